@@ -54,19 +54,30 @@ bool use_simt(const agent_attn_handle* h) {
     return h->cfg.dtype == AA_F32 || h->cfg.path == AA_PATH_SIMT;
 }
 
-// Large agent counts go to the tensor-memory kernel (the shape rule does not depend on the bias, so
-// that the workspace size is the same with and without one).
-bool use_umma(const agent_attn_handle* h, int n_tokens, int n_agents) {
+// Shapes that the tensor-memory kernels take (large agent counts, aligned rows).  The rule does not depend on the bias, so that
+// the workspace size is the same with and without one.
+bool umma_shape(const agent_attn_handle* h, int n_tokens, int n_agents) {
     return !use_simt(h) && auto_like(h) &&
            aggregate_umma_eligible(h->cfg.dtype, n_agents, n_tokens, h->cfg.head_dim, true);
+}
+// They win on long token axes (16384 tokens of 256 agents: 190 us against 247 us); below 8192 tokens their start and their
+// separate merge cost more than they save (4096 tokens: 60 us against 51 us; 464 tokens, 240 slabs: 157 us against 141 us) and
+// the register-tiled kernels run.
+bool use_umma(const agent_attn_handle* h, int n_tokens, int n_agents) {
+    return n_tokens >= 8192 && umma_shape(h, n_tokens, n_agents);
 }
 
 AggPlan plan_for(const agent_attn_handle* h, int n_tokens, int n_agents) {
     const int slabs = h->cfg.batch * h->cfg.heads;
     if (use_umma(h, n_tokens, n_agents))
         return plan_aggregate_umma(slabs, n_agents, n_tokens, h->cfg.head_dim, h->sm_count);
-    return use_simt(h) ? plan_aggregate_simt(slabs, n_agents, n_tokens, h->cfg.head_dim, h->sm_count)
-                       : plan_aggregate_mma(slabs, n_agents, n_tokens, h->cfg.head_dim, h->sm_count);
+    if (use_simt(h)) return plan_aggregate_simt(slabs, n_agents, n_tokens, h->cfg.head_dim, h->sm_count);
+    AggPlan pl;                     // register tiles: the states of a slab meet in shared memory
+    memset(&pl, 0, sizeof(pl));
+    pl.rows_pad = (n_agents + 15) / 16 * 16;
+    pl.dpad = h->cfg.head_dim;
+    pl.splits = pl.row_blocks = 1;
+    return pl;
 }
 
 // Plan of the streaming path for a call shape (cached in the handle); ok = false where it does not apply.
@@ -164,11 +175,27 @@ int do_pool(agent_attn_handle* h, const void* Q, int gh, int gw, int ph, int pw,
     return AA_OK;
 }
 
+TileArgs tile_args(const agent_attn_handle* h, int gh, int gw, int n, const CallLayout& cl) {
+    TileArgs t;
+    memset(&t, 0, sizeof(t));
+    t.slabs = h->cfg.batch * h->cfg.heads; t.heads = h->cfg.heads; t.N = gh * gw; t.n = n; t.d = h->cfg.head_dim;
+    t.H = gh; t.W = gw; t.scale1 = h->scale1; t.scale2 = h->scale2;
+    t.lin = cl.in; t.lout = cl.out;
+    return t;
+}
+
 int do_aggregate(agent_attn_handle* h, const void* A, const void* K, const void* V, const void* b1,
                  int N, int n, void* VA, float* partials, unsigned* tickets, cudaStream_t st,
                  const CallLayout* cl = nullptr) {
-    if (cl && cl->strided && !use_umma(h, N, n))
-        return fail(h, AA_ERR_UNSUPPORTED, "strided K and V need the fused or the tensor-memory kernels (16-bit, d <= 64, n <= 256)");
+    const bool umma = use_umma(h, N, n);
+    if (!umma && !use_simt(h)) {
+        TileArgs t = tile_args(h, 1, N, n, cl ? *cl : dense_call(h, N));
+        t.a = A; t.k = K; t.v = V; t.b1 = b1; t.va = VA;
+        const cudaError_t e = launch_tile_aggregate(h->cfg.dtype, t, h->sm_count, false, st);
+        if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "aggregation launch failed: %s", cudaGetErrorString(e));
+        h->launches++;
+        return AA_OK;
+    }
     const AggPlan pl = plan_for(h, N, n);
     cudaError_t e = cudaMemsetAsync(tickets, 0, (size_t)h->cfg.batch * h->cfg.heads * sizeof(unsigned), st);
     if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "ticket reset failed: %s", cudaGetErrorString(e));
@@ -183,17 +210,24 @@ int do_aggregate(agent_attn_handle* h, const void* A, const void* K, const void*
     a.lin = cl ? cl->in : dense_layout(h->cfg.heads, N, h->cfg.head_dim);
     a.lout = a.lin;
     a.strided = cl && cl->strided;
-    e = use_umma(h, N, n) ? launch_aggregate_umma(h->cfg.dtype, a, pl, st)
-        : use_simt(h)     ? launch_aggregate_simt(h->cfg.dtype, a, pl, st)
-                          : launch_aggregate_mma(h->cfg.dtype, a, pl, st);
+    e = umma ? launch_aggregate_umma(h->cfg.dtype, a, pl, st) : launch_aggregate_simt(h->cfg.dtype, a, pl, st);
     if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "aggregation launch failed: %s", cudaGetErrorString(e));
-    h->launches += use_umma(h, N, n) ? 2 : 1;      // the tensor-memory path merges in a second kernel
+    h->launches += umma ? 2 : 1;      // the tensor-memory path merges in a second kernel
     return AA_OK;
 }
 
 int do_broadcast(agent_attn_handle* h, const void* Q, const void* A, const void* VA, const void* V,
                  const void* b2, const void* wd, int gh, int gw, int n, void* out, cudaStream_t st,
                  const CallLayout* cl = nullptr) {
+    const bool umma = use_umma(h, gh * gw, n) && broadcast_umma_eligible(h->cfg.dtype, n, gh * gw, h->cfg.head_dim);
+    if (!umma && !use_simt(h)) {
+        TileArgs t = tile_args(h, gh, gw, n, cl ? *cl : dense_call(h, gh * gw));
+        t.q = Q; t.a = A; t.va = const_cast<void*>(VA); t.v = V; t.b2 = b2; t.wd = wd; t.out = out;
+        const cudaError_t e = launch_tile_broadcast(h->cfg.dtype, t, h->sm_count, false, st);
+        if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "broadcast launch failed: %s", cudaGetErrorString(e));
+        h->launches++;
+        return AA_OK;
+    }
     AttnArgs a;
     memset(&a, 0, sizeof(a));
     a.qm = Q; a.km = A; a.vm = VA; a.bias = b2; a.out = out;
@@ -205,13 +239,7 @@ int do_broadcast(agent_attn_handle* h, const void* Q, const void* A, const void*
     a.lin = cl ? cl->in : dense_layout(h->cfg.heads, (long long)gh * gw, h->cfg.head_dim);
     a.lout = cl ? cl->out : a.lin;
     a.strided = cl && cl->strided;
-    const bool umma = !use_simt(h) && auto_like(h) &&
-                      broadcast_umma_eligible(h->cfg.dtype, n, gh * gw, h->cfg.head_dim);
-    if (a.strided && !umma)
-        return fail(h, AA_ERR_UNSUPPORTED, "strided Q, V and out need the fused or the tensor-memory kernels (16-bit, d <= 64, n a multiple of 8 up to 256)");
-    cudaError_t e = umma          ? launch_broadcast_umma(h->cfg.dtype, a, h->sm_count, st)
-                    : use_simt(h) ? launch_broadcast_simt(h->cfg.dtype, a, st)
-                                  : launch_broadcast_mma(h->cfg.dtype, a, st);
+    const cudaError_t e = umma ? launch_broadcast_umma(h->cfg.dtype, a, h->sm_count, st) : launch_broadcast_simt(h->cfg.dtype, a, st);
     if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "broadcast launch failed: %s", cudaGetErrorString(e));
     h->launches++;
     return AA_OK;
@@ -396,6 +424,13 @@ static int forward_impl(agent_attn_handle* h, const void* Q, const void* K, cons
     cudaStream_t st = (cudaStream_t)stream;
     char* ws = static_cast<char*>(workspace);
     const CallLayout cl = clp ? *clp : dense_call(h, N);
+    // strided tensors: 16-bit types, pooled agents on grids of the task-queue kernel's kind, or large agent counts
+    if (cl.strided && !(auto_like(h) && !use_simt(h) &&
+                        ((!A && fused_parts_per_slab(h->cfg.dtype, grid_h, grid_w, h->cfg.head_dim, n_agents) > 0) ||
+                         (umma_shape(h, N, n_agents) && broadcast_umma_eligible(h->cfg.dtype, n_agents, N, h->cfg.head_dim)))))
+        return fail(h, AA_ERR_UNSUPPORTED,
+                    "strided tensors need 16-bit elements and either d = 64, n <= 64, pooled agents and W <= 64, or d <= 64 and n a "
+                    "multiple of 8 in 72..256");
     if (h->cfg.path == AA_PATH_AUTO && h->cfg.dtype != AA_F32 && !cl.strided) {
         // long token grids with few agents: three streaming kernels, phase by phase over the batch
         const StreamPlan& sp = stream_plan_for(h, grid_h, grid_w, n_agents, A == nullptr);
@@ -433,7 +468,7 @@ static int forward_impl(agent_attn_handle* h, const void* Q, const void* K, cons
             return AA_OK;
         }
     }
-    if (!A && auto_like(h) && h->cfg.dtype != AA_F32) {
+    if (!A && (h->cfg.path == AA_PATH_QUEUE || (h->cfg.path == AA_PATH_AUTO && cl.strided && N >= 1024)) && h->cfg.dtype != AA_F32) {
         // one persistent kernel for the whole module where the shape allows it
         if (h->fused_key[0] != grid_h || h->fused_key[1] != grid_w || h->fused_key[2] != n_agents) {
             h->fused_plan = plan_fused(h->cfg.dtype, h->cfg.batch * h->cfg.heads, grid_h, grid_w, h->cfg.head_dim,
@@ -462,13 +497,14 @@ static int forward_impl(agent_attn_handle* h, const void* Q, const void* K, cons
             return AA_OK;
         }
     }
-    // strided tensors are read in place only by the task-queue and the tensor-memory kernels: decide before anything
-    // is launched
-    if (cl.strided && !(use_umma(h, N, n_agents) && !use_simt(h) && auto_like(h) &&
-                        broadcast_umma_eligible(h->cfg.dtype, n_agents, N, h->cfg.head_dim)))
-        return fail(h, AA_ERR_UNSUPPORTED,
-                    "strided tensors need the task-queue kernel (16-bit, d = 64, n <= 64, pooled agents, W <= 64) or the "
-                    "tensor-memory kernels (16-bit, d <= 64, n a multiple of 8 in 72..256)");
+    if (!use_simt(h) && !use_umma(h, N, n_agents)) {
+        TileArgs t = tile_args(h, grid_h, grid_w, n_agents, cl);
+        t.q = Q; t.k = K; t.v = V; t.a = A ? A : ws + w.a_off; t.va = ws + w.va_off; t.pool = p;
+        t.b1 = b1; t.b2 = b2; t.wd = dwc_weight; t.out = out;
+        const cudaError_t e = launch_tile_forward(h->cfg.dtype, t, h->sm_count, h->cfg.path != AA_PATH_UNFUSED && tile_one_kernel(t), st, &h->launches);
+        if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "forward launch failed: %s", cudaGetErrorString(e));
+        return AA_OK;
+    }
     const void* agents = A;
     if (!A) {
         if (int rc = do_pool(h, Q, grid_h, grid_w, p, p, ws + w.a_off, st, &cl)) return rc;
@@ -750,7 +786,7 @@ extern "C" int agent_attn_aggregate_static(agent_attn_handle* h, const void* A, 
     // scratch layout: [partials | arrival counters], each 256-byte aligned
     const size_t slabs = (size_t)h->cfg.batch * h->cfg.heads;
     const AggPlan pl = plan_for(h, n_tokens, n_agents);
-    const size_t part_bytes = align_up(slabs * pl.parts * partial_floats(pl.rows_pad, pl.dpad) * sizeof(float), 256);
+    const size_t part_bytes = align_up(slabs * (pl.parts > 0 ? pl.parts : 1) * partial_floats(pl.rows_pad, pl.dpad) * sizeof(float), 256);
     const size_t need = part_bytes + align_up(slabs * sizeof(unsigned), 256);
     if (need > AA_STATIC_SCRATCH_BYTES)
         return fail(h, AA_ERR_WORKSPACE,

@@ -84,19 +84,33 @@ struct AggPlan {
     int row_blocks;   // blocks per slab along the agent axis (fp32 FMA path only)
 };
 
-// per-path planners and launchers (attn_simt.cu / aggregate_mma.cu / broadcast_mma.cu)
+// per-path planners and launchers (attn_simt.cu)
 AggPlan plan_aggregate_simt(int slabs, int n_agents, int n_tokens, int d, int sm_count);
-AggPlan plan_aggregate_mma(int slabs, int n_agents, int n_tokens, int d, int sm_count);
 cudaError_t launch_aggregate_simt(int dtype, const AttnArgs& p, const AggPlan& plan, cudaStream_t st);
 cudaError_t launch_broadcast_simt(int dtype, const AttnArgs& p, cudaStream_t st);
-cudaError_t launch_aggregate_mma(int dtype, const AttnArgs& p, const AggPlan& plan, cudaStream_t st);
-cudaError_t launch_broadcast_mma(int dtype, const AttnArgs& p, cudaStream_t st);
 // tensor-memory (tcgen05) kernels for large agent counts (aggregate_umma.cu)
 bool aggregate_umma_eligible(int dtype, int n_agents, int n_tokens, int d, bool has_bias);
 AggPlan plan_aggregate_umma(int slabs, int n_agents, int n_tokens, int d, int sm_count);
 cudaError_t launch_aggregate_umma(int dtype, const AttnArgs& p, const AggPlan& plan, cudaStream_t st);
 bool broadcast_umma_eligible(int dtype, int n_agents, int n_tokens, int d);
 cudaError_t launch_broadcast_umma(int dtype, const AttnArgs& p, int sm_count, cudaStream_t st);
+
+// Register-tiled kernels (tile_fwd.cuh): any 16-bit shape, grid and strides.
+struct TileArgs {
+    const void *q, *k, *v, *a;            // a: agents [slabs][n][d] (written first when `pool` is set)
+    void* va;                             // agent features [slabs][n][d]
+    const void *b1, *b2, *wd;
+    void* out;
+    int slabs, heads, N, n, d, H, W;
+    int pool;                             // pool x pool agents are pooled from q; 0: the caller's agents
+    float scale1, scale2;
+    TokLayout lin, lout;
+    int rg, kg, agg_tokens, bc_tokens;    // row groups and key groups of an aggregation block; tokens per block of either stage
+};
+cudaError_t launch_tile_forward(int dtype, TileArgs a, int sm_count, bool one_kernel, cudaStream_t st, int* launches);
+cudaError_t launch_tile_aggregate(int dtype, TileArgs a, int sm_count, bool dependent, cudaStream_t st);
+cudaError_t launch_tile_broadcast(int dtype, TileArgs a, int sm_count, bool dependent, cudaStream_t st);
+bool tile_one_kernel(const TileArgs& a);                 // the shape can run as one kernel
 
 // Whole module (Eq. 6) in one persistent kernel for small agent counts (n <= 64, d = 64,
 // block pooling, W <= 64).  Blocks take tasks from a device-side queue: "G" tasks pool their token

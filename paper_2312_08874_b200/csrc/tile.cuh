@@ -1,0 +1,257 @@
+// Building blocks of the register-tiled attention kernels (mma.sync m16n8k16, 16-bit operands, fp32 accumulators).
+//
+// A warp owns kMT x 16 rows of one softmax attention and walks its columns in blocks of 32: logits (kMT x 16 x 32) and
+// outputs (kMT x 16 x DK) stay in registers.  Rows are agents and columns tokens in the aggregation (Eq. 3, inner
+// attention); rows are tokens and columns agents in the broadcast (outer attention).
+//
+// Column order: inside a block, thread t of a quad owns columns 8 t .. 8 t + 7 (so its biases are one 16-byte load):
+// MMA column (j, 2 t + e), j = n-tile, stands for column 8 t + 2 j + e.  Key and value rows are put into shared memory in
+// that order (col_to_row), so the permutation costs nothing afterwards.
+#pragma once
+#include "common.cuh"
+#include "kernels.h"
+
+namespace aa {
+
+// Two m-tiles per warp halve the shared-memory reads per MMA (an operand fragment serves both); from 80 channels on the
+// accumulators leave registers for one only.
+template <int DK> struct TileGeom {
+    static constexpr int kMT = 1;
+    static constexpr int kRows = 16 * kMT;          // rows of a warp
+    static constexpr int kPitch = DK * 2 + 16;      // bytes between rows in shared memory: ldmatrix without bank conflicts
+    static constexpr int kKS = DK / 16;             // k steps of the logits
+    static constexpr int kNT = DK / 8;              // 8-channel tiles of the output
+};
+
+__device__ __forceinline__ int col_to_row(int c) { return (c & ~31) | ((c & 6) << 2) | ((c >> 2) & 6) | (c & 1); }
+
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+// D = A B (+ D): pure functions of their registers, so the compiler may interleave them with the softmax arithmetic.
+template <typename T> __device__ __forceinline__ void mma_acc(float* c, const uint32_t* a, uint32_t b0, uint32_t b1);
+template <typename T> __device__ __forceinline__ void mma_set(float* c, const uint32_t* a, uint32_t b0, uint32_t b1);
+#define AA_MMA_FORMS(TYPE, NAME)                                                                                          \
+    template <> __device__ __forceinline__ void mma_acc<TYPE>(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {      \
+        asm("mma.sync.aligned.m16n8k16.row.col.f32." NAME "." NAME ".f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n" \
+            : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1)); \
+    }                                                                                                                     \
+    template <> __device__ __forceinline__ void mma_set<TYPE>(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {      \
+        asm("mma.sync.aligned.m16n8k16.row.col.f32." NAME "." NAME ".f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};\n" \
+            : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])                                                              \
+            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));                                    \
+    }
+AA_MMA_FORMS(__nv_bfloat16, "bf16")
+AA_MMA_FORMS(__half, "f16")
+#undef AA_MMA_FORMS
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float d;
+    asm("max.f32 %0, %1, %2, %3;\n" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+__device__ __forceinline__ void cp_async16s(uint32_t dst, const void* src, int src_bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+}
+__device__ __forceinline__ void pdl_wait_prior() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_release_next() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync_all() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync_all(int csize) {
+    if (csize == 1) __syncthreads();
+    else cluster_sync_all();
+}
+__device__ __forceinline__ float ld_dsmem_f32(uint32_t addr, uint32_t rank) {
+    uint32_t a;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ float2 ld_dsmem_f32x2(uint32_t addr, uint32_t rank) {
+    uint32_t a;
+    float2 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.v2.f32 {%0,%1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ float quad_max(float v) {
+    v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 1));
+    return fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 2));
+}
+__device__ __forceinline__ float quad_sum(float v) {
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v + __shfl_xor_sync(0xffffffffu, v, 2);
+}
+
+// Byte offset (inside a block of key or value rows) that a lane hands to ldmatrix.
+template <int DK> __device__ __forceinline__ uint32_t key_lane_offset(int lane) {
+    return ((lane & 7) + ((lane >> 4) & 1) * 8) * TileGeom<DK>::kPitch + ((lane >> 3) & 1) * 16;
+}
+template <int DK> __device__ __forceinline__ uint32_t val_lane_offset(int lane) {
+    return (lane & 15) * TileGeom<DK>::kPitch + (lane >> 4) * 16;
+}
+
+// s = rows . keys^T for one block of 32 key rows at `kb` (lane offset included).
+template <typename T, int DK>
+__device__ __forceinline__ void tile_logits(float (&s)[TileGeom<DK>::kMT][4][4], const uint32_t (&a)[TileGeom<DK>::kMT][TileGeom<DK>::kKS][4],
+                                            uint32_t kb) {
+    using G = TileGeom<DK>;
+#pragma unroll
+    for (int ks = 0; ks < G::kKS; ++ks)
+#pragma unroll
+        for (int j2 = 0; j2 < 2; ++j2) {
+            uint32_t b[4];
+            ldsm4(b, kb + j2 * 16 * G::kPitch + ks * 32);
+#pragma unroll
+            for (int mt = 0; mt < G::kMT; ++mt) {
+                if (ks == 0) {
+                    mma_set<T>(s[mt][2 * j2], a[mt][ks], b[0], b[1]);
+                    mma_set<T>(s[mt][2 * j2 + 1], a[mt][ks], b[2], b[3]);
+                } else {
+                    mma_acc<T>(s[mt][2 * j2], a[mt][ks], b[0], b[1]);
+                    mma_acc<T>(s[mt][2 * j2 + 1], a[mt][ks], b[2], b[3]);
+                }
+            }
+        }
+}
+
+// o += p . values for one block of 32 value rows at `vb` (lane offset included).
+template <typename T, int DK>
+__device__ __forceinline__ void tile_values(float (&o)[TileGeom<DK>::kMT][TileGeom<DK>::kNT][4], const uint32_t (&p)[TileGeom<DK>::kMT][2][4],
+                                            uint32_t vb) {
+    using G = TileGeom<DK>;
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+        for (int c2 = 0; c2 < G::kNT / 2; ++c2) {
+            uint32_t b[4];
+            ldsm4t(b, vb + ks * 16 * G::kPitch + c2 * 32);
+#pragma unroll
+            for (int mt = 0; mt < G::kMT; ++mt) {
+                mma_acc<T>(o[mt][2 * c2], p[mt][ks], b[0], b[1]);
+                mma_acc<T>(o[mt][2 * c2 + 1], p[mt][ks], b[2], b[3]);
+            }
+        }
+}
+
+// Eight consecutive bias elements whose row starts at any element: `align` is the alignment (in elements: 8, 2 or 1)
+// that every row of the tensor has; the first `cnt` elements exist.
+template <typename T> __device__ __forceinline__ uint4 load_bias8(const T* p, int align, int cnt) {
+    uint4 r = make_uint4(0u, 0u, 0u, 0u);
+    if (cnt <= 0) return r;
+    if (align == 8) return __ldg(reinterpret_cast<const uint4*>(p));      // then cnt is a multiple of 8 too
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+    if (align == 2) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (2 * i < cnt) w[i] = __ldg(reinterpret_cast<const uint32_t*>(p) + i);
+    } else {
+        const unsigned short* u = reinterpret_cast<const unsigned short*>(p);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t lo = 2 * i < cnt ? __ldg(u + 2 * i) : 0, hi = 2 * i + 1 < cnt ? __ldg(u + 2 * i + 1) : 0;
+            w[i] = lo | (hi << 16);
+        }
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Running state of the softmax of a warp's rows (row index: m-tile, half).  `ref` is the exponent reference in log2
+// units, taken from the row's first block; it moves only when a logit exceeds it by more than 8 (so the products are
+// rescaled rarely, and probabilities stay below 2^8: inside fp16).  `lim` is that 8, or -inf while the row has no weight.
+template <int MT> struct SoftRows {
+    float ref[MT][2], lim[MT][2];
+    float2 sum[MT][2];
+    __device__ __forceinline__ void init() {
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) { ref[m][h] = 0.f; lim[m][h] = -INFINITY; sum[m][h] = make_float2(0.f, 0.f); }
+    }
+    __device__ __forceinline__ float total(int m, int h) const { return quad_sum(sum[m][h].x + sum[m][h].y); }
+};
+
+// Logits of one block -> probabilities as MMA operands.  x = s * c1 + bias * log2(e) - ref; columns at and past `valid`
+// (counted inside the block) are removed.
+template <typename T, int DK, int BIAS>
+__device__ __forceinline__ void tile_softmax(float (&s)[TileGeom<DK>::kMT][4][4], const uint4 (&bias)[TileGeom<DK>::kMT][2], float c1, int valid,
+                                             int t, SoftRows<TileGeom<DK>::kMT>& st, float (&o)[TileGeom<DK>::kMT][TileGeom<DK>::kNT][4],
+                                             uint32_t (&p)[TileGeom<DK>::kMT][2][4]) {
+    using G = TileGeom<DK>;
+    float2 x[G::kMT][2][4];
+#pragma unroll
+    for (int mt = 0; mt < G::kMT; ++mt)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float2 nref = make_float2(-st.ref[mt][h], -st.ref[mt][h]);
+            const uint32_t w[4] = {bias[mt][h].x, bias[mt][h].y, bias[mt][h].z, bias[mt][h].w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float2 y = nref;
+                if constexpr (BIAS != 0) y = ffma2(unpack2<T>(w[j]), make_float2(kLog2e, kLog2e), nref);
+                x[mt][h][j] = ffma2(make_float2(s[mt][j][2 * h], s[mt][j][2 * h + 1]), make_float2(c1, c1), y);
+            }
+        }
+    if (valid < 32) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int c = 8 * t + 2 * j;
+#pragma unroll
+            for (int mt = 0; mt < G::kMT; ++mt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (c >= valid) x[mt][h][j].x = -INFINITY;
+                    if (c + 1 >= valid) x[mt][h][j].y = -INFINITY;
+                }
+        }
+    }
+    float mx[G::kMT][2];
+    bool grow = false;
+#pragma unroll
+    for (int mt = 0; mt < G::kMT; ++mt)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float m = fmaxf(x[mt][h][0].x, x[mt][h][0].y);
+#pragma unroll
+            for (int j = 1; j < 4; ++j) m = max3(m, x[mt][h][j].x, x[mt][h][j].y);
+            mx[mt][h] = m;
+            grow |= m > st.lim[mt][h];
+        }
+    if (__any_sync(0xffffffffu, grow)) {
+#pragma unroll
+        for (int mt = 0; mt < G::kMT; ++mt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float m = quad_max(mx[mt][h]);
+                const bool first = st.lim[mt][h] < 0.f;                   // then nothing is accumulated yet
+                const float by = m > st.lim[mt][h] ? m : 0.f;
+                const float f = first ? 1.f : fast_exp2(-by);
+                if (m > -INFINITY) st.lim[mt][h] = 8.f;
+                st.ref[mt][h] += by;
+                st.sum[mt][h].x *= f;
+                st.sum[mt][h].y *= f;
+#pragma unroll
+                for (int c = 0; c < G::kNT; ++c) { o[mt][c][2 * h] *= f; o[mt][c][2 * h + 1] *= f; }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) { x[mt][h][j].x -= by; x[mt][h][j].y -= by; }
+            }
+    }
+#pragma unroll
+    for (int mt = 0; mt < G::kMT; ++mt)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 e = make_float2(fast_exp2(x[mt][h][j].x), fast_exp2(x[mt][h][j].y));
+                st.sum[mt][h] = fadd2(st.sum[mt][h], e);
+                p[mt][j >> 1][(j & 1) * 2 + h] = pack2<T>(e.x, e.y);
+            }
+}
+
+}  // namespace aa

@@ -1,0 +1,162 @@
+// Launch plans of the register-tiled forward kernels.
+#include "tile_launch.cuh"
+
+#include <algorithm>
+
+namespace aa {
+
+namespace {
+
+struct DkInfo {
+    int dk;
+};
+DkInfo dk_of(int d) {
+    DkInfo i;
+    i.dk = d <= 32 ? 32 : d <= 48 ? 48 : d <= 64 ? 64 : d <= 80 ? 80 : d <= 96 ? 96 : 128;
+    return i;
+}
+cudaError_t dispatch(TileKernel k, int dtype, int dk, int bias, const TileArgs& a, const TileLaunch& l) {
+    switch (dk) {
+        case 32: return tile_dispatch_32(k, dtype, bias, a, l);
+        case 48: return tile_dispatch_48(k, dtype, bias, a, l);
+        case 64: return tile_dispatch_64(k, dtype, bias, a, l);
+        case 80: return tile_dispatch_80(k, dtype, bias, a, l);
+        case 96: return tile_dispatch_96(k, dtype, bias, a, l);
+        default: return tile_dispatch_128(k, dtype, bias, a, l);
+    }
+}
+template <int DK> int agg_smem_dk(int kg) { return kg == 1 ? AggShape<DK, 1>::kSmem : kg == 2 ? AggShape<DK, 2>::kSmem : AggShape<DK, 4>::kSmem; }
+int agg_smem(int dk, int kg) {
+    switch (dk) {
+        case 32: return agg_smem_dk<32>(kg);
+        case 48: return agg_smem_dk<48>(kg);
+        case 64: return agg_smem_dk<64>(kg);
+        case 80: return agg_smem_dk<80>(kg);
+        case 96: return agg_smem_dk<96>(kg);
+        default: return agg_smem_dk<128>(kg);
+    }
+}
+int bc_smem(int dk, const TileArgs& a, int warps) {
+    const bool dwc = a.wd != nullptr;
+    switch (dk) {
+        case 32: return BcShape<32>::smem_bytes(a.n, warps, a.W, dwc);
+        case 48: return BcShape<48>::smem_bytes(a.n, warps, a.W, dwc);
+        case 64: return BcShape<64>::smem_bytes(a.n, warps, a.W, dwc);
+        case 80: return BcShape<80>::smem_bytes(a.n, warps, a.W, dwc);
+        case 96: return BcShape<96>::smem_bytes(a.n, warps, a.W, dwc);
+        default: return BcShape<128>::smem_bytes(a.n, warps, a.W, dwc);
+    }
+}
+int bias_align(int row) { return row % 8 == 0 ? 8 : 1; }
+int bias_kind(const void* b, int align) { return !b ? 0 : align == 8 ? 1 : 2; }
+int up32(int x) { return (x + 31) & ~31; }
+
+// Row and key groups of an aggregation block: at most eight warps, all of them with rows.
+int agg_rows(const TileArgs& a, const DkInfo& dk, TileArgs* out) {
+    const int rb = (a.n + 8 * 16 - 1) / (8 * 16);
+    out->rg = ((a.n + rb - 1) / rb + 16 - 1) / 16;
+    out->kg = out->rg <= 2 ? 4 : out->rg <= 4 ? 2 : 1;
+    return rb;
+}
+
+}  // namespace
+
+cudaError_t launch_tile_aggregate(int dtype, TileArgs a, int sm_count, bool dependent, cudaStream_t st) {
+    const DkInfo dk = dk_of(a.d);
+    const int rb = agg_rows(a, dk, &a);
+    
+    a.b2 = nullptr;
+    // Parts of the token axis (one block each, a cluster per slab).  Two blocks share an SM and hide each other's
+    // latencies, so the best split is the one with the shortest blocks in the fewest waves; a block's start and merge count as
+    // 128 tokens.
+    int best = 1;
+    long long best_cost = 0;
+    for (int c = 1; c <= 8; c *= 2) {
+        const int tokens = up32((a.N + c - 1) / c);
+        if (c > 1 && (tokens < 64 || c * a.kg > 32)) break;
+        const long long blocks = (long long)a.slabs * rb * c;
+        const long long cost = ((blocks + 2LL * sm_count - 1) / (2LL * sm_count)) * (tokens + 128LL);
+        if (c == 1 || cost < best_cost) { best = c; best_cost = cost; }
+    }
+    a.agg_tokens = up32((a.N + best - 1) / best);
+    TileLaunch l;
+    l.grid = dim3(best, rb, a.slabs);
+    l.threads = kAggThreads;
+    l.cluster = best;
+    l.smem = agg_smem(dk.dk, a.kg);
+    l.dependent = dependent;
+    l.stream = st;
+    return dispatch(kTileAggregate, dtype, dk.dk, bias_kind(a.b1, bias_align(a.N)), a, l);
+}
+
+cudaError_t launch_tile_broadcast(int dtype, TileArgs a, int sm_count, bool dependent, cudaStream_t st) {
+    const DkInfo dk = dk_of(a.d);
+    
+    a.b1 = nullptr;
+    // Small agent counts: blocks of eight warps, two to an SM.  Large ones: the agents and their features fill a third of
+    // the shared memory or more, so one block of sixteen warps shares them.
+    const bool pair = bc_smem(dk.dk, a, 8) <= 113 * 1024;
+    int warps = pair ? 8 : 16;
+    while (bc_smem(dk.dk, a, warps) > 227 * 1024) warps -= 4;      // (256 agents of 128 channels: 8; four always fit)
+    const int slots = pair ? 2 * sm_count : sm_count;
+    const int pass = warps * 16;                       // tokens of one pass of a block
+    int best = 1;
+    double best_cost = 0;
+    for (int k = 1; k <= 16; ++k) {
+        const long long blocks = (long long)a.slabs * ((a.N + (long long)pass * k - 1) / ((long long)pass * k));
+        const double cost = (double)((blocks + slots - 1) / slots) * (k + 0.4);
+        if (k == 1 || cost < best_cost) { best = k; best_cost = cost; }
+        if ((long long)pass * k >= a.N) break;
+    }
+    a.bc_tokens = pass * best;
+    TileLaunch l;
+    l.grid = dim3((a.N + a.bc_tokens - 1) / a.bc_tokens, a.slabs);
+    l.threads = warps * 32;
+    l.cluster = 0;
+    l.smem = bc_smem(dk.dk, a, warps);
+    l.dependent = dependent;
+    l.stream = st;
+    return dispatch(kTileBroadcast, dtype, dk.dk, bias_kind(a.b2, bias_align(a.n)), a, l);
+}
+
+bool tile_one_kernel(const TileArgs& a) {
+    const DkInfo dk = dk_of(a.d);
+    if (a.n > 8 * 16 || bc_smem(dk.dk, a, 8) > 113 * 1024) return false;
+    return a.N <= 1024;
+}
+
+cudaError_t launch_tile_forward(int dtype, TileArgs a, int sm_count, bool one_kernel, cudaStream_t st, int* launches) {
+    if (one_kernel) {
+        const DkInfo dk = dk_of(a.d);
+        agg_rows(a, dk, &a);
+        
+        
+        int c = 1;
+        while (c < 8 && (long long)a.slabs * 2 * c <= 2LL * sm_count && up32((a.N + 2 * c - 1) / (2 * c)) >= 32 && a.N > 32 * c) c *= 2;
+        a.agg_tokens = up32((a.N + c - 1) / c);
+        TileLaunch l;
+        l.grid = dim3(c, a.slabs);
+        l.threads = kAggThreads;
+        l.cluster = c;
+        l.smem = std::max(agg_smem(dk.dk, a.kg), bc_smem(dk.dk, a, 8));
+        l.dependent = false;
+        l.stream = st;
+        *launches += 1;
+        return dispatch(kTileSlab, dtype, dk.dk, !a.b1 && !a.b2 ? 0 : a.b1 && a.b2 && a.N % 8 == 0 && a.n % 8 == 0 ? 1 : 2, a, l);
+    }
+    if (a.pool) {
+        const unsigned blocks = (unsigned)(((long long)a.slabs * a.n + 7) / 8);
+        if (dtype == kBF16) tile_pool_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(a);
+        else tile_pool_kernel<__half><<<blocks, 256, 0, st>>>(a);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        *launches += 1;
+    }
+    cudaError_t e = launch_tile_aggregate(dtype, a, sm_count, a.pool != 0, st);
+    if (e != cudaSuccess) return e;
+    e = launch_tile_broadcast(dtype, a, sm_count, true, st);
+    *launches += 2;
+    return e;
+}
+
+}  // namespace aa

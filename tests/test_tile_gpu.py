@@ -1,0 +1,35 @@
+"""Register-tiled kernels at the edges of their tiles, against the fp64 oracle."""
+import pytest
+import torch
+
+from paper_2312_08874_b200 import Workload, make_inputs
+from tests.parity_util import assert_close, gpu_forward, make_module, oracle_forward
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [
+    # batch heads H   W   d   pool dtype  bias  dwc
+    (1, 1, 4, 4, 8, 4, "f16", True, True),           # as many agents as tokens, channels padded from 8 to 32
+    (2, 1, 31, 33, 72, 4, "bf16", True, True),       # 1023 tokens: one kernel; 16 agents, odd bias rows, channels padded
+    (2, 2, 32, 33, 64, 5, "bf16", True, True),       # 1056 tokens: three kernels; two row groups, ragged last tile
+    (1, 3, 5, 300, 64, 5, "f16", True, True),        # W > tile: the halo in three runs
+    (1, 1, 3, 131, 40, 3, "bf16", False, True),      # W one past the single-run halo
+    (1, 2, 130, 9, 104, 9, "bf16", True, True),      # 81 agents (six row groups), 104 channels padded to 128
+    (1, 1, 45, 45, 64, 11, "f16", True, True),       # 121 agents: the last block that fits one row block, unaligned bias rows
+    (1, 1, 40, 41, 32, 13, "bf16", True, False),     # 169 agents: two row blocks, bias rows read from global memory
+    (1, 1, 33, 32, 128, 16, "bf16", True, True),     # 256 agents of 128 channels
+    (160, 2, 11, 13, 64, 7, "bf16", True, True),     # more slabs than resident blocks: a cluster of one
+]
+
+
+@pytest.mark.parametrize("case", SHAPES, ids=[f"B{c[0]}h{c[1]}_{c[2]}x{c[3]}_d{c[4]}_p{c[5]}" for c in SHAPES])
+def test_tile_edges_match_oracle(case):
+    B, heads, H, W, d, pool, dtype, bias, dwc = case
+    w = Workload("tile", B, heads, H, W, d, pool, dtype, bias, dwc, 1.0, seed=700 + H * W + d)
+    inp = make_inputs(w, bias_std=0.5, dwc_std=0.2)
+    mod = make_module(w)
+    out = gpu_forward(mod, w, inp)
+    slabs = [(0, 0), (B - 1, heads - 1)]
+    for (b, h), ref in zip(slabs, oracle_forward(w, inp, slabs=slabs)):
+        assert_close(out[b:b + 1, h:h + 1], ref, dtype, f"{case} slab {(b, h)}")
+    assert torch.equal(out, gpu_forward(mod, w, inp)), "bit-reproducible"
