@@ -1,6 +1,6 @@
 // Aggregation on register tiles: V_A = softmax(scale1 A K^T + B1) V (Eq. 3 inner attention, bias of Eq. 5).
 //
-// A block of eight warps owns up to 128 agent rows of a slab and a range of its tokens: rg row groups of 16 agents times KG key
+// A block of NW warps owns up to 16 NW agent rows of a slab and a range of its tokens: rg row groups of 16 agents times KG key
 // groups that take alternate 32-token blocks.  Keys and values stream through a cp.async ring; the blocks of a slab form a
 // thread-block cluster and merge their softmax states through distributed shared memory at the end.
 #pragma once
@@ -8,20 +8,20 @@
 
 namespace aa {
 
-constexpr int kAggThreads = 256;
 constexpr int kAggStages = 3;
 
-template <int DK, int KG> struct AggShape {
+template <int DK, int KG, int NW> struct AggShape {
     using G = TileGeom<DK>;
-    static constexpr int kTokens = KG == 1 ? 64 : 128;                 // tokens of a stage
+    static constexpr int kThreads = NW * 32;
+    static constexpr int kTokens = KG == 1 || KG * NW == 8 ? 64 : 128;                 // tokens of a stage
     static constexpr int kStage = 2 * kTokens * G::kPitch;             // K rows, then V rows
     static constexpr int kAccPitch = DK + 8;                           // fp32 words between the rows of a partial state
-    static constexpr int kPart = 8 * 16 * (kAccPitch + 2) * 4;         // partial states of eight warps (over the ring, after the loop)
-    static constexpr int kMerge = kPart + 128 * 8 * KG * 4;            // and the merge weights
+    static constexpr int kPart = NW * 16 * (kAccPitch + 2) * 4;         // partial states of the warps (over the ring, after the loop)
+    static constexpr int kMerge = kPart + NW * 16 * 8 * KG * 4;            // and the merge weights
     static constexpr int kSmem = kAggStages * kStage > kMerge ? kAggStages * kStage : kMerge;
     // copies: a thread keeps its 16-byte channel chunk and steps by kRowStep rows
     static constexpr int kChunks = DK / 8;
-    static constexpr int kRowStep = kChunks <= 4 ? 64 : kChunks <= 8 ? 32 : 16;
+    static constexpr int kRowStep = (kChunks <= 4 ? 64 : kChunks <= 8 ? 32 : 16) * NW / 8;
 };
 
 template <typename T> struct AggCta {
@@ -54,16 +54,16 @@ template <typename T> __device__ __forceinline__ uint4 load_bias8_any(const T* p
 }
 
 // One stage of keys and values: token rows in block order, channels past d and tokens past the range zero.
-template <typename T, int DK, int KG>
+template <typename T, int DK, int KG, int NW>
 __device__ __forceinline__ void agg_load(const AggCta<T>& c, uint32_t dst, const T* kp, const T* vp, int left) {
     using G = TileGeom<DK>;
-    using S = AggShape<DK, KG>;
+    using S = AggShape<DK, KG, NW>;
     const long long step = S::kRowStep * c.kst;
     if (left >= S::kTokens) {
 #pragma unroll
         for (int i = 0; i < S::kTokens / S::kRowStep; ++i) {
             constexpr int R = S::kRowStep;
-            const int off = ((i * R & ~31) + ((i * R >> 2) & 6)) * G::kPitch;          // col_to_row(i * R): R is 16, 32 or 64
+            const int off = ((i * R & ~31) + ((i * R >> 2) & 6)) * G::kPitch;          // col_to_row(i * R): R is 8, 16, 32 or 64
             cp_async16s(dst + off, kp + i * step, 16);
             cp_async16s(dst + S::kTokens * G::kPitch + off, vp + i * step, 16);
         }
@@ -80,10 +80,10 @@ __device__ __forceinline__ void agg_load(const AggCta<T>& c, uint32_t dst, const
 
 // Aggregation over the block's token range; leaves the warps' partial states in `smem`.  `wait_agents` runs after the first
 // copies have been issued.  BIAS: 0 none, 1 rows of 16-byte pieces (N a multiple of 8), 2 any row length.
-template <typename T, int DK, int KG, int BIAS, typename F>
+template <typename T, int DK, int KG, int NW, int BIAS, typename F>
 __device__ __forceinline__ void agg_phase(const AggCta<T>& c, unsigned char* smem, F&& wait_agents) {
     using G = TileGeom<DK>;
-    using S = AggShape<DK, KG>;
+    using S = AggShape<DK, KG, NW>;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     int rgi = warp, kgi = 0;
     if (KG > 1 && rgi >= c.rg) { rgi -= c.rg; ++kgi; }
@@ -104,7 +104,7 @@ __device__ __forceinline__ void agg_phase(const AggCta<T>& c, unsigned char* sme
     const long long tile_step = (long long)S::kTokens * c.kst;
 #pragma unroll
     for (int i = 0; i < kAggStages - 1; ++i) {
-        if (loader && i < tiles) agg_load<T, DK, KG>(c, ldst + i * S::kStage, kp + i * tile_step, vp + i * tile_step, c.t1 - c.t0 - i * S::kTokens);
+        if (loader && i < tiles) agg_load<T, DK, KG, NW>(c, ldst + i * S::kStage, kp + i * tile_step, vp + i * tile_step, c.t1 - c.t0 - i * S::kTokens);
         cp_async_commit();
     }
     kp += (kAggStages - 1) * tile_step;
@@ -153,7 +153,7 @@ __device__ __forceinline__ void agg_phase(const AggCta<T>& c, unsigned char* sme
     for (int it = 0; it < tiles; ++it) {
         cp_async_wait<kAggStages - 2>();
         __syncthreads();
-        if (loader && left > 0) agg_load<T, DK, KG>(c, ldst + wr, kp, vp, left);
+        if (loader && left > 0) agg_load<T, DK, KG, NW>(c, ldst + wr, kp, vp, left);
         cp_async_commit();
         kp += tile_step; vp += tile_step; left -= S::kTokens;
         if (active) {
@@ -177,7 +177,7 @@ __device__ __forceinline__ void agg_phase(const AggCta<T>& c, unsigned char* sme
     cp_async_wait<0>();
     __syncthreads();
     float* acc = reinterpret_cast<float*>(smem) + warp * 16 * S::kAccPitch;
-    float2* ml = reinterpret_cast<float2*>(smem + 8 * 16 * S::kAccPitch * 4) + warp * 16;
+    float2* ml = reinterpret_cast<float2*>(smem + NW * 16 * S::kAccPitch * 4) + warp * 16;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int r = h * 8 + g;
@@ -193,11 +193,11 @@ __device__ __forceinline__ void agg_phase(const AggCta<T>& c, unsigned char* sme
 // agent rows (r = crank, crank + csize, ...).  A thread per row turns (reference, sum) pairs into weights, then a thread per two
 // channels adds up: loads of different sources are independent, so the latency is that of two of them.  Fixed order:
 // bit-reproducible.
-template <typename T, int DK, int KG>
+template <typename T, int DK, int KG, int NW>
 __device__ __forceinline__ void agg_merge(const AggCta<T>& c, unsigned char* smem, int crank, int csize) {
-    using S = AggShape<DK, KG>;
+    using S = AggShape<DK, KG, NW>;
     const int rows = min(c.rg * 16, c.n - c.row0);
-    const uint32_t acc0 = smem_u32(smem), ml0 = acc0 + 8 * 16 * S::kAccPitch * 4;
+    const uint32_t acc0 = smem_u32(smem), ml0 = acc0 + NW * 16 * S::kAccPitch * 4;
     float* wt = reinterpret_cast<float*>(smem + S::kPart);                    // [share][csize * KG], normalised
     const int nsrc = csize * KG, share = (rows - crank + csize - 1) / csize;
     if ((int)threadIdx.x < share) {
@@ -225,7 +225,7 @@ __device__ __forceinline__ void agg_merge(const AggCta<T>& c, unsigned char* sme
             if (q < nsrc) wt[threadIdx.x * nsrc + q] = m[q] * inv;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < share * (DK / 2); i += kAggThreads) {
+    for (int i = threadIdx.x; i < share * (DK / 2); i += S::kThreads) {
         const int k = i / (DK / 2), ch = 2 * (i - k * (DK / 2)), r = crank + k * csize;
         if (ch >= c.d) continue;
         const uint32_t src = acc0 + (r * S::kAccPitch + ch) * 4;

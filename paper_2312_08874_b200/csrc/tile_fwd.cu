@@ -25,15 +25,18 @@ cudaError_t dispatch(TileKernel k, int dtype, int dk, int bias, const TileArgs& 
         default: return tile_dispatch_128(k, dtype, bias, a, l);
     }
 }
-template <int DK> int agg_smem_dk(int kg) { return kg == 1 ? AggShape<DK, 1>::kSmem : kg == 2 ? AggShape<DK, 2>::kSmem : AggShape<DK, 4>::kSmem; }
-int agg_smem(int dk, int kg) {
+template <int DK> int agg_smem_dk(int kg, int warps) {
+    if (warps == 8) return kg == 1 ? AggShape<DK, 1, 8>::kSmem : kg == 2 ? AggShape<DK, 2, 8>::kSmem : AggShape<DK, 4, 8>::kSmem;
+    return kg == 1 ? AggShape<DK, 1, 4>::kSmem : kg == 2 ? AggShape<DK, 2, 4>::kSmem : AggShape<DK, 4, 4>::kSmem;
+}
+int agg_smem(int dk, int kg, int warps) {
     switch (dk) {
-        case 32: return agg_smem_dk<32>(kg);
-        case 48: return agg_smem_dk<48>(kg);
-        case 64: return agg_smem_dk<64>(kg);
-        case 80: return agg_smem_dk<80>(kg);
-        case 96: return agg_smem_dk<96>(kg);
-        default: return agg_smem_dk<128>(kg);
+        case 32: return agg_smem_dk<32>(kg, warps);
+        case 48: return agg_smem_dk<48>(kg, warps);
+        case 64: return agg_smem_dk<64>(kg, warps);
+        case 80: return agg_smem_dk<80>(kg, warps);
+        case 96: return agg_smem_dk<96>(kg, warps);
+        default: return agg_smem_dk<128>(kg, warps);
     }
 }
 int bc_smem(int dk, const TileArgs& a, int warps) {
@@ -81,9 +84,9 @@ cudaError_t launch_tile_aggregate(int dtype, TileArgs a, int sm_count, bool depe
     a.agg_tokens = up32((a.N + best - 1) / best);
     TileLaunch l;
     l.grid = dim3(best, rb, a.slabs);
-    l.threads = kAggThreads;
+    l.threads = 256;
     l.cluster = best;
-    l.smem = agg_smem(dk.dk, a.kg);
+    l.smem = agg_smem(dk.dk, a.kg, 8);
     l.dependent = dependent;
     l.stream = st;
     return dispatch(kTileAggregate, dtype, dk.dk, bias_kind(a.b1, bias_align(a.N)), a, l);
@@ -119,26 +122,28 @@ cudaError_t launch_tile_broadcast(int dtype, TileArgs a, int sm_count, bool depe
     return dispatch(kTileBroadcast, dtype, dk.dk, bias_kind(a.b2, bias_align(a.n)), a, l);
 }
 
+// Blocks of four warps (up to 64 agents) or eight: registers for sixteen warps an SM either way.
 bool tile_one_kernel(const TileArgs& a) {
     const DkInfo dk = dk_of(a.d);
-    if (a.n > 8 * 16 || bc_smem(dk.dk, a, 8) > 113 * 1024) return false;
-    return a.N <= 1024;
+    return a.N <= 1024 && a.n <= 128 && bc_smem(dk.dk, a, a.n <= 64 ? 4 : 8) <= 113 * 1024;
 }
 
 cudaError_t launch_tile_forward(int dtype, TileArgs a, int sm_count, bool one_kernel, cudaStream_t st, int* launches) {
     if (one_kernel) {
         const DkInfo dk = dk_of(a.d);
-        agg_rows(a, dk, &a);
-        
-        
-        int c = 1;
-        while (c < 8 && (long long)a.slabs * 2 * c <= 2LL * sm_count && up32((a.N + 2 * c - 1) / (2 * c)) >= 32 && a.N > 32 * c) c *= 2;
-        a.agg_tokens = up32((a.N + c - 1) / c);
+        const int warps = a.n <= 64 ? 4 : 8;
+        a.rg = (a.n + 15) / 16;
+        a.kg = warps == 8 || a.rg > 2 ? 1 : a.rg == 2 ? 2 : 4;
         TileLaunch l;
+        l.smem = std::max(agg_smem(dk.dk, a.kg, warps), bc_smem(dk.dk, a, warps));
+        // blocks per slab: as many as are resident at once
+        const long long slots = std::min<long long>(16 / warps, 227 * 1024 / (l.smem + 1024)) * sm_count;
+        int c = 1;
+        while (c < 8 && a.slabs * 2LL * c <= slots && a.N > 32 * c) c *= 2;
+        a.agg_tokens = up32((a.N + c - 1) / c);
         l.grid = dim3(c, a.slabs);
-        l.threads = kAggThreads;
+        l.threads = warps * 32;
         l.cluster = c;
-        l.smem = std::max(agg_smem(dk.dk, a.kg), bc_smem(dk.dk, a, 8));
         l.dependent = false;
         l.stream = st;
         *launches += 1;

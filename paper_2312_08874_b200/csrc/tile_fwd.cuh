@@ -122,13 +122,13 @@ __device__ __forceinline__ BcCta<T> bc_cta(const TileArgs& p, int slab, int part
 
 // grid (cluster of token parts, row blocks, slabs)
 template <typename T, int DK, int KG, int BIAS>
-__global__ void __launch_bounds__(kAggThreads, 2) tile_aggregate_kernel(const __grid_constant__ TileArgs p) {
+__global__ void __launch_bounds__(256, 2) tile_aggregate_kernel(const __grid_constant__ TileArgs p) {
     extern __shared__ __align__(128) unsigned char smem[];
     pdl_release_next();
     const AggCta<T> c = agg_cta<T>(p, blockIdx.z, blockIdx.x, blockIdx.y);
-    agg_phase<T, DK, KG, BIAS>(c, smem, [] { pdl_wait_prior(); });
+    agg_phase<T, DK, KG, 8, BIAS>(c, smem, [] { pdl_wait_prior(); });
     cluster_sync_all(gridDim.x);
-    agg_merge<T, DK, KG>(c, smem, blockIdx.x, gridDim.x);
+    agg_merge<T, DK, KG, 8>(c, smem, blockIdx.x, gridDim.x);
     if (gridDim.x > 1) cluster_sync_all();                                // siblings still read this block's shared memory
 }
 
@@ -146,37 +146,37 @@ __global__ void __launch_bounds__(512, 1) tile_broadcast_kernel(const __grid_con
 }
 
 // Short grids: a cluster of blocks per slab runs the three phases, tied by cluster barriers.  grid (cluster, slabs)
-template <typename T, int DK, int KG, int BIAS>
-__global__ void __launch_bounds__(kAggThreads, 2) tile_slab_kernel(const __grid_constant__ TileArgs p) {
+template <typename T, int DK, int KG, int NW, int BIAS>
+__global__ void __launch_bounds__(NW * 32, 16 / NW) tile_slab_kernel(const __grid_constant__ TileArgs p) {
     extern __shared__ __align__(128) unsigned char smem[];
     const int slab = blockIdx.y, crank = blockIdx.x, csize = gridDim.x, warp = threadIdx.x >> 5;
     const AggCta<T> c = agg_cta<T>(p, slab, crank, 0);
-    agg_phase<T, DK, KG, BIAS>(c, smem, [&] {
+    agg_phase<T, DK, KG, NW, BIAS>(c, smem, [&] {
         if (p.pool) {
             const T* q = static_cast<const T*>(p.q) + tok_offset(p.lin, slab, p.heads, 0);
             T* a = const_cast<T*>(c.a);
             if (p.H * p.W <= 32 * p.n) {                 // small windows: a thread per 16 bytes of an agent
                 const int cpt = p.d >> 3, items = (p.n - crank + csize - 1) / csize * cpt;
-                for (int i = threadIdx.x; i < items; i += kAggThreads) {
+                for (int i = threadIdx.x; i < items; i += NW * 32) {
                     const int agent = crank + i / cpt * csize, ch = i % cpt;
                     pool_chunk<T>(q + ch * 8, p.lin.st, p.H, p.W, p.pool, agent, a + (size_t)agent * p.d + ch * 8);
                 }
             } else {
-                for (int i = crank + warp * csize; i < p.n; i += csize * (kAggThreads / 32))
+                for (int i = crank + warp * csize; i < p.n; i += csize * (NW))
                     pool_window<T>(q, p.lin.st, p.H, p.W, p.pool, i, p.d, a + (size_t)i * p.d);
             }
             cluster_sync_all(csize);
         }
     });
     cluster_sync_all(csize);
-    agg_merge<T, DK, KG>(c, smem, crank, csize);
+    agg_merge<T, DK, KG, NW>(c, smem, crank, csize);
     cluster_sync_all(csize);
     const BcCta<T> b = bc_cta<T>(p, slab, crank, p.agg_tokens);
     bc_fill<T, DK>(b, smem);
     cp_async_commit();
     cp_async_wait<0>();
     __syncthreads();
-    bc_phase<T, DK, BIAS>(b, smem, kAggThreads / 32);
+    bc_phase<T, DK, BIAS>(b, smem, NW);
 }
 
 template <typename T>

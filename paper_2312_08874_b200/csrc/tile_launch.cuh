@@ -56,9 +56,10 @@ template <typename K> inline cudaError_t tile_launch(K kern, std::atomic<unsigne
 
 // BIAS: 0 none, 1 rows of 16-byte pieces, 2 any alignment
 template <typename T, int DK, int KG, int BIAS> cudaError_t tile_dispatch_kg(TileKernel k, const TileArgs& a, const TileLaunch& l) {
-    static std::atomic<unsigned long long> done[2];
+    static std::atomic<unsigned long long> done[3];
     if (k == kTileAggregate) return tile_launch(tile_aggregate_kernel<T, DK, KG, BIAS>, done[0], a, l);
-    return tile_launch(tile_slab_kernel<T, DK, KG, BIAS>, done[1], a, l);
+    if (KG == 1 && l.threads == 256) return tile_launch(tile_slab_kernel<T, DK, 1, 8, BIAS>, done[1], a, l);
+    return tile_launch(tile_slab_kernel<T, DK, KG, 4, BIAS>, done[2], a, l);
 }
 template <typename T, int DK, int BIAS> cudaError_t tile_dispatch_b(TileKernel k, const TileArgs& a, const TileLaunch& l) {
     static std::atomic<unsigned long long> done;
