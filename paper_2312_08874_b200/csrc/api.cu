@@ -648,8 +648,12 @@ int agent_attn_query_status(agent_attn_handle* h, void* stream) {
 // region 256-byte aligned (V_A, dV_A and dA are cleared with one memset, so their regions have one size).
 namespace {
 struct BwdLayout {
-    size_t a, va, dva, da, lse, dot, tab, part, total;
+    size_t a, va, dva, da, lse, dot, tab, part, terms, total;
 };
+// 16-bit inputs outside the mixed-precision kernels: fp32 operands as 16-bit terms on the tensor cores
+bool use_terms(const agent_attn_handle* h, int n) {
+    return auto_like(h) && !backward_mma_eligible(h->cfg.dtype, n, h->cfg.head_dim) && backward_terms_eligible(h->cfg.dtype, n, h->cfg.head_dim);
+}
 bool bwd_layout(const agent_attn_handle* h, int N, int n, BwdPlan* pl, BwdLayout* w) {
     const int slabs = h->cfg.batch * h->cfg.heads;
     if (!plan_backward(slabs, n, N, h->cfg.head_dim, h->sm_count, pl)) return false;
@@ -663,7 +667,8 @@ bool bwd_layout(const agent_attn_handle* h, int N, int n, BwdPlan* pl, BwdLayout
         const size_t mma_floats = backward_mma_part_floats(slabs, plan_backward_mma(slabs, N, h->sm_count));
         if (part_floats < mma_floats) part_floats = mma_floats;
     }
-    w->total = w->part + align_up(part_floats * sizeof(float), 256);
+    w->terms = w->part + align_up(part_floats * sizeof(float), 256);
+    w->total = w->terms + (use_terms(h, n) ? backward_terms_bytes(slabs, n, N, h->cfg.head_dim) : 0);
     return true;
 }
 }  // namespace
@@ -734,9 +739,10 @@ int agent_attn_backward(agent_attn_handle* h, const void* Q, const void* K, cons
     c.dtype = h->cfg.dtype;
     c.use_mma = auto_like(h) && backward_mma_eligible(h->cfg.dtype, n_agents, h->cfg.head_dim);
     if (c.use_mma) c.plan_mma = plan_backward_mma(c.slabs, N, h->sm_count);
+    c.ws_terms = use_terms(h, n_agents) ? ws + w.terms : nullptr;
     cudaError_t e = launch_backward(h->cfg.dtype, c, (cudaStream_t)stream);
     if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "backward launch failed: %s", cudaGetErrorString(e));
-    h->launches = backward_launch_count(c.use_mma != 0);
+    h->launches = backward_launch_count(c);
     return AA_OK;
 }
 

@@ -521,14 +521,18 @@ cudaError_t backward_typed(const BwdCall& c, BwdArgs a, cudaStream_t st) {
 #define AA_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
     AA_TRY(cudaMemsetAsync(c.ws_va, 0, c.clear_bytes, st));               // V_A, dV_A, dA are contiguous
     const size_t bias_elems = (size_t)a.heads * a.n * a.N;
-    if (c.db1) AA_TRY(cudaMemsetAsync(c.db1, 0, bias_elems * sizeof(float), st));
-    if (c.db2) AA_TRY(cudaMemsetAsync(c.db2, 0, bias_elems * sizeof(float), st));
+    const bool clear_bias = !c.ws_terms || a.slabs != a.heads;             // (a single batch entry stores its bias gradients)
+    if (c.db1 && clear_bias) AA_TRY(cudaMemsetAsync(c.db1, 0, bias_elems * sizeof(float), st));
+    if (c.db2 && clear_bias) AA_TRY(cudaMemsetAsync(c.db2, 0, bias_elems * sizeof(float), st));
     if (c.dwd) AA_TRY(cudaMemsetAsync(c.dwd, 0, (size_t)a.heads * a.d * 9 * sizeof(float), st));
 
     bwd_pool_kernel<T><<<(unsigned)((snd + 255) / 256), 256, 0, st>>>(a, c.q, c.ws_a);
     AA_TRY(cudaGetLastError());
     bwd_window_table_kernel<<<(unsigned)((a.N + 255) / 256), 256, 0, st>>>(a, c.ws_tab);
     AA_TRY(cudaGetLastError());
+    if (c.ws_terms) {
+        if constexpr (sizeof(T) == 2) AA_TRY(launch_backward_terms(c.dtype, c, c.ws_terms, st));
+    } else {
     // aggregation forward: row statistics, then V_A
     a.x = c.k; a.y = c.v; a.bias = c.b1; a.m0 = c.ws_a; a.m1 = nullptr; a.scale = c.scale1;
     a.part = c.ws_part; a.dbias = nullptr;
@@ -570,6 +574,7 @@ cudaError_t backward_typed(const BwdCall& c, BwdArgs a, cudaStream_t st) {
     } else {
         AA_TRY((launch_tile<T, kAgg1>(a, st)));
     }
+    }
     // pooling and depthwise terms
     {
         int chunks = (4 * c.sm_count + a.slabs - 1) / a.slabs;          // short loops (they are load-latency bound), few atomics
@@ -610,7 +615,7 @@ bool plan_backward(int slabs, int n, int N, int d, int sm_count, BwdPlan* out) {
     return true;
 }
 
-int backward_launch_count(bool use_mma) { return use_mma ? 8 : 9; }
+int backward_launch_count(const BwdCall& c) { return c.ws_terms ? 11 : c.use_mma ? 8 : 9; }
 
 cudaError_t launch_backward(int dtype, const BwdCall& c, cudaStream_t st) {
     BwdArgs a;

@@ -1,0 +1,684 @@
+// Gradient kernels on register tiles (mma.sync): operands that carry more than 16 bits are sums of 16-bit terms.
+//
+// Inputs (Q, K, V, dO) are NX terms of the MMA type E: one where E is their own type, two where fp16 inputs meet bf16 terms (a
+// bf16 pair holds all 11 bits).  Derived operands (A, V_A, dV_A: TA, TM terms; P, dS: TP terms) are split when they are made; a
+// product keeps the term pairs whose order is below that of the finer operand, so three bf16 terms give fp32 operands.
+//
+// Two orientations, so that no probability is ever transposed:
+//   sums  rows = agents, columns = tokens: everything summed over tokens (V_A, dV_A, dA) and dB1
+//   rows  rows = tokens, columns = agents: everything that a token owns (softmax statistics, dQ, dK, dV) and dB2
+#pragma once
+#include "tile_agg.cuh"
+
+namespace aa {
+
+enum BwdSums { kSumsForward, kSumsBroadcast, kSumsAggregate };
+enum BwdRows { kRowsStats, kRowsQuery, kRowsKeyValue };
+
+// term pairs of a product: i of NA, j of NB with i + j < max(NA, NB)
+template <int NA, int NB> struct TermPairs {
+    static constexpr int kOrder = NA > NB ? NA : NB;
+    __host__ __device__ static constexpr bool keep(int i, int j) { return i + j < kOrder; }
+};
+
+// two fp32 -> NT packed pairs of terms
+template <typename E, int NT> __device__ __forceinline__ void split_pair(float a, float b, uint32_t (&w)[NT]) {
+#pragma unroll
+    for (int i = 0; i < NT; ++i) {
+        w[i] = pack2<E>(a, b);
+        if (i + 1 < NT) {
+            const float2 u = unpack2<E>(w[i]);
+            a -= u.x;
+            b -= u.y;
+        }
+    }
+}
+__device__ __forceinline__ void red_add4(float* p, float a, float b, float c, float d) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};\n" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+__device__ __forceinline__ void red_add2(float* p, float a, float b) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1,%2};\n" ::"l"(p), "f"(a), "f"(b) : "memory");
+}
+// eight consecutive bias gradients of one row: added, or stored where the batch has one entry
+__device__ __forceinline__ void put_dbias8(float* p, const float* v, int cnt, bool aligned, bool store) {
+    if (cnt >= 8 && aligned) {
+        if (store) {
+            *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+            *reinterpret_cast<float4*>(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
+        } else {
+            red_add4(p, v[0], v[1], v[2], v[3]);
+            red_add4(p + 4, v[4], v[5], v[6], v[7]);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i < cnt) {
+                if (store) p[i] = v[i];
+                else atomicAdd(p + i, v[i]);
+            }
+    }
+}
+
+// A operand (16 rows x 16 channels) from a tile in natural row order
+template <int PITCH> __device__ __forceinline__ uint32_t a_lane_offset(int lane) { return (lane & 15) * PITCH + (lane >> 4) * 16; }
+
+// 16 bytes of a token row as NX chunks of terms
+template <typename T, typename E, int NX> __device__ __forceinline__ void split_chunk(const uint4& raw, uint4 (&out)[NX]) {
+    if constexpr (NX == 1) {
+        out[0] = raw;
+    } else {
+        const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+        uint32_t o[NX][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 f = unpack2<T>(w[i]);
+            uint32_t t[NX];
+            split_pair<E, NX>(f.x, f.y, t);
+#pragma unroll
+            for (int k = 0; k < NX; ++k) o[k][i] = t[k];
+        }
+#pragma unroll
+        for (int k = 0; k < NX; ++k) out[k] = make_uint4(o[k][0], o[k][1], o[k][2], o[k][3]);
+    }
+}
+
+struct BwdTermArgs {
+    const void *x, *y, *bias;              // [slabs][N][d] (Q, dO or K, V); B2 [heads][N][n] or B1 [heads][n][N], or null
+    const void *a_t, *m_t;                 // terms [terms][slabs][n][d] of A; of V_A or dV_A
+    float2* tok_stats;                     // [slabs][N]: (log2-sum-exp, row dot) of the broadcast softmax
+    float2* agent_stats;                   // [slabs][n]: (log2-sum-exp, D) of the aggregation softmax
+    float *outer0, *outer1;                // fp32 [slabs][n][d]
+    float *row0, *row1;                    // fp32 [slabs][N][d]
+    float* dbias;
+    void* va_t;                            // forward sums: terms of V_A
+    int slabs, heads, N, n, d;
+    int rg, tokens;                        // sums: row groups; tokens per block (either kernel)
+    float scale;
+};
+
+// ------------------------------------------------------------------------------------------------------------- sums
+template <int DK, int NX, int TA, int TM, int KG, int MODE> struct SumsShape {
+    static constexpr int kPitch = DK * 2 + 16;
+    static constexpr int kTokens = NX == 1 && KG < 2 ? 64 : 32 * KG;
+    static constexpr int kStages = NX == 1 ? 3 : 2;
+    static constexpr int kStats = MODE == kSumsBroadcast ? kTokens * 8 : 0;
+    static constexpr int kStage = 2 * NX * kTokens * kPitch + kStats;
+    static constexpr int kMats = TA + (MODE == kSumsForward ? 0 : TM);
+    static constexpr int kAccPitch = DK + 8;
+    static constexpr int kMerge = 8 * 16 * (kAccPitch + 2) * 4 + 8 * 16 * 8 * KG * 4;        // forward: partial states, over the ring
+    __host__ __device__ static constexpr int smem(int rows) {
+        const int ring = kStages * kStage, part = MODE == kSumsForward ? kMerge : 0;
+        return kMats * rows * kPitch + (ring > part ? ring : part);
+    }
+};
+
+template <typename T, typename E, int DK, int NX, int TA, int TM, int TP, int KG, int MODE>
+__global__ void __launch_bounds__(256, 1) bwd_sums_kernel(const __grid_constant__ BwdTermArgs p) {
+    using S = SumsShape<DK, NX, TA, TM, KG, MODE>;
+    constexpr int PITCH = S::kPitch, KS = DK / 16, NT = DK / 8, TOK = S::kTokens;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const int slab = blockIdx.z, head = slab % p.heads, rows = p.rg * 16, row0 = blockIdx.y * rows;
+    const int t0 = min(p.N, (int)blockIdx.x * p.tokens), t1 = min(p.N, t0 + p.tokens);
+    const int rgi = warp % p.rg, kgi = warp / p.rg;
+    const bool active = kgi < KG;
+    const uint32_t sm = smem_u32(smem), ring = sm + S::kMats * rows * PITCH;
+    // agents' terms
+    {
+        const int chunks = DK / 8;
+        for (int i = threadIdx.x; i < S::kMats * rows * chunks; i += 256) {
+            const int m = i / (rows * chunks), e = i - m * rows * chunks, r = e / chunks, ch = e - r * chunks;
+            const bool ok = row0 + r < p.n && ch * 8 < p.d;
+            const E* src = m < TA ? static_cast<const E*>(p.a_t) + (size_t)m * p.slabs * p.n * p.d
+                                  : static_cast<const E*>(p.m_t) + (size_t)(m - TA) * p.slabs * p.n * p.d;
+            const size_t off = ok ? ((size_t)slab * p.n + row0 + r) * p.d + ch * 8 : 0;
+            cp_async16s(sm + (m * rows + r) * PITCH + ch * 16, src + off, ok ? 16 : 0);
+        }
+        cp_async_commit();
+    }
+    const T* x = static_cast<const T*>(p.x) + (size_t)slab * p.N * p.d;
+    const T* y = static_cast<const T*>(p.y) + (size_t)slab * p.N * p.d;
+    auto load = [&](int tok, int stage) {
+        const uint32_t dst0 = ring + stage * S::kStage;
+        for (int i = threadIdx.x; i < TOK * (DK / 8); i += 256) {
+            const int r = i / (DK / 8), ch = i - r * (DK / 8);
+            const bool ok = tok + r < t1 && ch * 8 < p.d;
+            const size_t off = ok ? (size_t)(tok + r) * p.d + ch * 8 : 0;
+            const uint32_t o = col_to_row(r) * PITCH + ch * 16;
+            if constexpr (NX == 1) {
+                cp_async16s(dst0 + o, x + off, ok ? 16 : 0);
+                cp_async16s(dst0 + TOK * PITCH + o, y + off, ok ? 16 : 0);
+            } else {
+                uint4 a[NX], b[NX], z = make_uint4(0u, 0u, 0u, 0u);
+                split_chunk<T, E, NX>(ok ? __ldg(reinterpret_cast<const uint4*>(x + off)) : z, a);
+                split_chunk<T, E, NX>(ok ? __ldg(reinterpret_cast<const uint4*>(y + off)) : z, b);
+#pragma unroll
+                for (int k = 0; k < NX; ++k) {
+                    *reinterpret_cast<uint4*>(smem + (dst0 - sm) + k * TOK * PITCH + o) = a[k];
+                    *reinterpret_cast<uint4*>(smem + (dst0 - sm) + (NX + k) * TOK * PITCH + o) = b[k];
+                }
+            }
+        }
+        if (MODE == kSumsBroadcast && threadIdx.x < TOK) {
+            float2 s = make_float2(INFINITY, 0.f);                    // no such token: its probabilities are zero
+            if (tok + (int)threadIdx.x < t1) s = p.tok_stats[(size_t)slab * p.N + tok + threadIdx.x];
+            *reinterpret_cast<float2*>(smem + (dst0 - sm) + 2 * NX * TOK * PITCH + threadIdx.x * 8) = s;
+        }
+    };
+    const int tiles = (t1 - t0 + TOK - 1) / TOK;
+#pragma unroll
+    for (int i = 0; i < S::kStages - 1; ++i) {
+        if (i < tiles) load(t0 + i * TOK, i);
+        cp_async_commit();
+    }
+    float o0[NT][4], o1[NT][4];
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o0[j][e] = o1[j][e] = 0.f;
+    const int r0 = row0 + rgi * 16 + g;
+    float2 rs[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    if (MODE == kSumsAggregate)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (r0 + h * 8 < p.n) rs[h] = p.agent_stats[(size_t)slab * p.n + r0 + h * 8];
+    float ref[2] = {-INFINITY, -INFINITY}, sum[2] = {0.f, 0.f};
+    const float c1 = p.scale * kLog2e;
+    // bias element (row r, token c): B1 [n][N] in the aggregation, B2 [N][n] in the broadcast
+    const T* bias = p.bias ? static_cast<const T*>(p.bias) + (size_t)head * p.n * p.N : nullptr;
+    const T* bias_end = p.bias ? static_cast<const T*>(p.bias) + (size_t)p.heads * p.n * p.N : nullptr;
+    const uint32_t aoff = sm + rgi * 16 * PITCH + a_lane_offset<PITCH>(lane);
+    const uint32_t koff = key_lane_offset<DK>(lane) + kgi * 32 * PITCH, voff = val_lane_offset<DK>(lane) + kgi * 32 * PITCH;
+    for (int it = 0; it < tiles; ++it) {
+        if (NX == 1) cp_async_wait<S::kStages - 2>();
+        else cp_async_wait<0>();
+        __syncthreads();
+        if (it + S::kStages - 1 < tiles) load(t0 + (it + S::kStages - 1) * TOK, (it + S::kStages - 1) % S::kStages);
+        cp_async_commit();
+        if (!active) continue;
+        const uint32_t st = ring + (it % S::kStages) * S::kStage;
+#pragma unroll 1
+        for (int sub = 0; sub * 32 * KG < TOK; ++sub) {
+            const int tok = t0 + it * TOK + (sub * KG + kgi) * 32;
+            if (tok >= t1) break;
+            const uint32_t xs = st + sub * KG * 32 * PITCH, ys = xs + NX * TOK * PITCH;
+            float s[4][4], dp[4][4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) s[j][e] = dp[j][e] = 0.f;
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks) {
+                uint32_t a[TA][4], m[TM][4];
+#pragma unroll
+                for (int i = 0; i < TA; ++i) ldsm4(a[i], aoff + i * rows * PITCH + ks * 32);
+                if (MODE != kSumsForward)
+#pragma unroll
+                    for (int i = 0; i < TM; ++i) ldsm4(m[i], aoff + (TA + i) * rows * PITCH + ks * 32);
+#pragma unroll
+                for (int j2 = 0; j2 < 2; ++j2)
+#pragma unroll
+                    for (int k = 0; k < NX; ++k) {
+                        uint32_t b[4];
+                        ldsm4(b, xs + koff + k * TOK * PITCH + j2 * 16 * PITCH + ks * 32);
+#pragma unroll
+                        for (int i = 0; i < TA; ++i)
+                            if (TermPairs<TA, NX>::keep(i, k)) {
+                                mma_acc<E>(s[2 * j2], a[i], b[0], b[1]);
+                                mma_acc<E>(s[2 * j2 + 1], a[i], b[2], b[3]);
+                            }
+                        if (MODE != kSumsForward) {
+                            ldsm4(b, ys + koff + k * TOK * PITCH + j2 * 16 * PITCH + ks * 32);
+#pragma unroll
+                            for (int i = 0; i < TM; ++i)
+                                if (TermPairs<TM, NX>::keep(i, k)) {
+                                    mma_acc<E>(dp[2 * j2], m[i], b[0], b[1]);
+                                    mma_acc<E>(dp[2 * j2 + 1], m[i], b[2], b[3]);
+                                }
+                        }
+                    }
+            }
+            // logits in log2 units, then probabilities and logit gradients
+            const int left = t1 - tok - 8 * t;
+            float bs[2][8];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int r = r0 + h * 8;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) bs[h][i] = 0.f;
+                if (bias && r < p.n) {
+                    if (MODE == kSumsBroadcast) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            if (i < left) bs[h][i] = Elem<T>::to_f32(bias[(size_t)(tok + 8 * t + i) * p.n + r]) * kLog2e;
+                    } else {
+                        const T* bp = bias + (size_t)r * p.N + tok + 8 * t;
+                        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+                        if (left > 0) w = p.N % 8 == 0 ? __ldg(reinterpret_cast<const uint4*>(bp)) : load_bias8_any(bp, bias_end);
+                        unpack16<T>(w, bs[h]);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) bs[h][i] *= kLog2e;
+                    }
+                }
+            }
+            uint32_t pt[TP][2][4], dt[TP][2][4];
+            if constexpr (MODE == kSumsForward) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float mx = -INFINITY;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            float& v = s[j][2 * h + e];
+                            v = 2 * j + e < left ? fmaf(v, c1, bs[h][2 * j + e]) : -INFINITY;
+                            mx = fmaxf(mx, v);
+                        }
+                    mx = quad_max(mx);
+                    const float nr = fmaxf(ref[h], mx), f = ref[h] == -INFINITY ? 0.f : exp2f(ref[h] - nr);
+                    ref[h] = nr;
+                    sum[h] *= f;
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) { o0[j][2 * h] *= f; o0[j][2 * h + 1] *= f; }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float p0 = nr == -INFINITY ? 0.f : fast_exp2(s[j][2 * h] - nr), p1 = nr == -INFINITY ? 0.f : fast_exp2(s[j][2 * h + 1] - nr);
+                        sum[h] += p0 + p1;
+                        uint32_t w[TP];
+                        split_pair<E, TP>(p0, p1, w);
+#pragma unroll
+                        for (int i = 0; i < TP; ++i) pt[i][j >> 1][(j & 1) * 2 + h] = w[i];
+                    }
+                }
+            } else {
+                float2 cs[8];
+                if (MODE == kSumsBroadcast)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float4 v = *reinterpret_cast<const float4*>(smem + (st - sm) + 2 * NX * TOK * PITCH + ((sub * KG + kgi) * 32 + 8 * t + 2 * i) * 8);
+                        cs[2 * i] = make_float2(v.x, v.y);
+                        cs[2 * i + 1] = make_float2(v.z, v.w);
+                    }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float ds[8];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        float pv[2];
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const int i = 2 * j + e;
+                            const float2 q = MODE == kSumsBroadcast ? cs[i] : rs[h];
+                            pv[e] = fast_exp2(fmaf(s[j][2 * h + e], c1, bs[h][i] - q.x));
+                            if (MODE == kSumsAggregate && i >= left) pv[e] = 0.f;
+                            ds[i] = pv[e] * (dp[j][2 * h + e] - q.y);
+                        }
+                        uint32_t w[TP];
+                        if (MODE == kSumsBroadcast) {
+                            split_pair<E, TP>(pv[0], pv[1], w);
+#pragma unroll
+                            for (int i = 0; i < TP; ++i) pt[i][j >> 1][(j & 1) * 2 + h] = w[i];
+                        }
+                        split_pair<E, TP>(ds[2 * j], ds[2 * j + 1], w);
+#pragma unroll
+                        for (int i = 0; i < TP; ++i) dt[i][j >> 1][(j & 1) * 2 + h] = w[i];
+                    }
+                    if (MODE == kSumsAggregate && p.dbias && r0 + h * 8 < p.n)
+                        put_dbias8(p.dbias + ((size_t)head * p.n + r0 + h * 8) * p.N + tok + 8 * t, ds, left, p.N % 4 == 0, p.slabs == p.heads);
+                }
+            }
+#pragma unroll
+            for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+                for (int c2 = 0; c2 < NT / 2; ++c2)
+#pragma unroll
+                    for (int k = 0; k < NX; ++k) {
+                        uint32_t b[4];
+                        if (MODE != kSumsAggregate) {
+                            ldsm4t(b, ys + voff + k * TOK * PITCH + kk * 16 * PITCH + c2 * 32);
+#pragma unroll
+                            for (int i = 0; i < TP; ++i)
+                                if (TermPairs<TP, NX>::keep(i, k)) {
+                                    mma_acc<E>(o0[2 * c2], pt[i][kk], b[0], b[1]);
+                                    mma_acc<E>(o0[2 * c2 + 1], pt[i][kk], b[2], b[3]);
+                                }
+                        }
+                        if (MODE != kSumsForward) {
+                            ldsm4t(b, xs + voff + k * TOK * PITCH + kk * 16 * PITCH + c2 * 32);
+#pragma unroll
+                            for (int i = 0; i < TP; ++i)
+                                if (TermPairs<TP, NX>::keep(i, k)) {
+                                    mma_acc<E>(o1[2 * c2], dt[i][kk], b[0], b[1]);
+                                    mma_acc<E>(o1[2 * c2 + 1], dt[i][kk], b[2], b[3]);
+                                }
+                        }
+                    }
+        }
+    }
+    if constexpr (MODE != kSumsForward) {
+        if (!active) return;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = r0 + h * 8;
+            if (r >= p.n) continue;
+            const size_t off = ((size_t)slab * p.n + r) * p.d + 2 * t;
+#pragma unroll
+            for (int j = 0; j < NT; ++j)
+                if (j * 8 + 2 * t < p.d) {
+                    if (MODE == kSumsBroadcast) red_add2(p.outer0 + off + j * 8, o0[j][2 * h], o0[j][2 * h + 1]);
+                    red_add2(p.outer1 + off + j * 8, o1[j][2 * h] * p.scale, o1[j][2 * h + 1] * p.scale);
+                }
+        }
+    } else {
+        // partial states of the slab's blocks meet in shared memory (as in agg_merge); V_A in fp32 and as terms, and the row statistics
+        cp_async_wait<0>();
+        __syncthreads();
+        const int csize = gridDim.x, crank = blockIdx.x;
+        unsigned char* ms = smem + S::kMats * rows * PITCH;
+        float* acc = reinterpret_cast<float*>(ms) + warp * 16 * S::kAccPitch;
+        float2* ml = reinterpret_cast<float2*>(ms + 8 * 16 * S::kAccPitch * 4);
+        float* wt = reinterpret_cast<float*>(ms + 8 * 16 * (S::kAccPitch + 2) * 4);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float l = quad_sum(sum[h]);
+            if (t == 0) ml[warp * 16 + h * 8 + g] = make_float2(ref[h], active ? l : 0.f);
+#pragma unroll
+            for (int j = 0; j < NT; ++j)
+                *reinterpret_cast<float2*>(acc + (h * 8 + g) * S::kAccPitch + j * 8 + 2 * t) = make_float2(o0[j][2 * h], o0[j][2 * h + 1]);
+        }
+        cluster_sync_all(csize);
+        const int nrows = min(rows, p.n - row0), nsrc = csize * KG, share = (nrows - crank + csize - 1) / csize;
+        const uint32_t acc0 = smem_u32(ms), ml0 = acc0 + 8 * 16 * S::kAccPitch * 4;
+        if ((int)threadIdx.x < share) {
+            const int r = crank + threadIdx.x * csize;
+            float m[8 * KG], l[8 * KG], mm = -INFINITY, tot = 0.f;
+#pragma unroll
+            for (int q = 0; q < 8 * KG; ++q) {
+                m[q] = 0.f; l[q] = 0.f;
+                if (q < nsrc) {
+                    const float2 v = ld_dsmem_f32x2(ml0 + ((q % KG) * rows + r) * 8, q / KG);
+                    m[q] = v.x; l[q] = v.y;
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 8 * KG; ++q)
+                if (l[q] > 0.f) mm = fmaxf(mm, m[q]);
+#pragma unroll
+            for (int q = 0; q < 8 * KG; ++q) {
+                m[q] = l[q] > 0.f ? exp2f(m[q] - mm) : (l[q] == 0.f ? 0.f : l[q]);
+                tot += l[q] * m[q];
+            }
+            const float inv = 1.f / tot;
+#pragma unroll
+            for (int q = 0; q < 8 * KG; ++q)
+                if (q < nsrc) wt[threadIdx.x * nsrc + q] = m[q] * inv;
+            p.agent_stats[(size_t)slab * p.n + row0 + r].x = mm + log2f(tot);
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < share * (DK / 2); i += 256) {
+            const int k = i / (DK / 2), ch = 2 * (i - k * (DK / 2)), r = crank + k * csize;
+            if (ch >= p.d) continue;
+            float2 v = make_float2(0.f, 0.f);
+            for (int b = 0; b < csize; ++b)
+#pragma unroll
+                for (int q = 0; q < KG; ++q) {
+                    const float2 w = ld_dsmem_f32x2(acc0 + ((q * rows + r) * S::kAccPitch + ch) * 4, b);
+                    const float f = wt[k * nsrc + b * KG + q];
+                    v.x = fmaf(w.x, f, v.x);
+                    v.y = fmaf(w.y, f, v.y);
+                }
+            const size_t off = ((size_t)slab * p.n + row0 + r) * p.d + ch;
+            *reinterpret_cast<float2*>(p.outer0 + off) = v;
+            uint32_t w[TM];
+            split_pair<E, TM>(v.x, v.y, w);
+#pragma unroll
+            for (int q = 0; q < TM; ++q)
+                *reinterpret_cast<uint32_t*>(static_cast<E*>(p.va_t) + (size_t)q * p.slabs * p.n * p.d + off) = w[q];
+        }
+        if (csize > 1) cluster_sync_all();
+    }
+}
+
+// ------------------------------------------------------------------------------------------------------------- rows
+template <int DK, int TA, int TM> struct RowsShape {
+    static constexpr int kPitch = DK * 2 + 16;
+    __host__ __device__ static constexpr int smem(int n) { return (TA + TM) * ((n + 31) & ~31) * kPitch + ((n + 31) & ~31) * 8; }
+};
+
+template <typename T, typename E, int DK, int NX, int TA, int TM, int TP, int MODE>
+__global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant__ BwdTermArgs p) {
+    constexpr int PITCH = DK * 2 + 16, KS = DK / 16, NT = DK / 8;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const int slab = blockIdx.y, head = slab % p.heads, n32 = (p.n + 31) & ~31;
+    const int t0 = min(p.N, (int)blockIdx.x * p.tokens), t1 = min(p.N, t0 + p.tokens);
+    const uint32_t sm = smem_u32(smem);
+    float2* st_s = reinterpret_cast<float2*>(smem + (TA + TM) * n32 * PITCH);
+    {
+        const int chunks = DK / 8;
+        for (int i = threadIdx.x; i < (TA + TM) * n32 * chunks; i += 256) {
+            const int m = i / (n32 * chunks), e = i - m * n32 * chunks, r = e / chunks, ch = e - r * chunks;
+            const bool ok = r < p.n && ch * 8 < p.d;
+            const E* src = m < TA ? static_cast<const E*>(p.a_t) + (size_t)m * p.slabs * p.n * p.d
+                                  : static_cast<const E*>(p.m_t) + (size_t)(m - TA) * p.slabs * p.n * p.d;
+            const size_t off = ok ? ((size_t)slab * p.n + r) * p.d + ch * 8 : 0;
+            cp_async16s(sm + (m * n32 + col_to_row(r)) * PITCH + ch * 16, src + off, ok ? 16 : 0);
+        }
+        if (MODE == kRowsKeyValue)
+            for (int i = threadIdx.x; i < n32; i += 256)                  // (no such agent: its probabilities are zero)
+                st_s[i] = i < p.n ? p.agent_stats[(size_t)slab * p.n + i] : make_float2(INFINITY, 0.f);
+        cp_async_commit();
+        cp_async_wait<0>();
+        __syncthreads();
+    }
+    const T* x = static_cast<const T*>(p.x) + (size_t)slab * p.N * p.d;
+    const T* y = static_cast<const T*>(p.y) + (size_t)slab * p.N * p.d;
+    const T* bias = p.bias ? static_cast<const T*>(p.bias) + (size_t)head * p.n * p.N : nullptr;
+    const T* bias_end = p.bias ? static_cast<const T*>(p.bias) + (size_t)p.heads * p.n * p.N : nullptr;
+    const float c1 = p.scale * kLog2e;
+    const uint32_t koff = sm + key_lane_offset<DK>(lane), voff = sm + val_lane_offset<DK>(lane);
+    for (int tok = t0 + warp * 16; tok < t1; tok += 128) {
+        uint32_t xf[NX][KS][4], yf[NX][KS][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const size_t off = (size_t)min(tok + h * 8 + g, t1 - 1) * p.d + 2 * t;
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    uint32_t xw = 0u, yw = 0u;
+                    if (ks * 16 + k * 8 + 2 * t < p.d) {
+                        xw = __ldg(reinterpret_cast<const uint32_t*>(x + off + ks * 16 + k * 8));
+                        yw = __ldg(reinterpret_cast<const uint32_t*>(y + off + ks * 16 + k * 8));
+                    }
+                    if constexpr (NX == 1) {
+                        xf[0][ks][k * 2 + h] = xw;
+                        yf[0][ks][k * 2 + h] = yw;
+                    } else {
+                        uint32_t w[NX];
+                        float2 f = unpack2<T>(xw);
+                        split_pair<E, NX>(f.x, f.y, w);
+#pragma unroll
+                        for (int i = 0; i < NX; ++i) xf[i][ks][k * 2 + h] = w[i];
+                        f = unpack2<T>(yw);
+                        split_pair<E, NX>(f.x, f.y, w);
+#pragma unroll
+                        for (int i = 0; i < NX; ++i) yf[i][ks][k * 2 + h] = w[i];
+                    }
+                }
+        }
+        float o0[NT][4], o1[NT][4];
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o0[j][e] = o1[j][e] = 0.f;
+        float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f}, rd[2] = {0.f, 0.f};
+        float2 rs[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        if (MODE == kRowsQuery)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) rs[h] = p.tok_stats[(size_t)slab * p.N + min(tok + h * 8 + g, t1 - 1)];
+#pragma unroll 1
+        for (int blk = 0; blk < n32; blk += 32) {
+            float bs[2][8];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int tk = tok + h * 8 + g, left = p.n - blk - 8 * t;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) bs[h][i] = 0.f;
+                if (bias && tk < t1) {
+                    if (MODE == kRowsKeyValue) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            if (i < left) bs[h][i] = Elem<T>::to_f32(bias[(size_t)(blk + 8 * t + i) * p.N + tk]) * kLog2e;
+                    } else {
+                        const T* bp = bias + (size_t)tk * p.n + blk + 8 * t;
+                        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+                        if (left > 0) w = p.n % 8 == 0 ? __ldg(reinterpret_cast<const uint4*>(bp)) : load_bias8_any(bp, bias_end);
+                        unpack16<T>(w, bs[h]);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) bs[h][i] *= kLog2e;
+                    }
+                }
+            }
+            float s[4][4], dp[4][4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) s[j][e] = dp[j][e] = 0.f;
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+                for (int j2 = 0; j2 < 2; ++j2) {
+#pragma unroll
+                    for (int i = 0; i < TA; ++i) {
+                        uint32_t b[4];
+                        ldsm4(b, koff + (i * n32 + blk + j2 * 16) * PITCH + ks * 32);
+#pragma unroll
+                        for (int k = 0; k < NX; ++k)
+                            if (TermPairs<TA, NX>::keep(i, k)) {
+                                mma_acc<E>(s[2 * j2], xf[k][ks], b[0], b[1]);
+                                mma_acc<E>(s[2 * j2 + 1], xf[k][ks], b[2], b[3]);
+                            }
+                    }
+#pragma unroll
+                    for (int i = 0; i < TM; ++i) {
+                        uint32_t b[4];
+                        ldsm4(b, koff + ((TA + i) * n32 + blk + j2 * 16) * PITCH + ks * 32);
+#pragma unroll
+                        for (int k = 0; k < NX; ++k)
+                            if (TermPairs<TM, NX>::keep(i, k)) {
+                                mma_acc<E>(dp[2 * j2], yf[k][ks], b[0], b[1]);
+                                mma_acc<E>(dp[2 * j2 + 1], yf[k][ks], b[2], b[3]);
+                            }
+                    }
+                }
+            const int left = p.n - blk - 8 * t;
+            if constexpr (MODE == kRowsStats) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {          // every thread keeps its own reference; the quad meets at the end
+                    float mx = m[h];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        float& v = s[i >> 1][2 * h + (i & 1)];
+                        v = i < left ? fmaf(v, c1, bs[h][i]) : -INFINITY;
+                        mx = fmaxf(mx, v);
+                    }
+                    const float base = mx == -INFINITY ? 0.f : mx, f = exp2f(m[h] - base);
+                    m[h] = mx;
+                    l[h] *= f;
+                    rd[h] *= f;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float e = fast_exp2(s[i >> 1][2 * h + (i & 1)] - base);
+                        l[h] += e;
+                        rd[h] = fmaf(e, dp[i >> 1][2 * h + (i & 1)], rd[h]);
+                    }
+                }
+            } else {
+                uint32_t pt[TP][2][4], dt[TP][2][4];
+                float2 cs[8];
+                if (MODE == kRowsKeyValue)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float4 v = *reinterpret_cast<const float4*>(st_s + blk + 8 * t + 2 * i);
+                        cs[2 * i] = make_float2(v.x, v.y);
+                        cs[2 * i + 1] = make_float2(v.z, v.w);
+                    }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float ds[8];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        float pv[2];
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const int i = 2 * j + e;
+                            const float2 q = MODE == kRowsKeyValue ? cs[i] : rs[h];
+                            pv[e] = fast_exp2(fmaf(s[j][2 * h + e], c1, bs[h][i] - q.x));
+                            if (MODE == kRowsQuery && i >= left) pv[e] = 0.f;
+                            ds[i] = pv[e] * (dp[j][2 * h + e] - q.y);
+                        }
+                        uint32_t w[TP];
+                        if (MODE == kRowsKeyValue) {
+                            split_pair<E, TP>(pv[0], pv[1], w);
+#pragma unroll
+                            for (int i = 0; i < TP; ++i) pt[i][j >> 1][(j & 1) * 2 + h] = w[i];
+                        }
+                        split_pair<E, TP>(ds[2 * j], ds[2 * j + 1], w);
+#pragma unroll
+                        for (int i = 0; i < TP; ++i) dt[i][j >> 1][(j & 1) * 2 + h] = w[i];
+                    }
+                    if (MODE == kRowsQuery && p.dbias && tok + h * 8 + g < t1)
+                        put_dbias8(p.dbias + ((size_t)head * p.N + tok + h * 8 + g) * p.n + blk + 8 * t, ds, left, p.n % 4 == 0, p.slabs == p.heads);
+                }
+#pragma unroll
+                for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+                    for (int c2 = 0; c2 < NT / 2; ++c2) {
+#pragma unroll
+                        for (int i = 0; i < TA; ++i) {
+                            uint32_t b[4];
+                            ldsm4t(b, voff + (i * n32 + blk + kk * 16) * PITCH + c2 * 32);
+#pragma unroll
+                            for (int k = 0; k < TP; ++k)
+                                if (TermPairs<TP, TA>::keep(k, i)) {
+                                    mma_acc<E>(o0[2 * c2], dt[k][kk], b[0], b[1]);
+                                    mma_acc<E>(o0[2 * c2 + 1], dt[k][kk], b[2], b[3]);
+                                }
+                        }
+                        if (MODE == kRowsKeyValue)
+#pragma unroll
+                            for (int i = 0; i < TM; ++i) {
+                                uint32_t b[4];
+                                ldsm4t(b, voff + ((TA + i) * n32 + blk + kk * 16) * PITCH + c2 * 32);
+#pragma unroll
+                                for (int k = 0; k < TP; ++k)
+                                    if (TermPairs<TP, TM>::keep(k, i)) {
+                                        mma_acc<E>(o1[2 * c2], pt[k][kk], b[0], b[1]);
+                                        mma_acc<E>(o1[2 * c2 + 1], pt[k][kk], b[2], b[3]);
+                                    }
+                            }
+                    }
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int tk = tok + h * 8 + g;
+            if constexpr (MODE == kRowsStats) {
+                const float mm = quad_max(m[h]), f = m[h] == -INFINITY ? 0.f : exp2f(m[h] - mm);
+                const float tot = quad_sum(l[h] * f), dot = quad_sum(rd[h] * f);
+                if (t == 0 && tk < t1) p.tok_stats[(size_t)slab * p.N + tk] = make_float2(mm + log2f(tot), dot / tot);
+            } else if (tk < t1) {
+                const size_t off = ((size_t)slab * p.N + tk) * p.d + 2 * t;
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+                    if (j * 8 + 2 * t < p.d) {
+                        *reinterpret_cast<float2*>(p.row0 + off + j * 8) = make_float2(o0[j][2 * h] * p.scale, o0[j][2 * h + 1] * p.scale);
+                        if (MODE == kRowsKeyValue) *reinterpret_cast<float2*>(p.row1 + off + j * 8) = make_float2(o1[j][2 * h], o1[j][2 * h + 1]);
+                    }
+            }
+        }
+    }
+}
+
+}  // namespace aa

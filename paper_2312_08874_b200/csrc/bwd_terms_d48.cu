@@ -1,0 +1,6 @@
+// Term-split gradient kernels for head sizes padded to 48 channels.
+#include "bwd_terms_launch.cuh"
+
+namespace aa {
+AA_BWD_TERMS_DEFINE(48)
+}  // namespace aa

@@ -234,9 +234,14 @@ struct BwdCall {
     int dtype;                                // element type of the inputs (kF32, kBF16, kF16)
     int use_mma;                              // the two gradient stages run on the tensor-core kernels
     BwdPlan plan_mma;                         // their tiling
+    void* ws_terms;                           // term-split kernels (bwd_terms.cu) run the attention stages; null: they do not
 };
+// Gradient stages with fp32 operands split into 16-bit terms (16-bit inputs, any shape whose agents fit in shared memory)
+bool backward_terms_eligible(int dtype, int n, int d);
+size_t backward_terms_bytes(int slabs, int n, int N, int d);
+cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStream_t st);
 bool plan_backward(int slabs, int n, int N, int d, int sm_count, BwdPlan* out);   // false: shape not supported
-int backward_launch_count(bool use_mma);
+int backward_launch_count(const BwdCall& c);
 cudaError_t launch_backward(int dtype, const BwdCall& c, cudaStream_t st);
 // Tensor-core kernels of the two gradient stages (16-bit inputs, n <= 64, d = 64)
 bool backward_mma_eligible(int dtype, int n, int d);
