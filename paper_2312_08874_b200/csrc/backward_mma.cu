@@ -180,7 +180,8 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_mma_kernel(BwdArgs p) {
                     const int col = 8 * j + 2 * t4 + (e & 1);
                     const float pr = fast_exp2(sc[j][e] - sStat[col]);     // exp2(-inf) = 0 for masked entries
                     sc[j][e] = pr;
-                    dp[j][e] = pr * (dp[j][e] - sStat[kNP + col]);
+                    // (a softmax over one token has no gradient; the two roundings of its dot product need not agree)
+                    dp[j][e] = N == 1 ? 0.f : pr * (dp[j][e] - sStat[kNP + col]);
                 }
         }
         // sc = P, dp = dS (fp32).  Bias gradient, then both as 16-bit operands (registers and shared memory).

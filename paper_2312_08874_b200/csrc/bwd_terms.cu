@@ -127,7 +127,7 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
     a.x = c.k; a.y = c.v; a.bias = c.b1; a.scale = c.scale1; a.outer0 = c.ws_va; a.va_t = va_t;
     AA_TRY(sums(kTermForward, true));
     // broadcast stage: token statistics, then dV_A and its share of dA
-    a.x = c.q; a.y = c.d_out; a.bias = c.b2; a.scale = c.scale2; a.m_t = va_t;
+    a.x = c.q; a.y = c.d_out; a.bias = c.b2; a.scale = a.out_scale = c.scale2; a.m_t = va_t;
     AA_TRY(rows(kTermStats));
     a.outer0 = c.ws_dva; a.outer1 = c.ws_da;
     AA_TRY(sums(kTermBroadcast, false));
@@ -135,7 +135,7 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
     AA_TRY(rows(kTermQuery));
     bwd_dot_split_kernel<<<(unsigned)((slabs * n + 7) / 8), 256, 0, st>>>(c.ws_va, c.ws_dva, agent_stats, dva_t, slabs * n, d);
     // aggregation stage
-    a.x = c.k; a.y = c.v; a.bias = c.b1; a.scale = c.scale1; a.m_t = dva_t; a.dbias = c.db1;
+    a.x = c.k; a.y = c.v; a.bias = c.b1; a.scale = c.scale1; a.out_scale = N == 1 ? 0.f : c.scale1; a.m_t = dva_t; a.dbias = c.db1;
     AA_TRY(sums(kTermAggregate, false));
     a.row0 = c.dk; a.row1 = c.dv; a.dbias = nullptr;
     AA_TRY(rows(kTermKeyValue));

@@ -93,7 +93,8 @@ struct BwdTermArgs {
     void* va_t;                            // forward sums: terms of V_A
     int slabs, heads, N, n, d;
     int rg, tokens;                        // sums: row groups; tokens per block (either kernel)
-    float scale;
+    float scale;                           // of the logits
+    float out_scale;                       // of dQ, dK and dA: the same; 0 where the softmax has one column (its logit gradients are exactly zero)
 };
 
 // ------------------------------------------------------------------------------------------------------------- sums
@@ -310,7 +311,7 @@ __global__ void __launch_bounds__(256, 1) bwd_sums_kernel(const __grid_constant_
                             const int i = 2 * j + e;
                             const float2 q = MODE == kSumsBroadcast ? cs[i] : rs[h];
                             pv[e] = fast_exp2(fmaf(s[j][2 * h + e], c1, bs[h][i] - q.x));
-                            if (MODE == kSumsAggregate && i >= left) pv[e] = 0.f;
+                            if (MODE == kSumsAggregate && (i >= left || p.N == 1)) pv[e] = 0.f;      // (a softmax over one token has no gradient)
                             ds[i] = pv[e] * (dp[j][2 * h + e] - q.y);
                         }
                         uint32_t w[TP];
@@ -366,7 +367,7 @@ __global__ void __launch_bounds__(256, 1) bwd_sums_kernel(const __grid_constant_
             for (int j = 0; j < NT; ++j)
                 if (j * 8 + 2 * t < p.d) {
                     if (MODE == kSumsBroadcast) red_add2(p.outer0 + off + j * 8, o0[j][2 * h], o0[j][2 * h + 1]);
-                    red_add2(p.outer1 + off + j * 8, o1[j][2 * h] * p.scale, o1[j][2 * h + 1] * p.scale);
+                    red_add2(p.outer1 + off + j * 8, o1[j][2 * h] * p.out_scale, o1[j][2 * h + 1] * p.out_scale);
                 }
         }
     } else {
@@ -673,7 +674,7 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
 #pragma unroll
                 for (int j = 0; j < NT; ++j)
                     if (j * 8 + 2 * t < p.d) {
-                        *reinterpret_cast<float2*>(p.row0 + off + j * 8) = make_float2(o0[j][2 * h] * p.scale, o0[j][2 * h + 1] * p.scale);
+                        *reinterpret_cast<float2*>(p.row0 + off + j * 8) = make_float2(o0[j][2 * h] * p.out_scale, o0[j][2 * h + 1] * p.out_scale);
                         if (MODE == kRowsKeyValue) *reinterpret_cast<float2*>(p.row1 + off + j * 8) = make_float2(o1[j][2 * h], o1[j][2 * h + 1]);
                     }
             }

@@ -226,7 +226,6 @@ struct BwdCall {
     float *ws_a, *ws_va, *ws_dva, *ws_da;     // [slabs][n][d] each; V_A, dV_A, dA contiguous in this order
     float *ws_lse, *ws_dot;                   // [slabs][n]
     float* ws_part;                           // [slabs][chunks][n][2]
-    int4* ws_tab;                             // [N][3]: pooling windows of each token
     size_t clear_bytes;                       // bytes from ws_va to the end of ws_da
     int slabs, heads, H, W, d, n, p, sm_count;
     float scale1, scale2;
@@ -240,6 +239,8 @@ struct BwdCall {
 bool backward_terms_eligible(int dtype, int n, int d);
 size_t backward_terms_bytes(int slabs, int n, int N, int d);
 cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStream_t st);
+// token-wise tail: dQ += Pooling^T(dA), dV += DWC^T(dO), dWd
+cudaError_t launch_backward_tail(int dtype, const BwdCall& c, cudaStream_t st);
 bool plan_backward(int slabs, int n, int N, int d, int sm_count, BwdPlan* out);   // false: shape not supported
 int backward_launch_count(const BwdCall& c);
 cudaError_t launch_backward(int dtype, const BwdCall& c, cudaStream_t st);

@@ -3,80 +3,9 @@
 // its own (long grids) and by one kernel that runs all three per slab (short grids).
 #pragma once
 #include "tile_bc.cuh"
+#include "tile_pool.cuh"
 
 namespace aa {
-
-// --------------------------------------------------------------------------------------------------------- pooling
-// One warp: mean of the window of agent (ay, ax) -> d elements at `out` (fixed order, fp32).
-template <typename T>
-__device__ __forceinline__ void pool_window(const T* q, long long qst, int H, int W, int p, int agent, int d, T* out) {
-    const int lane = threadIdx.x & 31;
-    const int ay = agent / p, ax = agent - ay * p;
-    const int y0 = (ay * H) / p, y1 = ((ay + 1) * H + p - 1) / p, x0 = (ax * W) / p, x1 = ((ax + 1) * W + p - 1) / p;
-    const int ww = x1 - x0, cnt = (y1 - y0) * ww;
-    // lanes = (token sub-lane, 16-byte chunk): a power of two of chunks, so that shuffles reduce over the sub-lanes
-    const int cpt = d / 8, cp2 = cpt <= 1 ? 1 : cpt <= 2 ? 2 : cpt <= 4 ? 4 : cpt <= 8 ? 8 : 16, tpl = 32 / cp2;
-    const int ch = lane & (cp2 - 1), ts = lane / cp2;
-    float2 acc[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) acc[k] = make_float2(0.f, 0.f);
-    int wy = ts / ww, wx = ts - wy * ww;
-    const T* base = q + ((size_t)y0 * W + x0) * qst + ch * 8;
-    for (int i = ts; i < cnt; i += 8 * tpl) {
-        uint4 raw[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            raw[u] = make_uint4(0u, 0u, 0u, 0u);
-            if (i + u * tpl < cnt && ch < cpt) raw[u] = __ldg(reinterpret_cast<const uint4*>(base + ((size_t)wy * W + wx) * qst));
-            wx += tpl;
-            while (wx >= ww) { wx -= ww; ++wy; }
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            acc[0] = fadd2(acc[0], unpack2<T>(raw[u].x));
-            acc[1] = fadd2(acc[1], unpack2<T>(raw[u].y));
-            acc[2] = fadd2(acc[2], unpack2<T>(raw[u].z));
-            acc[3] = fadd2(acc[3], unpack2<T>(raw[u].w));
-        }
-    }
-    for (int o = cp2; o < 32; o <<= 1)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            acc[k].x += __shfl_xor_sync(0xffffffffu, acc[k].x, o);
-            acc[k].y += __shfl_xor_sync(0xffffffffu, acc[k].y, o);
-        }
-    if (ts == 0 && ch < cpt) {
-        const float inv = 1.f / (float)cnt;
-        const float f[8] = {acc[0].x * inv, acc[0].y * inv, acc[1].x * inv, acc[1].y * inv,
-                            acc[2].x * inv, acc[2].y * inv, acc[3].x * inv, acc[3].y * inv};
-        *reinterpret_cast<uint4*>(out + ch * 8) = pack16<T>(f);
-    }
-}
-
-// One thread: eight channels of one agent, for small windows (independent loads, no shuffles; fixed order, fp32).
-template <typename T>
-__device__ __forceinline__ void pool_chunk(const T* q, long long qst, int H, int W, int p, int agent, T* out) {
-    const int ay = agent / p, ax = agent - ay * p;
-    const int y0 = (ay * H) / p, y1 = ((ay + 1) * H + p - 1) / p, x0 = (ax * W) / p, x1 = ((ax + 1) * W + p - 1) / p;
-    float2 acc[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) acc[k] = make_float2(0.f, 0.f);
-    for (int y = y0; y < y1; ++y) {
-        const T* row = q + (long long)(y * W) * qst;
-#pragma unroll 4
-        for (int x = x0; x < x1; ++x) {
-            const uint4 raw = __ldg(reinterpret_cast<const uint4*>(row + x * qst));
-            acc[0] = fadd2(acc[0], unpack2<T>(raw.x));
-            acc[1] = fadd2(acc[1], unpack2<T>(raw.y));
-            acc[2] = fadd2(acc[2], unpack2<T>(raw.z));
-            acc[3] = fadd2(acc[3], unpack2<T>(raw.w));
-        }
-    }
-    const float inv = 1.f / (float)((y1 - y0) * (x1 - x0));
-    const float f[8] = {acc[0].x * inv, acc[0].y * inv, acc[1].x * inv, acc[1].y * inv,
-                        acc[2].x * inv, acc[2].y * inv, acc[3].x * inv, acc[3].y * inv};
-    *reinterpret_cast<uint4*>(out) = pack16<T>(f);
-}
 
 // --------------------------------------------------------------------------------------------------------- kernels
 template <typename T>
@@ -159,11 +88,13 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) tile_slab_kernel(const __gri
                 const int cpt = p.d >> 3, items = (p.n - crank + csize - 1) / csize * cpt;
                 for (int i = threadIdx.x; i < items; i += NW * 32) {
                     const int agent = crank + i / cpt * csize, ch = i % cpt;
-                    pool_chunk<T>(q + ch * 8, p.lin.st, p.H, p.W, p.pool, agent, a + (size_t)agent * p.d + ch * 8);
+                    pool_chunk<T>(q + ch * 8, p.lin.st, p.H, p.W, p.pool, agent,
+                                  [&](const float (&f)[8]) { *reinterpret_cast<uint4*>(a + (size_t)agent * p.d + ch * 8) = pack16<T>(f); });
                 }
             } else {
                 for (int i = crank + warp * csize; i < p.n; i += csize * (NW))
-                    pool_window<T>(q, p.lin.st, p.H, p.W, p.pool, i, p.d, a + (size_t)i * p.d);
+                    pool_window<T>(q, p.lin.st, p.H, p.W, p.pool, i, p.d,
+                                   [&](int ch, const float (&f)[8]) { *reinterpret_cast<uint4*>(a + (size_t)i * p.d + ch * 8) = pack16<T>(f); });
             }
             cluster_sync_all(csize);
         }
@@ -185,8 +116,9 @@ __global__ void __launch_bounds__(256) tile_pool_kernel(const __grid_constant__ 
     const long long cell = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (cell >= (long long)p.slabs * p.n) return;
     const int slab = (int)(cell / p.n), agent = (int)(cell - (long long)slab * p.n);
+    T* a = static_cast<T*>(const_cast<void*>(p.a)) + (size_t)cell * p.d;
     pool_window<T>(static_cast<const T*>(p.q) + tok_offset(p.lin, slab, p.heads, 0), p.lin.st, p.H, p.W, p.pool, agent, p.d,
-                   static_cast<T*>(const_cast<void*>(p.a)) + (size_t)cell * p.d);
+                   [&](int ch, const float (&f)[8]) { *reinterpret_cast<uint4*>(a + ch * 8) = pack16<T>(f); });
 }
 
 }  // namespace aa

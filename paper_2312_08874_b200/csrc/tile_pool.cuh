@@ -1,0 +1,78 @@
+// Agent tokens by average pooling (text under Eq. 6): means of eight channels handed to the caller.
+#pragma once
+#include "tile.cuh"
+
+namespace aa {
+
+// One warp: mean of the window of agent (ay, ax) -> put(chunk, eight means) for every 8-channel chunk (fixed order, fp32).
+template <typename T, typename F>
+__device__ __forceinline__ void pool_window(const T* q, long long qst, int H, int W, int p, int agent, int d, F&& put) {
+    const int lane = threadIdx.x & 31;
+    const int ay = agent / p, ax = agent - ay * p;
+    const int y0 = (ay * H) / p, y1 = ((ay + 1) * H + p - 1) / p, x0 = (ax * W) / p, x1 = ((ax + 1) * W + p - 1) / p;
+    const int ww = x1 - x0, cnt = (y1 - y0) * ww;
+    // lanes = (token sub-lane, 16-byte chunk): a power of two of chunks, so that shuffles reduce over the sub-lanes
+    const int cpt = d / 8, cp2 = cpt <= 1 ? 1 : cpt <= 2 ? 2 : cpt <= 4 ? 4 : cpt <= 8 ? 8 : 16, tpl = 32 / cp2;
+    const int ch = lane & (cp2 - 1), ts = lane / cp2;
+    float2 acc[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[k] = make_float2(0.f, 0.f);
+    int wy = ts / ww, wx = ts - wy * ww;
+    const T* base = q + ((size_t)y0 * W + x0) * qst + ch * 8;
+    for (int i = ts; i < cnt; i += 8 * tpl) {
+        uint4 raw[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            raw[u] = make_uint4(0u, 0u, 0u, 0u);
+            if (i + u * tpl < cnt && ch < cpt) raw[u] = __ldg(reinterpret_cast<const uint4*>(base + ((size_t)wy * W + wx) * qst));
+            wx += tpl;
+            while (wx >= ww) { wx -= ww; ++wy; }
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            acc[0] = fadd2(acc[0], unpack2<T>(raw[u].x));
+            acc[1] = fadd2(acc[1], unpack2<T>(raw[u].y));
+            acc[2] = fadd2(acc[2], unpack2<T>(raw[u].z));
+            acc[3] = fadd2(acc[3], unpack2<T>(raw[u].w));
+        }
+    }
+    for (int o = cp2; o < 32; o <<= 1)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            acc[k].x += __shfl_xor_sync(0xffffffffu, acc[k].x, o);
+            acc[k].y += __shfl_xor_sync(0xffffffffu, acc[k].y, o);
+        }
+    if (ts == 0 && ch < cpt) {
+        const float inv = 1.f / (float)cnt;
+        const float f[8] = {acc[0].x * inv, acc[0].y * inv, acc[1].x * inv, acc[1].y * inv,
+                            acc[2].x * inv, acc[2].y * inv, acc[3].x * inv, acc[3].y * inv};
+        put(ch, f);
+    }
+}
+
+// One thread: eight channels of one agent, for small windows (independent loads, no shuffles; fixed order, fp32).
+template <typename T, typename F>
+__device__ __forceinline__ void pool_chunk(const T* q, long long qst, int H, int W, int p, int agent, F&& put) {
+    const int ay = agent / p, ax = agent - ay * p;
+    const int y0 = (ay * H) / p, y1 = ((ay + 1) * H + p - 1) / p, x0 = (ax * W) / p, x1 = ((ax + 1) * W + p - 1) / p;
+    float2 acc[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[k] = make_float2(0.f, 0.f);
+    for (int y = y0; y < y1; ++y) {
+        const T* row = q + (long long)(y * W) * qst;
+#pragma unroll 4
+        for (int x = x0; x < x1; ++x) {
+            const uint4 raw = __ldg(reinterpret_cast<const uint4*>(row + x * qst));
+            acc[0] = fadd2(acc[0], unpack2<T>(raw.x));
+            acc[1] = fadd2(acc[1], unpack2<T>(raw.y));
+            acc[2] = fadd2(acc[2], unpack2<T>(raw.z));
+            acc[3] = fadd2(acc[3], unpack2<T>(raw.w));
+        }
+    }
+    const float inv = 1.f / (float)((y1 - y0) * (x1 - x0));
+    const float f[8] = {acc[0].x * inv, acc[0].y * inv, acc[1].x * inv, acc[1].y * inv,
+                        acc[2].x * inv, acc[2].y * inv, acc[3].x * inv, acc[3].y * inv};
+    put(f);
+}
+
+}  // namespace aa
