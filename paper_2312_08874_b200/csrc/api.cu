@@ -645,7 +645,8 @@ int agent_attn_query_status(agent_attn_handle* h, void* stream) {
 }
 
 // Workspace of the backward pass: [A | V_A | dV_A | dA | lse | dot | partial (max, sum) | terms], fp32, each
-// region 256-byte aligned (V_A, dV_A and dA are cleared with one memset, so their regions have one size).
+// region 256-byte aligned (V_A, dV_A and dA are cleared as one, so their regions have one size).  The mixed-precision kernels
+// keep A in 16 bits in its region, the terms of V_A in that of the partials and (log-sum-exp, -) pairs over lse and dot.
 namespace {
 struct BwdLayout {
     size_t a, va, dva, da, lse, dot, part, terms, total;
@@ -663,10 +664,7 @@ bool bwd_layout(const agent_attn_handle* h, int N, int n, BwdPlan* pl, BwdLayout
     w->lse = 4 * snd; w->dot = w->lse + sn;
     w->part = w->dot + sn;
     size_t part_floats = (size_t)slabs * pl->chunks * n * 2;
-    if (backward_mma_eligible(h->cfg.dtype, n, h->cfg.head_dim)) {      // partials of the tensor-core stage 1
-        const size_t mma_floats = backward_mma_part_floats(slabs, plan_backward_mma(slabs, N, h->sm_count));
-        if (part_floats < mma_floats) part_floats = mma_floats;
-    }
+    if (part_floats * sizeof(float) < snd) part_floats = snd / sizeof(float);       // (mixed precision: two 16-bit terms of V_A)
     w->terms = w->part + align_up(part_floats * sizeof(float), 256);
     w->total = w->terms + (use_terms(h, n) ? backward_terms_bytes(slabs, n, N, h->cfg.head_dim) : 0);
     return true;
@@ -731,7 +729,7 @@ int agent_attn_backward(agent_attn_handle* h, const void* Q, const void* K, cons
     c.ws_dva = reinterpret_cast<float*>(ws + w.dva); c.ws_da = reinterpret_cast<float*>(ws + w.da);
     c.ws_lse = reinterpret_cast<float*>(ws + w.lse); c.ws_dot = reinterpret_cast<float*>(ws + w.dot);
     c.ws_part = reinterpret_cast<float*>(ws + w.part);
-    c.clear_bytes = w.lse - w.va;
+    c.region_bytes = w.va;
     c.slabs = h->cfg.batch * h->cfg.heads; c.heads = h->cfg.heads; c.H = grid_h; c.W = grid_w;
     c.d = h->cfg.head_dim; c.n = n_agents; c.p = p; c.sm_count = h->sm_count;
     c.scale1 = h->scale1; c.scale2 = h->scale2;

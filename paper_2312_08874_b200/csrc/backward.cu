@@ -389,60 +389,51 @@ cudaError_t backward_typed(const BwdCall& c, BwdArgs a, cudaStream_t st) {
     const size_t sn = (size_t)a.slabs * a.n, snd = sn * a.d;
     cudaError_t e;
 #define AA_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
-    AA_TRY(cudaMemsetAsync(c.ws_va, 0, c.clear_bytes, st));               // V_A, dV_A, dA are contiguous
+    if (c.ws_terms) {
+        if constexpr (sizeof(T) == 2) AA_TRY(launch_backward_terms(c.dtype, c, c.ws_terms, st));
+        return launch_backward_tail(c.dtype, c, st);
+    }
+    if (c.use_mma) {
+        AA_TRY(launch_backward_mixed_forward(c.dtype, c, st));
+        BwdArgs m = a;
+        m.np = c.plan_mma.np; m.tile = c.plan_mma.tile; m.tiles = c.plan_mma.tiles;
+        m.chunks = c.plan_mma.chunks; m.tiles_per_chunk = c.plan_mma.tiles_per_chunk;
+        m.a_t = c.ws_a; m.va_t = c.ws_part; m.stats = reinterpret_cast<const float2*>(c.ws_lse);
+        m.x = c.q; m.y = c.d_out; m.bias = c.b2; m.scale = c.scale2;
+        m.outer0 = c.ws_dva; m.outer1 = c.ws_da; m.row0 = c.dq; m.dbias = c.db2;
+        AA_TRY(launch_backward_mma(c.dtype, true, m, st));
+        m.x = c.k; m.y = c.v; m.bias = c.b1; m.m0 = c.ws_va; m.m1 = c.ws_dva; m.scale = c.scale1;
+        m.row0 = c.dk; m.row1 = c.dv; m.dbias = c.db1;
+        AA_TRY(launch_backward_mma(c.dtype, false, m, st));
+        return launch_backward_tail(c.dtype, c, st);
+    }
+    AA_TRY(cudaMemsetAsync(c.ws_va, 0, 3 * c.region_bytes, st));          // V_A, dV_A, dA are contiguous
     const size_t bias_elems = (size_t)a.heads * a.n * a.N;
-    const bool clear_bias = !c.ws_terms || a.slabs != a.heads;             // (a single batch entry stores its bias gradients)
-    if (c.db1 && clear_bias) AA_TRY(cudaMemsetAsync(c.db1, 0, bias_elems * sizeof(float), st));
-    if (c.db2 && clear_bias) AA_TRY(cudaMemsetAsync(c.db2, 0, bias_elems * sizeof(float), st));
+    if (c.db1) AA_TRY(cudaMemsetAsync(c.db1, 0, bias_elems * sizeof(float), st));
+    if (c.db2) AA_TRY(cudaMemsetAsync(c.db2, 0, bias_elems * sizeof(float), st));
     if (c.dwd) AA_TRY(cudaMemsetAsync(c.dwd, 0, (size_t)a.heads * a.d * 9 * sizeof(float), st));
 
     bwd_pool_kernel<T><<<(unsigned)((snd + 255) / 256), 256, 0, st>>>(a, c.q, c.ws_a);
     AA_TRY(cudaGetLastError());
-    if (c.ws_terms) {
-        if constexpr (sizeof(T) == 2) AA_TRY(launch_backward_terms(c.dtype, c, c.ws_terms, st));
-    } else {
     // aggregation forward: row statistics, then V_A
     a.x = c.k; a.y = c.v; a.bias = c.b1; a.m0 = c.ws_a; a.m1 = nullptr; a.scale = c.scale1;
     a.part = c.ws_part; a.dbias = nullptr;
-    if (c.use_mma) {
-        BwdArgs m = a;
-        m.np = c.plan_mma.np; m.tile = c.plan_mma.tile; m.tiles = c.plan_mma.tiles;
-        m.chunks = c.plan_mma.chunks; m.tiles_per_chunk = c.plan_mma.tiles_per_chunk;
-        AA_TRY(launch_backward_fwd1_mma(c.dtype, m, c.ws_va, c.ws_lse, st));
-        a.lse = c.ws_lse;
-    } else {
-        AA_TRY((launch_tile<T, kStats1>(a, st)));
-        bwd_lse_kernel<<<(unsigned)((sn + 255) / 256), 256, 0, st>>>(a, c.ws_lse);
-        AA_TRY(cudaGetLastError());
-        a.lse = c.ws_lse; a.outer0 = c.ws_va;
-        AA_TRY((launch_tile<T, kVa1>(a, st)));
-    }
+    AA_TRY((launch_tile<T, kStats1>(a, st)));
+    bwd_lse_kernel<<<(unsigned)((sn + 255) / 256), 256, 0, st>>>(a, c.ws_lse);
+    AA_TRY(cudaGetLastError());
+    a.lse = c.ws_lse; a.outer0 = c.ws_va;
+    AA_TRY((launch_tile<T, kVa1>(a, st)));
     // broadcast backward
     a.x = c.q; a.y = c.d_out; a.bias = c.b2; a.m0 = c.ws_a; a.m1 = c.ws_va; a.scale = c.scale2;
     a.outer0 = c.ws_dva; a.outer1 = c.ws_da; a.row0 = c.dq; a.row1 = nullptr; a.dbias = c.db2;
-    if (c.use_mma) {
-        BwdArgs m = a;
-        m.np = c.plan_mma.np; m.tile = c.plan_mma.tile; m.tiles = c.plan_mma.tiles;
-        m.chunks = c.plan_mma.chunks; m.tiles_per_chunk = c.plan_mma.tiles_per_chunk;
-        AA_TRY(launch_backward_mma(c.dtype, true, m, st));
-    } else {
-        AA_TRY((launch_tile<T, kBcast2>(a, st)));
-    }
+    AA_TRY((launch_tile<T, kBcast2>(a, st)));
     bwd_dot_kernel<<<(unsigned)((sn + 7) / 8), 256, 0, st>>>(a, c.ws_va, c.ws_dva, c.ws_dot);
     AA_TRY(cudaGetLastError());
     // aggregation backward
     a.x = c.k; a.y = c.v; a.bias = c.b1; a.m0 = c.ws_a; a.m1 = c.ws_dva; a.scale = c.scale1;
     a.lse = c.ws_lse; a.dot = c.ws_dot;
     a.outer0 = nullptr; a.outer1 = c.ws_da; a.row0 = c.dk; a.row1 = c.dv; a.dbias = c.db1;
-    if (c.use_mma) {
-        BwdArgs m = a;
-        m.np = c.plan_mma.np; m.tile = c.plan_mma.tile; m.tiles = c.plan_mma.tiles;
-        m.chunks = c.plan_mma.chunks; m.tiles_per_chunk = c.plan_mma.tiles_per_chunk;
-        AA_TRY(launch_backward_mma(c.dtype, false, m, st));
-    } else {
-        AA_TRY((launch_tile<T, kAgg1>(a, st)));
-    }
-    }
+    AA_TRY((launch_tile<T, kAgg1>(a, st)));
     AA_TRY(launch_backward_tail(c.dtype, c, st));          // pooling and depthwise terms
 #undef AA_TRY
     return cudaSuccess;
@@ -476,7 +467,7 @@ bool plan_backward(int slabs, int n, int N, int d, int sm_count, BwdPlan* out) {
     return true;
 }
 
-int backward_launch_count(const BwdCall& c) { return (c.ws_terms ? 9 : c.use_mma ? 6 : 7) + 1 + (c.dwd ? 1 : 0); }
+int backward_launch_count(const BwdCall& c) { return (c.ws_terms ? 8 : c.use_mma ? 4 : 7) + 1 + (c.dwd ? 1 : 0); }
 
 cudaError_t launch_backward(int dtype, const BwdCall& c, cudaStream_t st) {
     BwdArgs a;

@@ -66,6 +66,8 @@ __global__ void __launch_bounds__(256, DWC ? 3 : 4) bwd_tail_kernel(const TailAr
     const int t0 = blockIdx.x * tokens, t1 = min(N, t0 + tokens);
     const int groups = d >> 2, cols = 256 / groups;               // d <= 128: at least eight tokens at once
     const int cg = threadIdx.x % groups, cl = threadIdx.x / groups;
+    pdl_wait_prior();
+    pdl_release_next();
     const int ylo = t0 / W, rows = (t1 - 1) / W - ylo + 1;
     for (int i = threadIdx.x; i < min(rows, kAxis); i += 256) yw[i] = windows_of(ylo + i, H, p);
     for (int i = threadIdx.x; i < min(W, kAxis); i += 256) xw[i] = windows_of(i, W, p);
@@ -175,6 +177,7 @@ __global__ void __launch_bounds__(256, 2) bwd_filter_kernel(const TailArgs a) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) red[threadIdx.x][k][q] = acc[k][q];
     __syncthreads();
+    pdl_wait_prior();                                             // (before that: inputs only)
     for (int o = threadIdx.x; o < d * 9; o += 256) {              // o = channel * 9 + tap
         const int c = o / 9, k = o - c * 9;
         float s = 0.f;
@@ -195,15 +198,12 @@ template <typename T> cudaError_t launch_tail(TailArgs a, int slabs, int sm_coun
     const int parts = (int)((N + tokens - 1) / tokens);
     tokens = (N + parts - 1) / parts;
     const dim3 grid(parts, slabs);
-    if (a.wd) bwd_tail_kernel<T, true><<<grid, 256, 0, st>>>(a, (int)tokens);
-    else bwd_tail_kernel<T, false><<<grid, 256, 0, st>>>(a, (int)tokens);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_dependent(a.wd ? bwd_tail_kernel<T, true> : bwd_tail_kernel<T, false>, grid, 256, 0, st, a, (int)tokens);
     if (e != cudaSuccess || !a.dwd) return e;
     // strips: two blocks per SM are resident, at least six rows each (a strip reads two more)
     const int strip = (int)(((long long)a.H * slabs + 2LL * sm_count - 1) / (2LL * sm_count));
     a.strip = ((strip < 6 ? 6 : strip) + 2) / 3 * 3;
-    bwd_filter_kernel<T><<<dim3((a.H + a.strip - 1) / a.strip, slabs), 256, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(bwd_filter_kernel<T>, dim3((a.H + a.strip - 1) / a.strip, slabs), 256, 0, st, a);
 }
 
 }  // namespace

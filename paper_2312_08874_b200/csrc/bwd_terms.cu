@@ -1,6 +1,7 @@
 // Gradients of the attention stages with fp32 operands on the tensor cores: launch plans and the small kernels between the
 // stages (term splits, D = dV_A . V_A).
 #include "bwd_terms_launch.cuh"
+#include "tile_pool.cuh"
 
 #include <algorithm>
 #include <cstring>
@@ -22,31 +23,72 @@ cudaError_t stage(int dtype, int d, int st, const BwdTermArgs& a, const BwdTermL
     }
 }
 
-// fp32 pairs -> three bf16 terms
-__global__ void __launch_bounds__(256) bwd_split_kernel(const float2* src, __nv_bfloat16* dst, size_t pairs) {
-    const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
-    if (i >= pairs) return;
-    const float2 v = src[i];
-    uint32_t w[kTerms];
-    split_pair<__nv_bfloat16, kTerms>(v.x, v.y, w);
+// Buffers that later kernels add to, cleared by extra blocks of the first kernel.
+struct ClearList {
+    float* p[4];
+    size_t words[4];
+    int pool_blocks;
+};
+constexpr int kClearWords = 256 * 32;              // words that a block clears
+
+// Pooled agents as NT terms of E: a warp per window, or (windows of at most 32 tokens on average) a thread per 8 channels.
+template <typename T, typename E, int NT>
+__global__ void __launch_bounds__(256) bwd_pool_terms_kernel(const T* q, E* dst, int slabs, int n, int H, int W, int pool, int d, bool small, ClearList cl) {
+    pdl_release_next();
+    if ((int)blockIdx.x >= cl.pool_blocks) {
+        size_t b = (size_t)(blockIdx.x - cl.pool_blocks) * kClearWords;
 #pragma unroll
-    for (int k = 0; k < kTerms; ++k) reinterpret_cast<uint32_t*>(dst)[k * pairs + i] = w[k];
+        for (int k = 0; k < 4; ++k) {
+            const size_t room = (cl.words[k] + kClearWords - 1) / kClearWords * kClearWords;
+            if (b < room) {
+                const size_t e = min(b + kClearWords, cl.words[k]), e4 = b + ((e - b) & ~(size_t)3);
+                for (size_t i = b + 4 * threadIdx.x; i < e4; i += 1024) *reinterpret_cast<float4*>(cl.p[k] + i) = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (threadIdx.x < e - e4) cl.p[k][e4 + threadIdx.x] = 0.f;
+                return;
+            }
+            b -= room;
+        }
+        return;
+    }
+    const size_t plane = (size_t)slabs * n * d;
+    auto put = [&](size_t off, const float (&f)[8]) {
+        uint32_t w[4][NT];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) split_pair<E, NT>(f[2 * i], f[2 * i + 1], w[i]);
+#pragma unroll
+        for (int k = 0; k < NT; ++k) *reinterpret_cast<uint4*>(dst + k * plane + off) = make_uint4(w[0][k], w[1][k], w[2][k], w[3][k]);
+    };
+    if (small) {
+        const int cpt = d >> 3;
+        const long long i = (long long)blockIdx.x * 256 + threadIdx.x, cell = i / cpt;
+        if (cell >= (long long)slabs * n) return;
+        const int slab = (int)(cell / n), agent = (int)(cell - (long long)slab * n), ch = (int)(i - cell * cpt);
+        pool_chunk<T>(q + (size_t)slab * H * W * d + ch * 8, d, H, W, pool, agent, [&](const float (&f)[8]) { put((size_t)cell * d + ch * 8, f); });
+    } else {
+        const long long cell = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+        if (cell >= (long long)slabs * n) return;
+        const int slab = (int)(cell / n), agent = (int)(cell - (long long)slab * n);
+        pool_window<T>(q + (size_t)slab * H * W * d, d, H, W, pool, agent, d, [&](int ch, const float (&f)[8]) { put((size_t)cell * d + ch * 8, f); });
+    }
 }
 
-// one warp per agent row: D = dV_A . V_A, and the terms of dV_A
-__global__ void __launch_bounds__(256) bwd_dot_split_kernel(const float* va, const float* dva, float2* stats, __nv_bfloat16* dst, int rows, int d) {
+// One warp per agent row: D = dV_A . V_A, and the terms of dV_A.
+template <typename E, int NT>
+__global__ void __launch_bounds__(256) bwd_dot_split_kernel(const float* va, const float* dva, float2* stats, E* dst, int rows, int d) {
     const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    pdl_wait_prior();
+    pdl_release_next();
     if (r >= rows) return;
-    const size_t pairs = (size_t)rows * d / 2;
+    const size_t plane = (size_t)rows * d;
     float acc = 0.f;
     for (int c = 2 * lane; c < d; c += 64) {
         const size_t off = (size_t)r * d + c;
         const float2 a = *reinterpret_cast<const float2*>(va + off), b = *reinterpret_cast<const float2*>(dva + off);
         acc = fmaf(a.x, b.x, fmaf(a.y, b.y, acc));
-        uint32_t w[kTerms];
-        split_pair<__nv_bfloat16, kTerms>(b.x, b.y, w);
+        uint32_t w[NT];
+        split_pair<E, NT>(b.x, b.y, w);
 #pragma unroll
-        for (int k = 0; k < kTerms; ++k) reinterpret_cast<uint32_t*>(dst)[k * pairs + off / 2] = w[k];
+        for (int k = 0; k < NT; ++k) *reinterpret_cast<uint32_t*>(dst + k * plane + off) = w[k];
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -64,17 +106,36 @@ SumsPlan sums_plan(int n, int d) {
     s.kg = s.rg <= 2 && dk <= 80 ? 4 : s.rg <= 4 ? 2 : 1;
     return s;
 }
-// Parts of the token axis: one block per SM is resident, a block's start (agents' terms into shared memory) costs about 256 tokens.
-int token_parts(long long others, int N, int unit, int most, bool pow2, int sm_count) {
+// Parts of the token axis for `slots` resident blocks; a block's start (agents' terms into shared memory) costs about 256 tokens.
+int token_parts(long long others, int N, int unit, int most, bool pow2, int slots) {
     int best = 1;
     double cost = 0;
     for (int c = 1; c <= most; c = pow2 ? 2 * c : c + 1) {
         const int tokens = ((N + c - 1) / c + unit - 1) / unit * unit;
         if (c > 1 && (tokens < 2 * unit || (long long)tokens * (c - 1) >= N)) continue;
-        const double k = (double)((others * c + sm_count - 1) / sm_count) * (tokens + 256);
+        const double k = (double)((others * c + slots - 1) / slots) * (tokens + 256);
         if (c == 1 || k < cost) { best = c; cost = k; }
     }
     return best;
+}
+
+size_t up256(size_t x) { return (x + 255) / 256 * 256; }
+
+// Pooling, and the clearing of the sums that the stages add to.
+template <typename T, typename E, int NT> cudaError_t pool_and_clear(const BwdCall& c, void* a_t, bool clear_bias, cudaStream_t st) {
+    const int N = c.H * c.W;
+    const bool small = N <= 32 * c.n;
+    ClearList cl = {};
+    cl.pool_blocks = (int)(small ? ((long long)c.slabs * c.n * (c.d / 8) + 255) / 256 : ((long long)c.slabs * c.n + 7) / 8);
+    const size_t bias = clear_bias ? (size_t)c.heads * c.n * N : 0;
+    cl.p[0] = c.ws_dva; cl.words[0] = 2 * c.region_bytes / sizeof(float);          // dV_A, dA
+    cl.p[1] = c.db1; cl.words[1] = c.db1 ? bias : 0;
+    cl.p[2] = c.db2; cl.words[2] = c.db2 ? bias : 0;
+    cl.p[3] = c.dwd; cl.words[3] = c.dwd ? (size_t)c.heads * c.d * 9 : 0;
+    size_t clear = 0;
+    for (size_t w : cl.words) clear += (w + kClearWords - 1) / kClearWords;
+    bwd_pool_terms_kernel<T, E, NT><<<(unsigned)(cl.pool_blocks + clear), 256, 0, st>>>(static_cast<const T*>(c.q), static_cast<E*>(a_t), c.slabs, c.n, c.H, c.W, c.p, c.d, small, cl);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -82,22 +143,43 @@ int token_parts(long long others, int N, int unit, int most, bool pow2, int sm_c
 bool backward_terms_eligible(int dtype, int n, int d) {
     if (dtype != kBF16 && dtype != kF16) return false;
     const int dk = dk_of_terms(d), pitch = dk * 2 + 16, n32 = (n + 31) & ~31;
-    return 2 * kTerms * n32 * pitch + n32 * 8 <= 227 * 1024;
+    return 6 * n32 * pitch + n32 * 8 <= 227 * 1024;
 }
 size_t backward_terms_bytes(int slabs, int n, int N, int d) {
-    const size_t terms = ((size_t)slabs * n * d * 2 * kTerms + 255) / 256 * 256;
-    return 3 * terms + ((size_t)slabs * N * 8 + 255) / 256 * 256 + ((size_t)slabs * n * 8 + 255) / 256 * 256;
+    return 3 * up256((size_t)slabs * n * d * 2 * 3) + up256((size_t)slabs * N * 8) + up256((size_t)slabs * n * 8);
+}
+
+cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStream_t st) {
+    cudaError_t e = dtype == kBF16 ? pool_and_clear<__nv_bfloat16, __nv_bfloat16, 1>(c, c.ws_a, true, st) : pool_and_clear<__half, __half, 1>(c, c.ws_a, true, st);
+    if (e != cudaSuccess) return e;
+    BwdTermArgs a;
+    memset(&a, 0, sizeof(a));
+    a.slabs = c.slabs; a.heads = c.heads; a.N = c.H * c.W; a.n = c.n; a.d = c.d;
+    a.x = c.k; a.y = c.v; a.bias = c.b1; a.scale = c.scale1;
+    a.a_t = c.ws_a; a.outer0 = c.ws_va; a.va_t = c.ws_part; a.agent_stats = reinterpret_cast<float2*>(c.ws_lse);
+    a.rg = (c.n + 15) / 16;                            // four warps, three blocks on an SM
+    BwdTermLaunch l;
+    l.stream = st;
+    l.kg = a.rg == 1 ? 4 : a.rg == 2 ? 2 : 1;
+    const int parts = token_parts(c.slabs, a.N, 64, 8, true, 3 * c.sm_count);
+    a.tokens = ((a.N + parts - 1) / parts + 63) / 64 * 64;
+    l.grid = dim3(parts, 1, c.slabs);
+    l.cluster = parts;
+    return bwd_terms_mixed(dtype, a, l);
 }
 
 cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStream_t st) {
     const int N = c.H * c.W, n = c.n, d = c.d, slabs = c.slabs;
     char* w = static_cast<char*>(ws);
-    const size_t terms = ((size_t)slabs * n * d * 2 * kTerms + 255) / 256 * 256;
-    __nv_bfloat16 *a_t = reinterpret_cast<__nv_bfloat16*>(w), *va_t = reinterpret_cast<__nv_bfloat16*>(w + terms), *dva_t = reinterpret_cast<__nv_bfloat16*>(w + 2 * terms);
+    const size_t terms = up256((size_t)slabs * n * d * 2 * 3);
+    void *a_t = w, *va_t = w + terms, *dva_t = w + 2 * terms;
     float2* tok_stats = reinterpret_cast<float2*>(w + 3 * terms);
-    float2* agent_stats = reinterpret_cast<float2*>(w + 3 * terms + ((size_t)slabs * N * 8 + 255) / 256 * 256);
-    const size_t pairs = (size_t)slabs * n * d / 2;
-    bwd_split_kernel<<<(unsigned)((pairs + 255) / 256), 256, 0, st>>>(reinterpret_cast<const float2*>(c.ws_a), a_t, pairs);
+    float2* agent_stats = reinterpret_cast<float2*>(w + 3 * terms + up256((size_t)slabs * N * 8));
+    using B = __nv_bfloat16;
+    cudaError_t e;
+#define AA_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
+    const bool clear_bias = slabs != c.heads;          // (a single batch entry stores its bias gradients)
+    AA_TRY(dtype == kBF16 ? (pool_and_clear<B, B, 3>(c, a_t, clear_bias, st)) : (pool_and_clear<__half, B, 3>(c, a_t, clear_bias, st)));
 
     BwdTermArgs a;
     memset(&a, 0, sizeof(a));
@@ -121,8 +203,6 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
         l.cluster = 0;
         return stage(dtype, d, which, a, l);
     };
-    cudaError_t e;
-#define AA_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
     // V_A and the statistics of the aggregation softmax
     a.x = c.k; a.y = c.v; a.bias = c.b1; a.scale = c.scale1; a.outer0 = c.ws_va; a.va_t = va_t;
     AA_TRY(sums(kTermForward, true));
@@ -133,14 +213,14 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
     AA_TRY(sums(kTermBroadcast, false));
     a.row0 = c.dq; a.dbias = c.db2;
     AA_TRY(rows(kTermQuery));
-    bwd_dot_split_kernel<<<(unsigned)((slabs * n + 7) / 8), 256, 0, st>>>(c.ws_va, c.ws_dva, agent_stats, dva_t, slabs * n, d);
+    AA_TRY((launch_dependent(bwd_dot_split_kernel<B, 3>, dim3((slabs * n + 7) / 8), 256, 0, st, (const float*)c.ws_va, (const float*)c.ws_dva, agent_stats, static_cast<B*>(dva_t), slabs * n, d)));
     // aggregation stage
     a.x = c.k; a.y = c.v; a.bias = c.b1; a.scale = c.scale1; a.out_scale = N == 1 ? 0.f : c.scale1; a.m_t = dva_t; a.dbias = c.db1;
     AA_TRY(sums(kTermAggregate, false));
     a.row0 = c.dk; a.row1 = c.dv; a.dbias = nullptr;
     AA_TRY(rows(kTermKeyValue));
 #undef AA_TRY
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 }  // namespace aa

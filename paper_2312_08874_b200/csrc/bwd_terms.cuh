@@ -36,9 +36,6 @@ template <typename E, int NT> __device__ __forceinline__ void split_pair(float a
 __device__ __forceinline__ void red_add4(float* p, float a, float b, float c, float d) {
     asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};\n" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
-__device__ __forceinline__ void red_add2(float* p, float a, float b) {
-    asm volatile("red.global.add.v2.f32 [%0], {%1,%2};\n" ::"l"(p), "f"(a), "f"(b) : "memory");
-}
 // eight consecutive bias gradients of one row: added, or stored where the batch has one entry
 __device__ __forceinline__ void put_dbias8(float* p, const float* v, int cnt, bool aligned, bool store) {
     if (cnt >= 8 && aligned) {
@@ -98,24 +95,24 @@ struct BwdTermArgs {
 };
 
 // ------------------------------------------------------------------------------------------------------------- sums
-template <int DK, int NX, int TA, int TM, int KG, int MODE> struct SumsShape {
+template <int DK, int NX, int TA, int TM, int KG, int NW, int MODE> struct SumsShape {
     static constexpr int kPitch = DK * 2 + 16;
     static constexpr int kTokens = NX == 1 && KG < 2 ? 64 : 32 * KG;
-    static constexpr int kStages = NX == 1 ? 3 : 2;
+    static constexpr int kStages = NX == 1 && NW == 8 ? 3 : 2;
     static constexpr int kStats = MODE == kSumsBroadcast ? kTokens * 8 : 0;
     static constexpr int kStage = 2 * NX * kTokens * kPitch + kStats;
     static constexpr int kMats = TA + (MODE == kSumsForward ? 0 : TM);
     static constexpr int kAccPitch = DK + 8;
-    static constexpr int kMerge = 8 * 16 * (kAccPitch + 2) * 4 + 8 * 16 * 8 * KG * 4;        // forward: partial states, over the ring
+    static constexpr int kMerge = NW * 16 * (kAccPitch + 2) * 4 + NW * 16 * 8 * KG * 4;        // forward: partial states, over the ring
     __host__ __device__ static constexpr int smem(int rows) {
         const int ring = kStages * kStage, part = MODE == kSumsForward ? kMerge : 0;
         return kMats * rows * kPitch + (ring > part ? ring : part);
     }
 };
 
-template <typename T, typename E, int DK, int NX, int TA, int TM, int TP, int KG, int MODE>
-__global__ void __launch_bounds__(256, 1) bwd_sums_kernel(const __grid_constant__ BwdTermArgs p) {
-    using S = SumsShape<DK, NX, TA, TM, KG, MODE>;
+template <typename T, typename E, int DK, int NX, int TA, int TM, int TP, int KG, int NW, int MODE>
+__global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(const __grid_constant__ BwdTermArgs p) {
+    using S = SumsShape<DK, NX, TA, TM, KG, NW, MODE>;
     constexpr int PITCH = S::kPitch, KS = DK / 16, NT = DK / 8, TOK = S::kTokens;
     extern __shared__ __align__(128) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
@@ -124,10 +121,12 @@ __global__ void __launch_bounds__(256, 1) bwd_sums_kernel(const __grid_constant_
     const int rgi = warp % p.rg, kgi = warp / p.rg;
     const bool active = kgi < KG;
     const uint32_t sm = smem_u32(smem), ring = sm + S::kMats * rows * PITCH;
+    pdl_wait_prior();
+    pdl_release_next();
     // agents' terms
     {
         const int chunks = DK / 8;
-        for (int i = threadIdx.x; i < S::kMats * rows * chunks; i += 256) {
+        for (int i = threadIdx.x; i < S::kMats * rows * chunks; i += NW * 32) {
             const int m = i / (rows * chunks), e = i - m * rows * chunks, r = e / chunks, ch = e - r * chunks;
             const bool ok = row0 + r < p.n && ch * 8 < p.d;
             const E* src = m < TA ? static_cast<const E*>(p.a_t) + (size_t)m * p.slabs * p.n * p.d
@@ -141,7 +140,7 @@ __global__ void __launch_bounds__(256, 1) bwd_sums_kernel(const __grid_constant_
     const T* y = static_cast<const T*>(p.y) + (size_t)slab * p.N * p.d;
     auto load = [&](int tok, int stage) {
         const uint32_t dst0 = ring + stage * S::kStage;
-        for (int i = threadIdx.x; i < TOK * (DK / 8); i += 256) {
+        for (int i = threadIdx.x; i < TOK * (DK / 8); i += NW * 32) {
             const int r = i / (DK / 8), ch = i - r * (DK / 8);
             const bool ok = tok + r < t1 && ch * 8 < p.d;
             const size_t off = ok ? (size_t)(tok + r) * p.d + ch * 8 : 0;
@@ -377,8 +376,8 @@ __global__ void __launch_bounds__(256, 1) bwd_sums_kernel(const __grid_constant_
         const int csize = gridDim.x, crank = blockIdx.x;
         unsigned char* ms = smem + S::kMats * rows * PITCH;
         float* acc = reinterpret_cast<float*>(ms) + warp * 16 * S::kAccPitch;
-        float2* ml = reinterpret_cast<float2*>(ms + 8 * 16 * S::kAccPitch * 4);
-        float* wt = reinterpret_cast<float*>(ms + 8 * 16 * (S::kAccPitch + 2) * 4);
+        float2* ml = reinterpret_cast<float2*>(ms + NW * 16 * S::kAccPitch * 4);
+        float* wt = reinterpret_cast<float*>(ms + NW * 16 * (S::kAccPitch + 2) * 4);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const float l = quad_sum(sum[h]);
@@ -389,7 +388,7 @@ __global__ void __launch_bounds__(256, 1) bwd_sums_kernel(const __grid_constant_
         }
         cluster_sync_all(csize);
         const int nrows = min(rows, p.n - row0), nsrc = csize * KG, share = (nrows - crank + csize - 1) / csize;
-        const uint32_t acc0 = smem_u32(ms), ml0 = acc0 + 8 * 16 * S::kAccPitch * 4;
+        const uint32_t acc0 = smem_u32(ms), ml0 = acc0 + NW * 16 * S::kAccPitch * 4;
         if ((int)threadIdx.x < share) {
             const int r = crank + threadIdx.x * csize;
             float m[8 * KG], l[8 * KG], mm = -INFINITY, tot = 0.f;
@@ -416,7 +415,7 @@ __global__ void __launch_bounds__(256, 1) bwd_sums_kernel(const __grid_constant_
             p.agent_stats[(size_t)slab * p.n + row0 + r].x = mm + log2f(tot);
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < share * (DK / 2); i += 256) {
+        for (int i = threadIdx.x; i < share * (DK / 2); i += NW * 32) {
             const int k = i / (DK / 2), ch = 2 * (i - k * (DK / 2)), r = crank + k * csize;
             if (ch >= p.d) continue;
             float2 v = make_float2(0.f, 0.f);
@@ -455,6 +454,8 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
     const int t0 = min(p.N, (int)blockIdx.x * p.tokens), t1 = min(p.N, t0 + p.tokens);
     const uint32_t sm = smem_u32(smem);
     float2* st_s = reinterpret_cast<float2*>(smem + (TA + TM) * n32 * PITCH);
+    pdl_wait_prior();
+    pdl_release_next();
     {
         const int chunks = DK / 8;
         for (int i = threadIdx.x; i < (TA + TM) * n32 * chunks; i += 256) {

@@ -209,7 +209,9 @@ struct BwdPlan {
 struct BwdArgs {
     const void *x, *y;        // token rows [slabs][N][d]: operand of the logits, second operand
     const void* bias;         // B1 [heads][n][N] or B2 [heads][N][n], or null
-    const float *m0, *m1;     // fp32 [slabs][n][d]: A; V_A or dV_A
+    const float *m0, *m1;     // fp32 [slabs][n][d]: A; V_A or dV_A  (mixed precision: V_A, dV_A)
+    const void *a_t, *va_t;   // mixed precision: 16-bit A [slabs][n][d]; two terms of V_A [2][slabs][n][d]
+    const float2* stats;      // mixed precision: .x = log2-sum-exp of the aggregation rows [slabs][n]
     const float *lse, *dot;   // fp32 [slabs][n]: log-sum-exp of the aggregation rows; dV_A . V_A
     float* part;              // fp32 [slabs][chunks][n][2]: per-block (max, sum) of the aggregation logits
     float *outer0, *outer1;   // fp32 [slabs][n][d]: sums over tokens (atomics)
@@ -226,7 +228,7 @@ struct BwdCall {
     float *ws_a, *ws_va, *ws_dva, *ws_da;     // [slabs][n][d] each; V_A, dV_A, dA contiguous in this order
     float *ws_lse, *ws_dot;                   // [slabs][n]
     float* ws_part;                           // [slabs][chunks][n][2]
-    size_t clear_bytes;                       // bytes from ws_va to the end of ws_da
+    size_t region_bytes;                      // bytes from ws_va to ws_dva and from ws_dva to ws_da
     int slabs, heads, H, W, d, n, p, sm_count;
     float scale1, scale2;
     BwdPlan plan;
@@ -239,6 +241,8 @@ struct BwdCall {
 bool backward_terms_eligible(int dtype, int n, int d);
 size_t backward_terms_bytes(int slabs, int n, int N, int d);
 cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStream_t st);
+// mixed precision, 16-bit inputs: A (16 bits, in ws_a), V_A (fp32 in ws_va, terms in ws_part), statistics (in ws_lse); clears the sums
+cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStream_t st);
 // token-wise tail: dQ += Pooling^T(dA), dV += DWC^T(dO), dWd
 cudaError_t launch_backward_tail(int dtype, const BwdCall& c, cudaStream_t st);
 bool plan_backward(int slabs, int n, int N, int d, int sm_count, BwdPlan* out);   // false: shape not supported
@@ -248,8 +252,5 @@ cudaError_t launch_backward(int dtype, const BwdCall& c, cudaStream_t st);
 bool backward_mma_eligible(int dtype, int n, int d);
 BwdPlan plan_backward_mma(int slabs, int N, int sm_count);
 cudaError_t launch_backward_mma(int dtype, bool broadcast_stage, const BwdArgs& a, cudaStream_t st);
-// aggregation stage recomputed: per-block partials into a.part, then V_A and the log-sum-exp per agent
-cudaError_t launch_backward_fwd1_mma(int dtype, const BwdArgs& a, float* va, float* lse, cudaStream_t st);
-size_t backward_mma_part_floats(int slabs, const BwdPlan& pl);
 
 }  // namespace aa
