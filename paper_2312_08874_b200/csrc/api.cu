@@ -3,6 +3,7 @@
 #include "../../include/agent_attn.h"
 #include "kernels.h"
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -11,6 +12,15 @@
 #include <new>
 
 using namespace aa;
+
+constexpr int kHostParts = 4;
+
+// What a call on host buffers keeps between calls: copy streams, events and the handles of its parts.
+struct HostPipe {
+    cudaStream_t in, out;
+    cudaEvent_t start, finish, ready[kHostParts], done[kHostParts];
+    agent_attn_handle* part[kHostParts];
+};
 
 struct agent_attn_handle {
     agent_attn_config cfg;
@@ -27,6 +37,7 @@ struct agent_attn_handle {
     bool stream_args_valid;
     unsigned poll_limit;    // flag-poll limit of the task-queue kernel (test hook; 0xffffffff = the kernel's own)
     unsigned stage_mask;    // which of the three streaming kernels a forward call launches (measurement hook; 7 = all)
+    HostPipe* pipe;         // made by the first host call that is split
     char err[512];
 };
 
@@ -304,10 +315,25 @@ int agent_attn_create(agent_attn_handle** out, const agent_attn_config* cfg) {
     return AA_OK;
 }
 
+static void destroy_pipe(HostPipe* p) {
+    if (!p) return;
+    if (p->in) cudaStreamDestroy(p->in);
+    if (p->out) cudaStreamDestroy(p->out);
+    if (p->start) cudaEventDestroy(p->start);
+    if (p->finish) cudaEventDestroy(p->finish);
+    for (int i = 0; i < kHostParts; ++i) {
+        if (p->ready[i]) cudaEventDestroy(p->ready[i]);
+        if (p->done[i]) cudaEventDestroy(p->done[i]);
+    }
+    for (agent_attn_handle* q : p->part) delete q;
+    delete p;
+}
+
 int agent_attn_destroy(agent_attn_handle* h) {
     if (!h) return AA_OK;
     {
         DeviceGuard guard(h->cfg.device);
+        destroy_pipe(h->pipe);
         if (h->d_status) cudaFree(h->d_status);
     }
     delete h;
@@ -572,14 +598,81 @@ int agent_attn_compose_bias(agent_attn_handle* h, const void* col, const void* r
     return AA_OK;
 }
 
+// A call on host buffers is bound by its copies (56 x 56 grid, 64 slabs: 78 MB in, 26 MB out, 1.98 ms in one piece).  It is cut into
+// parts along the batch, or along the heads of a single batch entry: the copies in, the kernels and the copies out of different
+// parts overlap, and what follows the last copy in is the work of the last part.  So parts halve: a half, a quarter, two eighths (few
+// copies, each costs 4 us of its own: eight even parts took 1.95 ms), but no less than 2 MB of input in the smaller half.
+constexpr size_t kBiasSlack = 256 * kHostParts;        // (parts by heads: each part's biases start at a multiple of 256 bytes)
+struct HostParts {
+    int count, units, size[kHostParts];
+};
+static HostParts host_parts(const agent_attn_handle* h, size_t qkv_bytes) {
+    HostParts p = {};
+    p.units = h->cfg.batch > 1 ? h->cfg.batch : h->cfg.heads;
+    for (int left = p.units; left > 0;) {
+        const bool cut = p.count + 1 < kHostParts && left > 1 && 3 * qkv_bytes / p.units * (left / 2) >= (2u << 20);
+        p.size[p.count] = cut ? (left + 1) / 2 : left;
+        left -= p.size[p.count++];
+    }
+    return p;
+}
+// Copy of a handle for `units` batch entries (or heads), without what was cached for the whole.
+static void part_handle(const agent_attn_handle* h, int units, agent_attn_handle* out) {
+    *out = *h;
+    (h->cfg.batch > 1 ? out->cfg.batch : out->cfg.heads) = units;
+    memset(out->fused_key, 0, sizeof(out->fused_key));
+    memset(out->stream_key, 0, sizeof(out->stream_key));
+    out->stream_args_valid = false;
+    out->pipe = nullptr;
+}
+
 size_t agent_attn_staging_bytes(const agent_attn_handle* h, int grid_h, int grid_w, int n_agents) {
-    const size_t ws = agent_attn_workspace_bytes(h, grid_h, grid_w, n_agents);
+    size_t ws = agent_attn_workspace_bytes(h, grid_h, grid_w, n_agents);
     if (!ws) return 0;
     const size_t es = h->elem_bytes, slabs = (size_t)h->cfg.batch * h->cfg.heads;
     const size_t N = (size_t)grid_h * grid_w, d = h->cfg.head_dim, n = n_agents, heads = h->cfg.heads;
+    const HostParts parts = host_parts(h, slabs * N * d * es);
+    for (int i = 0; parts.count > 1 && i < parts.count; ++i) {
+        agent_attn_handle part;
+        part_handle(h, parts.size[i], &part);
+        ws = std::max(ws, agent_attn_workspace_bytes(&part, grid_h, grid_w, n_agents));
+    }
     const size_t qkv = align_up(slabs * N * d * es, 256);
-    return 4 * qkv + align_up(slabs * n * d * es, 256) + 2 * align_up(heads * n * N * es, 256) +
+    return 4 * qkv + align_up(slabs * n * d * es, 256) + 2 * (align_up(heads * n * N * es, 256) + kBiasSlack) +
            align_up(heads * d * 9 * es, 256) + align_up(ws, 256);
+}
+
+// The handle's copy streams and events, and part handles of these sizes.
+static HostPipe* host_pipe(agent_attn_handle* h, const HostParts& parts) {
+    if (!h->pipe) {
+        HostPipe* p = new (std::nothrow) HostPipe;
+        if (!p) return nullptr;
+        memset(p, 0, sizeof(*p));
+        bool ok = cudaStreamCreateWithFlags(&p->in, cudaStreamNonBlocking) == cudaSuccess &&
+                  cudaStreamCreateWithFlags(&p->out, cudaStreamNonBlocking) == cudaSuccess;
+        for (cudaEvent_t* e : {&p->start, &p->finish}) ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+        for (int i = 0; i < kHostParts; ++i)
+            ok = ok && cudaEventCreateWithFlags(&p->ready[i], cudaEventDisableTiming) == cudaSuccess &&
+                 cudaEventCreateWithFlags(&p->done[i], cudaEventDisableTiming) == cudaSuccess;
+        for (agent_attn_handle*& q : p->part) {
+            q = new (std::nothrow) agent_attn_handle;
+            if (q) part_handle(h, 0, q);
+            ok = ok && q;
+        }
+        if (!ok) {
+            destroy_pipe(p);
+            return nullptr;
+        }
+        h->pipe = p;
+    }
+    for (int i = 0; i < parts.count; ++i) {
+        agent_attn_handle* q = h->pipe->part[i];
+        const int u = parts.size[i];
+        if ((h->cfg.batch > 1 ? q->cfg.batch : q->cfg.heads) != u) part_handle(h, u, q);
+        q->poll_limit = h->poll_limit;
+        q->stage_mask = h->stage_mask;
+    }
+    return h->pipe;
 }
 
 int agent_attn_forward_host(agent_attn_handle* h, const void* Q, const void* K, const void* V, const void* A,
@@ -598,33 +691,86 @@ int agent_attn_forward_host(agent_attn_handle* h, const void* Q, const void* K, 
     const size_t es = h->elem_bytes, slabs = (size_t)h->cfg.batch * h->cfg.heads;
     const size_t N = (size_t)grid_h * grid_w, d = h->cfg.head_dim, n = n_agents, heads = h->cfg.heads;
     const size_t qkv_b = slabs * N * d * es, a_b = slabs * n * d * es, bias_b = heads * n * N * es, w_b = heads * d * 9 * es;
+    // device regions, and the host pointers they are filled from
+    enum { kQ, kK, kV, kA, kB1, kB2, kW, kO, kRegions };
+    const void* src[kRegions] = {Q, K, V, A, bias ? bias->b1 : nullptr, bias ? bias->b2 : nullptr, dwc_weight, out};
+    const size_t bytes[kRegions] = {qkv_b, qkv_b, qkv_b, a_b, bias_b, bias_b, w_b, qkv_b};
+    char* dev[kRegions];
     char* s = static_cast<char*>(staging);
-    char* dQ = s;                       s += align_up(qkv_b, 256);
-    char* dK = s;                       s += align_up(qkv_b, 256);
-    char* dV = s;                       s += align_up(qkv_b, 256);
-    char* dO = s;                       s += align_up(qkv_b, 256);
-    char* dA = s;                       s += align_up(a_b, 256);
-    char* dB1 = s;                      s += align_up(bias_b, 256);
-    char* dB2 = s;                      s += align_up(bias_b, 256);
-    char* dW = s;                       s += align_up(w_b, 256);
+    for (int i = 0; i < kRegions; ++i) { dev[i] = s; s += align_up(bytes[i], 256) + (i == kB1 || i == kB2 ? kBiasSlack : 0); }
     char* dWs = s;
-    const size_t ws_bytes = agent_attn_workspace_bytes(h, grid_h, grid_w, n_agents);
-    struct Cp { void* dst; const void* src; size_t bytes; } cps[] = {
-        {dQ, Q, qkv_b}, {dK, K, qkv_b}, {dV, V, qkv_b}, {dA, A, a_b},
-        {dB1, bias ? bias->b1 : nullptr, bias_b}, {dB2, bias ? bias->b2 : nullptr, bias_b}, {dW, dwc_weight, w_b}};
-    for (const Cp& c : cps) {
-        if (!c.src) continue;
-        cudaError_t e = cudaMemcpyAsync(c.dst, c.src, c.bytes, cudaMemcpyHostToDevice, st);
-        if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "host-to-device copy failed: %s", cudaGetErrorString(e));
+    const size_t ws_bytes = staging_bytes - (size_t)(s - static_cast<char*>(staging));
+
+    HostParts parts = host_parts(h, qkv_b);
+    bool split = parts.count > 1;
+    if (split) {
+        // pageable memory is copied by the host itself, piece by piece: nothing to overlap
+        cudaPointerAttributes pa;
+        for (const void* p : {Q, K, V, (const void*)out})
+            if (cudaPointerGetAttributes(&pa, p) != cudaSuccess || pa.type != cudaMemoryTypeHost) { cudaGetLastError(); split = false; }
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) { cudaGetLastError(); split = false; }
     }
-    agent_attn_bias db;
-    db.b1 = (bias && bias->b1) ? dB1 : nullptr;
-    db.b2 = (bias && bias->b2) ? dB2 : nullptr;
-    int rc = agent_attn_forward(h, dQ, dK, dV, A ? dA : nullptr, grid_h, grid_w, n_agents, bias ? &db : nullptr,
-                                dwc_weight ? dW : nullptr, dO, dWs, ws_bytes, stream);
-    if (rc) return rc;
-    cudaError_t e = cudaMemcpyAsync(out, dO, qkv_b, cudaMemcpyDeviceToHost, st);
-    if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "device-to-host copy failed: %s", cudaGetErrorString(e));
+    HostPipe* pipe = split ? host_pipe(h, parts) : nullptr;
+    if (!pipe) { parts.count = 1; parts.size[0] = parts.units; }
+    cudaError_t e = cudaSuccess;
+#define AA_STEP(x) do { if (e == cudaSuccess) e = (x); } while (0)
+    cudaStream_t cin = pipe ? pipe->in : st, cout = pipe ? pipe->out : st;
+    if (pipe) {
+        AA_STEP(cudaEventRecord(pipe->start, st));                 // the staging memory is the caller's, in the order of its stream
+        AA_STEP(cudaStreamWaitEvent(cin, pipe->start, 0));
+        AA_STEP(cudaStreamWaitEvent(cout, pipe->start, 0));
+    }
+    const bool by_heads = h->cfg.batch == 1;
+    int launches = 0, rc = AA_OK;
+    for (int k = 0, u0 = 0; k < parts.count && e == cudaSuccess; u0 += parts.size[k++]) {
+        // per-head operands go with their part where the heads are cut, else with the first part
+        auto range = [&](int i, size_t* off, size_t* len) {
+            const bool shared = !by_heads && (i == kB1 || i == kB2 || i == kW);
+            *off = shared ? 0 : bytes[i] / parts.units * u0;
+            *len = shared ? (k == 0 ? bytes[i] : 0) : bytes[i] / parts.units * parts.size[k];
+        };
+        const void* in[kRegions];
+        for (int i = 0; i < kRegions; ++i) {
+            size_t off, len;
+            range(i, &off, &len);
+            char* dst = dev[i] + (i == kB1 || i == kB2 ? align_up(off, 256) + (off ? 256 * k : 0) : off);
+            in[i] = src[i] ? dst : nullptr;
+            if (i != kO && src[i] && len) AA_STEP(cudaMemcpyAsync(dst, static_cast<const char*>(src[i]) + off, len, cudaMemcpyHostToDevice, cin));
+        }
+        if (pipe) {
+            AA_STEP(cudaEventRecord(pipe->ready[k], cin));
+            AA_STEP(cudaStreamWaitEvent(st, pipe->ready[k], 0));
+        }
+        if (e != cudaSuccess) break;
+        agent_attn_bias db;
+        db.b1 = in[kB1];
+        db.b2 = in[kB2];
+        agent_attn_handle* ph = pipe ? pipe->part[k] : h;
+        rc = agent_attn_forward(ph, in[kQ], in[kK], in[kV], in[kA], grid_h, grid_w, n_agents, bias ? &db : nullptr, in[kW], const_cast<void*>(in[kO]), dWs,
+                                ws_bytes, stream);
+        launches += ph->launches;
+        if (rc != AA_OK && pipe) memcpy(h->err, ph->err, sizeof(h->err));
+        if (rc != AA_OK) break;
+        size_t off, len;
+        range(kO, &off, &len);
+        if (pipe) {
+            AA_STEP(cudaEventRecord(pipe->done[k], st));
+            AA_STEP(cudaStreamWaitEvent(cout, pipe->done[k], 0));
+        }
+        AA_STEP(cudaMemcpyAsync(static_cast<char*>(out) + off, dev[kO] + off, len, cudaMemcpyDeviceToHost, cout));
+    }
+    if (pipe) {                                                    // (after an error too: the caller's stream ends after the copies)
+        cudaError_t f = cudaEventRecord(pipe->finish, cin);
+        if (f == cudaSuccess) f = cudaStreamWaitEvent(st, pipe->finish, 0);
+        if (f == cudaSuccess) f = cudaEventRecord(pipe->finish, cout);
+        if (f == cudaSuccess) f = cudaStreamWaitEvent(st, pipe->finish, 0);
+        AA_STEP(f);
+    }
+#undef AA_STEP
+    if (rc != AA_OK) return rc;
+    if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "copying between host and device failed: %s", cudaGetErrorString(e));
+    h->launches = launches;
     return AA_OK;
 }
 
