@@ -121,12 +121,15 @@ def load_library(build_if_missing: bool = True) -> ctypes.CDLL:
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream_ptr(stream: Optional[torch.cuda.Stream]):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    return (torch.cuda.current_stream() if stream is None else stream).cuda_stream
+
+
+def _bias(b1: Optional[torch.Tensor], b2: Optional[torch.Tensor]):
+    return None if b1 is None and b2 is None else ctypes.byref(AgentAttnBias(_ptr(b1), _ptr(b2)))
 
 
 class AgentAttention:
@@ -148,6 +151,7 @@ class AgentAttention:
             raise AgentAttnError(rc, "agent_attn_create failed (is an sm_100 GPU present?)")
         self._ws: Optional[torch.Tensor] = None
         self._staging: Optional[torch.Tensor] = None
+        self._bytes: dict = {}             # scratch sizes by call shape: they depend on nothing else
 
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:
@@ -164,15 +168,24 @@ class AgentAttention:
     def _chk_tensor(self, t: Optional[torch.Tensor], shape, name: str, cuda: bool = True):
         if t is None:
             return
-        if tuple(t.shape) != tuple(shape) or t.dtype != self.dtype or not t.is_contiguous() or t.is_cuda != cuda:
+        if t.shape != shape or t.dtype is not self.dtype or not t.is_contiguous() or t.is_cuda is not cuda:
             raise ValueError(f"{name}: expected contiguous {'cuda' if cuda else 'cpu'} {self.dtype} tensor of "
                              f"shape {tuple(shape)}, got {tuple(t.shape)} {t.dtype} on {t.device}")
 
+    def _scratch_bytes(self, query: str, grid_h: int, grid_w: int, n_agents: int) -> int:
+        key = (query, grid_h, grid_w, n_agents)
+        need = self._bytes.get(key)
+        if need is None:
+            if len(self._bytes) >= 64:
+                self._bytes.clear()
+            need = self._bytes[key] = int(getattr(self.lib, query)(self._h, grid_h, grid_w, n_agents))
+        return need
+
     def workspace_bytes(self, grid_h: int, grid_w: int, n_agents: int) -> int:
-        return int(self.lib.agent_attn_workspace_bytes(self._h, grid_h, grid_w, n_agents))
+        return self._scratch_bytes("agent_attn_workspace_bytes", grid_h, grid_w, n_agents)
 
     def staging_bytes(self, grid_h: int, grid_w: int, n_agents: int) -> int:
-        return int(self.lib.agent_attn_staging_bytes(self._h, grid_h, grid_w, n_agents))
+        return self._scratch_bytes("agent_attn_staging_bytes", grid_h, grid_w, n_agents)
 
     def workspace(self, grid_h: int, grid_w: int, n_agents: int) -> torch.Tensor:
         need = self.workspace_bytes(grid_h, grid_w, n_agents)
@@ -219,10 +232,9 @@ class AgentAttention:
             out = torch.empty_like(q)
         self._chk_tensor(out, (B, h, N, d), "out")
         ws = self.workspace(grid_h, grid_w, n_agents) if workspace is None else workspace
-        bias = AgentAttnBias(_ptr(b1), _ptr(b2)) if (b1 is not None or b2 is not None) else None
         self._check(self.lib.agent_attn_forward(
             self._h, _ptr(q), _ptr(k), _ptr(v), _ptr(agents), grid_h, grid_w, n_agents,
-            ctypes.byref(bias) if bias is not None else None, _ptr(dwc_weight), _ptr(out), _ptr(ws),
+            _bias(b1, b2), _ptr(dwc_weight), _ptr(out), _ptr(ws),
             ws.numel(), _stream_ptr(stream)))
         return out
 
@@ -238,7 +250,7 @@ class AgentAttention:
         for t, nm in ((q, "q"), (k, "k"), (v, "v"), (out, "out")):
             if t is None:
                 continue
-            if tuple(t.shape) != (B, h, N, d) or t.dtype != self.dtype or not t.is_cuda or t.stride(3) != 1:
+            if t.shape != (B, h, N, d) or t.dtype is not self.dtype or not t.is_cuda or t.stride(3) != 1:
                 raise ValueError(f"{nm}: expected a cuda {self.dtype} view of shape {(B, h, N, d)} with contiguous channels")
         if q.stride() != k.stride() or q.stride() != v.stride():
             raise ValueError("q, k and v must have the same strides")
@@ -249,17 +261,16 @@ class AgentAttention:
         if out is None:
             out = torch.empty((B, N, h, d), dtype=self.dtype, device=self.device).permute(0, 2, 1, 3)
         ws = self.workspace(grid_h, grid_w, n_agents) if workspace is None else workspace
-        bias = AgentAttnBias(_ptr(b1), _ptr(b2)) if (b1 is not None or b2 is not None) else None
         sin = (ctypes.c_longlong * 3)(q.stride(0), q.stride(1), q.stride(2))
         sout = (ctypes.c_longlong * 3)(out.stride(0), out.stride(1), out.stride(2))
         self._check(self.lib.agent_attn_forward_strided(
             self._h, _ptr(q), _ptr(k), _ptr(v), _ptr(agents), sin, grid_h, grid_w, n_agents,
-            ctypes.byref(bias) if bias is not None else None, _ptr(dwc_weight), _ptr(out), sout, _ptr(ws),
+            _bias(b1, b2), _ptr(dwc_weight), _ptr(out), sout, _ptr(ws),
             ws.numel(), _stream_ptr(stream)))
         return out
 
     def backward_workspace(self, grid_h: int, grid_w: int, n_agents: int) -> torch.Tensor:
-        nbytes = self.lib.agent_attn_backward_workspace_bytes(self._h, grid_h, grid_w, n_agents)
+        nbytes = self._scratch_bytes("agent_attn_backward_workspace_bytes", grid_h, grid_w, n_agents)
         if nbytes == 0:
             raise AgentAttnError(2, f"backward does not support grid {grid_h}x{grid_w} with {n_agents} agents")
         return torch.empty(nbytes, dtype=torch.uint8, device=self.device)
@@ -280,22 +291,20 @@ class AgentAttention:
         self._chk_tensor(b1, (h, n_agents, N), "b1")
         self._chk_tensor(b2, (h, N, n_agents), "b2")
         self._chk_tensor(dwc_weight, (h, d, 3, 3), "dwc_weight")
-        f32 = dict(dtype=torch.float32, device=self.device)
-        g = {"dq": torch.empty((B, h, N, d), **f32), "dk": torch.empty((B, h, N, d), **f32),
-             "dv": torch.empty((B, h, N, d), **f32)}
+        f32, dev = torch.float32, self.device
+        g = {k: torch.empty((B, h, N, d), dtype=f32, device=dev) for k in ("dq", "dk", "dv")}
         if b1 is not None and need_bias_grads:
-            g["db1"] = torch.empty((h, n_agents, N), **f32)
+            g["db1"] = torch.empty((h, n_agents, N), dtype=f32, device=dev)
         if b2 is not None and need_bias_grads:
-            g["db2"] = torch.empty((h, N, n_agents), **f32)
+            g["db2"] = torch.empty((h, N, n_agents), dtype=f32, device=dev)
         if dwc_weight is not None and need_filter_grad:
-            g["dwd"] = torch.empty((h, d, 3, 3), **f32)
+            g["dwd"] = torch.empty((h, d, 3, 3), dtype=f32, device=dev)
         ws = self.backward_workspace(grid_h, grid_w, n_agents) if workspace is None else workspace
-        bias = AgentAttnBias(_ptr(b1), _ptr(b2)) if (b1 is not None or b2 is not None) else None
         grads = AgentAttnGrads(_ptr(g["dq"]), _ptr(g["dk"]), _ptr(g["dv"]), _ptr(g.get("db1")), _ptr(g.get("db2")),
                                _ptr(g.get("dwd")))
         self._check(self.lib.agent_attn_backward(
             self._h, _ptr(q), _ptr(k), _ptr(v), _ptr(d_out), grid_h, grid_w, n_agents,
-            ctypes.byref(bias) if bias is not None else None, _ptr(dwc_weight), ctypes.byref(grads), _ptr(ws),
+            _bias(b1, b2), _ptr(dwc_weight), ctypes.byref(grads), _ptr(ws),
             ws.numel(), _stream_ptr(stream)))
         return g
 
@@ -404,12 +413,11 @@ class AgentAttention:
             if self._staging is None or self._staging.numel() < need:
                 self._staging = torch.empty(need, dtype=torch.uint8, device=self.device)
             staging = self._staging
-        bias = AgentAttnBias(_ptr(b1), _ptr(b2)) if (b1 is not None or b2 is not None) else None
         s = torch.cuda.current_stream() if stream is None else stream
         self._check(self.lib.agent_attn_forward_host(
             self._h, _ptr(q), _ptr(k), _ptr(v), _ptr(agents), grid_h, grid_w, n_agents,
-            ctypes.byref(bias) if bias is not None else None, _ptr(dwc_weight), _ptr(out),
-            _ptr(staging), staging.numel(), ctypes.c_void_p(s.cuda_stream)))
+            _bias(b1, b2), _ptr(dwc_weight), _ptr(out),
+            _ptr(staging), staging.numel(), s.cuda_stream))
         if synchronize:
             s.synchronize()
         return out
