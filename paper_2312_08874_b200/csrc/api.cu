@@ -65,6 +65,10 @@ bool use_simt(const agent_attn_handle* h) {
     return h->cfg.dtype == AA_F32 || h->cfg.path == AA_PATH_SIMT;
 }
 
+// fp32 tensors on the tensor cores, as 16-bit terms
+bool use_terms_forward(const agent_attn_handle* h, int n_agents) {
+    return h->cfg.dtype == AA_F32 && auto_like(h) && terms_forward_eligible(n_agents, h->cfg.head_dim);
+}
 // Shapes that the tensor-memory kernels take (large agent counts, aligned rows).  The rule does not depend on the bias, so that
 // the workspace size is the same with and without one.
 bool umma_shape(const agent_attn_handle* h, int n_tokens, int n_agents) {
@@ -139,6 +143,7 @@ WsLayout ws_layout(const agent_attn_handle* h, int n_tokens, int n_agents, int g
             extra = stream_extra_bytes((int)slabs, h->cfg.heads, n_tokens, n_agents);
         }
     }
+    if (use_terms_forward(h, n_agents)) extra = terms_forward_bytes((int)slabs, n_agents, h->cfg.head_dim);
     w.ticket_off = w.part_off + align_up(part_floats * sizeof(float), 256);
     w.extra_off = w.ticket_off + align_up(fused_counter_words((int)slabs) * sizeof(unsigned), 256);
     w.total = w.extra_off + extra;
@@ -523,6 +528,16 @@ static int forward_impl(agent_attn_handle* h, const void* Q, const void* K, cons
             return AA_OK;
         }
     }
+    if (use_terms_forward(h, n_agents)) {
+        TermsForward t = {static_cast<const float*>(Q), static_cast<const float*>(K), static_cast<const float*>(V), static_cast<const float*>(A),
+                          static_cast<const float*>(b1), static_cast<const float*>(b2), static_cast<const float*>(dwc_weight),
+                          reinterpret_cast<float*>(ws + w.a_off), reinterpret_cast<float*>(ws + w.va_off), static_cast<float*>(out), ws + w.extra_off,
+                          h->cfg.batch * h->cfg.heads, h->cfg.heads, grid_h, grid_w, h->cfg.head_dim, n_agents, p, h->sm_count, h->scale1, h->scale2};
+        const cudaError_t e = launch_terms_forward(t, st);
+        if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "forward launch failed: %s", cudaGetErrorString(e));
+        h->launches = 3;
+        return AA_OK;
+    }
     if (!use_simt(h) && !use_umma(h, N, n_agents)) {
         TileArgs t = tile_args(h, grid_h, grid_w, n_agents, cl);
         t.q = Q; t.k = K; t.v = V; t.a = A ? A : ws + w.a_off; t.va = ws + w.va_off; t.pool = p;
@@ -797,7 +812,7 @@ namespace {
 struct BwdLayout {
     size_t a, va, dva, da, lse, dot, part, terms, total;
 };
-// 16-bit inputs outside the mixed-precision kernels: fp32 operands as 16-bit terms on the tensor cores
+// inputs outside the mixed-precision kernels: fp32 operands as 16-bit terms on the tensor cores
 bool use_terms(const agent_attn_handle* h, int n) {
     return auto_like(h) && !backward_mma_eligible(h->cfg.dtype, n, h->cfg.head_dim) && backward_terms_eligible(h->cfg.dtype, n, h->cfg.head_dim);
 }

@@ -390,7 +390,7 @@ cudaError_t backward_typed(const BwdCall& c, BwdArgs a, cudaStream_t st) {
     cudaError_t e;
 #define AA_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
     if (c.ws_terms) {
-        if constexpr (sizeof(T) == 2) AA_TRY(launch_backward_terms(c.dtype, c, c.ws_terms, st));
+        AA_TRY(launch_backward_terms(c.dtype, c, c.ws_terms, st));
         return launch_backward_tail(c.dtype, c, st);
     }
     if (c.use_mma) {

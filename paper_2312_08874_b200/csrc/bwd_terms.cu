@@ -1,5 +1,5 @@
-// Gradients of the attention stages with fp32 operands on the tensor cores: launch plans and the small kernels between the
-// stages (term splits, D = dV_A . V_A).
+// The attention stages with fp32 operands on the tensor cores (the gradients, and the forward pass of fp32 tensors): launch plans
+// and the small kernels between the stages (term splits, D = dV_A . V_A).
 #include "bwd_terms_launch.cuh"
 #include "tile_pool.cuh"
 
@@ -31,9 +31,17 @@ struct ClearList {
 };
 constexpr int kClearWords = 256 * 32;              // words that a block clears
 
+struct PoolArgs8 {
+    const void *q, *given;             // tokens, or the caller's agents
+    float* plain;                      // the agents in fp32 too, or null
+    int slabs, n, H, W, pool, d;
+    bool small;
+};
 // Pooled agents as NT terms of E: a warp per window, or (windows of at most 32 tokens on average) a thread per 8 channels.
 template <typename T, typename E, int NT>
-__global__ void __launch_bounds__(256) bwd_pool_terms_kernel(const T* q, E* dst, int slabs, int n, int H, int W, int pool, int d, bool small, ClearList cl) {
+__global__ void __launch_bounds__(256) bwd_pool_terms_kernel(PoolArgs8 pa, E* dst, ClearList cl) {
+    const T *q = static_cast<const T*>(pa.q), *given = static_cast<const T*>(pa.given);
+    const int slabs = pa.slabs, n = pa.n, H = pa.H, W = pa.W, pool = pa.pool, d = pa.d;
     pdl_release_next();
     if ((int)blockIdx.x >= cl.pool_blocks) {
         size_t b = (size_t)(blockIdx.x - cl.pool_blocks) * kClearWords;
@@ -52,17 +60,28 @@ __global__ void __launch_bounds__(256) bwd_pool_terms_kernel(const T* q, E* dst,
     }
     const size_t plane = (size_t)slabs * n * d;
     auto put = [&](size_t off, const float (&f)[8]) {
+        if (pa.plain) {
+            *reinterpret_cast<float4*>(pa.plain + off) = make_float4(f[0], f[1], f[2], f[3]);
+            *reinterpret_cast<float4*>(pa.plain + off + 4) = make_float4(f[4], f[5], f[6], f[7]);
+        }
         uint32_t w[4][NT];
 #pragma unroll
         for (int i = 0; i < 4; ++i) split_pair<E, NT>(f[2 * i], f[2 * i + 1], w[i]);
 #pragma unroll
         for (int k = 0; k < NT; ++k) *reinterpret_cast<uint4*>(dst + k * plane + off) = make_uint4(w[0][k], w[1][k], w[2][k], w[3][k]);
     };
-    if (small) {
+    if (pa.small) {
         const int cpt = d >> 3;
         const long long i = (long long)blockIdx.x * 256 + threadIdx.x, cell = i / cpt;
         if (cell >= (long long)slabs * n) return;
         const int slab = (int)(cell / n), agent = (int)(cell - (long long)slab * n), ch = (int)(i - cell * cpt);
+        if (given) {
+            float2 a[4] = {};
+            add_raw8<T>(a, ld_raw8<T>(given + (size_t)cell * d + ch * 8));
+            const float f[8] = {a[0].x, a[0].y, a[1].x, a[1].y, a[2].x, a[2].y, a[3].x, a[3].y};
+            put((size_t)cell * d + ch * 8, f);
+            return;
+        }
         pool_chunk<T>(q + (size_t)slab * H * W * d + ch * 8, d, H, W, pool, agent, [&](const float (&f)[8]) { put((size_t)cell * d + ch * 8, f); });
     } else {
         const long long cell = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -98,12 +117,15 @@ __global__ void __launch_bounds__(256) bwd_dot_split_kernel(const float* va, con
 struct SumsPlan {
     int rb, rg, kg;
 };
-SumsPlan sums_plan(int n, int d) {
+SumsPlan sums_plan(int dtype, int n, int d) {
     const int dk = dk_of_terms(d), most = dk <= 64 ? 128 : dk <= 80 ? 64 : 32;       // agent rows of a block: six term tiles of them, and the ring, in shared memory
     SumsPlan s;
     s.rb = (n + most - 1) / most;
     s.rg = ((n + s.rb - 1) / s.rb + 15) / 16;
     s.kg = s.rg <= 2 && dk <= 80 ? 4 : s.rg <= 4 ? 2 : 1;
+    // fp32 tokens are three terms: two stages of 32 kg of them, K and V, beside the agents'
+    if (dtype == kF32)
+        while (s.kg > 1 && (6 * s.rg * 16 + 2 * 6 * 32 * s.kg) * (dk * 2 + 16) + 2 * 32 * s.kg * 8 > 227 * 1024) s.kg /= 2;
     return s;
 }
 // Parts of the token axis for `slots` resident blocks; a block's start (agents' terms into shared memory) costs about 256 tokens.
@@ -121,27 +143,30 @@ int token_parts(long long others, int N, int unit, int most, bool pow2, int slot
 
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 
+template <typename T, typename E, int NT> cudaError_t launch_pool_terms(PoolArgs8 pa, void* a_t, ClearList cl, cudaStream_t st) {
+    pa.small = pa.given || pa.H * pa.W <= 32 * pa.n;
+    cl.pool_blocks = (int)(pa.small ? ((long long)pa.slabs * pa.n * (pa.d / 8) + 255) / 256 : ((long long)pa.slabs * pa.n + 7) / 8);
+    size_t clear = 0;
+    for (size_t w : cl.words) clear += (w + kClearWords - 1) / kClearWords;
+    bwd_pool_terms_kernel<T, E, NT><<<(unsigned)(cl.pool_blocks + clear), 256, 0, st>>>(pa, static_cast<E*>(a_t), cl);
+    return cudaGetLastError();
+}
 // Pooling, and the clearing of the sums that the stages add to.
 template <typename T, typename E, int NT> cudaError_t pool_and_clear(const BwdCall& c, void* a_t, bool clear_bias, cudaStream_t st) {
-    const int N = c.H * c.W;
-    const bool small = N <= 32 * c.n;
+    const PoolArgs8 pa = {c.q, nullptr, nullptr, c.slabs, c.n, c.H, c.W, c.p, c.d, false};
     ClearList cl = {};
-    cl.pool_blocks = (int)(small ? ((long long)c.slabs * c.n * (c.d / 8) + 255) / 256 : ((long long)c.slabs * c.n + 7) / 8);
-    const size_t bias = clear_bias ? (size_t)c.heads * c.n * N : 0;
+    const size_t bias = clear_bias ? (size_t)c.heads * c.n * c.H * c.W : 0;
     cl.p[0] = c.ws_dva; cl.words[0] = 2 * c.region_bytes / sizeof(float);          // dV_A, dA
     cl.p[1] = c.db1; cl.words[1] = c.db1 ? bias : 0;
     cl.p[2] = c.db2; cl.words[2] = c.db2 ? bias : 0;
     cl.p[3] = c.dwd; cl.words[3] = c.dwd ? (size_t)c.heads * c.d * 9 : 0;
-    size_t clear = 0;
-    for (size_t w : cl.words) clear += (w + kClearWords - 1) / kClearWords;
-    bwd_pool_terms_kernel<T, E, NT><<<(unsigned)(cl.pool_blocks + clear), 256, 0, st>>>(static_cast<const T*>(c.q), static_cast<E*>(a_t), c.slabs, c.n, c.H, c.W, c.p, c.d, small, cl);
-    return cudaGetLastError();
+    return launch_pool_terms<T, E, NT>(pa, a_t, cl, st);
 }
 
 }  // namespace
 
 bool backward_terms_eligible(int dtype, int n, int d) {
-    if (dtype != kBF16 && dtype != kF16) return false;
+    if (dtype == kF32 && (d % 8 || dk_of_terms(d) > kTermGradientsF32)) return false;
     const int dk = dk_of_terms(d), pitch = dk * 2 + 16, n32 = (n + 31) & ~31;
     return 6 * n32 * pitch + n32 * 8 <= 227 * 1024;
 }
@@ -179,13 +204,13 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
     cudaError_t e;
 #define AA_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
     const bool clear_bias = slabs != c.heads;          // (a single batch entry stores its bias gradients)
-    AA_TRY(dtype == kBF16 ? (pool_and_clear<B, B, 3>(c, a_t, clear_bias, st)) : (pool_and_clear<__half, B, 3>(c, a_t, clear_bias, st)));
+    AA_TRY(dtype == kBF16 ? (pool_and_clear<B, B, 3>(c, a_t, clear_bias, st)) : dtype == kF16 ? (pool_and_clear<__half, B, 3>(c, a_t, clear_bias, st)) : (pool_and_clear<float, B, 3>(c, a_t, clear_bias, st)));
 
     BwdTermArgs a;
     memset(&a, 0, sizeof(a));
     a.slabs = slabs; a.heads = c.heads; a.N = N; a.n = n; a.d = d;
     a.a_t = a_t; a.tok_stats = tok_stats; a.agent_stats = agent_stats;
-    const SumsPlan sp = sums_plan(n, d);
+    const SumsPlan sp = sums_plan(dtype, n, d);
     a.rg = sp.rg;
     BwdTermLaunch l;
     l.stream = st; l.kg = sp.kg;
@@ -221,6 +246,44 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
     AA_TRY(rows(kTermKeyValue));
 #undef AA_TRY
     return cudaSuccess;
+}
+
+// fp32 forward pass: three kernels.  (The CUDA-core kernels took 119 us for one image of 196 tokens, three heads of 64 channels and
+// 49 agents.)
+bool terms_forward_eligible(int n, int d) {
+    const int dk = dk_of_terms(d), n32 = (n + 31) & ~31;
+    return d % 8 == 0 && 6 * n32 * (dk * 2 + 16) + 9 * dk * 4 <= 227 * 1024;
+}
+size_t terms_forward_bytes(int slabs, int n, int d) { return 2 * up256((size_t)slabs * n * d * 2 * 3) + up256((size_t)slabs * n * 8); }
+
+cudaError_t launch_terms_forward(const TermsForward& c, cudaStream_t st) {
+    const int N = c.H * c.W;
+    char* w = static_cast<char*>(c.ws);
+    const size_t terms = up256((size_t)c.slabs * c.n * c.d * 2 * 3);
+    const PoolArgs8 pa = {c.q, c.agents, c.agents ? nullptr : c.a_ws, c.slabs, c.n, c.H, c.W, c.p, c.d, false};
+    cudaError_t e = launch_pool_terms<float, __nv_bfloat16, 3>(pa, w, ClearList{}, st);
+    if (e != cudaSuccess) return e;
+    BwdTermArgs a;
+    memset(&a, 0, sizeof(a));
+    a.slabs = c.slabs; a.heads = c.heads; a.N = N; a.n = c.n; a.d = c.d; a.H = c.H; a.W = c.W;
+    a.a_t = w; a.va_t = w + terms; a.agent_stats = reinterpret_cast<float2*>(w + 2 * terms);
+    const SumsPlan sp = sums_plan(kF32, c.n, c.d);
+    a.rg = sp.rg;
+    BwdTermLaunch l;
+    l.stream = st; l.kg = sp.kg;
+    a.x = c.k; a.y = c.v; a.bias = c.b1; a.scale = c.scale1; a.outer0 = c.va_ws;
+    int parts = token_parts((long long)c.slabs * sp.rb, N, 64, 8, true, c.sm_count);
+    a.tokens = ((N + parts - 1) / parts + 63) / 64 * 64;
+    l.grid = dim3(parts, sp.rb, c.slabs);
+    l.cluster = parts;
+    e = stage(kF32, c.d, kTermForward, a, l);
+    if (e != cudaSuccess) return e;
+    a.x = c.q; a.y = c.v; a.bias = c.b2; a.scale = c.scale2; a.m_t = w + terms; a.row0 = c.out; a.wd = c.wd;
+    parts = token_parts(c.slabs, N, 128, 512, false, c.sm_count);
+    a.tokens = ((N + parts - 1) / parts + 127) / 128 * 128;
+    l.grid = dim3(parts, c.slabs);
+    l.cluster = 0;
+    return stage(kF32, c.d, kTermOut, a, l);
 }
 
 }  // namespace aa

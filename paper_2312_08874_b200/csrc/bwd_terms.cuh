@@ -13,7 +13,7 @@
 namespace aa {
 
 enum BwdSums { kSumsForward, kSumsBroadcast, kSumsAggregate };
-enum BwdRows { kRowsStats, kRowsQuery, kRowsKeyValue };
+enum BwdRows { kRowsStats, kRowsQuery, kRowsKeyValue, kRowsOut };
 
 // term pairs of a product: i of NA, j of NB with i + j < max(NA, NB)
 template <int NA, int NB> struct TermPairs {
@@ -59,24 +59,50 @@ __device__ __forceinline__ void put_dbias8(float* p, const float* v, int cnt, bo
 // A operand (16 rows x 16 channels) from a tile in natural row order
 template <int PITCH> __device__ __forceinline__ uint32_t a_lane_offset(int lane) { return (lane & 15) * PITCH + (lane >> 4) * 16; }
 
-// 16 bytes of a token row as NX chunks of terms
-template <typename T, typename E, int NX> __device__ __forceinline__ void split_chunk(const uint4& raw, uint4 (&out)[NX]) {
-    if constexpr (NX == 1) {
-        out[0] = raw;
-    } else {
-        const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-        uint32_t o[NX][4];
+// Eight channels of a token row as NX chunks of terms (zeros where there are none)
+template <typename T, typename E, int NX> __device__ __forceinline__ void load_terms(const T* src, bool ok, uint4 (&out)[NX]) {
+    uint32_t o[NX][4];
+    uint4 raw[sizeof(T) / 2];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 f = unpack2<T>(w[i]);
-            uint32_t t[NX];
-            split_pair<E, NX>(f.x, f.y, t);
+    for (int i = 0; i < (int)sizeof(T) / 2; ++i) raw[i] = ok ? __ldg(reinterpret_cast<const uint4*>(src) + i) : make_uint4(0u, 0u, 0u, 0u);
+    float f[8];
+    unpack16<T>(raw[0], f);
+    if constexpr (sizeof(T) == 4) unpack16<T>(raw[1], f + 4);
 #pragma unroll
-            for (int k = 0; k < NX; ++k) o[k][i] = t[k];
-        }
+    for (int i = 0; i < 4; ++i) {
+        uint32_t t[NX];
+        split_pair<E, NX>(f[2 * i], f[2 * i + 1], t);
 #pragma unroll
-        for (int k = 0; k < NX; ++k) out[k] = make_uint4(o[k][0], o[k][1], o[k][2], o[k][3]);
+        for (int k = 0; k < NX; ++k) o[k][i] = t[k];
     }
+#pragma unroll
+    for (int k = 0; k < NX; ++k) out[k] = make_uint4(o[k][0], o[k][1], o[k][2], o[k][3]);
+}
+// Two channels of a token row in fp32
+template <typename T> __device__ __forceinline__ float2 load_pair(const T* src) {
+    if constexpr (sizeof(T) == 4) return __ldg(reinterpret_cast<const float2*>(src));
+    else return unpack2<T>(__ldg(reinterpret_cast<const uint32_t*>(src)));
+}
+// Eight consecutive biases of a row of `row` elements times log2(e); the first `left` exist (the others are not used).
+template <typename T> __device__ __forceinline__ void load_bias_row(const T* p, int left, int row, const T* end, float (&bs)[8]) {
+    if constexpr (sizeof(T) == 4) {
+        if (row % 4 == 0) {
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+            if (left > 0) a = __ldg(reinterpret_cast<const float4*>(p));
+            if (left > 4) b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+            bs[0] = a.x; bs[1] = a.y; bs[2] = a.z; bs[3] = a.w;
+            bs[4] = b.x; bs[5] = b.y; bs[6] = b.z; bs[7] = b.w;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) bs[i] = i < left ? __ldg(p + i) : 0.f;
+        }
+    } else {
+        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+        if (left > 0) w = row % 8 == 0 ? __ldg(reinterpret_cast<const uint4*>(p)) : load_bias8_any(p, end);
+        unpack16<T>(w, bs);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) bs[i] *= kLog2e;
 }
 
 struct BwdTermArgs {
@@ -90,6 +116,8 @@ struct BwdTermArgs {
     void* va_t;                            // forward sums: terms of V_A
     int slabs, heads, N, n, d;
     int rg, tokens;                        // sums: row groups; tokens per block (either kernel)
+    const void* wd;                        // rows out: depthwise filter [heads][d][3][3] over y, or null
+    int H, W;
     float scale;                           // of the logits
     float out_scale;                       // of dQ, dK and dA: the same; 0 where the softmax has one column (its logit gradients are exactly zero)
 };
@@ -149,9 +177,9 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(cons
                 cp_async16s(dst0 + o, x + off, ok ? 16 : 0);
                 cp_async16s(dst0 + TOK * PITCH + o, y + off, ok ? 16 : 0);
             } else {
-                uint4 a[NX], b[NX], z = make_uint4(0u, 0u, 0u, 0u);
-                split_chunk<T, E, NX>(ok ? __ldg(reinterpret_cast<const uint4*>(x + off)) : z, a);
-                split_chunk<T, E, NX>(ok ? __ldg(reinterpret_cast<const uint4*>(y + off)) : z, b);
+                uint4 a[NX], b[NX];
+                load_terms<T, E, NX>(x + off, ok, a);
+                load_terms<T, E, NX>(y + off, ok, b);
 #pragma unroll
                 for (int k = 0; k < NX; ++k) {
                     *reinterpret_cast<uint4*>(smem + (dst0 - sm) + k * TOK * PITCH + o) = a[k];
@@ -252,12 +280,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(cons
                         for (int i = 0; i < 8; ++i)
                             if (i < left) bs[h][i] = Elem<T>::to_f32(bias[(size_t)(tok + 8 * t + i) * p.n + r]) * kLog2e;
                     } else {
-                        const T* bp = bias + (size_t)r * p.N + tok + 8 * t;
-                        uint4 w = make_uint4(0u, 0u, 0u, 0u);
-                        if (left > 0) w = p.N % 8 == 0 ? __ldg(reinterpret_cast<const uint4*>(bp)) : load_bias8_any(bp, bias_end);
-                        unpack16<T>(w, bs[h]);
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) bs[h][i] *= kLog2e;
+                        load_bias_row<T>(bias + (size_t)r * p.N + tok + 8 * t, left, p.N, bias_end, bs[h]);
                     }
                 }
             }
@@ -442,18 +465,21 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(cons
 // ------------------------------------------------------------------------------------------------------------- rows
 template <int DK, int TA, int TM> struct RowsShape {
     static constexpr int kPitch = DK * 2 + 16;
-    __host__ __device__ static constexpr int smem(int n) { return (TA + TM) * ((n + 31) & ~31) * kPitch + ((n + 31) & ~31) * 8; }
+    __host__ __device__ static constexpr int smem(int n) { return (TA + TM) * ((n + 31) & ~31) * kPitch + ((n + 31) & ~31) * 8; }      // (or 9 DK filter words, rows out)
+    __host__ __device__ static constexpr int smem_out(int n) { return (TA + TM) * ((n + 31) & ~31) * kPitch + 9 * DK * 4; }
 };
 
 template <typename T, typename E, int DK, int NX, int TA, int TM, int TP, int MODE>
 __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant__ BwdTermArgs p) {
     constexpr int PITCH = DK * 2 + 16, KS = DK / 16, NT = DK / 8;
+    constexpr bool kRaw = sizeof(T) == 4;
     extern __shared__ __align__(128) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const int slab = blockIdx.y, head = slab % p.heads, n32 = (p.n + 31) & ~31;
     const int t0 = min(p.N, (int)blockIdx.x * p.tokens), t1 = min(p.N, t0 + p.tokens);
     const uint32_t sm = smem_u32(smem);
     float2* st_s = reinterpret_cast<float2*>(smem + (TA + TM) * n32 * PITCH);
+    float* wt_s = reinterpret_cast<float*>(st_s);
     pdl_wait_prior();
     pdl_release_next();
     {
@@ -466,6 +492,8 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
             const size_t off = ok ? ((size_t)slab * p.n + r) * p.d + ch * 8 : 0;
             cp_async16s(sm + (m * n32 + col_to_row(r)) * PITCH + ch * 16, src + off, ok ? 16 : 0);
         }
+        if (MODE == kRowsOut && p.wd)
+            for (int i = threadIdx.x; i < p.d * 9; i += 256) wt_s[(i % 9) * DK + i / 9] = Elem<T>::to_f32(static_cast<const T*>(p.wd)[(size_t)head * p.d * 9 + i]);
         if (MODE == kRowsKeyValue)
             for (int i = threadIdx.x; i < n32; i += 256)                  // (no such agent: its probabilities are zero)
                 st_s[i] = i < p.n ? p.agent_stats[(size_t)slab * p.n + i] : make_float2(INFINITY, 0.f);
@@ -480,7 +508,9 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
     const float c1 = p.scale * kLog2e;
     const uint32_t koff = sm + key_lane_offset<DK>(lane), voff = sm + val_lane_offset<DK>(lane);
     for (int tok = t0 + warp * 16; tok < t1; tok += 128) {
-        uint32_t xf[NX][KS][4], yf[NX][KS][4];
+        // operand rows: as terms, or (fp32) as they are, split when they are used: three terms of both do not fit in registers
+        uint32_t xf[kRaw ? 1 : NX][kRaw ? 1 : KS][4], yf[kRaw ? 1 : NX][kRaw ? 1 : KS][4];
+        float2 xr[kRaw ? KS : 1][4], yr[kRaw ? KS : 1][4];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const size_t off = (size_t)min(tok + h * 8 + g, t1 - 1) * p.d + 2 * t;
@@ -488,24 +518,26 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
             for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
-                    uint32_t xw = 0u, yw = 0u;
-                    if (ks * 16 + k * 8 + 2 * t < p.d) {
-                        xw = __ldg(reinterpret_cast<const uint32_t*>(x + off + ks * 16 + k * 8));
-                        yw = __ldg(reinterpret_cast<const uint32_t*>(y + off + ks * 16 + k * 8));
-                    }
+                    const bool in = ks * 16 + k * 8 + 2 * t < p.d;
                     if constexpr (NX == 1) {
-                        xf[0][ks][k * 2 + h] = xw;
-                        yf[0][ks][k * 2 + h] = yw;
+                        xf[0][ks][k * 2 + h] = in ? __ldg(reinterpret_cast<const uint32_t*>(x + off + ks * 16 + k * 8)) : 0u;
+                        yf[0][ks][k * 2 + h] = in && MODE != kRowsOut ? __ldg(reinterpret_cast<const uint32_t*>(y + off + ks * 16 + k * 8)) : 0u;
                     } else {
-                        uint32_t w[NX];
-                        float2 f = unpack2<T>(xw);
-                        split_pair<E, NX>(f.x, f.y, w);
+                        float2 fx = make_float2(0.f, 0.f), fy = fx;
+                        if (in) fx = load_pair<T>(x + off + ks * 16 + k * 8);
+                        if (in && MODE != kRowsOut) fy = load_pair<T>(y + off + ks * 16 + k * 8);
+                        if constexpr (kRaw) {
+                            xr[ks][k * 2 + h] = fx;
+                            yr[ks][k * 2 + h] = fy;
+                        } else {
+                            uint32_t w[NX];
+                            split_pair<E, NX>(fx.x, fx.y, w);
 #pragma unroll
-                        for (int i = 0; i < NX; ++i) xf[i][ks][k * 2 + h] = w[i];
-                        f = unpack2<T>(yw);
-                        split_pair<E, NX>(f.x, f.y, w);
+                            for (int i = 0; i < NX; ++i) xf[i][ks][k * 2 + h] = w[i];
+                            split_pair<E, NX>(fy.x, fy.y, w);
 #pragma unroll
-                        for (int i = 0; i < NX; ++i) yf[i][ks][k * 2 + h] = w[i];
+                            for (int i = 0; i < NX; ++i) yf[i][ks][k * 2 + h] = w[i];
+                        }
                     }
                 }
         }
@@ -533,12 +565,7 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                         for (int i = 0; i < 8; ++i)
                             if (i < left) bs[h][i] = Elem<T>::to_f32(bias[(size_t)(blk + 8 * t + i) * p.N + tk]) * kLog2e;
                     } else {
-                        const T* bp = bias + (size_t)tk * p.n + blk + 8 * t;
-                        uint4 w = make_uint4(0u, 0u, 0u, 0u);
-                        if (left > 0) w = p.n % 8 == 0 ? __ldg(reinterpret_cast<const uint4*>(bp)) : load_bias8_any(bp, bias_end);
-                        unpack16<T>(w, bs[h]);
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) bs[h][i] *= kLog2e;
+                        load_bias_row<T>(bias + (size_t)tk * p.n + blk + 8 * t, left, p.n, bias_end, bs[h]);
                     }
                 }
             }
@@ -548,7 +575,23 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
 #pragma unroll
                 for (int e = 0; e < 4; ++e) s[j][e] = dp[j][e] = 0.f;
 #pragma unroll
-            for (int ks = 0; ks < KS; ++ks)
+            for (int ks = 0; ks < KS; ++ks) {
+                uint32_t xt[NX][4], yt[NX][4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if constexpr (kRaw) {
+                        uint32_t w[NX];
+                        split_pair<E, NX>(xr[ks][q].x, xr[ks][q].y, w);
+#pragma unroll
+                        for (int k = 0; k < NX; ++k) xt[k][q] = w[k];
+                        if (MODE != kRowsOut) split_pair<E, NX>(yr[ks][q].x, yr[ks][q].y, w);
+#pragma unroll
+                        for (int k = 0; k < NX; ++k) yt[k][q] = w[k];
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < NX; ++k) { xt[k][q] = xf[k][ks][q]; yt[k][q] = yf[k][ks][q]; }
+                    }
+                }
 #pragma unroll
                 for (int j2 = 0; j2 < 2; ++j2) {
 #pragma unroll
@@ -558,22 +601,24 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
 #pragma unroll
                         for (int k = 0; k < NX; ++k)
                             if (TermPairs<TA, NX>::keep(i, k)) {
-                                mma_acc<E>(s[2 * j2], xf[k][ks], b[0], b[1]);
-                                mma_acc<E>(s[2 * j2 + 1], xf[k][ks], b[2], b[3]);
+                                mma_acc<E>(s[2 * j2], xt[k], b[0], b[1]);
+                                mma_acc<E>(s[2 * j2 + 1], xt[k], b[2], b[3]);
                             }
                     }
+                    if (MODE != kRowsOut)
 #pragma unroll
-                    for (int i = 0; i < TM; ++i) {
-                        uint32_t b[4];
-                        ldsm4(b, koff + ((TA + i) * n32 + blk + j2 * 16) * PITCH + ks * 32);
+                        for (int i = 0; i < TM; ++i) {
+                            uint32_t b[4];
+                            ldsm4(b, koff + ((TA + i) * n32 + blk + j2 * 16) * PITCH + ks * 32);
 #pragma unroll
-                        for (int k = 0; k < NX; ++k)
-                            if (TermPairs<TM, NX>::keep(i, k)) {
-                                mma_acc<E>(dp[2 * j2], yf[k][ks], b[0], b[1]);
-                                mma_acc<E>(dp[2 * j2 + 1], yf[k][ks], b[2], b[3]);
-                            }
-                    }
+                            for (int k = 0; k < NX; ++k)
+                                if (TermPairs<TM, NX>::keep(i, k)) {
+                                    mma_acc<E>(dp[2 * j2], yt[k], b[0], b[1]);
+                                    mma_acc<E>(dp[2 * j2 + 1], yt[k], b[2], b[3]);
+                                }
+                        }
                 }
+            }
             const int left = p.n - blk - 8 * t;
             if constexpr (MODE == kRowsStats) {
 #pragma unroll
@@ -596,6 +641,48 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                         rd[h] = fmaf(e, dp[i >> 1][2 * h + (i & 1)], rd[h]);
                     }
                 }
+            } else if constexpr (MODE == kRowsOut) {
+                uint32_t pt[TP][2][4];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float mx = m[h];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        float& v = s[i >> 1][2 * h + (i & 1)];
+                        v = i < left ? fmaf(v, c1, bs[h][i]) : -INFINITY;
+                        mx = fmaxf(mx, v);
+                    }
+                    mx = quad_max(mx);
+                    const float f = m[h] == -INFINITY ? 0.f : exp2f(m[h] - mx);
+                    m[h] = mx;
+                    l[h] *= f;
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) { o0[j][2 * h] *= f; o0[j][2 * h + 1] *= f; }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float p0 = fast_exp2(s[j][2 * h] - mx), p1 = fast_exp2(s[j][2 * h + 1] - mx);
+                        l[h] += p0 + p1;
+                        uint32_t w[TP];
+                        split_pair<E, TP>(p0, p1, w);
+#pragma unroll
+                        for (int i = 0; i < TP; ++i) pt[i][j >> 1][(j & 1) * 2 + h] = w[i];
+                    }
+                }
+#pragma unroll
+                for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+                    for (int c2 = 0; c2 < NT / 2; ++c2)
+#pragma unroll
+                        for (int i = 0; i < TM; ++i) {
+                            uint32_t b[4];
+                            ldsm4t(b, voff + ((TA + i) * n32 + blk + kk * 16) * PITCH + c2 * 32);
+#pragma unroll
+                            for (int k = 0; k < TP; ++k)
+                                if (TermPairs<TP, TM>::keep(k, i)) {
+                                    mma_acc<E>(o0[2 * c2], pt[k][kk], b[0], b[1]);
+                                    mma_acc<E>(o0[2 * c2 + 1], pt[k][kk], b[2], b[3]);
+                                }
+                        }
             } else {
                 uint32_t pt[TP][2][4], dt[TP][2][4];
                 float2 cs[8];
@@ -670,6 +757,29 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                 const float mm = quad_max(m[h]), f = m[h] == -INFINITY ? 0.f : exp2f(m[h] - mm);
                 const float tot = quad_sum(l[h] * f), dot = quad_sum(rd[h] * f);
                 if (t == 0 && tk < t1) p.tok_stats[(size_t)slab * p.N + tk] = make_float2(mm + log2f(tot), dot / tot);
+            } else if constexpr (MODE == kRowsOut) {
+                const float inv = 1.f / quad_sum(l[h]);
+                if (tk < t1) {
+                    const size_t off = ((size_t)slab * p.N + tk) * p.d + 2 * t;
+                    const int gy = tk / p.W, gx = tk - gy * p.W;
+#pragma unroll
+                    for (int j = 0; j < NT; ++j)
+                        if (j * 8 + 2 * t < p.d) {
+                            float2 v = make_float2(o0[j][2 * h] * inv, o0[j][2 * h + 1] * inv);
+                            if (p.wd)
+#pragma unroll
+                                for (int k = 0; k < 9; ++k) {
+                                    const int dy = k / 3 - 1, dx = k % 3 - 1;
+                                    if ((unsigned)(gy + dy) < (unsigned)p.H && (unsigned)(gx + dx) < (unsigned)p.W) {
+                                        const float2 u = load_pair<T>(y + (size_t)(tk + dy * p.W + dx) * p.d + j * 8 + 2 * t);
+                                        const float2 w = *reinterpret_cast<const float2*>(wt_s + k * DK + j * 8 + 2 * t);
+                                        v.x = fmaf(u.x, w.x, v.x);
+                                        v.y = fmaf(u.y, w.y, v.y);
+                                    }
+                                }
+                            *reinterpret_cast<float2*>(p.row0 + off + j * 8) = v;
+                        }
+                }
             } else if (tk < t1) {
                 const size_t off = ((size_t)slab * p.N + tk) * p.d + 2 * t;
 #pragma unroll

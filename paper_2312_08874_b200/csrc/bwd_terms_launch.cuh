@@ -33,7 +33,7 @@ template <typename K> inline cudaError_t bwd_launch(K kern, std::atomic<unsigned
 // sums of up to 64 agents of 64 channels): A rounded once to the element type, the probabilities and V_A two terms of it.
 template <typename T> struct TermsFull {
     using E = __nv_bfloat16;
-    static constexpr int NX = Elem<T>::kIsBf16 ? 1 : 2, TA = 3, TM = 3, TP = 3, NW = 8;
+    static constexpr int NX = sizeof(T) == 4 ? 3 : Elem<T>::kIsBf16 ? 1 : 2, TA = 3, TM = 3, TP = 3, NW = 8;
 };
 template <typename T> struct TermsMixed {
     using E = T;
@@ -51,24 +51,31 @@ template <typename T, typename C, int DK, int MODE> cudaError_t bwd_sums(const B
 template <typename T, int DK, int MODE> cudaError_t bwd_rows(const BwdTermArgs& a, const BwdTermLaunch& l) {
     using C = TermsFull<T>;
     static std::atomic<unsigned long long> done;
-    return bwd_launch(bwd_rows_kernel<T, typename C::E, DK, C::NX, C::TA, C::TM, C::TP, MODE>, done, a, l, 256, RowsShape<DK, C::TA, C::TM>::smem(a.n));
+    return bwd_launch(bwd_rows_kernel<T, typename C::E, DK, C::NX, C::TA, C::TM, C::TP, MODE>, done, a, l, 256, MODE == kRowsOut ? RowsShape<DK, C::TA, C::TM>::smem_out(a.n) : RowsShape<DK, C::TA, C::TM>::smem(a.n));
 }
 
-enum BwdTermStage { kTermForward, kTermStats, kTermBroadcast, kTermAggregate, kTermKeyValue, kTermQuery };
+enum BwdTermStage { kTermForward, kTermStats, kTermBroadcast, kTermAggregate, kTermKeyValue, kTermQuery, kTermOut };
+constexpr int kTermGradientsF32 = 80;      // fp32 inputs: the gradient kernels' accumulators and operand rows fit in registers up to here
 template <typename T, int DK> cudaError_t bwd_terms_stage(int stage, const BwdTermArgs& a, const BwdTermLaunch& l) {
-    switch (stage) {
-        case kTermForward:   return bwd_sums<T, TermsFull<T>, DK, kSumsForward>(a, l);
-        case kTermStats:     return bwd_rows<T, DK, kRowsStats>(a, l);
-        case kTermBroadcast: return bwd_sums<T, TermsFull<T>, DK, kSumsBroadcast>(a, l);
-        case kTermAggregate: return bwd_sums<T, TermsFull<T>, DK, kSumsAggregate>(a, l);
-        case kTermKeyValue:  return bwd_rows<T, DK, kRowsKeyValue>(a, l);
-        default:             return bwd_rows<T, DK, kRowsQuery>(a, l);
+    if (stage == kTermForward) return bwd_sums<T, TermsFull<T>, DK, kSumsForward>(a, l);
+    if constexpr (sizeof(T) == 4)
+        if (stage == kTermOut) return bwd_rows<T, DK, kRowsOut>(a, l);
+    if constexpr (sizeof(T) == 2 || DK <= kTermGradientsF32) {
+        switch (stage) {
+            case kTermStats:     return bwd_rows<T, DK, kRowsStats>(a, l);
+            case kTermBroadcast: return bwd_sums<T, TermsFull<T>, DK, kSumsBroadcast>(a, l);
+            case kTermAggregate: return bwd_sums<T, TermsFull<T>, DK, kSumsAggregate>(a, l);
+            case kTermKeyValue:  return bwd_rows<T, DK, kRowsKeyValue>(a, l);
+            case kTermQuery:     return bwd_rows<T, DK, kRowsQuery>(a, l);
+        }
     }
+    return cudaErrorInvalidValue;
 }
 #define AA_BWD_TERMS_DECLARE(DK) cudaError_t bwd_terms_##DK(int dtype, int stage, const BwdTermArgs& a, const BwdTermLaunch& l)
 #define AA_BWD_TERMS_DEFINE(DK)                                                                            \
     AA_BWD_TERMS_DECLARE(DK) {                                                                             \
-        return dtype == kBF16 ? bwd_terms_stage<__nv_bfloat16, DK>(stage, a, l) : bwd_terms_stage<__half, DK>(stage, a, l); \
+        return dtype == kBF16 ? bwd_terms_stage<__nv_bfloat16, DK>(stage, a, l)                            \
+               : dtype == kF16 ? bwd_terms_stage<__half, DK>(stage, a, l) : bwd_terms_stage<float, DK>(stage, a, l); \
     }
 AA_BWD_TERMS_DECLARE(32); AA_BWD_TERMS_DECLARE(48); AA_BWD_TERMS_DECLARE(64); AA_BWD_TERMS_DECLARE(80); AA_BWD_TERMS_DECLARE(96); AA_BWD_TERMS_DECLARE(128);
 cudaError_t bwd_terms_mixed(int dtype, const BwdTermArgs& a, const BwdTermLaunch& l);         // forward sums

@@ -237,7 +237,18 @@ struct BwdCall {
     BwdPlan plan_mma;                         // their tiling
     void* ws_terms;                           // term-split kernels (bwd_terms.cu) run the attention stages; null: they do not
 };
-// Gradient stages with fp32 operands split into 16-bit terms (16-bit inputs, any shape whose agents fit in shared memory)
+// fp32 forward pass with operands split into 16-bit terms
+struct TermsForward {
+    const float *q, *k, *v, *agents, *b1, *b2, *wd;      // agents: the caller's, or null (pooled)
+    float *a_ws, *va_ws, *out;
+    void* ws;                                            // terms_forward_bytes
+    int slabs, heads, H, W, d, n, p, sm_count;
+    float scale1, scale2;
+};
+bool terms_forward_eligible(int n, int d);
+size_t terms_forward_bytes(int slabs, int n, int d);
+cudaError_t launch_terms_forward(const TermsForward& c, cudaStream_t st);
+// Gradient stages with fp32 operands split into 16-bit terms (any shape whose agents fit in shared memory; fp32 inputs up to 80 channels)
 bool backward_terms_eligible(int dtype, int n, int d);
 size_t backward_terms_bytes(int slabs, int n, int N, int d);
 cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStream_t st);

@@ -4,6 +4,29 @@
 
 namespace aa {
 
+// Eight channels as loaded, and added to four pairs of sums.
+template <typename T> struct Raw8 { uint4 w[sizeof(T) / 2]; };
+template <typename T> __device__ __forceinline__ Raw8<T> ld_raw8(const T* p) {
+    Raw8<T> r;
+#pragma unroll
+    for (int i = 0; i < (int)sizeof(T) / 2; ++i) r.w[i] = __ldg(reinterpret_cast<const uint4*>(p) + i);
+    return r;
+}
+template <typename T> __device__ __forceinline__ void add_raw8(float2 (&acc)[4], const Raw8<T>& r) {
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            acc[2 * i] = fadd2(acc[2 * i], make_float2(__uint_as_float(r.w[i].x), __uint_as_float(r.w[i].y)));
+            acc[2 * i + 1] = fadd2(acc[2 * i + 1], make_float2(__uint_as_float(r.w[i].z), __uint_as_float(r.w[i].w)));
+        }
+    } else {
+        acc[0] = fadd2(acc[0], unpack2<T>(r.w[0].x));
+        acc[1] = fadd2(acc[1], unpack2<T>(r.w[0].y));
+        acc[2] = fadd2(acc[2], unpack2<T>(r.w[0].z));
+        acc[3] = fadd2(acc[3], unpack2<T>(r.w[0].w));
+    }
+}
+
 // One warp: mean of the window of agent (ay, ax) -> put(chunk, eight means) for every 8-channel chunk (fixed order, fp32).
 template <typename T, typename F>
 __device__ __forceinline__ void pool_window(const T* q, long long qst, int H, int W, int p, int agent, int d, F&& put) {
@@ -11,7 +34,7 @@ __device__ __forceinline__ void pool_window(const T* q, long long qst, int H, in
     const int ay = agent / p, ax = agent - ay * p;
     const int y0 = (ay * H) / p, y1 = ((ay + 1) * H + p - 1) / p, x0 = (ax * W) / p, x1 = ((ax + 1) * W + p - 1) / p;
     const int ww = x1 - x0, cnt = (y1 - y0) * ww;
-    // lanes = (token sub-lane, 16-byte chunk): a power of two of chunks, so that shuffles reduce over the sub-lanes
+    // lanes = (token sub-lane, 8-channel chunk): a power of two of chunks, so that shuffles reduce over the sub-lanes
     const int cpt = d / 8, cp2 = cpt <= 1 ? 1 : cpt <= 2 ? 2 : cpt <= 4 ? 4 : cpt <= 8 ? 8 : 16, tpl = 32 / cp2;
     const int ch = lane & (cp2 - 1), ts = lane / cp2;
     float2 acc[4];
@@ -20,21 +43,16 @@ __device__ __forceinline__ void pool_window(const T* q, long long qst, int H, in
     int wy = ts / ww, wx = ts - wy * ww;
     const T* base = q + ((size_t)y0 * W + x0) * qst + ch * 8;
     for (int i = ts; i < cnt; i += 8 * tpl) {
-        uint4 raw[8];
+        Raw8<T> raw[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            raw[u] = make_uint4(0u, 0u, 0u, 0u);
-            if (i + u * tpl < cnt && ch < cpt) raw[u] = __ldg(reinterpret_cast<const uint4*>(base + ((size_t)wy * W + wx) * qst));
+            raw[u] = Raw8<T>{};
+            if (i + u * tpl < cnt && ch < cpt) raw[u] = ld_raw8<T>(base + ((size_t)wy * W + wx) * qst);
             wx += tpl;
             while (wx >= ww) { wx -= ww; ++wy; }
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            acc[0] = fadd2(acc[0], unpack2<T>(raw[u].x));
-            acc[1] = fadd2(acc[1], unpack2<T>(raw[u].y));
-            acc[2] = fadd2(acc[2], unpack2<T>(raw[u].z));
-            acc[3] = fadd2(acc[3], unpack2<T>(raw[u].w));
-        }
+        for (int u = 0; u < 8; ++u) add_raw8<T>(acc, raw[u]);
     }
     for (int o = cp2; o < 32; o <<= 1)
 #pragma unroll
@@ -61,13 +79,7 @@ __device__ __forceinline__ void pool_chunk(const T* q, long long qst, int H, int
     for (int y = y0; y < y1; ++y) {
         const T* row = q + (long long)(y * W) * qst;
 #pragma unroll 4
-        for (int x = x0; x < x1; ++x) {
-            const uint4 raw = __ldg(reinterpret_cast<const uint4*>(row + x * qst));
-            acc[0] = fadd2(acc[0], unpack2<T>(raw.x));
-            acc[1] = fadd2(acc[1], unpack2<T>(raw.y));
-            acc[2] = fadd2(acc[2], unpack2<T>(raw.z));
-            acc[3] = fadd2(acc[3], unpack2<T>(raw.w));
-        }
+        for (int x = x0; x < x1; ++x) add_raw8<T>(acc, ld_raw8<T>(row + x * qst));
     }
     const float inv = 1.f / (float)((y1 - y0) * (x1 - x0));
     const float f[8] = {acc[0].x * inv, acc[0].y * inv, acc[1].x * inv, acc[1].y * inv,

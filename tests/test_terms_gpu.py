@@ -1,0 +1,53 @@
+"""fp32 tensors on the tensor cores (operands as sums of 16-bit terms) at the edges of their tiles, against the fp64 oracle."""
+import pytest
+import torch
+
+from paper_2312_08874_b200 import AA_PATH_AUTO, Workload, make_inputs
+from tests.parity_util import assert_close, make_module, oracle_forward, to_dev
+from tests.test_backward_gpu import check, run_both
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [
+    # batch heads H  W   d   pool bias  dwc
+    (1, 1, 4, 4, 8, 4, True, True),           # as many agents as tokens, channels padded from 8 to 32
+    (2, 1, 31, 33, 72, 3, True, True),        # one row group, unaligned bias rows, channels padded to 80
+    (1, 2, 37, 36, 64, 6, True, True),        # 36 agents: three row groups, ragged last tile
+    (1, 2, 20, 20, 48, 9, True, False),       # 81 agents: six row groups
+    (1, 1, 40, 41, 64, 16, True, True),       # 256 agents: two row blocks
+    (1, 1, 33, 12, 128, 8, True, True),       # 128 channels: two row blocks of 32 agents
+    (2, 1, 9, 300, 32, 5, False, True),
+    (40, 4, 7, 7, 40, 7, True, True),         # every token its own agent, many slabs
+]
+IDS = [f"B{c[0]}h{c[1]}_{c[2]}x{c[3]}_d{c[4]}_p{c[5]}" for c in SHAPES]
+
+
+def workload(case):
+    B, heads, H, W, d, pool, bias, dwc = case
+    return Workload("terms", B, heads, H, W, d, pool, "f32", bias, dwc, 1.0, seed=800 + H * W + d)
+
+
+@pytest.mark.parametrize("case", SHAPES, ids=IDS)
+def test_fp32_forward_matches_oracle(case):
+    w = workload(case)
+    inp = make_inputs(w, bias_std=0.5, dwc_std=0.2)
+    mod = make_module(w)
+    ws = mod.workspace(w.grid_h, w.grid_w, w.agents)
+    out = mod.forward(to_dev(inp["q"]), to_dev(inp["k"]), to_dev(inp["v"]), w.grid_h, w.grid_w, w.agents, b1=to_dev(inp["b1"]),
+                      b2=to_dev(inp["b2"]), dwc_weight=to_dev(inp["dwc"]), workspace=ws)
+    assert mod.last_launch_count() == 3
+    slabs = [(0, 0), (w.batch - 1, w.heads - 1)]
+    for (b, h), ref in zip(slabs, oracle_forward(w, inp, slabs=slabs)):
+        assert_close(out[b:b + 1, h:h + 1], ref, "f32", f"{case} slab {(b, h)}")
+    # the same with the agents handed in
+    agents, va = (t.clone() for t in mod.intermediates(ws, w.agents))
+    again = mod.forward(to_dev(inp["q"]), to_dev(inp["k"]), to_dev(inp["v"]), w.grid_h, w.grid_w, w.agents, agents=agents, b1=to_dev(inp["b1"]),
+                        b2=to_dev(inp["b2"]), dwc_weight=to_dev(inp["dwc"]))
+    assert torch.equal(out, again) and bool(torch.isfinite(va).all())
+
+
+@pytest.mark.parametrize("case", [c for c in SHAPES if c[4] <= 80], ids=[i for i, c in zip(IDS, SHAPES) if c[4] <= 80])
+def test_fp32_backward_matches_oracle(case):
+    w = workload(case)
+    _, got, ref = run_both(w, make_inputs(w, bias_std=0.5, dwc_std=0.2), path=AA_PATH_AUTO)
+    check(got, ref, str(case))
