@@ -128,19 +128,19 @@ SumsPlan sums_plan(int dtype, int n, int d) {
         while (s.kg > 1 && (6 * s.rg * 16 + 2 * 6 * 32 * s.kg) * (dk * 2 + 16) + 2 * 32 * s.kg * 8 > 227 * 1024) s.kg /= 2;
     return s;
 }
-// Parts of the token axis for `slots` resident blocks; a block's start (agents' terms into shared memory) costs about 256 tokens.
-int token_parts(long long others, int N, int unit, int most, bool pow2, int slots) {
+// Parts of the token axis for `slots` resident blocks, of whole units of tokens.  A block takes `pass` tokens at a time, and its start
+// (agents' terms into shared memory) costs about 256.
+int token_parts(long long others, int N, int unit, int pass, int most, bool pow2, int slots) {
     int best = 1;
     double cost = 0;
     for (int c = 1; c <= most; c = pow2 ? 2 * c : c + 1) {
         const int tokens = ((N + c - 1) / c + unit - 1) / unit * unit;
-        if (c > 1 && (tokens < 2 * unit || (long long)tokens * (c - 1) >= N)) continue;
-        const double k = (double)((others * c + slots - 1) / slots) * (tokens + 256);
+        if (c > 1 && (long long)tokens * (c - 1) >= N) continue;
+        const double k = (double)((others * c + slots - 1) / slots) * ((tokens + pass - 1) / pass * pass + 256);
         if (c == 1 || k < cost) { best = c; cost = k; }
     }
     return best;
 }
-
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 
 template <typename T, typename E, int NT> cudaError_t launch_pool_terms(PoolArgs8 pa, void* a_t, ClearList cl, cudaStream_t st) {
@@ -186,7 +186,7 @@ cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStrea
     BwdTermLaunch l;
     l.stream = st;
     l.kg = a.rg == 1 ? 4 : a.rg == 2 ? 2 : 1;
-    const int parts = token_parts(c.slabs, a.N, 64, 8, true, 3 * c.sm_count);
+    const int parts = token_parts(c.slabs, a.N, 64, 64, 8, true, 3 * c.sm_count);
     a.tokens = ((a.N + parts - 1) / parts + 63) / 64 * 64;
     l.grid = dim3(parts, 1, c.slabs);
     l.cluster = parts;
@@ -215,15 +215,15 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
     BwdTermLaunch l;
     l.stream = st; l.kg = sp.kg;
     auto sums = [&](int which, bool cluster) {
-        const int parts = token_parts((long long)slabs * sp.rb, N, 64, cluster ? 8 : 64, cluster, c.sm_count);
+        const int parts = token_parts((long long)slabs * sp.rb, N, 64, 64, cluster ? 8 : 64, cluster, c.sm_count);
         a.tokens = ((N + parts - 1) / parts + 63) / 64 * 64;
         l.grid = dim3(parts, sp.rb, slabs);
         l.cluster = cluster ? parts : 0;
         return stage(dtype, d, which, a, l);
     };
     auto rows = [&](int which) {
-        const int parts = token_parts(slabs, N, 128, 512, false, c.sm_count);
-        a.tokens = ((N + parts - 1) / parts + 127) / 128 * 128;
+        const int parts = token_parts(slabs, N, 16, 128, 512, false, c.sm_count);
+        a.tokens = ((N + parts - 1) / parts + 15) / 16 * 16;
         l.grid = dim3(parts, slabs);
         l.cluster = 0;
         return stage(dtype, d, which, a, l);
@@ -272,15 +272,15 @@ cudaError_t launch_terms_forward(const TermsForward& c, cudaStream_t st) {
     BwdTermLaunch l;
     l.stream = st; l.kg = sp.kg;
     a.x = c.k; a.y = c.v; a.bias = c.b1; a.scale = c.scale1; a.outer0 = c.va_ws;
-    int parts = token_parts((long long)c.slabs * sp.rb, N, 64, 8, true, c.sm_count);
+    int parts = token_parts((long long)c.slabs * sp.rb, N, 64, 64, 8, true, c.sm_count);
     a.tokens = ((N + parts - 1) / parts + 63) / 64 * 64;
     l.grid = dim3(parts, sp.rb, c.slabs);
     l.cluster = parts;
     e = stage(kF32, c.d, kTermForward, a, l);
     if (e != cudaSuccess) return e;
     a.x = c.q; a.y = c.v; a.bias = c.b2; a.scale = c.scale2; a.m_t = w + terms; a.row0 = c.out; a.wd = c.wd;
-    parts = token_parts(c.slabs, N, 128, 512, false, c.sm_count);
-    a.tokens = ((N + parts - 1) / parts + 127) / 128 * 128;
+    parts = token_parts(c.slabs, N, 16, 128, 512, false, c.sm_count);
+    a.tokens = ((N + parts - 1) / parts + 15) / 16 * 16;
     l.grid = dim3(parts, c.slabs);
     l.cluster = 0;
     return stage(kF32, c.d, kTermOut, a, l);

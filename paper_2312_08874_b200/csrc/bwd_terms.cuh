@@ -750,6 +750,51 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                     }
             }
         }
+        if constexpr (MODE == kRowsOut) {
+            // neighbouring threads swap halves of two 8-channel tiles: then a thread has four channels of tile j + (t & 1) of both rows,
+            // and the eighteen 16-byte loads of its two depthwise windows are in flight at once
+            const bool odd = t & 1;
+            bool in[2][9];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float inv = 1.f / quad_sum(l[h]);
+#pragma unroll
+                for (int j = 0; j < NT; ++j) { o0[j][2 * h] *= inv; o0[j][2 * h + 1] *= inv; }
+                const int tk = tok + h * 8 + g, gy = tk / p.W, gx = tk - gy * p.W;
+#pragma unroll
+                for (int k = 0; k < 9; ++k) in[h][k] = p.wd && tk < t1 && (unsigned)(gy + k / 3 - 1) < (unsigned)p.H && (unsigned)(gx + k % 3 - 1) < (unsigned)p.W;
+            }
+#pragma unroll
+            for (int j = 0; j < NT; j += 2) {
+                const int ch = 8 * (j + (t & 1)) + 4 * (t >> 1);
+                const bool live = ch < p.d;
+                float4 u[2][9];
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int k = 0; k < 9; ++k) {
+                        u[h][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (in[h][k] && live) u[h][k] = __ldg(reinterpret_cast<const float4*>(y + (size_t)(tok + h * 8 + g + (k / 3 - 1) * p.W + k % 3 - 1) * p.d + ch));
+                    }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float sx = odd ? o0[j][2 * h] : o0[j + 1][2 * h], sy = odd ? o0[j][2 * h + 1] : o0[j + 1][2 * h + 1];
+                    const float rx = __shfl_xor_sync(0xffffffffu, sx, 1), ry = __shfl_xor_sync(0xffffffffu, sy, 1);
+                    float4 v = odd ? make_float4(rx, ry, o0[j + 1][2 * h], o0[j + 1][2 * h + 1]) : make_float4(o0[j][2 * h], o0[j][2 * h + 1], rx, ry);
+                    if (p.wd)
+#pragma unroll
+                        for (int k = 0; k < 9; ++k) {
+                            const float4 w = *reinterpret_cast<const float4*>(wt_s + k * DK + ch);
+                            v.x = fmaf(u[h][k].x, w.x, v.x);
+                            v.y = fmaf(u[h][k].y, w.y, v.y);
+                            v.z = fmaf(u[h][k].z, w.z, v.z);
+                            v.w = fmaf(u[h][k].w, w.w, v.w);
+                        }
+                    if (live && tok + h * 8 + g < t1) *reinterpret_cast<float4*>(p.row0 + ((size_t)slab * p.N + tok + h * 8 + g) * p.d + ch) = v;
+                }
+            }
+            continue;
+        }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int tk = tok + h * 8 + g;
@@ -757,29 +802,6 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                 const float mm = quad_max(m[h]), f = m[h] == -INFINITY ? 0.f : exp2f(m[h] - mm);
                 const float tot = quad_sum(l[h] * f), dot = quad_sum(rd[h] * f);
                 if (t == 0 && tk < t1) p.tok_stats[(size_t)slab * p.N + tk] = make_float2(mm + log2f(tot), dot / tot);
-            } else if constexpr (MODE == kRowsOut) {
-                const float inv = 1.f / quad_sum(l[h]);
-                if (tk < t1) {
-                    const size_t off = ((size_t)slab * p.N + tk) * p.d + 2 * t;
-                    const int gy = tk / p.W, gx = tk - gy * p.W;
-#pragma unroll
-                    for (int j = 0; j < NT; ++j)
-                        if (j * 8 + 2 * t < p.d) {
-                            float2 v = make_float2(o0[j][2 * h] * inv, o0[j][2 * h + 1] * inv);
-                            if (p.wd)
-#pragma unroll
-                                for (int k = 0; k < 9; ++k) {
-                                    const int dy = k / 3 - 1, dx = k % 3 - 1;
-                                    if ((unsigned)(gy + dy) < (unsigned)p.H && (unsigned)(gx + dx) < (unsigned)p.W) {
-                                        const float2 u = load_pair<T>(y + (size_t)(tk + dy * p.W + dx) * p.d + j * 8 + 2 * t);
-                                        const float2 w = *reinterpret_cast<const float2*>(wt_s + k * DK + j * 8 + 2 * t);
-                                        v.x = fmaf(u.x, w.x, v.x);
-                                        v.y = fmaf(u.y, w.y, v.y);
-                                    }
-                                }
-                            *reinterpret_cast<float2*>(p.row0 + off + j * 8) = v;
-                        }
-                }
             } else if (tk < t1) {
                 const size_t off = ((size_t)slab * p.N + tk) * p.d + 2 * t;
 #pragma unroll
