@@ -202,9 +202,10 @@ __device__ __forceinline__ void agg_merge(const AggCta<T>& c, unsigned char* sme
     const int nsrc = csize * KG, share = (rows - crank + csize - 1) / csize;
     if ((int)threadIdx.x < share) {
         const int r = crank + threadIdx.x * csize;
-        float m[8 * KG], l[8 * KG], mm = -INFINITY, tot = 0.f;
+        constexpr int kSrc = KG == 1 ? 16 : 32;                               // at most
+        float m[kSrc], l[kSrc], mm = -INFINITY, tot = 0.f;
 #pragma unroll
-        for (int q = 0; q < 8 * KG; ++q) {
+        for (int q = 0; q < kSrc; ++q) {
             m[q] = 0.f; l[q] = 0.f;
             if (q < nsrc) {
                 const float2 v = ld_dsmem_f32x2(ml0 + ((q % KG) * c.rg * 16 + r) * 8, q / KG);
@@ -212,16 +213,16 @@ __device__ __forceinline__ void agg_merge(const AggCta<T>& c, unsigned char* sme
             }
         }
 #pragma unroll
-        for (int q = 0; q < 8 * KG; ++q)
+        for (int q = 0; q < kSrc; ++q)
             if (l[q] > 0.f) mm = fmaxf(mm, m[q]);
 #pragma unroll
-        for (int q = 0; q < 8 * KG; ++q) {
+        for (int q = 0; q < kSrc; ++q) {
             m[q] = l[q] > 0.f ? fast_exp2(m[q] - mm) : (l[q] == 0.f ? 0.f : l[q]);      // (a NaN sum stays one)
             tot += l[q] * m[q];
         }
         const float inv = 1.f / tot;
 #pragma unroll
-        for (int q = 0; q < 8 * KG; ++q)
+        for (int q = 0; q < kSrc; ++q)
             if (q < nsrc) wt[threadIdx.x * nsrc + q] = m[q] * inv;
     }
     __syncthreads();

@@ -71,12 +71,15 @@ cudaError_t launch_tile_aggregate(int dtype, TileArgs a, int sm_count, bool depe
     a.b2 = nullptr;
     // Parts of the token axis (one block each, a cluster per slab).  Two blocks share an SM and hide each other's
     // latencies, so the best split is the one with the shortest blocks in the fewest waves; a block's start and merge count as
-    // 128 tokens.
+    // 128 tokens.  Clusters of sixteen are for few slabs with long token axes (eight slabs of 8775 tokens: 42 us in eights, 28 us):
+    // two such blocks share an SM, so that a cluster asks for eight SMs of one GPC.
     int best = 1;
     long long best_cost = 0;
-    for (int c = 1; c <= 8; c *= 2) {
+    const int smem = agg_smem(dk.dk, a.kg, 8);
+    for (int c = 1; c <= 16; c *= 2) {
         const int tokens = up32((a.N + c - 1) / c);
         if (c > 1 && (tokens < 64 || c * a.kg > 32)) break;
+        if (c == 16 && (a.slabs * rb > 8 || smem > 112 * 1024)) break;
         const long long blocks = (long long)a.slabs * rb * c;
         const long long cost = ((blocks + 2LL * sm_count - 1) / (2LL * sm_count)) * (tokens + 128LL);
         if (c == 1 || cost < best_cost) { best = c; best_cost = cost; }
@@ -86,7 +89,7 @@ cudaError_t launch_tile_aggregate(int dtype, TileArgs a, int sm_count, bool depe
     l.grid = dim3(best, rb, a.slabs);
     l.threads = 256;
     l.cluster = best;
-    l.smem = agg_smem(dk.dk, a.kg, 8);
+    l.smem = smem;
     l.dependent = dependent;
     l.stream = st;
     return dispatch(kTileAggregate, dtype, dk.dk, bias_kind(a.b1, bias_align(a.N)), a, l);
@@ -150,9 +153,12 @@ cudaError_t launch_tile_forward(int dtype, TileArgs a, int sm_count, bool one_ke
         return dispatch(kTileSlab, dtype, dk.dk, !a.b1 && !a.b2 ? 0 : a.b1 && a.b2 && a.N % 8 == 0 && a.n % 8 == 0 ? 1 : 2, a, l);
     }
     if (a.pool) {
-        const unsigned blocks = (unsigned)(((long long)a.slabs * a.n + 7) / 8);
-        if (dtype == kBF16) tile_pool_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(a);
-        else tile_pool_kernel<__half><<<blocks, 256, 0, st>>>(a);
+        // a warp per window, or (few windows, more than 32 tokens each) a block per window
+        const long long cells = (long long)a.slabs * a.n;
+        const bool wide = cells < 8LL * sm_count && a.N > 32 * a.n;
+        const unsigned blocks = (unsigned)(wide ? cells : (cells + 7) / 8);
+        if (dtype == kBF16) wide ? tile_pool_kernel<__nv_bfloat16, true><<<blocks, 256, 0, st>>>(a) : tile_pool_kernel<__nv_bfloat16, false><<<blocks, 256, 0, st>>>(a);
+        else wide ? tile_pool_kernel<__half, true><<<blocks, 256, 0, st>>>(a) : tile_pool_kernel<__half, false><<<blocks, 256, 0, st>>>(a);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         *launches += 1;

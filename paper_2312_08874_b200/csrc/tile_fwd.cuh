@@ -110,15 +110,33 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) tile_slab_kernel(const __gri
     bc_phase<T, DK, BIAS>(b, smem, NW);
 }
 
-template <typename T>
+// WIDE: the eight warps of a block share a window
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(256) tile_pool_kernel(const __grid_constant__ TileArgs p) {
     pdl_release_next();
-    const long long cell = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int warp = threadIdx.x >> 5;
+    const long long cell = WIDE ? blockIdx.x : (long long)blockIdx.x * 8 + warp;
     if (cell >= (long long)p.slabs * p.n) return;
     const int slab = (int)(cell / p.n), agent = (int)(cell - (long long)slab * p.n);
     T* a = static_cast<T*>(const_cast<void*>(p.a)) + (size_t)cell * p.d;
-    pool_window<T>(static_cast<const T*>(p.q) + tok_offset(p.lin, slab, p.heads, 0), p.lin.st, p.H, p.W, p.pool, agent, p.d,
-                   [&](int ch, const float (&f)[8]) { *reinterpret_cast<uint4*>(a + ch * 8) = pack16<T>(f); });
+    const T* q = static_cast<const T*>(p.q) + tok_offset(p.lin, slab, p.heads, 0);
+    if constexpr (WIDE) {
+        __shared__ __align__(16) float part[8][128];
+        pool_window<T>(q, p.lin.st, p.H, p.W, p.pool, agent, p.d, [&](int ch, const float (&f)[8]) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) part[warp][ch * 8 + i] = f[i];
+        }, warp, 8);
+        __syncthreads();
+        if ((int)threadIdx.x < p.d / 2) {
+            float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int w = 0; w < 8; ++w) s = fadd2(s, *reinterpret_cast<const float2*>(&part[w][2 * threadIdx.x]));
+            *reinterpret_cast<uint32_t*>(a + 2 * threadIdx.x) = pack2<T>(s.x, s.y);
+        }
+    } else {
+        pool_window<T>(q, p.lin.st, p.H, p.W, p.pool, agent, p.d,
+                       [&](int ch, const float (&f)[8]) { *reinterpret_cast<uint4*>(a + ch * 8) = pack16<T>(f); });
+    }
 }
 
 }  // namespace aa

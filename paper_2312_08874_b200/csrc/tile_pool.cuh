@@ -27,28 +27,28 @@ template <typename T> __device__ __forceinline__ void add_raw8(float2 (&acc)[4],
     }
 }
 
-// One warp: mean of the window of agent (ay, ax) -> put(chunk, eight means) for every 8-channel chunk (fixed order, fp32).
+// One warp (of `parts` that take turns; the shares add up): mean of the window of agent (ay, ax) -> put(chunk, eight means) for every 8-channel chunk (fixed order, fp32).
 template <typename T, typename F>
-__device__ __forceinline__ void pool_window(const T* q, long long qst, int H, int W, int p, int agent, int d, F&& put) {
+__device__ __forceinline__ void pool_window(const T* q, long long qst, int H, int W, int p, int agent, int d, F&& put, int part = 0, int parts = 1) {
     const int lane = threadIdx.x & 31;
     const int ay = agent / p, ax = agent - ay * p;
     const int y0 = (ay * H) / p, y1 = ((ay + 1) * H + p - 1) / p, x0 = (ax * W) / p, x1 = ((ax + 1) * W + p - 1) / p;
     const int ww = x1 - x0, cnt = (y1 - y0) * ww;
     // lanes = (token sub-lane, 8-channel chunk): a power of two of chunks, so that shuffles reduce over the sub-lanes
     const int cpt = d / 8, cp2 = cpt <= 1 ? 1 : cpt <= 2 ? 2 : cpt <= 4 ? 4 : cpt <= 8 ? 8 : 16, tpl = 32 / cp2;
-    const int ch = lane & (cp2 - 1), ts = lane / cp2;
+    const int ch = lane & (cp2 - 1), ts = lane / cp2, step = tpl * parts, t0 = ts + part * tpl;
     float2 acc[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) acc[k] = make_float2(0.f, 0.f);
-    int wy = ts / ww, wx = ts - wy * ww;
+    int wy = t0 / ww, wx = t0 - wy * ww;
     const T* base = q + ((size_t)y0 * W + x0) * qst + ch * 8;
-    for (int i = ts; i < cnt; i += 8 * tpl) {
+    for (int i = t0; i < cnt; i += 8 * step) {
         Raw8<T> raw[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             raw[u] = Raw8<T>{};
-            if (i + u * tpl < cnt && ch < cpt) raw[u] = ld_raw8<T>(base + ((size_t)wy * W + wx) * qst);
-            wx += tpl;
+            if (i + u * step < cnt && ch < cpt) raw[u] = ld_raw8<T>(base + ((size_t)wy * W + wx) * qst);
+            wx += step;
             while (wx >= ww) { wx -= ww; ++wy; }
         }
 #pragma unroll

@@ -1,0 +1,26 @@
+"""Token-wise tail of the backward pass (pooling, depthwise and filter gradients) at the edges of its tiles, against the fp64 oracle."""
+import pytest
+
+from paper_2312_08874_b200 import AA_PATH_AUTO, Workload, make_inputs
+from tests.test_backward_gpu import check, run_both
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [
+    # batch heads H   W   d   pool dtype
+    (1, 1, 3, 131, 40, 3, "bf16"),        # W one past the single-run halo, channels padded from 40 to 48
+    (1, 2, 5, 300, 64, 5, "f16"),         # the halo in three runs, unequal windows
+    (2, 1, 130, 9, 104, 4, "bf16"),       # seven channel groups
+    (3, 1, 8, 16, 16, 2, "f16"),          # exactly one tile, one channel group
+    (1, 1, 43, 3, 8, 3, "bf16"),          # one token past a tile, half a channel group
+    (160, 2, 9, 15, 80, 3, "bf16"),       # more slabs than resident blocks
+    (2, 2, 30, 41, 128, 6, "f16"),
+]
+
+
+@pytest.mark.parametrize("case", SHAPES, ids=[f"B{c[0]}h{c[1]}_{c[2]}x{c[3]}_d{c[4]}_p{c[5]}" for c in SHAPES])
+def test_tail_edges_match_oracle(case):
+    B, heads, H, W, d, pool, dtype = case
+    w = Workload("tail", B, heads, H, W, d, pool, dtype, True, True, 1.0, seed=600 + H * W + d)
+    _, got, ref = run_both(w, make_inputs(w, bias_std=0.5, dwc_std=0.2), path=AA_PATH_AUTO)
+    check(got, ref, str(case), tc=d == 64)
