@@ -103,6 +103,8 @@ __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_cons
     __syncthreads();
     tc_fence_after_sync();
     pp.tmem = s_tmem;
+    pdl_wait_prior();                                     // the agents come from the preceding kernel
+    pdl_release_next();
 
     const uint32_t sA = smem_u32(smem + OFF_A), ring = smem_u32(smem + OFF_RING);
     const size_t pf = partial_floats(g.rows_pad, 64);
@@ -218,13 +220,10 @@ __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_cons
 #pragma unroll
                     for (int k = 0; k < 32; ++k) if (k >= valid) sv[k] = -INFINITY;
                 }
-                float mx0 = fmaxf(sv[0], sv[1]), mx1 = fmaxf(sv[2], sv[3]), mx2 = fmaxf(sv[4], sv[5]), mx3 = fmaxf(sv[6], sv[7]);
+                float mx0 = sv[0], mx1 = sv[1];
 #pragma unroll
-                for (int k = 8; k < 32; k += 8) {
-                    mx0 = fmaxf(mx0, fmaxf(sv[k], sv[k + 1]));     mx1 = fmaxf(mx1, fmaxf(sv[k + 2], sv[k + 3]));
-                    mx2 = fmaxf(mx2, fmaxf(sv[k + 4], sv[k + 5])); mx3 = fmaxf(mx3, fmaxf(sv[k + 6], sv[k + 7]));
-                }
-                const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
+                for (int k = 2; k < 30; k += 4) { mx0 = max3(mx0, sv[k], sv[k + 1]); mx1 = max3(mx1, sv[k + 2], sv[k + 3]); }
+                const float mx = max3(mx0, mx1, fmaxf(sv[30], sv[31]));
                 if (mx > m_ref + kTau) {                       // also the first tile (m_ref = -inf)
                     corr = fast_exp2((m_ref - mx) * kLog2e);
                     resc = started;
@@ -325,6 +324,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) merge_umma_kernel(const float* __restrict__ partials, int parts, int rows_pad,
                                                          int n, int d, T* __restrict__ out) {
     const int slab = blockIdx.y;
+    pdl_wait_prior();
+    pdl_release_next();
     const size_t pf = partial_floats(rows_pad, 64);
     const float* base = partials + (size_t)slab * parts * pf;
     const int groups = d >> 2;                             // d is a multiple of 8
@@ -333,7 +334,7 @@ __global__ void __launch_bounds__(256) merge_umma_kernel(const float* __restrict
     if (r >= n || cg >= groups) return;
     float mx = -INFINITY, den = 0.f;
     float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 16
+#pragma unroll 8
     for (int q = 0; q < parts; ++q) {
         const float* pq = base + q * pf;
         const float mq = __ldcg(pq + r);
@@ -386,12 +387,10 @@ static cudaError_t launch_umma_t(const UmmaAggArgs& g, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     dim3 grid(g.a.splits, g.a.slabs);
-    kern<<<grid, NT, kSmemBytes, st>>>(g);
-    e = cudaGetLastError();
+    e = launch_dependent(kern, grid, NT, kSmemBytes, st, g);
     if (e != cudaSuccess) return e;
     dim3 mgrid((g.a.rows + 15) / 16, g.a.slabs);
-    merge_umma_kernel<T><<<mgrid, 256, 0, st>>>(g.a.partials, g.a.splits, g.rows_pad, g.a.rows, g.a.d, static_cast<T*>(g.a.out));
-    return cudaGetLastError();
+    return launch_dependent(merge_umma_kernel<T>, mgrid, 256, 0, st, (const float*)g.a.partials, g.a.splits, g.rows_pad, g.a.rows, g.a.d, static_cast<T*>(g.a.out));
 }
 
 // cudaErrorNotSupported: a tensor map could not be encoded; the caller falls back to the mma.sync kernel.

@@ -213,7 +213,8 @@ int do_aggregate(agent_attn_handle* h, const void* A, const void* K, const void*
         return AA_OK;
     }
     const AggPlan pl = plan_for(h, N, n);
-    cudaError_t e = cudaMemsetAsync(tickets, 0, (size_t)h->cfg.batch * h->cfg.heads * sizeof(unsigned), st);
+    cudaError_t e = cudaSuccess;
+    if (!umma) e = cudaMemsetAsync(tickets, 0, (size_t)h->cfg.batch * h->cfg.heads * sizeof(unsigned), st);
     if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "ticket reset failed: %s", cudaGetErrorString(e));
     AttnArgs a;
     memset(&a, 0, sizeof(a));

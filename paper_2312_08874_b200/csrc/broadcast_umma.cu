@@ -10,9 +10,13 @@
 //                         instruction stream delays the other).
 //   warps 0-15 "row warps": thread (query row, agent group g of 32 columns per step): online softmax over
 //                         the steps with its own running maximum, sum and accumulator O_g in tensor memory
-//                         (no reduction crosses threads inside the loop).  At the end of a tile the four
-//                         groups of a row exchange (max, sum), every thread combines 16 output channels from
-//                         the four accumulators, adds the depthwise 3x3 term, rounds once and stores.
+//                         (no reduction crosses threads inside the loop).  At the end of a tile a warp owns
+//                         32 rows x 16 channels in mma.sync accumulator layout: the depthwise 3x3 term by MMAs
+//                         with the filter as a diagonal operand (k = (tap of a pair, channel of eight); rows of
+//                         taps outside the grid are the address of zeros), while the last product is in flight;
+//                         then the four groups' accumulators, read in the same layout and weighted by the row's
+//                         (max, sum) exchange; rounded once and stored.  (With the depthwise term as 144 FMAs
+//                         and the combination per thread: 113 us for 16 slabs of a 128 x 128 grid; this way 100 us.)
 // The probabilities of a step overwrite, in place, the bias values that the same thread has just read (same
 // rows, same columns of the B2 stage), so P needs no buffer of its own; the room holds the V tokens of the
 // depthwise window instead: three runs of 130 consecutive tokens (the tile's own, and those one grid row above
@@ -37,7 +41,8 @@ constexpr int kTimeoutTile = 3, kTimeoutLoads = 4, kTimeoutRole = 6;
 // shared memory (bytes from a 1024-aligned base)
 constexpr int OFF_BAR = 0;
 constexpr int OFF_ML = 1024;                             // [4 groups][128 rows] (max, sum)
-constexpr int OFF_W = OFF_ML + 4 * 128 * 8;              // filter taps [9][64] fp32
+constexpr int OFF_WGT = OFF_ML + 4 * 128 * 8;            // [4 groups][128 rows] weights of the groups' accumulators
+constexpr int OFF_ZERO = OFF_WGT + 4 * 128 * 4;          // 16 zero bytes
 constexpr int OFF_A = 8192;                              // agents [256][128 B]
 constexpr int OFF_VA = OFF_A + 4 * kTile;                // agent features [256][128 B]
 constexpr int OFF_Q = OFF_VA + 4 * kTile;                // 2 x query tile [128][128 B]
@@ -45,8 +50,9 @@ constexpr int OFF_B2 = OFF_Q + 4 * kTile;                // 2 stages x (2 column
 constexpr int kHaloRows = 136;                           // 130 tokens of a run, rounded up to whole swizzle atoms
 constexpr int kHaloSeg = kHaloRows * 128;
 constexpr int OFF_H = OFF_B2 + 2 * 4 * kTile;            // 3 runs of V tokens [136][128 B]
-constexpr int kSmemBytes = OFF_H + 3 * kHaloSeg + 1024;
-static_assert(OFF_W + 9 * 64 * 4 <= OFF_A, "small buffers");
+constexpr int OFF_TAB = OFF_H + 3 * kHaloSeg;            // filter: [10 taps][64 channels] words, the weight in the half that the channel has in a pair
+constexpr int kSmemBytes = OFF_TAB + 10 * 64 * 4 + 1024;
+static_assert(OFF_ZERO + 16 <= OFF_A, "small buffers");
 static_assert(kSmemBytes <= 232448 && kSmemBytes > 116 * 1024, "one block per SM");
 
 // mbarriers                                   count          waiter
@@ -112,6 +118,8 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
     __syncthreads();
     tc_fence_after_sync();
     pp.tmem = s_tmem;
+    pdl_wait_prior();                                     // A and V_A come from the preceding kernels
+    pdl_release_next();
 
     const uint32_t sA = smem_u32(smem + OFF_A), sVA = smem_u32(smem + OFF_VA), sQ = smem_u32(smem + OFF_Q);
     const uint32_t sB2 = smem_u32(smem + OFF_B2), sH = smem_u32(smem + OFF_H);
@@ -211,19 +219,21 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
         const int row = 32 * (warp & 3) + lane;                // query row of the tile = tensor-memory lane
         const uint32_t lane_base = ((uint32_t)(32 * (warp & 3))) << 16;
         const uint32_t tO = pp.tmem + TM_O + 64 * gq + lane_base;
-        float* sW = reinterpret_cast<float*>(smem + OFF_W);
+        float* sWgt = reinterpret_cast<float*>(smem + OFF_WGT);
+        uint32_t* sTab = reinterpret_cast<uint32_t*>(smem + OFF_TAB);
+        const int lg = lane >> 2, lt = lane & 3;               // mma.sync coordinates
         float2* sML = reinterpret_cast<float2*>(smem + OFF_ML);
         const int H = p.H, W = p.W;
         const int c0 = 16 * gq;                                // this thread's output channels
-        const int nch = max(0, min(16, d - c0));               // 0, 8 or 16
         // set-up: filter taps, zero rows of V_A past the last agent (0 * NaN is not 0)
         if (has_dwc) {
-            const T* w = static_cast<const T*>(p.dwc_w) + (size_t)head * d * 9;
-            for (int e = tid; e < 9 * 64; e += NROW) {
+            const uint16_t* w = static_cast<const uint16_t*>(p.dwc_w) + (size_t)head * d * 9;
+            for (int e = tid; e < 10 * 64; e += NROW) {
                 const int tap = e >> 6, ch = e & 63;
-                sW[e] = ch < d ? Elem<T>::to_f32(w[ch * 9 + tap]) : 0.f;
+                sTab[e] = tap < 9 && ch < d ? (uint32_t)w[ch * 9 + tap] << (16 * (ch & 1)) : 0u;
             }
         }
+        if (tid < 4) reinterpret_cast<uint32_t*>(smem + OFF_ZERO)[tid] = 0u;
         pipe_wait_one(pp, BAR_AG, kTimeoutLoads);
         for (int e = tid; e < (128 * MB - n) * 8; e += NROW)
             *(reinterpret_cast<uint4*>(smem + OFF_VA + (n + (e >> 3)) * 128) + (e & 7)) = make_uint4(0u, 0u, 0u, 0u);
@@ -277,13 +287,10 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
 #pragma unroll
                         for (int k = 0; k < 32; ++k) if (k >= valid) sv[k] = -INFINITY;
                     }
-                    float mx0 = fmaxf(sv[0], sv[1]), mx1 = fmaxf(sv[2], sv[3]), mx2 = fmaxf(sv[4], sv[5]), mx3 = fmaxf(sv[6], sv[7]);
+                    float mx0 = sv[0], mx1 = sv[1];
 #pragma unroll
-                    for (int k = 8; k < 32; k += 8) {
-                        mx0 = fmaxf(mx0, fmaxf(sv[k], sv[k + 1]));     mx1 = fmaxf(mx1, fmaxf(sv[k + 2], sv[k + 3]));
-                        mx2 = fmaxf(mx2, fmaxf(sv[k + 4], sv[k + 5])); mx3 = fmaxf(mx3, fmaxf(sv[k + 6], sv[k + 7]));
-                    }
-                    const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
+                    for (int k = 2; k < 30; k += 4) { mx0 = max3(mx0, sv[k], sv[k + 1]); mx1 = max3(mx1, sv[k + 2], sv[k + 3]); }
+                    const float mx = max3(mx0, mx1, fmaxf(sv[30], sv[31]));
                     if (mx > m_ref + kTau) {                   // also the first step (m_ref = -inf)
                         corr = fast_exp2((m_ref - mx) * kLog2e);
                         resc = started;
@@ -330,84 +337,102 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
                 tc_fence_before_sync();
                 pipe_arrive(pp, BAR_P_FULL);
             }
-            // depthwise 3x3 term for this thread's 16 channels of its token, while the last product is in flight
-            float2 dw[8];
+            // depthwise 3x3 term of this warp's 32 rows x 16 channels, while the last product is in flight
+            float o[2][2][4];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) dw[k] = make_float2(0.f, 0.f);
+            for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                for (int jj = 0; jj < 2; ++jj)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) o[mt][jj][e] = 0.f;
+            const int tile0 = (i0 + i) * QT + 32 * (warp & 3);
             if (has_dwc) {
-                // tap (u, v) of this thread's token sits at row (row + v) of run u; taps outside the grid
-                // (or in another slab, or past the head dim) contribute nothing
+                uint32_t in[2];                                // per 16-row tile, bit k: window position k of this lane's row lies in the grid
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt) {
+                    const int tk = tile0 + 16 * mt + (lane & 15), y = (int)((unsigned)tk / (unsigned)W), x = tk - y * W;
+                    in[mt] = 0x1ffu & (x == 0 ? ~0x49u : ~0u) & (x == W - 1 ? ~0x124u : ~0u) & (y == 0 ? ~7u : ~0u) & (y == H - 1 ? ~0x1c0u : ~0u);
+                    if (tk >= N) in[mt] = 0u;
+                }
                 pipe_wait_one(pp, BAR_H_FULL, kTimeoutLoads);
-                const int tk = min(tok, N - 1);
-                const int y = tk / W, x = tk - y * W;
-                const bool live = tok < N && nch > 0;
+                const uint32_t zero = smem_u32(smem + OFF_ZERO);
+                const uint32_t* tab = lt == (lg >> 1) ? sTab + c0 + lg : reinterpret_cast<const uint32_t*>(smem + OFF_ZERO);
+                const int tstep = lt == (lg >> 1) ? 64 : 0, jstep = lt == (lg >> 1) ? 8 : 0;
 #pragma unroll
-                for (int u = 0; u < 3; ++u) {
-                    const int yy = y + u - 1;
-                    const bool rowok = live && yy >= 0 && yy < H;
+                for (int pr = 0; pr < 5; ++pr) {
+                    // lanes 0-15 address tap 2 pr, lanes 16-31 tap 2 pr + 1 (the tenth: weights zero)
+                    const int ka = 2 * pr, kb = pr < 4 ? 2 * pr + 1 : 8;
+                    const int u = lane < 16 ? ka / 3 : kb / 3, v = lane < 16 ? ka % 3 : kb % 3;
+                    uint32_t w[2][2];
 #pragma unroll
-                    for (int v = 0; v < 3; ++v) {
-                        const int xx = x + v - 1;
-                        const bool ok = rowok && xx >= 0 && xx < W;
-                        const int r = row + v;
-                        const unsigned char* src = smem + OFF_H + u * kHaloSeg + r * 128;
-                        const float4* wt = reinterpret_cast<const float4*>(sW + (u * 3 + v) * 64 + c0);
+                    for (int jj = 0; jj < 2; ++jj) {
+                        w[jj][0] = tab[2 * pr * tstep + jj * jstep];
+                        w[jj][1] = tab[(2 * pr + 1) * tstep + jj * jstep];
+                    }
 #pragma unroll
-                        for (int hh = 0; hh < 2; ++hh) {
-                            uint4 rr = *reinterpret_cast<const uint4*>(src + ((((c0 >> 3) + hh) ^ (r & 7)) << 4));
-                            if (!ok || (hh == 1 && nch <= 8)) rr = make_uint4(0u, 0u, 0u, 0u);
-                            const float4 w0 = wt[2 * hh], w1 = wt[2 * hh + 1];
-                            dw[4 * hh + 0] = ffma2(make_float2(w0.x, w0.y), unpack2<T>(rr.x), dw[4 * hh + 0]);
-                            dw[4 * hh + 1] = ffma2(make_float2(w0.z, w0.w), unpack2<T>(rr.y), dw[4 * hh + 1]);
-                            dw[4 * hh + 2] = ffma2(make_float2(w1.x, w1.y), unpack2<T>(rr.z), dw[4 * hh + 2]);
-                            dw[4 * hh + 3] = ffma2(make_float2(w1.z, w1.w), unpack2<T>(rr.w), dw[4 * hh + 3]);
+                    for (int mt = 0; mt < 2; ++mt) {
+                        // tap (u, v) of a row sits at row (row + v) of run u
+                        const int r = 32 * (warp & 3) + 16 * mt + (lane & 15) + v;
+                        const bool ok = in[mt] >> (3 * u + v) & 1;
+                        const uint32_t src = sH + u * kHaloSeg + r * 128;
+#pragma unroll
+                        for (int jj = 0; jj < 2; ++jj) {
+                            uint32_t f[4];
+                            const uint32_t addr = ok ? src + (((2 * gq + jj) ^ (r & 7)) << 4) : zero;
+                            asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                                         : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3]) : "r"(addr) : "memory");
+                            mma16816<T>(o[mt][jj], f, w[jj][0], w[jj][1]);
                         }
                     }
                 }
                 pipe_arrive(pp, BAR_H_EMPTY);
             }
+            // weights of the row's four accumulators (the four warps of a row quarter meet)
             sML[gq * 128 + row] = make_float2(started ? m_ref : -INFINITY, started ? l : 0.f);
-            pipe_wait_one(pp, BAR_PV, kTimeoutTile);
-            tc_fence_after_sync();
-            asm volatile("bar.sync 1, %0;\n" ::"n"(NROW) : "memory");
+            asm volatile("bar.sync %0, 128;\n" ::"r"(2 + (warp & 3)) : "memory");
             {
                 float2 ml[4];
-                float mm = -INFINITY;
+                float mm = -INFINITY, den = 0.f;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) { ml[q] = sML[q * 128 + row]; mm = fmaxf(mm, ml[q].x); }
-                float wgt[4], den = 0.f;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    wgt[q] = fast_exp2((ml[q].x - mm) * kLog2e);        // exp2(-inf) = 0 for a group without agents
-                    den += wgt[q] * ml[q].y;
-                }
-                float acc[16];
-#pragma unroll
-                for (int k = 0; k < 16; ++k) acc[k] = 0.f;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    uint32_t ro[16];
-                    tmem_ld16(pp.tmem + TM_O + 64 * q + c0 + lane_base, ro);
-                    tmem_ld_wait();
-                    if (ml[q].y > 0.f) {                               // uniform enough: skip accumulators never written
-#pragma unroll
-                        for (int k = 0; k < 16; ++k) acc[k] = fmaf(wgt[q], __uint_as_float(ro[k]), acc[k]);
-                    }
-                }
-                tc_fence_before_sync();
-                const float inv = 1.f / den;
-                if (tok < N && nch > 0) {
-                    float o8[8];
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) o8[k] = fmaf(acc[k], inv, (k & 1) ? dw[k >> 1].y : dw[k >> 1].x);
-                    *reinterpret_cast<uint4*>(gO + (size_t)tok * so + c0) = pack16<T>(o8);
-                    if (nch > 8) {
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) o8[k] = fmaf(acc[8 + k], inv, (k & 1) ? dw[4 + (k >> 1)].y : dw[4 + (k >> 1)].x);
-                        *(reinterpret_cast<uint4*>(gO + (size_t)tok * so + c0) + 1) = pack16<T>(o8);
-                    }
-                }
+                for (int q = 0; q < 4; ++q) den += fast_exp2((ml[q].x - mm) * kLog2e) * ml[q].y;      // exp2(-inf) = 0 for a group without agents
+                sWgt[gq * 128 + row] = started ? fast_exp2((m_ref - mm) * kLog2e) / den : 0.f;
             }
+            asm volatile("bar.sync %0, 128;\n" ::"r"(2 + (warp & 3)) : "memory");
+            pipe_wait_one(pp, BAR_PV, kTimeoutTile);
+            tc_fence_after_sync();
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+                const float* wg = sWgt + 32 * (warp & 3) + 16 * mt + lg;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (32 * q < n) {                          // (accumulators of groups without agents are never written)
+                        uint32_t ro[8];
+                        tmem_ld_16x256b_x2(pp.tmem + TM_O + 64 * q + c0 + lane_base + (16u * mt << 16), ro);
+                        const float w0 = wg[q * 128], w1 = wg[q * 128 + 8];
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int jj = 0; jj < 2; ++jj) {
+                            o[mt][jj][0] = fmaf(w0, __uint_as_float(ro[4 * jj]), o[mt][jj][0]);
+                            o[mt][jj][1] = fmaf(w0, __uint_as_float(ro[4 * jj + 1]), o[mt][jj][1]);
+                            o[mt][jj][2] = fmaf(w1, __uint_as_float(ro[4 * jj + 2]), o[mt][jj][2]);
+                            o[mt][jj][3] = fmaf(w1, __uint_as_float(ro[4 * jj + 3]), o[mt][jj][3]);
+                        }
+                    }
+            }
+            tc_fence_before_sync();
+            // neighbouring threads swap the channels of one 8-channel tile: eight bytes a thread, a row's 32 bytes a store
+            const int ch = c0 + 8 * (lt & 1) + 4 * (lt >> 1);
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) {
+                    const uint32_t wa = pack2<T>(o[mt][0][2 * hh], o[mt][0][2 * hh + 1]), wb = pack2<T>(o[mt][1][2 * hh], o[mt][1][2 * hh + 1]);
+                    const uint32_t got = __shfl_xor_sync(0xffffffffu, (lt & 1) ? wa : wb, 1);
+                    const int to = tile0 + 16 * mt + 8 * hh + lg;
+                    if (to < N && ch < d) *reinterpret_cast<uint2*>(gO + (size_t)to * so + ch) = (lt & 1) ? make_uint2(got, wb) : make_uint2(wa, got);
+                }
         }
     }
     tc_fence_before_sync();
@@ -428,8 +453,7 @@ static cudaError_t launch_bc_umma_t(const UmmaBcArgs& g, int splits, cudaStream_
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     dim3 grid(splits, g.a.slabs);
-    kern<<<grid, NT, kSmemBytes, st>>>(g);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, NT, kSmemBytes, st, g);
 }
 
 // cudaErrorNotSupported: a tensor map could not be encoded.

@@ -82,12 +82,12 @@ __global__ void __launch_bounds__(256) bwd_pool_terms_kernel(PoolArgs8 pa, E* ds
             put((size_t)cell * d + ch * 8, f);
             return;
         }
-        pool_chunk<T>(q + (size_t)slab * H * W * d + ch * 8, d, H, W, pool, agent, [&](const float (&f)[8]) { put((size_t)cell * d + ch * 8, f); });
+        pool_chunk<T>(q + (size_t)slab * H * W * d + ch * 8, d, H, W, pool, pool, agent, [&](const float (&f)[8]) { put((size_t)cell * d + ch * 8, f); });
     } else {
         const long long cell = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
         if (cell >= (long long)slabs * n) return;
         const int slab = (int)(cell / n), agent = (int)(cell - (long long)slab * n);
-        pool_window<T>(q + (size_t)slab * H * W * d, d, H, W, pool, agent, d, [&](int ch, const float (&f)[8]) { put((size_t)cell * d + ch * 8, f); });
+        pool_window<T>(q + (size_t)slab * H * W * d, d, H, W, pool, pool, agent, d, [&](int ch, const float (&f)[8]) { put((size_t)cell * d + ch * 8, f); });
     }
 }
 

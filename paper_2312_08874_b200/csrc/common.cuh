@@ -114,6 +114,11 @@ __device__ __forceinline__ float fast_exp2(float x) {       // ex2.approx: exp2(
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float d;
+    asm("max.f32 %0, %1, %2, %3;\n" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
 // packed pairs of fp32 (sm_100): d = a * b + c, a + b, a * b on both halves in one instruction.  (Same arithmetic
 // throughput as the scalar forms, half the issue slots; the intrinsics let the compiler keep the pairs in
 // adjacent registers.)

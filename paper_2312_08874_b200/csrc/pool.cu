@@ -1,10 +1,10 @@
 // Agent tokens by average pooling of Q over the token grid (text under Eq. 6: A = Pooling(Q)).
 //
-// One warp owns one pooled cell of one slab.  Its lanes are laid out as (token sub-lane, 16-byte
-// channel chunk), so a warp-wide load covers whole contiguous token rows of the window; sums are
-// kept in fp32 and reduced across the token sub-lanes in a fixed order (no atomics: results are
-// bit-reproducible).
-#include "common.cuh"
+// One warp owns one pooled cell of one slab.  Its lanes are laid out as (token sub-lane, channel chunk), so a warp-wide load covers
+// whole contiguous token rows of the window; sums are kept in fp32 and reduced across the token sub-lanes in a fixed order (no
+// atomics: results are bit-reproducible).  16-bit elements: eight loads in flight per lane (pool_window); reading Q is the bound (16
+// slabs of a 256 x 256 grid: 27.7 us with a division per load and four in flight, 24.5 us).
+#include "tile_pool.cuh"
 #include "kernels.h"
 
 namespace aa {
@@ -55,13 +55,26 @@ __global__ void __launch_bounds__(256) pool_kernel(PoolArgs p) {
     }
 }
 
+template <typename T>
+__global__ void __launch_bounds__(256) pool_window_kernel(PoolArgs p) {
+    pdl_wait_prior();                                              // (its output may still be read by the kernels before)
+    pdl_release_next();
+    const int n = p.ph * p.pw;
+    const long long cell = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (cell >= (long long)p.slabs * n) return;
+    const int slab = (int)(cell / n), agent = (int)(cell - (long long)slab * n);
+    T* a = static_cast<T*>(p.a) + (size_t)cell * p.d;
+    pool_window<T>(static_cast<const T*>(p.q) + tok_offset(p.lq, slab, p.heads, 0), p.lq.st, p.H, p.W, p.ph, p.pw, agent, p.d,
+                   [&](int ch, const float (&f)[8]) { *reinterpret_cast<uint4*>(a + ch * 8) = pack16<T>(f); });
+}
+
 cudaError_t launch_pool(int dtype, const PoolArgs& p, cudaStream_t st) {
     const long long cells = (long long)p.slabs * p.ph * p.pw;
     const unsigned blocks = (unsigned)((cells + 7) / 8);
     switch (dtype) {
         case kF32:  pool_kernel<float><<<blocks, 256, 0, st>>>(p); break;
-        case kBF16: pool_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(p); break;
-        case kF16:  pool_kernel<__half><<<blocks, 256, 0, st>>>(p); break;
+        case kBF16: pool_window_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(p); break;
+        case kF16:  pool_window_kernel<__half><<<blocks, 256, 0, st>>>(p); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -64,12 +64,6 @@ template <> struct Pair<__half> {
 // 16-bit formats, and probabilities are never negative.
 constexpr uint32_t kPairGe2 = 0x40004000u;
 
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-
 // Bounded wait for the phase of mbarrier i with the given parity (the caller derives the parity from its
 // loop counter).  On expiry the block's `dead` flag is set, every later wait of the block returns at once,
 // and `code` goes to the device status word: a logic error ends as a status code, never as a hang.

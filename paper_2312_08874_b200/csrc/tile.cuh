@@ -49,11 +49,6 @@ template <typename T> __device__ __forceinline__ void mma_set(float* c, const ui
 AA_MMA_FORMS(__nv_bfloat16, "bf16")
 AA_MMA_FORMS(__half, "f16")
 #undef AA_MMA_FORMS
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float d;
-    asm("max.f32 %0, %1, %2, %3;\n" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
 __device__ __forceinline__ void cp_async16s(uint32_t dst, const void* src, int src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }

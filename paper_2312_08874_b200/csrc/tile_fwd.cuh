@@ -88,12 +88,12 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) tile_slab_kernel(const __gri
                 const int cpt = p.d >> 3, items = (p.n - crank + csize - 1) / csize * cpt;
                 for (int i = threadIdx.x; i < items; i += NW * 32) {
                     const int agent = crank + i / cpt * csize, ch = i % cpt;
-                    pool_chunk<T>(q + ch * 8, p.lin.st, p.H, p.W, p.pool, agent,
+                    pool_chunk<T>(q + ch * 8, p.lin.st, p.H, p.W, p.pool, p.pool, agent,
                                   [&](const float (&f)[8]) { *reinterpret_cast<uint4*>(a + (size_t)agent * p.d + ch * 8) = pack16<T>(f); });
                 }
             } else {
                 for (int i = crank + warp * csize; i < p.n; i += csize * (NW))
-                    pool_window<T>(q, p.lin.st, p.H, p.W, p.pool, i, p.d,
+                    pool_window<T>(q, p.lin.st, p.H, p.W, p.pool, p.pool, i, p.d,
                                    [&](int ch, const float (&f)[8]) { *reinterpret_cast<uint4*>(a + (size_t)i * p.d + ch * 8) = pack16<T>(f); });
             }
             cluster_sync_all(csize);
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(256) tile_pool_kernel(const __grid_constant__ 
     const T* q = static_cast<const T*>(p.q) + tok_offset(p.lin, slab, p.heads, 0);
     if constexpr (WIDE) {
         __shared__ __align__(16) float part[8][128];
-        pool_window<T>(q, p.lin.st, p.H, p.W, p.pool, agent, p.d, [&](int ch, const float (&f)[8]) {
+        pool_window<T>(q, p.lin.st, p.H, p.W, p.pool, p.pool, agent, p.d, [&](int ch, const float (&f)[8]) {
 #pragma unroll
             for (int i = 0; i < 8; ++i) part[warp][ch * 8 + i] = f[i];
         }, warp, 8);
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(256) tile_pool_kernel(const __grid_constant__ 
             *reinterpret_cast<uint32_t*>(a + 2 * threadIdx.x) = pack2<T>(s.x, s.y);
         }
     } else {
-        pool_window<T>(q, p.lin.st, p.H, p.W, p.pool, agent, p.d,
+        pool_window<T>(q, p.lin.st, p.H, p.W, p.pool, p.pool, agent, p.d,
                        [&](int ch, const float (&f)[8]) { *reinterpret_cast<uint4*>(a + ch * 8) = pack16<T>(f); });
     }
 }

@@ -29,10 +29,10 @@ template <typename T> __device__ __forceinline__ void add_raw8(float2 (&acc)[4],
 
 // One warp (of `parts` that take turns; the shares add up): mean of the window of agent (ay, ax) -> put(chunk, eight means) for every 8-channel chunk (fixed order, fp32).
 template <typename T, typename F>
-__device__ __forceinline__ void pool_window(const T* q, long long qst, int H, int W, int p, int agent, int d, F&& put, int part = 0, int parts = 1) {
+__device__ __forceinline__ void pool_window(const T* q, long long qst, int H, int W, int ph, int pw, int agent, int d, F&& put, int part = 0, int parts = 1) {
     const int lane = threadIdx.x & 31;
-    const int ay = agent / p, ax = agent - ay * p;
-    const int y0 = (ay * H) / p, y1 = ((ay + 1) * H + p - 1) / p, x0 = (ax * W) / p, x1 = ((ax + 1) * W + p - 1) / p;
+    const int ay = agent / pw, ax = agent - ay * pw;
+    const int y0 = (ay * H) / ph, y1 = ((ay + 1) * H + ph - 1) / ph, x0 = (ax * W) / pw, x1 = ((ax + 1) * W + pw - 1) / pw;
     const int ww = x1 - x0, cnt = (y1 - y0) * ww;
     // lanes = (token sub-lane, 8-channel chunk): a power of two of chunks, so that shuffles reduce over the sub-lanes
     const int cpt = d / 8, cp2 = cpt <= 1 ? 1 : cpt <= 2 ? 2 : cpt <= 4 ? 4 : cpt <= 8 ? 8 : 16, tpl = 32 / cp2;
@@ -70,9 +70,9 @@ __device__ __forceinline__ void pool_window(const T* q, long long qst, int H, in
 
 // One thread: eight channels of one agent, for small windows (independent loads, no shuffles; fixed order, fp32).
 template <typename T, typename F>
-__device__ __forceinline__ void pool_chunk(const T* q, long long qst, int H, int W, int p, int agent, F&& put) {
-    const int ay = agent / p, ax = agent - ay * p;
-    const int y0 = (ay * H) / p, y1 = ((ay + 1) * H + p - 1) / p, x0 = (ax * W) / p, x1 = ((ax + 1) * W + p - 1) / p;
+__device__ __forceinline__ void pool_chunk(const T* q, long long qst, int H, int W, int ph, int pw, int agent, F&& put) {
+    const int ay = agent / pw, ax = agent - ay * pw;
+    const int y0 = (ay * H) / ph, y1 = ((ay + 1) * H + ph - 1) / ph, x0 = (ax * W) / pw, x1 = ((ax + 1) * W + pw - 1) / pw;
     float2 acc[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) acc[k] = make_float2(0.f, 0.f);
