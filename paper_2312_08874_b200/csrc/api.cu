@@ -463,7 +463,7 @@ static int forward_impl(agent_attn_handle* h, const void* Q, const void* K, cons
         return fail(h, AA_ERR_UNSUPPORTED,
                     "strided tensors need 16-bit elements and either d = 64, n <= 64, pooled agents and W <= 64, or d <= 64 and n a "
                     "multiple of 8 in 72..256");
-    if (h->cfg.path == AA_PATH_AUTO && h->cfg.dtype != AA_F32 && !cl.strided) {
+    if (h->cfg.path == AA_PATH_AUTO && h->cfg.dtype != AA_F32) {
         // long token grids with few agents: three streaming kernels, phase by phase over the batch
         const StreamPlan& sp = stream_plan_for(h, grid_h, grid_w, n_agents, A == nullptr);
         if (sp.ok) {
@@ -481,23 +481,28 @@ static int forward_impl(agent_attn_handle* h, const void* Q, const void* K, cons
             sa.tickets = reinterpret_cast<unsigned*>(ws + w.ticket_off);
             sa.status = h->d_status;
             sa.slabs = slabs; sa.heads = h->cfg.heads; sa.H = grid_h; sa.W = grid_w; sa.n = n_agents; sa.p = p;
-            sa.scale1 = h->scale1; sa.scale2 = h->scale2; sa.sm_count = h->sm_count; sa.plan = sp;
+            sa.scale1 = h->scale1; sa.scale2 = h->scale2; sa.sm_count = h->sm_count; sa.lin = cl.in; sa.lout = cl.out; sa.plan = sp;
+            sa.hf = sa.heads > 1 && cl.in.sh < cl.in.st;
             // the tensor maps depend on the pointers and the shape only: reuse them while both repeat
             const size_t key_bytes = offsetof(StreamArgs, tm_k);
+            bool maps = true;
             if (h->stream_args_valid && memcmp(&sa, &h->stream_args, key_bytes) == 0) {
                 sa = h->stream_args;
             } else {
-                if (!stream_make_maps(&sa)) return fail(h, AA_ERR_CUDA, "tensor map encoding failed");
-                h->stream_args = sa;
-                h->stream_args_valid = true;
+                maps = stream_make_maps(&sa);
+                if (!maps && !cl.strided) return fail(h, AA_ERR_CUDA, "tensor map encoding failed");
+                if (maps) h->stream_args = sa;
+                h->stream_args_valid = maps;
             }
             cudaError_t e = cudaSuccess;
-            h->launches = 0;
-            if (e == cudaSuccess && (h->stage_mask & 1u)) { e = launch_stream_prep(h->cfg.dtype, sa, st); h->launches++; }
-            if (e == cudaSuccess && (h->stage_mask & 2u)) { e = launch_stream_aggregate(h->cfg.dtype, sa, st); h->launches++; }
-            if (e == cudaSuccess && (h->stage_mask & 4u)) { e = launch_stream_broadcast(h->cfg.dtype, sa, st); h->launches++; }
-            if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "streaming launch failed: %s", cudaGetErrorString(e));
-            return AA_OK;
+            if (maps) {                           // (strides that no map expresses: the kernels below)
+                h->launches = 0;
+                if (e == cudaSuccess && (h->stage_mask & 1u)) { e = launch_stream_prep(h->cfg.dtype, sa, st); h->launches++; }
+                if (e == cudaSuccess && (h->stage_mask & 2u)) { e = launch_stream_aggregate(h->cfg.dtype, sa, st); h->launches++; }
+                if (e == cudaSuccess && (h->stage_mask & 4u)) { e = launch_stream_broadcast(h->cfg.dtype, sa, st); h->launches++; }
+                if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "streaming launch failed: %s", cudaGetErrorString(e));
+                return AA_OK;
+            }
         }
     }
     if (!A && (h->cfg.path == AA_PATH_QUEUE || (h->cfg.path == AA_PATH_AUTO && cl.strided && N >= 1024)) && h->cfg.dtype != AA_F32) {

@@ -188,6 +188,8 @@ struct StreamArgs {
     int slabs, heads, H, W, n, p;
     float scale1, scale2;
     int sm_count;
+    TokLayout lin, lout;       // of Q, K, V and of the output
+    int hf;                    // dimension order of their maps (heads before tokens)
     StreamPlan plan;
     alignas(64) CUtensorMap tm_k, tm_v, tm_b1, tm_q, tm_b2, tm_h, tm_a2, tm_va;
 };

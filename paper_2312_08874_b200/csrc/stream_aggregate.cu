@@ -155,8 +155,8 @@ __global__ void __launch_bounds__(NT, 1) stream_aggregate_kernel(const __grid_co
             for (int i = 0; i < first; ++i) {
                 const uint32_t bar = pipe_bar(pp, BAR_FULL + i), dst = ring + i * kStage;
                 mbar_arrive_expect_tx(bar, tx);
-                tma_load_3d(dst, &p.tm_k, 0, (t0 + i) * TK, slab, bar);
-                tma_load_3d(dst + kTile, &p.tm_v, 0, (t0 + i) * TK, slab, bar);
+                tma_load_tok(dst, &p.tm_k, p.hf, (t0 + i) * TK, head, slab / p.heads, bar);
+                tma_load_tok(dst + kTile, &p.tm_v, p.hf, (t0 + i) * TK, head, slab / p.heads, bar);
             }
             pdl_wait();
             if (has_bias)
@@ -167,8 +167,8 @@ __global__ void __launch_bounds__(NT, 1) stream_aggregate_kernel(const __grid_co
                 wait_spin(pp, BAR_EMPTY + s, (i / STAGES) - 1, kTimeoutRole);
                 const uint32_t bar = pipe_bar(pp, BAR_FULL + s), dst = ring + s * kStage;
                 mbar_arrive_expect_tx(bar, tx);
-                tma_load_3d(dst, &p.tm_k, 0, c0, slab, bar);
-                tma_load_3d(dst + kTile, &p.tm_v, 0, c0, slab, bar);
+                tma_load_tok(dst, &p.tm_k, p.hf, c0, head, slab / p.heads, bar);
+                tma_load_tok(dst + kTile, &p.tm_v, p.hf, c0, head, slab / p.heads, bar);
                 if (has_bias) tma_load_3d(dst + 2 * kTile, &p.tm_b1, 0, c0, head, bar);
             }
         }

@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(NT, 1) stream_broadcast_kernel(const __grid_co
                 for (int i = 0; i < min(T_, 2); ++i, ih.next()) {
                     const uint32_t bar = pipe_bar(pp, BAR_H_FULL + i);
                     mbar_arrive_expect_tx(bar, h_tx);
-                    tma_load_4d(sH + i * L.hsz + 1024, &p.tm_h, 0, -1, ih.tb * R - 1, ih.slab, bar);
+                    tma_load_grid(sH + i * L.hsz + 1024, &p.tm_h, p.hf, -1, ih.tb * R - 1, ih.slab % p.heads, ih.slab / p.heads, bar);
                 }
             pdl_wait();      // A, V_A, the padded B2 and the weight slices come from the preceding kernels
             int cur = -1, ord = -1;
@@ -174,13 +174,13 @@ __global__ void __launch_bounds__(NT, 1) stream_broadcast_kernel(const __grid_co
                 if (i >= 2) wait_spin(pp, BAR_QB_EMPTY + s2, (i >> 1) - 1, kTimeoutRole);
                 const uint32_t bar = pipe_bar(pp, BAR_QB_FULL + s2), dst = sQB + s2 * 2 * L.qsz;
                 mbar_arrive_expect_tx(bar, qb_tx);
-                tma_load_4d(dst, &p.tm_q, 0, -1, it.tb * R, it.slab, bar);
+                tma_load_grid(dst, &p.tm_q, p.hf, -1, it.tb * R, it.slab % p.heads, it.slab / p.heads, bar);
                 tma_load_4d(dst + L.qsz, &p.tm_b2, 0, -1, it.tb * R, p.b2 ? it.slab % p.heads : 0, bar);
                 if (has_dwc && i >= 2) {
                     wait_spin(pp, BAR_H_EMPTY + s2, (i >> 1) - 1, kTimeoutRole);
                     const uint32_t hb = pipe_bar(pp, BAR_H_FULL + s2);
                     mbar_arrive_expect_tx(hb, h_tx);
-                    tma_load_4d(sH + s2 * L.hsz + 1024, &p.tm_h, 0, -1, it.tb * R - 1, it.slab, hb);
+                    tma_load_grid(sH + s2 * L.hsz + 1024, &p.tm_h, p.hf, -1, it.tb * R - 1, it.slab % p.heads, it.slab / p.heads, hb);
                 }
             }
         }
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(NT, 1) stream_broadcast_kernel(const __grid_co
             const int rows = min(R, H - it.tb * R);
             const bool live = r < rows && xp >= 1 && xp <= W;
             const uint32_t tO = pp.tmem + TM_O + 64 * b + lane_base, tD = pp.tmem + TM_D + 64 * b + lane_base;
-            uint4* dst = reinterpret_cast<uint4*>(static_cast<T*>(p.out) + ((size_t)it.slab * N + (size_t)(it.tb * R + r) * W + (xp - 1)) * 64);
+            uint4* dst = reinterpret_cast<uint4*>(static_cast<T*>(p.out) + tok_offset(p.lout, it.slab, p.heads, (long long)(it.tb * R + r) * W + (xp - 1)));
             wait_par(pp, BAR_O_FULL + b, i >> 1, kTimeoutTile);
             if (has_dwc) wait_par(pp, BAR_D_FULL + b, i >> 1, kTimeoutTile);
             tc_fence_after_sync();
@@ -425,11 +425,12 @@ size_t stream_extra_bytes(int slabs, int heads, int N, int n_agents) {
 
 bool stream_make_maps(StreamArgs* a) {
     const uint64_t N = (uint64_t)a->H * a->W, S = a->slabs;
-    if (!make_map_rows3d_u16(&a->tm_k, a->k, S, N, 128, true)) return false;
-    if (!make_map_rows3d_u16(&a->tm_v, a->v, S, N, 128, true)) return false;
-    if (!make_map_grid4d_u16(&a->tm_q, a->q, S, (uint64_t)a->H, (uint64_t)a->W, (uint32_t)a->plan.rows_b, (uint32_t)(a->W + 2), true)) return false;
+    const int batch = a->slabs / a->heads;
+    if (!make_map_tok_u16(&a->tm_k, &a->hf, a->k, a->lin, batch, a->heads, (long long)N, 64, 128, true)) return false;
+    if (!make_map_tok_u16(&a->tm_v, &a->hf, a->v, a->lin, batch, a->heads, (long long)N, 64, 128, true)) return false;
+    if (!make_map_grid5d_u16(&a->tm_q, a->hf, a->q, a->lin, batch, a->heads, (uint64_t)a->H, (uint64_t)a->W, (uint32_t)a->plan.rows_b, (uint32_t)(a->W + 2))) return false;
     if (!make_map_grid4d_u16(&a->tm_b2, a->b2p, a->b2 ? (uint64_t)a->heads : 1u, (uint64_t)a->H, (uint64_t)a->W, (uint32_t)a->plan.rows_b, (uint32_t)(a->W + 2), true)) return false;
-    if (a->dwc_w && !make_map_grid4d_u16(&a->tm_h, a->v, S, (uint64_t)a->H, (uint64_t)a->W, (uint32_t)(a->plan.rows_b + 2), (uint32_t)(a->W + 2), true)) return false;
+    if (a->dwc_w && !make_map_grid5d_u16(&a->tm_h, a->hf, a->v, a->lin, batch, a->heads, (uint64_t)a->H, (uint64_t)a->W, (uint32_t)(a->plan.rows_b + 2), (uint32_t)(a->W + 2))) return false;
     if (a->b1 && !make_map_rows3d_u16(&a->tm_b1, a->b1c, (uint64_t)a->heads, N, 128, true)) return false;
     if (!make_map_2d_u16(&a->tm_a2, a->a2s, S * a->n, 64, (uint32_t)a->n, 64)) return false;
     if (!make_map_2d_u16(&a->tm_va, a->va_ws, S * a->n, 64, (uint32_t)a->n, 64)) return false;

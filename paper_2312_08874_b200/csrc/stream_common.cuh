@@ -110,6 +110,15 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
 }
 
+// 5-D tiled load of a token grid with heads and batch: box at (0, x, y, head, b), the head dimension after the grid's or
+// (head_first) before it; coordinates outside the grid are zero-filled.
+__device__ __forceinline__ void tma_load_grid(uint32_t dst, const CUtensorMap* map, int head_first, int x, int y, int head, int b, uint32_t bar) {
+    const int c1 = head_first ? head : x, c2 = head_first ? x : y, c3 = head_first ? y : head;
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];\n"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(c1), "r"(c2), "r"(c3), "r"(b), "r"(bar) : "memory");
+}
+
 // 4-D tiled load of a [slab][y][x][64] view: box at (0, x, y, slab); coordinates outside the grid (x = -1, x = W,
 // y = -1, y = H) are zero-filled, which is the zero padding of the depthwise window.
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c, int x, int y, int z, uint32_t bar) {
@@ -136,6 +145,28 @@ inline bool make_map_rows3d_u16(CUtensorMap* out, const void* base, uint64_t zs,
     return fn(out, CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, const_cast<void*>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Host: map of the token grid of a tensor with layout l for tma_load_grid (64 channels, box of 64 x box_w x box_h, 128-byte swizzle).
+// The dimension order is that of make_map_tok_u16; false if the strides cannot be expressed.
+inline bool make_map_grid5d_u16(CUtensorMap* out, int head_first, const void* base, const TokLayout& l, int batch, int heads, uint64_t H, uint64_t W, uint32_t box_h, uint32_t box_w) {
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    if ((reinterpret_cast<uintptr_t>(base) & 15u) || box_h > 256 || box_w > 256 || box_h < 1 || box_w < 1) return false;
+    if ((l.sb & 7) || (l.sh & 7) || (l.st & 7) || l.st < 64) return false;
+    const cuuint64_t st = (cuuint64_t)l.st * 2, row = st * W;
+    cuuint64_t sh = (cuuint64_t)l.sh * 2, sb = (cuuint64_t)l.sb * 2;
+    if (heads == 1 && !head_first && sh < row * H) sh = row * H;             // strides of single heads or entries are never used
+    const cuuint64_t last = head_first ? row * H : sh * heads;
+    if (batch == 1 && sb < last) sb = last;
+    const cuuint64_t dims[5] = {64, head_first ? (cuuint64_t)heads : W, head_first ? W : H, head_first ? H : (cuuint64_t)heads, (cuuint64_t)batch};
+    const cuuint64_t strides[4] = {head_first ? sh : st, head_first ? st : row, head_first ? row : sh, sb};
+    for (int i = 1; i < 4; ++i)
+        if (strides[i] < strides[i - 1]) return false;
+    const cuuint32_t box[5] = {64, head_first ? 1u : box_w, head_first ? box_w : box_h, head_first ? box_h : 1u, 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return fn(out, CU_TENSOR_MAP_DATA_TYPE_UINT16, 5, const_cast<void*>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // Host: map of a dense [z][H][W][64] tensor of 16-bit elements with a box of 64 x box_w x box_h x 1, 128-byte swizzle or none.

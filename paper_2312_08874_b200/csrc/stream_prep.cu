@@ -41,7 +41,8 @@ __global__ void __launch_bounds__(NT, 4) stream_prep_kernel(const StreamArgs p, 
             const int y0 = (a / p.p) * win_h, x0 = (a % p.p) * win_w;
             // lane (c, ts) walks the window's tokens ts, ts + 4, ... in row-major order; (wy, wx) is kept
             // incrementally, so the loads of a batch cost an add and a compare each
-            const uint4* gq = reinterpret_cast<const uint4*>(static_cast<const T*>(p.q) + ((size_t)slab * N + (size_t)y0 * p.W + x0) * 64) + c;
+            const uint4* gq = reinterpret_cast<const uint4*>(static_cast<const T*>(p.q) + tok_offset(p.lin, slab, p.heads, (long long)y0 * p.W + x0)) + c;
+            const size_t qst = (size_t)p.lin.st / 8;
             inv = 1.f / (float)cnt;
             int wy = ts / win_w, wx = ts - wy * win_w;
             float2 acc2[4];
@@ -52,7 +53,7 @@ __global__ void __launch_bounds__(NT, 4) stream_prep_kernel(const StreamArgs p, 
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     raw[u] = make_uint4(0u, 0u, 0u, 0u);
-                    if (ib + 4 * u < cnt) raw[u] = __ldg(gq + ((size_t)wy * p.W + wx) * 8);
+                    if (ib + 4 * u < cnt) raw[u] = __ldg(gq + ((size_t)wy * p.W + wx) * qst);
                     wx += 4;
                     while (wx >= win_w) { wx -= win_w; ++wy; }
                 }
