@@ -124,8 +124,17 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()
 
 
+# torch.cuda.current_stream() builds a stream object (3.2 us); the raw handle costs 0.1 us
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream_ptr(stream: Optional[torch.cuda.Stream]):
-    return (torch.cuda.current_stream() if stream is None else stream).cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None and _raw_device is not None:
+        return _raw_stream(_raw_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _bias(b1: Optional[torch.Tensor], b2: Optional[torch.Tensor]):
@@ -291,14 +300,14 @@ class AgentAttention:
         self._chk_tensor(b1, (h, n_agents, N), "b1")
         self._chk_tensor(b2, (h, N, n_agents), "b2")
         self._chk_tensor(dwc_weight, (h, d, 3, 3), "dwc_weight")
-        f32, dev = torch.float32, self.device
-        g = {k: torch.empty((B, h, N, d), dtype=f32, device=dev) for k in ("dq", "dk", "dv")}
+        f32, like = torch.float32, torch.empty_like
+        g = {"dq": like(q, dtype=f32), "dk": like(q, dtype=f32), "dv": like(q, dtype=f32)}
         if b1 is not None and need_bias_grads:
-            g["db1"] = torch.empty((h, n_agents, N), dtype=f32, device=dev)
+            g["db1"] = like(b1, dtype=f32)
         if b2 is not None and need_bias_grads:
-            g["db2"] = torch.empty((h, N, n_agents), dtype=f32, device=dev)
+            g["db2"] = like(b2, dtype=f32)
         if dwc_weight is not None and need_filter_grad:
-            g["dwd"] = torch.empty((h, d, 3, 3), dtype=f32, device=dev)
+            g["dwd"] = like(dwc_weight, dtype=f32)
         ws = self.backward_workspace(grid_h, grid_w, n_agents) if workspace is None else workspace
         grads = AgentAttnGrads(_ptr(g["dq"]), _ptr(g["dk"]), _ptr(g["dv"]), _ptr(g.get("db1")), _ptr(g.get("db2")),
                                _ptr(g.get("dwd")))

@@ -42,6 +42,7 @@ template <typename T, typename E, int NT>
 __global__ void __launch_bounds__(256) bwd_pool_terms_kernel(PoolArgs8 pa, E* dst, ClearList cl) {
     const T *q = static_cast<const T*>(pa.q), *given = static_cast<const T*>(pa.given);
     const int slabs = pa.slabs, n = pa.n, H = pa.H, W = pa.W, pool = pa.pool, d = pa.d;
+    pdl_wait_prior();
     pdl_release_next();
     if ((int)blockIdx.x >= cl.pool_blocks) {
         size_t b = (size_t)(blockIdx.x - cl.pool_blocks) * kClearWords;
@@ -148,8 +149,7 @@ template <typename T, typename E, int NT> cudaError_t launch_pool_terms(PoolArgs
     cl.pool_blocks = (int)(pa.small ? ((long long)pa.slabs * pa.n * (pa.d / 8) + 255) / 256 : ((long long)pa.slabs * pa.n + 7) / 8);
     size_t clear = 0;
     for (size_t w : cl.words) clear += (w + kClearWords - 1) / kClearWords;
-    bwd_pool_terms_kernel<T, E, NT><<<(unsigned)(cl.pool_blocks + clear), 256, 0, st>>>(pa, static_cast<E*>(a_t), cl);
-    return cudaGetLastError();
+    return launch_dependent(bwd_pool_terms_kernel<T, E, NT>, dim3((unsigned)(cl.pool_blocks + clear)), 256, 0, st, pa, static_cast<E*>(a_t), cl);
 }
 // Pooling, and the clearing of the sums that the stages add to.
 template <typename T, typename E, int NT> cudaError_t pool_and_clear(const BwdCall& c, void* a_t, bool clear_bias, cudaStream_t st) {

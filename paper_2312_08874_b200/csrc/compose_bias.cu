@@ -11,6 +11,8 @@ namespace aa {
 template <typename T, bool TRANSPOSE>
 __global__ void __launch_bounds__(256) compose_bias_kernel(ComposeArgs p) {
     const int N = p.h * p.w;
+    pdl_wait_prior();
+    pdl_release_next();
     const long long total = (long long)p.heads * p.n * N;
     const long long e0 = 8 * ((long long)blockIdx.x * 256 + threadIdx.x);
     if (e0 >= total) return;
@@ -72,21 +74,19 @@ __global__ void __launch_bounds__(256) compose_bias_kernel(ComposeArgs p) {
     }
 }
 
-template <typename T> static void launch_compose(const ComposeArgs& p, unsigned blocks, cudaStream_t st) {
-    if (p.transpose) compose_bias_kernel<T, true><<<blocks, 256, 0, st>>>(p);
-    else compose_bias_kernel<T, false><<<blocks, 256, 0, st>>>(p);
+template <typename T> static cudaError_t launch_compose(const ComposeArgs& p, unsigned blocks, cudaStream_t st) {
+    return launch_dependent(p.transpose ? compose_bias_kernel<T, true> : compose_bias_kernel<T, false>, dim3(blocks), 256, 0, st, p);
 }
 
 cudaError_t launch_compose_bias(int dtype, const ComposeArgs& p, cudaStream_t st) {
     const long long total = (long long)p.heads * p.n * p.h * p.w;
     const unsigned blocks = (unsigned)((total + 2047) / 2048);
     switch (dtype) {
-        case kF32:  launch_compose<float>(p, blocks, st); break;
-        case kBF16: launch_compose<__nv_bfloat16>(p, blocks, st); break;
-        case kF16:  launch_compose<__half>(p, blocks, st); break;
+        case kF32:  return launch_compose<float>(p, blocks, st);
+        case kBF16: return launch_compose<__nv_bfloat16>(p, blocks, st);
+        case kF16:  return launch_compose<__half>(p, blocks, st);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 }  // namespace aa

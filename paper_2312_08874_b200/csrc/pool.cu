@@ -73,8 +73,8 @@ cudaError_t launch_pool(int dtype, const PoolArgs& p, cudaStream_t st) {
     const unsigned blocks = (unsigned)((cells + 7) / 8);
     switch (dtype) {
         case kF32:  pool_kernel<float><<<blocks, 256, 0, st>>>(p); break;
-        case kBF16: pool_window_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(p); break;
-        case kF16:  pool_window_kernel<__half><<<blocks, 256, 0, st>>>(p); break;
+        case kBF16: return launch_dependent(pool_window_kernel<__nv_bfloat16>, dim3(blocks), 256, 0, st, p);
+        case kF16:  return launch_dependent(pool_window_kernel<__half>, dim3(blocks), 256, 0, st, p);
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

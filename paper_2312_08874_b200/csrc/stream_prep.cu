@@ -19,6 +19,7 @@ constexpr int NT = 256;
 
 template <typename T>
 __global__ void __launch_bounds__(NT, 4) stream_prep_kernel(const StreamArgs p, int bias_blocks) {
+    pdl_wait();                       // the workspace may still be read by the kernels before
     pdl_launch_dependents();          // the aggregation kernel may set itself up while this one runs
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int N = p.H * p.W, n = p.n;
@@ -149,10 +150,9 @@ cudaError_t launch_stream_prep(int dtype, const StreamArgs& a, cudaStream_t st) 
     if (bias_blocks > 8LL * a.sm_count) bias_blocks = 8LL * a.sm_count;
     if (bias_blocks < 1) bias_blocks = 1;
     const unsigned grid = (unsigned)(pool_blocks + bias_blocks);
-    if (dtype == kBF16) stream_prep_kernel<__nv_bfloat16><<<grid, NT, 0, st>>>(a, (int)bias_blocks);
-    else if (dtype == kF16) stream_prep_kernel<__half><<<grid, NT, 0, st>>>(a, (int)bias_blocks);
-    else return cudaErrorInvalidValue;
-    return cudaGetLastError();
+    if (dtype == kBF16) return launch_dependent(stream_prep_kernel<__nv_bfloat16>, dim3(grid), NT, 0, st, a, (int)bias_blocks);
+    if (dtype == kF16) return launch_dependent(stream_prep_kernel<__half>, dim3(grid), NT, 0, st, a, (int)bias_blocks);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace aa

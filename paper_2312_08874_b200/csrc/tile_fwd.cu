@@ -147,7 +147,7 @@ cudaError_t launch_tile_forward(int dtype, TileArgs a, int sm_count, bool one_ke
         l.grid = dim3(c, a.slabs);
         l.threads = warps * 32;
         l.cluster = c;
-        l.dependent = false;
+        l.dependent = true;
         l.stream = st;
         *launches += 1;
         return dispatch(kTileSlab, dtype, dk.dk, !a.b1 && !a.b2 ? 0 : a.b1 && a.b2 && a.N % 8 == 0 && a.n % 8 == 0 ? 1 : 2, a, l);
@@ -157,9 +157,8 @@ cudaError_t launch_tile_forward(int dtype, TileArgs a, int sm_count, bool one_ke
         const long long cells = (long long)a.slabs * a.n;
         const bool wide = cells < 8LL * sm_count && a.N > 32 * a.n;
         const unsigned blocks = (unsigned)(wide ? cells : (cells + 7) / 8);
-        if (dtype == kBF16) wide ? tile_pool_kernel<__nv_bfloat16, true><<<blocks, 256, 0, st>>>(a) : tile_pool_kernel<__nv_bfloat16, false><<<blocks, 256, 0, st>>>(a);
-        else wide ? tile_pool_kernel<__half, true><<<blocks, 256, 0, st>>>(a) : tile_pool_kernel<__half, false><<<blocks, 256, 0, st>>>(a);
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e = dtype == kBF16 ? launch_dependent(wide ? tile_pool_kernel<__nv_bfloat16, true> : tile_pool_kernel<__nv_bfloat16, false>, dim3(blocks), 256, 0, st, a)
+                                       : launch_dependent(wide ? tile_pool_kernel<__half, true> : tile_pool_kernel<__half, false>, dim3(blocks), 256, 0, st, a);
         if (e != cudaSuccess) return e;
         *launches += 1;
     }

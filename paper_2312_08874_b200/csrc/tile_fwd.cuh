@@ -79,6 +79,7 @@ template <typename T, int DK, int KG, int NW, int BIAS>
 __global__ void __launch_bounds__(NW * 32, 16 / NW) tile_slab_kernel(const __grid_constant__ TileArgs p) {
     extern __shared__ __align__(128) unsigned char smem[];
     const int slab = blockIdx.y, crank = blockIdx.x, csize = gridDim.x, warp = threadIdx.x >> 5;
+    pdl_wait_prior();           // (no early release: blocks of the next call would take the slots that balance this one)
     const AggCta<T> c = agg_cta<T>(p, slab, crank, 0);
     agg_phase<T, DK, KG, NW, BIAS>(c, smem, [&] {
         if (p.pool) {
@@ -113,6 +114,7 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) tile_slab_kernel(const __gri
 // WIDE: the eight warps of a block share a window
 template <typename T, bool WIDE>
 __global__ void __launch_bounds__(256) tile_pool_kernel(const __grid_constant__ TileArgs p) {
+    pdl_wait_prior();
     pdl_release_next();
     const int warp = threadIdx.x >> 5;
     const long long cell = WIDE ? blockIdx.x : (long long)blockIdx.x * 8 + warp;
