@@ -504,7 +504,7 @@ def main():
             mod.forward_host(pin["q"], pin["k"], pin["v"], w.grid_h, w.grid_w, w.agents, b1=pin["b1"],
                              b2=pin["b2"], dwc_weight=pin["dwc"], out=out_h, stream=stream)
         # two calls in flight on two streams, each with its own staging and result buffer: the copy back of one
-        # step overlaps the copy in of the next (the copies of a step itself stay in order on its stream)
+        # step overlaps the copy in of the next
         need = mod.staging_bytes(w.grid_h, w.grid_w, w.agents)
         lanes = [(torch.cuda.Stream(device=dev), torch.empty(need, dtype=torch.uint8, device=dev),
                   torch.empty_like(pin["q"]).pin_memory()) for _ in range(2)]

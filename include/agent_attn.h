@@ -229,7 +229,9 @@ size_t agent_attn_staging_bytes(const agent_attn_handle* h, int grid_h, int grid
  * members, dwc_weight and out are host pointers (pinned memory makes the copies asynchronous).
  * `staging` is device memory of >= agent_attn_staging_bytes(...) owned by the caller.
  * Enqueues host-to-device copies of every input, the forward pass and the device-to-host copy
- * of out on `stream`; the caller synchronises the stream before reading `out`. */
+ * of out, in order on `stream`; the caller synchronises the stream before reading `out`.  Large
+ * calls on pinned memory are cut into up to four parts whose copies run on two streams of the
+ * handle, tied to `stream` by events, so that copies and kernels of different parts overlap. */
 int agent_attn_forward_host(agent_attn_handle* h,
                             const void* Q, const void* K, const void* V, const void* A,
                             int grid_h, int grid_w, int n_agents,
