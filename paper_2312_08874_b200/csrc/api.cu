@@ -75,11 +75,19 @@ bool umma_shape(const agent_attn_handle* h, int n_tokens, int n_agents) {
     return !use_simt(h) && auto_like(h) &&
            aggregate_umma_eligible(h->cfg.dtype, n_agents, n_tokens, h->cfg.head_dim, true);
 }
-// They win on long token axes (16384 tokens of 256 agents: 190 us against 247 us); below 8192 tokens their start and their
-// separate merge cost more than they save (4096 tokens: 60 us against 51 us; 464 tokens, 240 slabs: 157 us against 141 us) and
-// the register-tiled kernels run.
+// They pad agents to 128 and channels to 64 and pay a start and a separate merge; the register tiles pay for neither.  Where the agents and
+// channels fill the padded blocks they win as soon as the token axis is long or there is work for several tiles of every block (256 agents
+// of 64 channels: 24 slabs of 7920 tokens 127 us against 163 us, 128 slabs of 4096 tokens 319 against 374; 32 slabs of 4096 tokens 105 by
+// either).  Elsewhere they win on long axes only (144 agents, 16 slabs of 16384 tokens: 162 us against 207 us), and not with few channels
+// and either many tokens or half-filled blocks (40 channels, 64 slabs of 10400 tokens: 315 us against 287 us; 144 agents of 32 channels, the
+// same: 359 against 241).
 bool use_umma(const agent_attn_handle* h, int n_tokens, int n_agents) {
-    return n_tokens >= 8192 && umma_shape(h, n_tokens, n_agents);
+    if (n_tokens < 2048 || !umma_shape(h, n_tokens, n_agents)) return false;
+    const int d = h->cfg.head_dim;
+    const long long work = (long long)h->cfg.batch * h->cfg.heads * n_tokens;
+    const bool filled = n_agents * 4 >= (n_agents + 127) / 128 * 128 * 3;
+    if (filled && d > 48) return n_tokens >= 6144 || work >= 150000;
+    return n_tokens >= 8192 && (filled || d > 32) && (d > 48 || work < 400000);
 }
 
 AggPlan plan_for(const agent_attn_handle* h, int n_tokens, int n_agents) {
@@ -299,16 +307,18 @@ int agent_attn_create(agent_attn_handle** out, const agent_attn_config* cfg) {
     }
     DeviceGuard guard(cfg->device);
     if (!guard.ok) return AA_ERR_CUDA;
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, cfg->device) != cudaSuccess) return AA_ERR_CUDA;
-    if (prop.major != 10) return AA_ERR_CUDA;       // the kernels are built for sm_100a only
+    int major = 0, sms = 0;                         // (cudaGetDeviceProperties takes 2.6 ms)
+    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, cfg->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cfg->device) != cudaSuccess)
+        return AA_ERR_CUDA;
+    if (major != 10) return AA_ERR_CUDA;            // the kernels are built for sm_100a only
 
     agent_attn_handle* h = new (std::nothrow) agent_attn_handle;
     if (!h) return AA_ERR_INVALID_ARG;
     memset(h, 0, sizeof(*h));
     h->cfg = *cfg;
     h->elem_bytes = es;
-    h->sm_count = prop.multiProcessorCount;
+    h->sm_count = sms;
     const float def = 1.0f / std::sqrt((float)cfg->head_dim);
     h->scale1 = cfg->scale1 > 0.f ? cfg->scale1 : def;
     h->scale2 = cfg->scale2 > 0.f ? cfg->scale2 : def;

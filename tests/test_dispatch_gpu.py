@@ -1,0 +1,29 @@
+"""Either side of the lines between the tensor-memory kernels and the register-tiled ones, against the fp64 oracle."""
+import pytest
+
+from paper_2312_08874_b200 import Workload, make_inputs
+from tests.parity_util import assert_close, gpu_forward, make_module, oracle_forward
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [
+    # batch heads H   W   d   pool launches
+    (1, 1, 64, 96, 64, 16, 4),        # 6144 tokens, filled blocks: tensor memory
+    (1, 1, 64, 95, 64, 16, 3),        # fewer: register tiles
+    (20, 2, 47, 80, 64, 16, 4),       # short axis, 150400 tokens in all: tensor memory
+    (1, 2, 64, 128, 64, 12, 4),       # half-filled blocks on a long axis: tensor memory
+    (1, 2, 64, 128, 32, 12, 3),       # and of few channels: register tiles
+]
+
+
+@pytest.mark.parametrize("case", SHAPES, ids=[f"B{c[0]}h{c[1]}_{c[2]}x{c[3]}_d{c[4]}_p{c[5]}" for c in SHAPES])
+def test_dispatch_lines(case):
+    B, heads, H, W, d, pool, launches = case
+    w = Workload("dispatch", B, heads, H, W, d, pool, "bf16", True, True, 1.0, seed=400 + H * W + d)
+    inp = make_inputs(w, bias_std=0.5, dwc_std=0.2)
+    mod = make_module(w)
+    out = gpu_forward(mod, w, inp)
+    assert mod.last_launch_count() == launches
+    slabs = [(0, 0), (B - 1, heads - 1)]
+    for (b, h), ref in zip(slabs, oracle_forward(w, inp, slabs=slabs)):
+        assert_close(out[b:b + 1, h:h + 1], ref, "bf16", f"{case} slab {(b, h)}")
