@@ -133,28 +133,6 @@ __device__ __forceinline__ void tile_values(float (&o)[TileGeom<DK>::kMT][TileGe
         }
 }
 
-// Eight consecutive bias elements whose row starts at any element: `align` is the alignment (in elements: 8, 2 or 1)
-// that every row of the tensor has; the first `cnt` elements exist.
-template <typename T> __device__ __forceinline__ uint4 load_bias8(const T* p, int align, int cnt) {
-    uint4 r = make_uint4(0u, 0u, 0u, 0u);
-    if (cnt <= 0) return r;
-    if (align == 8) return __ldg(reinterpret_cast<const uint4*>(p));      // then cnt is a multiple of 8 too
-    uint32_t w[4] = {0u, 0u, 0u, 0u};
-    if (align == 2) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (2 * i < cnt) w[i] = __ldg(reinterpret_cast<const uint32_t*>(p) + i);
-    } else {
-        const unsigned short* u = reinterpret_cast<const unsigned short*>(p);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint32_t lo = 2 * i < cnt ? __ldg(u + 2 * i) : 0, hi = 2 * i + 1 < cnt ? __ldg(u + 2 * i + 1) : 0;
-            w[i] = lo | (hi << 16);
-        }
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
 // Running state of the softmax of a warp's rows (row index: m-tile, half).  `ref` is the exponent reference in log2
 // units, taken from the row's first block; it moves only when a logit exceeds it by more than 8 (so the products are
 // rescaled rarely, and probabilities stay below 2^8: inside fp16).  `lim` is that 8, or -inf while the row has no weight.
