@@ -653,14 +653,14 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                         mx = fmaxf(mx, v);
                     }
                     mx = quad_max(mx);
-                    const float f = m[h] == -INFINITY ? 0.f : exp2f(m[h] - mx);
+                    const float base = mx == -INFINITY ? 0.f : mx, f = exp2f(m[h] - base);      // (every agent so far may be masked)
                     m[h] = mx;
                     l[h] *= f;
 #pragma unroll
                     for (int j = 0; j < NT; ++j) { o0[j][2 * h] *= f; o0[j][2 * h + 1] *= f; }
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const float p0 = fast_exp2(s[j][2 * h] - mx), p1 = fast_exp2(s[j][2 * h + 1] - mx);
+                        const float p0 = fast_exp2(s[j][2 * h] - base), p1 = fast_exp2(s[j][2 * h + 1] - base);
                         l[h] += p0 + p1;
                         uint32_t w[TP];
                         split_pair<E, TP>(p0, p1, w);
