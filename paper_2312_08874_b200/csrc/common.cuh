@@ -9,6 +9,9 @@
 namespace aa {
 
 constexpr float kLog2e = 1.4426950408889634f;
+// Least reference of an online softmax in natural units: finite in log2 units too, so that a row whose entries are all removed so far
+// (-inf, or a type's lowest value) has probabilities exp2(-inf) = 0 and not exp2(-inf + inf).
+constexpr float kRefFloor = -2e38f;
 
 // ----------------------------------------------------------------------------- element types
 template <typename T> struct Elem;

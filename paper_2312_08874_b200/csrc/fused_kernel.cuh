@@ -385,8 +385,7 @@ __device__ __forceinline__ void run_g_task(const FusedArgs& p, int slab, int sub
         mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
         mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
         const float mn0 = fmaxf(m0, mx0), mn1 = fmaxf(m1, mx1);
-        const float base0 = (mn0 == -INFINITY) ? 0.f : mn0;
-        const float base1 = (mn1 == -INFINITY) ? 0.f : mn1;
+        const float base0 = fmaxf(mn0, kRefFloor), base1 = fmaxf(mn1, kRefFloor);
         const float nb0 = -base0 * kLog2e, nb1 = -base1 * kLog2e;
         // rescale the running state only when some row of the warp saw a new maximum
         if (__any_sync(0xffffffffu, (mn0 != m0) || (mn1 != m1))) {

@@ -2,7 +2,7 @@
 import pytest
 import torch
 
-from paper_2312_08874_b200 import AA_PATH_AUTO, AA_PATH_SIMT, Workload, make_inputs
+from paper_2312_08874_b200 import AA_PATH_AUTO, AA_PATH_QUEUE, AA_PATH_SIMT, Workload, make_inputs
 from paper_2312_08874_b200.workloads import TORCH_DTYPE
 from tests.parity_util import assert_close, gpu_forward, make_module, oracle_forward
 from tests.test_backward_gpu import check, run_both, tensor_core_path
@@ -17,6 +17,7 @@ SHAPES = [
     (2, 2, 14, 14, 64, 7, "bf16", AA_PATH_AUTO),      # register tiles, one kernel
     (1, 1, 40, 41, 32, 13, "f16", AA_PATH_AUTO),      # register tiles, two row blocks, unaligned bias rows
     (1, 2, 32, 32, 64, 7, "bf16", AA_PATH_AUTO),      # streaming kernels
+    (1, 2, 14, 14, 64, 7, "bf16", AA_PATH_QUEUE),     # task queue
 ]
 IDS = [f"{c[6]}_{c[2]}x{c[3]}_d{c[4]}_p{c[5]}_path{c[7]}" for c in SHAPES]
 
