@@ -18,6 +18,8 @@ SHAPES = [
     (1, 1, 40, 41, 32, 13, "f16", AA_PATH_AUTO),      # register tiles, two row blocks, unaligned bias rows
     (1, 2, 32, 32, 64, 7, "bf16", AA_PATH_AUTO),      # streaming kernels
     (1, 2, 14, 14, 64, 7, "bf16", AA_PATH_QUEUE),     # task queue
+    (1, 1, 64, 96, 64, 16, "bf16", AA_PATH_AUTO),     # tensor memory: every agent group of a step closed
+    (1, 1, 96, 96, 40, 12, "f16", AA_PATH_AUTO),      # the same, half-filled blocks
 ]
 IDS = [f"{c[6]}_{c[2]}x{c[3]}_d{c[4]}_p{c[5]}_path{c[7]}" for c in SHAPES]
 
