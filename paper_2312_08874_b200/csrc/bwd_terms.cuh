@@ -21,6 +21,61 @@ template <int NA, int NB> struct TermPairs {
     __host__ __device__ static constexpr bool keep(int i, int j) { return i + j < kOrder; }
 };
 
+// Products of two 8-column tiles (MMA operands A: terms of 16 rows, B: terms of 16 columns).  An mma.sync rounds its sum towards
+// zero, so a long chain of them in one accumulator drifts: with chains over a block's whole token range the forward pass of 16384
+// tokens was 1.4e-5 off, 1.2e-7 this way (fp32 FMAs: 1.4e-7).  So the pairs of leading terms are kept apart from the small ones, and
+// sums over tokens or agents take 32 of them at a time (TermSum) and join in fp32 additions, which round to nearest.
+template <typename E> __device__ __forceinline__ void mma_two(float (&c0)[4], float (&c1)[4], const uint32_t (&a)[4], const uint32_t (&b)[4], bool fresh) {
+    if (fresh) {
+        mma_set<E>(c0, a, b[0], b[1]);
+        mma_set<E>(c1, a, b[2], b[3]);
+    } else {
+        mma_acc<E>(c0, a, b[0], b[1]);
+        mma_acc<E>(c1, a, b[2], b[3]);
+    }
+}
+// every pair of A's terms with term k of B, but for that of the leading terms; `fresh`: the first one starts the sum
+template <typename E, int NA, int NB> __device__ __forceinline__ void mma_low(float (&c0)[4], float (&c1)[4], const uint32_t (&a)[NA][4], const uint32_t (&b)[4], int k, bool fresh) {
+#pragma unroll
+    for (int i = NA - 1; i >= 0; --i)
+        if (TermPairs<NA, NB>::keep(i, k) && i + k > 0) {
+            mma_two<E>(c0, c1, a[i], b, fresh);
+            fresh = false;
+        }
+}
+__device__ __forceinline__ void add4(float (&c)[4], const float (&t)[4]) {
+#pragma unroll
+    for (int e = 0; e < 4; e += 2) {
+        const float2 u = fadd2(make_float2(c[e], c[e + 1]), make_float2(t[e], t[e + 1]));
+        c[e] = u.x;
+        c[e + 1] = u.y;
+    }
+}
+// A product over 32 tokens or agents (two k steps), added to o0 and o1: `load(b, kk, k)` fetches term k of B.  The small pairs come
+// first, so that only the two leading ones are rounded at full magnitude.  FULL false (A rounded to 16 bits): straight into o0, o1.
+template <typename E, int NA, int NB, bool FULL, typename F>
+__device__ __forceinline__ void term_sum(float (&o0)[4], float (&o1)[4], const uint32_t (&a)[2][NA][4], F&& load) {
+    float t[2][4];
+    uint32_t b[2][4];
+#pragma unroll
+    for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+        for (int k = NB - 1; k >= 0; --k) {
+            load(b[kk], kk, k);
+            if (FULL) mma_low<E, NA, NB>(t[0], t[1], a[kk], b[kk], k, kk == 0 && k == NB - 1);
+            else mma_low<E, NA, NB>(o0, o1, a[kk], b[kk], k, false);
+        }
+#pragma unroll
+    for (int kk = 0; kk < 2; ++kk) {
+        if (FULL) mma_two<E>(t[0], t[1], a[kk][0], b[kk], false);
+        else mma_two<E>(o0, o1, a[kk][0], b[kk], false);
+    }
+    if (FULL) {
+        add4(o0, t[0]);
+        add4(o1, t[1]);
+    }
+}
+
 // two fp32 -> NT packed pairs of terms
 template <typename E, int NT> __device__ __forceinline__ void split_pair(float a, float b, uint32_t (&w)[NT]) {
 #pragma unroll
@@ -142,6 +197,7 @@ template <typename T, typename E, int DK, int NX, int TA, int TM, int TP, int KG
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(const __grid_constant__ BwdTermArgs p) {
     using S = SumsShape<DK, NX, TA, TM, KG, NW, MODE>;
     constexpr int PITCH = S::kPitch, KS = DK / 16, NT = DK / 8, TOK = S::kTokens;
+    constexpr bool FULL = TA > 1;                      // (mixed precision: A is rounded to 16 bits)
     extern __shared__ __align__(128) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const int slab = blockIdx.z, head = slab % p.heads, rows = p.rg * 16, row0 = blockIdx.y * rows;
@@ -230,11 +286,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(cons
             const int tok = t0 + it * TOK + (sub * KG + kgi) * 32;
             if (tok >= t1) break;
             const uint32_t xs = st + sub * KG * 32 * PITCH, ys = xs + NX * TOK * PITCH;
-            float s[4][4], dp[4][4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) s[j][e] = dp[j][e] = 0.f;
+            float s[4][4], dp[4][4], sl[4][4], dl[4][4];                  // leading terms, small ones
 #pragma unroll
             for (int ks = 0; ks < KS; ++ks) {
                 uint32_t a[TA][4], m[TM][4];
@@ -249,22 +301,19 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(cons
                     for (int k = 0; k < NX; ++k) {
                         uint32_t b[4];
                         ldsm4(b, xs + koff + k * TOK * PITCH + j2 * 16 * PITCH + ks * 32);
-#pragma unroll
-                        for (int i = 0; i < TA; ++i)
-                            if (TermPairs<TA, NX>::keep(i, k)) {
-                                mma_acc<E>(s[2 * j2], a[i], b[0], b[1]);
-                                mma_acc<E>(s[2 * j2 + 1], a[i], b[2], b[3]);
-                            }
+                        if (k == 0) mma_two<E>(s[2 * j2], s[2 * j2 + 1], a[0], b, ks == 0);
+                        mma_low<E, TA, NX>(sl[2 * j2], sl[2 * j2 + 1], a, b, k, ks == 0 && k == 0);
                         if (MODE != kSumsForward) {
                             ldsm4(b, ys + koff + k * TOK * PITCH + j2 * 16 * PITCH + ks * 32);
-#pragma unroll
-                            for (int i = 0; i < TM; ++i)
-                                if (TermPairs<TM, NX>::keep(i, k)) {
-                                    mma_acc<E>(dp[2 * j2], m[i], b[0], b[1]);
-                                    mma_acc<E>(dp[2 * j2 + 1], m[i], b[2], b[3]);
-                                }
+                            if (k == 0) mma_two<E>(dp[2 * j2], dp[2 * j2 + 1], m[0], b, ks == 0);
+                            mma_low<E, TM, NX>(dl[2 * j2], dl[2 * j2 + 1], m, b, k, ks == 0 && k == 0);
                         }
                     }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (FULL) add4(s[j], sl[j]);
+                if (MODE != kSumsForward) add4(dp[j], dl[j]);
             }
             // logits in log2 units, then probabilities and logit gradients
             const int left = t1 - tok - 8 * t;
@@ -284,7 +333,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(cons
                     }
                 }
             }
-            uint32_t pt[TP][2][4], dt[TP][2][4];
+            uint32_t pt[2][TP][4], dt[2][TP][4];
             if constexpr (MODE == kSumsForward) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -310,7 +359,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(cons
                         uint32_t w[TP];
                         split_pair<E, TP>(p0, p1, w);
 #pragma unroll
-                        for (int i = 0; i < TP; ++i) pt[i][j >> 1][(j & 1) * 2 + h] = w[i];
+                        for (int i = 0; i < TP; ++i) pt[j >> 1][i][(j & 1) * 2 + h] = w[i];
                     }
                 }
             } else {
@@ -340,42 +389,24 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(cons
                         if (MODE == kSumsBroadcast) {
                             split_pair<E, TP>(pv[0], pv[1], w);
 #pragma unroll
-                            for (int i = 0; i < TP; ++i) pt[i][j >> 1][(j & 1) * 2 + h] = w[i];
+                            for (int i = 0; i < TP; ++i) pt[j >> 1][i][(j & 1) * 2 + h] = w[i];
                         }
                         split_pair<E, TP>(ds[2 * j], ds[2 * j + 1], w);
 #pragma unroll
-                        for (int i = 0; i < TP; ++i) dt[i][j >> 1][(j & 1) * 2 + h] = w[i];
+                        for (int i = 0; i < TP; ++i) dt[j >> 1][i][(j & 1) * 2 + h] = w[i];
                     }
                     if (MODE == kSumsAggregate && p.dbias && r0 + h * 8 < p.n)
                         put_dbias8(p.dbias + ((size_t)head * p.n + r0 + h * 8) * p.N + tok + 8 * t, ds, left, p.N % 4 == 0, p.slabs == p.heads);
                 }
             }
 #pragma unroll
-            for (int kk = 0; kk < 2; ++kk)
-#pragma unroll
-                for (int c2 = 0; c2 < NT / 2; ++c2)
-#pragma unroll
-                    for (int k = 0; k < NX; ++k) {
-                        uint32_t b[4];
-                        if (MODE != kSumsAggregate) {
-                            ldsm4t(b, ys + voff + k * TOK * PITCH + kk * 16 * PITCH + c2 * 32);
-#pragma unroll
-                            for (int i = 0; i < TP; ++i)
-                                if (TermPairs<TP, NX>::keep(i, k)) {
-                                    mma_acc<E>(o0[2 * c2], pt[i][kk], b[0], b[1]);
-                                    mma_acc<E>(o0[2 * c2 + 1], pt[i][kk], b[2], b[3]);
-                                }
-                        }
-                        if (MODE != kSumsForward) {
-                            ldsm4t(b, xs + voff + k * TOK * PITCH + kk * 16 * PITCH + c2 * 32);
-#pragma unroll
-                            for (int i = 0; i < TP; ++i)
-                                if (TermPairs<TP, NX>::keep(i, k)) {
-                                    mma_acc<E>(o1[2 * c2], dt[i][kk], b[0], b[1]);
-                                    mma_acc<E>(o1[2 * c2 + 1], dt[i][kk], b[2], b[3]);
-                                }
-                        }
-                    }
+            for (int c2 = 0; c2 < NT / 2; ++c2) {
+                auto rows = [&](uint32_t base) {
+                    return [&, base](uint32_t (&b)[4], int kk, int k) { ldsm4t(b, base + voff + k * TOK * PITCH + kk * 16 * PITCH + c2 * 32); };
+                };
+                if constexpr (MODE != kSumsAggregate) term_sum<E, TP, NX, FULL>(o0[2 * c2], o0[2 * c2 + 1], pt, rows(ys));
+                if constexpr (MODE != kSumsForward) term_sum<E, TP, NX, FULL>(o1[2 * c2], o1[2 * c2 + 1], dt, rows(xs));
+            }
         }
     }
     if constexpr (MODE != kSumsForward) {
@@ -569,11 +600,7 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                     }
                 }
             }
-            float s[4][4], dp[4][4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) s[j][e] = dp[j][e] = 0.f;
+            float s[4][4], dp[4][4], sl[4][4], dl[4][4];                  // leading terms, small ones
 #pragma unroll
             for (int ks = 0; ks < KS; ++ks) {
                 uint32_t xt[NX][4], yt[NX][4];
@@ -598,26 +625,23 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                     for (int i = 0; i < TA; ++i) {
                         uint32_t b[4];
                         ldsm4(b, koff + (i * n32 + blk + j2 * 16) * PITCH + ks * 32);
-#pragma unroll
-                        for (int k = 0; k < NX; ++k)
-                            if (TermPairs<TA, NX>::keep(i, k)) {
-                                mma_acc<E>(s[2 * j2], xt[k], b[0], b[1]);
-                                mma_acc<E>(s[2 * j2 + 1], xt[k], b[2], b[3]);
-                            }
+                        if (i == 0) mma_two<E>(s[2 * j2], s[2 * j2 + 1], xt[0], b, ks == 0);
+                        mma_low<E, NX, TA>(sl[2 * j2], sl[2 * j2 + 1], xt, b, i, ks == 0 && i == (NX == 1));
                     }
                     if (MODE != kRowsOut)
 #pragma unroll
                         for (int i = 0; i < TM; ++i) {
                             uint32_t b[4];
                             ldsm4(b, koff + ((TA + i) * n32 + blk + j2 * 16) * PITCH + ks * 32);
-#pragma unroll
-                            for (int k = 0; k < NX; ++k)
-                                if (TermPairs<TM, NX>::keep(i, k)) {
-                                    mma_acc<E>(dp[2 * j2], yt[k], b[0], b[1]);
-                                    mma_acc<E>(dp[2 * j2 + 1], yt[k], b[2], b[3]);
-                                }
+                            if (i == 0) mma_two<E>(dp[2 * j2], dp[2 * j2 + 1], yt[0], b, ks == 0);
+                            mma_low<E, NX, TM>(dl[2 * j2], dl[2 * j2 + 1], yt, b, i, ks == 0 && i == (NX == 1));
                         }
                 }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                add4(s[j], sl[j]);
+                if (MODE != kRowsOut) add4(dp[j], dl[j]);
             }
             const int left = p.n - blk - 8 * t;
             if constexpr (MODE == kRowsStats) {
@@ -642,7 +666,7 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                     }
                 }
             } else if constexpr (MODE == kRowsOut) {
-                uint32_t pt[TP][2][4];
+                uint32_t pt[2][TP][4];
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     float mx = m[h];
@@ -665,26 +689,14 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                         uint32_t w[TP];
                         split_pair<E, TP>(p0, p1, w);
 #pragma unroll
-                        for (int i = 0; i < TP; ++i) pt[i][j >> 1][(j & 1) * 2 + h] = w[i];
+                        for (int i = 0; i < TP; ++i) pt[j >> 1][i][(j & 1) * 2 + h] = w[i];
                     }
                 }
 #pragma unroll
-                for (int kk = 0; kk < 2; ++kk)
-#pragma unroll
-                    for (int c2 = 0; c2 < NT / 2; ++c2)
-#pragma unroll
-                        for (int i = 0; i < TM; ++i) {
-                            uint32_t b[4];
-                            ldsm4t(b, voff + ((TA + i) * n32 + blk + kk * 16) * PITCH + c2 * 32);
-#pragma unroll
-                            for (int k = 0; k < TP; ++k)
-                                if (TermPairs<TP, TM>::keep(k, i)) {
-                                    mma_acc<E>(o0[2 * c2], pt[k][kk], b[0], b[1]);
-                                    mma_acc<E>(o0[2 * c2 + 1], pt[k][kk], b[2], b[3]);
-                                }
-                        }
+                for (int c2 = 0; c2 < NT / 2; ++c2)
+                    term_sum<E, TP, TM, true>(o0[2 * c2], o0[2 * c2 + 1], pt, [&](uint32_t (&b)[4], int kk, int i) { ldsm4t(b, voff + ((TA + i) * n32 + blk + kk * 16) * PITCH + c2 * 32); });
             } else {
-                uint32_t pt[TP][2][4], dt[TP][2][4];
+                uint32_t pt[2][TP][4], dt[2][TP][4];
                 float2 cs[8];
                 if (MODE == kRowsKeyValue)
 #pragma unroll
@@ -711,43 +723,21 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                         if (MODE == kRowsKeyValue) {
                             split_pair<E, TP>(pv[0], pv[1], w);
 #pragma unroll
-                            for (int i = 0; i < TP; ++i) pt[i][j >> 1][(j & 1) * 2 + h] = w[i];
+                            for (int i = 0; i < TP; ++i) pt[j >> 1][i][(j & 1) * 2 + h] = w[i];
                         }
                         split_pair<E, TP>(ds[2 * j], ds[2 * j + 1], w);
 #pragma unroll
-                        for (int i = 0; i < TP; ++i) dt[i][j >> 1][(j & 1) * 2 + h] = w[i];
+                        for (int i = 0; i < TP; ++i) dt[j >> 1][i][(j & 1) * 2 + h] = w[i];
                     }
                     if (MODE == kRowsQuery && p.dbias && tok + h * 8 + g < t1)
                         put_dbias8(p.dbias + ((size_t)head * p.N + tok + h * 8 + g) * p.n + blk + 8 * t, ds, left, p.n % 4 == 0, p.slabs == p.heads);
                 }
 #pragma unroll
-                for (int kk = 0; kk < 2; ++kk)
-#pragma unroll
-                    for (int c2 = 0; c2 < NT / 2; ++c2) {
-#pragma unroll
-                        for (int i = 0; i < TA; ++i) {
-                            uint32_t b[4];
-                            ldsm4t(b, voff + (i * n32 + blk + kk * 16) * PITCH + c2 * 32);
-#pragma unroll
-                            for (int k = 0; k < TP; ++k)
-                                if (TermPairs<TP, TA>::keep(k, i)) {
-                                    mma_acc<E>(o0[2 * c2], dt[k][kk], b[0], b[1]);
-                                    mma_acc<E>(o0[2 * c2 + 1], dt[k][kk], b[2], b[3]);
-                                }
-                        }
-                        if (MODE == kRowsKeyValue)
-#pragma unroll
-                            for (int i = 0; i < TM; ++i) {
-                                uint32_t b[4];
-                                ldsm4t(b, voff + ((TA + i) * n32 + blk + kk * 16) * PITCH + c2 * 32);
-#pragma unroll
-                                for (int k = 0; k < TP; ++k)
-                                    if (TermPairs<TP, TM>::keep(k, i)) {
-                                        mma_acc<E>(o1[2 * c2], pt[k][kk], b[0], b[1]);
-                                        mma_acc<E>(o1[2 * c2 + 1], pt[k][kk], b[2], b[3]);
-                                    }
-                            }
-                    }
+                for (int c2 = 0; c2 < NT / 2; ++c2) {
+                    term_sum<E, TP, TA, true>(o0[2 * c2], o0[2 * c2 + 1], dt, [&](uint32_t (&b)[4], int kk, int i) { ldsm4t(b, voff + (i * n32 + blk + kk * 16) * PITCH + c2 * 32); });
+                    if (MODE == kRowsKeyValue)
+                        term_sum<E, TP, TM, true>(o1[2 * c2], o1[2 * c2 + 1], pt, [&](uint32_t (&b)[4], int kk, int i) { ldsm4t(b, voff + ((TA + i) * n32 + blk + kk * 16) * PITCH + c2 * 32); });
+                }
             }
         }
         if constexpr (MODE == kRowsOut) {

@@ -2,8 +2,9 @@
 import pytest
 import torch
 
-from paper_2312_08874_b200 import AA_PATH_AUTO, Workload, make_inputs
-from tests.parity_util import assert_close, make_module, oracle_forward, to_dev
+from oracle import agent_attention_oracle as orc
+from paper_2312_08874_b200 import AA_PATH_AUTO, Workload, make_inputs, make_upstream_grad
+from tests.parity_util import assert_close, errors, make_module, oracle_forward, to_dev, to_np
 from tests.test_backward_gpu import check, run_both
 
 pytestmark = pytest.mark.gpu
@@ -51,3 +52,31 @@ def test_fp32_backward_matches_oracle(case):
     w = workload(case)
     _, got, ref = run_both(w, make_inputs(w, bias_std=0.5, dwc_std=0.2), path=AA_PATH_AUTO)
     check(got, ref, str(case))
+
+
+# Many slabs: a block takes thousands of tokens of one.  fp32 arithmetic that rounds to nearest: an output passes through about eight
+# rounded stages (operands, logits, exponential, weights, two sums, the merge) of 2^-24 each, random sums of their errors well below
+# 16 x 2^-24 = 1e-6; the logit gradients are differences dP - rowsum(P dP) that cancel up to three quarters of dP: 4e-6.
+LONG_FORWARD, LONG_BACKWARD = 1e-6, 4e-6
+
+
+def test_fp32_forward_of_many_long_slabs_stays_fp32_accurate():
+    w = Workload("long", 2, 8, 128, 128, 64, 7, "f32", True, False, 1.0, seed=31)
+    inp = make_inputs(w, bias_std=0.2)
+    out = make_module(w).forward(to_dev(inp["q"]), to_dev(inp["k"]), to_dev(inp["v"]), w.grid_h, w.grid_w, w.agents, b1=to_dev(inp["b1"]), b2=to_dev(inp["b2"]))
+    slabs = [(0, 0), (1, 7)]
+    for (b, h), ref in zip(slabs, oracle_forward(w, inp, slabs=slabs)):
+        assert errors(out[b:b + 1, h:h + 1], ref)["rel_l2"] <= LONG_FORWARD
+
+
+def test_term_gradients_of_many_long_slabs_stay_fp32_accurate():
+    w = Workload("long", 2, 8, 128, 128, 64, 16, "bf16", True, False, 1.0, seed=32)
+    inp, go = make_inputs(w, bias_std=0.2), make_upstream_grad(w)
+    got = make_module(w).backward(to_dev(inp["q"]), to_dev(inp["k"]), to_dev(inp["v"]), to_dev(go), w.grid_h, w.grid_w, w.agents,
+                                  b1=to_dev(inp["b1"]), b2=to_dev(inp["b2"]))
+    b, h = 1, 6
+    one = lambda t: to_np(t[b:b + 1, h:h + 1])
+    ref = orc.backward(one(inp["q"]), one(inp["k"]), one(inp["v"]), one(go), w.grid_h, w.grid_w, (w.pool, w.pool),
+                       b1=to_np(inp["b1"][h:h + 1]), b2=to_np(inp["b2"][h:h + 1]))
+    for key in ("dq", "dk", "dv"):
+        assert errors(got[key][b:b + 1, h:h + 1], ref[key])["rel_l2"] <= LONG_BACKWARD, key
