@@ -24,7 +24,7 @@ template <int NA, int NB> struct TermPairs {
 // Products of two 8-column tiles (MMA operands A: terms of 16 rows, B: terms of 16 columns).  An mma.sync rounds its sum towards
 // zero, so a long chain of them in one accumulator drifts: with chains over a block's whole token range the forward pass of 16384
 // tokens was 1.4e-5 off, 1.2e-7 this way (fp32 FMAs: 1.4e-7).  So the pairs of leading terms are kept apart from the small ones, and
-// sums over tokens or agents take 32 of them at a time (TermSum) and join in fp32 additions, which round to nearest.
+// sums over tokens or agents take 32 of them at a time (term_sum) and join in fp32 additions, which round to nearest.
 template <typename E> __device__ __forceinline__ void mma_two(float (&c0)[4], float (&c1)[4], const uint32_t (&a)[4], const uint32_t (&b)[4], bool fresh) {
     if (fresh) {
         mma_set<E>(c0, a, b[0], b[1]);
@@ -52,9 +52,10 @@ __device__ __forceinline__ void add4(float (&c)[4], const float (&t)[4]) {
     }
 }
 // A product over 32 tokens or agents (two k steps), added to o0 and o1: `load(b, kk, k)` fetches term k of B.  The small pairs come
-// first, so that only the two leading ones are rounded at full magnitude.  FULL false (A rounded to 16 bits): straight into o0, o1.
-template <typename E, int NA, int NB, bool FULL, typename F>
+// first, so that only the two leading ones are rounded at full magnitude.
+template <typename E, int NA, int NB, typename F>
 __device__ __forceinline__ void term_sum(float (&o0)[4], float (&o1)[4], const uint32_t (&a)[2][NA][4], F&& load) {
+    static_assert(NA > 1 || NB > 1, "small pairs start the sum");
     float t[2][4];
     uint32_t b[2][4];
 #pragma unroll
@@ -62,18 +63,12 @@ __device__ __forceinline__ void term_sum(float (&o0)[4], float (&o1)[4], const u
 #pragma unroll
         for (int k = NB - 1; k >= 0; --k) {
             load(b[kk], kk, k);
-            if (FULL) mma_low<E, NA, NB>(t[0], t[1], a[kk], b[kk], k, kk == 0 && k == NB - 1);
-            else mma_low<E, NA, NB>(o0, o1, a[kk], b[kk], k, false);
+            mma_low<E, NA, NB>(t[0], t[1], a[kk], b[kk], k, kk == 0 && k == NB - 1);
         }
 #pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {
-        if (FULL) mma_two<E>(t[0], t[1], a[kk][0], b[kk], false);
-        else mma_two<E>(o0, o1, a[kk][0], b[kk], false);
-    }
-    if (FULL) {
-        add4(o0, t[0]);
-        add4(o1, t[1]);
-    }
+    for (int kk = 0; kk < 2; ++kk) mma_two<E>(t[0], t[1], a[kk][0], b[kk], false);
+    add4(o0, t[0]);
+    add4(o1, t[1]);
 }
 
 // two fp32 -> NT packed pairs of terms
@@ -197,7 +192,7 @@ template <typename T, typename E, int DK, int NX, int TA, int TM, int TP, int KG
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(const __grid_constant__ BwdTermArgs p) {
     using S = SumsShape<DK, NX, TA, TM, KG, NW, MODE>;
     constexpr int PITCH = S::kPitch, KS = DK / 16, NT = DK / 8, TOK = S::kTokens;
-    constexpr bool FULL = TA > 1;                      // (mixed precision: A is rounded to 16 bits)
+    constexpr bool kLow = TA > 1 || NX > 1;            // (mixed precision: the logits have one pair of terms)
     extern __shared__ __align__(128) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const int slab = blockIdx.z, head = slab % p.heads, rows = p.rg * 16, row0 = blockIdx.y * rows;
@@ -312,7 +307,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(cons
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                if (FULL) add4(s[j], sl[j]);
+                if (kLow) add4(s[j], sl[j]);
                 if (MODE != kSumsForward) add4(dp[j], dl[j]);
             }
             // logits in log2 units, then probabilities and logit gradients
@@ -404,8 +399,8 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(cons
                 auto rows = [&](uint32_t base) {
                     return [&, base](uint32_t (&b)[4], int kk, int k) { ldsm4t(b, base + voff + k * TOK * PITCH + kk * 16 * PITCH + c2 * 32); };
                 };
-                if constexpr (MODE != kSumsAggregate) term_sum<E, TP, NX, FULL>(o0[2 * c2], o0[2 * c2 + 1], pt, rows(ys));
-                if constexpr (MODE != kSumsForward) term_sum<E, TP, NX, FULL>(o1[2 * c2], o1[2 * c2 + 1], dt, rows(xs));
+                if constexpr (MODE != kSumsAggregate) term_sum<E, TP, NX>(o0[2 * c2], o0[2 * c2 + 1], pt, rows(ys));
+                if constexpr (MODE != kSumsForward) term_sum<E, TP, NX>(o1[2 * c2], o1[2 * c2 + 1], dt, rows(xs));
             }
         }
     }
@@ -694,7 +689,7 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                 }
 #pragma unroll
                 for (int c2 = 0; c2 < NT / 2; ++c2)
-                    term_sum<E, TP, TM, true>(o0[2 * c2], o0[2 * c2 + 1], pt, [&](uint32_t (&b)[4], int kk, int i) { ldsm4t(b, voff + ((TA + i) * n32 + blk + kk * 16) * PITCH + c2 * 32); });
+                    term_sum<E, TP, TM>(o0[2 * c2], o0[2 * c2 + 1], pt, [&](uint32_t (&b)[4], int kk, int i) { ldsm4t(b, voff + ((TA + i) * n32 + blk + kk * 16) * PITCH + c2 * 32); });
             } else {
                 uint32_t pt[2][TP][4], dt[2][TP][4];
                 float2 cs[8];
@@ -734,9 +729,9 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                 }
 #pragma unroll
                 for (int c2 = 0; c2 < NT / 2; ++c2) {
-                    term_sum<E, TP, TA, true>(o0[2 * c2], o0[2 * c2 + 1], dt, [&](uint32_t (&b)[4], int kk, int i) { ldsm4t(b, voff + (i * n32 + blk + kk * 16) * PITCH + c2 * 32); });
+                    term_sum<E, TP, TA>(o0[2 * c2], o0[2 * c2 + 1], dt, [&](uint32_t (&b)[4], int kk, int i) { ldsm4t(b, voff + (i * n32 + blk + kk * 16) * PITCH + c2 * 32); });
                     if (MODE == kRowsKeyValue)
-                        term_sum<E, TP, TM, true>(o1[2 * c2], o1[2 * c2 + 1], pt, [&](uint32_t (&b)[4], int kk, int i) { ldsm4t(b, voff + ((TA + i) * n32 + blk + kk * 16) * PITCH + c2 * 32); });
+                        term_sum<E, TP, TM>(o1[2 * c2], o1[2 * c2 + 1], pt, [&](uint32_t (&b)[4], int kk, int i) { ldsm4t(b, voff + ((TA + i) * n32 + blk + kk * 16) * PITCH + c2 * 32); });
                 }
             }
         }

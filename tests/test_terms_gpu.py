@@ -80,3 +80,22 @@ def test_term_gradients_of_many_long_slabs_stay_fp32_accurate():
                        b1=to_np(inp["b1"][h:h + 1]), b2=to_np(inp["b2"][h:h + 1]))
     for key in ("dq", "dk", "dv"):
         assert errors(got[key][b:b + 1, h:h + 1], ref[key])["rel_l2"] <= LONG_BACKWARD, key
+
+
+def test_mixed_precision_gradients_carry_agent_features_as_two_terms_hold_them():
+    """The mixed-precision backward pass keeps V_A in fp32 (the second region of its workspace) and reads it as two bf16 terms, good to
+    2^-17 = 8e-6.  444 slabs fill 148 SMs, so that a block sums 3136 tokens, which must not lose that; the values have a mean, so rounding does not average out."""
+    w = Workload("mixed", 444, 1, 56, 56, 64, 7, "bf16", False, False, 1.0, seed=33)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(w.seed)
+    q, k, v, go = (torch.randn((w.batch, 1, w.tokens, 64), generator=g, device="cuda").to(torch.bfloat16) for _ in range(4))
+    v += 1
+    mod = make_module(w)
+    ws = mod.backward_workspace(56, 56, 49)
+    mod.backward(q, k, v, go, 56, 56, 49, workspace=ws)
+    size = w.slabs * 49 * 64 * 4
+    va = ws[size:2 * size].view(torch.float32).view(w.slabs, 49, 64)
+    for s in (0, w.slabs - 1):
+        a = q[s, 0].view(7, 8, 7, 8, 64).double().mean(dim=(1, 3)).view(49, 64).to(torch.bfloat16).double()
+        ref = torch.softmax(a @ k[s, 0].double().T / 8, dim=1) @ v[s, 0].double()
+        assert float((va[s] - ref).norm() / ref.norm()) <= 8e-6 / 4
