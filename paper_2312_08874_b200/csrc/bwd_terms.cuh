@@ -71,11 +71,18 @@ __device__ __forceinline__ void term_sum(float (&o0)[4], float (&o1)[4], const u
     add4(o1, t[1]);
 }
 
-// two fp32 -> NT packed pairs of terms
+// pack2 of finite values that never rounds up to infinity (fp32 reaches half a bf16 step past the largest bf16)
+template <typename E> __device__ __forceinline__ uint32_t pack2_finite(float lo, float hi) {
+    uint32_t w;
+    if constexpr (Elem<E>::kIsBf16) asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;\n" : "=r"(w) : "f"(hi), "f"(lo));
+    else w = pack2<E>(lo, hi);
+    return w;
+}
+// two fp32 -> NT packed pairs of terms.  Finite values are finite sums of terms; an infinite one has a NaN among its terms.
 template <typename E, int NT> __device__ __forceinline__ void split_pair(float a, float b, uint32_t (&w)[NT]) {
 #pragma unroll
     for (int i = 0; i < NT; ++i) {
-        w[i] = pack2<E>(a, b);
+        w[i] = i == 0 && NT > 1 ? pack2_finite<E>(a, b) : pack2<E>(a, b);
         if (i + 1 < NT) {
             const float2 u = unpack2<E>(w[i]);
             a -= u.x;

@@ -99,3 +99,19 @@ def test_mixed_precision_gradients_carry_agent_features_as_two_terms_hold_them()
         a = q[s, 0].view(7, 8, 7, 8, 64).double().mean(dim=(1, 3)).view(49, 64).to(torch.bfloat16).double()
         ref = torch.softmax(a @ k[s, 0].double().T / 8, dim=1) @ v[s, 0].double()
         assert float((va[s] - ref).norm() / ref.norm()) <= 8e-6 / 4
+
+
+@pytest.mark.parametrize("pool", [4, 7])
+def test_fp32_forward_of_values_at_the_end_of_the_range(pool):
+    """fp32 reaches half a bf16 step past the largest bf16: such a value must not become infinite when it is split into bf16 terms."""
+    w = Workload("range", 1, 2, 14, 14, 64, pool, "f32", True, True, 1.0, seed=34)
+    inp = make_inputs(w, bias_std=0.5, dwc_std=0.2)
+    inp["v"][0, 0, 5, 7] = torch.finfo(torch.float32).max
+    inp["v"][0, 0, 90, 9] = -torch.finfo(torch.float32).max
+    dev = {k: to_dev(v) for k, v in inp.items()}
+    out = make_module(w).forward(dev["q"], dev["k"], dev["v"], 14, 14, w.agents, b1=dev["b1"], b2=dev["b2"], dwc_weight=dev["dwc"])
+    ref = oracle_forward(w, inp)
+    for ch in (7, 9):
+        assert_close(out[:, :1, :, ch] * 1e-38, ref[:, :1, :, ch] * 1e-38, "f32", f"channel {ch}")
+    rest = [c for c in range(64) if c not in (7, 9)]
+    assert_close(out[:, :, :, rest], ref[:, :, :, rest], "f32", "the others")
