@@ -252,7 +252,7 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
 // 49 agents.)
 bool terms_forward_eligible(int n, int d) {
     const int dk = dk_of_terms(d), n32 = (n + 31) & ~31;
-    return d % 8 == 0 && 6 * n32 * (dk * 2 + 16) + 9 * dk * 4 <= 227 * 1024;
+    return d % 8 == 0 && 6 * n32 * (dk * 2 + 16) + 10 * dk * 4 <= 227 * 1024;
 }
 size_t terms_forward_bytes(int slabs, int n, int d) { return 2 * up256((size_t)slabs * n * d * 2 * 3) + up256((size_t)slabs * n * 8); }
 

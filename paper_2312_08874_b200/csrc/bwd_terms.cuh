@@ -113,6 +113,17 @@ __device__ __forceinline__ void put_dbias8(float* p, const float* v, int cnt, bo
     }
 }
 
+// Sum of the infinities and NaNs of a column: what a weighted sum over it comes to (zero: all are finite).  The terms of an infinite value
+// hold a NaN, so the forward kernels ask here where a sum is NaN and its weights are not; never on finite inputs.
+static __device__ __noinline__ float nonfinite_sum(const float* p, int stride, int count) {
+    float s = 0.f;
+    for (int i = 0; i < count; ++i) {
+        const float v = p[(size_t)i * stride];
+        if (!(fabsf(v) < INFINITY)) s += v;
+    }
+    return s;
+}
+
 // A operand (16 rows x 16 channels) from a tile in natural row order
 template <int PITCH> __device__ __forceinline__ uint32_t a_lane_offset(int lane) { return (lane & 15) * PITCH + (lane >> 4) * 16; }
 
@@ -167,7 +178,7 @@ struct BwdTermArgs {
     const void *a_t, *m_t;                 // terms [terms][slabs][n][d] of A; of V_A or dV_A
     float2* tok_stats;                     // [slabs][N]: (log2-sum-exp, row dot) of the broadcast softmax
     float2* agent_stats;                   // [slabs][n]: (log2-sum-exp, D) of the aggregation softmax
-    float *outer0, *outer1;                // fp32 [slabs][n][d]
+    float *outer0, *outer1;                // fp32 [slabs][n][d]  (rows out: V_A)
     float *row0, *row1;                    // fp32 [slabs][N][d]
     float* dbias;
     void* va_t;                            // forward sums: terms of V_A
@@ -483,6 +494,10 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(cons
                     v.x = fmaf(w.x, f, v.x);
                     v.y = fmaf(w.y, f, v.y);
                 }
+            if constexpr (sizeof(T) == 4) {
+                if (isnan(v.x) && !isnan(wt[k * nsrc])) { const float f = nonfinite_sum(y + ch, p.d, p.N); if (f != 0.f) v.x = f; }
+                if (isnan(v.y) && !isnan(wt[k * nsrc])) { const float f = nonfinite_sum(y + ch + 1, p.d, p.N); if (f != 0.f) v.y = f; }
+            }
             const size_t off = ((size_t)slab * p.n + row0 + r) * p.d + ch;
             *reinterpret_cast<float2*>(p.outer0 + off) = v;
             uint32_t w[TM];
@@ -498,8 +513,8 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 1 : 3) bwd_sums_kernel(cons
 // ------------------------------------------------------------------------------------------------------------- rows
 template <int DK, int TA, int TM> struct RowsShape {
     static constexpr int kPitch = DK * 2 + 16;
-    __host__ __device__ static constexpr int smem(int n) { return (TA + TM) * ((n + 31) & ~31) * kPitch + ((n + 31) & ~31) * 8; }      // (or 9 DK filter words, rows out)
-    __host__ __device__ static constexpr int smem_out(int n) { return (TA + TM) * ((n + 31) & ~31) * kPitch + 9 * DK * 4; }
+    __host__ __device__ static constexpr int smem(int n) { return (TA + TM) * ((n + 31) & ~31) * kPitch + ((n + 31) & ~31) * 8; }      // (rows out: 9 DK filter words and DK sums)
+    __host__ __device__ static constexpr int smem_out(int n) { return (TA + TM) * ((n + 31) & ~31) * kPitch + 10 * DK * 4; }
 };
 
 template <typename T, typename E, int DK, int NX, int TA, int TM, int TP, int MODE>
@@ -513,6 +528,8 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
     const uint32_t sm = smem_u32(smem);
     float2* st_s = reinterpret_cast<float2*>(smem + (TA + TM) * n32 * PITCH);
     float* wt_s = reinterpret_cast<float*>(st_s);
+    float* inf_s = wt_s + 9 * DK;                      // (rows out) per channel: nonfinite_sum of V_A
+    bool infinite = false;
     pdl_wait_prior();
     pdl_release_next();
     {
@@ -532,7 +549,24 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                 st_s[i] = i < p.n ? p.agent_stats[(size_t)slab * p.n + i] : make_float2(INFINITY, 0.f);
         cp_async_commit();
         cp_async_wait<0>();
-        __syncthreads();
+        if constexpr (MODE == kRowsOut) {              // a NaN among the last terms of V_A (of those that this thread has copied)
+            float2 z = make_float2(0.f, 0.f);
+            const int last = (TA + TM - 1) * n32;
+            for (int e = (threadIdx.x - last * chunks) & 255; e < n32 * chunks; e += 256) {
+                const int r = e / chunks, ch = e - r * chunks;
+                const uint4 w = *reinterpret_cast<const uint4*>(smem + (last + col_to_row(r)) * PITCH + ch * 16);
+                const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) z = ffma2(unpack2<E>(u[k]), make_float2(0.f, 0.f), z);
+            }
+            infinite = __syncthreads_or(isnan(z.x + z.y));
+            if (infinite) {
+                for (int c = threadIdx.x; c < DK; c += 256) inf_s[c] = c < p.d ? nonfinite_sum(p.outer0 + (size_t)slab * p.n * p.d + c, p.d, p.n) : 0.f;
+                __syncthreads();
+            }
+        } else {
+            __syncthreads();
+        }
     }
     const T* x = static_cast<const T*>(p.x) + (size_t)slab * p.N * p.d;
     const T* y = static_cast<const T*>(p.y) + (size_t)slab * p.N * p.d;
@@ -752,6 +786,12 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                 const float inv = 1.f / quad_sum(l[h]);
 #pragma unroll
                 for (int j = 0; j < NT; ++j) { o0[j][2 * h] *= inv; o0[j][2 * h + 1] *= inv; }
+                if (infinite && !isnan(inv))
+#pragma unroll
+                    for (int j = 0; j < NT; ++j)
+#pragma unroll
+                        for (int c = 0; c < 2; ++c)
+                            if (inf_s[j * 8 + 2 * t + c] != 0.f) o0[j][2 * h + c] = inf_s[j * 8 + 2 * t + c];
                 const int tk = tok + h * 8 + g, gy = tk / p.W, gx = tk - gy * p.W;
 #pragma unroll
                 for (int k = 0; k < 9; ++k) in[h][k] = p.wd && tk < t1 && (unsigned)(gy + k / 3 - 1) < (unsigned)p.H && (unsigned)(gx + k % 3 - 1) < (unsigned)p.W;

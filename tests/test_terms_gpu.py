@@ -115,3 +115,26 @@ def test_fp32_forward_of_values_at_the_end_of_the_range(pool):
         assert_close(out[:, :1, :, ch] * 1e-38, ref[:, :1, :, ch] * 1e-38, "f32", f"channel {ch}")
     rest = [c for c in range(64) if c not in (7, 9)]
     assert_close(out[:, :, :, rest], ref[:, :, :, rest], "f32", "the others")
+
+
+@pytest.mark.parametrize("case", [(14, 14, 64, 7), (20, 21, 24, 5), (40, 41, 64, 16)], ids=["short", "padded_channels", "two_row_blocks"])
+def test_fp32_forward_of_an_infinite_value(case):
+    """An infinite value makes its own channel infinite (NaN where infinities of both signs meet) and touches no other."""
+    H, W, d, pool = case
+    w = Workload("infinite", 1, 2, H, W, d, pool, "f32", True, True, 1.0, seed=35)
+    inp = make_inputs(w, bias_std=0.5, dwc_std=0.2)
+    clean = oracle_forward(w, inp)
+    t1, t2 = 2 * W + 2, (H - 3) * W + 5
+    inp["v"][0, 0, t1, 7] = float("inf")
+    inp["v"][0, 0, t1, 9] = -float("inf")
+    inp["v"][0, 0, t1, 11] = float("inf")
+    inp["v"][0, 0, t2, 11] = -float("inf")
+    dev = {k: to_dev(v) for k, v in inp.items()}
+    out = make_module(w).forward(dev["q"], dev["k"], dev["v"], H, W, w.agents, b1=dev["b1"], b2=dev["b2"], dwc_weight=dev["dwc"])
+    rest = [c for c in range(d) if c not in (7, 9, 11)]
+    assert_close(out[:, :, :, rest], clean[:, :, :, rest], "f32", "the other channels")
+    assert_close(out[:, 1], clean[:, 1], "f32", "the other head")
+    far = [t for t in range(w.tokens) if abs(t // W - t1 // W) > 1]        # (beside the value the depthwise term adds an infinity of its own)
+    assert torch.equal(out[0, 0, far, 7], torch.full((len(far),), float("inf"), device="cuda"))
+    assert torch.equal(out[0, 0, far, 9], torch.full((len(far),), -float("inf"), device="cuda"))
+    assert bool(torch.isnan(out[0, 0, :, 11]).all())
