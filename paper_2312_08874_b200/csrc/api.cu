@@ -13,12 +13,17 @@
 
 using namespace aa;
 
-constexpr int kHostParts = 4;
+constexpr int kHostParts = 4, kHostLanes = 4;
 
-// What a call on host buffers keeps between calls: copy streams, events and the handles of its parts.
-struct HostPipe {
+// What a call on host buffers keeps between calls: copy streams and events, and the handles of its parts.  A lane serves one stream of
+// the caller's at a time, so that calls on different streams never wait for one another.
+struct HostLane {
+    unsigned long long user;      // id of the stream whose calls it serves (0: none yet)
     cudaStream_t in, out;
     cudaEvent_t start, finish, ready[kHostParts], done[kHostParts];
+};
+struct HostPipe {
+    HostLane lane[kHostLanes];
     agent_attn_handle* part[kHostParts];
 };
 
@@ -332,16 +337,20 @@ int agent_attn_create(agent_attn_handle** out, const agent_attn_config* cfg) {
     return AA_OK;
 }
 
+static void destroy_lane(HostLane* l) {
+    if (l->in) cudaStreamDestroy(l->in);
+    if (l->out) cudaStreamDestroy(l->out);
+    if (l->start) cudaEventDestroy(l->start);
+    if (l->finish) cudaEventDestroy(l->finish);
+    for (int i = 0; i < kHostParts; ++i) {
+        if (l->ready[i]) cudaEventDestroy(l->ready[i]);
+        if (l->done[i]) cudaEventDestroy(l->done[i]);
+    }
+    memset(l, 0, sizeof(*l));
+}
 static void destroy_pipe(HostPipe* p) {
     if (!p) return;
-    if (p->in) cudaStreamDestroy(p->in);
-    if (p->out) cudaStreamDestroy(p->out);
-    if (p->start) cudaEventDestroy(p->start);
-    if (p->finish) cudaEventDestroy(p->finish);
-    for (int i = 0; i < kHostParts; ++i) {
-        if (p->ready[i]) cudaEventDestroy(p->ready[i]);
-        if (p->done[i]) cudaEventDestroy(p->done[i]);
-    }
+    for (HostLane& l : p->lane) destroy_lane(&l);
     for (agent_attn_handle* q : p->part) delete q;
     delete p;
 }
@@ -675,18 +684,13 @@ size_t agent_attn_staging_bytes(const agent_attn_handle* h, int grid_h, int grid
            align_up(heads * d * 9 * es, 256) + align_up(ws, 256);
 }
 
-// The handle's copy streams and events, and part handles of these sizes.
+// Part handles of these sizes.
 static HostPipe* host_pipe(agent_attn_handle* h, const HostParts& parts) {
     if (!h->pipe) {
         HostPipe* p = new (std::nothrow) HostPipe;
         if (!p) return nullptr;
         memset(p, 0, sizeof(*p));
-        bool ok = cudaStreamCreateWithFlags(&p->in, cudaStreamNonBlocking) == cudaSuccess &&
-                  cudaStreamCreateWithFlags(&p->out, cudaStreamNonBlocking) == cudaSuccess;
-        for (cudaEvent_t* e : {&p->start, &p->finish}) ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
-        for (int i = 0; i < kHostParts; ++i)
-            ok = ok && cudaEventCreateWithFlags(&p->ready[i], cudaEventDisableTiming) == cudaSuccess &&
-                 cudaEventCreateWithFlags(&p->done[i], cudaEventDisableTiming) == cudaSuccess;
+        bool ok = true;
         for (agent_attn_handle*& q : p->part) {
             q = new (std::nothrow) agent_attn_handle;
             if (q) part_handle(h, 0, q);
@@ -706,6 +710,38 @@ static HostPipe* host_pipe(agent_attn_handle* h, const HostParts& parts) {
         q->stage_mask = h->stage_mask;
     }
     return h->pipe;
+}
+// A lane for a call on stream `st`: the one that serves the stream already (its earlier calls precede this one on the stream anyway),
+// else one whose last call has ended, else a new one.  Null where all are at work for other streams: the call then runs in one piece
+// on its own stream.
+static HostLane* host_lane(HostPipe* p, cudaStream_t st) {
+    unsigned long long id = 0;
+    if (cudaStreamGetId(st, &id) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    ++id;                                              // (0 marks a lane without a user)
+    // another stream of this thread may be under capture: queries and creations are not part of it
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    HostLane* found = nullptr;
+    for (HostLane& l : p->lane)
+        if (!found && l.user == id) found = &l;
+    for (HostLane& l : p->lane)
+        if (!found && l.user && cudaEventQuery(l.finish) == cudaSuccess) found = &l;
+    cudaGetLastError();                                // (cudaErrorNotReady of the lanes at work)
+    for (HostLane& l : p->lane)
+        if (!found && !l.user) {
+            bool ok = cudaStreamCreateWithFlags(&l.in, cudaStreamNonBlocking) == cudaSuccess &&
+                      cudaStreamCreateWithFlags(&l.out, cudaStreamNonBlocking) == cudaSuccess;
+            for (cudaEvent_t* e : {&l.start, &l.finish}) ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+            for (int i = 0; i < kHostParts; ++i)
+                ok = ok && cudaEventCreateWithFlags(&l.ready[i], cudaEventDisableTiming) == cudaSuccess &&
+                     cudaEventCreateWithFlags(&l.done[i], cudaEventDisableTiming) == cudaSuccess;
+            if (ok) found = &l;
+            else { destroy_lane(&l); cudaGetLastError(); }
+            break;
+        }
+    if (found) found->user = id;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return found;
 }
 
 int agent_attn_forward_host(agent_attn_handle* h, const void* Q, const void* K, const void* V, const void* A,
@@ -745,14 +781,15 @@ int agent_attn_forward_host(agent_attn_handle* h, const void* Q, const void* K, 
         if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) { cudaGetLastError(); split = false; }
     }
     HostPipe* pipe = split ? host_pipe(h, parts) : nullptr;
-    if (!pipe) { parts.count = 1; parts.size[0] = parts.units; }
+    HostLane* lane = pipe ? host_lane(pipe, st) : nullptr;
+    if (!lane) { parts.count = 1; parts.size[0] = parts.units; }
     cudaError_t e = cudaSuccess;
 #define AA_STEP(x) do { if (e == cudaSuccess) e = (x); } while (0)
-    cudaStream_t cin = pipe ? pipe->in : st, cout = pipe ? pipe->out : st;
-    if (pipe) {
-        AA_STEP(cudaEventRecord(pipe->start, st));                 // the staging memory is the caller's, in the order of its stream
-        AA_STEP(cudaStreamWaitEvent(cin, pipe->start, 0));
-        AA_STEP(cudaStreamWaitEvent(cout, pipe->start, 0));
+    cudaStream_t cin = lane ? lane->in : st, cout = lane ? lane->out : st;
+    if (lane) {
+        AA_STEP(cudaEventRecord(lane->start, st));                 // the staging memory is the caller's, in the order of its stream
+        AA_STEP(cudaStreamWaitEvent(cin, lane->start, 0));
+        AA_STEP(cudaStreamWaitEvent(cout, lane->start, 0));
     }
     const bool by_heads = h->cfg.batch == 1;
     int launches = 0, rc = AA_OK;
@@ -771,33 +808,34 @@ int agent_attn_forward_host(agent_attn_handle* h, const void* Q, const void* K, 
             in[i] = src[i] ? dst : nullptr;
             if (i != kO && src[i] && len) AA_STEP(cudaMemcpyAsync(dst, static_cast<const char*>(src[i]) + off, len, cudaMemcpyHostToDevice, cin));
         }
-        if (pipe) {
-            AA_STEP(cudaEventRecord(pipe->ready[k], cin));
-            AA_STEP(cudaStreamWaitEvent(st, pipe->ready[k], 0));
+        if (lane) {
+            AA_STEP(cudaEventRecord(lane->ready[k], cin));
+            AA_STEP(cudaStreamWaitEvent(st, lane->ready[k], 0));
         }
         if (e != cudaSuccess) break;
         agent_attn_bias db;
         db.b1 = in[kB1];
         db.b2 = in[kB2];
-        agent_attn_handle* ph = pipe ? pipe->part[k] : h;
+        agent_attn_handle* ph = lane ? pipe->part[k] : h;
         rc = agent_attn_forward(ph, in[kQ], in[kK], in[kV], in[kA], grid_h, grid_w, n_agents, bias ? &db : nullptr, in[kW], const_cast<void*>(in[kO]), dWs,
                                 ws_bytes, stream);
         launches += ph->launches;
-        if (rc != AA_OK && pipe) memcpy(h->err, ph->err, sizeof(h->err));
+        if (rc != AA_OK && lane) memcpy(h->err, ph->err, sizeof(h->err));
         if (rc != AA_OK) break;
         size_t off, len;
         range(kO, &off, &len);
-        if (pipe) {
-            AA_STEP(cudaEventRecord(pipe->done[k], st));
-            AA_STEP(cudaStreamWaitEvent(cout, pipe->done[k], 0));
+        if (lane) {
+            AA_STEP(cudaEventRecord(lane->done[k], st));
+            AA_STEP(cudaStreamWaitEvent(cout, lane->done[k], 0));
         }
         AA_STEP(cudaMemcpyAsync(static_cast<char*>(out) + off, dev[kO] + off, len, cudaMemcpyDeviceToHost, cout));
     }
-    if (pipe) {                                                    // (after an error too: the caller's stream ends after the copies)
-        cudaError_t f = cudaEventRecord(pipe->finish, cin);
-        if (f == cudaSuccess) f = cudaStreamWaitEvent(st, pipe->finish, 0);
-        if (f == cudaSuccess) f = cudaEventRecord(pipe->finish, cout);
-        if (f == cudaSuccess) f = cudaStreamWaitEvent(st, pipe->finish, 0);
+    if (lane) {                                                    // (after an error too: the caller's stream ends after the copies)
+        // (`finish` ends as work of `cout` that follows `cin`'s, so that a query of it speaks for the whole lane)
+        cudaError_t f = cudaEventRecord(lane->finish, cin);
+        if (f == cudaSuccess) f = cudaStreamWaitEvent(cout, lane->finish, 0);
+        if (f == cudaSuccess) f = cudaEventRecord(lane->finish, cout);
+        if (f == cudaSuccess) f = cudaStreamWaitEvent(st, lane->finish, 0);
         AA_STEP(f);
     }
 #undef AA_STEP

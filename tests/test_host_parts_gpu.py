@@ -36,3 +36,40 @@ def test_split_host_call_matches_oracle(case):
     torch.cuda.synchronize()
     assert all(torch.equal(o, out) for _, _, o in lanes)
     assert mod.query_status() == 0
+
+
+def test_split_host_calls_on_different_streams_do_not_wait_for_one_another():
+    w = Workload("host", 8, 2, 56, 56, 64, 7, "bf16", True, True, 1.0, seed=901)
+    inp = make_inputs(w, bias_std=0.5, dwc_std=0.2)
+    mod = make_module(w)
+    pin = {k: v.pin_memory() for k, v in inp.items()}
+    args = (pin["q"], pin["k"], pin["v"], w.grid_h, w.grid_w, w.agents)
+    ops = dict(b1=pin["b1"], b2=pin["b2"], dwc_weight=pin["dwc"])
+    want = mod.forward_host(*args, **ops)
+    assert mod.last_launch_count() > 3, "expected several parts"
+    lanes = [(torch.cuda.Stream(), torch.empty(mod.staging_bytes(w.grid_h, w.grid_w, w.agents), dtype=torch.uint8, device="cuda"), torch.empty_like(want).pin_memory())
+             for _ in range(6)]
+
+    def call(s, stg, o):
+        mod.forward_host(*args, **ops, out=o, stream=s, synchronize=False, staging=stg)
+
+    for lane in lanes[:2]:                                 # both streams have called before
+        call(*lane)
+    torch.cuda.synchronize()
+    busy, idle = lanes[:2]
+    with torch.cuda.stream(busy[0]):
+        torch.cuda._sleep(1_000_000_000)                   # half a second of work before its call
+    call(*busy)
+    ended = torch.cuda.Event()
+    ended.record(busy[0])
+    call(*idle)
+    idle[0].synchronize()
+    assert not ended.query(), "the call on the idle stream waited for the busy one"
+    # more streams at work than the handle keeps copy streams for
+    for s, _, _ in lanes:
+        with torch.cuda.stream(s):
+            torch.cuda._sleep(2_000_000)
+    for lane in lanes + lanes:
+        call(*lane)
+    torch.cuda.synchronize()
+    assert all(torch.equal(o, want) for _, _, o in lanes) and mod.query_status() == 0
