@@ -232,9 +232,10 @@ size_t agent_attn_staging_bytes(const agent_attn_handle* h, int grid_h, int grid
  * of out, in order on `stream`; the caller synchronises the stream before reading `out`.  Large
  * calls on pinned memory are cut into up to four parts whose copies run on two streams of the
  * library's, tied to `stream` by events, so that copies and kernels of different parts overlap.
- * The handle keeps up to four such pairs of streams, each for the calls of one `stream`: calls on
- * different streams do not wait for one another.  (With four streams at work, calls on a fifth run
- * in one piece on that stream.) */
+ * Calls on different streams do not wait for one another: the handle keeps up to four such pairs
+ * of streams, each for the calls of one `stream`, and a call runs in one piece on its own stream
+ * where the call before it was on another one or such a call is still in flight (the calls then
+ * overlap one another). */
 int agent_attn_forward_host(agent_attn_handle* h,
                             const void* Q, const void* K, const void* V, const void* A,
                             int grid_h, int grid_w, int n_agents,

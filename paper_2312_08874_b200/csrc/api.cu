@@ -24,6 +24,7 @@ struct HostLane {
 };
 struct HostPipe {
     HostLane lane[kHostLanes];
+    unsigned long long last;      // id of the stream of the last call
     agent_attn_handle* part[kHostParts];
 };
 
@@ -711,35 +712,46 @@ static HostPipe* host_pipe(agent_attn_handle* h, const HostParts& parts) {
     }
     return h->pipe;
 }
+// Copy streams and events of a lane, made when it first cuts a call (a stream made while others work can take a millisecond).
+static bool lane_ready(HostLane* l) {
+    if (l->done[kHostParts - 1]) return true;
+    bool ok = cudaStreamCreateWithFlags(&l->in, cudaStreamNonBlocking) == cudaSuccess && cudaStreamCreateWithFlags(&l->out, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaEventCreateWithFlags(&l->start, cudaEventDisableTiming) == cudaSuccess;
+    for (int i = 0; i < kHostParts; ++i)
+        ok = ok && cudaEventCreateWithFlags(&l->ready[i], cudaEventDisableTiming) == cudaSuccess &&
+             cudaEventCreateWithFlags(&l->done[i], cudaEventDisableTiming) == cudaSuccess;
+    return ok;
+}
 // A lane for a call on stream `st`: the one that serves the stream already (its earlier calls precede this one on the stream anyway),
-// else one whose last call has ended, else a new one.  Null where all are at work for other streams: the call then runs in one piece
-// on its own stream.
-static HostLane* host_lane(HostPipe* p, cudaStream_t st) {
+// else one whose last call has ended, else a new one.  Null where all are at work for other streams.  *alone: the last call was on this
+// stream too, no other lane is at work, and this one can cut the call.
+static HostLane* host_lane(HostPipe* p, cudaStream_t st, bool* alone) {
+    *alone = false;
     unsigned long long id = 0;
     if (cudaStreamGetId(st, &id) != cudaSuccess) { cudaGetLastError(); return nullptr; }
     ++id;                                              // (0 marks a lane without a user)
     // another stream of this thread may be under capture: queries and creations are not part of it
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-    HostLane* found = nullptr;
+    HostLane *own = nullptr, *ended = nullptr, *unused = nullptr;
+    bool busy = p->last && p->last != id;
+    p->last = id;
     for (HostLane& l : p->lane)
-        if (!found && l.user == id) found = &l;
-    for (HostLane& l : p->lane)
-        if (!found && l.user && cudaEventQuery(l.finish) == cudaSuccess) found = &l;
-    cudaGetLastError();                                // (cudaErrorNotReady of the lanes at work)
-    for (HostLane& l : p->lane)
-        if (!found && !l.user) {
-            bool ok = cudaStreamCreateWithFlags(&l.in, cudaStreamNonBlocking) == cudaSuccess &&
-                      cudaStreamCreateWithFlags(&l.out, cudaStreamNonBlocking) == cudaSuccess;
-            for (cudaEvent_t* e : {&l.start, &l.finish}) ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
-            for (int i = 0; i < kHostParts; ++i)
-                ok = ok && cudaEventCreateWithFlags(&l.ready[i], cudaEventDisableTiming) == cudaSuccess &&
-                     cudaEventCreateWithFlags(&l.done[i], cudaEventDisableTiming) == cudaSuccess;
-            if (ok) found = &l;
-            else { destroy_lane(&l); cudaGetLastError(); }
-            break;
+        if (!l.user) unused = &l;
+        else if (l.user == id) own = &l;
+        else if (cudaEventQuery(l.finish) == cudaSuccess) ended = &l;
+        else busy = true;
+    HostLane* found = own ? own : ended;
+    if (!found && unused && cudaEventCreateWithFlags(&unused->finish, cudaEventDisableTiming) == cudaSuccess) found = unused;
+    if (found) {
+        found->user = id;
+        *alone = !busy && lane_ready(found);
+        if (!busy && !*alone) {                        // (no copy streams to be had)
+            destroy_lane(found);
+            found = nullptr;
         }
-    if (found) found->user = id;
+    }
+    cudaGetLastError();                                // (cudaErrorNotReady of the lanes at work)
     cudaThreadExchangeStreamCaptureMode(&mode);
     return found;
 }
@@ -781,7 +793,11 @@ int agent_attn_forward_host(agent_attn_handle* h, const void* Q, const void* K, 
         if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) { cudaGetLastError(); split = false; }
     }
     HostPipe* pipe = split ? host_pipe(h, parts) : nullptr;
-    HostLane* lane = pipe ? host_lane(pipe, st) : nullptr;
+    // Calls in flight on several streams overlap one another's copies and kernels by themselves; parts would only cost them (64 slabs of
+    // 3136 tokens, forty calls: two streams 1.66 ms a call in parts, 1.54 in one piece; one stream 1.77 and 1.95).
+    bool alone = false;
+    HostLane* const own = pipe ? host_lane(pipe, st, &alone) : nullptr;
+    HostLane* const lane = alone ? own : nullptr;
     if (!lane) { parts.count = 1; parts.size[0] = parts.units; }
     cudaError_t e = cudaSuccess;
 #define AA_STEP(x) do { if (e == cudaSuccess) e = (x); } while (0)
@@ -837,6 +853,8 @@ int agent_attn_forward_host(agent_attn_handle* h, const void* Q, const void* K, 
         if (f == cudaSuccess) f = cudaEventRecord(lane->finish, cout);
         if (f == cudaSuccess) f = cudaStreamWaitEvent(st, lane->finish, 0);
         AA_STEP(f);
+    } else if (own) {
+        AA_STEP(cudaEventRecord(own->finish, st));                 // (other streams' calls see this one in flight)
     }
 #undef AA_STEP
     if (rc != AA_OK) return rc;

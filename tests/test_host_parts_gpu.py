@@ -53,16 +53,18 @@ def test_split_host_calls_on_different_streams_do_not_wait_for_one_another():
     def call(s, stg, o):
         mod.forward_host(*args, **ops, out=o, stream=s, synchronize=False, staging=stg)
 
-    for lane in lanes[:2]:                                 # both streams have called before
+    busy, idle = lanes[:2]
+    for lane in (idle, busy, busy):                        # both streams have called before
         call(*lane)
     torch.cuda.synchronize()
-    busy, idle = lanes[:2]
     with torch.cuda.stream(busy[0]):
         torch.cuda._sleep(1_000_000_000)                   # half a second of work before its call
     call(*busy)
+    assert mod.last_launch_count() > 3, "expected several parts"
     ended = torch.cuda.Event()
     ended.record(busy[0])
     call(*idle)
+    assert mod.last_launch_count() == 3, "beside a call in flight: one piece"
     idle[0].synchronize()
     assert not ended.query(), "the call on the idle stream waited for the busy one"
     # more streams at work than the handle keeps copy streams for
