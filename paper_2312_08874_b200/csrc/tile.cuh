@@ -136,16 +136,24 @@ __device__ __forceinline__ void tile_values(float (&o)[TileGeom<DK>::kMT][TileGe
 // Running state of the softmax of a warp's rows (row index: m-tile, half).  `ref` is the exponent reference in log2
 // units, taken from the row's first block; it moves only when a logit exceeds it by more than 8 (so the products are
 // rescaled rarely, and probabilities stay below 2^8: inside fp16).  `lim` is that 8, or -inf while the row has no weight.
+// The sums of the rounded probabilities come out of one more MMA per k step, against ones (every column of it holds them).
 template <int MT> struct SoftRows {
     float ref[MT][2], lim[MT][2];
-    float2 sum[MT][2];
+    float sum[MT][4];
     __device__ __forceinline__ void init() {
 #pragma unroll
         for (int m = 0; m < MT; ++m)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) { ref[m][h] = 0.f; lim[m][h] = -INFINITY; sum[m][h] = make_float2(0.f, 0.f); }
+            for (int h = 0; h < 2; ++h) { ref[m][h] = 0.f; lim[m][h] = -INFINITY; sum[m][2 * h] = sum[m][2 * h + 1] = 0.f; }
     }
-    __device__ __forceinline__ float total(int m, int h) const { return quad_sum(sum[m][h].x + sum[m][h].y); }
+    __device__ __forceinline__ float total(int m, int h) const { return sum[m][2 * h]; }
+    template <typename T> __device__ __forceinline__ void add(const uint32_t (&p)[MT][2][4]) {
+        constexpr uint32_t kOnes = Elem<T>::kIsBf16 ? 0x3f803f80u : 0x3c003c00u;
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+            for (int m = 0; m < MT; ++m) mma_acc<T>(sum[m], p[m][ks], kOnes, kOnes);
+    }
 };
 
 // Logits of one block -> probabilities as MMA operands.  x = s * c1 + bias * log2(e) - ref; columns at and past `valid`
@@ -205,8 +213,8 @@ __device__ __forceinline__ void tile_softmax(float (&s)[TileGeom<DK>::kMT][4][4]
                 const float f = first ? 1.f : fast_exp2(-by);
                 if (m > -INFINITY) st.lim[mt][h] = 8.f;
                 st.ref[mt][h] += by;
-                st.sum[mt][h].x *= f;
-                st.sum[mt][h].y *= f;
+                st.sum[mt][2 * h] *= f;
+                st.sum[mt][2 * h + 1] *= f;
 #pragma unroll
                 for (int c = 0; c < G::kNT; ++c) { o[mt][c][2 * h] *= f; o[mt][c][2 * h + 1] *= f; }
 #pragma unroll
@@ -220,9 +228,9 @@ __device__ __forceinline__ void tile_softmax(float (&s)[TileGeom<DK>::kMT][4][4]
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const float2 e = make_float2(fast_exp2(x[mt][h][j].x), fast_exp2(x[mt][h][j].y));
-                st.sum[mt][h] = fadd2(st.sum[mt][h], e);
                 p[mt][j >> 1][(j & 1) * 2 + h] = pack2<T>(e.x, e.y);
             }
+    st.template add<T>(p);
 }
 
 }  // namespace aa

@@ -33,3 +33,16 @@ def test_tile_edges_match_oracle(case):
     for (b, h), ref in zip(slabs, oracle_forward(w, inp, slabs=slabs)):
         assert_close(out[b:b + 1, h:h + 1], ref, dtype, f"{case} slab {(b, h)}")
     assert torch.equal(out, gpu_forward(mod, w, inp)), "bit-reproducible"
+
+
+@pytest.mark.parametrize("case", [(2, 2, 14, 14, 64, 7, "bf16"), (1, 2, 45, 45, 64, 11, "f16"), (1, 1, 33, 32, 40, 16, "bf16")], ids=["one_kernel", "three_kernels", "d40"])
+def test_weights_and_their_sums_agree(case):
+    """Values that are all one, less themselves through the depthwise term: what is left is how far the rounded weights are from adding up to
+    their normaliser.  Both are sums of the same 16-bit numbers, rounded once per 16 of at most 256: 2 x 16 x 2^-23 = 4e-6.  (A normaliser of
+    the weights before rounding leaves 2^-9 / sqrt(agents) in bf16.)"""
+    B, heads, H, W, d, pool, dtype = case
+    w = Workload("weights", B, heads, H, W, d, pool, dtype, True, True, 1.0, seed=36)
+    inp = make_inputs(w, bias_std=0.5)
+    inp["v"].fill_(1)
+    inp["dwc"].zero_()[:, :, 1, 1] = -1
+    assert float(gpu_forward(make_module(w), w, inp).abs().max()) <= 4e-6
