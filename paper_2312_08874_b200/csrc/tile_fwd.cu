@@ -71,15 +71,16 @@ cudaError_t launch_tile_aggregate(int dtype, TileArgs a, int sm_count, bool depe
     a.b2 = nullptr;
     // Parts of the token axis (one block each, a cluster per slab).  Two blocks share an SM and hide each other's
     // latencies, so the best split is the one with the shortest blocks in the fewest waves; a block's start and merge count as
-    // 128 tokens.  Clusters of sixteen are for few slabs with long token axes (eight slabs of 8775 tokens: 42 us in eights, 28 us):
-    // two such blocks share an SM, so that a cluster asks for eight SMs of one GPC.
+    // 128 tokens.  A cluster of sixteen asks for eight SMs of one GPC (two blocks share an SM): fourteen of them are resident at once, the
+    // fifteenth waits for one to end (49 agents, whole forward pass, eights against sixteens: 14 slabs of 8775 tokens 83 and 69 us, 16 slabs
+    // 85 and 92 us; 16640 tokens 115 and 98, 124 and 125 us; 2800 tokens 37 and 35, 38 and 44 us).
     int best = 1;
     long long best_cost = 0;
     const int smem = agg_smem(dk.dk, a.kg, 8);
     for (int c = 1; c <= 16; c *= 2) {
         const int tokens = up32((a.N + c - 1) / c);
         if (c > 1 && (tokens < 64 || c * a.kg > 32)) break;
-        if (c == 16 && (a.slabs * rb > 8 || smem > 112 * 1024)) break;
+        if (c == 16 && (a.slabs * rb > 14 || smem > 112 * 1024)) break;
         const long long blocks = (long long)a.slabs * rb * c;
         const long long cost = ((blocks + 2LL * sm_count - 1) / (2LL * sm_count)) * (tokens + 128LL);
         if (c == 1 || cost < best_cost) { best = c; best_cost = cost; }

@@ -19,6 +19,8 @@ SHAPES = [
     (1, 1, 40, 41, 32, 13, "bf16", True, False),     # 169 agents: two row blocks, bias rows read from global memory
     (1, 1, 33, 32, 128, 16, "bf16", True, True),     # 256 agents of 128 channels
     (160, 2, 11, 13, 64, 7, "bf16", True, True),     # more slabs than resident blocks: a cluster of one
+    (7, 2, 23, 70, 64, 5, "f16", True, True),        # fourteen slabs: clusters of sixteen, the last one without tokens
+    (5, 3, 23, 70, 64, 5, "f16", True, True),        # fifteen: clusters of eight
 ]
 
 
