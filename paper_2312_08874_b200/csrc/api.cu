@@ -570,7 +570,7 @@ static int forward_impl(agent_attn_handle* h, const void* Q, const void* K, cons
         TileArgs t = tile_args(h, grid_h, grid_w, n_agents, cl);
         t.q = Q; t.k = K; t.v = V; t.a = A ? A : ws + w.a_off; t.va = ws + w.va_off; t.pool = p;
         t.b1 = b1; t.b2 = b2; t.wd = dwc_weight; t.out = out;
-        const cudaError_t e = launch_tile_forward(h->cfg.dtype, t, h->sm_count, h->cfg.path != AA_PATH_UNFUSED && tile_one_kernel(t), st, &h->launches);
+        const cudaError_t e = launch_tile_forward(h->cfg.dtype, t, h->sm_count, h->cfg.path != AA_PATH_UNFUSED && tile_one_kernel(t, h->sm_count), st, &h->launches);
         if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "forward launch failed: %s", cudaGetErrorString(e));
         return AA_OK;
     }

@@ -110,7 +110,7 @@ struct TileArgs {
 cudaError_t launch_tile_forward(int dtype, TileArgs a, int sm_count, bool one_kernel, cudaStream_t st, int* launches);
 cudaError_t launch_tile_aggregate(int dtype, TileArgs a, int sm_count, bool dependent, cudaStream_t st);
 cudaError_t launch_tile_broadcast(int dtype, TileArgs a, int sm_count, bool dependent, cudaStream_t st);
-bool tile_one_kernel(const TileArgs& a);                 // the shape can run as one kernel
+bool tile_one_kernel(const TileArgs& a, int sm_count);   // short grids: one kernel for the whole pass
 
 // Whole module (Eq. 6) in one persistent kernel for small agent counts (n <= 64, d = 64,
 // block pooling, W <= 64).  Blocks take tasks from a device-side queue: "G" tasks pool their token

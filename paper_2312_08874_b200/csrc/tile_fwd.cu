@@ -54,6 +54,21 @@ int bias_align(int row) { return row % 8 == 0 ? 8 : 1; }
 int bias_kind(const void* b, int align) { return !b ? 0 : align == 8 ? 1 : 2; }
 int up32(int x) { return (x + 31) & ~31; }
 
+// The one-kernel path: blocks of four warps (up to 64 agents; eight warps have rows for 128), registers for sixteen warps an SM either way.
+struct SlabPlan {
+    int warps, rg, kg, smem;
+    long long slots;               // blocks resident at once
+};
+SlabPlan slab_plan(const TileArgs& a, int sm_count) {
+    const DkInfo dk = dk_of(a.d);
+    SlabPlan s;
+    s.warps = a.n <= 64 ? 4 : 8;
+    s.rg = (a.n + 15) / 16;
+    s.kg = s.warps == 8 || s.rg > 2 ? 1 : s.rg == 2 ? 2 : 4;
+    s.smem = std::max(agg_smem(dk.dk, s.kg, s.warps), bc_smem(dk.dk, a, s.warps));
+    s.slots = std::min<long long>(16 / s.warps, 227 * 1024 / (s.smem + 1024)) * sm_count;
+    return s;
+}
 // Row and key groups of an aggregation block: at most eight warps, all of them with rows.
 int agg_rows(const TileArgs& a, const DkInfo& dk, TileArgs* out) {
     const int rb = (a.n + 8 * 16 - 1) / (8 * 16);
@@ -126,32 +141,35 @@ cudaError_t launch_tile_broadcast(int dtype, TileArgs a, int sm_count, bool depe
     return dispatch(kTileBroadcast, dtype, dk.dk, bias_kind(a.b2, bias_align(a.n)), a, l);
 }
 
-// Blocks of four warps (up to 64 agents) or eight: registers for sixteen warps an SM either way.
-bool tile_one_kernel(const TileArgs& a) {
-    const DkInfo dk = dk_of(a.d);
-    return a.N <= 1024 && a.n <= 128 && bc_smem(dk.dk, a, a.n <= 64 ? 4 : 8) <= 113 * 1024;
+// It saves two launches and the agents' way through memory; a slab's chain runs in at most eight blocks, so the longer the grid, the less it
+// saves (three kernels against one, 49 agents of 64 channels, 1 to 384 slabs: 196 tokens 1.18 to 1.32 times its time, 400 tokens 0.89 to
+// 1.07, 784 tokens 0.77 to 1.04; 64 agents, 784 tokens 0.88 to 1.23).  Slabs beyond the resident blocks start when others end, which only the
+// shortest chains can afford (384 slabs on 296 slots: 49 agents of 128 channels, 49 tokens 1.23, 100 tokens 0.77, 196 tokens 0.73; 81
+// agents of 64 channels, 100 tokens 1.28, 196 tokens 1.02, 256 tokens 0.88).
+bool tile_one_kernel(const TileArgs& a, int sm_count) {
+    if (a.N > 1024 || a.n > 128) return false;
+    const SlabPlan s = slab_plan(a, sm_count);
+    return bc_smem(dk_of(a.d).dk, a, s.warps) <= 113 * 1024 && (a.slabs <= s.slots || a.N <= (a.n > 64 ? 196 : 64));
 }
 
 cudaError_t launch_tile_forward(int dtype, TileArgs a, int sm_count, bool one_kernel, cudaStream_t st, int* launches) {
     if (one_kernel) {
-        const DkInfo dk = dk_of(a.d);
-        const int warps = a.n <= 64 ? 4 : 8;
-        a.rg = (a.n + 15) / 16;
-        a.kg = warps == 8 || a.rg > 2 ? 1 : a.rg == 2 ? 2 : 4;
+        const SlabPlan s = slab_plan(a, sm_count);
+        a.rg = s.rg;
+        a.kg = s.kg;
         TileLaunch l;
-        l.smem = std::max(agg_smem(dk.dk, a.kg, warps), bc_smem(dk.dk, a, warps));
+        l.smem = s.smem;
         // blocks per slab: as many as are resident at once
-        const long long slots = std::min<long long>(16 / warps, 227 * 1024 / (l.smem + 1024)) * sm_count;
         int c = 1;
-        while (c < 8 && a.slabs * 2LL * c <= slots && a.N > 32 * c) c *= 2;
+        while (c < 8 && a.slabs * 2LL * c <= s.slots && a.N > 32 * c) c *= 2;
         a.agg_tokens = up32((a.N + c - 1) / c);
         l.grid = dim3(c, a.slabs);
-        l.threads = warps * 32;
+        l.threads = s.warps * 32;
         l.cluster = c;
         l.dependent = true;
         l.stream = st;
         *launches += 1;
-        return dispatch(kTileSlab, dtype, dk.dk, !a.b1 && !a.b2 ? 0 : a.b1 && a.b2 && a.N % 8 == 0 && a.n % 8 == 0 ? 1 : 2, a, l);
+        return dispatch(kTileSlab, dtype, dk_of(a.d).dk, !a.b1 && !a.b2 ? 0 : a.b1 && a.b2 && a.N % 8 == 0 && a.n % 8 == 0 ? 1 : 2, a, l);
     }
     if (a.pool) {
         // a warp per window, or (few windows, more than 32 tokens each) a block per window

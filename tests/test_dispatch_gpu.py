@@ -1,4 +1,5 @@
-"""Either side of the lines between the tensor-memory kernels and the register-tiled ones, against the fp64 oracle."""
+"""Either side of the lines between the tensor-memory kernels and the register-tiled ones, and between one kernel and three, against the fp64
+oracle."""
 import pytest
 
 from paper_2312_08874_b200 import Workload, make_inputs
@@ -13,6 +14,11 @@ SHAPES = [
     (20, 2, 47, 80, 64, 16, 4),       # short axis, 150400 tokens in all: tensor memory
     (1, 2, 64, 128, 64, 12, 4),       # half-filled blocks on a long axis: tensor memory
     (1, 2, 64, 128, 32, 12, 3),       # and of few channels: register tiles
+    (2, 1, 31, 33, 64, 8, 1),         # 1023 tokens: one kernel
+    (2, 1, 15, 69, 64, 8, 3),         # 1035 on a grid too wide for the streaming kernels: three
+    (48, 6, 9, 9, 128, 5, 1),         # slabs all resident: one kernel
+    (50, 6, 9, 9, 128, 5, 3),         # more than fit: three
+    (50, 6, 8, 8, 128, 5, 1),         # but not on the shortest grids
 ]
 
 
