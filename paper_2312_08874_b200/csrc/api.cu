@@ -81,19 +81,22 @@ bool umma_shape(const agent_attn_handle* h, int n_tokens, int n_agents) {
     return !use_simt(h) && auto_like(h) &&
            aggregate_umma_eligible(h->cfg.dtype, n_agents, n_tokens, h->cfg.head_dim, true);
 }
-// They pad agents to 128 and channels to 64 and pay a start and a separate merge; the register tiles pay for neither.  Where the agents and
-// channels fill the padded blocks they win as soon as the token axis is long or there is work for several tiles of every block (256 agents
-// of 64 channels: 24 slabs of 7920 tokens 127 us against 163 us, 128 slabs of 4096 tokens 319 against 374; 32 slabs of 4096 tokens 105 by
-// either).  Elsewhere they win on long axes only (144 agents, 16 slabs of 16384 tokens: 162 us against 207 us), and not with few channels
-// and either many tokens or half-filled blocks (40 channels, 64 slabs of 10400 tokens: 315 us against 287 us; 144 agents of 32 channels, the
-// same: 359 against 241).
+// They pad agents to 128 and channels to 64 and pay a start and a separate merge; the register tiles pay for neither.  Register tiles
+// against these, times of the whole pass (above 1: these are faster), bf16 with biases and depthwise term:
+//   256 agents of 56 or 64 channels, the blocks filled: 6144 tokens and more 1.07 to 1.75; shorter axes once there is a tile for every
+//     SM (3072 tokens: 8 slabs 0.93 to 0.96, 16 slabs 1.26 to 1.32, 32 slabs 1.01)
+//   144 agents of 64 channels, half-filled: 6144 tokens, 1 to 16 slabs 0.99 to 1.17, 32 and 64 slabs 0.93 to 0.98; 16384 tokens 1.16
+//     to 1.39, 32 slabs 0.97
+//   256 agents of 40 channels: 7920 tokens 0.92 to 1.17, 16384 tokens 1.10 to 1.30; 24 slabs of 12960 tokens 1.05, 32 slabs 0.82 and 0.89
+//     (four blocks a slab: 20 SMs idle)
+//   256 agents of 32 channels 0.58 to 1.02 (one slab of 16384 tokens 1.12); 144 agents of 32 or 40 channels 0.50 to 1.02
 bool use_umma(const agent_attn_handle* h, int n_tokens, int n_agents) {
     if (n_tokens < 2048 || !umma_shape(h, n_tokens, n_agents)) return false;
-    const int d = h->cfg.head_dim;
-    const long long work = (long long)h->cfg.batch * h->cfg.heads * n_tokens;
+    const int d = h->cfg.head_dim, slabs = h->cfg.batch * h->cfg.heads;
+    const long long work = (long long)slabs * n_tokens;
     const bool filled = n_agents * 4 >= (n_agents + 127) / 128 * 128 * 3;
-    if (filled && d > 48) return n_tokens >= 6144 || work >= 150000;
-    return n_tokens >= 8192 && (filled || d > 32) && (d > 48 || work < 400000);
+    if (d > 48) return filled ? n_tokens >= 6144 || work >= 32768 : n_tokens >= 8192 || (n_tokens >= 6144 && slabs <= 16);
+    return filled && d > 32 && n_tokens >= 8192 && slabs <= 24;
 }
 
 AggPlan plan_for(const agent_attn_handle* h, int n_tokens, int n_agents) {

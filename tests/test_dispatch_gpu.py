@@ -14,6 +14,12 @@ SHAPES = [
     (20, 2, 47, 80, 64, 16, 4),       # short axis, 150400 tokens in all: tensor memory
     (1, 2, 64, 128, 64, 12, 4),       # half-filled blocks on a long axis: tensor memory
     (1, 2, 64, 128, 32, 12, 3),       # and of few channels: register tiles
+    (4, 4, 32, 64, 64, 16, 4),        # filled blocks, a tile for every SM: tensor memory
+    (3, 5, 32, 64, 64, 16, 3),        # fewer: register tiles
+    (1, 1, 64, 96, 64, 12, 4),        # half-filled blocks, 6144 tokens of few slabs: tensor memory
+    (17, 1, 64, 96, 64, 12, 3),       # of many: register tiles
+    (2, 1, 64, 128, 40, 16, 4),       # filled with agents, 40 channels: tensor memory
+    (2, 1, 64, 128, 32, 16, 3),       # 32: register tiles
     (2, 1, 31, 33, 64, 8, 1),         # 1023 tokens: one kernel
     (2, 1, 15, 69, 64, 8, 3),         # 1035 on a grid too wide for the streaming kernels: three
     (48, 6, 9, 9, 128, 5, 1),         # slabs all resident: one kernel
