@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_cons
         const int row = 128 * mb + 32 * (warp & 3) + lane;     // agent row (padded)
         const uint32_t lane_base = ((uint32_t)(32 * (warp & 3))) << 16;
         const uint32_t tO = pp.tmem + TM_O + 64 * (2 * mb + c) + lane_base;
-        float m_ref = -INFINITY, l = 0.f;
+        float m_ref = kRefFloor, l = 0.f;
         bool started = false;
         for (int t = 0; t < tiles; ++t) {
             const int b = t & 1, s = t % STAGES;
@@ -223,8 +223,8 @@ __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_cons
                 float mx0 = sv[0], mx1 = sv[1];
 #pragma unroll
                 for (int k = 2; k < 30; k += 4) { mx0 = max3(mx0, sv[k], sv[k + 1]); mx1 = max3(mx1, sv[k + 2], sv[k + 3]); }
-                const float mx = fmaxf(max3(mx0, mx1, fmaxf(sv[30], sv[31])), kRefFloor);
-                if (mx > m_ref + kTau) {                       // also the first tile (m_ref = -inf)
+                const float mx = max3(mx0, mx1, fmaxf(sv[30], sv[31]));
+                if (mx > m_ref + kTau) {                       // also the first tile with an open key (m_ref = kRefFloor)
                     corr = fast_exp2((m_ref - mx) * kLog2e);
                     resc = started;
                     m_ref = mx;

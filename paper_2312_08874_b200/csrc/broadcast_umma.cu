@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
         const size_t so = (size_t)p.lout.st;
         for (int i = 0; i < tiles; ++i) {
             const int tok = (i0 + i) * QT + row;
-            float m_ref = -INFINITY, l = 0.f;
+            float m_ref = kRefFloor, l = 0.f;
             bool started = false;
             for (int a = 0; a < MB; ++a) {
                 const int j = i * MB + a, b = j & 1;
@@ -290,8 +290,8 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
                     float mx0 = sv[0], mx1 = sv[1];
 #pragma unroll
                     for (int k = 2; k < 30; k += 4) { mx0 = max3(mx0, sv[k], sv[k + 1]); mx1 = max3(mx1, sv[k + 2], sv[k + 3]); }
-                    const float mx = fmaxf(max3(mx0, mx1, fmaxf(sv[30], sv[31])), kRefFloor);
-                    if (mx > m_ref + kTau) {                   // also the first step (m_ref = -inf)
+                    const float mx = max3(mx0, mx1, fmaxf(sv[30], sv[31]));
+                    if (mx > m_ref + kTau) {                   // also the first step with an open agent (m_ref = kRefFloor)
                         corr = fast_exp2((m_ref - mx) * kLog2e);
                         resc = started;
                         m_ref = mx;
