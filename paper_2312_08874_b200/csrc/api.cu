@@ -140,9 +140,8 @@ WsLayout ws_layout(const agent_attn_handle* h, int n_tokens, int n_agents, int g
     w.a_off = 0;
     w.va_off = av;
     w.part_off = 2 * av;
-    // sized for either launch plan (per-step kernels or the fused kernel)
     size_t part_floats = slabs * pl.parts * partial_floats(pl.rows_pad, pl.dpad);
-    if (grid_h > 0 && auto_like(h)) {
+    if (grid_h > 0 && h->cfg.path == AA_PATH_QUEUE) {
         const size_t fused_floats = slabs * (size_t)fused_parts_per_slab(h->cfg.dtype, grid_h, grid_w, h->cfg.head_dim, n_agents) *
                                     partial_floats(64, h->cfg.head_dim);
         if (part_floats < fused_floats) part_floats = fused_floats;
@@ -154,10 +153,7 @@ WsLayout ws_layout(const agent_attn_handle* h, int n_tokens, int n_agents, int g
             const StreamPlan sp = (h->cfg.path == AA_PATH_AUTO && h->cfg.dtype != AA_F32)
                                       ? plan_stream(h->cfg.dtype, (int)slabs, grid_h, grid_w, h->cfg.head_dim, n_agents, pooled != 0, h->sm_count)
                                       : StreamPlan{};
-            if (!sp.ok) continue;
-            const size_t sf = slabs * (size_t)sp.splits * partial_floats(64, 64);
-            if (part_floats < sf) part_floats = sf;
-            extra = stream_extra_bytes((int)slabs, h->cfg.heads, n_tokens, n_agents);
+            if (sp.ok) extra = stream_extra_bytes((int)slabs, h->cfg.heads, n_tokens, n_agents);
         }
     }
     if (use_terms_forward(h, n_agents)) extra = terms_forward_bytes((int)slabs, n_agents, h->cfg.head_dim);
@@ -501,8 +497,6 @@ static int forward_impl(agent_attn_handle* h, const void* Q, const void* K, cons
             sa.b1c = ws + w.extra_off + 2 * av;
             sa.b2p = ws + w.extra_off + 2 * av + align_up((size_t)h->cfg.heads * N * 64 * 2, 256);
             sa.wt = ws + w.extra_off + 2 * av + 2 * align_up((size_t)h->cfg.heads * N * 64 * 2, 256);
-            sa.partials = reinterpret_cast<float*>(ws + w.part_off);
-            sa.tickets = reinterpret_cast<unsigned*>(ws + w.ticket_off);
             sa.status = h->d_status;
             sa.slabs = slabs; sa.heads = h->cfg.heads; sa.H = grid_h; sa.W = grid_w; sa.n = n_agents; sa.p = p;
             sa.scale1 = h->scale1; sa.scale2 = h->scale2; sa.sm_count = h->sm_count; sa.lin = cl.in; sa.lout = cl.out; sa.plan = sp;

@@ -23,8 +23,6 @@ __global__ void __launch_bounds__(NT, 4) stream_prep_kernel(const StreamArgs p, 
     pdl_launch_dependents();          // the aggregation kernel may set itself up while this one runs
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int N = p.H * p.W, n = p.n;
-    if (blockIdx.x == 0)
-        for (int e = tid; e < p.slabs; e += NT) p.tickets[e] = 0u;
     // the bias blocks come first in the grid: they are few, latency-bound, and would otherwise form the kernel's tail
     if ((int)blockIdx.x >= bias_blocks) {
         const long long wi = (long long)(blockIdx.x - bias_blocks) * (NT / 32) + warp;
