@@ -110,7 +110,7 @@ __device__ __forceinline__ void agg_phase(const AggCta<T>& c, unsigned char* sme
     kp += (kAggStages - 1) * tile_step;
     vp += (kAggStages - 1) * tile_step;
     wait_agents();
-    uint32_t a[1][G::kKS][4];
+    uint32_t a[G::kKS][4];
     const int r0 = c.row0 + rgi * 16 + g;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -120,28 +120,28 @@ __device__ __forceinline__ void agg_phase(const AggCta<T>& c, unsigned char* sme
         for (int ks = 0; ks < G::kKS; ++ks)
 #pragma unroll
             for (int q = 0; q < 2; ++q)
-                a[0][ks][q * 2 + h] = (ok && ks * 16 + q * 8 + 2 * t < c.d) ? *reinterpret_cast<const uint32_t*>(ap + ks * 16 + q * 8) : 0u;
+                a[ks][q * 2 + h] = (ok && ks * 16 + q * 8 + 2 * t < c.d) ? *reinterpret_cast<const uint32_t*>(ap + ks * 16 + q * 8) : 0u;
     }
-    float o[1][G::kNT][4];
+    float o[G::kNT][4];
 #pragma unroll
     for (int j = 0; j < G::kNT; ++j)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) o[0][j][e] = 0.f;
-    SoftRows<1> st;
+        for (int e = 0; e < 4; ++e) o[j][e] = 0.f;
+    SoftRows st;
     st.init();
-    uint4 bias[1][2];
+    uint4 bias[2];
     // rows past n read the last row's bias (their results are not stored); columns past the end are masked, their loads clamped
     const T* brow = c.b1 + (size_t)min(r0, c.n - 1) * c.N;
     const long long brow8 = (long long)(min(r0 + 8, c.n - 1) - min(r0, c.n - 1)) * c.N;
     auto fetch_bias = [&](int tok) {
         if constexpr (BIAS == 1) {
             const int col = min(tok + 8 * t, c.N - 8);
-            bias[0][0] = __ldg(reinterpret_cast<const uint4*>(brow + col));
-            bias[0][1] = __ldg(reinterpret_cast<const uint4*>(brow + brow8 + col));
+            bias[0] = __ldg(reinterpret_cast<const uint4*>(brow + col));
+            bias[1] = __ldg(reinterpret_cast<const uint4*>(brow + brow8 + col));
         } else if constexpr (BIAS == 2) {
             const int col = min(tok + 8 * t, c.N - 1);
-            bias[0][0] = load_bias8_any(brow + col, c.b1_end);
-            bias[0][1] = load_bias8_any(brow + brow8 + col, c.b1_end);
+            bias[0] = load_bias8_any(brow + col, c.b1_end);
+            bias[1] = load_bias8_any(brow + brow8 + col, c.b1_end);
         }
     };
     int tok = c.t0 + kgi * 32;
@@ -161,8 +161,8 @@ __device__ __forceinline__ void agg_phase(const AggCta<T>& c, unsigned char* sme
             for (int sub = 0; sub < S::kTokens / (32 * KG); ++sub) {
                 if (tok < c.t1) {
                     const uint32_t so = sm + rd + sub * KG * 32 * G::kPitch;
-                    float s[1][4][4];
-                    uint32_t p[1][2][4];
+                    float s[4][4];
+                    uint32_t p[2][4];
                     tile_logits<T, DK>(s, a, so + koff);
                     tile_softmax<T, DK, BIAS>(s, bias, c.c1, c.t1 - tok, t, st, o, p);
                     tok += 32 * KG;
@@ -181,11 +181,11 @@ __device__ __forceinline__ void agg_phase(const AggCta<T>& c, unsigned char* sme
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int r = h * 8 + g;
-        const float l = st.total(0, h);
-        if (t == 0) ml[r] = make_float2(st.ref[0][h], l);
+        const float l = st.total(h);
+        if (t == 0) ml[r] = make_float2(st.ref[h], l);
 #pragma unroll
         for (int j = 0; j < G::kNT; ++j)
-            *reinterpret_cast<float2*>(acc + r * S::kAccPitch + j * 8 + 2 * t) = make_float2(o[0][j][2 * h], o[0][j][2 * h + 1]);
+            *reinterpret_cast<float2*>(acc + r * S::kAccPitch + j * 8 + 2 * t) = make_float2(o[j][2 * h], o[j][2 * h + 1]);
     }
 }
 

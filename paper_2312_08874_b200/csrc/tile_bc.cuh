@@ -116,8 +116,8 @@ __device__ __forceinline__ void bc_phase(const BcCta<T>& c, unsigned char* smem,
     if (dwc) bc_fill_filter<T, DK>(c, vtile, tab, halo);
 
     const bool full = c.d == DK;
-    uint32_t a[1][G::kKS][4];
-    uint4 bias[1][2];
+    uint32_t a[G::kKS][4];
+    uint4 bias[2];
     auto fetch_q = [&](int tok) {                      // tokens past the range read its last row (results not stored)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -126,7 +126,7 @@ __device__ __forceinline__ void bc_phase(const BcCta<T>& c, unsigned char* smem,
             for (int ks = 0; ks < G::kKS; ++ks)
 #pragma unroll
                 for (int k = 0; k < 2; ++k)
-                    a[0][ks][k * 2 + h] = (full || ks * 16 + k * 8 + 2 * t < c.d) ? __ldg(reinterpret_cast<const uint32_t*>(q + ks * 16 + k * 8)) : 0u;
+                    a[ks][k * 2 + h] = (full || ks * 16 + k * 8 + 2 * t < c.d) ? __ldg(reinterpret_cast<const uint32_t*>(q + ks * 16 + k * 8)) : 0u;
         }
     };
     int shift = 0;
@@ -148,15 +148,15 @@ __device__ __forceinline__ void bc_phase(const BcCta<T>& c, unsigned char* smem,
             for (int h = 0; h < 2; ++h) {
                 const int r = min(tok + h * 8 + g, c.t1 - 1);
                 if constexpr (BIAS == 1) {
-                    bias[0][h] = __ldg(reinterpret_cast<const uint4*>(c.b2 + (size_t)r * c.n + min(col, c.n - 8)));
+                    bias[h] = __ldg(reinterpret_cast<const uint4*>(c.b2 + (size_t)r * c.n + min(col, c.n - 8)));
                 } else if (staged) {
                     const unsigned short* u = reinterpret_cast<const unsigned short*>(bstage + shift) + (r - tok) * c.n;
                     uint32_t w[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) w[i] = u[min(col + 2 * i, c.n - 1)] | ((uint32_t)u[min(col + 2 * i + 1, c.n - 1)] << 16);
-                    bias[0][h] = make_uint4(w[0], w[1], w[2], w[3]);
+                    bias[h] = make_uint4(w[0], w[1], w[2], w[3]);
                 } else {
-                    bias[0][h] = load_bias8_any(c.b2 + (size_t)r * c.n + min(col, c.n - 1), c.b2_end);
+                    bias[h] = load_bias8_any(c.b2 + (size_t)r * c.n + min(col, c.n - 1), c.b2_end);
                 }
             }
         }
@@ -168,22 +168,22 @@ __device__ __forceinline__ void bc_phase(const BcCta<T>& c, unsigned char* smem,
     for (int base = c.t0; base < c.t1; base += tokens, tok += tokens) {
         if (dwc) bc_load_halo<T, DK>(c, vt, base, tokens);
         cp_async_commit();
-        float o[1][G::kNT][4];
+        float o[G::kNT][4];
         if (tok < c.t1) {
-            SoftRows<1> st;
+            SoftRows st;
             st.init();
 #pragma unroll
             for (int j = 0; j < G::kNT; ++j)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) o[0][j][e] = 0.f;
+                for (int e = 0; e < 4; ++e) o[j][e] = 0.f;
             if (BIAS == 2 && staged) {
                 cp_async_wait<1>();
                 __syncwarp();
                 fetch_bias(tok, 0);
             }
             for (int blk = 0; blk < rows; blk += 32) {
-                float s[1][4][4];
-                uint32_t p[1][2][4];
+                float s[4][4];
+                uint32_t p[2][4];
                 tile_logits<T, DK>(s, a, ka + blk * G::kPitch);
                 tile_softmax<T, DK, BIAS>(s, bias, c.c1, c.n - blk, t, st, o, p);
                 if (blk + 32 < rows) fetch_bias(tok, blk + 32);
@@ -192,9 +192,9 @@ __device__ __forceinline__ void bc_phase(const BcCta<T>& c, unsigned char* smem,
             fetch_q(tok + tokens);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const float inv = 1.f / st.total(0, h);
+                const float inv = 1.f / st.total(h);
 #pragma unroll
-                for (int j = 0; j < G::kNT; ++j) { o[0][j][2 * h] *= inv; o[0][j][2 * h + 1] *= inv; }
+                for (int j = 0; j < G::kNT; ++j) { o[j][2 * h] *= inv; o[j][2 * h + 1] *= inv; }
             }
         }
         stage_bias(tok + tokens);
@@ -218,7 +218,7 @@ __device__ __forceinline__ void bc_phase(const BcCta<T>& c, unsigned char* smem,
                         uint32_t f[4];
                         ldsm4(f, addr + j * 16);
                         const uint2 w = tp[(pr * G::kNT + j) * 32];
-                        mma_acc<T>(o[0][j], f, w.x, w.y);
+                        mma_acc<T>(o[j], f, w.x, w.y);
                     }
                 }
             }
@@ -228,8 +228,8 @@ __device__ __forceinline__ void bc_phase(const BcCta<T>& c, unsigned char* smem,
             const uint32_t os = vt + warp * 16 * G::kPitch;
 #pragma unroll
             for (int j = 0; j < G::kNT; j += 2)
-                stsm4(os + (lane & 15) * G::kPitch + (j + (lane >> 4)) * 16, pack2<T>(o[0][j][0], o[0][j][1]), pack2<T>(o[0][j][2], o[0][j][3]),
-                      pack2<T>(o[0][j + 1][0], o[0][j + 1][1]), pack2<T>(o[0][j + 1][2], o[0][j + 1][3]));
+                stsm4(os + (lane & 15) * G::kPitch + (j + (lane >> 4)) * 16, pack2<T>(o[j][0], o[j][1]), pack2<T>(o[j][2], o[j][3]),
+                      pack2<T>(o[j + 1][0], o[j + 1][1]), pack2<T>(o[j + 1][2], o[j + 1][3]));
             __syncwarp();
             const unsigned char* op = vtile + warp * 16 * G::kPitch;
 #pragma unroll

@@ -7,14 +7,7 @@ namespace aa {
 
 namespace {
 
-struct DkInfo {
-    int dk;
-};
-DkInfo dk_of(int d) {
-    DkInfo i;
-    i.dk = d <= 32 ? 32 : d <= 48 ? 48 : d <= 64 ? 64 : d <= 80 ? 80 : d <= 96 ? 96 : 128;
-    return i;
-}
+int dk_of(int d) { return d <= 32 ? 32 : d <= 48 ? 48 : d <= 64 ? 64 : d <= 80 ? 80 : d <= 96 ? 96 : 128; }
 cudaError_t dispatch(TileKernel k, int dtype, int dk, int bias, const TileArgs& a, const TileLaunch& l) {
     switch (dk) {
         case 32: return tile_dispatch_32(k, dtype, bias, a, l);
@@ -60,17 +53,17 @@ struct SlabPlan {
     long long slots;               // blocks resident at once
 };
 SlabPlan slab_plan(const TileArgs& a, int sm_count) {
-    const DkInfo dk = dk_of(a.d);
+    const int dk = dk_of(a.d);
     SlabPlan s;
     s.warps = a.n <= 64 ? 4 : 8;
     s.rg = (a.n + 15) / 16;
     s.kg = s.warps == 8 || s.rg > 2 ? 1 : s.rg == 2 ? 2 : 4;
-    s.smem = std::max(agg_smem(dk.dk, s.kg, s.warps), bc_smem(dk.dk, a, s.warps));
+    s.smem = std::max(agg_smem(dk, s.kg, s.warps), bc_smem(dk, a, s.warps));
     s.slots = std::min<long long>(16 / s.warps, 227 * 1024 / (s.smem + 1024)) * sm_count;
     return s;
 }
 // Row and key groups of an aggregation block: at most eight warps, all of them with rows.
-int agg_rows(const TileArgs& a, const DkInfo& dk, TileArgs* out) {
+int agg_rows(const TileArgs& a, TileArgs* out) {
     const int rb = (a.n + 8 * 16 - 1) / (8 * 16);
     out->rg = ((a.n + rb - 1) / rb + 16 - 1) / 16;
     out->kg = out->rg <= 2 ? 4 : out->rg <= 4 ? 2 : 1;
@@ -80,9 +73,8 @@ int agg_rows(const TileArgs& a, const DkInfo& dk, TileArgs* out) {
 }  // namespace
 
 cudaError_t launch_tile_aggregate(int dtype, TileArgs a, int sm_count, bool dependent, cudaStream_t st) {
-    const DkInfo dk = dk_of(a.d);
-    const int rb = agg_rows(a, dk, &a);
-    
+    const int dk = dk_of(a.d);
+    const int rb = agg_rows(a, &a);
     a.b2 = nullptr;
     // Parts of the token axis (one block each, a cluster per slab).  Two blocks share an SM and hide each other's
     // latencies, so the best split is the one with the shortest blocks in the fewest waves; a block's start and merge count as
@@ -91,7 +83,7 @@ cudaError_t launch_tile_aggregate(int dtype, TileArgs a, int sm_count, bool depe
     // 85 and 92 us; 16640 tokens 115 and 98, 124 and 125 us; 2800 tokens 37 and 35, 38 and 44 us).
     int best = 1;
     long long best_cost = 0;
-    const int smem = agg_smem(dk.dk, a.kg, 8);
+    const int smem = agg_smem(dk, a.kg, 8);
     for (int c = 1; c <= 16; c *= 2) {
         const int tokens = up32((a.N + c - 1) / c);
         if (c > 1 && (tokens < 64 || c * a.kg > 32)) break;
@@ -108,18 +100,17 @@ cudaError_t launch_tile_aggregate(int dtype, TileArgs a, int sm_count, bool depe
     l.smem = smem;
     l.dependent = dependent;
     l.stream = st;
-    return dispatch(kTileAggregate, dtype, dk.dk, bias_kind(a.b1, bias_align(a.N)), a, l);
+    return dispatch(kTileAggregate, dtype, dk, bias_kind(a.b1, bias_align(a.N)), a, l);
 }
 
 cudaError_t launch_tile_broadcast(int dtype, TileArgs a, int sm_count, bool dependent, cudaStream_t st) {
-    const DkInfo dk = dk_of(a.d);
-    
+    const int dk = dk_of(a.d);
     a.b1 = nullptr;
     // Small agent counts: blocks of eight warps, two to an SM.  Large ones: the agents and their features fill a third of
     // the shared memory or more, so one block of sixteen warps shares them.
-    const bool pair = bc_smem(dk.dk, a, 8) <= 113 * 1024;
+    const bool pair = bc_smem(dk, a, 8) <= 113 * 1024;
     int warps = pair ? 8 : 16;
-    while (bc_smem(dk.dk, a, warps) > 227 * 1024) warps -= 4;      // (256 agents of 128 channels: 8; four always fit)
+    while (bc_smem(dk, a, warps) > 227 * 1024) warps -= 4;      // (256 agents of 128 channels: 8; four always fit)
     const int slots = pair ? 2 * sm_count : sm_count;
     const int pass = warps * 16;                       // tokens of one pass of a block
     int best = 1;
@@ -135,10 +126,10 @@ cudaError_t launch_tile_broadcast(int dtype, TileArgs a, int sm_count, bool depe
     l.grid = dim3((a.N + a.bc_tokens - 1) / a.bc_tokens, a.slabs);
     l.threads = warps * 32;
     l.cluster = 0;
-    l.smem = bc_smem(dk.dk, a, warps);
+    l.smem = bc_smem(dk, a, warps);
     l.dependent = dependent;
     l.stream = st;
-    return dispatch(kTileBroadcast, dtype, dk.dk, bias_kind(a.b2, bias_align(a.n)), a, l);
+    return dispatch(kTileBroadcast, dtype, dk, bias_kind(a.b2, bias_align(a.n)), a, l);
 }
 
 // It saves two launches and the agents' way through memory; a slab's chain runs in at most eight blocks, so the longer the grid, the less it
@@ -149,7 +140,7 @@ cudaError_t launch_tile_broadcast(int dtype, TileArgs a, int sm_count, bool depe
 bool tile_one_kernel(const TileArgs& a, int sm_count) {
     if (a.N > 1024 || a.n > 128) return false;
     const SlabPlan s = slab_plan(a, sm_count);
-    return bc_smem(dk_of(a.d).dk, a, s.warps) <= 113 * 1024 && (a.slabs <= s.slots || a.N <= (a.n > 64 ? 196 : 64));
+    return bc_smem(dk_of(a.d), a, s.warps) <= 113 * 1024 && (a.slabs <= s.slots || a.N <= (a.n > 64 ? 196 : 64));
 }
 
 cudaError_t launch_tile_forward(int dtype, TileArgs a, int sm_count, bool one_kernel, cudaStream_t st, int* launches) {
@@ -169,7 +160,7 @@ cudaError_t launch_tile_forward(int dtype, TileArgs a, int sm_count, bool one_ke
         l.dependent = true;
         l.stream = st;
         *launches += 1;
-        return dispatch(kTileSlab, dtype, dk_of(a.d).dk, !a.b1 && !a.b2 ? 0 : a.b1 && a.b2 && a.N % 8 == 0 && a.n % 8 == 0 ? 1 : 2, a, l);
+        return dispatch(kTileSlab, dtype, dk_of(a.d), !a.b1 && !a.b2 ? 0 : a.b1 && a.b2 && a.N % 8 == 0 && a.n % 8 == 0 ? 1 : 2, a, l);
     }
     if (a.pool) {
         // a warp per window, or (few windows, more than 32 tokens each) a block per window
