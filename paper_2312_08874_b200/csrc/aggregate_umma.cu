@@ -426,7 +426,7 @@ static cudaError_t launch_umma_t(const UmmaAggArgs& g, cudaStream_t st) {
                             (const float*)g.a.partials, g.a.splits, g.rows_pad, g.a.rows, g.a.d, static_cast<T*>(g.a.out));
 }
 
-// cudaErrorNotSupported: a tensor map could not be encoded; the caller falls back to the mma.sync kernel.
+// cudaErrorNotSupported: a tensor map could not be encoded.
 cudaError_t launch_aggregate_umma(int dtype, const AttnArgs& p, const AggPlan& plan, cudaStream_t st) {
     UmmaAggArgs g;
     memset(&g, 0, sizeof(g));

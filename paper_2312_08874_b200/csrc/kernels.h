@@ -20,6 +20,24 @@ inline TokLayout dense_layout(int heads, long long n_tokens, int d) {
     l.sb = (long long)heads * n_tokens * d; l.sh = n_tokens * d; l.st = d;
     return l;
 }
+// Extents and byte strides of the outer dimensions of a tensor map over such a tensor (16-bit elements): head and token in the order of
+// their strides, then batch.  False where they do not nest in that order: no map, the register-tiled kernels read the tensor.
+inline bool tok_map_dims(const TokLayout& l, int batch, int heads, long long n_tokens, bool* head_first, unsigned long long (&n)[2], unsigned long long (&s)[3]) {
+    const bool hf = heads > 1 && l.sh < l.st;
+    *head_first = hf;
+    n[0] = hf ? heads : n_tokens; n[1] = hf ? n_tokens : heads;
+    s[0] = (unsigned long long)(hf ? l.sh : l.st) * 2;
+    s[1] = (unsigned long long)(hf ? l.st : l.sh) * 2;
+    if (heads == 1 && s[1] < s[0] * n[0]) s[1] = s[0] * n[0];          // a single head: its stride is never used
+    s[2] = (unsigned long long)l.sb * 2;
+    if (batch == 1 && s[2] < s[1] * n[1]) s[2] = s[1] * n[1];          // a single batch item: its stride is never used
+    return s[1] >= s[0] && s[2] >= s[1] && s[2] < (1ull << 40);
+}
+inline bool tok_map_exists(const TokLayout& l, int batch, int heads, long long n_tokens) {
+    bool hf;
+    unsigned long long n[2], s[3];
+    return tok_map_dims(l, batch, heads, n_tokens, &hf, n, s);
+}
 __host__ __device__ inline long long tok_offset(const TokLayout& l, int slab, int heads, long long tok) {
     return (long long)(slab / heads) * l.sb + (long long)(slab % heads) * l.sh + tok * l.st;
 }

@@ -125,17 +125,12 @@ inline bool make_map_tok_u16(CUtensorMap* out, int* head_first, const void* base
     if (!fn) return false;
     if ((reinterpret_cast<uintptr_t>(base) & 15u) || box_tokens > 256 || d > 64 || d % 8 != 0) return false;
     if ((l.sb & 7) || (l.sh & 7) || (l.st & 7) || l.st < d) return false;
-    const int hf = (heads > 1 && l.sh < l.st) ? 1 : 0;
-    *head_first = hf;
-    const cuuint64_t n1 = hf ? (cuuint64_t)heads : (cuuint64_t)n_tokens, n2 = hf ? (cuuint64_t)n_tokens : (cuuint64_t)heads;
-    const cuuint64_t s1 = (cuuint64_t)(hf ? l.sh : l.st) * 2;
-    cuuint64_t s2 = (cuuint64_t)(hf ? l.st : l.sh) * 2;
-    if (heads == 1 && s2 < s1 * n1) s2 = s1 * n1;          // a single head: its stride is never used
-    cuuint64_t s3 = (cuuint64_t)l.sb * 2;
-    if (batch == 1 && s3 < s2 * n2) s3 = s2 * n2;          // a single batch item: its stride is never used
-    const cuuint64_t dims[4] = {(cuuint64_t)d, n1, n2, (cuuint64_t)batch};
-    const cuuint64_t strides[3] = {s1, s2, s3};
-    if (strides[1] < strides[0] || strides[2] < strides[1]) return false;
+    bool hf;
+    unsigned long long n[2], st[3];
+    if (!tok_map_dims(l, batch, heads, n_tokens, &hf, n, st)) return false;
+    *head_first = hf ? 1 : 0;
+    const cuuint64_t dims[4] = {(cuuint64_t)d, n[0], n[1], (cuuint64_t)batch};
+    const cuuint64_t strides[3] = {st[0], st[1], st[2]};
     const cuuint32_t box[4] = {64u, hf ? 1u : box_tokens, hf ? box_tokens : 1u, 1u};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     return fn(out, CU_TENSOR_MAP_DATA_TYPE_UINT16, 4, const_cast<void*>(base), dims, strides, box, estr,

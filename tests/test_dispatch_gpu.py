@@ -3,7 +3,7 @@ oracle."""
 import pytest
 
 from paper_2312_08874_b200 import Workload, make_inputs
-from tests.parity_util import assert_close, gpu_forward, make_module, oracle_forward
+from tests.parity_util import assert_close, gpu_forward, make_module, oracle_forward, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -39,3 +39,25 @@ def test_dispatch_lines(case):
     slabs = [(0, 0), (B - 1, heads - 1)]
     for (b, h), ref in zip(slabs, oracle_forward(w, inp, slabs=slabs)):
         assert_close(out[b:b + 1, h:h + 1], ref, "bf16", f"{case} slab {(b, h)}")
+
+
+@pytest.mark.parametrize("case", [(4, 4, 32, 64), (1, 2, 64, 96), (3, 1, 64, 128)], ids=["short", "one_entry", "one_head"])
+def test_token_major_views_that_no_tensor_map_expresses(case):
+    """[N, B, heads, d] storage, or heads outside the batch: strides do not nest as tensor maps want them, so the shapes of the tensor-memory
+    kernels run on register tiles (with one batch entry or one head they nest)."""
+    B, heads, H, W = case
+    w = Workload("dispatch", B, heads, H, W, 64, 16, "bf16", True, True, 1.0, seed=500 + H * W)
+    inp = make_inputs(w, bias_std=0.5, dwc_std=0.2)
+    mod = make_module(w)
+    kw = dict(b1=to_dev(inp["b1"]), b2=to_dev(inp["b2"]), dwc_weight=to_dev(inp["dwc"]))
+    slabs = [(0, 0), (B - 1, heads - 1)]
+    refs = oracle_forward(w, inp, slabs=slabs)
+    for order in ((2, 0, 1, 3), (1, 2, 0, 3)):                 # storage [N, B, heads, d], and [heads, N, B, d]
+        back = [order.index(i) for i in range(4)]
+        views = [to_dev(inp[x]).permute(order).contiguous().permute(back) for x in ("q", "k", "v")]
+        out = mod.forward_strided(*views, H, W, w.agents, **kw)
+        assert mod.query_status() == 0
+        if B > 1 and heads > 1:
+            assert mod.last_launch_count() == 3
+        for (b, h), ref in zip(slabs, refs):
+            assert_close(out[b:b + 1, h:h + 1].contiguous(), ref, "bf16", f"{case} {order} slab {(b, h)}")
