@@ -709,45 +709,43 @@ static HostPipe* host_pipe(agent_attn_handle* h, const HostParts& parts) {
     }
     return h->pipe;
 }
-// Copy streams and events of a lane, made when it first cuts a call (a stream made while others work can take a millisecond).
+// Copy streams and events of a lane, made when it is first used.
 static bool lane_ready(HostLane* l) {
-    if (l->done[kHostParts - 1]) return true;
-    bool ok = cudaStreamCreateWithFlags(&l->in, cudaStreamNonBlocking) == cudaSuccess && cudaStreamCreateWithFlags(&l->out, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaEventCreateWithFlags(&l->start, cudaEventDisableTiming) == cudaSuccess;
+    if (l->user) return true;
+    bool ok = cudaStreamCreateWithFlags(&l->in, cudaStreamNonBlocking) == cudaSuccess && cudaStreamCreateWithFlags(&l->out, cudaStreamNonBlocking) == cudaSuccess;
+    for (cudaEvent_t* e : {&l->start, &l->finish}) ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
     for (int i = 0; i < kHostParts; ++i)
         ok = ok && cudaEventCreateWithFlags(&l->ready[i], cudaEventDisableTiming) == cudaSuccess &&
              cudaEventCreateWithFlags(&l->done[i], cudaEventDisableTiming) == cudaSuccess;
     return ok;
 }
 // A lane for a call on stream `st`: the one that serves the stream already (its earlier calls precede this one on the stream anyway),
-// else one whose last call has ended, else a new one.  Null where all are at work for other streams.  *alone: the last call was on this
-// stream too, no other lane is at work, and this one can cut the call.
-static HostLane* host_lane(HostPipe* p, cudaStream_t st, bool* alone) {
-    *alone = false;
+// else one whose last call has ended, else a new one.  Null, for a call in one piece, where the call before it was on another stream:
+// streams that take turns overlap one another's copies and kernels by themselves, and parts would only cost them (64 slabs of 3136
+// tokens, forty calls: two streams 1.66 ms a call in parts, 1.54 in one piece; one stream 1.73 and 1.94).  (Not whether others are in
+// flight: parts and whole calls round differently, and a result must not depend on the time at which it was asked for.)  Null also where
+// every lane is at work for other streams.
+static HostLane* host_lane(HostPipe* p, cudaStream_t st) {
     unsigned long long id = 0;
     if (cudaStreamGetId(st, &id) != cudaSuccess) { cudaGetLastError(); return nullptr; }
     ++id;                                              // (0 marks a lane without a user)
+    const bool turns = p->last && p->last != id;
+    p->last = id;
+    if (turns) return nullptr;
     // another stream of this thread may be under capture: queries and creations are not part of it
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) { cudaGetLastError(); return nullptr; }
     HostLane *own = nullptr, *ended = nullptr, *unused = nullptr;
-    bool busy = p->last && p->last != id;
-    p->last = id;
     for (HostLane& l : p->lane)
         if (!l.user) unused = &l;
         else if (l.user == id) own = &l;
         else if (cudaEventQuery(l.finish) == cudaSuccess) ended = &l;
-        else busy = true;
-    HostLane* found = own ? own : ended;
-    if (!found && unused && cudaEventCreateWithFlags(&unused->finish, cudaEventDisableTiming) == cudaSuccess) found = unused;
-    if (found) {
-        found->user = id;
-        *alone = !busy && lane_ready(found);
-        if (!busy && !*alone) {                        // (no copy streams to be had)
-            destroy_lane(found);
-            found = nullptr;
-        }
+    HostLane* found = own ? own : ended ? ended : unused;
+    if (found && !lane_ready(found)) {                 // (no copy streams to be had)
+        destroy_lane(found);
+        found = nullptr;
     }
+    if (found) found->user = id;
     cudaGetLastError();                                // (cudaErrorNotReady of the lanes at work)
     cudaThreadExchangeStreamCaptureMode(&mode);
     return found;
@@ -790,11 +788,7 @@ int agent_attn_forward_host(agent_attn_handle* h, const void* Q, const void* K, 
         if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) { cudaGetLastError(); split = false; }
     }
     HostPipe* pipe = split ? host_pipe(h, parts) : nullptr;
-    // Calls in flight on several streams overlap one another's copies and kernels by themselves; parts would only cost them (64 slabs of
-    // 3136 tokens, forty calls: two streams 1.66 ms a call in parts, 1.54 in one piece; one stream 1.77 and 1.95).
-    bool alone = false;
-    HostLane* const own = pipe ? host_lane(pipe, st, &alone) : nullptr;
-    HostLane* const lane = alone ? own : nullptr;
+    HostLane* const lane = pipe ? host_lane(pipe, st) : nullptr;
     if (!lane) { parts.count = 1; parts.size[0] = parts.units; }
     cudaError_t e = cudaSuccess;
 #define AA_STEP(x) do { if (e == cudaSuccess) e = (x); } while (0)
@@ -850,8 +844,6 @@ int agent_attn_forward_host(agent_attn_handle* h, const void* Q, const void* K, 
         if (f == cudaSuccess) f = cudaEventRecord(lane->finish, cout);
         if (f == cudaSuccess) f = cudaStreamWaitEvent(st, lane->finish, 0);
         AA_STEP(f);
-    } else if (own) {
-        AA_STEP(cudaEventRecord(own->finish, st));                 // (other streams' calls see this one in flight)
     }
 #undef AA_STEP
     if (rc != AA_OK) return rc;
