@@ -25,7 +25,12 @@
  *    for AA_ERR_CUDA, the launch failed) and agent_attn_last_error() describes the reason.
  *    No call throws, aborts or traps.
  *  - Results are bit-identical from run to run for the same inputs, handle configuration and
- *    device.
+ *    device (exceptions: agent_attn_backward, and parts of host calls, see there).
+ *  - Infinities and NaNs in the inputs make non-finite what depends on them: an infinite query, key
+ *    or agent its softmax rows, an infinite value its channel of the slab.  With a depthwise filter
+ *    and 16-bit types it also makes NaN the other channels of its group of 8 or 16 at the tokens of
+ *    its 3x3 neighbourhood.  A bias of -inf, or of the type's lowest value, removes a key or an
+ *    agent; a row that has none left is unspecified.
  */
 #ifndef AGENT_ATTN_H_
 #define AGENT_ATTN_H_
@@ -50,13 +55,16 @@ typedef enum {
 } aa_status;
 
 typedef enum {
-    AA_PATH_AUTO = 0,         /* tensor-core kernels for bf16/f16: three streaming kernels for long token grids
-                                 with few agents (n <= 64, d = 64, N >= 1024), one persistent task-queue kernel
-                                 for short ones, tensor-memory kernels for n > 64; fp32 FMA kernels for f32 */
+    AA_PATH_AUTO = 0,         /* bf16/f16: three streaming kernels for long token grids with few agents (n <= 64, d = 64,
+                                 N >= 1024, W <= 64), tensor-memory kernels for many agents (72 <= n <= 256, d <= 64)
+                                 on long axes or large batches, register-tiled kernels for everything else, in one
+                                 kernel on short grids.  f32: operands as three bf16 terms on the tensor cores (fp32
+                                 accuracy) where the agents' terms fit in shared memory, else fp32 FMA kernels */
     AA_PATH_SIMT = 1,         /* fp32 FMA kernels for every dtype (slow; for cross-checks) */
-    AA_PATH_UNFUSED = 2,      /* like AUTO, but always one kernel per step (pool, aggregate, broadcast) */
-    AA_PATH_QUEUE = 3         /* like AUTO, but without the streaming kernels: the task-queue kernel wherever it
-                                 applies (n <= 64, d = 64, W <= 64), whatever the number of tokens */
+    AA_PATH_UNFUSED = 2,      /* always one kernel per step (pool, aggregate, broadcast): register-tiled kernels for
+                                 bf16/f16, fp32 FMA kernels for f32 */
+    AA_PATH_QUEUE = 3         /* like AUTO, but the persistent task-queue kernel wherever it applies (16-bit, n <= 64,
+                                 d = 64, 8 <= W <= 64, windows that tile the grid), and no streaming kernels */
 } aa_path;
 
 typedef struct {
@@ -131,11 +139,11 @@ int agent_attn_forward(agent_attn_handle* h,
  *   out          device; element (b, head, token, c) at base + b * out_strides[0] + head * out_strides[1]
  *                + token * out_strides[2] + c
  *   everything else as in agent_attn_forward (A, biases and the filter are dense).
- * Dense strides {heads*N*d, N*d, d} make this call identical to agent_attn_forward.  Other strides run on the
- * fused and the tensor-memory kernels only: AA_ERR_UNSUPPORTED for fp32, head_dim > 64 (or != 64 with
- * n_agents <= 64), caller-supplied A with n_agents <= 64, n_agents > 64 not a multiple of 8, N not a multiple
- * of 8 with a bias, and handles created with a path other than AA_PATH_AUTO.  Other errors as in
- * agent_attn_forward.  No host synchronisation, no allocation. */
+ * Dense strides {heads*N*d, N*d, d} make this call identical to agent_attn_forward.  Other strides are read in
+ * place by the same kernels, or by the register-tiled ones where no tensor map expresses them.  AA_ERR_UNSUPPORTED
+ * for fp32; with n_agents <= 64: head_dim != 64, caller-supplied A, W outside 8..64 or windows that do not tile
+ * the grid; with n_agents > 64: head_dim > 64, n_agents not a multiple of 8, N < 128 or not a multiple of 8; and
+ * for handles created with AA_PATH_SIMT or AA_PATH_UNFUSED.  Other errors as in agent_attn_forward.  No host synchronisation, no allocation. */
 int agent_attn_forward_strided(agent_attn_handle* h,
                                const void* Q, const void* K, const void* V, const void* A,
                                const long long in_strides[3],
@@ -172,10 +180,12 @@ size_t agent_attn_backward_workspace_bytes(const agent_attn_handle* h, int grid_
  * Arithmetic: handles created with AA_PATH_AUTO run the three attention stages on the tensor cores for 16-bit
  * element types with n_agents <= 64 and head_dim == 64 (A, the probabilities and the logit gradients are
  * rounded to the element type before they enter a product, as in the forward pass; V_A, dV_A and the
- * probabilities that form V_A are carried as two 16-bit terms); every other shape, fp32 inputs, and handles
- * created with AA_PATH_SIMT or AA_PATH_UNFUSED compute in fp32 on CUDA cores throughout.  Sums over tokens
- * and over the batch are accumulated with floating-point atomics, so the low-order bits of the results may
- * differ from run to run (the one exception to the reproducibility rule above).
+ * probabilities that form V_A are carried as two 16-bit terms).  Every other shape and fp32 inputs compute with
+ * fp32 accuracy: on the tensor cores with operands as three bf16 terms (16-bit types, and f32 up to 80 channels,
+ * where the agents' terms fit in shared memory), else, and for handles created with AA_PATH_SIMT or
+ * AA_PATH_UNFUSED, on the CUDA cores.  Sums over tokens and over the batch are accumulated with floating-point
+ * atomics, so the low-order bits of the results may differ from run to run (an exception to the reproducibility
+ * rule above).
  * Errors: AA_ERR_INVALID_ARG (null, misaligned or aliasing buffers, n not a square, dwd without a
  * filter), AA_ERR_UNSUPPORTED (shape limits), AA_ERR_WORKSPACE, AA_ERR_CUDA.  No host synchronisation,
  * no allocation. */
@@ -195,8 +205,8 @@ int agent_attn_pool(agent_attn_handle* h, const void* Q, int grid_h, int grid_w,
  * A device [B][heads][n][d]; K, V device [B][heads][N][d]; b1 device [heads][n][N] or NULL;
  * VA_out device [B][heads][n][d].  The N keys of a slab are split over thread blocks; the
  * workspace (>= agent_attn_workspace_bytes for any grid with grid_h * grid_w = n_tokens)
- * receives their partial (max, sum, acc) states, which the last block to finish merges in a
- * fixed order. */
+ * receives their partial (max, sum, acc) states where they do not meet in shared memory; they are
+ * merged in a fixed order. */
 int agent_attn_aggregate(agent_attn_handle* h, const void* A, const void* K, const void* V,
                          const void* b1, int n_tokens, int n_agents, void* VA_out,
                          void* workspace, size_t workspace_bytes, void* stream);
@@ -234,8 +244,9 @@ size_t agent_attn_staging_bytes(const agent_attn_handle* h, int grid_h, int grid
  * library's, tied to `stream` by events, so that copies and kernels of different parts overlap.
  * Calls on different streams do not wait for one another: the handle keeps up to four such pairs
  * of streams, each for the calls of one `stream`, and a call runs in one piece on its own stream
- * where the call before it was on another one or such a call is still in flight (the calls then
- * overlap one another). */
+ * where the call before it was on another one (streams that take turns overlap one another), or
+ * where all pairs are at work for others.  Parts split the token axis in another way than the
+ * whole does, so that 16-bit results of the two may differ by a rounding. */
 int agent_attn_forward_host(agent_attn_handle* h,
                             const void* Q, const void* K, const void* V, const void* A,
                             int grid_h, int grid_w, int n_agents,
