@@ -21,8 +21,8 @@ NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
     "--use_fast_math", "-Xcompiler", "-fPIC", "-Xptxas", "-v",
 ]
-# --use_fast_math is wanted only in the tensor-core kernels' exponent path, which uses explicit
-# ex2.approx anyway; the fp32 path must keep IEEE division and exp2f, so it is compiled without it.
+# --use_fast_math serves the 16-bit kernels' divisions; the fp32 kernels keep IEEE division, logarithms and denormals, and exp2f
+# where they call it (the term kernels' probabilities are explicit ex2.approx, as accurate on their range), so they go without.
 PRECISE_FILES = {"attn_simt.cu", "pool.cu", "api.cu", "backward.cu", "bwd_terms.cu"} | {f"bwd_terms_d{d}.cu" for d in (32, 48, 64, 80, 96, 128)}
 
 

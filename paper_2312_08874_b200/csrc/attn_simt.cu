@@ -1,7 +1,7 @@
 // fp32 FMA kernels for both Softmax attentions of Eq. 3 (any element type, fp32 arithmetic).
 //
-// This is the path of the fp32 configuration (no tensor-core rounding is acceptable at its
-// 1e-4 tolerance) and a cross-check path for the 16-bit types.  One block owns 64 rows of the
+// This is the path of AA_PATH_SIMT, of fp32 tensors under AA_PATH_UNFUSED, and of fp32 shapes that
+// the term kernels do not take (agents' terms beyond shared memory).  One block owns 64 rows of the
 // attention (agents in the aggregation, tokens in the broadcast) and walks its columns in tiles
 // of 32 with an online softmax; the accumulator lives in registers.
 #include "common.cuh"
