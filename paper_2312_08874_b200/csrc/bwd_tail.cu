@@ -2,9 +2,12 @@
 //   dQ  += Pooling^T(dA)   a window spreads its agent's gradient evenly over its tokens
 //   dV  += DWC^T(dO)       tap (u, v) of output token (y - u + 1, x - v + 1) read V[y][x]
 //   dWd += corr(dO, V)     dWd[c][u][v] = sum over tokens of dO[y - u + 1][x - v + 1][c] V[y][x][c]
-// The first two are one pass with a thread per token and four channels and all its loads in flight at once (dQ and dV are read and
-// written in fp32: that traffic is the bound).  The third is a pass of its own: its 36 sums per thread would halve the threads of
-// the first.  64 slabs of a 56 x 56 grid: one pass for all three 156 us, these two 74 + 31 us.
+// Two kernels of threads that slide down a strip of rows of a grid column.  bwd_conv_tail does dV and dWd, two channels a thread: a row
+// brings three new window entries, the other six come from registers, an entry serves both its tap and its sum, and rows are requested
+// two ahead.  (Four channels a thread need twice the registers for taps and sums: with the taps in shared memory and two blocks of
+// eight warps an SM 60 us.)  bwd_pool_tail is a stream over dQ, four rows in flight.  dQ and dV are read and written in fp32, which is
+// the bound.  64 slabs of a 56 x 56 grid: 47 us (154 MB, 24 us at the copy bandwidth) and 16 us (103 MB, 16 us); one kernel for dQ and
+// dV with all nine window loads of a token, and one for dWd, took 74 and 31.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -16,27 +19,31 @@ struct TailArgs {
     const void *v, *go, *wd;
     const float* da;
     float *dq, *dv, *dwd;
-    int heads, H, W, d, n, p, strip;
+    int heads, H, W, d, n, p, strip, strips, passes;
 };
 
-// Four channels of a token, as loaded; channel pairs in fp32 on use.
-template <typename T> struct Raw4 { uint2 w; };
-template <> struct Raw4<float> { float4 w; };
-template <typename T> __device__ __forceinline__ Raw4<T> ld_raw4(const T* p) {
-    Raw4<T> r;
-    if constexpr (sizeof(T) == 4) r.w = __ldg(reinterpret_cast<const float4*>(p));
-    else r.w = __ldg(reinterpret_cast<const uint2*>(p));
+// Two channels of a token as loaded (zeros where there is no token; volatile: left to itself the compiler gathers the loads of several
+// rows and spills), and in fp32 on use.
+template <typename T> struct Raw2 { uint32_t w; };
+template <> struct Raw2<float> { float2 w; };
+template <typename T> __device__ __forceinline__ Raw2<T> ld_raw2(const T* p, bool ok) {
+    Raw2<T> r;
+    if constexpr (sizeof(T) == 4)
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\tmov.b32 %0, 0f00000000;\n\tmov.b32 %1, 0f00000000;\n\t@p ld.global.nc.v2.f32 {%0,%1}, [%2];\n\t}\n"
+                     : "=&f"(r.w.x), "=&f"(r.w.y) : "l"(p), "r"((int)ok));
+    else
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\tmov.b32 %0, 0;\n\t@p ld.global.nc.u32 %0, [%1];\n\t}\n" : "=&r"(r.w) : "l"(p), "r"((int)ok));
     return r;
 }
-template <typename T> __device__ __forceinline__ Raw4<T> zero_raw4() {
-    Raw4<T> r;
-    if constexpr (sizeof(T) == 4) r.w = make_float4(0.f, 0.f, 0.f, 0.f);
-    else r.w = make_uint2(0u, 0u);
+__device__ __forceinline__ float2 ld_pair(const float* p, bool ok) {
+    float2 r;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\tmov.b32 %0, 0f00000000;\n\tmov.b32 %1, 0f00000000;\n\t@p ld.global.v2.f32 {%0,%1}, [%2];\n\t}\n"
+                 : "=&f"(r.x), "=&f"(r.y) : "l"(p), "r"((int)ok) : "memory");
     return r;
 }
-template <typename T> __device__ __forceinline__ float2 pair(const Raw4<T>& r, int q) {
-    if constexpr (sizeof(T) == 4) return q == 0 ? make_float2(r.w.x, r.w.y) : make_float2(r.w.z, r.w.w);
-    else return unpack2<T>(q == 0 ? r.w.x : r.w.y);
+template <typename T> __device__ __forceinline__ float2 pair(const Raw2<T>& r) {
+    if constexpr (sizeof(T) == 4) return r.w;
+    else return unpack2<T>(r.w);
 }
 
 // Pooling windows over position i of an axis of L positions and p cells: first cell, and the lengths of it and of the next
@@ -56,154 +63,181 @@ __device__ __forceinline__ Windows windows_of(int i, int L, int p) {
     return w;
 }
 
-constexpr int kAxis = 512;         // positions of an axis whose windows are kept in shared memory
+constexpr int kAxis = 512;         // rows whose windows are kept in shared memory
+constexpr int kThreadsQ = 256, kThreadsV = 128;
 
-template <typename T, bool DWC>
-__global__ void __launch_bounds__(256, DWC ? 3 : 4) bwd_tail_kernel(const TailArgs a, int tokens) {
-    __shared__ __align__(16) float wt[DWC ? 9 * 128 : 4];
-    __shared__ Windows yw[kAxis], xw[kAxis];
-    const int d = a.d, H = a.H, W = a.W, p = a.p, N = H * W, slab = blockIdx.y;
-    const int t0 = blockIdx.x * tokens, t1 = min(N, t0 + tokens);
-    const int groups = d >> 2, cols = 256 / groups;               // d <= 128: at least eight tokens at once
+// Columns of a slab's strips, one after the other: a block takes `passes` times `cols` of them.
+struct Column {
+    int x, y0, y1;
+};
+__device__ __forceinline__ Column column_of(const TailArgs& a, int i) {
+    const int s = i / a.W;
+    return {i - s * a.W, s * a.strip, min(a.H, (s + 1) * a.strip)};
+}
+
+__global__ void __launch_bounds__(kThreadsQ, 4) bwd_pool_tail_kernel(const TailArgs a) {
+    __shared__ Windows yw[kAxis];
+    const int d = a.d, H = a.H, W = a.W, p = a.p, slab = blockIdx.y;
+    const int groups = d >> 2, cols = kThreadsQ / groups;         // d <= 128: at least eight columns at once
     const int cg = threadIdx.x % groups, cl = threadIdx.x / groups;
+    for (int i = threadIdx.x; i < min(H, kAxis); i += kThreadsQ) yw[i] = windows_of(i, H, p);
     pdl_wait_prior();
     pdl_release_next();
-    const int ylo = t0 / W, rows = (t1 - 1) / W - ylo + 1;
-    for (int i = threadIdx.x; i < min(rows, kAxis); i += 256) yw[i] = windows_of(ylo + i, H, p);
-    for (int i = threadIdx.x; i < min(W, kAxis); i += 256) xw[i] = windows_of(i, W, p);
-    if (DWC) {
-        const T* w = static_cast<const T*>(a.wd) + (size_t)(slab % a.heads) * d * 9;
-        for (int i = threadIdx.x; i < d * 9; i += 256) wt[(i % 9) * d + i / 9] = Elem<T>::to_f32(w[i]);
-    }
     __syncthreads();
     if (cl >= cols) return;
-    const size_t base = (size_t)slab * N * d + 4 * cg;
-    const T* go = static_cast<const T*>(a.go) + base;
     const float* da = a.da + (size_t)slab * a.n * d + 4 * cg;
-    int tok = t0 + cl, y = tok / W, x = tok - y * W;
-    for (; tok < t1; tok += cols) {
-        float4 q = *reinterpret_cast<const float4*>(a.dq + base + (size_t)tok * d), o = make_float4(0.f, 0.f, 0.f, 0.f);
-        Raw4<T> win[9];
-        if (DWC) {
-            o = *reinterpret_cast<const float4*>(a.dv + base + (size_t)tok * d);
+    const int first = blockIdx.x * a.passes * cols, last = min(first + a.passes * cols, a.strips * W);
+    for (int i = first + cl; i < last; i += cols) {
+        const Column c = column_of(a, i);
+        const Windows wx = windows_of(c.x, W, p);
+        float* dq = a.dq + ((size_t)slab * H * W + (size_t)c.y0 * W + c.x) * d + 4 * cg;
+        float4 pooled = make_float4(0.f, 0.f, 0.f, 0.f);
+        Windows wy = {-1, 0, 0};
+        for (int y = c.y0; y < c.y1; y += 4) {
+            float4 q[4];
 #pragma unroll
-            for (int k = 0; k < 9; ++k) {                         // window position k: token (y + k / 3 - 1, x + k % 3 - 1)
-                const int dy = k / 3 - 1, dx = k % 3 - 1;
-                win[k] = zero_raw4<T>();
-                if ((unsigned)(y + dy) < (unsigned)H && (unsigned)(x + dx) < (unsigned)W) win[k] = ld_raw4<T>(go + (long long)(tok + dy * W + dx) * d);
+            for (int k = 0; k < 4; ++k)
+                if (y + k < c.y1) q[k] = *reinterpret_cast<const float4*>(dq + (size_t)k * W * d);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (y + k >= c.y1) break;
+                const Windows w = y + k < kAxis ? yw[y + k] : windows_of(y + k, H, p);
+                if (w.first != wy.first || w.len0 != wy.len0 || w.len1 != wy.len1) {       // another window row: its agents' gradients
+                    wy = w;
+                    pooled = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j)
+#pragma unroll
+                        for (int l = 0; l < 2; ++l) {
+                            const int area = (j ? wy.len1 : wy.len0) * (l ? wx.len1 : wx.len0);
+                            if (area == 0) continue;
+                            const float4 g = __ldg(reinterpret_cast<const float4*>(da + (size_t)((wy.first + j) * p + wx.first + l) * d));
+                            const float inv = 1.f / (float)area;
+                            pooled.x = fmaf(g.x, inv, pooled.x); pooled.y = fmaf(g.y, inv, pooled.y);
+                            pooled.z = fmaf(g.z, inv, pooled.z); pooled.w = fmaf(g.w, inv, pooled.w);
+                        }
+                }
+                q[k].x += pooled.x; q[k].y += pooled.y; q[k].z += pooled.z; q[k].w += pooled.w;
+                *reinterpret_cast<float4*>(dq + (size_t)k * W * d) = q[k];
             }
+            dq += (size_t)4 * W * d;
         }
-        const Windows wy = y - ylo < kAxis ? yw[y - ylo] : windows_of(y, H, p), wx = x < kAxis ? xw[x] : windows_of(x, W, p);
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const int area = (i ? wy.len1 : wy.len0) * (k ? wx.len1 : wx.len0);
-                if (area == 0) continue;
-                const float4 g = __ldg(reinterpret_cast<const float4*>(da + (size_t)((wy.first + i) * p + wx.first + k) * d));
-                const float inv = 1.f / (float)area;
-                q.x = fmaf(g.x, inv, q.x); q.y = fmaf(g.y, inv, q.y);
-                q.z = fmaf(g.z, inv, q.z); q.w = fmaf(g.w, inv, q.w);
-            }
-        *reinterpret_cast<float4*>(a.dq + base + (size_t)tok * d) = q;
-        if (DWC) {
-            float2 c[2] = {make_float2(o.x, o.y), make_float2(o.z, o.w)};
-#pragma unroll
-            for (int k = 0; k < 9; ++k) {                         // window position k meets tap 8 - k
-                const float4 f = *reinterpret_cast<const float4*>(wt + (8 - k) * d + 4 * cg);
-                c[0] = ffma2(pair<T>(win[k], 0), make_float2(f.x, f.y), c[0]);
-                c[1] = ffma2(pair<T>(win[k], 1), make_float2(f.z, f.w), c[1]);
-            }
-            *reinterpret_cast<float4*>(a.dv + base + (size_t)tok * d) = make_float4(c[0].x, c[0].y, c[1].x, c[1].y);
-        }
-        x += cols;
-        while (x >= W) { x -= W; ++y; }
     }
 }
 
-// A thread owns four channels of a grid column and slides down a strip of rows, three rows at a time: twelve loads in flight, and
-// the window rows above come from registers.
-template <typename T>
-__global__ void __launch_bounds__(256, 2) bwd_filter_kernel(const TailArgs a) {
-    __shared__ float2 red[256][9][2];
+template <typename T, bool DWD>
+__global__ void __launch_bounds__(kThreadsV, sizeof(T) == 4 ? 4 : 5) bwd_conv_tail_kernel(const TailArgs a) {
+    __shared__ float2 red[DWD ? kThreadsV : 1][9];
     const int d = a.d, H = a.H, W = a.W, slab = blockIdx.y;
-    const int y0 = blockIdx.x * a.strip, y1 = min(H, y0 + a.strip);
-    const int groups = d >> 2, cols = 256 / groups;
+    const int groups = d >> 1, cols = kThreadsV / groups;         // d <= 128: at least two columns at once
     const int cg = threadIdx.x % groups, cl = threadIdx.x / groups;
-    const size_t base = (size_t)slab * H * W * d + 4 * cg;
-    const T* v = static_cast<const T*>(a.v) + base;
-    const T* go = static_cast<const T*>(a.go) + base;
-    float2 acc[9][2];
+    float2 tap[9], acc[DWD ? 9 : 1];
+    {
+        const T* w = static_cast<const T*>(a.wd) + ((size_t)(slab % a.heads) * d + 2 * cg) * 9;
 #pragma unroll
-    for (int k = 0; k < 9; ++k) acc[k][0] = acc[k][1] = make_float2(0.f, 0.f);
-    if (cl < cols)
-        for (int x = cl; x < W; x += cols) {
-            Raw4<T> win[5][3], t[3];                              // dO rows y - 1 .. y + 3 around V rows y .. y + 2
-            auto row = [&](Raw4<T> (&r)[3], int y) {
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    r[c] = zero_raw4<T>();
-                    if ((unsigned)y < (unsigned)H && (unsigned)(x + c - 1) < (unsigned)W) r[c] = ld_raw4<T>(go + (long long)(y * W + x + c - 1) * d);
-                }
-            };
-            row(win[0], y0 - 1);
-            row(win[1], y0);
-            for (int y = y0; y < y1; y += 3) {
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    row(win[2 + i], y + 1 + i);
-                    t[i] = zero_raw4<T>();
-                    if (y + i < y1) t[i] = ld_raw4<T>(v + (long long)((y + i) * W + x) * d);
-                }
-#pragma unroll
-                for (int i = 0; i < 3; ++i)
-#pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        const float2 s = pair<T>(t[i], q);
-#pragma unroll
-                        for (int u = 0; u < 3; ++u)
-#pragma unroll
-                            for (int w = 0; w < 3; ++w) acc[3 * u + w][q] = ffma2(pair<T>(win[i + 2 - u][2 - w], q), s, acc[3 * u + w][q]);
-                    }
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    win[0][c] = win[3][c];
-                    win[1][c] = win[4][c];
-                }
-            }
-        }
-#pragma unroll
-    for (int k = 0; k < 9; ++k)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) red[threadIdx.x][k][q] = acc[k][q];
-    __syncthreads();
-    pdl_wait_prior();                                             // (before that: inputs only)
-    for (int o = threadIdx.x; o < d * 9; o += 256) {              // o = channel * 9 + tap
-        const int c = o / 9, k = o - c * 9;
-        float s = 0.f;
-        for (int l = 0; l < cols; ++l) {
-            const float2 t = red[l * groups + (c >> 2)][k][(c >> 1) & 1];
-            s += (c & 1) ? t.y : t.x;
-        }
-        atomicAdd(a.dwd + (size_t)(slab % a.heads) * d * 9 + o, s);
+        for (int k = 0; k < 9; ++k) tap[k] = make_float2(Elem<T>::to_f32(w[k]), Elem<T>::to_f32(w[9 + k]));
     }
+    pdl_wait_prior();                                             // (before that: inputs only)
+    pdl_release_next();
+    if (DWD)
+#pragma unroll
+        for (int k = 0; k < 9; ++k) acc[k] = make_float2(0.f, 0.f);
+    const int first = blockIdx.x * a.passes * cols, last = min(first + a.passes * cols, a.strips * W);
+    const size_t pitch = (size_t)W * d;
+    if (cl < cols)
+        for (int i = first + cl; i < last; i += cols) {
+            const Column c = column_of(a, i);
+            const bool left = c.x > 0, right = c.x + 1 < W;
+            const size_t base = ((size_t)slab * H * W + (size_t)c.y0 * W + c.x) * d + 2 * cg;
+            const T *v = static_cast<const T*>(a.v) + base, *go = static_cast<const T*>(a.go) + base;
+            float* dv = a.dv + base;
+            // rings of three rows: dO in fp32 (y - 1 .. y + 1), the dO rows on their way (y + 2, y + 3), dV and V (y .. y + 2)
+            float2 win[3][3], o[3];
+            Raw2<T> raw[3][3], rv[3];
+            auto row = [&](Raw2<T> (&r)[3], const T* g, int y) {
+                const bool in = (unsigned)y < (unsigned)H;
+                r[0] = ld_raw2<T>(g - d, in && left);
+                r[1] = ld_raw2<T>(g, in);
+                r[2] = ld_raw2<T>(g + d, in && right);
+            };
+            auto convert = [&](float2 (&f)[3], const Raw2<T> (&r)[3]) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) f[k] = pair<T>(r[k]);
+            };
+            row(raw[2], go - pitch, c.y0 - 1);
+            row(raw[0], go, c.y0);
+            o[0] = ld_pair(dv, true);
+            if (DWD) rv[0] = ld_raw2<T>(v, true);
+            o[1] = ld_pair(dv + pitch, c.y0 + 1 < c.y1);
+            if (DWD) rv[1] = ld_raw2<T>(v + pitch, c.y0 + 1 < c.y1);
+            row(raw[1], go + pitch, c.y0 + 1);
+            convert(win[2], raw[2]);
+            convert(win[0], raw[0]);
+            go += 2 * pitch;
+            row(raw[2], go, c.y0 + 2);
+            for (int y = c.y0; y < c.y1; y += 3)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {                     // row y + k (rows past the strip: zeros, not stored)
+                    const int y2 = y + k + 2;
+                    go += pitch;
+                    row(raw[k], go, y2 + 1);
+                    o[(k + 2) % 3] = ld_pair(dv + 2 * pitch, y2 < c.y1);
+                    if (DWD) rv[(k + 2) % 3] = ld_raw2<T>(v + 2 * pitch, y2 < c.y1);
+                    convert(win[(k + 1) % 3], raw[(k + 1) % 3]);
+                    float2 s = o[k];
+                    const float2 t = DWD ? pair<T>(rv[k]) : make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int j = 0; j < 9; ++j) {                 // window position j = token (y + j / 3 - 1, x + j % 3 - 1) meets tap 8 - j
+                        const float2 g = win[(k + j / 3 + 2) % 3][j % 3];
+                        s = ffma2(g, tap[8 - j], s);
+                        if (DWD) acc[8 - j] = ffma2(g, t, acc[8 - j]);
+                    }
+                    if (y + k < c.y1) *reinterpret_cast<float2*>(dv) = s;
+                    dv += pitch;
+                    v += pitch;
+                }
+        }
+    if (DWD) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) red[threadIdx.x][k] = acc[k];
+        __syncthreads();
+        for (int o = threadIdx.x; o < d * 9; o += kThreadsV) {    // o = channel * 9 + tap
+            const int c = o / 9, k = o - c * 9;
+            float s = 0.f;
+            for (int l = 0; l < cols; ++l) {
+                const float2 t = red[l * groups + (c >> 1)][k];
+                s += (c & 1) ? t.y : t.x;
+            }
+            atomicAdd(a.dwd + (size_t)(slab % a.heads) * d * 9 + o, s);
+        }
+    }
+}
+
+// Strips of rows, and passes of a block over `cols` columns: the least rows that a slot (a resident block) goes through, when a strip
+// costs `halo` rows more than it has and the start of a block `start` rows.
+dim3 plan_strips(TailArgs* a, int slabs, int cols, int slots, int halo, int start) {
+    long long best = 0;
+    int blocks = 1;
+    for (int strips = 1; strips <= 32 && (strips == 1 || strips * 4 <= a->H); ++strips) {
+        const int rows = (a->H + strips - 1) / strips, used = (a->H + rows - 1) / rows, total = (int)(((long long)used * a->W + cols - 1) / cols);
+        for (int passes = 1; passes <= 8 && passes <= total; ++passes) {
+            const int per_slab = (total + passes - 1) / passes;
+            const long long cost = ((long long)slabs * per_slab + slots - 1) / slots * (passes * (rows + halo) + start);
+            if (best == 0 || cost < best) { best = cost; blocks = per_slab; a->strip = rows; a->strips = used; a->passes = passes; }
+        }
+    }
+    return dim3(blocks, slabs);
 }
 
 template <typename T> cudaError_t launch_tail(TailArgs a, int slabs, int sm_count, cudaStream_t st) {
-    const int N = a.H * a.W, cols = 256 / (a.d / 4);
-    // runs of tokens: three blocks per SM are resident; at least eight passes of a block, for its tables and taps
-    const long long want = 3LL * sm_count;
-    long long tokens = ((long long)N * slabs + want - 1) / want;
-    tokens = tokens < 8 * cols ? 8 * cols : tokens;
-    const int parts = (int)((N + tokens - 1) / tokens);
-    tokens = (N + parts - 1) / parts;
-    const dim3 grid(parts, slabs);
-    cudaError_t e = launch_dependent(a.wd ? bwd_tail_kernel<T, true> : bwd_tail_kernel<T, false>, grid, 256, 0, st, a, (int)tokens);
-    if (e != cudaSuccess || !a.dwd) return e;
-    // strips: two blocks per SM are resident, at least six rows each (a strip reads two more)
-    const int strip = (int)(((long long)a.H * slabs + 2LL * sm_count - 1) / (2LL * sm_count));
-    a.strip = ((strip < 6 ? 6 : strip) + 2) / 3 * 3;
-    return launch_dependent(bwd_filter_kernel<T>, dim3((a.H + a.strip - 1) / a.strip, slabs), 256, 0, st, a);
+    // dV first: the stage before has just written it
+    if (a.wd) {
+        const dim3 grid = plan_strips(&a, slabs, kThreadsV / (a.d / 2), (sizeof(T) == 4 ? 4 : 5) * sm_count, 2, 4);
+        const cudaError_t e = launch_dependent(a.dwd ? bwd_conv_tail_kernel<T, true> : bwd_conv_tail_kernel<T, false>, grid, kThreadsV, 0, st, a);
+        if (e != cudaSuccess) return e;
+    }
+    const dim3 grid = plan_strips(&a, slabs, kThreadsQ / (a.d / 4), 4 * sm_count, 0, 4);
+    return launch_dependent(bwd_pool_tail_kernel, grid, kThreadsQ, 0, st, a);
 }
 
 }  // namespace
@@ -211,7 +245,7 @@ template <typename T> cudaError_t launch_tail(TailArgs a, int slabs, int sm_coun
 cudaError_t launch_backward_tail(int dtype, const BwdCall& c, cudaStream_t st) {
     TailArgs a;
     a.v = c.v; a.go = c.d_out; a.wd = c.wd; a.da = c.ws_da; a.dq = c.dq; a.dv = c.dv; a.dwd = c.dwd;
-    a.heads = c.heads; a.H = c.H; a.W = c.W; a.d = c.d; a.n = c.n; a.p = c.p; a.strip = 0;
+    a.heads = c.heads; a.H = c.H; a.W = c.W; a.d = c.d; a.n = c.n; a.p = c.p; a.strip = a.strips = a.passes = 0;
     switch (dtype) {
         case kF32:  return launch_tail<float>(a, c.slabs, c.sm_count, st);
         case kBF16: return launch_tail<__nv_bfloat16>(a, c.slabs, c.sm_count, st);

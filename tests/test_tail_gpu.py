@@ -24,3 +24,23 @@ def test_tail_edges_match_oracle(case):
     w = Workload("tail", B, heads, H, W, d, pool, dtype, True, True, 1.0, seed=600 + H * W + d)
     _, got, ref = run_both(w, make_inputs(w, bias_std=0.5, dwc_std=0.2), path=AA_PATH_AUTO)
     check(got, ref, str(case), tc=d == 64)
+
+
+# strips of rows and runs of columns: fewer rows than a strip starts ahead, more rows than the window table holds, strips and columns
+# that do not divide, several passes of a block, the smallest and largest head sizes, fp32
+STRIPS = [
+    (1, 1, 1, 70, 64, 1, "bf16"),
+    (2, 1, 2, 5, 8, 2, "f32"),
+    (1, 1, 600, 4, 16, 4, "f16"),
+    (1, 2, 37, 33, 48, 7, "f32"),
+    (40, 2, 29, 31, 64, 4, "bf16"),
+    (1, 1, 25, 27, 128, 5, "bf16"),
+]
+
+
+@pytest.mark.parametrize("case", STRIPS, ids=[f"B{c[0]}h{c[1]}_{c[2]}x{c[3]}_d{c[4]}_p{c[5]}_{c[6]}" for c in STRIPS])
+def test_strips_match_oracle(case):
+    B, heads, H, W, d, pool, dtype = case
+    w = Workload("tail", B, heads, H, W, d, pool, dtype, True, True, 1.0, seed=700 + H * W + d)
+    _, got, ref = run_both(w, make_inputs(w, bias_std=0.5, dwc_std=0.2), path=AA_PATH_AUTO)
+    check(got, ref, str(case), tc=d == 64 and dtype != "f32")
