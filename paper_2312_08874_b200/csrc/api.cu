@@ -870,14 +870,16 @@ int agent_attn_query_status(agent_attn_handle* h, void* stream) {
 
 // Workspace of the backward pass: [A | V_A | dV_A | dA | lse | dot | partial (max, sum) | terms], fp32, each
 // region 256-byte aligned (V_A, dV_A and dA are cleared as one, so their regions have one size).  The mixed-precision kernels
-// keep A in 16 bits in its region, the terms of V_A in that of the partials and (log-sum-exp, -) pairs over lse and dot.
+// keep A in 16 bits in its region, the terms of V_A in that of the partials, (log-sum-exp, D) pairs over lse and dot, and the terms of
+// dV_A and the padded biases in that of the terms.
 namespace {
 struct BwdLayout {
     size_t a, va, dva, da, lse, dot, part, terms, total;
 };
+bool use_mixed(const agent_attn_handle* h, int n) { return auto_like(h) && backward_umma_eligible(h->cfg.dtype, n, h->cfg.head_dim); }
 // inputs outside the mixed-precision kernels: fp32 operands as 16-bit terms on the tensor cores
 bool use_terms(const agent_attn_handle* h, int n) {
-    return auto_like(h) && !backward_mma_eligible(h->cfg.dtype, n, h->cfg.head_dim) && backward_terms_eligible(h->cfg.dtype, n, h->cfg.head_dim);
+    return auto_like(h) && !backward_umma_eligible(h->cfg.dtype, n, h->cfg.head_dim) && backward_terms_eligible(h->cfg.dtype, n, h->cfg.head_dim);
 }
 bool bwd_layout(const agent_attn_handle* h, int N, int n, BwdPlan* pl, BwdLayout* w) {
     const int slabs = h->cfg.batch * h->cfg.heads;
@@ -890,7 +892,7 @@ bool bwd_layout(const agent_attn_handle* h, int N, int n, BwdPlan* pl, BwdLayout
     size_t part_floats = (size_t)slabs * pl->chunks * n * 2;
     if (part_floats * sizeof(float) < snd) part_floats = snd / sizeof(float);       // (mixed precision: two 16-bit terms of V_A)
     w->terms = w->part + align_up(part_floats * sizeof(float), 256);
-    w->total = w->terms + (use_terms(h, n) ? backward_terms_bytes(slabs, n, N, h->cfg.head_dim) : 0);
+    w->total = w->terms + (use_mixed(h, n) ? backward_umma_bytes(slabs, h->cfg.heads, n, N) : use_terms(h, n) ? backward_terms_bytes(slabs, n, N, h->cfg.head_dim) : 0);
     return true;
 }
 }  // namespace
@@ -958,8 +960,8 @@ int agent_attn_backward(agent_attn_handle* h, const void* Q, const void* K, cons
     c.d = h->cfg.head_dim; c.n = n_agents; c.p = p; c.sm_count = h->sm_count;
     c.scale1 = h->scale1; c.scale2 = h->scale2;
     c.dtype = h->cfg.dtype;
-    c.use_mma = auto_like(h) && backward_mma_eligible(h->cfg.dtype, n_agents, h->cfg.head_dim);
-    if (c.use_mma) c.plan_mma = plan_backward_mma(c.slabs, N, h->sm_count);
+    c.status = h->d_status;
+    c.ws_mixed = use_mixed(h, n_agents) ? ws + w.terms : nullptr;
     c.ws_terms = use_terms(h, n_agents) ? ws + w.terms : nullptr;
     cudaError_t e = launch_backward(h->cfg.dtype, c, (cudaStream_t)stream);
     if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "backward launch failed: %s", cudaGetErrorString(e));

@@ -393,18 +393,11 @@ cudaError_t backward_typed(const BwdCall& c, BwdArgs a, cudaStream_t st) {
         AA_TRY(launch_backward_terms(c.dtype, c, c.ws_terms, st));
         return launch_backward_tail(c.dtype, c, st);
     }
-    if (c.use_mma) {
+    if (c.ws_mixed) {
         AA_TRY(launch_backward_mixed_forward(c.dtype, c, st));
-        BwdArgs m = a;
-        m.np = c.plan_mma.np; m.tile = c.plan_mma.tile; m.tiles = c.plan_mma.tiles;
-        m.chunks = c.plan_mma.chunks; m.tiles_per_chunk = c.plan_mma.tiles_per_chunk;
-        m.a_t = c.ws_a; m.va_t = c.ws_part; m.stats = reinterpret_cast<const float2*>(c.ws_lse);
-        m.x = c.q; m.y = c.d_out; m.bias = c.b2; m.scale = c.scale2;
-        m.outer0 = c.ws_dva; m.outer1 = c.ws_da; m.row0 = c.dq; m.dbias = c.db2;
-        AA_TRY(launch_backward_mma(c.dtype, true, m, st));
-        m.x = c.k; m.y = c.v; m.bias = c.b1; m.m0 = c.ws_va; m.m1 = c.ws_dva; m.scale = c.scale1;
-        m.row0 = c.dk; m.row1 = c.dv; m.dbias = c.db1;
-        AA_TRY(launch_backward_mma(c.dtype, false, m, st));
+        AA_TRY(launch_backward_umma(c.dtype, true, c, st));
+        AA_TRY(launch_backward_mixed_dot(c.dtype, c, st));
+        AA_TRY(launch_backward_umma(c.dtype, false, c, st));
         return launch_backward_tail(c.dtype, c, st);
     }
     AA_TRY(cudaMemsetAsync(c.ws_va, 0, 3 * c.region_bytes, st));          // V_A, dV_A, dA are contiguous
@@ -467,7 +460,7 @@ bool plan_backward(int slabs, int n, int N, int d, int sm_count, BwdPlan* out) {
     return true;
 }
 
-int backward_launch_count(const BwdCall& c) { return (c.ws_terms ? 8 : c.use_mma ? 4 : 7) + 1 + (c.wd ? 1 : 0); }
+int backward_launch_count(const BwdCall& c) { return (c.ws_terms ? 8 : c.ws_mixed ? 5 : 7) + 1 + (c.wd ? 1 : 0); }
 
 cudaError_t launch_backward(int dtype, const BwdCall& c, cudaStream_t st) {
     BwdArgs a;

@@ -30,6 +30,27 @@ struct ClearList {
     int pool_blocks;
 };
 constexpr int kClearWords = 256 * 32;              // words that a block clears
+// Biases as rows of 64 agents per token [heads][N][64] (zeros past n), by further blocks of the first kernel: B1 transposed, B2.
+struct PadList {
+    const void *b1, *b2;
+    void *p1, *p2;
+    int heads, n, N, blocks1, blocks2;
+};
+template <typename T> __device__ __forceinline__ void pad_bias(const T* src, uint4* dst, bool transposed, const PadList& pl, int block) {
+    const long long rows = (long long)pl.heads * pl.N, i = (long long)block * 256 + threadIdx.x;
+    // neighbouring threads: B1 is read along its tokens, B2 along its agents
+    const long long row = transposed ? i % rows : i >> 3;
+    const int c0 = 8 * (int)(transposed ? i / rows : i & 7);
+    if (c0 >= 64 || row >= rows) return;
+    const int head = (int)(row / pl.N), tok = (int)(row - (long long)head * pl.N);
+    __align__(16) T v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int c = c0 + k;
+        v[k] = c >= pl.n ? Elem<T>::from_f32(0.f) : transposed ? src[((size_t)head * pl.n + c) * pl.N + tok] : src[(size_t)row * pl.n + c];
+    }
+    dst[row * 8 + (c0 >> 3)] = *reinterpret_cast<const uint4*>(v);
+}
 
 struct PoolArgs8 {
     const void *q, *given;             // tokens, or the caller's agents
@@ -39,7 +60,7 @@ struct PoolArgs8 {
 };
 // Pooled agents as NT terms of E: a warp per window, or (windows of at most 32 tokens on average) a thread per 8 channels.
 template <typename T, typename E, int NT>
-__global__ void __launch_bounds__(256) bwd_pool_terms_kernel(PoolArgs8 pa, E* dst, ClearList cl) {
+__global__ void __launch_bounds__(256) bwd_pool_terms_kernel(PoolArgs8 pa, E* dst, ClearList cl, PadList pl) {
     const T *q = static_cast<const T*>(pa.q), *given = static_cast<const T*>(pa.given);
     const int slabs = pa.slabs, n = pa.n, H = pa.H, W = pa.W, pool = pa.pool, d = pa.d;
     pdl_wait_prior();
@@ -56,6 +77,11 @@ __global__ void __launch_bounds__(256) bwd_pool_terms_kernel(PoolArgs8 pa, E* ds
                 return;
             }
             b -= room;
+        }
+        if constexpr (NT == 1) {
+            const int block = (int)(b / kClearWords);
+            if (block < pl.blocks1) pad_bias<T>(static_cast<const T*>(pl.b1), static_cast<uint4*>(pl.p1), true, pl, block);
+            else pad_bias<T>(static_cast<const T*>(pl.b2), static_cast<uint4*>(pl.p2), false, pl, block - pl.blocks1);
         }
         return;
     }
@@ -144,15 +170,15 @@ int token_parts(long long others, int N, int unit, int pass, int most, bool pow2
 }
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 
-template <typename T, typename E, int NT> cudaError_t launch_pool_terms(PoolArgs8 pa, void* a_t, ClearList cl, cudaStream_t st) {
+template <typename T, typename E, int NT> cudaError_t launch_pool_terms(PoolArgs8 pa, void* a_t, ClearList cl, PadList pl, cudaStream_t st) {
     pa.small = pa.given || pa.H * pa.W <= 32 * pa.n;
     cl.pool_blocks = (int)(pa.small ? ((long long)pa.slabs * pa.n * (pa.d / 8) + 255) / 256 : ((long long)pa.slabs * pa.n + 7) / 8);
     size_t clear = 0;
     for (size_t w : cl.words) clear += (w + kClearWords - 1) / kClearWords;
-    return launch_dependent(bwd_pool_terms_kernel<T, E, NT>, dim3((unsigned)(cl.pool_blocks + clear)), 256, 0, st, pa, static_cast<E*>(a_t), cl);
+    return launch_dependent(bwd_pool_terms_kernel<T, E, NT>, dim3((unsigned)(cl.pool_blocks + clear + pl.blocks1 + pl.blocks2)), 256, 0, st, pa, static_cast<E*>(a_t), cl, pl);
 }
 // Pooling, and the clearing of the sums that the stages add to.
-template <typename T, typename E, int NT> cudaError_t pool_and_clear(const BwdCall& c, void* a_t, bool clear_bias, cudaStream_t st) {
+template <typename T, typename E, int NT> cudaError_t pool_and_clear(const BwdCall& c, void* a_t, bool clear_bias, const PadList& pl, cudaStream_t st) {
     const PoolArgs8 pa = {c.q, nullptr, nullptr, c.slabs, c.n, c.H, c.W, c.p, c.d, false};
     ClearList cl = {};
     const size_t bias = clear_bias ? (size_t)c.heads * c.n * c.H * c.W : 0;
@@ -160,7 +186,7 @@ template <typename T, typename E, int NT> cudaError_t pool_and_clear(const BwdCa
     cl.p[1] = c.db1; cl.words[1] = c.db1 ? bias : 0;
     cl.p[2] = c.db2; cl.words[2] = c.db2 ? bias : 0;
     cl.p[3] = c.dwd; cl.words[3] = c.dwd ? (size_t)c.heads * c.d * 9 : 0;
-    return launch_pool_terms<T, E, NT>(pa, a_t, cl, st);
+    return launch_pool_terms<T, E, NT>(pa, a_t, cl, pl, st);
 }
 
 }  // namespace
@@ -175,7 +201,11 @@ size_t backward_terms_bytes(int slabs, int n, int N, int d) {
 }
 
 cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStream_t st) {
-    cudaError_t e = dtype == kBF16 ? pool_and_clear<__nv_bfloat16, __nv_bfloat16, 1>(c, c.ws_a, true, st) : pool_and_clear<__half, __half, 1>(c, c.ws_a, true, st);
+    const size_t rows = (size_t)c.heads * c.H * c.W;
+    char* padded = static_cast<char*>(c.ws_mixed) + up256((size_t)2 * c.slabs * c.n * 64 * 2);          // (see backward_umma_bytes)
+    const int blocks = (int)((rows * 8 + 255) / 256);
+    const PadList pl = {c.b1, c.b2, padded, padded + rows * 128, c.heads, c.n, c.H * c.W, c.b1 ? blocks : 0, c.b2 ? blocks : 0};
+    cudaError_t e = dtype == kBF16 ? pool_and_clear<__nv_bfloat16, __nv_bfloat16, 1>(c, c.ws_a, true, pl, st) : pool_and_clear<__half, __half, 1>(c, c.ws_a, true, pl, st);
     if (e != cudaSuccess) return e;
     BwdTermArgs a;
     memset(&a, 0, sizeof(a));
@@ -193,6 +223,15 @@ cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStrea
     return bwd_terms_mixed(dtype, a, l);
 }
 
+// D = dV_A . V_A and the two terms of dV_A, between the two gradient stages
+cudaError_t launch_backward_mixed_dot(int dtype, const BwdCall& c, cudaStream_t st) {
+    const int rows = c.slabs * c.n;
+    const float *va = c.ws_va, *dva = c.ws_dva;
+    float2* stats = reinterpret_cast<float2*>(c.ws_lse);
+    if (dtype == kBF16) return launch_dependent(bwd_dot_split_kernel<__nv_bfloat16, 2>, dim3((rows + 7) / 8), 256, 0, st, va, dva, stats, static_cast<__nv_bfloat16*>(c.ws_mixed), rows, c.d);
+    return launch_dependent(bwd_dot_split_kernel<__half, 2>, dim3((rows + 7) / 8), 256, 0, st, va, dva, stats, static_cast<__half*>(c.ws_mixed), rows, c.d);
+}
+
 cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStream_t st) {
     const int N = c.H * c.W, n = c.n, d = c.d, slabs = c.slabs;
     char* w = static_cast<char*>(ws);
@@ -204,7 +243,7 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
     cudaError_t e;
 #define AA_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
     const bool clear_bias = slabs != c.heads;          // (a single batch entry stores its bias gradients)
-    AA_TRY(dtype == kBF16 ? (pool_and_clear<B, B, 3>(c, a_t, clear_bias, st)) : dtype == kF16 ? (pool_and_clear<__half, B, 3>(c, a_t, clear_bias, st)) : (pool_and_clear<float, B, 3>(c, a_t, clear_bias, st)));
+    AA_TRY(dtype == kBF16 ? (pool_and_clear<B, B, 3>(c, a_t, clear_bias, PadList{}, st)) : dtype == kF16 ? (pool_and_clear<__half, B, 3>(c, a_t, clear_bias, PadList{}, st)) : (pool_and_clear<float, B, 3>(c, a_t, clear_bias, PadList{}, st)));
 
     BwdTermArgs a;
     memset(&a, 0, sizeof(a));
@@ -261,7 +300,7 @@ cudaError_t launch_terms_forward(const TermsForward& c, cudaStream_t st) {
     char* w = static_cast<char*>(c.ws);
     const size_t terms = up256((size_t)c.slabs * c.n * c.d * 2 * 3);
     const PoolArgs8 pa = {c.q, c.agents, c.agents ? nullptr : c.a_ws, c.slabs, c.n, c.H, c.W, c.p, c.d, false};
-    cudaError_t e = launch_pool_terms<float, __nv_bfloat16, 3>(pa, w, ClearList{}, st);
+    cudaError_t e = launch_pool_terms<float, __nv_bfloat16, 3>(pa, w, ClearList{}, PadList{}, st);
     if (e != cudaSuccess) return e;
     BwdTermArgs a;
     memset(&a, 0, sizeof(a));

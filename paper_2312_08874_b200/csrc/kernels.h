@@ -227,9 +227,7 @@ struct BwdPlan {
 struct BwdArgs {
     const void *x, *y;        // token rows [slabs][N][d]: operand of the logits, second operand
     const void* bias;         // B1 [heads][n][N] or B2 [heads][N][n], or null
-    const float *m0, *m1;     // fp32 [slabs][n][d]: A; V_A or dV_A  (mixed precision: V_A, dV_A)
-    const void *a_t, *va_t;   // mixed precision: 16-bit A [slabs][n][d]; two terms of V_A [2][slabs][n][d]
-    const float2* stats;      // mixed precision: .x = log2-sum-exp of the aggregation rows [slabs][n]
+    const float *m0, *m1;     // fp32 [slabs][n][d]: A; V_A or dV_A
     const float *lse, *dot;   // fp32 [slabs][n]: log-sum-exp of the aggregation rows; dV_A . V_A
     float* part;              // fp32 [slabs][chunks][n][2]: per-block (max, sum) of the aggregation logits
     float *outer0, *outer1;   // fp32 [slabs][n][d]: sums over tokens (atomics)
@@ -251,8 +249,8 @@ struct BwdCall {
     float scale1, scale2;
     BwdPlan plan;
     int dtype;                                // element type of the inputs (kF32, kBF16, kF16)
-    int use_mma;                              // the two gradient stages run on the tensor-core kernels
-    BwdPlan plan_mma;                         // their tiling
+    int* status;                              // status word of the kernels with bounded waits
+    void* ws_mixed;                           // mixed precision on the tensor cores (bwd_umma.cu) runs the attention stages; null: it does not
     void* ws_terms;                           // term-split kernels (bwd_terms.cu) run the attention stages; null: they do not
 };
 // fp32 forward pass with operands split into 16-bit terms
@@ -272,14 +270,15 @@ size_t backward_terms_bytes(int slabs, int n, int N, int d);
 cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStream_t st);
 // mixed precision, 16-bit inputs: A (16 bits, in ws_a), V_A (fp32 in ws_va, terms in ws_part), statistics (in ws_lse); clears the sums
 cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStream_t st);
+cudaError_t launch_backward_mixed_dot(int dtype, const BwdCall& c, cudaStream_t st);
 // token-wise tail: dQ += Pooling^T(dA), dV += DWC^T(dO), dWd
 cudaError_t launch_backward_tail(int dtype, const BwdCall& c, cudaStream_t st);
 bool plan_backward(int slabs, int n, int N, int d, int sm_count, BwdPlan* out);   // false: shape not supported
 int backward_launch_count(const BwdCall& c);
 cudaError_t launch_backward(int dtype, const BwdCall& c, cudaStream_t st);
 // Tensor-core kernels of the two gradient stages (16-bit inputs, n <= 64, d = 64)
-bool backward_mma_eligible(int dtype, int n, int d);
-BwdPlan plan_backward_mma(int slabs, int N, int sm_count);
-cudaError_t launch_backward_mma(int dtype, bool broadcast_stage, const BwdArgs& a, cudaStream_t st);
+bool backward_umma_eligible(int dtype, int n, int d);
+size_t backward_umma_bytes(int slabs, int heads, int n, int N);
+cudaError_t launch_backward_umma(int dtype, bool broadcast_stage, const BwdCall& c, cudaStream_t st);
 
 }  // namespace aa
