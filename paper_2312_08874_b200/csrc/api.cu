@@ -868,13 +868,13 @@ int agent_attn_query_status(agent_attn_handle* h, void* stream) {
     return AA_OK;
 }
 
-// Workspace of the backward pass: [A | V_A | dV_A | dA | lse | dot | partial (max, sum) | terms], fp32, each
+// Workspace of the backward pass: [A | V_A | dV_A | dA | lse | dot | dWd copies | partial (max, sum) | terms], fp32, each
 // region 256-byte aligned (V_A, dV_A and dA are cleared as one, so their regions have one size).  The mixed-precision kernels
 // keep A in 16 bits in its region, the terms of V_A in that of the partials, (log-sum-exp, D) pairs over lse and dot, and the terms of
 // dV_A and the padded biases in that of the terms.
 namespace {
 struct BwdLayout {
-    size_t a, va, dva, da, lse, dot, part, terms, total;
+    size_t a, va, dva, da, lse, dot, dwd, part, terms, total;
 };
 bool use_mixed(const agent_attn_handle* h, int n) { return auto_like(h) && backward_umma_eligible(h->cfg.dtype, n, h->cfg.head_dim); }
 // inputs outside the mixed-precision kernels: fp32 operands as 16-bit terms on the tensor cores
@@ -888,7 +888,8 @@ bool bwd_layout(const agent_attn_handle* h, int N, int n, BwdPlan* pl, BwdLayout
     const size_t sn = align_up((size_t)slabs * n * sizeof(float), 256);
     w->a = 0; w->va = snd; w->dva = 2 * snd; w->da = 3 * snd;
     w->lse = 4 * snd; w->dot = w->lse + sn;
-    w->part = w->dot + sn;
+    w->dwd = w->dot + sn;
+    w->part = w->dwd + align_up((size_t)kFilterCopies * h->cfg.heads * h->cfg.head_dim * 9 * sizeof(float), 256);
     size_t part_floats = (size_t)slabs * pl->chunks * n * 2;
     if (part_floats * sizeof(float) < snd) part_floats = snd / sizeof(float);       // (mixed precision: two 16-bit terms of V_A)
     w->terms = w->part + align_up(part_floats * sizeof(float), 256);
@@ -954,7 +955,7 @@ int agent_attn_backward(agent_attn_handle* h, const void* Q, const void* K, cons
     c.ws_a = reinterpret_cast<float*>(ws + w.a); c.ws_va = reinterpret_cast<float*>(ws + w.va);
     c.ws_dva = reinterpret_cast<float*>(ws + w.dva); c.ws_da = reinterpret_cast<float*>(ws + w.da);
     c.ws_lse = reinterpret_cast<float*>(ws + w.lse); c.ws_dot = reinterpret_cast<float*>(ws + w.dot);
-    c.ws_part = reinterpret_cast<float*>(ws + w.part);
+    c.ws_part = reinterpret_cast<float*>(ws + w.part); c.ws_dwd = reinterpret_cast<float*>(ws + w.dwd);
     c.region_bytes = w.va;
     c.slabs = h->cfg.batch * h->cfg.heads; c.heads = h->cfg.heads; c.H = grid_h; c.W = grid_w;
     c.d = h->cfg.head_dim; c.n = n_agents; c.p = p; c.sm_count = h->sm_count;

@@ -404,7 +404,7 @@ cudaError_t backward_typed(const BwdCall& c, BwdArgs a, cudaStream_t st) {
     const size_t bias_elems = (size_t)a.heads * a.n * a.N;
     if (c.db1) AA_TRY(cudaMemsetAsync(c.db1, 0, bias_elems * sizeof(float), st));
     if (c.db2) AA_TRY(cudaMemsetAsync(c.db2, 0, bias_elems * sizeof(float), st));
-    if (c.dwd) AA_TRY(cudaMemsetAsync(c.dwd, 0, (size_t)a.heads * a.d * 9 * sizeof(float), st));
+    if (c.dwd) AA_TRY(cudaMemsetAsync(c.ws_dwd, 0, (size_t)kFilterCopies * a.heads * a.d * 9 * sizeof(float), st));
 
     bwd_pool_kernel<T><<<(unsigned)((snd + 255) / 256), 256, 0, st>>>(a, c.q, c.ws_a);
     AA_TRY(cudaGetLastError());

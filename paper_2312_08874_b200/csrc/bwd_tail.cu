@@ -3,11 +3,13 @@
 //   dV  += DWC^T(dO)       tap (u, v) of output token (y - u + 1, x - v + 1) read V[y][x]
 //   dWd += corr(dO, V)     dWd[c][u][v] = sum over tokens of dO[y - u + 1][x - v + 1][c] V[y][x][c]
 // Two kernels of threads that slide down a strip of rows of a grid column.  bwd_conv_tail does dV and dWd, two channels a thread: a row
-// brings three new window entries, the other six come from registers, an entry serves both its tap and its sum, and rows are requested
-// two ahead.  (Four channels a thread need twice the registers for taps and sums: with the taps in shared memory and two blocks of
-// eight warps an SM 60 us.)  bwd_pool_tail is a stream over dQ, four rows in flight.  dQ and dV are read and written in fp32, which is
-// the bound.  64 slabs of a 56 x 56 grid: 47 us (154 MB, 24 us at the copy bandwidth) and 16 us (103 MB, 16 us); one kernel for dQ and
-// dV with all nine window loads of a token, and one for dWd, took 74 and 31.
+// brings three new window entries, the other six come from registers, an entry serves both its tap and its sum, and dO is requested two
+// rows ahead.  (Four channels a thread need twice the registers for taps and sums: with the taps in shared memory and two blocks of
+// eight warps an SM 60 us; a spill of 100 bytes in the loop costs 26 us, so tokens are addressed by one offset.)  Its blocks add their
+// share of dWd to one of kFilterCopies copies, which the second kernel adds up: relative error 1.4e-7, against 5e-7 in a single copy.
+// bwd_pool_tail is a stream over dQ, four rows in flight.  dQ and dV are read and written in fp32, which is the bound.  64 slabs of a
+// 56 x 56 grid: 44 us (154 MB, 24 us at the copy bandwidth) and 16 us (103 MB, 16 us); one kernel for dQ and dV with all nine window
+// loads of a token, and one for dWd, took 74 and 31.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -18,7 +20,7 @@ namespace {
 struct TailArgs {
     const void *v, *go, *wd;
     const float* da;
-    float *dq, *dv, *dwd;
+    float *dq, *dv, *dwd, *dwd_copies;
     int heads, H, W, d, n, p, strip, strips, passes;
 };
 
@@ -78,6 +80,22 @@ __device__ __forceinline__ Column column_of(const TailArgs& a, int i) {
 __global__ void __launch_bounds__(kThreadsQ, 4) bwd_pool_tail_kernel(const TailArgs a) {
     __shared__ Windows yw[kAxis];
     const int d = a.d, H = a.H, W = a.W, p = a.p, slab = blockIdx.y;
+    if (a.dwd && blockIdx.x == gridDim.x - 1) {                   // the last column of blocks: the filter gradient's copies
+        pdl_wait_prior();
+        pdl_release_next();
+        const int words = a.heads * d * 9;
+        for (int o = slab * kThreadsQ + threadIdx.x; o < words; o += gridDim.y * kThreadsQ) {
+            float c[kFilterCopies];
+#pragma unroll
+            for (int k = 0; k < kFilterCopies; ++k) c[k] = a.dwd_copies[(size_t)k * words + o];
+#pragma unroll
+            for (int h = kFilterCopies / 2; h; h >>= 1)
+#pragma unroll
+                for (int k = 0; k < h; ++k) c[k] += c[k + h];
+            a.dwd[o] = c[0];
+        }
+        return;
+    }
     const int groups = d >> 2, cols = kThreadsQ / groups;         // d <= 128: at least eight columns at once
     const int cg = threadIdx.x % groups, cl = threadIdx.x / groups;
     for (int i = threadIdx.x; i < min(H, kAxis); i += kThreadsQ) yw[i] = windows_of(i, H, p);
@@ -148,41 +166,36 @@ __global__ void __launch_bounds__(kThreadsV, sizeof(T) == 4 ? 4 : 5) bwd_conv_ta
         for (int i = first + cl; i < last; i += cols) {
             const Column c = column_of(a, i);
             const bool left = c.x > 0, right = c.x + 1 < W;
-            const size_t base = ((size_t)slab * H * W + (size_t)c.y0 * W + c.x) * d + 2 * cg;
-            const T *v = static_cast<const T*>(a.v) + base, *go = static_cast<const T*>(a.go) + base;
-            float* dv = a.dv + base;
-            // rings of three rows: dO in fp32 (y - 1 .. y + 1), the dO rows on their way (y + 2, y + 3), dV and V (y .. y + 2)
+            size_t off = ((size_t)slab * H * W + (size_t)c.y0 * W + c.x) * d + 2 * cg;       // of row y + k
+            const T *v = static_cast<const T*>(a.v), *go = static_cast<const T*>(a.go);
+            // rings of three rows: dO in fp32 (y - 1 .. y + 1), the dO rows on their way (y + 2, y + 3), dV and V (y, y + 1)
             float2 win[3][3], o[3];
             Raw2<T> raw[3][3], rv[3];
-            auto row = [&](Raw2<T> (&r)[3], const T* g, int y) {
+            auto row = [&](Raw2<T> (&r)[3], size_t at, int y) {
                 const bool in = (unsigned)y < (unsigned)H;
-                r[0] = ld_raw2<T>(g - d, in && left);
-                r[1] = ld_raw2<T>(g, in);
-                r[2] = ld_raw2<T>(g + d, in && right);
+                r[0] = ld_raw2<T>(go + at - d, in && left);
+                r[1] = ld_raw2<T>(go + at, in);
+                r[2] = ld_raw2<T>(go + at + d, in && right);
             };
             auto convert = [&](float2 (&f)[3], const Raw2<T> (&r)[3]) {
 #pragma unroll
                 for (int k = 0; k < 3; ++k) f[k] = pair<T>(r[k]);
             };
-            row(raw[2], go - pitch, c.y0 - 1);
-            row(raw[0], go, c.y0);
-            o[0] = ld_pair(dv, true);
-            if (DWD) rv[0] = ld_raw2<T>(v, true);
-            o[1] = ld_pair(dv + pitch, c.y0 + 1 < c.y1);
-            if (DWD) rv[1] = ld_raw2<T>(v + pitch, c.y0 + 1 < c.y1);
-            row(raw[1], go + pitch, c.y0 + 1);
+            row(raw[2], off - pitch, c.y0 - 1);
+            row(raw[0], off, c.y0);
+            o[0] = ld_pair(a.dv + off, true);
+            if (DWD) rv[0] = ld_raw2<T>(v + off, true);
+            row(raw[1], off + pitch, c.y0 + 1);
             convert(win[2], raw[2]);
             convert(win[0], raw[0]);
-            go += 2 * pitch;
-            row(raw[2], go, c.y0 + 2);
+            row(raw[2], off + 2 * pitch, c.y0 + 2);
             for (int y = c.y0; y < c.y1; y += 3)
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {                     // row y + k (rows past the strip: zeros, not stored)
-                    const int y2 = y + k + 2;
-                    go += pitch;
-                    row(raw[k], go, y2 + 1);
-                    o[(k + 2) % 3] = ld_pair(dv + 2 * pitch, y2 < c.y1);
-                    if (DWD) rv[(k + 2) % 3] = ld_raw2<T>(v + 2 * pitch, y2 < c.y1);
+                    const bool more = y + k + 1 < c.y1;
+                    row(raw[k], off + 3 * pitch, y + k + 3);
+                    o[(k + 1) % 3] = ld_pair(a.dv + off + pitch, more);
+                    if (DWD) rv[(k + 1) % 3] = ld_raw2<T>(v + off + pitch, more);
                     convert(win[(k + 1) % 3], raw[(k + 1) % 3]);
                     float2 s = o[k];
                     const float2 t = DWD ? pair<T>(rv[k]) : make_float2(0.f, 0.f);
@@ -192,15 +205,16 @@ __global__ void __launch_bounds__(kThreadsV, sizeof(T) == 4 ? 4 : 5) bwd_conv_ta
                         s = ffma2(g, tap[8 - j], s);
                         if (DWD) acc[8 - j] = ffma2(g, t, acc[8 - j]);
                     }
-                    if (y + k < c.y1) *reinterpret_cast<float2*>(dv) = s;
-                    dv += pitch;
-                    v += pitch;
+                    if (y + k < c.y1) *reinterpret_cast<float2*>(a.dv + off) = s;
+                    off += pitch;
                 }
         }
     if (DWD) {
 #pragma unroll
         for (int k = 0; k < 9; ++k) red[threadIdx.x][k] = acc[k];
         __syncthreads();
+        // one of several copies: a sum of all blocks' shares in one word would round as often as there are blocks
+        float* copy = a.dwd_copies + ((size_t)((blockIdx.x + blockIdx.y) % kFilterCopies) * a.heads + slab % a.heads) * d * 9;
         for (int o = threadIdx.x; o < d * 9; o += kThreadsV) {    // o = channel * 9 + tap
             const int c = o / 9, k = o - c * 9;
             float s = 0.f;
@@ -208,7 +222,7 @@ __global__ void __launch_bounds__(kThreadsV, sizeof(T) == 4 ? 4 : 5) bwd_conv_ta
                 const float2 t = red[l * groups + (c >> 1)][k];
                 s += (c & 1) ? t.y : t.x;
             }
-            atomicAdd(a.dwd + (size_t)(slab % a.heads) * d * 9 + o, s);
+            atomicAdd(copy + o, s);
         }
     }
 }
@@ -236,7 +250,8 @@ template <typename T> cudaError_t launch_tail(TailArgs a, int slabs, int sm_coun
         const cudaError_t e = launch_dependent(a.dwd ? bwd_conv_tail_kernel<T, true> : bwd_conv_tail_kernel<T, false>, grid, kThreadsV, 0, st, a);
         if (e != cudaSuccess) return e;
     }
-    const dim3 grid = plan_strips(&a, slabs, kThreadsQ / (a.d / 4), 4 * sm_count, 0, 4);
+    dim3 grid = plan_strips(&a, slabs, kThreadsQ / (a.d / 4), 4 * sm_count, 0, 4);
+    if (a.dwd) ++grid.x;
     return launch_dependent(bwd_pool_tail_kernel, grid, kThreadsQ, 0, st, a);
 }
 
@@ -244,7 +259,7 @@ template <typename T> cudaError_t launch_tail(TailArgs a, int slabs, int sm_coun
 
 cudaError_t launch_backward_tail(int dtype, const BwdCall& c, cudaStream_t st) {
     TailArgs a;
-    a.v = c.v; a.go = c.d_out; a.wd = c.wd; a.da = c.ws_da; a.dq = c.dq; a.dv = c.dv; a.dwd = c.dwd;
+    a.v = c.v; a.go = c.d_out; a.wd = c.wd; a.da = c.ws_da; a.dq = c.dq; a.dv = c.dv; a.dwd = c.dwd; a.dwd_copies = c.ws_dwd;
     a.heads = c.heads; a.H = c.H; a.W = c.W; a.d = c.d; a.n = c.n; a.p = c.p; a.strip = a.strips = a.passes = 0;
     switch (dtype) {
         case kF32:  return launch_tail<float>(a, c.slabs, c.sm_count, st);

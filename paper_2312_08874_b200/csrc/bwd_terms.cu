@@ -185,7 +185,7 @@ template <typename T, typename E, int NT> cudaError_t pool_and_clear(const BwdCa
     cl.p[0] = c.ws_dva; cl.words[0] = 2 * c.region_bytes / sizeof(float);          // dV_A, dA
     cl.p[1] = c.db1; cl.words[1] = c.db1 ? bias : 0;
     cl.p[2] = c.db2; cl.words[2] = c.db2 ? bias : 0;
-    cl.p[3] = c.dwd; cl.words[3] = c.dwd ? (size_t)c.heads * c.d * 9 : 0;
+    cl.p[3] = c.ws_dwd; cl.words[3] = c.dwd ? (size_t)kFilterCopies * c.heads * c.d * 9 : 0;
     return launch_pool_terms<T, E, NT>(pa, a_t, cl, pl, st);
 }
 
