@@ -25,23 +25,28 @@ cudaError_t stage(int dtype, int d, int st, const BwdTermArgs& a, const BwdTermL
 
 // Buffers that later kernels add to, cleared by extra blocks of the first kernel.
 struct ClearList {
-    float* p[4];
-    size_t words[4];
+    float* p[7];
+    size_t words[7];
     int pool_blocks;
 };
 constexpr int kClearWords = 256 * 32;              // words that a block clears
-// Biases as rows of 64 agents per token [heads][N][64] (zeros past n), by further blocks of the first kernel: B1 transposed, B2.
+// Biases as rows of `width` agents per token [heads][N][width] (zeros past n), by further blocks of the first kernel: B1 transposed, B2.
 struct PadList {
     const void *b1, *b2;
     void *p1, *p2;
-    int heads, n, N, blocks1, blocks2;
+    int heads, n, N, width, blocks1, blocks2;
 };
+PadList pad_list(const void* b1, const void* b2, void* p1, void* p2, int heads, int n, int N) {
+    const int width = (n + 63) / 64 * 64, blocks = (int)(((size_t)heads * N * (width / 8) + 255) / 256);
+    return {b1, b2, p1, p2, heads, n, N, width, b1 && p1 ? blocks : 0, b2 && p2 ? blocks : 0};
+}
 template <typename T> __device__ __forceinline__ void pad_bias(const T* src, uint4* dst, bool transposed, const PadList& pl, int block) {
     const long long rows = (long long)pl.heads * pl.N, i = (long long)block * 256 + threadIdx.x;
     // neighbouring threads: B1 is read along its tokens, B2 along its agents
-    const long long row = transposed ? i % rows : i >> 3;
-    const int c0 = 8 * (int)(transposed ? i / rows : i & 7);
-    if (c0 >= 64 || row >= rows) return;
+    const int chunks = pl.width >> 3;
+    const long long row = transposed ? i % rows : i / chunks;
+    const int c0 = 8 * (int)(transposed ? i / rows : i % chunks);
+    if (c0 >= pl.width || row >= rows) return;
     const int head = (int)(row / pl.N), tok = (int)(row - (long long)head * pl.N);
     __align__(16) T v[8];
 #pragma unroll
@@ -49,7 +54,7 @@ template <typename T> __device__ __forceinline__ void pad_bias(const T* src, uin
         const int c = c0 + k;
         v[k] = c >= pl.n ? Elem<T>::from_f32(0.f) : transposed ? src[((size_t)head * pl.n + c) * pl.N + tok] : src[(size_t)row * pl.n + c];
     }
-    dst[row * 8 + (c0 >> 3)] = *reinterpret_cast<const uint4*>(v);
+    dst[row * chunks + (c0 >> 3)] = *reinterpret_cast<const uint4*>(v);
 }
 
 struct PoolArgs8 {
@@ -68,7 +73,7 @@ __global__ void __launch_bounds__(256) bwd_pool_terms_kernel(PoolArgs8 pa, E* ds
     if ((int)blockIdx.x >= cl.pool_blocks) {
         size_t b = (size_t)(blockIdx.x - cl.pool_blocks) * kClearWords;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < 7; ++k) {
             const size_t room = (cl.words[k] + kClearWords - 1) / kClearWords * kClearWords;
             if (b < room) {
                 const size_t e = min(b + kClearWords, cl.words[k]), e4 = b + ((e - b) & ~(size_t)3);
@@ -78,7 +83,7 @@ __global__ void __launch_bounds__(256) bwd_pool_terms_kernel(PoolArgs8 pa, E* ds
             }
             b -= room;
         }
-        if constexpr (NT == 1) {
+        if constexpr (sizeof(T) == 2) {
             const int block = (int)(b / kClearWords);
             if (block < pl.blocks1) pad_bias<T>(static_cast<const T*>(pl.b1), static_cast<uint4*>(pl.p1), true, pl, block);
             else pad_bias<T>(static_cast<const T*>(pl.b2), static_cast<uint4*>(pl.p2), false, pl, block - pl.blocks1);
@@ -178,7 +183,7 @@ template <typename T, typename E, int NT> cudaError_t launch_pool_terms(PoolArgs
     return launch_dependent(bwd_pool_terms_kernel<T, E, NT>, dim3((unsigned)(cl.pool_blocks + clear + pl.blocks1 + pl.blocks2)), 256, 0, st, pa, static_cast<E*>(a_t), cl, pl);
 }
 // Pooling, and the clearing of the sums that the stages add to.
-template <typename T, typename E, int NT> cudaError_t pool_and_clear(const BwdCall& c, void* a_t, bool clear_bias, const PadList& pl, cudaStream_t st) {
+template <typename T, typename E, int NT> cudaError_t pool_and_clear(const BwdCall& c, void* a_t, bool clear_bias, bool clear_rows, const PadList& pl, cudaStream_t st) {
     const PoolArgs8 pa = {c.q, nullptr, nullptr, c.slabs, c.n, c.H, c.W, c.p, c.d, false};
     ClearList cl = {};
     const size_t bias = clear_bias ? (size_t)c.heads * c.n * c.H * c.W : 0;
@@ -186,6 +191,8 @@ template <typename T, typename E, int NT> cudaError_t pool_and_clear(const BwdCa
     cl.p[1] = c.db1; cl.words[1] = c.db1 ? bias : 0;
     cl.p[2] = c.db2; cl.words[2] = c.db2 ? bias : 0;
     cl.p[3] = c.ws_dwd; cl.words[3] = c.dwd ? (size_t)kFilterCopies * c.heads * c.d * 9 : 0;
+    float* const rows[3] = {c.dq, c.dk, c.dv};
+    for (int k = 0; k < 3; ++k) { cl.p[4 + k] = rows[k]; cl.words[4 + k] = clear_rows ? (size_t)c.slabs * c.H * c.W * c.d : 0; }
     return launch_pool_terms<T, E, NT>(pa, a_t, cl, pl, st);
 }
 
@@ -196,16 +203,15 @@ bool backward_terms_eligible(int dtype, int n, int d) {
     const int dk = dk_of_terms(d), pitch = dk * 2 + 16, n32 = (n + 31) & ~31;
     return 6 * n32 * pitch + n32 * 8 <= 227 * 1024;
 }
-size_t backward_terms_bytes(int slabs, int n, int N, int d) {
-    return 3 * up256((size_t)slabs * n * d * 2 * 3) + up256((size_t)slabs * N * 8) + up256((size_t)slabs * n * 8);
+size_t backward_terms_bytes(int dtype, int slabs, int heads, int n, int N, int d) {
+    return (backward_terms_umma_eligible(dtype, n, N, d) ? backward_terms_umma_bytes(heads, n, N) : 0) + 3 * up256((size_t)slabs * n * d * 2 * 3) + up256((size_t)slabs * N * 8) + up256((size_t)slabs * n * 8);
 }
 
 cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStream_t st) {
     const size_t rows = (size_t)c.heads * c.H * c.W;
     char* padded = static_cast<char*>(c.ws_mixed) + up256((size_t)2 * c.slabs * c.n * 64 * 2);          // (see backward_umma_bytes)
-    const int blocks = (int)((rows * 8 + 255) / 256);
-    const PadList pl = {c.b1, c.b2, padded, padded + rows * 128, c.heads, c.n, c.H * c.W, c.b1 ? blocks : 0, c.b2 ? blocks : 0};
-    cudaError_t e = dtype == kBF16 ? pool_and_clear<__nv_bfloat16, __nv_bfloat16, 1>(c, c.ws_a, true, pl, st) : pool_and_clear<__half, __half, 1>(c, c.ws_a, true, pl, st);
+    const PadList pl = pad_list(c.b1, c.b2, padded, padded + rows * 128, c.heads, c.n, c.H * c.W);
+    cudaError_t e = dtype == kBF16 ? pool_and_clear<__nv_bfloat16, __nv_bfloat16, 1>(c, c.ws_a, true, false, pl, st) : pool_and_clear<__half, __half, 1>(c, c.ws_a, true, false, pl, st);
     if (e != cudaSuccess) return e;
     BwdTermArgs a;
     memset(&a, 0, sizeof(a));
@@ -243,7 +249,10 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
     cudaError_t e;
 #define AA_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
     const bool clear_bias = slabs != c.heads;          // (a single batch entry stores its bias gradients)
-    AA_TRY(dtype == kBF16 ? (pool_and_clear<B, B, 3>(c, a_t, clear_bias, PadList{}, st)) : dtype == kF16 ? (pool_and_clear<__half, B, 3>(c, a_t, clear_bias, PadList{}, st)) : (pool_and_clear<float, B, 3>(c, a_t, clear_bias, PadList{}, st)));
+    const bool umma = backward_terms_umma_eligible(dtype, n, N, d), clear_rows = umma && n > 64;      // (blocks of 64 agents add to the rows)
+    void *pad1 = nullptr, *pad2 = nullptr;
+    if (umma) backward_terms_umma_padded(c.heads, n, N, w + 3 * terms + up256((size_t)slabs * N * 8) + up256((size_t)slabs * n * 8), &pad1, &pad2);
+    AA_TRY(dtype == kBF16 ? (pool_and_clear<B, B, 3>(c, a_t, clear_bias, clear_rows, pad_list(c.b1, c.b2, pad1, pad2, c.heads, n, N), st)) : dtype == kF16 ? (pool_and_clear<__half, B, 3>(c, a_t, clear_bias, clear_rows, PadList{}, st)) : (pool_and_clear<float, B, 3>(c, a_t, clear_bias, clear_rows, PadList{}, st)));
 
     BwdTermArgs a;
     memset(&a, 0, sizeof(a));
@@ -273,12 +282,17 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
     // broadcast stage: token statistics, then dV_A and its share of dA
     a.x = c.q; a.y = c.d_out; a.bias = c.b2; a.scale = a.out_scale = c.scale2; a.m_t = va_t;
     AA_TRY(rows(kTermStats));
-    a.outer0 = c.ws_dva; a.outer1 = c.ws_da;
-    AA_TRY(sums(kTermBroadcast, false));
-    a.row0 = c.dq; a.dbias = c.db2;
-    AA_TRY(rows(kTermQuery));
+    if (umma) {
+        AA_TRY(launch_backward_terms_umma(true, c, a_t, va_t, tok_stats, pad2, st));
+    } else {
+        a.outer0 = c.ws_dva; a.outer1 = c.ws_da;
+        AA_TRY(sums(kTermBroadcast, false));
+        a.row0 = c.dq; a.dbias = c.db2;
+        AA_TRY(rows(kTermQuery));
+    }
     AA_TRY((launch_dependent(bwd_dot_split_kernel<B, 3>, dim3((slabs * n + 7) / 8), 256, 0, st, (const float*)c.ws_va, (const float*)c.ws_dva, agent_stats, static_cast<B*>(dva_t), slabs * n, d)));
     // aggregation stage
+    if (umma) return launch_backward_terms_umma(false, c, a_t, dva_t, agent_stats, pad1, st);
     a.x = c.k; a.y = c.v; a.bias = c.b1; a.scale = c.scale1; a.out_scale = N == 1 ? 0.f : c.scale1; a.m_t = dva_t; a.dbias = c.db1;
     AA_TRY(sums(kTermAggregate, false));
     a.row0 = c.dk; a.row1 = c.dv; a.dbias = nullptr;

@@ -1,0 +1,504 @@
+// Backward pass with fp32 accuracy on the 5th-generation tensor cores: the two gradient stages for bf16 tensors of up to 64 channels.
+//
+// Broadcast stage (X = Q, Y = dO, M = V_A):   S = X A^T, dP = Y M^T, P = exp(S - lse[token]), dS = P o (dP - dot[token]);
+//     dQ += scale dS A,  dV_A += P^T Y,  dA += scale dS^T X,  dB2 += dS.
+// Aggregation stage (X = K, Y = V, M = dV_A): S = X A^T, dP = Y M^T, P = exp(S - lse[agent]), dS = P o (dP - D[agent]);
+//     dK += scale dS A,  dV += P M,  dA += scale dS^T X,  dB1 += dS.
+// A, M, P and dS are sums of three bf16 terms, a product keeps the six pairs of order below three (bwd_terms.cuh).
+//
+// Unit of work: 64 agents of a slab x 128 tokens.  One block per SM takes a contiguous run of the (slab, tile) sequence for its 64 agents;
+// blocks for the other agents of a slab run beside it, so that X and Y come from DRAM once.  The terms of A and M stay in shared memory.  Roles as in bwd_umma.cu: eight row warps (thread = token, half of the agents), four
+// output warps, a TMA warp, an issuer of S and dP, an issuer of the products of P and dS.  P and dS are in fp32 registers while the
+// products of the tile before run, and are split into terms once those have read theirs: 96 KB of term tiles fit once, not twice.
+//
+// Accuracy: an accumulation in tensor memory does not round to nearest, so a chain drifts with its length (see term_sum).  The small pairs
+// therefore come first, sums over tokens leave tensor memory after every tile and join in fp32 registers, and the agents' share of a
+// token's gradient leaves after 64 of them.
+//
+// What bounds it: fp32 reductions, about 2 TB/s (a tile adds 32 KB of bias gradients and 32 KB per output); without them a tile takes
+// 6000 cycles of 9400, of which splitting and storing terms is 2000 beside operand reads of the tensor pipe (shared memory at 60 %).
+// 16 slabs of a 128 x 128 grid, 256 agents, biases: broadcast 328 us, aggregation 378 us; as two mma.sync kernels each (bwd_sums_kernel,
+// bwd_rows_kernel) 828 and 1010 us.  96 slabs of 14 x 14, 81 agents, whole pass: 313 -> 215 us; one slab of 40 x 23, 49 agents of 32
+// channels: 62 -> 52 us.
+#include "bwd_terms_launch.cuh"
+#include "stream_common.cuh"
+
+#include <algorithm>
+#include <cstring>
+
+namespace aa {
+
+namespace {
+
+constexpr int kTok = 128;                    // tokens per tile
+constexpr int kTile = kTok * 128;            // bytes of a swizzled [128][64] tile of 16-bit elements
+constexpr int kMat = 64 * 128;               // bytes of a [64][64] tile
+constexpr int kStages = 2, kTerms = 3;
+constexpr int kStage = 2 * kTile;            // X | Y
+constexpr int kRowThreads = 256, kThreads = kRowThreads + 128 + 96;
+
+// shared memory (bytes from a 1024-aligned base; mbarriers and two words of the block at its start)
+constexpr int OFF_DEAD = 128, OFF_TMEM = 132;
+constexpr int OFF_RING = 1024;
+constexpr int OFF_AM = OFF_RING + kStages * kStage;          // terms of A, terms of M
+constexpr int OFF_P = OFF_AM + 2 * kTerms * kMat;            // per term: P | dS
+constexpr int OFF_BIAS = OFF_P + 2 * kTerms * kTile;         // [128 tokens][64 agents], or twice [64 agents][64 tokens]
+constexpr int OFF_STAT = OFF_BIAS + kTile;                   // aggregation: [2][64] (lse, D)
+constexpr int kSmemBytes = OFF_STAT + 2 * 64 * 8 + 1024;
+static_assert(kSmemBytes <= 232448 && kSmemBytes > 116 * 1024, "one block per SM");
+
+// mbarriers                        count             waiter
+constexpr int BAR_FULL = 0;   // [2] tx               issuer of S and dP
+constexpr int BAR_AM = 2;     //     tx               the same
+constexpr int BAR_S = 3;      //     commit           row warps: S and dP of a tile
+constexpr int BAR_READ = 4;   //     row warps        issuer of S and dP: they have been read
+constexpr int BAR_P = 5;      //     row warps        issuer of the products: P and dS written
+constexpr int BAR_DONE = 6;   // [2] commit           row warps, output warps: every product of a tile (producer: the last tile of a slab)
+constexpr int BAR_OUT = 8;    // [2] output warps     issuer of the products: outputs and sums read
+constexpr int BAR_DRAIN = 10; // [2] commit           each issuer, once, at its end
+constexpr int BAR_BIAS = 12;  //     tx               row warps
+constexpr int BAR_BREAD = 13; //     row warps        producer: the biases have been read
+constexpr int BAR_FREE = 14;  // [2] commit           producer: the sums of a tile, the last to read its X and Y
+constexpr int kBars = 16;
+static_assert(8 * kBars <= OFF_DEAD, "mbarriers");
+constexpr int kTimeoutTile = 3, kTimeoutRole = 6;
+
+// tensor memory columns: S | dP; then twice (broadcast) sums of P^T [X | Y] and dS^T [X | Y] | dQ, (aggregation) dK | dV | sums of dS^T X
+constexpr uint32_t TM_S = 0, TM_BUF = 128, kBufCols = 192;
+
+struct Args {
+    const float2* stats;      // broadcast: (log2-sum-exp, row dot) [slabs][N]; aggregation: (log2-sum-exp, D) [slabs][n]
+    float *outer0, *outer1;   // fp32 [slabs][n][d]: dV_A (broadcast) and dA (added)
+    float *row0, *row1;       // fp32 [slabs][N][d]: dQ, or dK and dV (added where there are several blocks of agents)
+    float* dbias;             // fp32 [heads][N][n] (broadcast) or [heads][n][N] (added; stored where the batch has one entry), or null
+    int* status;
+    int slabs, heads, N, n, d, tiles, blocks;
+    int bias;                 // 0: none; 1: tiles of token rows; 2: tiles of agent rows
+    float scale;
+    alignas(64) CUtensorMap tm_x, tm_y, tm_a, tm_m, tm_b;
+};
+
+__device__ __forceinline__ uint64_t desc_mn(uint32_t addr, uint32_t lead) {       // MN-major operand: two tiles of 64, `lead` bytes apart
+    return (umma_desc_sw128(addr) & ~((uint64_t)0x3fffu << 16)) | ((uint64_t)(lead >> 4) << 16);
+}
+// 16 lanes x 64 fp32 columns in mma.sync accumulator layout: r[4 j + 2 h + e] = (row g + 8 h, column 8 j + 2 t + e)
+__device__ __forceinline__ void tmem_ld_16x256b_x8(uint32_t taddr, float (&r)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
+        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]),
+          "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15]),
+          "=f"(r[16]), "=f"(r[17]), "=f"(r[18]), "=f"(r[19]), "=f"(r[20]), "=f"(r[21]), "=f"(r[22]), "=f"(r[23]),
+          "=f"(r[24]), "=f"(r[25]), "=f"(r[26]), "=f"(r[27]), "=f"(r[28]), "=f"(r[29]), "=f"(r[30]), "=f"(r[31])
+        : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void st_shared4(uint32_t addr, const uint32_t (&v)[4]) {
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+// split_pair of three bf16 terms, the residuals by packed arithmetic
+__device__ __forceinline__ void split3(float2 v, uint32_t (&w)[kTerms]) {
+    w[0] = pack2_finite<__nv_bfloat16>(v.x, v.y);
+#pragma unroll
+    for (int i = 1; i < kTerms; ++i) {
+        v = ffma2(unpack2<__nv_bfloat16>(w[i - 1]), make_float2(-1.f, -1.f), v);
+        w[i] = pack2<__nv_bfloat16>(v.x, v.y);
+    }
+}
+
+template <bool BCAST>
+__global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __grid_constant__ Args p) {
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int N = p.N, n = p.n, d = p.d;
+    const int ab = blockIdx.x % p.blocks, lanes = gridDim.x / p.blocks, me = blockIdx.x / p.blocks;      // block of 64 agents; runs of its sequence
+    const long long total = (long long)p.slabs * p.tiles, first = total * me / lanes;
+    const int count = (int)(total * (me + 1) / lanes - first);
+    int slab = (int)(first / p.tiles), tile = (int)(first - (long long)slab * p.tiles);     // of the role's current tile
+    const uint32_t base = smem_u32(smem);
+
+    Pipe pp;
+    pp.status = p.status;
+    pp.dead = reinterpret_cast<int*>(smem + OFF_DEAD);
+    pp.bars = base;
+    pp.ph = 0u;
+    if (tid == 0) {
+        *pp.dead = 0;
+        for (int i = 0; i < kBars; ++i) mbar_init(pp.bars + 8 * i, i == BAR_READ || i == BAR_P || i == BAR_BREAD ? 8u : i >= BAR_OUT && i < BAR_DRAIN ? 4u : 1u);
+        mbar_fence_init();
+    }
+    if (warp == 0) tmem_alloc<512>(base + OFF_TMEM);
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    pp.tmem = *reinterpret_cast<const volatile uint32_t*>(smem + OFF_TMEM);
+    pdl_wait_prior();
+    pdl_release_next();
+    auto advance = [&] {
+        if (++tile == p.tiles) { tile = 0; ++slab; }
+    };
+
+    if (warp == 12) {
+        // ------------------------------------------------------------------ producer
+        if (lane == 0) {
+            for (int i = 0; i < count && !pipe_dead(pp); ++i, advance()) {
+                const int b = i & 1;
+                if (i >= 2) wait_spin(pp, BAR_FREE + b, (i >> 1) - 1, kTimeoutRole);
+                const uint32_t bar = pipe_bar(pp, BAR_FULL + b), dst = base + OFF_RING + b * kStage;
+                mbar_arrive_expect_tx(bar, kStage);
+                tma_load_3d(dst, &p.tm_x, 0, tile * kTok, slab, bar);
+                tma_load_3d(dst + kTile, &p.tm_y, 0, tile * kTok, slab, bar);
+                if (p.bias) {
+                    if (i > 0) wait_spin(pp, BAR_BREAD, i - 1, kTimeoutRole);
+                    const uint32_t bb = pipe_bar(pp, BAR_BIAS), to = base + OFF_BIAS;
+                    const int head = slab % p.heads;
+                    mbar_arrive_expect_tx(bb, kTile);
+                    if (p.bias == 1) {
+                        tma_load_3d(to, &p.tm_b, ab * 64, tile * kTok, head, bb);
+                    } else {
+                        tma_load_3d(to, &p.tm_b, tile * kTok, ab * 64, head, bb);
+                        tma_load_3d(to + kMat, &p.tm_b, tile * kTok + 64, ab * 64, head, bb);
+                    }
+                }
+                if (i == 0 || tile == 0) {
+                    if (i > 0) wait_spin(pp, BAR_DONE + (b ^ 1), (i - 1) >> 1, kTimeoutRole);  // the last tile of the slab before
+                    const uint32_t bam = pipe_bar(pp, BAR_AM), am = base + OFF_AM;
+                    mbar_arrive_expect_tx(bam, 2 * kTerms * kMat);
+                    for (int t = 0; t < kTerms; ++t) {
+                        tma_load_3d(am + t * kMat, &p.tm_a, 0, ab * 64, t * p.slabs + slab, bam);
+                        tma_load_3d(am + (kTerms + t) * kMat, &p.tm_m, 0, ab * 64, t * p.slabs + slab, bam);
+                    }
+                }
+            }
+        }
+        __syncwarp();
+    } else if (warp == 13) {
+        // ------------------------------------------------------------------ S and dP
+        const uint32_t id = umma_idesc(1, 128, 64, 0), ts = pp.tmem + TM_S;
+        const uint64_t da = umma_desc_sw128(base + OFF_AM);
+        int groups = 0;
+        for (int i = 0; i < count && !pipe_dead(pp); ++i, advance()) {
+            const int b = i & 1;
+            if (i == 0 || tile == 0) wait_spin(pp, BAR_AM, groups++, kTimeoutTile);
+            wait_spin(pp, BAR_FULL + b, i >> 1, kTimeoutTile);
+            if (i > 0) wait_spin(pp, BAR_READ, i - 1, kTimeoutRole);
+            tc_fence_after_sync();
+            const uint64_t dx = umma_desc_sw128(base + OFF_RING + b * kStage);
+            // descriptor start addresses count 16-byte units: + 2 per k step of a K-major operand (32 bytes)
+#pragma unroll
+            for (int which = 0; which < 2; ++which)
+#pragma unroll
+                for (int t = kTerms - 1; t >= 0; --t)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        umma_ss_w(ts + 64 * which, dx + which * (kTile >> 4) + 2 * k, da + (which * kTerms + t) * (kMat >> 4) + 2 * k, id, t < kTerms - 1 || k > 0);
+            umma_commit_w(pipe_bar(pp, BAR_S));
+        }
+        umma_drain_w(pp, BAR_DRAIN);
+        __syncwarp();
+    } else if (warp == 14) {
+        // ------------------------------------------------------------------ products of P and dS
+        const uint32_t id_out = umma_idesc(1, 128, 64, 1), id_sum = umma_idesc(1, 128, BCAST ? 128 : 64, 1) | (1u << 15);
+        const uint64_t dp = umma_desc_sw128(base + OFF_P), da = umma_desc_sw128(base + OFF_AM), dps = desc_mn(base + OFF_P, kTile);
+        for (int i = 0; i < count && !pipe_dead(pp); ++i) {
+            const int b = i & 1;
+            wait_spin(pp, BAR_P, i, kTimeoutRole);
+            if (i >= 2) wait_spin(pp, BAR_OUT + b, (i >> 1) - 1, kTimeoutRole);
+            tc_fence_after_sync();
+            const uint64_t dxy = desc_mn(base + OFF_RING + b * kStage, kTile);
+            const uint32_t tb = pp.tmem + TM_BUF + kBufCols * b;
+            // + 128 per k step of an MN-major operand (16 rows of 128 bytes)
+#pragma unroll
+            for (int t = kTerms - 1; t >= 0; --t)
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    umma_ss_w(tb + (BCAST ? 0 : 128), dps + t * (2 * kTile >> 4) + 128 * k, dxy + 128 * k, id_sum, t < kTerms - 1 || k > 0);
+            umma_commit_w(pipe_bar(pp, BAR_FREE + b));
+            // pairs of terms (t of dS or P, u of A or M), the smallest first
+#pragma unroll
+            for (int which = 0; which < (BCAST ? 1 : 2); ++which)
+#pragma unroll
+                for (int order = kTerms - 1; order >= 0; --order)
+#pragma unroll
+                    for (int t = 0; t <= order; ++t)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            umma_ss_w(tb + (BCAST ? 128 : 64 * which), dp + (2 * t + 1 - which) * (kTile >> 4) + 2 * k,
+                                      da + (which * kTerms + order - t) * (kMat >> 4) + 128 * k, id_out, order < kTerms - 1 || t > 0 || k > 0);
+            umma_commit_w(pipe_bar(pp, BAR_DONE + b));
+        }
+        umma_drain_w(pp, BAR_DRAIN + 1);
+        __syncwarp();
+    } else if (warp >= 8) {
+        // ------------------------------------------------------------------ outputs
+        const int q = warp & 3, g = lane >> 2, t = lane & 3;
+        const bool second = q >= 2, sums = BCAST || second;            // lanes 64 ..: rows of dS
+        float acc[2][32];                                              // rows 16 f + g + 8 h of the warp's 32
+#pragma unroll
+        for (int f = 0; f < 2; ++f)
+#pragma unroll
+            for (int k = 0; k < 32; ++k) acc[f][k] = 0.f;
+        for (int i = 0; i < count; ++i, advance()) {
+            const int b = i & 1;
+            const uint32_t rows = pp.tmem + TM_BUF + kBufCols * b + ((uint32_t)(32 * q) << 16);
+            wait_par(pp, BAR_DONE + b, i >> 1, kTimeoutTile);
+            tc_fence_after_sync();
+            float o[32];
+            if (sums)
+#pragma unroll
+                for (int f = 0; f < 2; ++f) {
+                    tmem_ld_16x256b_x8(rows + (BCAST ? (second ? 0u : 64u) : 128u) + ((uint32_t)(16 * f) << 16), o);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int k = 0; k < 32; k += 2) {
+                        const float2 v = fadd2(make_float2(acc[f][k], acc[f][k + 1]), make_float2(o[k], o[k + 1]));
+                        acc[f][k] = v.x;
+                        acc[f][k + 1] = v.y;
+                    }
+                }
+            const int tok0 = tile * kTok + 32 * q + g;
+#pragma unroll
+            for (int which = 0; which < (BCAST ? 1 : 2); ++which) {
+                float* dst = which == 0 ? p.row0 : p.row1;
+                const float scale = which == 0 ? p.scale : 1.f;
+#pragma unroll
+                for (int f = 0; f < 2; ++f) {
+                    tmem_ld_16x256b_x8(rows + (BCAST ? 128u : 64u * which) + ((uint32_t)(16 * f) << 16), o);
+                    tmem_ld_wait();
+                    if (which == (BCAST ? 0 : 1) && f == 1) {          // everything is in registers: hand the buffer back before the stores
+                        tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) pipe_arrive(pp, BAR_OUT + b);
+                    }
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int tok = tok0 + 16 * f + 8 * h;
+                        if (tok >= N) continue;
+                        float* r = dst + ((size_t)slab * N + tok) * d + 2 * t;
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            if (8 * j >= d) break;
+                            const float2 v = make_float2(scale * o[4 * j + 2 * h], scale * o[4 * j + 2 * h + 1]);
+                            if (p.blocks == 1) *reinterpret_cast<float2*>(r + 8 * j) = v;
+                            else red_add2(r + 8 * j, v.x, v.y);
+                        }
+                    }
+                }
+            }
+            if (sums && (tile == p.tiles - 1 || i == count - 1)) {     // the last tile of the slab in this block
+                float* dst = second ? p.outer1 : p.outer0;
+                const float scale = second ? p.scale : 1.f;
+#pragma unroll
+                for (int f = 0; f < 2; ++f)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int r = ab * 64 + 32 * (q & 1) + 16 * f + 8 * h + g;
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            if (r < n && 8 * j < d) red_add2(dst + ((size_t)slab * n + r) * d + 8 * j + 2 * t, scale * acc[f][4 * j + 2 * h], scale * acc[f][4 * j + 2 * h + 1]);
+                            acc[f][4 * j + 2 * h] = acc[f][4 * j + 2 * h + 1] = 0.f;
+                        }
+                    }
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ row warps
+        const int q = warp & 3, half = warp >> 2, r = 32 * q + lane;
+        const uint32_t ts = pp.tmem + TM_S + ((uint32_t)(32 * q) << 16) + 32 * half;
+        const float c1 = p.scale * kLog2e;
+        const bool store = p.slabs == p.heads;
+        float2* s_stat = reinterpret_cast<float2*>(smem + OFF_STAT);
+        int parity = 0;
+        const float2 none = make_float2(INFINITY, 0.f);                // (a token or an agent that does not exist: its probabilities are zero)
+        const int c0 = ab * 64 + 32 * half, lim = n - c0;              // columns of this half that exist
+        float2 next = none;
+        if (BCAST && tile * kTok + r < N) next = __ldg(p.stats + (size_t)slab * N + tile * kTok + r);
+        uint32_t bw[16];                                               // 32 biases as pairs, read a tile ahead
+        auto load_bias = [&](int i) {
+            if (p.bias) wait_par(pp, BAR_BIAS, i, kTimeoutTile);
+            if (BCAST || p.bias != 2) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    uint4 w = make_uint4(0u, 0u, 0u, 0u);
+                    if (p.bias) w = *reinterpret_cast<const uint4*>(smem + OFF_BIAS + r * 128 + (((4 * half + c) ^ (r & 7)) << 4));
+                    bw[4 * c] = w.x; bw[4 * c + 1] = w.y; bw[4 * c + 2] = w.z; bw[4 * c + 3] = w.w;
+                }
+            } else {
+                const unsigned char* src = smem + OFF_BIAS + (r >> 6) * kMat + (32 * half) * 128 + (r & 7) * 2;
+                const int ch = (r & 63) >> 3;
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const uint32_t lo = *reinterpret_cast<const unsigned short*>(src + 2 * j * 128 + ((ch ^ (2 * j & 7)) << 4));
+                    const uint32_t hi = *reinterpret_cast<const unsigned short*>(src + (2 * j + 1) * 128 + ((ch ^ ((2 * j + 1) & 7)) << 4));
+                    bw[j] = lo | hi << 16;
+                }
+            }
+            // Every lane's words must be in registers before the buffer is handed back: loads that queue behind reductions were overtaken by
+            // the arrival and then by the next tile.  So the arriving lane is chosen by a vote on the words themselves.
+            uint32_t x = bw[0];
+#pragma unroll
+            for (int j = 1; j < 16; ++j) x ^= bw[j];
+            if (p.bias && lane == (__all_sync(0xffffffffu, x == 0x5bd1e995u) ? 31 : 0)) pipe_arrive(pp, BAR_BREAD);
+        };
+        load_bias(0);
+        for (int i = 0; i < count; ++i, advance()) {
+            const int b = i & 1, tok = tile * kTok + r, head = slab % p.heads;
+            const bool ok = tok < N;
+            const float2 st = next;
+            if (BCAST) {
+                const int nt = tile + 1 == p.tiles ? 0 : tile + 1, ns = slab + (nt == 0);
+                next = none;
+                if (i + 1 < count && nt * kTok + r < N) next = __ldg(p.stats + (size_t)ns * N + nt * kTok + r);
+            } else if (i == 0 || tile == 0) {                          // another slab: its statistics
+                parity ^= 1;
+                if (tid < 64) s_stat[parity * 64 + tid] = ab * 64 + tid < n ? __ldg(p.stats + (size_t)slab * n + ab * 64 + tid) : none;
+                asm volatile("bar.sync 1, %0;\n" ::"n"(kRowThreads) : "memory");
+            }
+            wait_par(pp, BAR_S, i, kTimeoutTile);
+            tc_fence_after_sync();
+            uint32_t sr[32], dr[32];
+            tmem_ld32(ts, sr);
+            tmem_ld32(ts + 64, dr);
+            tmem_ld_wait();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) pipe_arrive(pp, BAR_READ);
+            // probabilities and logit gradients
+            float2 pr[16], ds[16];
+            const float4* sst = reinterpret_cast<const float4*>(s_stat + parity * 64 + 32 * half);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                float4 v = make_float4(st.x, st.y, st.x, st.y);
+                if (!BCAST) v = sst[j];                                // (lse, D) of two agents
+                const float2 t = ffma2(unpack2<__nv_bfloat16>(bw[j]), make_float2(kLog2e, kLog2e), make_float2(-v.x, -v.z));
+                const float2 x = ffma2(make_float2(__uint_as_float(sr[2 * j]), __uint_as_float(sr[2 * j + 1])), make_float2(c1, c1), t);
+                pr[j] = make_float2(fast_exp2(x.x), fast_exp2(x.y));
+                if (BCAST && 2 * j >= lim) pr[j].x = 0.f;
+                if (BCAST && 2 * j + 1 >= lim) pr[j].y = 0.f;
+                if (!BCAST && !ok) pr[j] = make_float2(0.f, 0.f);
+                ds[j] = fmul2(pr[j], fadd2(make_float2(__uint_as_float(dr[2 * j]), __uint_as_float(dr[2 * j + 1])), make_float2(-v.y, -v.w)));
+            }
+            // as operands, once the products of the tile before have read theirs
+            if (i > 0) wait_par(pp, BAR_DONE + (b ^ 1), (i - 1) >> 1, kTimeoutTile);
+            const uint32_t prow = base + OFF_P + r * 128;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const uint32_t off = prow + (((4 * half + c) ^ (r & 7)) << 4);
+                uint32_t u[kTerms][4], v[kTerms][4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    uint32_t w[kTerms];
+                    split3(pr[4 * c + k], w);
+#pragma unroll
+                    for (int t = 0; t < kTerms; ++t) u[t][k] = w[t];
+                    split3(ds[4 * c + k], w);
+#pragma unroll
+                    for (int t = 0; t < kTerms; ++t) v[t][k] = w[t];
+                }
+#pragma unroll
+                for (int t = 0; t < kTerms; ++t) {
+                    st_shared4(off + 2 * t * kTile, u[t]);
+                    st_shared4(off + (2 * t + 1) * kTile, v[t]);
+                }
+            }
+            tc_fence_before_sync();
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) pipe_arrive(pp, BAR_P);
+            if (p.dbias && lim > 0) {
+                if (BCAST) {
+                    // [token][agent]: this warp's terms of dS, read back so that neighbouring lanes add to neighbouring agents
+                    const int t0 = tile * kTok + 32 * q;
+                    float* g = p.dbias + ((size_t)head * N + t0) * n + c0;
+                    const unsigned char* src = smem + OFF_P + kTile + 32 * q * 128;
+                    if (n % 4 == 0) {
+                        const int cc = lane >> 3;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int rr = 8 * k + (lane & 7);
+                            float2 v[4];
+#pragma unroll
+                            for (int t = kTerms - 1; t >= 0; --t) {
+                                const uint4 w = *reinterpret_cast<const uint4*>(src + 2 * t * kTile + rr * 128 + (((4 * half + cc) ^ (rr & 7)) << 4));
+                                const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) v[e] = t == kTerms - 1 ? unpack2<__nv_bfloat16>(u[e]) : fadd2(v[e], unpack2<__nv_bfloat16>(u[e]));
+                            }
+                            if (t0 + rr < N) put_dbias8(g + (size_t)rr * n + 8 * cc, reinterpret_cast<const float*>(v), lim - 8 * cc, true, store);
+                        }
+                    } else if (lane < lim) {
+                        const int left = min(32, N - t0), ch = 4 * half + (lane >> 3);
+                        for (int rr = 0; rr < left; ++rr) {
+                            const unsigned char* e = src + rr * 128 + ((ch ^ (rr & 7)) << 4) + (lane & 7) * 2;
+                            float v = 0.f;
+#pragma unroll
+                            for (int t = kTerms - 1; t >= 0; --t) v += __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(e + 2 * t * kTile));
+                            if (store) g[(size_t)rr * n + lane] = v;
+                            else atomicAdd(g + (size_t)rr * n + lane, v);
+                        }
+                    }
+                    __syncwarp();
+                } else if (ok) {
+                    float* g = p.dbias + ((size_t)head * n + c0) * N + tok;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {
+                        const float v = j & 1 ? ds[j >> 1].y : ds[j >> 1].x;
+                        if (j >= lim) break;
+                        if (store) g[(size_t)j * N] = v;
+                        else atomicAdd(g + (size_t)j * N, v);
+                    }
+                }
+            }
+            if (i + 1 < count) load_bias(i + 1);
+        }
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc<512>(pp.tmem);
+}
+
+template <bool BCAST> cudaError_t launch(const Args& a, int sm_count, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(bwd_terms_umma_kernel<BCAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e != cudaSuccess) return e;
+    const long long total = (long long)a.slabs * a.tiles, lanes = std::min<long long>(total, std::max(1, sm_count / a.blocks));
+    return launch_dependent(bwd_terms_umma_kernel<BCAST>, dim3((unsigned)(lanes * a.blocks)), kThreads, kSmemBytes, st, a);
+}
+
+}  // namespace
+
+// Faster than the mma.sync kernels on every shape of a sweep from 147 tokens x 9 agents (61 -> 57 us) to 16384 x 256.
+// (One agent or one token: a softmax over it has no gradient, which the recomputed products give exactly only where both passes agree)
+bool backward_terms_umma_eligible(int dtype, int n, int N, int d) { return dtype == kBF16 && d <= 64 && d % 8 == 0 && n > 1 && n <= 256 && N > 1; }
+
+// TMA takes a bias as it is where its rows are multiples of 16 bytes; others are copied to token rows of whole blocks of agents.
+static size_t padded_bias_bytes(int heads, int n, int N) { return ((size_t)heads * N * ((n + 63) / 64) * 128 + 255) / 256 * 256; }
+size_t backward_terms_umma_bytes(int heads, int n, int N) { return (N % 8 ? padded_bias_bytes(heads, n, N) : 0) + (n % 8 ? padded_bias_bytes(heads, n, N) : 0); }
+void backward_terms_umma_padded(int heads, int n, int N, void* ws, void** b1, void** b2) {
+    *b1 = N % 8 ? ws : nullptr;
+    *b2 = n % 8 ? static_cast<char*>(ws) + (N % 8 ? padded_bias_bytes(heads, n, N) : 0) : nullptr;
+}
+
+cudaError_t launch_backward_terms_umma(bool broadcast_stage, const BwdCall& c, const void* a_t, const void* m_t, const float2* stats, const void* padded, cudaStream_t st) {
+    Args a;
+    memset(&a, 0, sizeof(a));
+    const int N = c.H * c.W;
+    a.slabs = c.slabs; a.heads = c.heads; a.N = N; a.n = c.n; a.d = c.d; a.tiles = (N + kTok - 1) / kTok; a.blocks = (c.n + 63) / 64;
+    a.status = c.status;
+    a.stats = stats;
+    const void* bias = broadcast_stage ? c.b2 : c.b1;
+    a.bias = !bias ? 0 : broadcast_stage || padded ? 1 : 2;
+    a.outer0 = c.ws_dva; a.outer1 = c.ws_da;
+    a.row0 = broadcast_stage ? c.dq : c.dk; a.row1 = c.dv;
+    a.dbias = broadcast_stage ? c.db2 : c.db1;
+    a.scale = broadcast_stage ? c.scale2 : c.scale1;
+    if (!make_map_rows3d_u16(&a.tm_x, broadcast_stage ? c.q : c.k, c.slabs, N, kTok, true, c.d) || !make_map_rows3d_u16(&a.tm_y, broadcast_stage ? c.d_out : c.v, c.slabs, N, kTok, true, c.d) ||
+        !make_map_rows3d_u16(&a.tm_a, a_t, (uint64_t)kTerms * c.slabs, c.n, 64, true, c.d) || !make_map_rows3d_u16(&a.tm_m, m_t, (uint64_t)kTerms * c.slabs, c.n, 64, true, c.d))
+        return cudaErrorInvalidValue;
+    if (bias && !(padded ? make_map_rows3d_u16(&a.tm_b, padded, c.heads, N, kTok, true, 64 * (uint64_t)a.blocks)
+                  : broadcast_stage ? make_map_rows3d_u16(&a.tm_b, bias, c.heads, N, kTok, true, c.n) : make_map_rows3d_u16(&a.tm_b, bias, c.heads, c.n, 64, true, N)))
+        return cudaErrorInvalidValue;
+    return broadcast_stage ? launch<true>(a, c.sm_count, st) : launch<false>(a, c.sm_count, st);
+}
+
+}  // namespace aa

@@ -268,8 +268,13 @@ size_t terms_forward_bytes(int slabs, int n, int d);
 cudaError_t launch_terms_forward(const TermsForward& c, cudaStream_t st);
 // Gradient stages with fp32 operands split into 16-bit terms (any shape whose agents fit in shared memory; fp32 inputs up to 80 channels)
 bool backward_terms_eligible(int dtype, int n, int d);
-size_t backward_terms_bytes(int slabs, int n, int N, int d);
+size_t backward_terms_bytes(int dtype, int slabs, int heads, int n, int N, int d);
 cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStream_t st);
+// the gradient stages of that on the 5th-generation tensor cores (bf16 inputs of up to 64 channels)
+bool backward_terms_umma_eligible(int dtype, int n, int N, int d);
+size_t backward_terms_umma_bytes(int heads, int n, int N);                        // biases as token rows of whole blocks of 64 agents,
+void backward_terms_umma_padded(int heads, int n, int N, void* ws, void** b1, void** b2);       // or null where they are read as they are
+cudaError_t launch_backward_terms_umma(bool broadcast_stage, const BwdCall& c, const void* a_t, const void* m_t, const float2* stats, const void* padded, cudaStream_t st);
 // mixed precision, 16-bit inputs: A (16 bits, in ws_a), V_A (fp32 in ws_va, terms in ws_part), statistics (in ws_lse); clears the sums
 cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStream_t st);
 cudaError_t launch_backward_mixed_dot(int dtype, const BwdCall& c, cudaStream_t st);

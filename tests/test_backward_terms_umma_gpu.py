@@ -1,0 +1,27 @@
+"""Gradients with fp32 accuracy on tensor memory (bf16, up to 64 channels) at the edges of tiles, agent blocks and runs, against the fp64 oracle."""
+import pytest
+
+from paper_2312_08874_b200 import AA_PATH_AUTO, Workload, make_inputs
+from tests.test_backward_gpu import check, run_both
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [
+    # batch heads H   W   d  pool dtype bias
+    (1, 1, 2, 63, 32, 2, "bf16", True),       # two tokens short of a tile, few agents
+    (2, 1, 8, 16, 40, 6, "bf16", True),       # exactly one tile, agents in both halves, ragged channels
+    (1, 3, 9, 43, 64, 9, "bf16", True),       # a batch of one: bias gradients are stored; odd rows of both biases
+    (2, 2, 16, 16, 64, 16, "bf16", False),    # four full blocks of agents, two full tiles, no bias
+    (75, 2, 15, 20, 64, 9, "bf16", True),     # more units than blocks: runs that start and end inside a block of agents
+    (40, 3, 12, 12, 48, 12, "bf16", True),    # runs of several blocks of agents of two ragged tiles
+    (2, 1, 61, 83, 64, 14, "bf16", True),     # many tiles per block of agents
+]
+
+
+@pytest.mark.parametrize("case", SHAPES, ids=[f"B{c[0]}h{c[1]}_{c[2]}x{c[3]}_d{c[4]}_p{c[5]}" for c in SHAPES])
+def test_tiles_and_agent_blocks_match_oracle(case):
+    B, heads, H, W, d, pool, dtype, bias = case
+    w = Workload("terms_umma", B, heads, H, W, d, pool, dtype, bias, True, 1.0, seed=900 + H * W + pool)
+    mod, got, ref = run_both(w, make_inputs(w, bias_std=0.5, dwc_std=0.2), path=AA_PATH_AUTO)
+    check(got, ref, str(case))
+    assert mod.last_launch_count() == 8, "expected the tensor-memory gradient kernels"
