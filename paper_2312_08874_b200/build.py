@@ -23,7 +23,7 @@ NVCC_FLAGS = [
 ]
 # --use_fast_math serves the 16-bit kernels' divisions; the fp32 kernels keep IEEE division, logarithms and denormals, and exp2f
 # where they call it (the term kernels' probabilities are explicit ex2.approx, as accurate on their range), so they go without.
-PRECISE_FILES = {"attn_simt.cu", "pool.cu", "api.cu", "backward.cu", "bwd_terms.cu", "bwd_terms_umma.cu"} | {f"bwd_terms_d{d}.cu" for d in (32, 48, 64, 80, 96, 128)}
+PRECISE_FILES = {"attn_simt.cu", "pool.cu", "api.cu", "backward.cu", "bwd_terms.cu", "bwd_terms_umma.cu", "bwd_values_umma.cu"} | {f"bwd_terms_d{d}.cu" for d in (32, 48, 64, 80, 96, 128)}
 
 
 def _nvcc() -> str:

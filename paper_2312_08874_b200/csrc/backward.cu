@@ -460,7 +460,12 @@ bool plan_backward(int slabs, int n, int N, int d, int sm_count, BwdPlan* out) {
     return true;
 }
 
-int backward_launch_count(const BwdCall& c) { return (c.ws_terms ? (backward_terms_umma_eligible(c.dtype, c.n, c.H * c.W, c.d) ? 6 : 8) : c.ws_mixed ? 5 : 7) + 1 + (c.wd ? 1 : 0); }
+int backward_launch_count(const BwdCall& c) {
+    const int N = c.H * c.W;
+    const bool umma = c.ws_mixed || (c.ws_terms && backward_terms_umma_eligible(c.dtype, c.n, N, c.d));
+    const int values = umma && backward_values_eligible(c.slabs, c.n, N);
+    return (c.ws_mixed ? 5 + values : !c.ws_terms ? 7 : umma ? 6 + values + (c.n > 64) : 8) + 1 + (c.wd ? 1 : 0);
+}
 
 cudaError_t launch_backward(int dtype, const BwdCall& c, cudaStream_t st) {
     BwdArgs a;

@@ -203,8 +203,8 @@ bool backward_terms_eligible(int dtype, int n, int d) {
     const int dk = dk_of_terms(d), pitch = dk * 2 + 16, n32 = (n + 31) & ~31;
     return 6 * n32 * pitch + n32 * 8 <= 227 * 1024;
 }
-size_t backward_terms_bytes(int dtype, int slabs, int heads, int n, int N, int d) {
-    return (backward_terms_umma_eligible(dtype, n, N, d) ? backward_terms_umma_bytes(heads, n, N) : 0) + 3 * up256((size_t)slabs * n * d * 2 * 3) + up256((size_t)slabs * N * 8) + up256((size_t)slabs * n * 8);
+size_t backward_terms_bytes(int dtype, int slabs, int heads, int n, int N, int d, int sm_count) {
+    return (backward_terms_umma_eligible(dtype, n, N, d) ? backward_terms_umma_bytes(slabs, heads, n, N) + backward_values_bytes(slabs, n, N, sm_count) : 0) + 3 * up256((size_t)slabs * n * d * 2 * 3) + up256((size_t)slabs * N * 8) + up256((size_t)slabs * n * 8);
 }
 
 cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStream_t st) {
@@ -213,6 +213,8 @@ cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStrea
     const PadList pl = pad_list(c.b1, c.b2, padded, padded + rows * 128, c.heads, c.n, c.H * c.W);
     cudaError_t e = dtype == kBF16 ? pool_and_clear<__nv_bfloat16, __nv_bfloat16, 1>(c, c.ws_a, true, false, pl, st) : pool_and_clear<__half, __half, 1>(c, c.ws_a, true, false, pl, st);
     if (e != cudaSuccess) return e;
+    if (backward_values_eligible(c.slabs, c.n, c.H * c.W))
+        return launch_backward_values(dtype, false, c, c.ws_a, c.ws_part, reinterpret_cast<float2*>(c.ws_lse), padded, static_cast<char*>(c.ws_mixed) + backward_umma_bytes(c.slabs, c.heads, c.n, c.H * c.W), st);
     BwdTermArgs a;
     memset(&a, 0, sizeof(a));
     a.slabs = c.slabs; a.heads = c.heads; a.N = c.H * c.W; a.n = c.n; a.d = c.d;
@@ -250,8 +252,9 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
 #define AA_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
     const bool clear_bias = slabs != c.heads;          // (a single batch entry stores its bias gradients)
     const bool umma = backward_terms_umma_eligible(dtype, n, N, d), clear_rows = umma && n > 64;      // (blocks of 64 agents add to the rows)
-    void *pad1 = nullptr, *pad2 = nullptr;
-    if (umma) backward_terms_umma_padded(c.heads, n, N, w + 3 * terms + up256((size_t)slabs * N * 8) + up256((size_t)slabs * n * 8), &pad1, &pad2);
+    void *pad1 = nullptr, *pad2 = nullptr, *partial = nullptr;
+    char* umma_ws = w + 3 * terms + up256((size_t)slabs * N * 8) + up256((size_t)slabs * n * 8);          // padded biases, partial states of V_A
+    if (umma) backward_terms_umma_padded(c.heads, n, N, umma_ws, &pad1, &pad2, &partial);
     AA_TRY(dtype == kBF16 ? (pool_and_clear<B, B, 3>(c, a_t, clear_bias, clear_rows, pad_list(c.b1, c.b2, pad1, pad2, c.heads, n, N), st)) : dtype == kF16 ? (pool_and_clear<__half, B, 3>(c, a_t, clear_bias, clear_rows, PadList{}, st)) : (pool_and_clear<float, B, 3>(c, a_t, clear_bias, clear_rows, PadList{}, st)));
 
     BwdTermArgs a;
@@ -278,13 +281,15 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
     };
     // V_A and the statistics of the aggregation softmax
     a.x = c.k; a.y = c.v; a.bias = c.b1; a.scale = c.scale1; a.outer0 = c.ws_va; a.va_t = va_t;
-    AA_TRY(sums(kTermForward, true));
+    if (umma && backward_values_eligible(slabs, n, N)) AA_TRY(launch_backward_values(dtype, true, c, a_t, va_t, agent_stats, pad1, umma_ws + backward_terms_umma_bytes(slabs, c.heads, n, N), st));
+    else AA_TRY(sums(kTermForward, true));
     // broadcast stage: token statistics, then dV_A and its share of dA
     a.x = c.q; a.y = c.d_out; a.bias = c.b2; a.scale = a.out_scale = c.scale2; a.m_t = va_t;
-    AA_TRY(rows(kTermStats));
     if (umma) {
-        AA_TRY(launch_backward_terms_umma(true, c, a_t, va_t, tok_stats, pad2, st));
+        AA_TRY(launch_backward_terms_umma(kUmmaStats, c, a_t, va_t, tok_stats, pad2, partial, st));
+        AA_TRY(launch_backward_terms_umma(kUmmaBroadcast, c, a_t, va_t, tok_stats, pad2, nullptr, st));
     } else {
+        AA_TRY(rows(kTermStats));
         a.outer0 = c.ws_dva; a.outer1 = c.ws_da;
         AA_TRY(sums(kTermBroadcast, false));
         a.row0 = c.dq; a.dbias = c.db2;
@@ -292,7 +297,7 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
     }
     AA_TRY((launch_dependent(bwd_dot_split_kernel<B, 3>, dim3((slabs * n + 7) / 8), 256, 0, st, (const float*)c.ws_va, (const float*)c.ws_dva, agent_stats, static_cast<B*>(dva_t), slabs * n, d)));
     // aggregation stage
-    if (umma) return launch_backward_terms_umma(false, c, a_t, dva_t, agent_stats, pad1, st);
+    if (umma) return launch_backward_terms_umma(kUmmaAggregate, c, a_t, dva_t, agent_stats, pad1, nullptr, st);
     a.x = c.k; a.y = c.v; a.bias = c.b1; a.scale = c.scale1; a.out_scale = N == 1 ? 0.f : c.scale1; a.m_t = dva_t; a.dbias = c.db1;
     AA_TRY(sums(kTermAggregate, false));
     a.row0 = c.dk; a.row1 = c.dv; a.dbias = nullptr;

@@ -1,5 +1,7 @@
-// Backward pass with fp32 accuracy on the 5th-generation tensor cores: the two gradient stages for bf16 tensors of up to 64 channels.
+// Backward pass with fp32 accuracy on the 5th-generation tensor cores: the two gradient stages for bf16 tensors of up to 64 channels, and
+// the token statistics of the first.
 //
+// Statistics (X = Q, Y = dO, M = V_A):        S = X A^T, dP = Y M^T; lse[token] = log-sum-exp of S, dot[token] = its softmax . dP
 // Broadcast stage (X = Q, Y = dO, M = V_A):   S = X A^T, dP = Y M^T, P = exp(S - lse[token]), dS = P o (dP - dot[token]);
 //     dQ += scale dS A,  dV_A += P^T Y,  dA += scale dS^T X,  dB2 += dS.
 // Aggregation stage (X = K, Y = V, M = dV_A): S = X A^T, dP = Y M^T, P = exp(S - lse[agent]), dS = P o (dP - D[agent]);
@@ -12,14 +14,14 @@
 // products of the tile before run, and are split into terms once those have read theirs: 96 KB of term tiles fit once, not twice.
 //
 // Accuracy: an accumulation in tensor memory does not round to nearest, so a chain drifts with its length (see term_sum).  The small pairs
-// therefore come first, sums over tokens leave tensor memory after every tile and join in fp32 registers, and the agents' share of a
+// of S and dP therefore have accumulators of their own and those of the other products come first, sums over tokens leave tensor memory after every tile and join in fp32 registers, and the agents' share of a
 // token's gradient leaves after 64 of them.
 //
 // What bounds it: fp32 reductions, about 2 TB/s (a tile adds 32 KB of bias gradients and 32 KB per output); without them a tile takes
 // 6000 cycles of 9400, of which splitting and storing terms is 2000 beside operand reads of the tensor pipe (shared memory at 60 %).
-// 16 slabs of a 128 x 128 grid, 256 agents, biases: broadcast 328 us, aggregation 378 us; as two mma.sync kernels each (bwd_sums_kernel,
-// bwd_rows_kernel) 828 and 1010 us.  96 slabs of 14 x 14, 81 agents, whole pass: 313 -> 215 us; one slab of 40 x 23, 49 agents of 32
-// channels: 62 -> 52 us.
+// 16 slabs of a 128 x 128 grid, 256 agents, biases: broadcast 336 us, aggregation 412 us, statistics 88 + 6 us; on mma.sync (bwd_sums_kernel,
+// bwd_rows_kernel) 828, 1010 and 242 us.  192 slabs of 14 x 14, 81 agents, whole pass: 313 -> 187 us; one slab of 40 x 23, 49 agents of 32
+// channels: 62 -> 51 us.
 #include "bwd_terms_launch.cuh"
 #include "stream_common.cuh"
 
@@ -44,6 +46,7 @@ constexpr int OFF_AM = OFF_RING + kStages * kStage;          // terms of A, term
 constexpr int OFF_P = OFF_AM + 2 * kTerms * kMat;            // per term: P | dS
 constexpr int OFF_BIAS = OFF_P + 2 * kTerms * kTile;         // [128 tokens][64 agents], or twice [64 agents][64 tokens]
 constexpr int OFF_STAT = OFF_BIAS + kTile;                   // aggregation: [2][64] (lse, D)
+constexpr int OFF_EX = OFF_P;                                // statistics: [2 tiles][2 halves][128] (max, sum, dot)
 constexpr int kSmemBytes = OFF_STAT + 2 * 64 * 8 + 1024;
 static_assert(kSmemBytes <= 232448 && kSmemBytes > 116 * 1024, "one block per SM");
 
@@ -54,20 +57,25 @@ constexpr int BAR_S = 3;      //     commit           row warps: S and dP of a t
 constexpr int BAR_READ = 4;   //     row warps        issuer of S and dP: they have been read
 constexpr int BAR_P = 5;      //     row warps        issuer of the products: P and dS written
 constexpr int BAR_DONE = 6;   // [2] commit           row warps, output warps: every product of a tile (producer: the last tile of a slab)
-constexpr int BAR_OUT = 8;    // [2] output warps     issuer of the products: outputs and sums read
+constexpr int BAR_OUT = 8;    //     output warps     issuer of the products: outputs and sums read
 constexpr int BAR_DRAIN = 10; // [2] commit           each issuer, once, at its end
 constexpr int BAR_BIAS = 12;  //     tx               row warps
 constexpr int BAR_BREAD = 13; //     row warps        producer: the biases have been read
-constexpr int BAR_FREE = 14;  // [2] commit           producer: the sums of a tile, the last to read its X and Y
+constexpr int BAR_FREE = 14;  // [2] commit           producer: the sums of a tile (statistics: S and dP), the last to read its X and Y
 constexpr int kBars = 16;
 static_assert(8 * kBars <= OFF_DEAD, "mbarriers");
 constexpr int kTimeoutTile = 3, kTimeoutRole = 6;
 
-// tensor memory columns: S | dP; then twice (broadcast) sums of P^T [X | Y] and dS^T [X | Y] | dQ, (aggregation) dK | dV | sums of dS^T X
-constexpr uint32_t TM_S = 0, TM_BUF = 128, kBufCols = 192;
+// tensor memory columns: leading and small pairs of S, of dP; then (broadcast) sums of P^T [X | Y] and dS^T [X | Y] | dQ, (aggregation)
+// dK | dV | sums of dS^T X
+constexpr uint32_t TM_S = 0, TM_DP = 128, TM_BUF = 256;
+
+enum Mode { kStats, kBcast, kAgg };
 
 struct Args {
     const float2* stats;      // broadcast: (log2-sum-exp, row dot) [slabs][N]; aggregation: (log2-sum-exp, D) [slabs][n]
+    float2* tok_stats;        // statistics: the former, where one block holds all agents,
+    float4* partial;          // else (max, sum, dot) [blocks][slabs][N]
     float *outer0, *outer1;   // fp32 [slabs][n][d]: dV_A (broadcast) and dA (added)
     float *row0, *row1;       // fp32 [slabs][N][d]: dQ, or dK and dV (added where there are several blocks of agents)
     float* dbias;             // fp32 [heads][N][n] (broadcast) or [heads][n][N] (added; stored where the batch has one entry), or null
@@ -93,6 +101,24 @@ __device__ __forceinline__ void tmem_ld_16x256b_x8(uint32_t taddr, float (&r)[32
           "=f"(r[24]), "=f"(r[25]), "=f"(r[26]), "=f"(r[27]), "=f"(r[28]), "=f"(r[29]), "=f"(r[30]), "=f"(r[31])
         : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
+        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]),
+          "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15]) : "r"(taddr) : "memory");
+}
+// 32 columns of leading pairs and of small ones (64 columns on), joined
+__device__ __forceinline__ void load_joined(uint32_t taddr, float2 (&v)[16]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float a[16], b[16];
+        tmem_ld16(taddr + 16 * h, a);
+        tmem_ld16(taddr + 64 + 16 * h, b);
+        tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[8 * h + j] = fadd2(make_float2(a[2 * j], a[2 * j + 1]), make_float2(b[2 * j], b[2 * j + 1]));
+    }
+}
 __device__ __forceinline__ void st_shared4(uint32_t addr, const uint32_t (&v)[4]) {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
 }
@@ -106,8 +132,9 @@ __device__ __forceinline__ void split3(float2 v, uint32_t (&w)[kTerms]) {
     }
 }
 
-template <bool BCAST>
+template <int MODE>
 __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __grid_constant__ Args p) {
+    constexpr bool BCAST = MODE == kBcast, AGG = MODE == kAgg, STATS = MODE == kStats;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -125,7 +152,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
     pp.ph = 0u;
     if (tid == 0) {
         *pp.dead = 0;
-        for (int i = 0; i < kBars; ++i) mbar_init(pp.bars + 8 * i, i == BAR_READ || i == BAR_P || i == BAR_BREAD ? 8u : i >= BAR_OUT && i < BAR_DRAIN ? 4u : 1u);
+        for (int i = 0; i < kBars; ++i) mbar_init(pp.bars + 8 * i, i == BAR_READ || i == BAR_P || i == BAR_BREAD ? 8u : i == BAR_OUT ? 4u : 1u);
         mbar_fence_init();
     }
     if (warp == 0) tmem_alloc<512>(base + OFF_TMEM);
@@ -162,7 +189,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
                     }
                 }
                 if (i == 0 || tile == 0) {
-                    if (i > 0) wait_spin(pp, BAR_DONE + (b ^ 1), (i - 1) >> 1, kTimeoutRole);  // the last tile of the slab before
+                    if (i > 0) wait_spin(pp, (STATS ? BAR_FREE : BAR_DONE) + (b ^ 1), (i - 1) >> 1, kTimeoutRole);  // the last tile of the slab before
                     const uint32_t bam = pipe_bar(pp, BAR_AM), am = base + OFF_AM;
                     mbar_arrive_expect_tx(bam, 2 * kTerms * kMat);
                     for (int t = 0; t < kTerms; ++t) {
@@ -192,22 +219,24 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
                 for (int t = kTerms - 1; t >= 0; --t)
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        umma_ss_w(ts + 64 * which, dx + which * (kTile >> 4) + 2 * k, da + (which * kTerms + t) * (kMat >> 4) + 2 * k, id, t < kTerms - 1 || k > 0);
+                        umma_ss_w(ts + (TM_DP - TM_S) * which + (t == 0 ? 0 : 64), dx + which * (kTile >> 4) + 2 * k, da + (which * kTerms + t) * (kMat >> 4) + 2 * k, id, t == 1 || k > 0);
+            if (STATS) umma_commit_w(pipe_bar(pp, BAR_FREE + b));
             umma_commit_w(pipe_bar(pp, BAR_S));
         }
         umma_drain_w(pp, BAR_DRAIN);
         __syncwarp();
     } else if (warp == 14) {
+        if (!STATS) {
         // ------------------------------------------------------------------ products of P and dS
         const uint32_t id_out = umma_idesc(1, 128, 64, 1), id_sum = umma_idesc(1, 128, BCAST ? 128 : 64, 1) | (1u << 15);
         const uint64_t dp = umma_desc_sw128(base + OFF_P), da = umma_desc_sw128(base + OFF_AM), dps = desc_mn(base + OFF_P, kTile);
         for (int i = 0; i < count && !pipe_dead(pp); ++i) {
             const int b = i & 1;
             wait_spin(pp, BAR_P, i, kTimeoutRole);
-            if (i >= 2) wait_spin(pp, BAR_OUT + b, (i >> 1) - 1, kTimeoutRole);
+            if (i > 0) wait_spin(pp, BAR_OUT, i - 1, kTimeoutRole);
             tc_fence_after_sync();
             const uint64_t dxy = desc_mn(base + OFF_RING + b * kStage, kTile);
-            const uint32_t tb = pp.tmem + TM_BUF + kBufCols * b;
+            const uint32_t tb = pp.tmem + TM_BUF;
             // + 128 per k step of an MN-major operand (16 rows of 128 bytes)
 #pragma unroll
             for (int t = kTerms - 1; t >= 0; --t)
@@ -229,8 +258,10 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
             umma_commit_w(pipe_bar(pp, BAR_DONE + b));
         }
         umma_drain_w(pp, BAR_DRAIN + 1);
+        }
         __syncwarp();
     } else if (warp >= 8) {
+        if (!STATS) {
         // ------------------------------------------------------------------ outputs
         const int q = warp & 3, g = lane >> 2, t = lane & 3;
         const bool second = q >= 2, sums = BCAST || second;            // lanes 64 ..: rows of dS
@@ -241,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
             for (int k = 0; k < 32; ++k) acc[f][k] = 0.f;
         for (int i = 0; i < count; ++i, advance()) {
             const int b = i & 1;
-            const uint32_t rows = pp.tmem + TM_BUF + kBufCols * b + ((uint32_t)(32 * q) << 16);
+            const uint32_t rows = pp.tmem + TM_BUF + ((uint32_t)(32 * q) << 16);
             wait_par(pp, BAR_DONE + b, i >> 1, kTimeoutTile);
             tc_fence_after_sync();
             float o[32];
@@ -269,7 +300,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
                     if (which == (BCAST ? 0 : 1) && f == 1) {          // everything is in registers: hand the buffer back before the stores
                         tc_fence_before_sync();
                         __syncwarp();
-                        if (lane == 0) pipe_arrive(pp, BAR_OUT + b);
+                        if (lane == 0) pipe_arrive(pp, BAR_OUT);
                     }
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
@@ -302,6 +333,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
                     }
             }
         }
+        }
     } else {
         // ------------------------------------------------------------------ row warps
         const int q = warp & 3, half = warp >> 2, r = 32 * q + lane;
@@ -317,7 +349,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
         uint32_t bw[16];                                               // 32 biases as pairs, read a tile ahead
         auto load_bias = [&](int i) {
             if (p.bias) wait_par(pp, BAR_BIAS, i, kTimeoutTile);
-            if (BCAST || p.bias != 2) {
+            if (!AGG || p.bias != 2) {
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     uint4 w = make_uint4(0u, 0u, 0u, 0u);
@@ -350,34 +382,67 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
                 const int nt = tile + 1 == p.tiles ? 0 : tile + 1, ns = slab + (nt == 0);
                 next = none;
                 if (i + 1 < count && nt * kTok + r < N) next = __ldg(p.stats + (size_t)ns * N + nt * kTok + r);
-            } else if (i == 0 || tile == 0) {                          // another slab: its statistics
+            } else if (AGG && (i == 0 || tile == 0)) {                 // another slab: its statistics
                 parity ^= 1;
                 if (tid < 64) s_stat[parity * 64 + tid] = ab * 64 + tid < n ? __ldg(p.stats + (size_t)slab * n + ab * 64 + tid) : none;
                 asm volatile("bar.sync 1, %0;\n" ::"n"(kRowThreads) : "memory");
             }
             wait_par(pp, BAR_S, i, kTimeoutTile);
             tc_fence_after_sync();
-            uint32_t sr[32], dr[32];
-            tmem_ld32(ts, sr);
-            tmem_ld32(ts + 64, dr);
-            tmem_ld_wait();
+            float2 pr[16], ds[16];
+            load_joined(ts, pr);
+            load_joined(ts + (TM_DP - TM_S), ds);
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) pipe_arrive(pp, BAR_READ);
+            // logits in log2 units
+#pragma unroll
+            for (int j = 0; j < 16; ++j) pr[j] = ffma2(pr[j], make_float2(c1, c1), fmul2(unpack2<__nv_bfloat16>(bw[j]), make_float2(kLog2e, kLog2e)));
+            if constexpr (STATS) {
+                if (lim < 32)
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        if (2 * j >= lim) pr[j].x = -INFINITY;
+                        if (2 * j + 1 >= lim) pr[j].y = -INFINITY;
+                    }
+                float m = fmaxf(pr[0].x, pr[0].y);
+#pragma unroll
+                for (int j = 1; j < 16; ++j) m = max3(m, pr[j].x, pr[j].y);
+                const float mb = m == -INFINITY ? 0.f : -m;            // (every agent of this half may be masked)
+                float2 l2 = make_float2(0.f, 0.f), d2 = l2;
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const float2 x = fadd2(pr[j], make_float2(mb, mb));
+                    pr[j] = make_float2(fast_exp2(x.x), fast_exp2(x.y));
+                    l2 = fadd2(l2, pr[j]);
+                    d2 = ffma2(pr[j], ds[j], d2);
+                }
+                const float l = l2.x + l2.y, dot = d2.x + d2.y;
+                float4* ex = reinterpret_cast<float4*>(smem + OFF_EX) + b * 256;
+                if (half) ex[r] = make_float4(m, l, dot, 0.f);
+                asm volatile("bar.sync %0, 64;\n" ::"r"(2 + q) : "memory");
+                if (!half && ok) {
+                    const float4 o = ex[r];
+                    const float mm = fmaxf(m, o.x), f = m == -INFINITY ? 0.f : exp2f(m - mm), fo = o.x == -INFINITY ? 0.f : exp2f(o.x - mm);
+                    const float tot = fmaf(l, f, o.y * fo), dt = fmaf(dot, f, o.z * fo);
+                    if (p.blocks == 1) p.tok_stats[(size_t)slab * N + tok] = make_float2(mm + log2f(tot), dt / tot);
+                    else p.partial[((size_t)ab * p.slabs + slab) * N + tok] = make_float4(mm, tot, dt, 0.f);
+                }
+                if (i + 1 < count) load_bias(i + 1);
+                continue;
+            }
             // probabilities and logit gradients
-            float2 pr[16], ds[16];
             const float4* sst = reinterpret_cast<const float4*>(s_stat + parity * 64 + 32 * half);
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 float4 v = make_float4(st.x, st.y, st.x, st.y);
-                if (!BCAST) v = sst[j];                                // (lse, D) of two agents
-                const float2 t = ffma2(unpack2<__nv_bfloat16>(bw[j]), make_float2(kLog2e, kLog2e), make_float2(-v.x, -v.z));
-                const float2 x = ffma2(make_float2(__uint_as_float(sr[2 * j]), __uint_as_float(sr[2 * j + 1])), make_float2(c1, c1), t);
+                if (AGG) v = sst[j];                                   // (lse, D) of two agents
+                const float2 x = fadd2(pr[j], make_float2(-v.x, -v.z));
                 pr[j] = make_float2(fast_exp2(x.x), fast_exp2(x.y));
                 if (BCAST && 2 * j >= lim) pr[j].x = 0.f;
                 if (BCAST && 2 * j + 1 >= lim) pr[j].y = 0.f;
-                if (!BCAST && !ok) pr[j] = make_float2(0.f, 0.f);
-                ds[j] = fmul2(pr[j], fadd2(make_float2(__uint_as_float(dr[2 * j]), __uint_as_float(dr[2 * j + 1])), make_float2(-v.y, -v.w)));
+                if (AGG && !ok) pr[j] = make_float2(0.f, 0.f);
+                ds[j] = fmul2(pr[j], fadd2(ds[j], make_float2(-v.y, -v.w)));
             }
             // as operands, once the products of the tile before have read theirs
             if (i > 0) wait_par(pp, BAR_DONE + (b ^ 1), (i - 1) >> 1, kTimeoutTile);
@@ -458,11 +523,28 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
     if (warp == 0) tmem_dealloc<512>(pp.tmem);
 }
 
-template <bool BCAST> cudaError_t launch(const Args& a, int sm_count, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(bwd_terms_umma_kernel<BCAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+// Token statistics from those of every block of agents
+__global__ void __launch_bounds__(256) bwd_stats_merge_kernel(const float4* partial, float2* stats, long long tokens, int blocks) {
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    pdl_wait_prior();
+    pdl_release_next();
+    if (i >= tokens) return;
+    float m = -INFINITY, l = 0.f, dot = 0.f;
+    for (int k = 0; k < blocks; ++k) {
+        const float4 v = partial[k * tokens + i];
+        const float mm = fmaxf(m, v.x), f = m == -INFINITY ? 0.f : exp2f(m - mm), fo = v.x == -INFINITY ? 0.f : exp2f(v.x - mm);
+        l = fmaf(l, f, v.y * fo);
+        dot = fmaf(dot, f, v.z * fo);
+        m = mm;
+    }
+    stats[i] = make_float2(m + log2f(l), dot / l);
+}
+
+template <int MODE> cudaError_t launch(const Args& a, int sm_count, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(bwd_terms_umma_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     const long long total = (long long)a.slabs * a.tiles, lanes = std::min<long long>(total, std::max(1, sm_count / a.blocks));
-    return launch_dependent(bwd_terms_umma_kernel<BCAST>, dim3((unsigned)(lanes * a.blocks)), kThreads, kSmemBytes, st, a);
+    return launch_dependent(bwd_terms_umma_kernel<MODE>, dim3((unsigned)(lanes * a.blocks)), kThreads, kSmemBytes, st, a);
 }
 
 }  // namespace
@@ -473,32 +555,44 @@ bool backward_terms_umma_eligible(int dtype, int n, int N, int d) { return dtype
 
 // TMA takes a bias as it is where its rows are multiples of 16 bytes; others are copied to token rows of whole blocks of agents.
 static size_t padded_bias_bytes(int heads, int n, int N) { return ((size_t)heads * N * ((n + 63) / 64) * 128 + 255) / 256 * 256; }
-size_t backward_terms_umma_bytes(int heads, int n, int N) { return (N % 8 ? padded_bias_bytes(heads, n, N) : 0) + (n % 8 ? padded_bias_bytes(heads, n, N) : 0); }
-void backward_terms_umma_padded(int heads, int n, int N, void* ws, void** b1, void** b2) {
-    *b1 = N % 8 ? ws : nullptr;
-    *b2 = n % 8 ? static_cast<char*>(ws) + (N % 8 ? padded_bias_bytes(heads, n, N) : 0) : nullptr;
+size_t backward_terms_umma_bytes(int slabs, int heads, int n, int N) {
+    return (N % 8 ? padded_bias_bytes(heads, n, N) : 0) + (n % 8 ? padded_bias_bytes(heads, n, N) : 0) + (n > 64 ? (size_t)((n + 63) / 64) * slabs * N * 16 : 0);
+}
+void backward_terms_umma_padded(int heads, int n, int N, void* ws, void** b1, void** b2, void** partial) {
+    char* w = static_cast<char*>(ws);
+    *b1 = N % 8 ? w : nullptr;
+    if (N % 8) w += padded_bias_bytes(heads, n, N);
+    *b2 = n % 8 ? w : nullptr;
+    if (n % 8) w += padded_bias_bytes(heads, n, N);
+    *partial = w;
 }
 
-cudaError_t launch_backward_terms_umma(bool broadcast_stage, const BwdCall& c, const void* a_t, const void* m_t, const float2* stats, const void* padded, cudaStream_t st) {
+cudaError_t launch_backward_terms_umma(BwdTermsUmma stage, const BwdCall& c, const void* a_t, const void* m_t, float2* stats, const void* padded, void* partial, cudaStream_t st) {
     Args a;
     memset(&a, 0, sizeof(a));
     const int N = c.H * c.W;
+    const bool queries = stage != kUmmaAggregate;
     a.slabs = c.slabs; a.heads = c.heads; a.N = N; a.n = c.n; a.d = c.d; a.tiles = (N + kTok - 1) / kTok; a.blocks = (c.n + 63) / 64;
     a.status = c.status;
-    a.stats = stats;
-    const void* bias = broadcast_stage ? c.b2 : c.b1;
-    a.bias = !bias ? 0 : broadcast_stage || padded ? 1 : 2;
+    a.stats = stats; a.tok_stats = stats; a.partial = static_cast<float4*>(partial);
+    const void* bias = queries ? c.b2 : c.b1;
+    a.bias = !bias ? 0 : queries || padded ? 1 : 2;
     a.outer0 = c.ws_dva; a.outer1 = c.ws_da;
-    a.row0 = broadcast_stage ? c.dq : c.dk; a.row1 = c.dv;
-    a.dbias = broadcast_stage ? c.db2 : c.db1;
-    a.scale = broadcast_stage ? c.scale2 : c.scale1;
-    if (!make_map_rows3d_u16(&a.tm_x, broadcast_stage ? c.q : c.k, c.slabs, N, kTok, true, c.d) || !make_map_rows3d_u16(&a.tm_y, broadcast_stage ? c.d_out : c.v, c.slabs, N, kTok, true, c.d) ||
+    a.row0 = queries ? c.dq : c.dk; a.row1 = c.dv;
+    a.dbias = queries ? c.db2 : c.db1;
+    a.scale = queries ? c.scale2 : c.scale1;
+    if (!make_map_rows3d_u16(&a.tm_x, queries ? c.q : c.k, c.slabs, N, kTok, true, c.d) || !make_map_rows3d_u16(&a.tm_y, queries ? c.d_out : c.v, c.slabs, N, kTok, true, c.d) ||
         !make_map_rows3d_u16(&a.tm_a, a_t, (uint64_t)kTerms * c.slabs, c.n, 64, true, c.d) || !make_map_rows3d_u16(&a.tm_m, m_t, (uint64_t)kTerms * c.slabs, c.n, 64, true, c.d))
         return cudaErrorInvalidValue;
     if (bias && !(padded ? make_map_rows3d_u16(&a.tm_b, padded, c.heads, N, kTok, true, 64 * (uint64_t)a.blocks)
-                  : broadcast_stage ? make_map_rows3d_u16(&a.tm_b, bias, c.heads, N, kTok, true, c.n) : make_map_rows3d_u16(&a.tm_b, bias, c.heads, c.n, 64, true, N)))
+                  : queries ? make_map_rows3d_u16(&a.tm_b, bias, c.heads, N, kTok, true, c.n) : make_map_rows3d_u16(&a.tm_b, bias, c.heads, c.n, 64, true, N)))
         return cudaErrorInvalidValue;
-    return broadcast_stage ? launch<true>(a, c.sm_count, st) : launch<false>(a, c.sm_count, st);
+    if (stage == kUmmaBroadcast) return launch<kBcast>(a, c.sm_count, st);
+    if (stage == kUmmaAggregate) return launch<kAgg>(a, c.sm_count, st);
+    cudaError_t e = launch<kStats>(a, c.sm_count, st);
+    if (e != cudaSuccess || a.blocks == 1) return e;
+    const long long tokens = (long long)c.slabs * N;
+    return launch_dependent(bwd_stats_merge_kernel, dim3((unsigned)((tokens + 255) / 256)), 256, 0, st, (const float4*)a.partial, stats, tokens, a.blocks);
 }
 
 }  // namespace aa

@@ -266,15 +266,23 @@ struct TermsForward {
 bool terms_forward_eligible(int n, int d);
 size_t terms_forward_bytes(int slabs, int n, int d);
 cudaError_t launch_terms_forward(const TermsForward& c, cudaStream_t st);
+// V_A (fp32 in ws_va and as terms) and the aggregation's row statistics on tensor memory: mixed precision, or (full) three bf16 terms.
+// `padded`: B1 as token rows of whole blocks of 64 agents, read where N is no multiple of 8; `ws`: backward_values_bytes.
+bool backward_values_eligible(int slabs, int n, int N);
+size_t backward_values_bytes(int slabs, int n, int N, int sm_count);
+cudaError_t launch_backward_values(int dtype, bool full, const BwdCall& c, const void* a_t, void* va_t, float2* stats, const void* padded, void* ws, cudaStream_t st);
 // Gradient stages with fp32 operands split into 16-bit terms (any shape whose agents fit in shared memory; fp32 inputs up to 80 channels)
 bool backward_terms_eligible(int dtype, int n, int d);
-size_t backward_terms_bytes(int dtype, int slabs, int heads, int n, int N, int d);
+size_t backward_terms_bytes(int dtype, int slabs, int heads, int n, int N, int d, int sm_count);
 cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStream_t st);
 // the gradient stages of that on the 5th-generation tensor cores (bf16 inputs of up to 64 channels)
 bool backward_terms_umma_eligible(int dtype, int n, int N, int d);
-size_t backward_terms_umma_bytes(int heads, int n, int N);                        // biases as token rows of whole blocks of 64 agents,
-void backward_terms_umma_padded(int heads, int n, int N, void* ws, void** b1, void** b2);       // or null where they are read as they are
-cudaError_t launch_backward_terms_umma(bool broadcast_stage, const BwdCall& c, const void* a_t, const void* m_t, const float2* stats, const void* padded, cudaStream_t st);
+enum BwdTermsUmma { kUmmaStats, kUmmaBroadcast, kUmmaAggregate };
+// Workspace: biases as token rows of whole blocks of 64 agents (null where they are read as they are), token statistics per block of agents
+size_t backward_terms_umma_bytes(int slabs, int heads, int n, int N);
+void backward_terms_umma_padded(int heads, int n, int N, void* ws, void** b1, void** b2, void** partial);
+// `stats`: of the tokens (statistics: written), or of the agents in the aggregation stage
+cudaError_t launch_backward_terms_umma(BwdTermsUmma stage, const BwdCall& c, const void* a_t, const void* m_t, float2* stats, const void* padded, void* partial, cudaStream_t st);
 // mixed precision, 16-bit inputs: A (16 bits, in ws_a), V_A (fp32 in ws_va, terms in ws_part), statistics (in ws_lse); clears the sums
 cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStream_t st);
 cudaError_t launch_backward_mixed_dot(int dtype, const BwdCall& c, cudaStream_t st);
