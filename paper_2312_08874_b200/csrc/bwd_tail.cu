@@ -7,11 +7,15 @@
 // rows ahead.  (Four channels a thread need twice the registers for taps and sums: with the taps in shared memory and two blocks of
 // eight warps an SM 60 us; a spill of 100 bytes in the loop costs 26 us, so tokens are addressed by one offset.)  Its blocks add their
 // share of dWd to one of kFilterCopies copies, which the second kernel adds up: relative error 1.4e-7, against 5e-7 in a single copy.
+// A block goes through several batch entries of its head where that fills one wave of blocks (384 slabs of a 14 x 14 grid: 24.3 -> 20.5 us;
+// 64 slabs of 56 x 56: 43 -> 39 us).
 // bwd_pool_tail is a stream over dQ, four rows in flight.  dQ and dV are read and written in fp32, which is the bound.  64 slabs of a
-// 56 x 56 grid: 44 us (154 MB, 24 us at the copy bandwidth) and 16 us (103 MB, 16 us); one kernel for dQ and dV with all nine window
+// 56 x 56 grid: 39 us (154 MB, 24 us at the copy bandwidth) and 16 us (103 MB, 16 us); one kernel for dQ and dV with all nine window
 // loads of a token, and one for dWd, took 74 and 31.
 #include "common.cuh"
 #include "kernels.h"
+
+#include <algorithm>
 
 namespace aa {
 
@@ -21,7 +25,7 @@ struct TailArgs {
     const void *v, *go, *wd;
     const float* da;
     float *dq, *dv, *dwd, *dwd_copies;
-    int heads, H, W, d, n, p, strip, strips, passes;
+    int heads, H, W, d, n, p, strip, strips, passes, batch;
 };
 
 // Two channels of a token as loaded (zeros where there is no token; volatile: left to itself the compiler gathers the loads of several
@@ -67,6 +71,7 @@ __device__ __forceinline__ Windows windows_of(int i, int L, int p) {
 
 constexpr int kAxis = 512;         // rows whose windows are kept in shared memory
 constexpr int kThreadsQ = 256, kThreadsV = 128;
+constexpr int kStartV = 8;         // the start and the end of a bwd_conv_tail block cost about so many rows
 
 // Columns of a slab's strips, one after the other: a block takes `passes` times `cols` of them.
 struct Column {
@@ -146,12 +151,12 @@ __global__ void __launch_bounds__(kThreadsQ, 4) bwd_pool_tail_kernel(const TailA
 template <typename T, bool DWD>
 __global__ void __launch_bounds__(kThreadsV, sizeof(T) == 4 ? 4 : 5) bwd_conv_tail_kernel(const TailArgs a) {
     __shared__ float2 red[DWD ? kThreadsV : 1][9];
-    const int d = a.d, H = a.H, W = a.W, slab = blockIdx.y;
+    const int d = a.d, H = a.H, W = a.W, head = blockIdx.y % a.heads;
     const int groups = d >> 1, cols = kThreadsV / groups;         // d <= 128: at least two columns at once
     const int cg = threadIdx.x % groups, cl = threadIdx.x / groups;
     float2 tap[9], acc[DWD ? 9 : 1];
     {
-        const T* w = static_cast<const T*>(a.wd) + ((size_t)(slab % a.heads) * d + 2 * cg) * 9;
+        const T* w = static_cast<const T*>(a.wd) + ((size_t)head * d + 2 * cg) * 9;
 #pragma unroll
         for (int k = 0; k < 9; ++k) tap[k] = make_float2(Elem<T>::to_f32(w[k]), Elem<T>::to_f32(w[9 + k]));
     }
@@ -162,7 +167,10 @@ __global__ void __launch_bounds__(kThreadsV, sizeof(T) == 4 ? 4 : 5) bwd_conv_ta
         for (int k = 0; k < 9; ++k) acc[k] = make_float2(0.f, 0.f);
     const int first = blockIdx.x * a.passes * cols, last = min(first + a.passes * cols, a.strips * W);
     const size_t pitch = (size_t)W * d;
-    if (cl < cols)
+    // its columns in every so many batch entries of one head: the filter and its gradient's sums stay in registers
+    for (int e = blockIdx.y / a.heads, step = gridDim.y / a.heads; e < a.batch; e += step) {
+        const int slab = e * a.heads + head;
+        if (cl < cols)
         for (int i = first + cl; i < last; i += cols) {
             const Column c = column_of(a, i);
             const bool left = c.x > 0, right = c.x + 1 < W;
@@ -209,12 +217,13 @@ __global__ void __launch_bounds__(kThreadsV, sizeof(T) == 4 ? 4 : 5) bwd_conv_ta
                     off += pitch;
                 }
         }
+    }
     if (DWD) {
 #pragma unroll
         for (int k = 0; k < 9; ++k) red[threadIdx.x][k] = acc[k];
         __syncthreads();
         // one of several copies: a sum of all blocks' shares in one word would round as often as there are blocks
-        float* copy = a.dwd_copies + ((size_t)((blockIdx.x + blockIdx.y) % kFilterCopies) * a.heads + slab % a.heads) * d * 9;
+        float* copy = a.dwd_copies + ((size_t)((blockIdx.x + blockIdx.y) % kFilterCopies) * a.heads + head) * d * 9;
         for (int o = threadIdx.x; o < d * 9; o += kThreadsV) {    // o = channel * 9 + tap
             const int c = o / 9, k = o - c * 9;
             float s = 0.f;
@@ -227,30 +236,35 @@ __global__ void __launch_bounds__(kThreadsV, sizeof(T) == 4 ? 4 : 5) bwd_conv_ta
     }
 }
 
-// Strips of rows, and passes of a block over `cols` columns: the least rows that a slot (a resident block) goes through, when a strip
-// costs `halo` rows more than it has and the start of a block `start` rows.
-dim3 plan_strips(TailArgs* a, int slabs, int cols, int slots, int halo, int start) {
+// Strips of rows, passes of a block over `cols` columns, and (`most` > 1) batch entries of a block: the least rows that a slot (a resident
+// block) goes through, when a strip costs `halo` rows more than it has and a block `start` rows.
+dim3 plan_strips(TailArgs* a, int most, int cols, int slots, int halo, int start) {
     long long best = 0;
-    int blocks = 1;
+    int blocks = 1, groups = a->batch;
     for (int strips = 1; strips <= 32 && (strips == 1 || strips * 4 <= a->H); ++strips) {
         const int rows = (a->H + strips - 1) / strips, used = (a->H + rows - 1) / rows, total = (int)(((long long)used * a->W + cols - 1) / cols);
         for (int passes = 1; passes <= 8 && passes <= total; ++passes) {
             const int per_slab = (total + passes - 1) / passes;
-            const long long cost = ((long long)slabs * per_slab + slots - 1) / slots * (passes * (rows + halo) + start);
-            if (best == 0 || cost < best) { best = cost; blocks = per_slab; a->strip = rows; a->strips = used; a->passes = passes; }
+            // batch entries: one each, or as many as leave a single wave of blocks
+            const int room = (int)std::max<long long>(1, slots / ((long long)per_slab * a->heads)), each = std::min(most, (a->batch + room - 1) / room);
+            for (int entries : {1, each}) {
+                const int gy = (a->batch + entries - 1) / entries;
+                const long long cost = ((long long)gy * a->heads * per_slab + slots - 1) / slots * ((long long)entries * passes * (rows + halo) + start);
+                if (best == 0 || cost < best) { best = cost; blocks = per_slab; groups = gy; a->strip = rows; a->strips = used; a->passes = passes; }
+            }
         }
     }
-    return dim3(blocks, slabs);
+    return dim3(blocks, groups * a->heads);
 }
 
-template <typename T> cudaError_t launch_tail(TailArgs a, int slabs, int sm_count, cudaStream_t st) {
+template <typename T> cudaError_t launch_tail(TailArgs a, int sm_count, cudaStream_t st) {
     // dV first: the stage before has just written it
     if (a.wd) {
-        const dim3 grid = plan_strips(&a, slabs, kThreadsV / (a.d / 2), (sizeof(T) == 4 ? 4 : 5) * sm_count, 2, 4);
+        const dim3 grid = plan_strips(&a, a.batch, kThreadsV / (a.d / 2), (sizeof(T) == 4 ? 4 : 5) * sm_count, 2, kStartV);
         const cudaError_t e = launch_dependent(a.dwd ? bwd_conv_tail_kernel<T, true> : bwd_conv_tail_kernel<T, false>, grid, kThreadsV, 0, st, a);
         if (e != cudaSuccess) return e;
     }
-    dim3 grid = plan_strips(&a, slabs, kThreadsQ / (a.d / 4), 4 * sm_count, 0, 4);
+    dim3 grid = plan_strips(&a, 1, kThreadsQ / (a.d / 4), 4 * sm_count, 0, 4);
     if (a.dwd) ++grid.x;
     return launch_dependent(bwd_pool_tail_kernel, grid, kThreadsQ, 0, st, a);
 }
@@ -260,11 +274,11 @@ template <typename T> cudaError_t launch_tail(TailArgs a, int slabs, int sm_coun
 cudaError_t launch_backward_tail(int dtype, const BwdCall& c, cudaStream_t st) {
     TailArgs a;
     a.v = c.v; a.go = c.d_out; a.wd = c.wd; a.da = c.ws_da; a.dq = c.dq; a.dv = c.dv; a.dwd = c.dwd; a.dwd_copies = c.ws_dwd;
-    a.heads = c.heads; a.H = c.H; a.W = c.W; a.d = c.d; a.n = c.n; a.p = c.p; a.strip = a.strips = a.passes = 0;
+    a.heads = c.heads; a.H = c.H; a.W = c.W; a.d = c.d; a.n = c.n; a.p = c.p; a.strip = a.strips = a.passes = 0; a.batch = c.slabs / c.heads;
     switch (dtype) {
-        case kF32:  return launch_tail<float>(a, c.slabs, c.sm_count, st);
-        case kBF16: return launch_tail<__nv_bfloat16>(a, c.slabs, c.sm_count, st);
-        default:    return launch_tail<__half>(a, c.slabs, c.sm_count, st);
+        case kF32:  return launch_tail<float>(a, c.sm_count, st);
+        case kBF16: return launch_tail<__nv_bfloat16>(a, c.sm_count, st);
+        default:    return launch_tail<__half>(a, c.sm_count, st);
     }
 }
 
