@@ -13,7 +13,7 @@
 namespace aa {
 
 enum BwdSums { kSumsForward, kSumsBroadcast, kSumsAggregate };
-enum BwdRows { kRowsStats, kRowsQuery, kRowsKeyValue, kRowsOut };
+enum BwdRows { kRowsStats, kRowsQuery, kRowsKeyValue, kRowsOut, kRowsOutSplit };       // (split: two warps per 16 tokens, half of the agents each)
 
 // term pairs of a product: i of NA, j of NB with i + j < max(NA, NB)
 template <int NA, int NB> struct TermPairs {
@@ -515,12 +515,15 @@ template <int DK, int TA, int TM> struct RowsShape {
     static constexpr int kPitch = DK * 2 + 16;
     __host__ __device__ static constexpr int smem(int n) { return (TA + TM) * ((n + 31) & ~31) * kPitch + ((n + 31) & ~31) * 8; }      // (rows out: 9 DK filter words and DK sums)
     __host__ __device__ static constexpr int smem_out(int n) { return (TA + TM) * ((n + 31) & ~31) * kPitch + 10 * DK * 4; }
+    // rows out, split: the 8-channel tiles up to kCut are finished by the first warp of a pair; per warp, what it gives away and its sums
+    static constexpr int kCut = (DK / 16 + 1) / 2 * 2, kGive = (kCut * 4 + 4) * 128;
+    __host__ __device__ static constexpr int smem_split(int n) { return smem_out(n) + 8 * kGive; }
 };
 
 template <typename T, typename E, int DK, int NX, int TA, int TM, int TP, int MODE>
 __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant__ BwdTermArgs p) {
     constexpr int PITCH = DK * 2 + 16, KS = DK / 16, NT = DK / 8;
-    constexpr bool kRaw = sizeof(T) == 4;
+    constexpr bool kRaw = sizeof(T) == 4, kOut = MODE == kRowsOut || MODE == kRowsOutSplit;
     extern __shared__ __align__(128) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const int slab = blockIdx.y, head = slab % p.heads, n32 = (p.n + 31) & ~31;
@@ -542,14 +545,14 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
             const size_t off = ok ? ((size_t)slab * p.n + r) * p.d + ch * 8 : 0;
             cp_async16s(sm + (m * n32 + col_to_row(r)) * PITCH + ch * 16, src + off, ok ? 16 : 0);
         }
-        if (MODE == kRowsOut && p.wd)
+        if (kOut && p.wd)
             for (int i = threadIdx.x; i < p.d * 9; i += 256) wt_s[(i % 9) * DK + i / 9] = Elem<T>::to_f32(static_cast<const T*>(p.wd)[(size_t)head * p.d * 9 + i]);
         if (MODE == kRowsKeyValue)
             for (int i = threadIdx.x; i < n32; i += 256)                  // (no such agent: its probabilities are zero)
                 st_s[i] = i < p.n ? p.agent_stats[(size_t)slab * p.n + i] : make_float2(INFINITY, 0.f);
         cp_async_commit();
         cp_async_wait<0>();
-        if constexpr (MODE == kRowsOut) {              // a NaN among the last terms of V_A (of those that this thread has copied)
+        if constexpr (kOut) {              // a NaN among the last terms of V_A (of those that this thread has copied)
             float2 z = make_float2(0.f, 0.f);
             const int last = (TA + TM - 1) * n32;
             for (int e = (threadIdx.x - last * chunks) & 255; e < n32 * chunks; e += 256) {
@@ -574,7 +577,11 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
     const T* bias_end = p.bias ? static_cast<const T*>(p.bias) + (size_t)p.heads * p.n * p.N : nullptr;
     const float c1 = p.scale * kLog2e;
     const uint32_t koff = sm + key_lane_offset<DK>(lane), voff = sm + val_lane_offset<DK>(lane);
-    for (int tok = t0 + warp * 16; tok < t1; tok += 128) {
+    // Few tokens for the chip: two warps share 16 of them, the blocks of 32 agents in turn, and meet over the running softmax states
+    constexpr bool split = MODE == kRowsOutSplit;
+    const int side = split ? warp >> 2 : 0, group = split ? warp & 3 : warp;
+    constexpr int CUT = RowsShape<DK, TA, TM>::kCut;
+    for (int tok = t0 + group * 16; tok < t1; tok += split ? 64 : 128) {
         // operand rows: as terms, or (fp32) as they are, split when they are used: three terms of both do not fit in registers
         uint32_t xf[kRaw ? 1 : NX][kRaw ? 1 : KS][4], yf[kRaw ? 1 : NX][kRaw ? 1 : KS][4];
         float2 xr[kRaw ? KS : 1][4], yr[kRaw ? KS : 1][4];
@@ -588,11 +595,11 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                     const bool in = ks * 16 + k * 8 + 2 * t < p.d;
                     if constexpr (NX == 1) {
                         xf[0][ks][k * 2 + h] = in ? __ldg(reinterpret_cast<const uint32_t*>(x + off + ks * 16 + k * 8)) : 0u;
-                        yf[0][ks][k * 2 + h] = in && MODE != kRowsOut ? __ldg(reinterpret_cast<const uint32_t*>(y + off + ks * 16 + k * 8)) : 0u;
+                        yf[0][ks][k * 2 + h] = in && !kOut ? __ldg(reinterpret_cast<const uint32_t*>(y + off + ks * 16 + k * 8)) : 0u;
                     } else {
                         float2 fx = make_float2(0.f, 0.f), fy = fx;
                         if (in) fx = load_pair<T>(x + off + ks * 16 + k * 8);
-                        if (in && MODE != kRowsOut) fy = load_pair<T>(y + off + ks * 16 + k * 8);
+                        if (in && !kOut) fy = load_pair<T>(y + off + ks * 16 + k * 8);
                         if constexpr (kRaw) {
                             xr[ks][k * 2 + h] = fx;
                             yr[ks][k * 2 + h] = fy;
@@ -619,7 +626,7 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
 #pragma unroll
             for (int h = 0; h < 2; ++h) rs[h] = p.tok_stats[(size_t)slab * p.N + min(tok + h * 8 + g, t1 - 1)];
 #pragma unroll 1
-        for (int blk = 0; blk < n32; blk += 32) {
+        for (int blk = side * 32; blk < n32; blk += split ? 64 : 32) {
             float bs[2][8];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -647,7 +654,7 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                         split_pair<E, NX>(xr[ks][q].x, xr[ks][q].y, w);
 #pragma unroll
                         for (int k = 0; k < NX; ++k) xt[k][q] = w[k];
-                        if (MODE != kRowsOut) split_pair<E, NX>(yr[ks][q].x, yr[ks][q].y, w);
+                        if (!kOut) split_pair<E, NX>(yr[ks][q].x, yr[ks][q].y, w);
 #pragma unroll
                         for (int k = 0; k < NX; ++k) yt[k][q] = w[k];
                     } else {
@@ -664,7 +671,7 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                         if (i == 0) mma_two<E>(s[2 * j2], s[2 * j2 + 1], xt[0], b, ks == 0);
                         mma_low<E, NX, TA>(sl[2 * j2], sl[2 * j2 + 1], xt, b, i, ks == 0 && i == (NX == 1));
                     }
-                    if (MODE != kRowsOut)
+                    if (!kOut)
 #pragma unroll
                         for (int i = 0; i < TM; ++i) {
                             uint32_t b[4];
@@ -677,7 +684,7 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 add4(s[j], sl[j]);
-                if (MODE != kRowsOut) add4(dp[j], dl[j]);
+                if (!kOut) add4(dp[j], dl[j]);
             }
             const int left = p.n - blk - 8 * t;
             if constexpr (MODE == kRowsStats) {
@@ -701,7 +708,7 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                         rd[h] = fmaf(e, dp[i >> 1][2 * h + (i & 1)], rd[h]);
                     }
                 }
-            } else if constexpr (MODE == kRowsOut) {
+            } else if constexpr (kOut) {
                 uint32_t pt[2][TP][4];
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -776,11 +783,38 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                 }
             }
         }
-        if constexpr (MODE == kRowsOut) {
+        if constexpr (kOut) {
             // neighbouring threads swap halves of two 8-channel tiles: then a thread has four channels of tile j + (t & 1) of both rows,
             // and the eighteen 16-byte loads of its two depthwise windows are in flight at once
             const bool odd = t & 1;
             bool in[2][9];
+            if (split) {                               // (the partner's elements belong to the same lane)
+                float* mine = reinterpret_cast<float*>(smem + RowsShape<DK, TA, TM>::smem_out(p.n) + warp * RowsShape<DK, TA, TM>::kGive) + lane;
+                const float* other = reinterpret_cast<const float*>(smem + RowsShape<DK, TA, TM>::smem_out(p.n) + (warp ^ 4) * RowsShape<DK, TA, TM>::kGive) + lane;
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+                    if ((j >= CUT) != side)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) mine[((j >= CUT ? j - CUT : j) * 4 + e) * 32] = o0[j][e];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    mine[(CUT * 4 + h) * 32] = m[h];
+                    mine[(CUT * 4 + 2 + h) * 32] = l[h];
+                }
+                asm volatile("bar.sync %0, 64;\n" ::"r"(1 + group) : "memory");
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float om = other[(CUT * 4 + h) * 32], ol = other[(CUT * 4 + 2 + h) * 32], mm = fmaxf(m[h], om), base = mm == -INFINITY ? 0.f : mm;
+                    const float f = exp2f(m[h] - base), fo = exp2f(om - base);
+                    l[h] = l[h] * f + ol * fo;
+#pragma unroll
+                    for (int j = 0; j < NT; ++j)
+                        if ((j >= CUT) == side)
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) o0[j][2 * h + e] = o0[j][2 * h + e] * f + other[((j >= CUT ? j - CUT : j) * 4 + 2 * h + e) * 32] * fo;
+                }
+                asm volatile("bar.sync %0, 64;\n" ::"r"(1 + group) : "memory");
+            }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const float inv = 1.f / quad_sum(l[h]);
@@ -798,6 +832,7 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
             }
 #pragma unroll
             for (int j = 0; j < NT; j += 2) {
+                if (split && (j >= CUT) != side) continue;
                 const int ch = 8 * (j + (t & 1)) + 4 * (t >> 1);
                 const bool live = ch < p.d;
                 float4 u[2][9];

@@ -51,15 +51,17 @@ template <typename T, typename C, int DK, int MODE> cudaError_t bwd_sums(const B
 template <typename T, int DK, int MODE> cudaError_t bwd_rows(const BwdTermArgs& a, const BwdTermLaunch& l) {
     using C = TermsFull<T>;
     static std::atomic<unsigned long long> done;
-    return bwd_launch(bwd_rows_kernel<T, typename C::E, DK, C::NX, C::TA, C::TM, C::TP, MODE>, done, a, l, 256, MODE == kRowsOut ? RowsShape<DK, C::TA, C::TM>::smem_out(a.n) : RowsShape<DK, C::TA, C::TM>::smem(a.n));
+    return bwd_launch(bwd_rows_kernel<T, typename C::E, DK, C::NX, C::TA, C::TM, C::TP, MODE>, done, a, l, 256, MODE == kRowsOutSplit ? RowsShape<DK, C::TA, C::TM>::smem_split(a.n) : MODE == kRowsOut ? RowsShape<DK, C::TA, C::TM>::smem_out(a.n) : RowsShape<DK, C::TA, C::TM>::smem(a.n));
 }
 
-enum BwdTermStage { kTermForward, kTermStats, kTermBroadcast, kTermAggregate, kTermKeyValue, kTermQuery, kTermOut };
+enum BwdTermStage { kTermForward, kTermStats, kTermBroadcast, kTermAggregate, kTermKeyValue, kTermQuery, kTermOut, kTermOutSplit };
 constexpr int kTermGradientsF32 = 80;      // fp32 inputs: the gradient kernels' accumulators and operand rows fit in registers up to here
 template <typename T, int DK> cudaError_t bwd_terms_stage(int stage, const BwdTermArgs& a, const BwdTermLaunch& l) {
     if (stage == kTermForward) return bwd_sums<T, TermsFull<T>, DK, kSumsForward>(a, l);
-    if constexpr (sizeof(T) == 4)
+    if constexpr (sizeof(T) == 4) {
         if (stage == kTermOut) return bwd_rows<T, DK, kRowsOut>(a, l);
+        if (stage == kTermOutSplit) return bwd_rows<T, DK, kRowsOutSplit>(a, l);
+    }
     if constexpr (sizeof(T) == 2 || DK <= kTermGradientsF32) {
         switch (stage) {
             case kTermStats:     return bwd_rows<T, DK, kRowsStats>(a, l);
