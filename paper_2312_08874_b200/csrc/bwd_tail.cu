@@ -16,6 +16,7 @@
 #include "kernels.h"
 
 #include <algorithm>
+#include <cmath>
 
 namespace aa {
 
@@ -239,18 +240,26 @@ __global__ void __launch_bounds__(kThreadsV, sizeof(T) == 4 ? 4 : 5) bwd_conv_ta
 // Strips of rows, passes of a block over `cols` columns, and (`most` > 1) batch entries of a block: the least rows that a slot (a resident
 // block) goes through, when a strip costs `halo` rows more than it has and a block `start` rows.
 dim3 plan_strips(TailArgs* a, int most, int cols, int slots, int halo, int start) {
-    long long best = 0;
-    int blocks = 1, groups = a->batch;
+    double best = 0;
+    int blocks = 1, groups = a->batch, tried = 0;
     for (int strips = 1; strips <= 32 && (strips == 1 || strips * 4 <= a->H); ++strips) {
-        const int rows = (a->H + strips - 1) / strips, used = (a->H + rows - 1) / rows, total = (int)(((long long)used * a->W + cols - 1) / cols);
-        for (int passes = 1; passes <= 8 && passes <= total; ++passes) {
-            const int per_slab = (total + passes - 1) / passes;
-            // batch entries: one each, or as many as leave a single wave of blocks
-            const int room = (int)std::max<long long>(1, slots / ((long long)per_slab * a->heads)), each = std::min(most, (a->batch + room - 1) / room);
-            for (int entries : {1, each}) {
-                const int gy = (a->batch + entries - 1) / entries;
-                const long long cost = ((long long)gy * a->heads * per_slab + slots - 1) / slots * ((long long)entries * passes * (rows + halo) + start);
+        const int rows = (a->H + strips - 1) / strips;
+        if (rows == tried) continue;                              // (this runs on every call: no plan twice, few divisions)
+        tried = rows;
+        const int used = (a->H + rows - 1) / rows;
+        const long long columns = ((long long)used * a->W + cols - 1) / cols;
+        for (int passes = 1; passes <= 8 && passes <= columns; ++passes) {
+            const int per_slab = (int)((columns + passes - 1) / passes);
+            auto consider = [&](int entries, int gy) {
+                const double cost = ceil((double)gy * a->heads * per_slab / slots) * ((double)entries * passes * (rows + halo) + start);
                 if (best == 0 || cost < best) { best = cost; blocks = per_slab; groups = gy; a->strip = rows; a->strips = used; a->passes = passes; }
+            };
+            consider(1, a->batch);
+            // or as many batch entries as leave a single wave of blocks
+            const double wave = (double)per_slab * a->heads;
+            if (most > 1 && wave * a->batch > slots) {
+                const int room = wave >= slots ? 1 : (int)(slots / wave), entries = std::min(most, (a->batch + room - 1) / room);
+                consider(entries, (a->batch + entries - 1) / entries);
             }
         }
     }

@@ -541,7 +541,8 @@ __global__ void __launch_bounds__(256) bwd_stats_merge_kernel(const float4* part
 }
 
 template <int MODE> cudaError_t launch(const Args& a, int sm_count, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(bwd_terms_umma_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    static std::atomic<unsigned long long> done;
+    cudaError_t e = allow_smem(bwd_terms_umma_kernel<MODE>, done, kSmemBytes);
     if (e != cudaSuccess) return e;
     const long long total = (long long)a.slabs * a.tiles, lanes = std::min<long long>(total, std::max(1, sm_count / a.blocks));
     return launch_dependent(bwd_terms_umma_kernel<MODE>, dim3((unsigned)(lanes * a.blocks)), kThreads, kSmemBytes, st, a);
@@ -581,11 +582,11 @@ cudaError_t launch_backward_terms_umma(BwdTermsUmma stage, const BwdCall& c, con
     a.row0 = queries ? c.dq : c.dk; a.row1 = c.dv;
     a.dbias = queries ? c.db2 : c.db1;
     a.scale = queries ? c.scale2 : c.scale1;
-    if (!make_map_rows3d_u16(&a.tm_x, queries ? c.q : c.k, c.slabs, N, kTok, true, c.d) || !make_map_rows3d_u16(&a.tm_y, queries ? c.d_out : c.v, c.slabs, N, kTok, true, c.d) ||
-        !make_map_rows3d_u16(&a.tm_a, a_t, (uint64_t)kTerms * c.slabs, c.n, 64, true, c.d) || !make_map_rows3d_u16(&a.tm_m, m_t, (uint64_t)kTerms * c.slabs, c.n, 64, true, c.d))
+    if (!make_map_3d_u16(&a.tm_x, queries ? c.q : c.k, c.slabs, N, c.d, kTok) || !make_map_3d_u16(&a.tm_y, queries ? c.d_out : c.v, c.slabs, N, c.d, kTok) ||
+        !make_map_3d_u16(&a.tm_a, a_t, (uint64_t)kTerms * c.slabs, c.n, c.d, 64) || !make_map_3d_u16(&a.tm_m, m_t, (uint64_t)kTerms * c.slabs, c.n, c.d, 64))
         return cudaErrorInvalidValue;
-    if (bias && !(padded ? make_map_rows3d_u16(&a.tm_b, padded, c.heads, N, kTok, true, 64 * (uint64_t)a.blocks)
-                  : queries ? make_map_rows3d_u16(&a.tm_b, bias, c.heads, N, kTok, true, c.n) : make_map_rows3d_u16(&a.tm_b, bias, c.heads, c.n, 64, true, N)))
+    if (bias && !(padded ? make_map_3d_u16(&a.tm_b, padded, c.heads, N, 64 * (uint64_t)a.blocks, kTok)
+                  : queries ? make_map_3d_u16(&a.tm_b, bias, c.heads, N, c.n, kTok) : make_map_3d_u16(&a.tm_b, bias, c.heads, c.n, N, 64)))
         return cudaErrorInvalidValue;
     if (stage == kUmmaBroadcast) return launch<kBcast>(a, c.sm_count, st);
     if (stage == kUmmaAggregate) return launch<kAgg>(a, c.sm_count, st);

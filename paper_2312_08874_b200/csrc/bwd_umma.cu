@@ -402,7 +402,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_umma_kernel(const __grid_cons
 }
 
 template <typename T, bool BCAST> cudaError_t launch(const UmmaArgs& a, int sm_count, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(bwd_umma_kernel<T, BCAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    static std::atomic<unsigned long long> done;
+    cudaError_t e = allow_smem(bwd_umma_kernel<T, BCAST>, done, kSmemBytes);
     if (e != cudaSuccess) return e;
     const long long total = (long long)a.slabs * a.tiles;
     return launch_dependent(bwd_umma_kernel<T, BCAST>, dim3((unsigned)(total < sm_count ? total : sm_count)), kThreads, kSmemBytes, st, a);

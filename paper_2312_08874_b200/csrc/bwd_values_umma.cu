@@ -425,7 +425,8 @@ Plan plan(int slabs, int n, int N, int sm_count) {
 }
 
 template <typename T, int TA, int TP, bool STACK> cudaError_t launch(const Args& a, int grid, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(bwd_values_umma_kernel<T, TA, TP, STACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem<TA>);
+    static std::atomic<unsigned long long> done;
+    cudaError_t e = allow_smem(bwd_values_umma_kernel<T, TA, TP, STACK>, done, kSmem<TA>);
     if (e != cudaSuccess) return e;
     return launch_dependent(bwd_values_umma_kernel<T, TA, TP, STACK>, dim3(grid), kThreads, kSmem<TA>, st, a);
 }
@@ -458,10 +459,10 @@ cudaError_t launch_backward_values(int dtype, bool full, const BwdCall& c, const
     a.scale = c.scale1;
     const bool rows = N % 8 == 0;                       // (TMA takes B1 as it is)
     a.bias = !c.b1 ? 0 : rows ? 2 : 1;
-    if (!make_map_rows3d_u16(&a.tm_k, c.k, c.slabs, N, kTok, true, c.d) || !make_map_rows3d_u16(&a.tm_v, c.v, c.slabs, N, kTok, true, c.d) ||
-        !make_map_rows3d_u16(&a.tm_a, a_t, (full ? 3 : 1) * (uint64_t)c.slabs, c.n, 64, true, c.d))
+    if (!make_map_3d_u16(&a.tm_k, c.k, c.slabs, N, c.d, kTok) || !make_map_3d_u16(&a.tm_v, c.v, c.slabs, N, c.d, kTok) ||
+        !make_map_3d_u16(&a.tm_a, a_t, (full ? 3 : 1) * (uint64_t)c.slabs, c.n, c.d, 64))
         return cudaErrorInvalidValue;
-    if (c.b1 && !(rows ? make_map_rows3d_u16(&a.tm_b, c.b1, c.heads, c.n, v.stack ? 64 : 128, true, N) : make_map_rows3d_u16(&a.tm_b, padded, c.heads, N, kTok, true, (c.n + 63) / 64 * 64)))
+    if (c.b1 && !(rows ? make_map_3d_u16(&a.tm_b, c.b1, c.heads, c.n, N, v.stack ? 64 : 128) : make_map_3d_u16(&a.tm_b, padded, c.heads, N, (c.n + 63) / 64 * 64, kTok)))
         return cudaErrorInvalidValue;
     using B = __nv_bfloat16;
     const int grid = v.lanes * v.blocks;

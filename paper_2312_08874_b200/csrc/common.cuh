@@ -1,6 +1,7 @@
 // Shared device helpers of the agent-attention kernels (sm_100a).
 #pragma once
 
+#include <atomic>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -153,6 +154,17 @@ __device__ __forceinline__ void red_add2(float* p, float a, float b) {
 // programmatic dependent launch: wait for the stream's previous kernel / let the next one start
 __device__ __forceinline__ void pdl_wait_prior() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_release_next() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+// Shared memory limit of a kernel, set once per device (the call costs more than a microsecond of the host's time)
+template <typename K> inline cudaError_t allow_smem(K kern, std::atomic<unsigned long long>& done, int bytes) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
+}
 // Launch that may start while its predecessor in the stream drains; the kernel calls pdl_wait_prior before it touches memory.
 template <typename... P, typename... Q> inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, Q&&... q) {
     cudaLaunchConfig_t cfg = {};

@@ -132,14 +132,14 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
-// Host: map of a dense [z][rows][d] tensor of 16-bit elements (d a multiple of 8; what lies outside reads zero) with a
+// Host: map of a [z][rows][64] tensor of 16-bit elements (row pitch 128 bytes, z pitch rows * 128 bytes) with a
 // box of 64 x box_rows x 1, 128-byte swizzle or none.
-inline bool make_map_rows3d_u16(CUtensorMap* out, const void* base, uint64_t zs, uint64_t rows, uint32_t box_rows, bool swizzle, uint64_t d = 64) {
+inline bool make_map_rows3d_u16(CUtensorMap* out, const void* base, uint64_t zs, uint64_t rows, uint32_t box_rows, bool swizzle) {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
     if ((reinterpret_cast<uintptr_t>(base) & 15u) || box_rows > 256 || box_rows < 1) return false;
-    const cuuint64_t dims[3] = {d, rows, zs};
-    const cuuint64_t strides[2] = {2 * d, rows * 2 * d};
+    const cuuint64_t dims[3] = {64, rows, zs};
+    const cuuint64_t strides[2] = {128, rows * 128};
     const cuuint32_t box[3] = {64, box_rows, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     return fn(out, CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, const_cast<void*>(base), dims, strides, box, estr,

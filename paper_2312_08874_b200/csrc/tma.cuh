@@ -116,6 +116,20 @@ inline bool make_map_2d_u16(CUtensorMap* out, const void* base, uint64_t rows, u
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Map of a dense [z][rows][cols] tensor of 16-bit elements (cols a multiple of 8) with a box of 64 columns x box_rows x 1 and the 128-byte
+// swizzle; what lies outside reads zero.
+inline bool make_map_3d_u16(CUtensorMap* out, const void* base, uint64_t zs, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    if ((reinterpret_cast<uintptr_t>(base) & 15u) || ((cols * 2) & 15u) || box_rows > 256 || box_rows < 1) return false;
+    const cuuint64_t dims[3] = {cols, rows, zs};
+    const cuuint64_t strides[2] = {2 * cols, rows * 2 * cols};
+    const cuuint32_t box[3] = {64, box_rows, 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return fn(out, CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Map of such a tensor of 16-bit elements for tma_load_tok: box = 64 channels (d <= 64: the rest is
 // zero-filled) x box_tokens, with the 128-byte swizzle or none.  *head_first receives the order.
 // False if the strides cannot be expressed (not multiples of 16 bytes, or not nested).
