@@ -18,7 +18,7 @@
 // token's gradient leaves after 64 of them.
 //
 // What bounds it: fp32 reductions, about 2 TB/s (a tile adds 32 KB of bias gradients and 32 KB per output); without them a tile takes
-// 6000 cycles of 9400, of which splitting and storing terms is 2000 beside operand reads of the tensor pipe (shared memory at 60 %).
+// 6000 cycles of 9400, of which splitting and storing terms is 2000 beside operand reads of the tensor pipe.
 // 16 slabs of a 128 x 128 grid, 256 agents, biases: broadcast 336 us, aggregation 412 us, statistics 88 + 6 us; on mma.sync (bwd_sums_kernel,
 // bwd_rows_kernel) 828, 1010 and 242 us.  192 slabs of 14 x 14, 81 agents, whole pass: 313 -> 187 us; one slab of 40 x 23, 49 agents of 32
 // channels: 62 -> 51 us.

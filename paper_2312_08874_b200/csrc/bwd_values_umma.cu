@@ -14,8 +14,8 @@
 //   warp 13, 14 issue the logits (a tile ahead) and P V
 // Runs that hold part of a slab leave partial states; bwd_values_merge_kernel joins them, one warp per row.
 //
-// What bounds it: full, the splits and the row warps' waits (16 slabs of a 128 x 128 grid, 256 agents: 104 + 8 us, 58 TFLOP/s of term pairs at
-// 0.33 of the tensor rate; bwd_sums_kernel 317 us); mixed, the start of the kernel (about 12 of 27 us at 64 slabs of 56 x 56).
+// What bounds it: full, the splits and the row warps' waits (16 slabs of a 128 x 128 grid, 256 agents: 104 + 8 us, 495 TFLOP/s of term
+// pairs, a third of the bf16 rate; bwd_sums_kernel 317 us); mixed, the start of the kernel (about 12 of 27 us at 64 slabs of 56 x 56).
 #include "bwd_terms_launch.cuh"
 #include "stream_common.cuh"
 
