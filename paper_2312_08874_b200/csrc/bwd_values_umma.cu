@@ -52,11 +52,15 @@ constexpr int BAR_A = 7;       // [2] tx              issuer of the logits
 constexpr int BAR_S = 9;       // [2] commit          row warps
 constexpr int BAR_READ = 11;   // [2] row warps       issuer of the logits: they have been read
 constexpr int BAR_P = 13;      //     row warps       issuer of P V: the probabilities are in tensor memory
-constexpr int BAR_DONE = 14;   // [2] commit          producer, row warps, output warps: P V of a tile
+constexpr int BAR_DONE = 14;   // [2] commit          row warps, output warps: P V of a tile
 constexpr int BAR_OUT = 16;    // [2] output warps    issuer of P V: its result has been read
 constexpr int BAR_DRAIN = 18;  // [2] commit          each issuer, once, at its end
-constexpr int kBars = 20;
+constexpr int BAR_FREE = 20;   // [3] commit          producer: P V of the tile in this stage, the last to read it
+constexpr int kBars = 23;
 static_assert(8 * kBars <= OFF_DEAD, "mbarriers");
+// A producer that is late must not find the barrier it waits on two phases further: the next phase of a stage's own barrier needs the
+// very load that the producer is about to issue.
+static_assert(kBars - BAR_FREE == kStages, "one release barrier per stage");
 constexpr int kTimeoutTile = 3, kTimeoutRole = 6;
 
 // tensor memory columns: logits, twice; terms of P (128 tokens = 64 columns each); products (twice where there is room)
@@ -136,7 +140,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_values_umma_kernel(const __gr
             int buf = 0;
             for (int i = 0; i < count && !pipe_dead(pp); ++i, advance()) {
                 const int s = i % kStages, b = i & 1;
-                if (i >= kStages) wait_spin(pp, BAR_DONE + ((i - kStages) & 1), (i - kStages) >> 1, kTimeoutRole);
+                if (i >= kStages) wait_spin(pp, BAR_FREE + s, i / kStages - 1, kTimeoutRole);
                 const uint32_t bar = pipe_bar(pp, BAR_FULL + s), dst = base + OFF_RING + s * 2 * kTile;
                 mbar_arrive_expect_tx(bar, 2 * kTile);
                 tma_load_3d(dst, &p.tm_k, 0, tile * kTok, slab, bar);
@@ -202,6 +206,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_values_umma_kernel(const __gr
             for (int t = TP - 1; t >= 0; --t)
 #pragma unroll
                 for (int k = 0; k < 8; ++k) umma_ts_w(pp.tmem + TM_D + 64 * db, pp.tmem + TM_P + 64 * t + 8 * k, dv + 128 * k, id, t < TP - 1 || k > 0);
+            umma_commit_w(pipe_bar(pp, BAR_FREE + s));
             umma_commit_w(pipe_bar(pp, BAR_DONE + b));
         }
         umma_drain_w(pp, BAR_DRAIN + 1);
