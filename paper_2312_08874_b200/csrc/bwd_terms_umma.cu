@@ -15,7 +15,10 @@
 //
 // Accuracy: an accumulation in tensor memory does not round to nearest, so a chain drifts with its length (see term_sum).  The small pairs
 // of S and dP therefore have accumulators of their own and those of the other products come first, sums over tokens leave tensor memory after every tile and join in fp32 registers, and the agents' share of a
-// token's gradient leaves after 64 of them.
+// token's gradient leaves after 64 of them.  Probabilities add up to one only where logits and statistics drift alike: the statistics above
+// come from the same instructions as the broadcast stage's logits, and the aggregation's logits are one chain, small pairs first, where
+// bwd_values_umma.cu made the statistics.  (With the pairs apart there, and a common part of 8 in the logits, dV of four slabs of 64 x 64 tokens,
+// 81 agents, was 3.8e-7 too large; 5e-8 in one chain.  With statistics from bwd_sums_kernel it is the other way round: 4e-8 and 4.5e-7.)
 //
 // What bounds it: fp32 reductions, about 2 TB/s (a tile adds 32 KB of bias gradients and 32 KB per output); without them a tile takes
 // 6000 cycles of 9400, of which splitting and storing terms is 2000 beside operand reads of the tensor pipe.
@@ -82,6 +85,7 @@ struct Args {
     int* status;
     int slabs, heads, N, n, d, tiles, blocks;
     int bias;                 // 0: none; 1: tiles of token rows; 2: tiles of agent rows
+    int chain;                // aggregation: all pairs of S in one accumulator, as where `stats` come from bwd_values_umma_kernel
     float scale;
     alignas(64) CUtensorMap tm_x, tm_y, tm_a, tm_m, tm_b;
 };
@@ -106,6 +110,16 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16]) {
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
         : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]),
           "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15]) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void load_pairs(uint32_t taddr, float2 (&v)[16]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float a[16];
+        tmem_ld16(taddr + 16 * h, a);
+        tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[8 * h + j] = make_float2(a[2 * j], a[2 * j + 1]);
+    }
 }
 // 32 columns of leading pairs and of small ones (64 columns on), joined
 __device__ __forceinline__ void load_joined(uint32_t taddr, float2 (&v)[16]) {
@@ -214,12 +228,15 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
             const uint64_t dx = umma_desc_sw128(base + OFF_RING + b * kStage);
             // descriptor start addresses count 16-byte units: + 2 per k step of a K-major operand (32 bytes)
 #pragma unroll
-            for (int which = 0; which < 2; ++which)
+            for (int which = 0; which < 2; ++which) {
+                const bool chain = AGG && which == 0 && p.chain;
 #pragma unroll
                 for (int t = kTerms - 1; t >= 0; --t)
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        umma_ss_w(ts + (TM_DP - TM_S) * which + (t == 0 ? 0 : 64), dx + which * (kTile >> 4) + 2 * k, da + (which * kTerms + t) * (kMat >> 4) + 2 * k, id, t == 1 || k > 0);
+                        umma_ss_w(ts + (TM_DP - TM_S) * which + (chain || t == 0 ? 0 : 64), dx + which * (kTile >> 4) + 2 * k, da + (which * kTerms + t) * (kMat >> 4) + 2 * k, id,
+                                  k > 0 || (chain ? t < kTerms - 1 : t == 1));
+            }
             if (STATS) umma_commit_w(pipe_bar(pp, BAR_FREE + b));
             umma_commit_w(pipe_bar(pp, BAR_S));
         }
@@ -390,7 +407,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
             wait_par(pp, BAR_S, i, kTimeoutTile);
             tc_fence_after_sync();
             float2 pr[16], ds[16];
-            load_joined(ts, pr);
+            if (AGG && p.chain) load_pairs(ts, pr);
+            else load_joined(ts, pr);
             load_joined(ts + (TM_DP - TM_S), ds);
             tc_fence_before_sync();
             __syncwarp();
@@ -581,6 +599,7 @@ cudaError_t launch_backward_terms_umma(BwdTermsUmma stage, const BwdCall& c, con
     a.outer0 = c.ws_dva; a.outer1 = c.ws_da;
     a.row0 = queries ? c.dq : c.dk; a.row1 = c.dv;
     a.dbias = queries ? c.db2 : c.db1;
+    a.chain = backward_values_eligible(c.slabs, c.n, N);
     a.scale = queries ? c.scale2 : c.scale1;
     if (!make_map_3d_u16(&a.tm_x, queries ? c.q : c.k, c.slabs, N, c.d, kTok) || !make_map_3d_u16(&a.tm_y, queries ? c.d_out : c.v, c.slabs, N, c.d, kTok) ||
         !make_map_3d_u16(&a.tm_a, a_t, (uint64_t)kTerms * c.slabs, c.n, c.d, 64) || !make_map_3d_u16(&a.tm_m, m_t, (uint64_t)kTerms * c.slabs, c.n, c.d, 64))

@@ -1,4 +1,5 @@
 """Gradients with fp32 accuracy on tensor memory (bf16, up to 64 channels) at the edges of tiles, agent blocks and runs, against the fp64 oracle."""
+import numpy as np
 import pytest
 
 from paper_2312_08874_b200 import AA_PATH_AUTO, Workload, make_inputs
@@ -29,3 +30,20 @@ def test_tiles_and_agent_blocks_match_oracle(case):
     check(got, ref, str(case))
     values = H * W > 1024 or (pool > 8 and B * heads * H * W >= 16384)
     assert mod.last_launch_count() == 8 + (pool > 8) + values, "expected the tensor-memory gradient kernels"
+
+
+@pytest.mark.parametrize("case", [(2, 2, 64, 64, 64, 9), (3, 2, 20, 20, 64, 9), (4, 2, 28, 28, 40, 5)], ids=["values_umma", "sums_n81", "sums_d40"])
+def test_probabilities_stay_normalised(case):
+    """Queries and keys with a common part, logits of 32 (46 in log2 units, whose fp32 unit is 2^-18).  Tensor memory rounds towards zero: a
+    step of an accumulation loses half a unit on average, which the statistics of the softmax have to share.  Else every probability, and dV
+    with them, is off by one factor of 2^-19 ln 2 = 1.3e-6 a step.  Bound: less than one step."""
+    B, heads, H, W, d, pool = case
+    w = Workload("mean", B, heads, H, W, d, pool, "bf16", False, False, 1.0, seed=950)
+    inp = make_inputs(w)
+    for k in ("q", "k"):
+        inp[k] = (inp[k].float() + 2.0).to(inp[k].dtype)
+    _, got, ref = run_both(w, inp, path=AA_PATH_AUTO)
+    g, r = got["dv"].double().cpu().numpy(), ref["dv"]
+    bias = float(((g - r) * np.sign(r)).sum() / np.abs(r).sum())
+    print(f"{case}: factor of dV 1 + {bias:.2e}")
+    assert abs(bias) < 1e-6, bias
