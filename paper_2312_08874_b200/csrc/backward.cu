@@ -396,7 +396,6 @@ cudaError_t backward_typed(const BwdCall& c, BwdArgs a, cudaStream_t st) {
     if (c.ws_mixed) {
         AA_TRY(launch_backward_mixed_forward(c.dtype, c, st));
         AA_TRY(launch_backward_umma(c.dtype, true, c, st));
-        AA_TRY(launch_backward_mixed_dot(c.dtype, c, st));
         AA_TRY(launch_backward_umma(c.dtype, false, c, st));
         return launch_backward_tail(c.dtype, c, st);
     }
@@ -464,7 +463,7 @@ int backward_launch_count(const BwdCall& c) {
     const int N = c.H * c.W;
     const bool umma = c.ws_mixed || (c.ws_terms && backward_terms_umma_eligible(c.dtype, c.n, N, c.d));
     const int values = umma && backward_values_eligible(c.slabs, c.n, N);
-    return (c.ws_mixed ? 5 + values : !c.ws_terms ? 7 : umma ? 6 + values + (c.n > 64) : 8) + 1 + (c.wd ? 1 : 0);
+    return (c.ws_mixed ? 4 + values : !c.ws_terms ? 7 : umma ? 6 + values + (c.n > 64) : 8) + 1 + (c.wd ? 1 : 0);
 }
 
 cudaError_t launch_backward(int dtype, const BwdCall& c, cudaStream_t st) {

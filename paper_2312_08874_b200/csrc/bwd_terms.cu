@@ -209,12 +209,12 @@ size_t backward_terms_bytes(int dtype, int slabs, int heads, int n, int N, int d
 
 cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStream_t st) {
     const size_t rows = (size_t)c.heads * c.H * c.W;
-    char* padded = static_cast<char*>(c.ws_mixed) + up256((size_t)2 * c.slabs * c.n * 64 * 2);          // (see backward_umma_bytes)
+    char* padded = static_cast<char*>(c.ws_mixed);                 // (see backward_umma_bytes)
     const PadList pl = pad_list(c.b1, c.b2, padded, padded + rows * 128, c.heads, c.n, c.H * c.W);
     cudaError_t e = dtype == kBF16 ? pool_and_clear<__nv_bfloat16, __nv_bfloat16, 1>(c, c.ws_a, true, false, pl, st) : pool_and_clear<__half, __half, 1>(c, c.ws_a, true, false, pl, st);
     if (e != cudaSuccess) return e;
     if (backward_values_eligible(c.slabs, c.n, c.H * c.W))
-        return launch_backward_values(dtype, false, c, c.ws_a, c.ws_part, reinterpret_cast<float2*>(c.ws_lse), padded, static_cast<char*>(c.ws_mixed) + backward_umma_bytes(c.slabs, c.heads, c.n, c.H * c.W), st);
+        return launch_backward_values(dtype, false, c, c.ws_a, c.ws_part, reinterpret_cast<float2*>(c.ws_lse), padded, static_cast<char*>(c.ws_mixed) + backward_umma_bytes(c.heads, c.H * c.W), st);
     BwdTermArgs a;
     memset(&a, 0, sizeof(a));
     a.slabs = c.slabs; a.heads = c.heads; a.N = c.H * c.W; a.n = c.n; a.d = c.d;
@@ -229,15 +229,6 @@ cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStrea
     l.grid = dim3(parts, 1, c.slabs);
     l.cluster = parts;
     return bwd_terms_mixed(dtype, a, l);
-}
-
-// D = dV_A . V_A and the two terms of dV_A, between the two gradient stages
-cudaError_t launch_backward_mixed_dot(int dtype, const BwdCall& c, cudaStream_t st) {
-    const int rows = c.slabs * c.n;
-    const float *va = c.ws_va, *dva = c.ws_dva;
-    float2* stats = reinterpret_cast<float2*>(c.ws_lse);
-    if (dtype == kBF16) return launch_dependent(bwd_dot_split_kernel<__nv_bfloat16, 2>, dim3((rows + 7) / 8), 256, 0, st, va, dva, stats, static_cast<__nv_bfloat16*>(c.ws_mixed), rows, c.d);
-    return launch_dependent(bwd_dot_split_kernel<__half, 2>, dim3((rows + 7) / 8), 256, 0, st, va, dva, stats, static_cast<__half*>(c.ws_mixed), rows, c.d);
 }
 
 cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStream_t st) {

@@ -13,7 +13,8 @@
 //   warps 0-7   "row warps": thread = (token, half of the agents).  Logits and dP from tensor memory, bias from the ring stage; P and dS as
 //               swizzled rows of 64 agents in shared memory: the same bytes are the K-major operand of the products per token and the
 //               MN-major operand of the sums over tokens, so nothing is transposed.  Then the bias gradient, by coalesced reductions.
-//   warps 8-11  outputs: per-token products from tensor memory to global memory; at the end of a slab its sums.
+//   warps 8-11  outputs: per-token products from tensor memory to global memory; at the end of a slab its sums.  Aggregation: a slab ahead,
+//               D and the terms of dV_A.
 //   warp 12     TMA: X, Y and the padded bias rows, two stages of 48 KB.
 //   warp 13, 14 issue S and dP (a tile ahead), and the products of P and dS.
 // The sums of both halves are one 128-row operand [P | dS] against [X | Y]: eight instructions of 128 columns, of whose four blocks two
@@ -22,6 +23,7 @@
 // What bounds it: the chain load -> logits -> softmax -> products -> stage free through two stages (tensor pipe about 0.8 us of it per tile),
 // and HBM: 64 slabs of a 56 x 56 grid, 49 agents: broadcast 36 us (103 MB, 16 us at the copy bandwidth), aggregation 41 us (154 MB, 24 us).
 // With mma.sync, 64-token tiles and scalar bias loads and reductions the two took 96 and 93 us.
+#include "bwd_terms.cuh"
 #include "stream_common.cuh"
 
 #include <cstring>
@@ -54,14 +56,16 @@ constexpr int BAR_P = 4;      // [2] row warps        both issuers: P and dS wri
 constexpr int BAR_DONE = 6;   // [2] commit           producer, row warps, output warps: every product of a tile
 constexpr int BAR_OUT = 8;    //     output warps     products issuer: outputs (and a finished slab's sums) read
 constexpr int BAR_DRAIN = 9;  // [2] commit           each issuer, once, at its end
-constexpr int kBars = 11;
+constexpr int BAR_M = 11;     // [2] output warps     logits issuer, row warps: terms of dV_A and statistics of a slab (aggregation)
+constexpr int kBars = 13;
 constexpr int kTimeoutTile = 3, kTimeoutRole = 6;
 
 // tensor memory columns: S | dP, twice; outputs; sums
 constexpr uint32_t TM_S = 0, TM_OUT = 256, TM_SUM = 384;
 
 struct UmmaArgs {
-    const float2* stats;      // aggregation: (log2-sum-exp, D) [slabs][n]
+    const float2* stats;      // aggregation: .x = log2-sum-exp [slabs][n]
+    const float *va, *dva;    // aggregation: V_A and dV_A, fp32 [slabs][n][64]
     float *outer0, *outer1;   // fp32 [slabs][n][64]: dV_A (broadcast) and dA (added)
     float *row0, *row1;       // fp32 [slabs][N][64]: dQ, or dK and dV
     float* dbias;             // fp32, B2's layout [heads][N][n] or B1's [heads][n][N] (added), or null
@@ -111,7 +115,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_umma_kernel(const __grid_cons
     pp.ph = 0u;
     if (tid == 0) {
         s_dead = 0;
-        for (int i = 0; i < kBars; ++i) mbar_init(pp.bars + 8 * i, i >= BAR_P && i < BAR_DONE ? 8u : i == BAR_OUT ? 4u : 1u);
+        for (int i = 0; i < kBars; ++i) mbar_init(pp.bars + 8 * i, i >= BAR_P && i < BAR_DONE ? 8u : i == BAR_OUT || i >= BAR_M ? 4u : 1u);
         mbar_fence_init();
     }
     if (warp == 0) tmem_alloc<512>(smem_u32(&s_tmem));
@@ -135,13 +139,15 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_umma_kernel(const __grid_cons
                 if (i >= 2) wait_spin(pp, BAR_DONE + b, (i >> 1) - 1, kTimeoutRole);
                 const bool fresh = i == 0 || tile == 0;
                 const uint32_t bar = pipe_bar(pp, BAR_FULL + b), dst = base + OFF_RING + b * kStage;
-                mbar_arrive_expect_tx(bar, (p.bias ? 3u : 2u) * kTile + (fresh ? 3u * kMat : 0u));
+                mbar_arrive_expect_tx(bar, (p.bias ? 3u : 2u) * kTile + (fresh ? (BCAST ? 3u : 1u) * kMat : 0u));
                 if (fresh) {
                     const uint32_t am = base + OFF_AM + buf * 3 * kMat;
                     buf ^= 1;
                     tma_load_3d(am, &p.tm_a, 0, 0, slab, bar);
-                    tma_load_3d(am + kMat, &p.tm_m, 0, 0, slab, bar);
-                    tma_load_3d(am + 2 * kMat, &p.tm_m, 0, 0, p.slabs + slab, bar);
+                    if (BCAST) {
+                        tma_load_3d(am + kMat, &p.tm_m, 0, 0, slab, bar);
+                        tma_load_3d(am + 2 * kMat, &p.tm_m, 0, 0, p.slabs + slab, bar);
+                    }
                 }
                 tma_load_3d(dst, &p.tm_x, 0, tile * kTok, slab, bar);
                 tma_load_3d(dst + kTile, &p.tm_y, 0, tile * kTok, slab, bar);
@@ -152,10 +158,13 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_umma_kernel(const __grid_cons
     } else if (warp == 13) {
         // ------------------------------------------------------------------ S and dP, a tile ahead
         const uint32_t id = umma_idesc(fmt, 128, 64, 0);
-        int buf = 1;
+        int buf = 1, order = 0;
         for (int i = 0; i < count && !pipe_dead(pp); ++i, advance()) {
             const int b = i & 1;
-            if (i == 0 || tile == 0) buf ^= 1;
+            if (i == 0 || tile == 0) {
+                buf ^= 1;
+                if (!BCAST) wait_spin(pp, BAR_M + buf, order++ >> 1, kTimeoutRole);
+            }
             if (i >= 2) wait_spin(pp, BAR_P + b, (i >> 1) - 1, kTimeoutRole);          // tile i - 2 has been read out of tensor memory
             wait_spin(pp, BAR_FULL + b, i >> 1, kTimeoutTile);
             tc_fence_after_sync();
@@ -204,8 +213,60 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_umma_kernel(const __grid_cons
         // ------------------------------------------------------------------ outputs
         const int q = warp & 3, g = lane >> 2, t = lane & 3;
         const uint32_t rows = pp.tmem + ((uint32_t)(32 * q) << 16);
+        // M of a slab for the aggregation: the two terms of dV_A, and (log2-sum-exp, D = dV_A . V_A) of its agents
+        auto prepare = [&](int of, int buf) {
+            const int c = lane & 7, r0 = 16 * q + (lane >> 3);         // rows r0 + 4 k, channels 8 c ..
+            float4 dva[4][2], va[4][2];
+            float lse[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const bool have = r0 + 4 * k < n;
+                const size_t row = (size_t)of * n + r0 + 4 * k;
+                lse[k] = INFINITY;                                 // (an agent that does not exist: its probabilities are zero)
+                if (have) lse[k] = __ldcg(&p.stats[row].x);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    dva[k][h] = va[k][h] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (have) dva[k][h] = __ldcg(reinterpret_cast<const float4*>(p.dva + row * 64 + 8 * c + 4 * h));
+                    if (have) va[k][h] = __ldcg(reinterpret_cast<const float4*>(p.va + row * 64 + 8 * c + 4 * h));
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int r = r0 + 4 * k;
+                uint32_t hi[4], lo[4];
+                float dot = 0.f;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float4 a = dva[k][h], v = va[k][h];
+                    dot = fmaf(a.x, v.x, fmaf(a.y, v.y, fmaf(a.z, v.z, fmaf(a.w, v.w, dot))));
+                    uint32_t w[2];
+                    split_pair<T, 2>(a.x, a.y, w);
+                    hi[2 * h] = w[0]; lo[2 * h] = w[1];
+                    split_pair<T, 2>(a.z, a.w, w);
+                    hi[2 * h + 1] = w[0]; lo[2 * h + 1] = w[1];
+                }
+                const uint32_t at = base + OFF_AM + (3 * buf + 1) * kMat + r * 128 + ((c ^ (r & 7)) << 4);
+                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(at), "r"(hi[0]), "r"(hi[1]), "r"(hi[2]), "r"(hi[3]) : "memory");
+                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(at + kMat), "r"(lo[0]), "r"(lo[1]), "r"(lo[2]), "r"(lo[3]) : "memory");
+#pragma unroll
+                for (int o = 4; o; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+                if (c == 0) reinterpret_cast<float2*>(smem + OFF_PATCH)[64 * buf + r] = make_float2(lse[k], dot);
+            }
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) pipe_arrive(pp, BAR_M + buf);
+        };
+        int prepared = 0, order = -1;                              // slabs of the run, in their order
         for (int i = 0; i < count; ++i, advance()) {
             const int b = i & 1;
+            if (!BCAST && (i == 0 || tile == 0)) {
+                // a slab ahead: every tile of the slab before this one is done, and with them the buffer of the next
+                ++order;
+                const int last = p.tiles - tile < count - i ? order + 1 : order;
+#pragma unroll 1
+                for (; prepared <= last; ++prepared) prepare(slab + prepared - order, prepared & 1);
+            }
             wait_par(pp, BAR_DONE + b, i >> 1, kTimeoutTile);
             tc_fence_after_sync();
             float o[2][32];                                        // rows 16 f + g + 8 h of the warp's 32
@@ -264,17 +325,13 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_umma_kernel(const __grid_cons
         float2* s_stat = reinterpret_cast<float2*>(smem + OFF_PATCH);
         float* patch = reinterpret_cast<float*>(smem + OFF_PATCH) + warp * 32 * kPatch;
         float4* ex = reinterpret_cast<float4*>(smem + OFF_EX);
-        int parity = 0;
-        float2 next = make_float2(INFINITY, 0.f);                  // (an agent that does not exist: its probabilities are zero)
-        if (!BCAST && tid < n) next = __ldg(p.stats + (size_t)slab * n + tid);
+        int order = -1;                                            // slab of the run
         for (int i = 0; i < count; ++i, advance()) {
             const int b = i & 1, tok = tile * kTok + r;
             const bool ok = tok < N;
             if (!BCAST && (i == 0 || tile == 0)) {                 // another slab: its statistics
-                parity ^= 1;
-                if (tid < 64) s_stat[parity * 64 + tid] = next;
-                if (tid < n && slab + 1 < p.slabs) next = __ldg(p.stats + (size_t)(slab + 1) * n + tid);
-                bar_named(1, kRowThreads);
+                ++order;
+                wait_par(pp, BAR_M + (order & 1), order >> 1, kTimeoutTile);
             }
             wait_par(pp, BAR_FULL + b, i >> 1, kTimeoutTile);
             wait_par(pp, BAR_S + b, i >> 1, kTimeoutTile);
@@ -338,7 +395,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_umma_kernel(const __grid_cons
                 }
             } else {
                 tmem_ld_wait();
-                const float4* st = reinterpret_cast<const float4*>(s_stat + parity * 64 + c0);
+                const float4* st = reinterpret_cast<const float4*>(s_stat + (order & 1) * 64 + c0);
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
                     const float4 v = st[j];                        // (lse, D) of two agents
@@ -421,16 +478,14 @@ cudaError_t launch_backward_umma(int dtype, bool broadcast_stage, const BwdCall&
     a.slabs = c.slabs; a.heads = c.heads; a.N = N; a.n = c.n; a.tiles = (N + kTok - 1) / kTok; a.bias = bias != nullptr;
     a.status = c.status;
     a.stats = reinterpret_cast<const float2*>(c.ws_lse);
+    a.va = c.ws_va; a.dva = c.ws_dva;
     a.outer0 = c.ws_dva; a.outer1 = c.ws_da;
     a.row0 = broadcast_stage ? c.dq : c.dk; a.row1 = c.dv;
     a.dbias = broadcast_stage ? c.db2 : c.db1;
     a.scale = broadcast_stage ? c.scale2 : c.scale1;
-    const size_t terms = ((size_t)2 * c.slabs * c.n * 64 * 2 + 255) / 256 * 256;
-    const char* w = static_cast<const char*>(c.ws_mixed);
-    const void* m = broadcast_stage ? static_cast<const void*>(c.ws_part) : w;
-    const void* padded = w + terms + (broadcast_stage ? (size_t)c.heads * N * 128 : 0);
+    const void* padded = static_cast<const char*>(c.ws_mixed) + (broadcast_stage ? (size_t)c.heads * N * 128 : 0);
     if (!make_map_rows3d_u16(&a.tm_x, broadcast_stage ? c.q : c.k, c.slabs, N, kTok, true) || !make_map_rows3d_u16(&a.tm_y, broadcast_stage ? c.d_out : c.v, c.slabs, N, kTok, true) ||
-        !make_map_rows3d_u16(&a.tm_a, c.ws_a, c.slabs, c.n, 64, true) || !make_map_rows3d_u16(&a.tm_m, m, 2 * (uint64_t)c.slabs, c.n, 64, true) ||
+        !make_map_rows3d_u16(&a.tm_a, c.ws_a, c.slabs, c.n, 64, true) || (broadcast_stage && !make_map_rows3d_u16(&a.tm_m, c.ws_part, 2 * (uint64_t)c.slabs, c.n, 64, true)) ||
         (bias && !make_map_rows3d_u16(&a.tm_b, padded, c.heads, N, kTok, true)))
         return cudaErrorInvalidValue;
     if (dtype == kBF16) return broadcast_stage ? launch<__nv_bfloat16, true>(a, c.sm_count, st) : launch<__nv_bfloat16, false>(a, c.sm_count, st);
@@ -438,9 +493,7 @@ cudaError_t launch_backward_umma(int dtype, bool broadcast_stage, const BwdCall&
     return cudaErrorInvalidValue;
 }
 
-// Workspace: two terms of dV_A, then B1 transposed and B2, both padded to 64 agents
-size_t backward_umma_bytes(int slabs, int heads, int n, int N) {
-    return ((size_t)2 * slabs * n * 64 * 2 + 255) / 256 * 256 + 2 * (size_t)heads * N * 128;
-}
+// Workspace: B1 transposed and B2, both padded to 64 agents
+size_t backward_umma_bytes(int heads, int N) { return 2 * (size_t)heads * N * 128; }
 
 }  // namespace aa

@@ -285,7 +285,6 @@ void backward_terms_umma_padded(int heads, int n, int N, void* ws, void** b1, vo
 cudaError_t launch_backward_terms_umma(BwdTermsUmma stage, const BwdCall& c, const void* a_t, const void* m_t, float2* stats, const void* padded, void* partial, cudaStream_t st);
 // mixed precision, 16-bit inputs: A (16 bits, in ws_a), V_A (fp32 in ws_va, terms in ws_part), statistics (in ws_lse); clears the sums
 cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStream_t st);
-cudaError_t launch_backward_mixed_dot(int dtype, const BwdCall& c, cudaStream_t st);
 // token-wise tail: dQ += Pooling^T(dA), dV += DWC^T(dO), dWd
 cudaError_t launch_backward_tail(int dtype, const BwdCall& c, cudaStream_t st);
 bool plan_backward(int slabs, int n, int N, int d, int sm_count, BwdPlan* out);   // false: shape not supported
@@ -293,7 +292,7 @@ int backward_launch_count(const BwdCall& c);
 cudaError_t launch_backward(int dtype, const BwdCall& c, cudaStream_t st);
 // Tensor-core kernels of the two gradient stages (16-bit inputs, n <= 64, d = 64)
 bool backward_umma_eligible(int dtype, int n, int d);
-size_t backward_umma_bytes(int slabs, int heads, int n, int N);
+size_t backward_umma_bytes(int heads, int N);
 cudaError_t launch_backward_umma(int dtype, bool broadcast_stage, const BwdCall& c, cudaStream_t st);
 
 }  // namespace aa
