@@ -223,8 +223,10 @@ __global__ void __launch_bounds__(kThreadsV, sizeof(T) == 4 ? 4 : 5) bwd_conv_ta
 #pragma unroll
         for (int k = 0; k < 9; ++k) red[threadIdx.x][k] = acc[k];
         __syncthreads();
-        // one of several copies: a sum of all blocks' shares in one word would round as often as there are blocks
-        float* copy = a.dwd_copies + ((size_t)((blockIdx.x + blockIdx.y) % kFilterCopies) * a.heads + head) * d * 9;
+        // one of several copies, by the block's rank in its head: a sum of all blocks' shares in one word would round as often as there are
+        // blocks
+        const unsigned rank = blockIdx.x + gridDim.x * (blockIdx.y / a.heads);
+        float* copy = a.dwd_copies + ((size_t)(rank % kFilterCopies) * a.heads + head) * d * 9;
         for (int o = threadIdx.x; o < d * 9; o += kThreadsV) {    // o = channel * 9 + tap
             const int c = o / 9, k = o - c * 9;
             float s = 0.f;

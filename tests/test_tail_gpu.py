@@ -1,7 +1,9 @@
 """Token-wise tail of the backward pass (pooling, depthwise and filter gradients) at the edges of its tiles, against the fp64 oracle."""
 import pytest
+import torch
 
-from paper_2312_08874_b200 import AA_PATH_AUTO, Workload, make_inputs
+from paper_2312_08874_b200 import AA_PATH_AUTO, Workload, make_inputs, make_upstream_grad
+from tests.parity_util import make_module, to_dev
 from tests.test_backward_gpu import check, run_both
 
 pytestmark = pytest.mark.gpu
@@ -44,3 +46,21 @@ def test_strips_match_oracle(case):
     w = Workload("tail", B, heads, H, W, d, pool, dtype, True, True, 1.0, seed=700 + H * W + d)
     _, got, ref = run_both(w, make_inputs(w, bias_std=0.5, dwc_std=0.2), path=AA_PATH_AUTO)
     check(got, ref, str(case), tc=d == 64 and dtype != "f32")
+
+
+@pytest.mark.parametrize("case", [(64, 8, 7), (64, 16, 7), (128, 4, 7), (32, 16, 14)], ids=lambda c: f"B{c[0]}h{c[1]}_{c[2]}x{c[2]}")
+def test_filter_gradient_is_shared_by_every_copy(case):
+    """Blocks add their share of a head's filter gradient to one of sixteen copies, so that a word takes a sixteenth of the roundings and of
+    the atomics.  Every copy of every head is in use where a head has at least as many blocks (here 40 to 90)."""
+    B, heads, grid = case
+    w = Workload("copies", B, heads, grid, grid, 64, 7, "bf16", False, True, 1.0, seed=770)
+    inp, mod = make_inputs(w, dwc_std=0.2), make_module(w)
+    ws = torch.zeros(mod.lib.agent_attn_backward_workspace_bytes(mod._h, grid, grid, 49), dtype=torch.uint8, device="cuda")
+    mod.backward(to_dev(inp["q"]), to_dev(inp["k"]), to_dev(inp["v"]), to_dev(make_upstream_grad(w)), grid, grid, 49,
+                 dwc_weight=to_dev(inp["dwc"]), workspace=ws)
+    torch.cuda.synchronize()
+    up = lambda x: (x + 255) // 256 * 256
+    at = 4 * up(B * heads * 49 * 64 * 4) + 2 * up(B * heads * 49 * 4)             # A, V_A, dV_A, dA, then two words per agent
+    copies = ws[at:at + 16 * heads * 64 * 9 * 4].view(torch.float32).view(16, heads, 64 * 9)
+    used = (copies != 0).any(dim=2).sum(dim=0).tolist()
+    assert used == [16] * heads, used
