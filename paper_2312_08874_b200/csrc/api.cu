@@ -893,7 +893,7 @@ bool bwd_layout(const agent_attn_handle* h, int N, int n, BwdPlan* pl, BwdLayout
     size_t part_floats = (size_t)slabs * pl->chunks * n * 2;
     if (part_floats * sizeof(float) < snd) part_floats = snd / sizeof(float);       // (mixed precision: two 16-bit terms of V_A)
     w->terms = w->part + align_up(part_floats * sizeof(float), 256);
-    w->total = w->terms + (use_mixed(h, n) ? backward_umma_bytes(h->cfg.heads, N) + backward_values_bytes(slabs, n, N, h->sm_count) : use_terms(h, n) ? backward_terms_bytes(h->cfg.dtype, slabs, h->cfg.heads, n, N, h->cfg.head_dim, h->sm_count) : 0);
+    w->total = w->terms + (use_mixed(h, n) ? backward_umma_bytes(h->cfg.heads, n, N) + backward_values_bytes(slabs, n, N, h->sm_count) : use_terms(h, n) ? backward_terms_bytes(h->cfg.dtype, slabs, h->cfg.heads, n, N, h->cfg.head_dim, h->sm_count) : 0);
     return true;
 }
 }  // namespace

@@ -30,14 +30,15 @@ struct ClearList {
     int pool_blocks;
 };
 constexpr int kClearWords = 256 * 32;              // words that a block clears
-// Biases as rows of `width` agents per token [heads][N][width] (zeros past n), by further blocks of the first kernel: B1 transposed, B2.
+// Biases as rows of bias_width(n) agents per token [heads][N][width] (zeros past n), by further blocks of the first kernel: B1 transposed, B2.
+// (Rows of whole blocks of 64 agents would be four times as much memory at 9 agents.)
 struct PadList {
     const void *b1, *b2;
     void *p1, *p2;
     int heads, n, N, width, blocks1, blocks2;
 };
 PadList pad_list(const void* b1, const void* b2, void* p1, void* p2, int heads, int n, int N) {
-    const int width = (n + 63) / 64 * 64, blocks = (int)(((size_t)heads * N * (width / 8) + 255) / 256);
+    const int width = bias_width(n), blocks = (int)(((size_t)heads * N * (width / 8) + 255) / 256);
     return {b1, b2, p1, p2, heads, n, N, width, b1 && p1 ? blocks : 0, b2 && p2 ? blocks : 0};
 }
 template <typename T> __device__ __forceinline__ void pad_bias(const T* src, uint4* dst, bool transposed, const PadList& pl, int block) {
@@ -208,16 +209,16 @@ size_t backward_terms_bytes(int dtype, int slabs, int heads, int n, int N, int d
 }
 
 cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStream_t st) {
-    const size_t rows = (size_t)c.heads * c.H * c.W;
+    const int N = c.H * c.W;
     char* padded = static_cast<char*>(c.ws_mixed);                 // (see backward_umma_bytes)
-    const PadList pl = pad_list(c.b1, c.b2, padded, padded + rows * 128, c.heads, c.n, c.H * c.W);
+    const PadList pl = pad_list(c.b1, c.b2, padded, c.n % 8 ? padded + padded_bias_bytes(c.heads, c.n, N) : nullptr, c.heads, c.n, N);
     cudaError_t e = dtype == kBF16 ? pool_and_clear<__nv_bfloat16, __nv_bfloat16, 1>(c, c.ws_a, true, false, pl, st) : pool_and_clear<__half, __half, 1>(c, c.ws_a, true, false, pl, st);
     if (e != cudaSuccess) return e;
-    if (backward_values_eligible(c.slabs, c.n, c.H * c.W))
-        return launch_backward_values(dtype, false, c, c.ws_a, c.ws_part, reinterpret_cast<float2*>(c.ws_lse), padded, static_cast<char*>(c.ws_mixed) + backward_umma_bytes(c.heads, c.H * c.W), st);
+    if (backward_values_eligible(c.slabs, c.n, N))
+        return launch_backward_values(dtype, false, c, c.ws_a, c.ws_part, reinterpret_cast<float2*>(c.ws_lse), padded, padded + backward_umma_bytes(c.heads, c.n, N), st);
     BwdTermArgs a;
     memset(&a, 0, sizeof(a));
-    a.slabs = c.slabs; a.heads = c.heads; a.N = c.H * c.W; a.n = c.n; a.d = c.d;
+    a.slabs = c.slabs; a.heads = c.heads; a.N = N; a.n = c.n; a.d = c.d;
     a.x = c.k; a.y = c.v; a.bias = c.b1; a.scale = c.scale1;
     a.a_t = c.ws_a; a.outer0 = c.ws_va; a.va_t = c.ws_part; a.agent_stats = reinterpret_cast<float2*>(c.ws_lse);
     a.rg = (c.n + 15) / 16;                            // four warps, three blocks on an SM

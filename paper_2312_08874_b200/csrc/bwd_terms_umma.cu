@@ -572,8 +572,6 @@ template <int MODE> cudaError_t launch(const Args& a, int sm_count, cudaStream_t
 // (One agent or one token: a softmax over it has no gradient, which the recomputed products give exactly only where both passes agree)
 bool backward_terms_umma_eligible(int dtype, int n, int N, int d) { return dtype == kBF16 && d <= 64 && d % 8 == 0 && n > 1 && n <= 256 && N > 1; }
 
-// TMA takes a bias as it is where its rows are multiples of 16 bytes; others are copied to token rows of whole blocks of agents.
-static size_t padded_bias_bytes(int heads, int n, int N) { return ((size_t)heads * N * ((n + 63) / 64) * 128 + 255) / 256 * 256; }
 size_t backward_terms_umma_bytes(int slabs, int heads, int n, int N) {
     return (N % 8 ? padded_bias_bytes(heads, n, N) : 0) + (n % 8 ? padded_bias_bytes(heads, n, N) : 0) + (n > 64 ? (size_t)((n + 63) / 64) * slabs * N * 16 : 0);
 }
@@ -604,7 +602,7 @@ cudaError_t launch_backward_terms_umma(BwdTermsUmma stage, const BwdCall& c, con
     if (!make_map_3d_u16(&a.tm_x, queries ? c.q : c.k, c.slabs, N, c.d, kTok) || !make_map_3d_u16(&a.tm_y, queries ? c.d_out : c.v, c.slabs, N, c.d, kTok) ||
         !make_map_3d_u16(&a.tm_a, a_t, (uint64_t)kTerms * c.slabs, c.n, c.d, 64) || !make_map_3d_u16(&a.tm_m, m_t, (uint64_t)kTerms * c.slabs, c.n, c.d, 64))
         return cudaErrorInvalidValue;
-    if (bias && !(padded ? make_map_3d_u16(&a.tm_b, padded, c.heads, N, 64 * (uint64_t)a.blocks, kTok)
+    if (bias && !(padded ? make_map_3d_u16(&a.tm_b, padded, c.heads, N, bias_width(c.n), kTok)
                   : queries ? make_map_3d_u16(&a.tm_b, bias, c.heads, N, c.n, kTok) : make_map_3d_u16(&a.tm_b, bias, c.heads, c.n, N, 64)))
         return cudaErrorInvalidValue;
     if (stage == kUmmaBroadcast) return launch<kBcast>(a, c.sm_count, st);

@@ -15,7 +15,7 @@
 //               MN-major operand of the sums over tokens, so nothing is transposed.  Then the bias gradient, by coalesced reductions.
 //   warps 8-11  outputs: per-token products from tensor memory to global memory; at the end of a slab its sums.  Aggregation: a slab ahead,
 //               D and the terms of dV_A.
-//   warp 12     TMA: X, Y and the padded bias rows, two stages of 48 KB.
+//   warp 12     TMA: X, Y and the bias as token rows, two stages of 48 KB.
 //   warp 13, 14 issue S and dP (a tile ahead), and the products of P and dS.
 // The sums of both halves are one 128-row operand [P | dS] against [X | Y]: eight instructions of 128 columns, of whose four blocks two
 // are used; as four products of 64 x 64 they would be sixteen.
@@ -483,17 +483,16 @@ cudaError_t launch_backward_umma(int dtype, bool broadcast_stage, const BwdCall&
     a.row0 = broadcast_stage ? c.dq : c.dk; a.row1 = c.dv;
     a.dbias = broadcast_stage ? c.db2 : c.db1;
     a.scale = broadcast_stage ? c.scale2 : c.scale1;
-    const void* padded = static_cast<const char*>(c.ws_mixed) + (broadcast_stage ? (size_t)c.heads * N * 128 : 0);
+    const void* rows = !broadcast_stage ? c.ws_mixed : c.n % 8 ? static_cast<const char*>(c.ws_mixed) + padded_bias_bytes(c.heads, c.n, N) : c.b2;       // (B2 as it is where TMA takes it)
     if (!make_map_rows3d_u16(&a.tm_x, broadcast_stage ? c.q : c.k, c.slabs, N, kTok, true) || !make_map_rows3d_u16(&a.tm_y, broadcast_stage ? c.d_out : c.v, c.slabs, N, kTok, true) ||
         !make_map_rows3d_u16(&a.tm_a, c.ws_a, c.slabs, c.n, 64, true) || (broadcast_stage && !make_map_rows3d_u16(&a.tm_m, c.ws_part, 2 * (uint64_t)c.slabs, c.n, 64, true)) ||
-        (bias && !make_map_rows3d_u16(&a.tm_b, padded, c.heads, N, kTok, true)))
+        (bias && !make_map_3d_u16(&a.tm_b, rows, c.heads, N, bias_width(c.n), kTok)))
         return cudaErrorInvalidValue;
     if (dtype == kBF16) return broadcast_stage ? launch<__nv_bfloat16, true>(a, c.sm_count, st) : launch<__nv_bfloat16, false>(a, c.sm_count, st);
     if (dtype == kF16) return broadcast_stage ? launch<__half, true>(a, c.sm_count, st) : launch<__half, false>(a, c.sm_count, st);
     return cudaErrorInvalidValue;
 }
 
-// Workspace: B1 transposed and B2, both padded to 64 agents
-size_t backward_umma_bytes(int heads, int N) { return 2 * (size_t)heads * N * 128; }
+size_t backward_umma_bytes(int heads, int n, int N) { return (n % 8 ? 2 : 1) * padded_bias_bytes(heads, n, N); }
 
 }  // namespace aa

@@ -467,7 +467,7 @@ cudaError_t launch_backward_values(int dtype, bool full, const BwdCall& c, const
     if (!make_map_3d_u16(&a.tm_k, c.k, c.slabs, N, c.d, kTok) || !make_map_3d_u16(&a.tm_v, c.v, c.slabs, N, c.d, kTok) ||
         !make_map_3d_u16(&a.tm_a, a_t, (full ? 3 : 1) * (uint64_t)c.slabs, c.n, c.d, 64))
         return cudaErrorInvalidValue;
-    if (c.b1 && !(rows ? make_map_3d_u16(&a.tm_b, c.b1, c.heads, c.n, N, v.stack ? 64 : 128) : make_map_3d_u16(&a.tm_b, padded, c.heads, N, (c.n + 63) / 64 * 64, kTok)))
+    if (c.b1 && !(rows ? make_map_3d_u16(&a.tm_b, c.b1, c.heads, c.n, N, v.stack ? 64 : 128) : make_map_3d_u16(&a.tm_b, padded, c.heads, N, bias_width(c.n), kTok)))
         return cudaErrorInvalidValue;
     using B = __nv_bfloat16;
     const int grid = v.lanes * v.blocks;

@@ -266,8 +266,12 @@ struct TermsForward {
 bool terms_forward_eligible(int n, int d);
 size_t terms_forward_bytes(int slabs, int n, int d);
 cudaError_t launch_terms_forward(const TermsForward& c, cudaStream_t st);
+// Biases for TMA, whose rows are multiples of 16 bytes: copied, where they are not, to token rows of `bias_width` agents (what a box reads
+// past them is zero).
+inline int bias_width(int n) { return (n + 7) / 8 * 8; }
+inline size_t padded_bias_bytes(int heads, int n, int N) { return ((size_t)heads * N * bias_width(n) * 2 + 255) / 256 * 256; }
 // V_A (fp32 in ws_va and as terms) and the aggregation's row statistics on tensor memory: mixed precision, or (full) three bf16 terms.
-// `padded`: B1 as token rows of whole blocks of 64 agents, read where N is no multiple of 8; `ws`: backward_values_bytes.
+// `padded`: B1 as token rows, read where N is no multiple of 8; `ws`: backward_values_bytes.
 bool backward_values_eligible(int slabs, int n, int N);
 size_t backward_values_bytes(int slabs, int n, int N, int sm_count);
 cudaError_t launch_backward_values(int dtype, bool full, const BwdCall& c, const void* a_t, void* va_t, float2* stats, const void* padded, void* ws, cudaStream_t st);
@@ -278,7 +282,7 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
 // the gradient stages of that on the 5th-generation tensor cores (bf16 inputs of up to 64 channels)
 bool backward_terms_umma_eligible(int dtype, int n, int N, int d);
 enum BwdTermsUmma { kUmmaStats, kUmmaBroadcast, kUmmaAggregate };
-// Workspace: biases as token rows of whole blocks of 64 agents (null where they are read as they are), token statistics per block of agents
+// Workspace: biases as token rows (null where they are read as they are), token statistics per block of agents
 size_t backward_terms_umma_bytes(int slabs, int heads, int n, int N);
 void backward_terms_umma_padded(int heads, int n, int N, void* ws, void** b1, void** b2, void** partial);
 // `stats`: of the tokens (statistics: written), or of the agents in the aggregation stage
@@ -292,7 +296,7 @@ int backward_launch_count(const BwdCall& c);
 cudaError_t launch_backward(int dtype, const BwdCall& c, cudaStream_t st);
 // Tensor-core kernels of the two gradient stages (16-bit inputs, n <= 64, d = 64)
 bool backward_umma_eligible(int dtype, int n, int d);
-size_t backward_umma_bytes(int heads, int N);
+size_t backward_umma_bytes(int heads, int n, int N);      // copies of the biases: B1, then B2 where it is not read as it is
 cudaError_t launch_backward_umma(int dtype, bool broadcast_stage, const BwdCall& c, cudaStream_t st);
 
 }  // namespace aa

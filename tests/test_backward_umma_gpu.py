@@ -2,6 +2,7 @@
 import pytest
 
 from paper_2312_08874_b200 import AA_PATH_AUTO, Workload, make_inputs
+from tests.parity_util import make_module
 from tests.test_backward_gpu import check, run_both
 
 pytestmark = pytest.mark.gpu
@@ -15,6 +16,7 @@ SHAPES = [
     (75, 2, 15, 20, 5, "bf16", True),     # more slabs than blocks: runs that start and end inside a slab
     (50, 3, 7, 7, 7, "f16", True),        # runs of several slabs of one ragged tile
     (1, 1, 61, 83, 7, "f16", True),       # several blocks per slab
+    (2, 2, 33, 32, 4, "bf16", True),      # 16 agents: B2 is read as it is, rows of 32 bytes; B1 with a row of agents in use past 1024 tokens
 ]
 
 
@@ -25,3 +27,13 @@ def test_tiles_and_runs_match_oracle(case):
     mod, got, ref = run_both(w, make_inputs(w, bias_std=0.5, dwc_std=0.2), path=AA_PATH_AUTO)
     check(got, ref, str(case), tc=True)
     assert mod.last_launch_count() == (7 if H * W > 1024 else 6), "expected the tensor-memory gradient kernels"
+
+
+@pytest.mark.parametrize("pool,copies", [(3, 2), (8, 1)], ids=["p3", "p8"])
+def test_workspace_holds_biases_as_wide_as_their_agents(pool, copies):
+    """Copies of the biases have rows of n agents rounded up to 8 (16 bytes), and B2 none where its rows are that already.  Beside them: four
+    fp32 words per agent and channel and the partial states of V_A, one 35 KB state per tile run, at most as many as blocks and slabs."""
+    w = Workload("ws", 1, 8, 256, 256, 64, pool, "bf16", True, True, 1.0)
+    mod, n = make_module(w), pool * pool
+    rows = 8 * 65536 * ((n + 7) // 8 * 8) * 2
+    assert mod.lib.agent_attn_backward_workspace_bytes(mod._h, 256, 256, n) <= copies * rows + (8 << 20)
