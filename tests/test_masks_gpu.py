@@ -20,6 +20,8 @@ SHAPES = [
     (1, 2, 14, 14, 64, 7, "bf16", AA_PATH_QUEUE),     # task queue
     (1, 1, 64, 96, 64, 16, "bf16", AA_PATH_AUTO),     # tensor memory: every agent group of a step closed
     (1, 1, 96, 96, 40, 12, "f16", AA_PATH_AUTO),      # the same, half-filled blocks
+    (48, 1, 14, 14, 64, 7, "f32", AA_PATH_AUTO),      # terms, a warp for all agents of 16 tokens (the first two shapes have two)
+    (2, 2, 50, 50, 32, 9, "f32", AA_PATH_AUTO),       # the same, two blocks closed
 ]
 IDS = [f"{c[6]}_{c[2]}x{c[3]}_d{c[4]}_p{c[5]}_path{c[7]}" for c in SHAPES]
 
@@ -50,11 +52,18 @@ BACKWARD = [
     (1, 1, 24, 24, 64, 12, "bf16", AA_PATH_AUTO),
     (2, 2, 14, 14, 64, 7, "bf16", AA_PATH_AUTO),
     (2, 1, 14, 14, 64, 7, "bf16", AA_PATH_SIMT),
+    # agent values on tensor memory: halves of a row, tiles and whole runs without a key
+    (1, 1, 61, 83, 64, 7, "bf16", AA_PATH_AUTO),      # two rows per agent, N odd: B1 by token rows
+    (1, 1, 61, 83, 64, 7, "f16", AA_PATH_AUTO),
+    (1, 2, 40, 40, 64, 7, "bf16", AA_PATH_AUTO),      # B1 by agent rows
+    (1, 1, 40, 41, 40, 7, "bf16", AA_PATH_AUTO),      # the same with three terms
+    (1, 1, 105, 79, 64, 11, "bf16", AA_PATH_AUTO),    # one block of 128 rows
+    (2, 1, 64, 43, 64, 13, "bf16", AA_PATH_AUTO),     # two
 ]
 
 
 @pytest.mark.parametrize("value", ["inf", "lowest"])
-@pytest.mark.parametrize("case", BACKWARD, ids=[f"{c[6]}_{c[2]}x{c[3]}_p{c[5]}_path{c[7]}" for c in BACKWARD])
+@pytest.mark.parametrize("case", BACKWARD, ids=[f"{c[6]}_{c[2]}x{c[3]}_d{c[4]}_p{c[5]}_path{c[7]}" for c in BACKWARD])
 def test_masked_backward_matches_oracle(case, value):
     w, inp = masked(case, value)
     _, got, ref = run_both(w, inp, path=case[7])
