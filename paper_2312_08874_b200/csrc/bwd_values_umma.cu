@@ -357,20 +357,25 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_values_umma_kernel(const __gr
     if (warp == 0) tmem_dealloc<512>(pp.tmem);
 }
 
-// One warp per (slab, agent): V_A from the partial states, in fp32 and as TM terms, and the log2-sum-exp of its row.
-template <typename T, int TM>
+// V_A from the partial states, in fp32 and as TM terms, and the log2-sum-exp of its row: one warp per (slab, agent), or (WARPS = 8) a block,
+// whose warps take the states in turn.
+template <typename T, int TM, int WARPS>
 __global__ void __launch_bounds__(256) bwd_values_merge_kernel(const float* states, float* va, T* terms, float2* stats, int slabs, int n, int d, int tiles, int blocks, int parts, int lanes, int stack) {
-    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    __shared__ float s_max[WARPS], s_tot[WARPS];
+    __shared__ float2 s_sum[WARPS][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, w0 = WARPS > 1 ? warp : 0;
+    const int row = WARPS > 1 ? blockIdx.x : blockIdx.x * 8 + warp;
     pdl_wait_prior();
     pdl_release_next();
     if (row >= slabs * n) return;
     const int slab = row / n, a = row - slab * n, rb = stack ? 0 : a >> 7, r = stack ? a : a & 127;
     const long long total = (long long)slabs * tiles, t0 = (long long)slab * tiles;
     const int have = owner(t0 + tiles - 1, lanes, total) - owner(t0, lanes, total) + 1, subs = stack ? 2 : 1;
-    const int cnt = have * subs;                                       // partial states of the row: a lane each, 32 at a time
+    // partial states of the row, the warp's own: a lane each, 32 at a time
+    const int cnt = (have * subs - w0 + WARPS - 1) / WARPS;
     const float* st = states + ((size_t)slab * parts * blocks + rb) * kState;
-    auto at = [&](int q) { return st + (size_t)(stack ? q >> 1 : q) * blocks * kState; };
-    auto sub_row = [&](int q) { return stack ? r + 64 * (q & 1) : r; };
+    auto at = [&](int q) { return st + (size_t)(stack ? (q * WARPS + w0) >> 1 : q * WARPS + w0) * blocks * kState; };
+    auto sub_row = [&](int q) { return stack ? r + 64 * ((q * WARPS + w0) & 1) : r; };
     auto head = [&](int q) {                                           // (reference, sum); nothing counts: (-inf, 0)
         float2 v = make_float2(-INFINITY, 0.f);
         if (q < cnt) {
@@ -387,6 +392,12 @@ __global__ void __launch_bounds__(256) bwd_values_merge_kernel(const float* stat
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
+    if (WARPS > 1) {
+        s_max[w0] = mm;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < WARPS; ++w) mm = fmaxf(mm, s_max[w]);
+    }
     float tot = 0.f;
     float2 o = make_float2(0.f, 0.f);
     for (int q0 = 0; q0 < cnt; q0 += 32) {
@@ -402,6 +413,17 @@ __global__ void __launch_bounds__(256) bwd_values_merge_kernel(const float* stat
     }
 #pragma unroll
     for (int k = 16; k; k >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, k);
+    if (WARPS > 1) {
+        s_tot[w0] = tot;
+        s_sum[w0][lane] = o;
+        __syncthreads();
+        if (w0 > 0) return;
+#pragma unroll
+        for (int w = 1; w < WARPS; ++w) {
+            tot += s_tot[w];
+            o = fadd2(o, s_sum[w][lane]);
+        }
+    }
     const float inv = 1.f / tot;
     if (lane == 0) stats[row].x = mm + log2f(tot);
     if (2 * lane >= d) return;
@@ -435,8 +457,12 @@ template <typename T, int TA, int TP, bool STACK> cudaError_t launch(const Args&
     if (e != cudaSuccess) return e;
     return launch_dependent(bwd_values_umma_kernel<T, TA, TP, STACK>, dim3(grid), kThreads, kSmem<TA>, st, a);
 }
+// A warp goes through about five states in a microsecond, so a block takes a row that may have more than sixteen (whole pass, 49 agents of
+// 64 channels, one slab: of 16384 tokens 127 -> 61 us, of 3136 tokens 47 -> 34; two slabs of 1640: 40.5 -> 34).
 template <typename T, int TM> cudaError_t merge(const Args& a, const Plan& v, float* va, void* terms, float2* stats, cudaStream_t st) {
-    return launch_dependent(bwd_values_merge_kernel<T, TM>, dim3((a.slabs * a.n + 7) / 8), 256, 0, st, (const float*)a.state, va, static_cast<T*>(terms), stats, a.slabs, a.n, a.d, v.tiles, v.blocks, v.parts, v.lanes, v.stack);
+    const bool wide = (v.parts << v.stack) > 16;
+    const int rows = a.slabs * a.n;
+    return launch_dependent(wide ? bwd_values_merge_kernel<T, TM, 8> : bwd_values_merge_kernel<T, TM, 1>, dim3(wide ? rows : (rows + 7) / 8), 256, 0, st, (const float*)a.state, va, static_cast<T*>(terms), stats, a.slabs, a.n, a.d, v.tiles, v.blocks, v.parts, v.lanes, v.stack);
 }
 
 }  // namespace

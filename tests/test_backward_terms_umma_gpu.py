@@ -19,6 +19,8 @@ SHAPES = [
     (1, 1, 33, 32, 40, 7, "bf16", True),      # agent values on tensor memory: two rows per agent, a token past a multiple of eight tiles
     (1, 2, 105, 79, 64, 11, "bf16", True),    # one block of 128 agents, N and n odd: both biases are padded
     (3, 2, 64, 43, 64, 13, "bf16", False),    # two blocks, runs that hold parts of two slabs
+    (1, 1, 70, 41, 64, 9, "bf16", True),      # agent values: 24 states a row, three for a warp
+    (1, 2, 64, 65, 40, 6, "bf16", True),      # two rows per agent, 66 states, slabs that begin inside a run
 ]
 
 
