@@ -461,7 +461,7 @@ bool plan_backward(int slabs, int n, int N, int d, int sm_count, BwdPlan* out) {
 
 int backward_launch_count(const BwdCall& c) {
     const int N = c.H * c.W;
-    const bool umma = c.ws_mixed || (c.ws_terms && backward_terms_umma_eligible(c.dtype, c.n, N, c.d));
+    const bool umma = c.ws_mixed || (c.ws_terms && backward_terms_umma_eligible(c.dtype, c.slabs, c.n, N, c.d));
     const int values = umma && backward_values_eligible(c.slabs, c.n, N);
     return (c.ws_mixed ? 4 + values : !c.ws_terms ? 7 : umma ? 6 + values + (c.n > 64) : 8) + 1 + (c.wd ? 1 : 0);
 }

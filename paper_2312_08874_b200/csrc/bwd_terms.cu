@@ -205,7 +205,7 @@ bool backward_terms_eligible(int dtype, int n, int d) {
     return 6 * n32 * pitch + n32 * 8 <= 227 * 1024;
 }
 size_t backward_terms_bytes(int dtype, int slabs, int heads, int n, int N, int d, int sm_count) {
-    return (backward_terms_umma_eligible(dtype, n, N, d) ? backward_terms_umma_bytes(slabs, heads, n, N) + backward_values_bytes(slabs, n, N, sm_count) : 0) + 3 * up256((size_t)slabs * n * d * 2 * 3) + up256((size_t)slabs * N * 8) + up256((size_t)slabs * n * 8);
+    return (backward_terms_umma_eligible(dtype, slabs, n, N, d) ? backward_terms_umma_bytes(slabs, heads, n, N) + backward_values_bytes(slabs, n, N, sm_count) : 0) + 3 * up256((size_t)slabs * n * d * 2 * 3) + up256((size_t)slabs * N * 8) + up256((size_t)slabs * n * 8);
 }
 
 cudaError_t launch_backward_mixed_forward(int dtype, const BwdCall& c, cudaStream_t st) {
@@ -243,7 +243,7 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
     cudaError_t e;
 #define AA_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
     const bool clear_bias = slabs != c.heads;          // (a single batch entry stores its bias gradients)
-    const bool umma = backward_terms_umma_eligible(dtype, n, N, d), clear_rows = umma && n > 64;      // (blocks of 64 agents add to the rows)
+    const bool umma = backward_terms_umma_eligible(dtype, slabs, n, N, d), clear_rows = umma && n > 64;      // (blocks of 64 agents add to the rows)
     void *pad1 = nullptr, *pad2 = nullptr, *partial = nullptr;
     char* umma_ws = w + 3 * terms + up256((size_t)slabs * N * 8) + up256((size_t)slabs * n * 8);          // padded biases, partial states of V_A
     if (umma) backward_terms_umma_padded(c.heads, n, N, umma_ws, &pad1, &pad2, &partial);

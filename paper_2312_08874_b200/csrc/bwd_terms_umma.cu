@@ -568,9 +568,21 @@ template <int MODE> cudaError_t launch(const Args& a, int sm_count, cudaStream_t
 
 }  // namespace
 
-// Faster than the mma.sync kernels on every shape of a sweep from 147 tokens x 9 agents (61 -> 57 us) to 16384 x 256.
-// (One agent or one token: a softmax over it has no gradient, which the recomputed products give exactly only where both passes agree)
-bool backward_terms_umma_eligible(int dtype, int n, int N, int d) { return dtype == kBF16 && d <= 64 && d % 8 == 0 && n > 1 && n <= 256 && N > 1; }
+// One agent or one token: a softmax over it has no gradient, which the recomputed products give exactly only where both passes agree.
+// A unit costs 64 agents of 64 channels whatever there are.  More than 32 agents are faster here than on mma.sync (some hundred shapes of 49
+// to 16384 tokens, whole pass: 0.33 to 1.05 times as long, the latter at 49 tokens).  Up to 32, one block of agents there, they are where
+// agents or channels fill the unit and tokens the chip, or where the token axis is long, or (lines of few agents) a large batch has short
+// slabs.  mma.sync -> here: 16 slabs of 196 tokens, 25 agents of 32 channels 42 -> 47 us, 48 slabs of 3136, 16 agents of 40 channels 214 -> 242;
+// but 192 slabs of 196, 25 agents of 40 channels 122 -> 104, one slab of 16384, 9 agents of 40 channels 129 -> 116, 16 slabs of 1023, 25 agents
+// of 56 channels 74 -> 66.
+bool backward_terms_umma_eligible(int dtype, int slabs, int n, int N, int d) {
+    if (dtype != kBF16 || d > 64 || d % 8 || n < 2 || n > 256 || N < 2) return false;
+    if (n > 32) return true;
+    const long long tokens = (long long)slabs * N;
+    if (d > 48) return n > 16 ? N >= 196 || tokens >= 9000 : N >= 1024 || tokens >= 16000;
+    if (d > 32) return n > 16 ? N >= 1024 || tokens >= 28000 : N >= 8192 || (N <= 512 && tokens >= 28000);
+    return n > 16 && (N >= 8192 || (N <= 256 && tokens >= 28000));
+}
 
 size_t backward_terms_umma_bytes(int slabs, int heads, int n, int N) {
     return (N % 8 ? padded_bias_bytes(heads, n, N) : 0) + (n % 8 ? padded_bias_bytes(heads, n, N) : 0) + (n > 64 ? (size_t)((n + 63) / 64) * slabs * N * 16 : 0);

@@ -280,7 +280,7 @@ bool backward_terms_eligible(int dtype, int n, int d);
 size_t backward_terms_bytes(int dtype, int slabs, int heads, int n, int N, int d, int sm_count);
 cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStream_t st);
 // the gradient stages of that on the 5th-generation tensor cores (bf16 inputs of up to 64 channels)
-bool backward_terms_umma_eligible(int dtype, int n, int N, int d);
+bool backward_terms_umma_eligible(int dtype, int slabs, int n, int N, int d);
 enum BwdTermsUmma { kUmmaStats, kUmmaBroadcast, kUmmaAggregate };
 // Workspace: biases as token rows (null where they are read as they are), token statistics per block of agents
 size_t backward_terms_umma_bytes(int slabs, int heads, int n, int N);

@@ -9,7 +9,8 @@ pytestmark = pytest.mark.gpu
 
 SHAPES = [
     # batch heads H   W   d  pool dtype bias
-    (1, 1, 2, 63, 32, 2, "bf16", True),       # two tokens short of a tile, few agents
+    (140, 1, 2, 63, 56, 2, "bf16", True),     # two tokens short of a tile, few agents
+    (1, 1, 96, 87, 32, 5, "bf16", True),      # 25 agents of 32 channels on a long axis
     (2, 1, 8, 16, 40, 6, "bf16", True),       # exactly one tile, agents in both halves, ragged channels
     (1, 3, 9, 43, 64, 9, "bf16", True),       # a batch of one: bias gradients are stored; odd rows of both biases
     (2, 2, 16, 16, 64, 16, "bf16", False),    # four full blocks of agents, two full tiles, no bias
@@ -32,6 +33,26 @@ def test_tiles_and_agent_blocks_match_oracle(case):
     check(got, ref, str(case))
     values = H * W > 1024 or (pool > 8 and B * heads * H * W >= 16384)
     assert mod.last_launch_count() == 8 + (pool > 8) + values, "expected the tensor-memory gradient kernels"
+
+
+# both sides of the lines between these kernels (8 launches, 9 past 1024 tokens) and those on mma.sync (10) for up to 32 agents
+LINES = [
+    # batch heads H   W   d  pool launches
+    (1, 1, 13, 15, 56, 5, 10), (1, 1, 14, 14, 56, 5, 8), (30, 2, 10, 15, 56, 5, 8),
+    (1, 1, 33, 31, 56, 3, 10), (1, 1, 32, 32, 56, 3, 8), (16, 4, 10, 25, 56, 4, 8),
+    (1, 1, 33, 31, 40, 5, 10), (1, 1, 32, 32, 48, 5, 8), (50, 4, 14, 10, 40, 5, 8),
+    (1, 1, 91, 90, 40, 4, 10), (1, 1, 64, 128, 40, 3, 9), (56, 1, 20, 25, 48, 2, 8), (50, 1, 27, 21, 40, 3, 10),
+    (1, 1, 2, 63, 32, 2, 10), (1, 1, 91, 90, 32, 5, 10), (1, 1, 64, 128, 32, 5, 9), (1, 1, 64, 128, 32, 4, 10), (110, 1, 16, 16, 24, 5, 8), (105, 1, 16, 17, 32, 5, 10),
+]
+
+
+@pytest.mark.parametrize("case", LINES, ids=[f"B{c[0]}h{c[1]}_{c[2]}x{c[3]}_d{c[4]}_p{c[5]}" for c in LINES])
+def test_lines_between_both_paths(case):
+    B, heads, H, W, d, pool, launches = case
+    w = Workload("lines", B, heads, H, W, d, pool, "bf16", True, True, 1.0, seed=970 + H * W + pool)
+    mod, got, ref = run_both(w, make_inputs(w, bias_std=0.5, dwc_std=0.2), path=AA_PATH_AUTO)
+    check(got, ref, str(case))
+    assert mod.last_launch_count() == launches
 
 
 @pytest.mark.parametrize("case", [(2, 2, 64, 64, 64, 9), (3, 2, 20, 20, 64, 9), (4, 2, 28, 28, 40, 5)], ids=["values_umma", "sums_n81", "sums_d40"])
