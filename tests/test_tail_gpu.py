@@ -1,4 +1,4 @@
-"""Token-wise tail of the backward pass (pooling, depthwise and filter gradients) at the edges of its tiles, against the fp64 oracle."""
+"""Token-wise tail of the backward pass (pooling, depthwise and filter gradients) at the edges of its strips and blocks, against the fp64 oracle."""
 import pytest
 import torch
 
@@ -10,12 +10,12 @@ pytestmark = pytest.mark.gpu
 
 SHAPES = [
     # batch heads H   W   d   pool dtype
-    (1, 1, 3, 131, 40, 3, "bf16"),        # W one past the single-run halo, channels padded from 40 to 48
-    (1, 2, 5, 300, 64, 5, "f16"),         # the halo in three runs, unequal windows
-    (2, 1, 130, 9, 104, 4, "bf16"),       # seven channel groups
-    (3, 1, 8, 16, 16, 2, "f16"),          # exactly one tile, one channel group
-    (1, 1, 43, 3, 8, 3, "bf16"),          # one token past a tile, half a channel group
-    (160, 2, 9, 15, 80, 3, "bf16"),       # more slabs than resident blocks
+    (1, 1, 3, 131, 40, 3, "bf16"),        # six columns at once (eight threads idle), the last group short
+    (1, 2, 5, 300, 64, 5, "f16"),         # many columns of few rows, unequal windows
+    (2, 1, 130, 9, 104, 4, "bf16"),       # several strips of rows, two columns at once (24 threads idle)
+    (3, 1, 8, 16, 16, 2, "f16"),          # every column of the grid at once, exactly
+    (1, 1, 43, 3, 8, 3, "bf16"),          # more columns at once than the grid has
+    (160, 2, 9, 15, 80, 3, "bf16"),       # blocks that go through several batch entries of their head
     (2, 2, 30, 41, 128, 6, "f16"),
 ]
 
