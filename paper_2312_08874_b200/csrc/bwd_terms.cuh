@@ -90,6 +90,16 @@ template <typename E, int NT> __device__ __forceinline__ void split_pair(float a
         }
     }
 }
+// the same, residuals by packed arithmetic (FINITE: the values may be past the largest E)
+template <typename E, int NT, bool FINITE = true> __device__ __forceinline__ void split_pair(float2 v, uint32_t (&w)[NT]) {
+    w[0] = FINITE ? pack2_finite<E>(v.x, v.y) : pack2<E>(v.x, v.y);
+#pragma unroll
+    for (int i = 1; i < NT; ++i) {
+        v = ffma2(unpack2<E>(w[i - 1]), make_float2(-1.f, -1.f), v);
+        w[i] = pack2<E>(v.x, v.y);
+    }
+}
+__device__ __forceinline__ void bar_named(int id, int threads) { asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory"); }
 __device__ __forceinline__ void red_add4(float* p, float a, float b, float c, float d) {
     asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};\n" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
@@ -801,7 +811,7 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
                     mine[(CUT * 4 + h) * 32] = m[h];
                     mine[(CUT * 4 + 2 + h) * 32] = l[h];
                 }
-                asm volatile("bar.sync %0, 64;\n" ::"r"(1 + group) : "memory");
+                bar_named(1 + group, 64);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const float om = other[(CUT * 4 + h) * 32], ol = other[(CUT * 4 + 2 + h) * 32], mm = fmaxf(m[h], om), base = mm == -INFINITY ? 0.f : mm;
@@ -813,7 +823,7 @@ __global__ void __launch_bounds__(256, 1) bwd_rows_kernel(const __grid_constant_
 #pragma unroll
                             for (int e = 0; e < 2; ++e) o0[j][2 * h + e] = o0[j][2 * h + e] * f + other[((j >= CUT ? j - CUT : j) * 4 + 2 * h + e) * 32] * fo;
                 }
-                asm volatile("bar.sync %0, 64;\n" ::"r"(1 + group) : "memory");
+                bar_named(1 + group, 64);
             }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {

@@ -90,21 +90,6 @@ struct Args {
     alignas(64) CUtensorMap tm_x, tm_y, tm_a, tm_m, tm_b;
 };
 
-__device__ __forceinline__ uint64_t desc_mn(uint32_t addr, uint32_t lead) {       // MN-major operand: two tiles of 64, `lead` bytes apart
-    return (umma_desc_sw128(addr) & ~((uint64_t)0x3fffu << 16)) | ((uint64_t)(lead >> 4) << 16);
-}
-// 16 lanes x 64 fp32 columns in mma.sync accumulator layout: r[4 j + 2 h + e] = (row g + 8 h, column 8 j + 2 t + e)
-__device__ __forceinline__ void tmem_ld_16x256b_x8(uint32_t taddr, float (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
-        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]),
-          "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15]),
-          "=f"(r[16]), "=f"(r[17]), "=f"(r[18]), "=f"(r[19]), "=f"(r[20]), "=f"(r[21]), "=f"(r[22]), "=f"(r[23]),
-          "=f"(r[24]), "=f"(r[25]), "=f"(r[26]), "=f"(r[27]), "=f"(r[28]), "=f"(r[29]), "=f"(r[30]), "=f"(r[31])
-        : "r"(taddr) : "memory");
-}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
@@ -136,16 +121,6 @@ __device__ __forceinline__ void load_joined(uint32_t taddr, float2 (&v)[16]) {
 __device__ __forceinline__ void st_shared4(uint32_t addr, const uint32_t (&v)[4]) {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
 }
-// split_pair of three bf16 terms, the residuals by packed arithmetic
-__device__ __forceinline__ void split3(float2 v, uint32_t (&w)[kTerms]) {
-    w[0] = pack2_finite<__nv_bfloat16>(v.x, v.y);
-#pragma unroll
-    for (int i = 1; i < kTerms; ++i) {
-        v = ffma2(unpack2<__nv_bfloat16>(w[i - 1]), make_float2(-1.f, -1.f), v);
-        w[i] = pack2<__nv_bfloat16>(v.x, v.y);
-    }
-}
-
 template <int MODE>
 __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __grid_constant__ Args p) {
     constexpr bool BCAST = MODE == kBcast, AGG = MODE == kAgg, STATS = MODE == kStats;
@@ -402,7 +377,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
             } else if (AGG && (i == 0 || tile == 0)) {                 // another slab: its statistics
                 parity ^= 1;
                 if (tid < 64) s_stat[parity * 64 + tid] = ab * 64 + tid < n ? __ldg(p.stats + (size_t)slab * n + ab * 64 + tid) : none;
-                asm volatile("bar.sync 1, %0;\n" ::"n"(kRowThreads) : "memory");
+                bar_named(1, kRowThreads);
             }
             wait_par(pp, BAR_S, i, kTimeoutTile);
             tc_fence_after_sync();
@@ -438,7 +413,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
                 const float l = l2.x + l2.y, dot = d2.x + d2.y;
                 float4* ex = reinterpret_cast<float4*>(smem + OFF_EX) + b * 256;
                 if (half) ex[r] = make_float4(m, l, dot, 0.f);
-                asm volatile("bar.sync %0, 64;\n" ::"r"(2 + q) : "memory");
+                bar_named(2 + q, 64);
                 if (!half && ok) {
                     const float4 o = ex[r];
                     const float mm = fmaxf(m, o.x), f = m == -INFINITY ? 0.f : exp2f(m - mm), fo = o.x == -INFINITY ? 0.f : exp2f(o.x - mm);
@@ -472,10 +447,10 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     uint32_t w[kTerms];
-                    split3(pr[4 * c + k], w);
+                    split_pair<__nv_bfloat16, kTerms>(pr[4 * c + k], w);
 #pragma unroll
                     for (int t = 0; t < kTerms; ++t) u[t][k] = w[t];
-                    split3(ds[4 * c + k], w);
+                    split_pair<__nv_bfloat16, kTerms>(ds[4 * c + k], w);
 #pragma unroll
                     for (int t = 0; t < kTerms; ++t) v[t][k] = w[t];
                 }

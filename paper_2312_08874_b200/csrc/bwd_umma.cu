@@ -75,24 +75,6 @@ struct UmmaArgs {
     alignas(64) CUtensorMap tm_x, tm_y, tm_a, tm_m, tm_b;
 };
 
-// MN-major operand of 128 rows: two tiles of 64, `lead` bytes apart
-__device__ __forceinline__ uint64_t desc_mn(uint32_t addr, uint32_t lead) {
-    return (umma_desc_sw128(addr) & ~((uint64_t)0x3fffu << 16)) | ((uint64_t)(lead >> 4) << 16);
-}
-// 16 lanes x 64 fp32 columns in mma.sync accumulator layout: r[4 j + 2 h + e] = (row g + 8 h, column 8 j + 2 t + e)
-__device__ __forceinline__ void tmem_ld_16x256b_x8(uint32_t taddr, float (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
-        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]),
-          "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15]),
-          "=f"(r[16]), "=f"(r[17]), "=f"(r[18]), "=f"(r[19]), "=f"(r[20]), "=f"(r[21]), "=f"(r[22]), "=f"(r[23]),
-          "=f"(r[24]), "=f"(r[25]), "=f"(r[26]), "=f"(r[27]), "=f"(r[28]), "=f"(r[29]), "=f"(r[30]), "=f"(r[31])
-        : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void bar_named(int id, int threads) { asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory"); }
-
 template <typename T, bool BCAST>
 __global__ void __launch_bounds__(kThreads, 1) bwd_umma_kernel(const __grid_constant__ UmmaArgs p) {
     extern __shared__ unsigned char smem_raw[];

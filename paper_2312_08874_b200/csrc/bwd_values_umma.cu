@@ -77,7 +77,7 @@ struct Args {
 // run (of `lanes`) that holds tile x of `total`
 __host__ __device__ inline int owner(long long x, long long lanes, long long total) {
     const unsigned long long v = (unsigned long long)(x + 1) * lanes - 1;
-    return v >> 32 ? (int)(v / total) : (int)((uint32_t)v / (uint32_t)total);         // (v < total * lanes: total fits where v does)
+    return (v | (unsigned long long)total) >> 32 ? (int)(v / total) : (int)((uint32_t)v / (uint32_t)total);
 }
 
 // 8 consecutive columns of this thread's tensor-memory row <- registers
@@ -85,16 +85,6 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8])
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]),
                  "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
 }
-// split_pair, the residuals by packed arithmetic
-template <typename T, int NT> __device__ __forceinline__ void split_terms(float2 v, uint32_t (&w)[NT]) {
-    w[0] = pack2<T>(v.x, v.y);
-#pragma unroll
-    for (int i = 1; i < NT; ++i) {
-        v = ffma2(unpack2<T>(w[i - 1]), make_float2(-1.f, -1.f), v);
-        w[i] = pack2<T>(v.x, v.y);
-    }
-}
-
 template <typename T, int TA, int TP, bool STACK>
 __global__ void __launch_bounds__(kThreads, 1) bwd_values_umma_kernel(const __grid_constant__ Args p) {
     constexpr int kFmt = Elem<T>::kIsBf16 ? 1 : 0, kCols = STACK ? 32 : 64, kD = TP == 2 ? 2 : 1;
@@ -311,7 +301,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_values_umma_kernel(const __gr
             for (int j = 1; j < kCols / 2; ++j) m = max3(m, s[j].x, s[j].y);
             tc_fence_before_sync();
             ex[(b * 2 + half) * 128 + r] = m;
-            asm volatile("bar.sync %0, 64;\n" ::"r"(1 + q) : "memory");
+            bar_named(1 + q, 64);
             if (lane == 0) {                                           // (every lane's loads have been consumed before the barrier)
                 pipe_arrive(pp, BAR_READ + b);
                 if (p.bias) pipe_arrive(pp, BAR_BREAD + b);
@@ -337,7 +327,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_values_umma_kernel(const __gr
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     uint32_t w[TP];
-                    split_terms<T, TP>(s[8 * g + k], w);
+                    split_pair<T, TP, false>(s[8 * g + k], w);              // (at most one, or NaN)
 #pragma unroll
                     for (int t = 0; t < TP; ++t) u[t][k] = w[t];
                 }
