@@ -163,9 +163,11 @@ typedef struct {
     void* dwd;                /* [heads][d][3][3], or NULL: gradient of the depthwise filter */
 } agent_attn_grads;
 
-/* Bytes of device workspace agent_attn_backward needs (fp32 copies of A, V_A, dV_A, dA, the row
- * statistics of the aggregation softmax and its per-block partial states).  0 on invalid arguments
- * or an unsupported shape. */
+/* Bytes of device workspace agent_attn_backward needs: A, V_A, dV_A and dA in fp32 (and as 16-bit
+ * terms), softmax statistics, sixteen copies of the filter gradient, partial states of V_A, and
+ * copies of biases whose rows are no multiple of 16 bytes (reserved whether or not a call has
+ * biases; B1 for 16-bit types with n_agents <= 64 and head_dim == 64 in any case).  0 on invalid
+ * arguments or an unsupported shape. */
 size_t agent_attn_backward_workspace_bytes(const agent_attn_handle* h, int grid_h, int grid_w, int n_agents);
 
 /* Gradients of Eq. 6 with pooled agents (A = Pooling(Q), so dQ includes the path through the agents):

@@ -330,7 +330,7 @@ cudaError_t launch_terms_forward(const TermsForward& c, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     a.x = c.q; a.y = c.v; a.bias = c.b2; a.scale = c.scale2; a.m_t = w + terms; a.row0 = c.out; a.wd = c.wd;
     // Fewer groups of 16 tokens than schedulers: two warps each (3 slabs of 196 tokens, 49 agents: whole pass
-    // 25.6 -> 23.4 us; 6 of 1200, 196 agents: 75 -> 68; 2 of 3000, 81 agents of 80 channels: 61 -> 55)
+    // 25.6 -> 22.9 us; 6 of 1200, 196 agents: 75 -> 68; 2 of 3000, 81 agents of 80 channels: 61 -> 55)
     const int dk = dk_of_terms(c.d), n32 = (c.n + 31) & ~31;
     const bool split = c.n > 32 && (long long)c.slabs * ((N + 15) / 16) <= 4 * c.sm_count && 6 * n32 * (dk * 2 + 16) + 10 * dk * 4 + 8 * ((dk / 16 + 1) / 2 * 8 + 4) * 128 <= 227 * 1024;
     parts = token_parts(c.slabs, N, 16, split ? 64 : 128, 512, false, c.sm_count);

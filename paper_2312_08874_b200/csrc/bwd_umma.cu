@@ -17,11 +17,12 @@
 //               D and the terms of dV_A.
 //   warp 12     TMA: X, Y and the bias as token rows, two stages of 48 KB.
 //   warp 13, 14 issue S and dP (a tile ahead), and the products of P and dS.
-// The sums of both halves are one 128-row operand [P | dS] against [X | Y]: eight instructions of 128 columns, of whose four blocks two
-// are used; as four products of 64 x 64 they would be sixteen.
+// Broadcast: the sums of both halves are one 128-row operand [P | dS] against [X | Y], eight instructions of 128 columns, of whose four
+// blocks two are used; as two products of 64 x 64 they would be sixteen.  (Aggregation: against X alone, 64 columns.)
 //
-// What bounds it: the chain load -> logits -> softmax -> products -> stage free through two stages (tensor pipe about 0.8 us of it per tile),
-// and HBM: 64 slabs of a 56 x 56 grid, 49 agents: broadcast 36 us (103 MB, 16 us at the copy bandwidth), aggregation 41 us (154 MB, 24 us).
+// What bounds it: the chain load -> logits -> softmax -> products -> stage free through two stages, and HBM: 64 slabs of a 56 x 56 grid, 49
+// agents (by ncu, cold caches): broadcast 40 us (103 MB, 16 us at the copy bandwidth), aggregation 47 us (154 MB, 24 us, and the start: D and
+// the terms of dV_A); tensor pipe 17 and 13 %, issue 32 and 30 %.
 // With mma.sync, 64-token tiles and scalar bias loads and reductions the two took 96 and 93 us.
 #include "bwd_terms.cuh"
 #include "stream_common.cuh"
