@@ -563,7 +563,7 @@ static int forward_impl(agent_attn_handle* h, const void* Q, const void* K, cons
         h->launches = 3;
         return AA_OK;
     }
-    if (!use_simt(h) && !(use_umma(h, N, n_agents) && (!cl.strided || tok_map_exists(cl.in, h->cfg.batch, h->cfg.heads, N)))) {
+    if (!use_simt(h) && !(use_umma(h, N, n_agents) && (!cl.strided || tok_grid_exists(cl.in, h->cfg.batch, h->cfg.heads, grid_h, grid_w)))) {
         TileArgs t = tile_args(h, grid_h, grid_w, n_agents, cl);
         t.q = Q; t.k = K; t.v = V; t.a = A ? A : ws + w.a_off; t.va = ws + w.va_off; t.pool = p;
         t.b1 = b1; t.b2 = b2; t.wd = dwc_weight; t.out = out;

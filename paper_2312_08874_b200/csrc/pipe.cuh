@@ -40,6 +40,12 @@ __device__ __forceinline__ void pipe_arrive(const Pipe& pp, int i) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(pipe_bar(pp, i)) : "memory");
 }
 
+// One arrival for a warp whose lanes have all done their part
+__device__ __forceinline__ void pipe_arrive_warp(const Pipe& pp, int i, int lane) {
+    __syncwarp();
+    if (lane == 0) pipe_arrive(pp, i);
+}
+
 // 32 consecutive fp32 columns of this thread's tensor-memory row <- registers
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
     asm volatile(
@@ -52,6 +58,9 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
           "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
         : "memory");
 }
+// Registers of a warp group's threads from here on; what others give up must cover what some take (the block's total at launch).
+template <int R> __device__ __forceinline__ void set_regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(R)); }
+template <int R> __device__ __forceinline__ void set_regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(R)); }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
 
 }  // namespace aa

@@ -16,6 +16,12 @@ __device__ __forceinline__ uint32_t tmem_ld1(uint32_t taddr) {
 }
 
 // 16 consecutive fp32 columns of this thread's tensor-memory row <- registers
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
+        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]),
+          "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15]) : "r"(taddr) : "memory");
+}
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
@@ -147,19 +153,19 @@ inline bool make_map_rows3d_u16(CUtensorMap* out, const void* base, uint64_t zs,
               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Host: map of the token grid of a tensor with layout l for tma_load_grid (64 channels, box of 64 x box_w x box_h, 128-byte swizzle).
+// Host: map of the token grid of a tensor with layout l for tma_load_grid (box of 64 x box_w x box_h, channels past d zero-filled, 128-byte swizzle).
 // The dimension order is that of make_map_tok_u16; false if the strides cannot be expressed.
-inline bool make_map_grid5d_u16(CUtensorMap* out, int head_first, const void* base, const TokLayout& l, int batch, int heads, uint64_t H, uint64_t W, uint32_t box_h, uint32_t box_w) {
+inline bool make_map_grid5d_u16(CUtensorMap* out, int head_first, const void* base, const TokLayout& l, int batch, int heads, uint64_t H, uint64_t W, uint32_t box_h, uint32_t box_w, int d = 64) {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
-    if ((reinterpret_cast<uintptr_t>(base) & 15u) || box_h > 256 || box_w > 256 || box_h < 1 || box_w < 1) return false;
-    if ((l.sb & 7) || (l.sh & 7) || (l.st & 7) || l.st < 64) return false;
+    if ((reinterpret_cast<uintptr_t>(base) & 15u) || box_h > 256 || box_w > 256 || box_h < 1 || box_w < 1 || d > 64 || d % 8) return false;
+    if ((l.sb & 7) || (l.sh & 7) || (l.st & 7) || l.st < d) return false;
     const cuuint64_t st = (cuuint64_t)l.st * 2, row = st * W;
     cuuint64_t sh = (cuuint64_t)l.sh * 2, sb = (cuuint64_t)l.sb * 2;
     if (heads == 1 && !head_first && sh < row * H) sh = row * H;             // strides of single heads or entries are never used
     const cuuint64_t last = head_first ? row * H : sh * heads;
     if (batch == 1 && sb < last) sb = last;
-    const cuuint64_t dims[5] = {64, head_first ? (cuuint64_t)heads : W, head_first ? W : H, head_first ? H : (cuuint64_t)heads, (cuuint64_t)batch};
+    const cuuint64_t dims[5] = {(cuuint64_t)d, head_first ? (cuuint64_t)heads : W, head_first ? W : H, head_first ? H : (cuuint64_t)heads, (cuuint64_t)batch};
     const cuuint64_t strides[4] = {head_first ? sh : st, head_first ? st : row, head_first ? row : sh, sb};
     for (int i = 1; i < 4; ++i)
         if (strides[i] < strides[i - 1]) return false;
