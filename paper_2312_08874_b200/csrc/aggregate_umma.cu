@@ -3,29 +3,28 @@
 //
 // Grid: (splits, slabs), one block of 19 warps per SM.  A block keeps the slab's agents resident (up to
 // two 128-row operand blocks) and streams its share of the slab's 64-token tiles (K, V and the matching
-// B1 columns) through a four-stage TMA ring.
+// B1 columns) through a four-stage TMA ring.  Two chains of eight row warps work beside one another: agents 0-127 and 128-255 of every
+// tile, or (up to 128 agents) the even and the odd tiles.  A chain's logits alternate between two buffers in tensor memory: while the
+// softmax of one tile runs, the products of the one before and the logits of the next are under way.
 //   warp 16 "producer":  one lane issues every TMA copy, ahead of the others through full/empty mbarriers.
-//   warps 17, 18 "MMA issuers": one lane each, one per agent block ("chain"): S = A_block K^T (tcgen05.mma,
-//                        accumulator in tensor memory) one tile ahead, and the products P V once the chain's
-//                        probabilities of a tile are written.  The two chains (agents 0-127, agents 128-255)
-//                        share the ring but have their own barriers, so that one computes while the other
-//                        waits for its products.
+//   warps 17, 18 "MMA issuers", one per chain: the products P V of a tile once its probabilities are written, then the logits
+//                        S = A_block K^T two tiles on over them (instructions of one thread run in their order).
 //   warps 0-15 "row warps": thread (agent row, token half): reads its 32 logits of the tile from tensor
 //                        memory, adds scale and bias, keeps its own running maximum / sum (no reduction
 //                        crosses threads: each token half has its own accumulator in tensor memory),
-//                        writes the probabilities back to shared memory as the A operand of P V, in place
-//                        of the bias values it has just read (so P needs no buffer and the ring has a
-//                        fourth stage).
-//                        A row's reference maximum moves only when exceeded by a margin; then the thread
+//                        writes the probabilities back over them as the A operand of P V.
+//                        A row's reference maximum moves only when exceeded by a margin; only then does the thread wait for products, and
 //                        rescales its accumulator row in tensor memory.
-// At the end the two token halves of a row meet in shared memory and the block writes one partial state;
+// At the end the two token halves of a row meet in shared memory and each chain (up to 128 agents), or the block, writes one partial state;
 // a second small kernel merges the slab's partials in a fixed order, spread over many blocks (a merge by
 // the slab's last block alone took longer than the streaming part).
 // Every wait is bounded (pipe.cuh).  No TMA multicast, no clusters.
-#include "common.cuh"
-#include "kernels.h"
+//
+// What bounds it: the row warps' instructions and exponentials (half of the time at the special-function rate), then HBM.  With probabilities through shared
+// memory, a wait for the products of the tile before in every tile and arrivals of single threads, 16 slabs of a 256 x 256 grid with 256
+// agents took 177 us; this way 133.
 #include "merge.cuh"
-#include "pipe.cuh"
+#include "stream_common.cuh"
 
 #include <cstring>
 
@@ -48,18 +47,18 @@ constexpr int kStage = 2 * kTile + 4 * kTile;
 constexpr int kSmemBytes = OFF_RING + STAGES * kStage + 1024;
 static_assert(kSmemBytes <= 232448 && kSmemBytes > 116 * 1024, "one block per SM");
 
-// mbarriers                                    count            waiter
-constexpr int BAR_FULL = 0;       // [STAGES]        tx             each chain's MMA issuer
-constexpr int BAR_EMPTY = 4;      // [STAGES]        one commit per chain     producer
-constexpr int BAR_S_FULL = 8;     // [chain][2]      commit         the chain's row warps
-constexpr int BAR_S_EMPTY = 12;   // [chain][2]      256 threads    the chain's MMA issuer
-constexpr int BAR_P_FULL = 16;    // [chain]         256 threads    the chain's MMA issuer
-constexpr int BAR_PV = 18;        // [chain]         commit         the chain's row warps
+// mbarriers (cb: + 2 chain + parity of the chain's tile)   count            waiter
+constexpr int BAR_FULL = 0;       // [STAGES]        tx             MMA issuers
+constexpr int BAR_EMPTY = 4;      // [STAGES]        one commit per chain that takes the tile     producer
+constexpr int BAR_S_FULL = 8;     // cb              commit         the chain's row warps
+constexpr int BAR_P_FULL = 12;    // cb              8 warps        the chain's MMA issuer        (logits and biases read as well)
+constexpr int BAR_PV = 16;        // cb              commit         the chain's row warps (where a reference moves, and at the end)
 constexpr int BAR_AG = 20;        //                 tx             both MMA issuers
-constexpr int kBars = 21;
+constexpr int BAR_DRAIN = 21;     // [chain]         commit         MMA issuer, once, at its end
+constexpr int kBars = 23;
 
-// tensor memory: logits 2 buffers x (2 agent blocks x 64), accumulators (agent block, token half) x 64
-constexpr uint32_t TM_S = 0, TM_O = 256;
+// tensor memory, columns of a chain: logits (then probabilities) of two tiles 64 each, accumulators of two token halves 64 each
+constexpr uint32_t TM_CHAIN = 256, TM_O = 128;
 
 struct UmmaAggArgs {
     AttnArgs a;
@@ -95,7 +94,7 @@ __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_cons
     if (tid == 0) {
         s_dead = 0;
         for (int i = 0; i < kBars; ++i)
-            mbar_init(pp.bars + 8 * i, (i >= BAR_S_EMPTY && i < BAR_PV) ? 256u : (i >= BAR_EMPTY && i < BAR_S_FULL) ? (uint32_t)MB : 1u);
+            mbar_init(pp.bars + 8 * i, (i >= BAR_P_FULL && i < BAR_PV) ? 8u : (i >= BAR_EMPTY && i < BAR_S_FULL) ? (uint32_t)MB : 1u);
         mbar_fence_init();
     }
     if (warp == 0) tmem_alloc<512>(smem_u32(&s_tmem));
@@ -108,7 +107,7 @@ __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_cons
 
     const uint32_t sA = smem_u32(smem + OFF_A), ring = smem_u32(smem + OFF_RING);
     const size_t pf = partial_floats(g.rows_pad, 64);
-    float* slab_parts = p.partials + (size_t)slab * gridDim.x * pf;
+    float* slab_parts = p.partials + (size_t)slab * gridDim.x * (MB == 1 ? 2 : 1) * pf;
 
     if (warp == 16) {
         // ------------------------------------------------------------------ producer
@@ -116,9 +115,9 @@ __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_cons
             mbar_arrive_expect_tx(pipe_bar(pp, BAR_AG), (uint32_t)MB * 2 * kTile);
             for (int mb = 0; mb < MB; ++mb) tma_load_2d(sA + mb * 2 * kTile, &g.tm_a, 0, slab * n + 128 * mb, pipe_bar(pp, BAR_AG));
             const uint32_t tx = 2 * kTile + (has_bias ? (uint32_t)MB * 2 * kTile : 0u);
-            for (int t = 0; t < tiles; ++t) {
+            for (int t = 0; t < tiles && !pipe_dead(pp); ++t) {
                 const int s = t % STAGES, c0 = (t0 + t) * KT;
-                if (t >= STAGES) pipe_wait_one(pp, BAR_EMPTY + s, kTimeoutRole);
+                if (t >= STAGES) wait_spin(pp, BAR_EMPTY + s, t / STAGES - 1, kTimeoutRole);
                 const uint32_t bar = pipe_bar(pp, BAR_FULL + s), dst = ring + s * kStage;
                 mbar_arrive_expect_tx(bar, tx);
                 tma_load_tok(dst, &g.tm_k, g.hf_k, c0, head, slab / p.heads, bar);
@@ -126,73 +125,67 @@ __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_cons
                 if (has_bias)
                     for (int mb = 0; mb < MB; ++mb) tma_load_2d(dst + 2 * kTile + mb * 2 * kTile, &g.tm_b, c0, head * n + 128 * mb, bar);
             }
-            for (int t = max(0, tiles - STAGES); t < tiles; ++t) pipe_wait_one(pp, BAR_EMPTY + t % STAGES, kTimeoutRole);
         }
         __syncwarp();
-    } else if (warp == 17 || warp == 18) {
-        // ------------------------------------------------------------------ MMA issuer of chain m = agent block m
-        const int m = warp - 17;
-        if (m < MB) {     // (the whole warp runs the loop; one elected lane issues)
+    } else if (warp >= 17) {
+        // ------------------------------------------------------------------ MMA issuer of a chain (the whole warp runs the loop; one elected lane issues)
+        const int m = warp - 17, first = MB == 1 ? m : 0, step = MB == 1 ? 2 : 1, count = (tiles - first + step - 1) / step;
+        if (count > 0) {
             const uint32_t idK = umma_idesc(fmt, 128, 64, 0), idMN = umma_idesc(fmt, 128, 64, 1);
-            const uint64_t dA = umma_desc_sw128(sA) + 1024 * m, dRing = umma_desc_sw128(ring);
-            // descriptor start addresses count 16-byte units: + 2 per K-step of a K-major operand (32 bytes),
-            // + 128 per K-step of an MN-major operand (16 rows of 128 bytes), + 1024 per 128-row block
-            auto issue_S = [&](int t) {
-                const int b = t & 1, s = t % STAGES;
-                if (t >= 2) pipe_wait_one(pp, BAR_S_EMPTY + 2 * m + b, kTimeoutRole);
-                pipe_wait_one(pp, BAR_FULL + s, kTimeoutTile);
+            const uint64_t dA = umma_desc_sw128(sA) + (MB == 1 ? 0 : 1024 * m), dRing = umma_desc_sw128(ring);
+            const uint32_t tc = pp.tmem + TM_CHAIN * m;
+            // descriptor start addresses count 16-byte units: + 2 per K-step of a K-major operand (32 bytes), + 128 per K-step of an MN-major
+            // operand (16 rows of 128 bytes), + 1024 per 128-row block; + 8 columns per K-step of an operand in tensor memory
+            auto logits = [&](int k) {
+                const int t = first + step * k, s = t % STAGES, b = k & 1;
+                wait_spin(pp, BAR_FULL + s, t / STAGES, kTimeoutTile);
                 tc_fence_after_sync();
                 const uint64_t dK = dRing + (uint64_t)(s * (kStage >> 4));
-                const uint32_t dd = pp.tmem + TM_S + 128 * b + 64 * m;
-                umma_ss_w(dd, dA, dK, idK, 0u);
-                umma_ss_w(dd, dA + 2, dK + 2, idK, 1u);
-                umma_ss_w(dd, dA + 4, dK + 4, idK, 1u);
-                umma_ss_w(dd, dA + 6, dK + 6, idK, 1u);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) umma_ss_w(tc + 64 * b, dA + 2 * i, dK + 2 * i, idK, i > 0);
                 umma_commit_w(pipe_bar(pp, BAR_S_FULL + 2 * m + b));
             };
-            pipe_wait_one(pp, BAR_AG, kTimeoutLoads);
-            issue_S(0);
-            for (int t = 0; t < tiles; ++t) {
-                if (t + 1 < tiles) issue_S(t + 1);
-                const int s = t % STAGES;
-                pipe_wait_one(pp, BAR_P_FULL + m, kTimeoutRole);
+            wait_spin(pp, BAR_AG, 0, kTimeoutLoads);
+            logits(0);
+            if (count > 1) logits(1);
+            for (int k = 0; k < count && !pipe_dead(pp); ++k) {
+                const int t = first + step * k, s = t % STAGES, b = k & 1;
+                wait_spin(pp, BAR_P_FULL + 2 * m + b, k >> 1, kTimeoutRole);
                 tc_fence_after_sync();
                 const int ntok = min(KT, N - (t0 + t) * KT);
                 const uint64_t dV = dRing + (uint64_t)(s * (kStage >> 4)) + (uint64_t)(kTile >> 4);
-                const uint64_t dP = dV + (uint64_t)(kTile >> 4) + 1024 * m;      // the probabilities replaced the stage's bias tile
-                for (int c = 0; c < 2; ++c) {
-                    if (32 * c >= ntok) break;
-                    const uint32_t dd = pp.tmem + TM_O + 64 * (2 * m + c);
-                    const uint64_t da = dP + 4 * c, db = dV + 256 * c;
-                    if (t > 0) umma_ss_w(dd, da, db, idMN, 1u); else umma_ss_w(dd, da, db, idMN, 0u);
-                    umma_ss_w(dd, da + 2, db + 128, idMN, 1u);
-                }
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+                    if (32 * c < ntok) {
+                        const uint32_t od = tc + TM_O + 64 * c, oa = tc + 64 * b + 32 * c;
+                        umma_ts_w(od, oa, dV + 256 * c, idMN, k > 0);
+                        umma_ts_w(od, oa + 8, dV + 256 * c + 128, idMN, 1u);
+                    }
                 umma_commit_w(pipe_bar(pp, BAR_EMPTY + s));
-                umma_commit_w(pipe_bar(pp, BAR_PV + m));
+                umma_commit_w(pipe_bar(pp, BAR_PV + 2 * m + b));
+                if (k + 2 < count) logits(k + 2);
             }
-            for (int t = max(0, tiles - 2); t < tiles; ++t) pipe_wait_one(pp, BAR_S_EMPTY + 2 * m + (t & 1), kTimeoutRole);
+            umma_drain_w(pp, BAR_DRAIN + m);
         }
         __syncwarp();
-    } else if ((warp >> 2 & 1) < MB) {
+    } else {
         // ------------------------------------------------------------------ row warps
-        const int mb = (warp >> 2) & 1, c = warp >> 3;         // agent block, token half
+        const int m = (warp >> 2) & 1, c = warp >> 3, mb = MB == 1 ? 0 : m;    // chain, token half, agent block
+        const int first = MB == 1 ? m : 0, step = MB == 1 ? 2 : 1, count = (tiles - first + step - 1) / step;
         const int row = 128 * mb + 32 * (warp & 3) + lane;     // agent row (padded)
         const uint32_t lane_base = ((uint32_t)(32 * (warp & 3))) << 16;
-        const uint32_t tO = pp.tmem + TM_O + 64 * (2 * mb + c) + lane_base;
+        const uint32_t tS = pp.tmem + TM_CHAIN * m + 32 * c + lane_base, tO = pp.tmem + TM_CHAIN * m + TM_O + 64 * c + lane_base;
         float m_ref = kRefFloor, l = 0.f;
         bool started = false;
-        for (int t = 0; t < tiles; ++t) {
-            const int b = t & 1, s = t % STAGES;
-            const int valid = min(32, N - ((t0 + t) * KT + 32 * c));      // tokens of this thread's half
-            pipe_wait_one(pp, BAR_S_FULL + 2 * mb + b, kTimeoutTile);
+        for (int k = 0; k < count; ++k) {
+            const int t = first + step * k, b = k & 1, s = t % STAGES;
+            const int valid = min(32, N - ((t0 + t) * KT + 32 * c));      // tokens of this thread's half (uniform; may be <= 0)
+            wait_par(pp, BAR_S_FULL + 2 * m + b, k >> 1, kTimeoutTile);
             tc_fence_after_sync();
-            float sv[32];
-            {
-                uint32_t ra[32];
-                tmem_ld32(pp.tmem + TM_S + 128 * b + 64 * mb + 32 * c + lane_base, ra);
+            if (valid > 0) {
+                float sv[32];
+                tmem_ld32(tS + 64 * b, *reinterpret_cast<uint32_t(*)[32]>(sv));
                 tmem_ld_wait();
-                tc_fence_before_sync();
-                pipe_arrive(pp, BAR_S_EMPTY + 2 * mb + b);
                 if (has_bias) {                              // logits in natural units: scale1 * a.k + b1
                     const unsigned char* sB = smem + OFF_RING + s * kStage + 2 * kTile + row * 128;
 #pragma unroll
@@ -200,80 +193,77 @@ __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_cons
                         const uint4 raw = *reinterpret_cast<const uint4*>(sB + (((4 * c + j) ^ (row & 7)) << 4));
                         const uint32_t w4[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {            // packed pairs: one instruction per two logits
-                            const float2 r2 = ffma2(make_float2(__uint_as_float(ra[8 * j + 2 * k]), __uint_as_float(ra[8 * j + 2 * k + 1])),
-                                                    make_float2(p.scale, p.scale), unpack2<T>(w4[k]));
-                            sv[8 * j + 2 * k] = r2.x; sv[8 * j + 2 * k + 1] = r2.y;
+                        for (int i = 0; i < 4; ++i) {            // packed pairs: one instruction per two logits
+                            const float2 r2 = ffma2(make_float2(sv[8 * j + 2 * i], sv[8 * j + 2 * i + 1]), make_float2(p.scale, p.scale), unpack2<T>(w4[i]));
+                            sv[8 * j + 2 * i] = r2.x; sv[8 * j + 2 * i + 1] = r2.y;
                         }
                     }
                 } else {
 #pragma unroll
-                    for (int k = 0; k < 32; ++k) sv[k] = __uint_as_float(ra[k]) * p.scale;
+                    for (int i = 0; i < 16; ++i) {
+                        const float2 r2 = fmul2(make_float2(sv[2 * i], sv[2 * i + 1]), make_float2(p.scale, p.scale));
+                        sv[2 * i] = r2.x; sv[2 * i + 1] = r2.y;
+                    }
                 }
-            }
-            uint32_t pk[16];
-            float corr = 1.f;
-            bool resc = false;
-            const bool tv = valid > 0;                         // uniform per warp
-            if (tv) {
                 if (valid < 32) {
 #pragma unroll
-                    for (int k = 0; k < 32; ++k) if (k >= valid) sv[k] = -INFINITY;
+                    for (int i = 0; i < 32; ++i) if (i >= valid) sv[i] = -INFINITY;
                 }
-                float mx0 = sv[0], mx1 = sv[1];
+                float mx0 = fmaxf(sv[0], sv[1]), mx1 = fmaxf(sv[2], sv[3]);
 #pragma unroll
-                for (int k = 2; k < 30; k += 4) { mx0 = max3(mx0, sv[k], sv[k + 1]); mx1 = max3(mx1, sv[k + 2], sv[k + 3]); }
-                const float mx = max3(mx0, mx1, fmaxf(sv[30], sv[31]));
-                if (mx > m_ref + kTau) {                       // also the first tile with an open key (m_ref = kRefFloor)
+                for (int i = 4; i < 32; i += 4) { mx0 = max3(mx0, sv[i], sv[i + 1]); mx1 = max3(mx1, sv[i + 2], sv[i + 3]); }
+                const float mx = fmaxf(mx0, mx1);
+                float corr = 1.f;
+                const bool moved = mx > m_ref + kTau;          // also the first tile with an open key (m_ref = kRefFloor)
+                if (moved) {
                     corr = fast_exp2((m_ref - mx) * kLog2e);
-                    resc = started;
                     m_ref = mx;
                     l *= corr;
                 }
-                const float nb = -m_ref * kLog2e;
-                float2 s01 = make_float2(0.f, 0.f), s23 = make_float2(0.f, 0.f);
-                const float2 l2e = make_float2(kLog2e, kLog2e), nb2 = make_float2(nb, nb);
+                uint32_t pk[16];
+                {
+                    const float nb = -m_ref * kLog2e;
+                    float2 s01 = make_float2(0.f, 0.f), s23 = make_float2(0.f, 0.f);
+                    const float2 l2e = make_float2(kLog2e, kLog2e), nb2 = make_float2(nb, nb);
 #pragma unroll
-                for (int k = 0; k < 16; k += 2) {
-                    const float2 a0 = ffma2(make_float2(sv[2 * k], sv[2 * k + 1]), l2e, nb2);
-                    const float2 a1 = ffma2(make_float2(sv[2 * k + 2], sv[2 * k + 3]), l2e, nb2);
-                    const float2 p01 = make_float2(fast_exp2(a0.x), fast_exp2(a0.y));     // exp2(-inf) = 0 past the range
-                    const float2 p23 = make_float2(fast_exp2(a1.x), fast_exp2(a1.y));
-                    s01 = fadd2(s01, p01); s23 = fadd2(s23, p23);
-                    pk[k] = pack2<T>(p01.x, p01.y);
-                    pk[k + 1] = pack2<T>(p23.x, p23.y);
+                    for (int i = 0; i < 16; i += 2) {
+                        const float2 a0 = ffma2(make_float2(sv[2 * i], sv[2 * i + 1]), l2e, nb2);
+                        const float2 a1 = ffma2(make_float2(sv[2 * i + 2], sv[2 * i + 3]), l2e, nb2);
+                        const float2 p01 = make_float2(fast_exp2(a0.x), fast_exp2(a0.y));     // exp2(-inf) = 0 past the range
+                        const float2 p23 = make_float2(fast_exp2(a1.x), fast_exp2(a1.y));
+                        s01 = fadd2(s01, p01); s23 = fadd2(s23, p23);
+                        pk[i] = pack2<T>(p01.x, p01.y);
+                        pk[i + 1] = pack2<T>(p23.x, p23.y);
+                    }
+                    l += (s01.x + s01.y) + (s23.x + s23.y);
                 }
-                l += (s01.x + s01.y) + (s23.x + s23.y);
+                tmem_st16(tS + 64 * b, pk);
+                if (started && __any_sync(0xffffffffu, moved)) {   // rare: the accumulator follows, once the products of the tile before are done
+                    wait_par(pp, BAR_PV + 2 * m + (b ^ 1), (k - 1) >> 1, kTimeoutTile);
+                    tc_fence_after_sync();
+#pragma unroll
+                    for (int hh = 0; hh < 4; ++hh) {
+                        float ra[16];
+                        uint32_t wa[16];
+                        tmem_ld16(tO + 16 * hh, ra);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) wa[i] = __float_as_uint(ra[i] * corr);
+                        tmem_st16(tO + 16 * hh, wa);
+                    }
+                }
                 started = true;
-            }
-            // P of the previous tile has been consumed (and every product into this thread's accumulator is done)
-            if (t > 0) { pipe_wait_one(pp, BAR_PV + mb, kTimeoutTile); tc_fence_after_sync(); }
-            if (__any_sync(0xffffffffu, resc)) {               // rare: the reference maximum of some row moved
-                uint32_t ra[32];
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
-                    tmem_ld32(tO + 32 * hh, ra);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int k = 0; k < 32; ++k) ra[k] = __float_as_uint(__uint_as_float(ra[k]) * corr);
-                    tmem_st32(tO + 32 * hh, ra);
-                }
                 tmem_st_wait();
             }
-            if (tv) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    *reinterpret_cast<uint4*>(smem + OFF_RING + s * kStage + 2 * kTile + row * 128 + (((4 * c + j) ^ (row & 7)) << 4)) =
-                        make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
-            }
-            fence_proxy_async();
             tc_fence_before_sync();
-            pipe_arrive(pp, BAR_P_FULL + mb);
+            pipe_arrive_warp(pp, BAR_P_FULL + 2 * m + b, lane);
         }
-        pipe_wait_one(pp, BAR_PV + mb, kTimeoutTile);
-        tc_fence_after_sync();
+        if (count > 0) {
+            wait_par(pp, BAR_PV + 2 * m + ((count - 1) & 1), (count - 1) >> 1, kTimeoutTile);
+            tc_fence_after_sync();
+        }
         // both chains are through with the ring before its memory is reused for the exchange below
-        asm volatile("bar.sync 3, %0;\n" ::"r"(256 * MB) : "memory");
+        asm volatile("bar.sync 3, %0;\n" ::"n"(NROW) : "memory");
         // the two token halves of a row meet in shared memory (the ring is drained: every product is done)
         float o[64];
         {
@@ -288,19 +278,19 @@ __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_cons
             }
         }
         tc_fence_before_sync();
-        float* sX = reinterpret_cast<float*>(smem + OFF_RING) + (size_t)row * 68;      // [256][68]: row, m, l
+        float* sX = reinterpret_cast<float*>(smem + OFF_RING) + (size_t)(128 * m + (row & 127)) * 68;      // [256][68]: row, m, l
         if (c == 1) {
 #pragma unroll
             for (int k = 0; k < 16; ++k) *reinterpret_cast<float4*>(sX + 4 * k) = make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
             sX[64] = m_ref; sX[65] = started ? l : 0.f;
         }
-        asm volatile("bar.sync %0, 256;\n" ::"r"(1 + mb) : "memory");      // the chain's own barrier
+        asm volatile("bar.sync %0, 256;\n" ::"r"(1 + m) : "memory");       // the chain's own barrier
         if (c == 0) {
             const float om = sX[64], ol = sX[65];
             const float mm = fmaxf(m_ref, om);
             const float bs = (mm == -INFINITY) ? 0.f : mm;
             const float wa = fast_exp2((m_ref - bs) * kLog2e), wb = fast_exp2((om - bs) * kLog2e);
-            float* part = slab_parts + (size_t)split * pf;
+            float* part = slab_parts + (size_t)(MB == 1 ? 2 * split + m : split) * pf;
             part[row] = mm * kLog2e;                       // the merge works in log2 units
             part[g.rows_pad + row] = (started ? l : 0.f) * wa + ol * wb;
             float* pacc = part + 2 * (size_t)g.rows_pad + (size_t)row * 64;
@@ -408,7 +398,7 @@ AggPlan plan_aggregate_umma(int slabs, int n_agents, int n_tokens, int d, int sm
     if (splits > 64) splits = 64;
     const int tps = (tiles + splits - 1) / splits;
     pl.splits = (tiles + tps - 1) / tps;
-    pl.parts = pl.splits;
+    pl.parts = pl.splits * (pl.rows_pad == 128 ? 2 : 1);          // (up to 128 agents: each chain writes its own)
     return pl;
 }
 
@@ -420,10 +410,11 @@ static cudaError_t launch_umma_t(const UmmaAggArgs& g, cudaStream_t st) {
     dim3 grid(g.a.splits, g.a.slabs);
     e = launch_dependent(kern, grid, NT, kSmemBytes, st, g);
     if (e != cudaSuccess) return e;
-    const bool one = g.a.splits <= 16;
+    const int parts = g.a.splits * (g.rows_pad == 128 ? 2 : 1);
+    const bool one = parts <= 16;
     const int rows = one ? 16 : 4;
     return launch_dependent(one ? merge_umma_kernel<T, 1> : merge_umma_kernel<T, 4>, dim3((g.a.rows + rows - 1) / rows, g.a.slabs), 256, 0, st,
-                            (const float*)g.a.partials, g.a.splits, g.rows_pad, g.a.rows, g.a.d, static_cast<T*>(g.a.out));
+                            (const float*)g.a.partials, parts, g.rows_pad, g.a.rows, g.a.d, static_cast<T*>(g.a.out));
 }
 
 // cudaErrorNotSupported: a tensor map could not be encoded.
