@@ -87,16 +87,11 @@ struct Args {
     int slabs, heads, N, n, d, tiles, blocks;
     int bias;                 // 0: none; 1: tiles of token rows; 2: tiles of agent rows
     int chain;                // aggregation: all pairs of S in one accumulator, as where `stats` come from bwd_values_umma_kernel
+    int owned;                // tiles of a stretch whose batch entries a block takes one after another (0: the sequence in its natural order)
     float scale;
     alignas(64) CUtensorMap tm_x, tm_y, tm_a, tm_m, tm_b;
 };
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
-        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]),
-          "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15]) : "r"(taddr) : "memory");
-}
 __device__ __forceinline__ void load_pairs(uint32_t taddr, float2 (&v)[16]) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -130,9 +125,23 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int N = p.N, n = p.n, d = p.d;
     const int ab = blockIdx.x % p.blocks, lanes = gridDim.x / p.blocks, me = blockIdx.x / p.blocks;      // block of 64 agents; runs of its sequence
-    const long long total = (long long)p.slabs * p.tiles, first = total * me / lanes;
-    const int count = (int)(total * (me + 1) / lanes - first);
-    int slab = (int)(first / p.tiles), tile = (int)(first - (long long)slab * p.tiles);     // of the role's current tile
+    // Natural order: a run of the (slab, tile) sequence.  Owned: a run of the (head, tile) sequence, cut into stretches of up to p.owned tiles of a
+    // head, all batch entries of a stretch in turn.
+    const int batch = p.owned ? p.slabs / p.heads : 1;
+    const long long total = (long long)p.slabs / batch * p.tiles, first = total * me / lanes, end = total * (me + 1) / lanes;
+    const int count = (int)(end - first) * batch;
+    long long at = first;                        // start of the role's current segment: tiles of one slab that follow one another
+    int entry = 0, slab = 0, tile = 0, left = 0, length = 0;                                // its current tile, and how many of the segment are left
+    bool fresh = true;                           // the first tile of a segment
+    auto segment = [&] {
+        slab = (int)(at / p.tiles);
+        tile = (int)(at - (long long)slab * p.tiles);
+        length = (int)min(end - at, (long long)(p.tiles - tile));
+        if (p.owned) length = min(length, p.owned);
+        left = length;
+        slab += entry * p.heads;
+    };
+    segment();
     const uint32_t base = smem_u32(smem);
 
     Pipe pp;
@@ -153,7 +162,11 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
     pdl_wait_prior();
     pdl_release_next();
     auto advance = [&] {
-        if (++tile == p.tiles) { tile = 0; ++slab; }
+        ++tile;
+        fresh = --left == 0;
+        if (!fresh) return;
+        if (++entry == batch) { entry = 0; at += length; }
+        segment();
     };
 
     if (warp == 12) {
@@ -178,8 +191,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
                         tma_load_3d(to + kMat, &p.tm_b, tile * kTok + 64, ab * 64, head, bb);
                     }
                 }
-                if (i == 0 || tile == 0) {
-                    if (i > 0) wait_spin(pp, (STATS ? BAR_FREE : BAR_DONE) + (b ^ 1), (i - 1) >> 1, kTimeoutRole);  // the last tile of the slab before
+                if (fresh) {
+                    if (i > 0) wait_spin(pp, (STATS ? BAR_FREE : BAR_DONE) + (b ^ 1), (i - 1) >> 1, kTimeoutRole);  // the last tile of the segment before
                     const uint32_t bam = pipe_bar(pp, BAR_AM), am = base + OFF_AM;
                     mbar_arrive_expect_tx(bam, 2 * kTerms * kMat);
                     for (int t = 0; t < kTerms; ++t) {
@@ -197,7 +210,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
         int groups = 0;
         for (int i = 0; i < count && !pipe_dead(pp); ++i, advance()) {
             const int b = i & 1;
-            if (i == 0 || tile == 0) wait_spin(pp, BAR_AM, groups++, kTimeoutTile);
+            if (fresh) wait_spin(pp, BAR_AM, groups++, kTimeoutTile);
             wait_spin(pp, BAR_FULL + b, i >> 1, kTimeoutTile);
             if (i > 0) wait_spin(pp, BAR_READ, i - 1, kTimeoutRole);
             tc_fence_after_sync();
@@ -310,7 +323,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
                     }
                 }
             }
-            if (sums && (tile == p.tiles - 1 || i == count - 1)) {     // the last tile of the slab in this block
+            if (sums && left == 1) {                                   // the last tile of the segment
                 float* dst = second ? p.outer1 : p.outer0;
                 const float scale = second ? p.scale : 1.f;
 #pragma unroll
@@ -332,7 +345,6 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
         const int q = warp & 3, half = warp >> 2, r = 32 * q + lane;
         const uint32_t ts = pp.tmem + TM_S + ((uint32_t)(32 * q) << 16) + 32 * half;
         const float c1 = p.scale * kLog2e;
-        const bool store = p.slabs == p.heads;
         float2* s_stat = reinterpret_cast<float2*>(smem + OFF_STAT);
         int parity = 0;
         const float2 none = make_float2(INFINITY, 0.f);                // (a token or an agent that does not exist: its probabilities are zero)
@@ -367,17 +379,19 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
             if (p.bias && lane == (__all_sync(0xffffffffu, x == 0x5bd1e995u) ? 31 : 0)) pipe_arrive(pp, BAR_BREAD);
         };
         load_bias(0);
-        for (int i = 0; i < count; ++i, advance()) {
-            const int b = i & 1, tok = tile * kTok + r, head = slab % p.heads;
-            const bool ok = tok < N;
+        for (int i = 0; i < count; ++i) {
+            const int now = slab, at_tile = tile;                      // this tile; the role's state goes on to the next
+            const bool first_tile = fresh;
+            if (i + 1 < count) advance();
+            const int b = i & 1, tok = at_tile * kTok + r, head = now % p.heads;
+            const bool ok = tok < N, store = p.slabs == p.heads || (p.owned && now < p.heads);      // a head's first batch entry, here before the others
             const float2 st = next;
             if (BCAST) {
-                const int nt = tile + 1 == p.tiles ? 0 : tile + 1, ns = slab + (nt == 0);
                 next = none;
-                if (i + 1 < count && nt * kTok + r < N) next = __ldg(p.stats + (size_t)ns * N + nt * kTok + r);
-            } else if (AGG && (i == 0 || tile == 0)) {                 // another slab: its statistics
+                if (i + 1 < count && tile * kTok + r < N) next = __ldg(p.stats + (size_t)slab * N + tile * kTok + r);
+            } else if (AGG && first_tile) {                                 // another segment: its statistics
                 parity ^= 1;
-                if (tid < 64) s_stat[parity * 64 + tid] = ab * 64 + tid < n ? __ldg(p.stats + (size_t)slab * n + ab * 64 + tid) : none;
+                if (tid < 64) s_stat[parity * 64 + tid] = ab * 64 + tid < n ? __ldg(p.stats + (size_t)now * n + ab * 64 + tid) : none;
                 bar_named(1, kRowThreads);
             }
             wait_par(pp, BAR_S, i, kTimeoutTile);
@@ -419,8 +433,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
                     const float4 o = ex[r];
                     const float mm = fmaxf(m, o.x), f = m == -INFINITY ? 0.f : exp2f(m - mm), fo = o.x == -INFINITY ? 0.f : exp2f(o.x - mm);
                     const float tot = fmaf(l, f, o.y * fo), dt = fmaf(dot, f, o.z * fo);
-                    if (p.blocks == 1) p.tok_stats[(size_t)slab * N + tok] = make_float2(mm + log2f(tot), dt / tot);
-                    else p.partial[((size_t)ab * p.slabs + slab) * N + tok] = make_float4(mm, tot, dt, 0.f);
+                    if (p.blocks == 1) p.tok_stats[(size_t)now * N + tok] = make_float2(mm + log2f(tot), dt / tot);
+                    else p.partial[((size_t)ab * p.slabs + now) * N + tok] = make_float4(mm, tot, dt, 0.f);
                 }
                 if (i + 1 < count) load_bias(i + 1);
                 continue;
@@ -468,7 +482,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
             if (p.dbias && lim > 0) {
                 if (BCAST) {
                     // [token][agent]: this warp's terms of dS, read back so that neighbouring lanes add to neighbouring agents
-                    const int t0 = tile * kTok + 32 * q;
+                    const int t0 = at_tile * kTok + 32 * q;
                     float* g = p.dbias + ((size_t)head * N + t0) * n + c0;
                     const unsigned char* src = smem + OFF_P + kTile + 32 * q * 128;
                     if (n % 4 == 0) {
@@ -538,7 +552,7 @@ template <int MODE> cudaError_t launch(const Args& a, int sm_count, cudaStream_t
     static std::atomic<unsigned long long> done;
     cudaError_t e = allow_smem(bwd_terms_umma_kernel<MODE>, done, kSmemBytes);
     if (e != cudaSuccess) return e;
-    const long long total = (long long)a.slabs * a.tiles, lanes = std::min<long long>(total, std::max(1, sm_count / a.blocks));
+    const long long total = (long long)(a.owned ? a.heads : a.slabs) * a.tiles, lanes = std::min<long long>(total, std::max(1, sm_count / a.blocks));
     return launch_dependent(bwd_terms_umma_kernel<MODE>, dim3((unsigned)(lanes * a.blocks)), kThreads, kSmemBytes, st, a);
 }
 
@@ -558,6 +572,17 @@ bool backward_terms_umma_eligible(int dtype, int slabs, int n, int N, int d) {
     if (d > 48) return n > 16 ? N >= 196 || tokens >= 9000 : N >= 1024 || tokens >= 16000;
     if (d > 32) return n > 16 ? N >= 1024 || tokens >= 28000 : N >= 8192 || (N <= 512 && tokens >= 28000);
     return n > 16 && (N >= 8192 || (N <= 256 && tokens >= 28000));
+}
+
+// Tiles of a stretch of the token axis whose batch entries one block takes in turn (0: runs of slabs).  A block that has all batch entries of its tiles
+// stores the first one's bias gradients and adds the others' to them: nothing is cleared, and what is added to is still in L2 (a reduction of 32 KB
+// on every SM: 1650 cycles where L2 holds the sums, 3400 where it does not).  A stretch ends with a change of A and M; two batch entries of
+// eight heads on a 128 x 128 grid, 256 agents, whole pass: 1176 us in the natural order; stretches of 28, 10, 4 and 2 tiles 1126, 1108, 1096 and 1084.
+int backward_terms_umma_owned(int slabs, int heads, int n, int N, int sm_count) {
+    constexpr int kStretch = 4;
+    const long long tiles = (long long)heads * ((N + kTok - 1) / kTok), blocks = (n + 63) / 64, lanes = std::max<long long>(1, sm_count / blocks);
+    if (slabs == heads || tiles < 8 * lanes) return 0;                  // (blocks have whole tiles of the axis: one more for some than for others)
+    return kStretch;
 }
 
 size_t backward_terms_umma_bytes(int slabs, int heads, int n, int N) {
@@ -586,6 +611,7 @@ cudaError_t launch_backward_terms_umma(BwdTermsUmma stage, const BwdCall& c, con
     a.row0 = queries ? c.dq : c.dk; a.row1 = c.dv;
     a.dbias = queries ? c.db2 : c.db1;
     a.chain = backward_values_eligible(c.slabs, c.n, N);
+    a.owned = a.dbias && stage != kUmmaStats ? backward_terms_umma_owned(c.slabs, c.heads, c.n, N, c.sm_count) : 0;
     a.scale = queries ? c.scale2 : c.scale1;
     if (!make_map_3d_u16(&a.tm_x, queries ? c.q : c.k, c.slabs, N, c.d, kTok) || !make_map_3d_u16(&a.tm_y, queries ? c.d_out : c.v, c.slabs, N, c.d, kTok) ||
         !make_map_3d_u16(&a.tm_a, a_t, (uint64_t)kTerms * c.slabs, c.n, c.d, 64) || !make_map_3d_u16(&a.tm_m, m_t, (uint64_t)kTerms * c.slabs, c.n, c.d, 64))
