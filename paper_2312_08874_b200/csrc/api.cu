@@ -81,22 +81,23 @@ bool umma_shape(const agent_attn_handle* h, int n_tokens, int n_agents) {
     return !use_simt(h) && auto_like(h) &&
            aggregate_umma_eligible(h->cfg.dtype, n_agents, n_tokens, h->cfg.head_dim, true);
 }
-// They pad agents to 128 and channels to 64 and pay a start and a separate merge; the register tiles pay for neither.  Register tiles
-// against these, times of the whole pass (above 1: these are faster), bf16 with biases and depthwise term:
-//   256 agents of 56 or 64 channels, the blocks filled: 6144 tokens and more 1.07 to 1.75; shorter axes once there is a tile for every
-//     SM (3072 tokens: 8 slabs 0.93 to 0.96, 16 slabs 1.26 to 1.32, 32 slabs 1.01)
-//   144 agents of 64 channels, half-filled: 6144 tokens, 1 to 16 slabs 0.99 to 1.17, 32 and 64 slabs 0.93 to 0.98; 16384 tokens 1.16
-//     to 1.39, 32 slabs 0.97
-//   256 agents of 40 channels: 7920 tokens 0.92 to 1.17, 16384 tokens 1.10 to 1.30; 24 slabs of 12960 tokens 1.05, 32 slabs 0.82 and 0.89
-//     (four blocks a slab: 20 SMs idle)
-//   256 agents of 32 channels 0.58 to 1.02 (one slab of 16384 tokens 1.12); 144 agents of 32 or 40 channels 0.50 to 1.02
+// They pad agents to 64 and channels to 64 and pay a start and a separate merge; the register tiles pay for neither.  Register tiles
+// against these, times of the whole pass (above 1: these are faster), bf16, with and without biases and depthwise term, 1 to 64 slabs:
+//   256 agents of 64 channels: 9216 tokens and more 1.41 to 2.39; 3072 and 4096 tokens, one slab 0.81 to 1.10, more 0.98 to 1.64; 768 to 1536
+//     tokens, up to 4 slabs 0.76 to 1.16, 32 and 64 slabs 0.96 to 1.33
+//   144 agents of 64 channels: 9216 tokens and more 1.12 to 2.01; 3072 and 4096 tokens 0.71 to 1.42
+//   256 agents of 40 channels: 9216 tokens and more 1.07 to 2.10; 3072 and 4096 tokens, 16 slabs and more 1.04 to 1.35, fewer 0.68 to 1.01
+//   144 agents of 40 channels: 16384 tokens and more 0.96 to 1.77; 9216 tokens, 8 slabs and more 1.06 to 1.40, fewer 0.87 to 1.05
+//   256 agents of 32 channels: 16384 tokens and more 1.04 to 1.75; 9216 tokens, one or two slabs 0.95 to 1.08, more 0.99 to 1.28
+//   144 agents of 32 channels: 32768 tokens 1.06 to 1.54 (32 slabs without biases 0.94); 16384 tokens, 8 slabs and more 0.94 to 1.39, fewer 0.91 to 1.12
 bool use_umma(const agent_attn_handle* h, int n_tokens, int n_agents) {
-    if (n_tokens < 2048 || !umma_shape(h, n_tokens, n_agents)) return false;
+    if (n_tokens < 768 || !umma_shape(h, n_tokens, n_agents)) return false;
     const int d = h->cfg.head_dim, slabs = h->cfg.batch * h->cfg.heads;
     const long long work = (long long)slabs * n_tokens;
     const bool filled = n_agents * 4 >= (n_agents + 127) / 128 * 128 * 3;
-    if (d > 48) return filled ? n_tokens >= 6144 || work >= 32768 : n_tokens >= 8192 || (n_tokens >= 6144 && slabs <= 16);
-    return filled && d > 32 && n_tokens >= 8192 && slabs <= 24;
+    if (d > 48) return filled ? work >= (n_tokens >= 3072 ? 6144 : 32768) : n_tokens >= 7168 || (n_tokens >= 6144 && slabs <= 16);
+    if (d > 32) return filled ? n_tokens >= 6144 || (n_tokens >= 1536 && work >= 49152) : n_tokens >= 12288 || (n_tokens >= 8192 && slabs >= 8);
+    return filled ? n_tokens >= 16384 || (n_tokens >= 8192 && slabs >= 4) : slabs <= 24 && (n_tokens >= 32768 || (n_tokens >= 16384 && slabs >= 8));
 }
 
 AggPlan plan_for(const agent_attn_handle* h, int n_tokens, int n_agents) {
@@ -567,6 +568,14 @@ static int forward_impl(agent_attn_handle* h, const void* Q, const void* K, cons
         TileArgs t = tile_args(h, grid_h, grid_w, n_agents, cl);
         t.q = Q; t.k = K; t.v = V; t.a = A ? A : ws + w.a_off; t.va = ws + w.va_off; t.pool = p;
         t.b1 = b1; t.b2 = b2; t.wd = dwc_weight; t.out = out;
+        if (auto_like(h) && slab_umma_eligible(h->cfg.dtype, t, h->sm_count)) {
+            const cudaError_t e = launch_slab_umma(h->cfg.dtype, t, h->d_status, st);
+            if (e != cudaErrorNotSupported) {
+                if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "forward launch failed: %s", cudaGetErrorString(e));
+                h->launches = 1;
+                return AA_OK;
+            }
+        }
         const cudaError_t e = launch_tile_forward(h->cfg.dtype, t, h->sm_count, h->cfg.path != AA_PATH_UNFUSED && tile_one_kernel(t, h->sm_count), st, &h->launches);
         if (e != cudaSuccess) return fail(h, AA_ERR_CUDA, "forward launch failed: %s", cudaGetErrorString(e));
         return AA_OK;

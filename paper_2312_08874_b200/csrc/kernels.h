@@ -138,6 +138,9 @@ cudaError_t launch_tile_forward(int dtype, TileArgs a, int sm_count, bool one_ke
 cudaError_t launch_tile_aggregate(int dtype, TileArgs a, int sm_count, bool dependent, cudaStream_t st);
 cudaError_t launch_tile_broadcast(int dtype, TileArgs a, int sm_count, bool dependent, cudaStream_t st);
 bool tile_one_kernel(const TileArgs& a, int sm_count);   // short grids: one kernel for the whole pass
+// Short grids on tensor memory: one block per slab (slab_umma.cu).
+bool slab_umma_eligible(int dtype, const TileArgs& a, int sm_count);
+cudaError_t launch_slab_umma(int dtype, const TileArgs& a, int* status, cudaStream_t st);
 
 // Whole module (Eq. 6) in one persistent kernel for small agent counts (n <= 64, d = 64,
 // block pooling, W <= 64).  Blocks take tasks from a device-side queue: "G" tasks pool their token
