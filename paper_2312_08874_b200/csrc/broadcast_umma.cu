@@ -62,7 +62,7 @@ constexpr int BAR_S_FULL = 14;     // ts          commit      row warps
 constexpr int BAR_P_FULL = 18;     // ts          8 warps     MMA issuer      (logits read as well)
 constexpr int BAR_PV = 22;         // ts          commit      row warps       products of a step (only where a reference moves)
 constexpr int BAR_O_FULL = 26;     // t           commit      output warps    every product of a tile
-constexpr int BAR_O_EMPTY = 28;    // t           8 warps     MMA issuer      accumulators read
+constexpr int BAR_O_EMPTY = 28;    // t           8 warps     MMA issuer, row warps    accumulators and (max, sum) read
 constexpr int BAR_ML = 30;         // t           8 warps     output warps
 constexpr int BAR_H_FULL = 32;     // i           tx          output warps    V tokens of the tile's depthwise window
 constexpr int BAR_H_EMPTY = 34;    // i           8 warps     their producer
@@ -228,7 +228,12 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
                 wait_par(pp, BAR_H_FULL + team, k, kTimeoutLoads);
                 // rows 16 mt .. of the warp are a row of the patch; those of the next one sit a row of the window on
                 dwc_rows<T, TW + 2>(o, sH + team * kHalo, 2 * q * (TW + 2) + (lane & 15), 64 * half, tab, lane, [](int u, int v) { return u * (TW + 2) + v; });
-                pipe_arrive_warp(pp, BAR_H_EMPTY + team, lane);
+                // The window goes back to TMA: an arrival overtakes loads that are still queued, so the arriving lane hangs on the products of
+                // what was loaded.
+                uint32_t x = 0u;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) x ^= __float_as_uint(o[k >> 2][k & 3][0]);
+                if (lane == (__all_sync(0xffffffffu, x == 0x5bd1e995u) ? 31 : 0)) pipe_arrive(pp, BAR_H_EMPTY + team);
             }
             wait_par(pp, BAR_ML + team, k, kTimeoutTile);
             float w0, w1;                                      // weights of row 32 q + lane's two accumulators
@@ -370,6 +375,8 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
                     }
                 }
                 if (a == steps - 1) {
+                    // (with two steps nothing else holds the (max, sum) of this tile back until those of the tile before have been read)
+                    if (steps == 2 && i >= 2) wait_par(pp, BAR_O_EMPTY + team, (i >> 1) - 1, kTimeoutRole);
                     reinterpret_cast<float2*>(smem + OFF_ML)[(team * 2 + ((i >> 1) & 1)) * 256 + half * 128 + row] = make_float2(m_ref, l);
                     pipe_arrive_warp(pp, BAR_ML + team, lane);
                 }
