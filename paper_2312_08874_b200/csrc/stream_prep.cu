@@ -1,6 +1,6 @@
 // First kernel of the streaming path for small agent counts: everything the two attention kernels need
 // besides Q, K and V themselves.
-//   * agents A = Pooling(Q) (text under Eq. 6): one warp per (slab, agent) window, 16-byte loads with eight in
+//   * agents A = Pooling(Q) (text under Eq. 6): one warp per (slab, agent) window (a block where there are few large ones), 16-byte loads with eight in
 //     flight per lane, fp32 sums in a fixed order; written as A and as scale1 * A, scale2 * A (each rounded
 //     once from the fp32 mean), the operands of the logit products of Eq. 3.  A caller's agents are only scaled.
 //   * agent biases (Eq. 5): B1 clamped to +-30000, transposed to [N][64] (pad columns zero); B2 clamped and
@@ -17,7 +17,7 @@ namespace aa {
 namespace {
 constexpr int NT = 256;
 
-template <typename T>
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(NT, 4) stream_prep_kernel(const StreamArgs p, int bias_blocks) {
     pdl_wait();                       // the workspace may still be read by the kernels before
     pdl_launch_dependents();          // the aggregation kernel may set itself up while this one runs
@@ -25,7 +25,8 @@ __global__ void __launch_bounds__(NT, 4) stream_prep_kernel(const StreamArgs p, 
     const int N = p.H * p.W, n = p.n;
     // the bias blocks come first in the grid: they are few, latency-bound, and would otherwise form the kernel's tail
     if ((int)blockIdx.x >= bias_blocks) {
-        const long long wi = (long long)(blockIdx.x - bias_blocks) * (NT / 32) + warp;
+        // WIDE: the eight warps share a window
+        const long long wi = WIDE ? (long long)(blockIdx.x - bias_blocks) : (long long)(blockIdx.x - bias_blocks) * (NT / 32) + warp;
         if (wi >= (long long)p.slabs * n) return;
         const int slab = (int)(wi / n), a = (int)(wi - (long long)slab * n);
         const int c = lane & 7, ts = lane >> 3;
@@ -36,24 +37,26 @@ __global__ void __launch_bounds__(NT, 4) stream_prep_kernel(const StreamArgs p, 
         if (p.a_user) {
             if (ts == 0) unpack16<T>(__ldg(reinterpret_cast<const uint4*>(static_cast<const T*>(p.a_user) + ((size_t)slab * n + a) * 64) + c), acc);
         } else {
-            const int win_h = p.H / p.p, win_w = p.W / p.p, cnt = win_h * win_w;
-            const int y0 = (a / p.p) * win_h, x0 = (a % p.p) * win_w;
+            const int ay = a / p.p, ax = a - ay * p.p;
+            const int y0 = ay * p.H / p.p, x0 = ax * p.W / p.p, win_w = ((ax + 1) * p.W + p.p - 1) / p.p - x0, cnt = (((ay + 1) * p.H + p.p - 1) / p.p - y0) * win_w;
             // lane (c, ts) walks the window's tokens ts, ts + 4, ... in row-major order; (wy, wx) is kept
             // incrementally, so the loads of a batch cost an add and a compare each
             const uint4* gq = reinterpret_cast<const uint4*>(static_cast<const T*>(p.q) + tok_offset(p.lin, slab, p.heads, (long long)y0 * p.W + x0)) + c;
             const size_t qst = (size_t)p.lin.st / 8;
             inv = 1.f / (float)cnt;
-            int wy = ts / win_w, wx = ts - wy * win_w;
+            constexpr int kStep = WIDE ? NT / 8 : 4;                   // token lanes that take turns
+            const int tw = WIDE ? ts + 4 * warp : ts;
+            int wy = tw / win_w, wx = tw - wy * win_w;
             float2 acc2[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) acc2[k] = make_float2(0.f, 0.f);
-            for (int ib = ts; ib < cnt; ib += 32) {          // eight loads in flight per lane, four blocks per SM
+            for (int ib = tw; ib < cnt; ib += 8 * kStep) {   // eight loads in flight per lane, four blocks per SM
                 uint4 raw[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     raw[u] = make_uint4(0u, 0u, 0u, 0u);
-                    if (ib + 4 * u < cnt) raw[u] = __ldg(gq + ((size_t)wy * p.W + wx) * qst);
-                    wx += 4;
+                    if (ib + kStep * u < cnt) raw[u] = __ldg(gq + ((size_t)wy * p.W + wx) * qst);
+                    wx += kStep;
                     while (wx >= win_w) { wx -= win_w; ++wy; }
                 }
 #pragma unroll
@@ -71,6 +74,18 @@ __global__ void __launch_bounds__(NT, 4) stream_prep_kernel(const StreamArgs p, 
         for (int o = 8; o < 32; o <<= 1) {
 #pragma unroll
             for (int k = 0; k < 8; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+        }
+        if constexpr (WIDE) {                                          // (their shares add up in the order of the warps)
+            __shared__ __align__(16) float part[NT / 32][64];
+            if (ts == 0)
+#pragma unroll
+                for (int k = 0; k < 8; ++k) part[warp][8 * c + k] = acc[k];
+            __syncthreads();
+            if (warp != 0) return;
+            if (!p.a_user)
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    for (int w = 1; w < NT / 32; ++w) acc[k] += part[w][8 * c + k];
         }
         if (ts == 0) {
             float m[8], s1[8], s2[8];
@@ -147,9 +162,12 @@ cudaError_t launch_stream_prep(int dtype, const StreamArgs& a, cudaStream_t st) 
     long long bias_blocks = (items + NT - 1) / NT;            // one output vector per thread where the grid allows it
     if (bias_blocks > 8LL * a.sm_count) bias_blocks = 8LL * a.sm_count;
     if (bias_blocks < 1) bias_blocks = 1;
-    const unsigned grid = (unsigned)(pool_blocks + bias_blocks);
-    if (dtype == kBF16) return launch_dependent(stream_prep_kernel<__nv_bfloat16>, dim3(grid), NT, 0, st, a, (int)bias_blocks);
-    if (dtype == kF16) return launch_dependent(stream_prep_kernel<__half>, dim3(grid), NT, 0, st, a, (int)bias_blocks);
+    // few windows of many tokens: a block each (one slab of 88 x 244 tokens, 9 agents: 77 us for the whole pass with a warp each, 37 this way)
+    const bool wide = !a.a_user && windows < 8LL * a.sm_count && N > 32LL * a.n;
+    const unsigned grid = (unsigned)((wide ? windows : pool_blocks) + bias_blocks);
+    auto go = [&](auto kern) { return launch_dependent(kern, dim3(grid), NT, 0, st, a, (int)bias_blocks); };
+    if (dtype == kBF16) return wide ? go(stream_prep_kernel<__nv_bfloat16, true>) : go(stream_prep_kernel<__nv_bfloat16, false>);
+    if (dtype == kF16) return wide ? go(stream_prep_kernel<__half, true>) : go(stream_prep_kernel<__half, false>);
     return cudaErrorInvalidValue;
 }
 
