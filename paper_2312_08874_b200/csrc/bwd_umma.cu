@@ -12,7 +12,8 @@
 // average; A and M of the next slab arrive with its first tile.  Roles:
 //   warps 0-7   "row warps": thread = (token, half of the agents).  Logits and dP from tensor memory, bias from the ring stage; P and dS as
 //               swizzled rows of 64 agents in shared memory: the same bytes are the K-major operand of the products per token and the
-//               MN-major operand of the sums over tokens, so nothing is transposed.  Then the bias gradient, by coalesced reductions.
+//               MN-major operand of the sums over tokens, so nothing is transposed.  Then the bias gradient: staged in fp32 and added by one bulk
+//               reduction a tile, which runs beside the next tile (rows that are no multiple of 16 bytes: by coalesced reductions of the warps).
 //   warps 8-11  outputs: per-token products from tensor memory to global memory; at the end of a slab its sums.  Aggregation: a slab ahead,
 //               D and the terms of dV_A.
 //   warp 12     TMA: X, Y and the bias as token rows, two stages of 48 KB.
@@ -21,8 +22,9 @@
 // blocks two are used; as two products of 64 x 64 they would be sixteen.  (Aggregation: against X alone, 64 columns.)
 //
 // What bounds it: the chain load -> logits -> softmax -> products -> stage free through two stages, and HBM: 64 slabs of a 56 x 56 grid, 49
-// agents (by ncu, cold caches): broadcast 40 us (103 MB, 16 us at the copy bandwidth), aggregation 47 us (154 MB, 24 us, and the start: D and
-// the terms of dV_A); tensor pipe 17 and 13 %, issue 32 and 30 %.
+// agents: broadcast 5500 cycles a tile (softmax 2000, probabilities as operands 670, waits 1500), aggregation 6500; 103 MB, 16 us at the copy
+// bandwidth, and 154 MB, 24 us.  Bias gradients by reductions of the row warps took them 1700 to 2500 cycles a tile; staged for the bulk
+// reduction 600: whole pass 184.9 -> 177.6 us, 384 slabs of 196 tokens 109.9 -> 106.5.
 // With mma.sync, 64-token tiles and scalar bias loads and reductions the two took 96 and 93 us.
 #include "bwd_terms.cuh"
 #include "stream_common.cuh"
@@ -45,7 +47,12 @@ constexpr int kPatch = 33;                   // row pitch of a warp's patch of l
 constexpr int OFF_RING = 1024;
 constexpr int OFF_AM = OFF_RING + kStages * kStage;          // two buffers of A | M | M's residual
 constexpr int OFF_P = OFF_AM + 2 * 3 * kMat;                 // P | dS
-constexpr int OFF_PATCH = OFF_P + 2 * kTile;                 // broadcast: [8 warps][32][kPatch] floats; aggregation: [2][64] (lse, D)
+constexpr int OFF_PATCH = OFF_P + 2 * kTile;                 // broadcast: logit gradients, staged (below) or as [8 warps][32][kPatch] floats;
+                                                             // aggregation: [2][64] (lse, D), then the stage
+// Stage of logit gradients for the bulk reduction.  Aggregation: [n][128 tokens].  Broadcast: n a multiple of four: twice [128 tokens][32 agents],
+// 128-byte swizzle; n odd: [128 tokens][n] (a thread's stores of one agent go to different banks).
+constexpr int kStageBytes = 128 * 64 * 4, kStatBytes = 2 * 64 * 8;
+static_assert(OFF_PATCH % 1024 == 0 && kStatBytes + kStageBytes <= 8 * 32 * kPatch * 4, "stage");
 constexpr int OFF_EX = OFF_PATCH + 8 * 32 * kPatch * 4;      // broadcast: [2 tiles][2 halves][128] (max, sum, dot)
 constexpr int kSmemBytes = OFF_EX + 2 * 256 * 16 + 1024;
 static_assert(kSmemBytes <= 232448 && kSmemBytes > 116 * 1024, "one block per SM");
@@ -72,9 +79,17 @@ struct UmmaArgs {
     float* dbias;             // fp32, B2's layout [heads][N][n] or B1's [heads][n][N] (added), or null
     int* status;
     int slabs, heads, N, n, tiles, bias;
+    int bulk;                 // bias gradients by bulk reductions
     float scale;
-    alignas(64) CUtensorMap tm_x, tm_y, tm_a, tm_m, tm_b;
+    alignas(64) CUtensorMap tm_x, tm_y, tm_a, tm_m, tm_b, tm_db;
 };
+
+__device__ __forceinline__ void st_shared_f32(uint32_t addr, float v) { asm volatile("st.shared.f32 [%0], %1;\n" ::"r"(addr), "f"(v) : "memory"); }
+// One bulk reduction (fp32 additions in L2) of a staged box; what lies outside the tensor is left out.
+__device__ __forceinline__ void reduce_add_3d(const CUtensorMap* map, int x, int y, int z, uint32_t src) {
+    asm volatile("cp.reduce.async.bulk.tensor.3d.global.shared::cta.add.tile.bulk_group [%0, {%1, %2, %3}], [%4];\n"
+                 ::"l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(src) : "memory");
+}
 
 template <typename T, bool BCAST>
 __global__ void __launch_bounds__(kThreads, 1) bwd_umma_kernel(const __grid_constant__ UmmaArgs p) {
@@ -409,7 +424,40 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_umma_kernel(const __grid_cons
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) pipe_arrive(pp, BAR_P + b);
-            if (p.dbias && lim > 0) {
+            if (p.dbias && p.bulk) {
+                const int head = slab % p.heads;
+                const uint32_t stage = base + OFF_PATCH + (BCAST ? 0 : kStatBytes);
+                // the reduction of the tile before has read the stage
+                if (tid == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+                bar_named(1, kRowThreads);
+                if (!BCAST) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        if (j < lim) st_shared_f32(stage + ((c0 + j) * 128 + r) * 4, j & 1 ? dp[j >> 1].y : dp[j >> 1].x);
+                } else if (n % 4 == 0) {
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        if (4 * c < lim)
+                            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"r"(stage + half * (kStageBytes / 2) + r * 128 + ((c ^ (r & 7)) << 4)),
+                                         "f"(dp[2 * c].x), "f"(dp[2 * c].y), "f"(dp[2 * c + 1].x), "f"(dp[2 * c + 1].y) : "memory");
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        if (j < lim) st_shared_f32(stage + (r * n + c0 + j) * 4, j & 1 ? dp[j >> 1].y : dp[j >> 1].x);
+                }
+                fence_proxy_async();
+                bar_named(1, kRowThreads);
+                if (tid == 0) {
+                    if (!BCAST) reduce_add_3d(&p.tm_db, tile * kTok, 0, head, stage);
+                    else if (n % 4 == 0) {
+                        reduce_add_3d(&p.tm_db, 0, tile * kTok, head, stage);
+                        if (n > 32) reduce_add_3d(&p.tm_db, 32, tile * kTok, head, stage + kStageBytes / 2);
+                    } else
+                        asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;\n"
+                                     ::"l"(p.dbias + ((size_t)head * N + (size_t)tile * kTok) * n), "r"(stage), "r"(min(kTok, N - tile * kTok) * n * 4) : "memory");
+                    asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+                }
+            } else if (p.dbias && lim > 0) {
                 const int head = slab % p.heads;
                 if (BCAST) {
                     // [token][agent]: through the warp's patch, so that the lanes of a reduction are neighbouring agents
@@ -435,6 +483,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_umma_kernel(const __grid_cons
                 }
             }
         }
+        if (p.bulk && tid == 0) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -450,6 +499,16 @@ template <typename T, bool BCAST> cudaError_t launch(const UmmaArgs& a, int sm_c
 }
 
 }  // namespace
+
+// Map of a bias gradient, fp32 [heads][rows][cols], for reduce_add_3d.
+static bool make_map_grad(CUtensorMap* out, void* base, uint64_t heads, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_cols, bool swizzle) {
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn || (reinterpret_cast<uintptr_t>(base) & 15u) || cols % 4) return false;
+    const cuuint64_t dims[3] = {cols, rows, heads}, strides[2] = {4 * cols, 4 * rows * cols};
+    const cuuint32_t box[3] = {box_cols, box_rows, 1}, estr[3] = {1, 1, 1};
+    return fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 bool backward_umma_eligible(int dtype, int n, int d) { return (dtype == kBF16 || dtype == kF16) && n <= 64 && d == 64; }
 
@@ -471,6 +530,10 @@ cudaError_t launch_backward_umma(int dtype, bool broadcast_stage, const BwdCall&
         !make_map_rows3d_u16(&a.tm_a, c.ws_a, c.slabs, c.n, 64, true) || (broadcast_stage && !make_map_rows3d_u16(&a.tm_m, c.ws_part, 2 * (uint64_t)c.slabs, c.n, 64, true)) ||
         (bias && !make_map_3d_u16(&a.tm_b, rows, c.heads, N, bias_width(c.n), kTok)))
         return cudaErrorInvalidValue;
+    // Rows of 16 bytes: tokens a multiple of four, and agents a multiple of four or odd (token rows that follow one another, 128 at a time).
+    a.bulk = a.dbias && N % 4 == 0 && (!broadcast_stage || c.n % 4 == 0 || c.n % 2);
+    if (a.bulk && !broadcast_stage && !make_map_grad(&a.tm_db, a.dbias, c.heads, c.n, N, c.n, kTok, false)) return cudaErrorInvalidValue;
+    if (a.bulk && broadcast_stage && c.n % 4 == 0 && !make_map_grad(&a.tm_db, a.dbias, c.heads, N, c.n, kTok, 32, true)) return cudaErrorInvalidValue;
     if (dtype == kBF16) return broadcast_stage ? launch<__nv_bfloat16, true>(a, c.sm_count, st) : launch<__nv_bfloat16, false>(a, c.sm_count, st);
     if (dtype == kF16) return broadcast_stage ? launch<__half, true>(a, c.sm_count, st) : launch<__half, false>(a, c.sm_count, st);
     return cudaErrorInvalidValue;

@@ -17,6 +17,8 @@ SHAPES = [
     (50, 3, 7, 7, 7, "f16", True),        # runs of several slabs of one ragged tile
     (1, 1, 61, 83, 7, "f16", True),       # several blocks per slab
     (2, 2, 33, 32, 4, "bf16", True),      # 16 agents: B2 is read as it is, rows of 32 bytes; B1 with a row of agents in use past 1024 tokens
+    (3, 2, 22, 14, 8, "f16", True),       # bias gradients by bulk reductions: 64 agents, a tile of 52 tokens
+    (2, 3, 20, 15, 7, "bf16", True),      # the same, token rows of 49 agents
     (1, 1, 200, 201, 3, "bf16", True),    # agent values: more than 32 states for each warp of a row's block
 ]
 
