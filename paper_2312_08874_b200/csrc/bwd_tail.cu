@@ -9,7 +9,7 @@
 // share of dWd to one of kFilterCopies copies, which the second kernel adds up: relative error 1.4e-7, against 5e-7 in a single copy.
 // A block goes through several batch entries of its head where that fills one wave of blocks (384 slabs of a 14 x 14 grid: 24.3 -> 20.5 us;
 // 64 slabs of 56 x 56: 43 -> 39 us).
-// bwd_pool_tail is a stream over dQ, four rows in flight.  dQ and dV are read and written in fp32, which is the bound.  64 slabs of a
+// bwd_pool_tail is a stream over dQ, four rows in flight, beside the blocks of the other (64 slabs of 56 x 56, whole pass: 177.6 -> 174.4 us).  dQ and dV are read and written in fp32, which is the bound.  64 slabs of a
 // 56 x 56 grid: 39 us (154 MB, 24 us at the copy bandwidth) and 16 us (103 MB, 16 us); one kernel for dQ and dV with all nine window
 // loads of a token, and one for dWd, took 74 and 31.
 #include "common.cuh"
@@ -83,6 +83,10 @@ __device__ __forceinline__ Column column_of(const TailArgs& a, int i) {
     return {i - s * a.W, s * a.strip, min(a.H, (s + 1) * a.strip)};
 }
 
+// BESIDE: the kernel before is bwd_conv_tail, whose blocks release this one once the gradient stages are complete and touch nothing that it
+// does; so it runs beside them, and waits for their end before its own (what comes next waits for this kernel alone).  What the stages wrote
+// is read past L1, which was not emptied since.
+template <bool BESIDE>
 __global__ void __launch_bounds__(kThreadsQ, 4) bwd_pool_tail_kernel(const TailArgs a) {
     __shared__ Windows yw[kAxis];
     const int d = a.d, H = a.H, W = a.W, p = a.p, slab = blockIdx.y;
@@ -105,10 +109,12 @@ __global__ void __launch_bounds__(kThreadsQ, 4) bwd_pool_tail_kernel(const TailA
     const int groups = d >> 2, cols = kThreadsQ / groups;         // d <= 128: at least eight columns at once
     const int cg = threadIdx.x % groups, cl = threadIdx.x / groups;
     for (int i = threadIdx.x; i < min(H, kAxis); i += kThreadsQ) yw[i] = windows_of(i, H, p);
-    pdl_wait_prior();
-    pdl_release_next();
+    if (!BESIDE) {
+        pdl_wait_prior();
+        pdl_release_next();
+    }
     __syncthreads();
-    if (cl >= cols) return;
+    if (cl < cols) {
     const float* da = a.da + (size_t)slab * a.n * d + 4 * cg;
     const int first = blockIdx.x * a.passes * cols, last = min(first + a.passes * cols, a.strips * W);
     for (int i = first + cl; i < last; i += cols) {
@@ -121,7 +127,7 @@ __global__ void __launch_bounds__(kThreadsQ, 4) bwd_pool_tail_kernel(const TailA
             float4 q[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if (y + k < c.y1) q[k] = *reinterpret_cast<const float4*>(dq + (size_t)k * W * d);
+                if (y + k < c.y1) q[k] = __ldcg(reinterpret_cast<const float4*>(dq + (size_t)k * W * d));
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 if (y + k >= c.y1) break;
@@ -135,7 +141,7 @@ __global__ void __launch_bounds__(kThreadsQ, 4) bwd_pool_tail_kernel(const TailA
                         for (int l = 0; l < 2; ++l) {
                             const int area = (j ? wy.len1 : wy.len0) * (l ? wx.len1 : wx.len0);
                             if (area == 0) continue;
-                            const float4 g = __ldg(reinterpret_cast<const float4*>(da + (size_t)((wy.first + j) * p + wx.first + l) * d));
+                            const float4 g = __ldcg(reinterpret_cast<const float4*>(da + (size_t)((wy.first + j) * p + wx.first + l) * d));
                             const float inv = 1.f / (float)area;
                             pooled.x = fmaf(g.x, inv, pooled.x); pooled.y = fmaf(g.y, inv, pooled.y);
                             pooled.z = fmaf(g.z, inv, pooled.z); pooled.w = fmaf(g.w, inv, pooled.w);
@@ -146,6 +152,11 @@ __global__ void __launch_bounds__(kThreadsQ, 4) bwd_pool_tail_kernel(const TailA
             }
             dq += (size_t)4 * W * d;
         }
+    }
+    }
+    if (BESIDE) {
+        pdl_release_next();
+        pdl_wait_prior();
     }
 }
 
@@ -277,7 +288,7 @@ template <typename T> cudaError_t launch_tail(TailArgs a, int sm_count, cudaStre
     }
     dim3 grid = plan_strips(&a, 1, kThreadsQ / (a.d / 4), 4 * sm_count, 0, 4);
     if (a.dwd) ++grid.x;
-    return launch_dependent(bwd_pool_tail_kernel, grid, kThreadsQ, 0, st, a);
+    return launch_dependent(a.wd ? bwd_pool_tail_kernel<true> : bwd_pool_tail_kernel<false>, grid, kThreadsQ, 0, st, a);
 }
 
 }  // namespace
