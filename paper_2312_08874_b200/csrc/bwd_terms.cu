@@ -243,8 +243,10 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
     cudaError_t e;
 #define AA_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
     const bool umma = backward_terms_umma_eligible(dtype, slabs, n, N, d);
-    // (a single batch entry stores its bias gradients, and so does the first one of a block that has them all)
-    const bool clear_bias = slabs != c.heads && !(umma && backward_terms_umma_owned(slabs, c.heads, n, N, c.sm_count)), clear_rows = umma && n > 64;      // (blocks of 64 agents add to the rows)
+    const UmmaOrder order = umma ? backward_terms_umma_order(slabs, c.heads, n, N, d, c.sm_count) : UmmaOrder{};
+    // (a single batch entry stores its bias gradients, and so does the first one of a block that has them all; blocks of 64 agents add to the rows,
+    // unless one block has them all)
+    const bool clear_bias = slabs != c.heads && !order.stretch, clear_rows = umma && n > 64 && !order.all_agents;
     void *pad1 = nullptr, *pad2 = nullptr, *partial = nullptr;
     char* umma_ws = w + 3 * terms + up256((size_t)slabs * N * 8) + up256((size_t)slabs * n * 8);          // padded biases, partial states of V_A
     if (umma) backward_terms_umma_padded(c.heads, n, N, umma_ws, &pad1, &pad2, &partial);

@@ -88,6 +88,7 @@ struct Args {
     int bias;                 // 0: none; 1: tiles of token rows; 2: tiles of agent rows
     int chain;                // aggregation: all pairs of S in one accumulator, as where `stats` come from bwd_values_umma_kernel
     int owned;                // tiles of a stretch whose batch entries a block takes one after another (0: the sequence in its natural order)
+    int all;                  // and all blocks of agents of each
     float scale;
     alignas(64) CUtensorMap tm_x, tm_y, tm_a, tm_m, tm_b;
 };
@@ -117,31 +118,34 @@ __device__ __forceinline__ void load_joined(uint32_t taddr, float2 (&v)[16]) {
 __device__ __forceinline__ void st_shared4(uint32_t addr, const uint32_t (&v)[4]) {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
 }
-template <int MODE>
+// OWN: in one of the orders that p.owned says (the natural one has instantiations of its own, up to 6 % faster without their bookkeeping)
+template <int MODE, bool OWN>
 __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __grid_constant__ Args p) {
     constexpr bool BCAST = MODE == kBcast, AGG = MODE == kAgg, STATS = MODE == kStats;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int N = p.N, n = p.n, d = p.d;
-    const int ab = blockIdx.x % p.blocks, lanes = gridDim.x / p.blocks, me = blockIdx.x / p.blocks;      // block of 64 agents; runs of its sequence
-    // Natural order: a run of the (slab, tile) sequence.  Owned: a run of the (head, tile) sequence, cut into stretches of up to p.owned tiles of a
-    // head, all batch entries of a stretch in turn.
-    const int batch = p.owned ? p.slabs / p.heads : 1;
+    // Natural order: a run of the (slab, tile) sequence for one block of 64 agents.  Owned: a run of the (head, tile) sequence, cut into stretches of
+    // up to p.owned tiles of a head, all batch entries of a stretch in turn; p.all: of each, all blocks of agents in turn.
+    const bool all = OWN && p.all;
+    const int side = all ? 1 : p.blocks, lanes = gridDim.x / side, me = blockIdx.x / side;            // blocks of agents side by side; runs of the sequence
+    const int batch = OWN ? p.slabs / p.heads : 1;
     const long long total = (long long)p.slabs / batch * p.tiles, first = total * me / lanes, end = total * (me + 1) / lanes;
-    const int count = (int)(end - first) * batch;
-    long long at = first;                        // start of the role's current segment: tiles of one slab that follow one another
-    int entry = 0, slab = 0, tile = 0, left = 0, length = 0;                                // its current tile, and how many of the segment are left
+    const int count = (int)(end - first) * batch * (all ? p.blocks : 1);
+    int slab = (int)(first / p.tiles), tile = (int)(first - (long long)slab * p.tiles), ab = all ? 0 : blockIdx.x % side;      // of the role's current tile
+    long long at = first;                        // start of its current segment: tiles of one slab that follow one another, for one block of agents
+    int entry = 0, left = 0, length = 0;         // its batch entry, how many of its tiles are left
     bool fresh = true;                           // the first tile of a segment
     auto segment = [&] {
         slab = (int)(at / p.tiles);
         tile = (int)(at - (long long)slab * p.tiles);
-        length = (int)min(end - at, (long long)(p.tiles - tile));
-        if (p.owned) length = min(length, p.owned);
-        left = length;
+        left = length = min((int)min(end - at, (long long)(p.tiles - tile)), p.owned);
         slab += entry * p.heads;
     };
-    segment();
+    if (OWN) segment();
+    auto is_fresh = [&](int i) { return OWN ? fresh : i == 0 || tile == 0; };
+    auto is_last = [&](int i) { return OWN ? left == 1 : tile == p.tiles - 1 || i == count - 1; };
     const uint32_t base = smem_u32(smem);
 
     Pipe pp;
@@ -163,9 +167,16 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
     pdl_release_next();
     auto advance = [&] {
         ++tile;
+        if (!OWN) {
+            if (tile == p.tiles) { tile = 0; ++slab; }
+            return;
+        }
         fresh = --left == 0;
         if (!fresh) return;
-        if (++entry == batch) { entry = 0; at += length; }
+        if (!all || ++ab == p.blocks) {
+            if (all) ab = 0;
+            if (++entry == batch) { entry = 0; at += length; }
+        }
         segment();
     };
 
@@ -191,7 +202,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
                         tma_load_3d(to + kMat, &p.tm_b, tile * kTok + 64, ab * 64, head, bb);
                     }
                 }
-                if (fresh) {
+                if (is_fresh(i)) {
                     if (i > 0) wait_spin(pp, (STATS ? BAR_FREE : BAR_DONE) + (b ^ 1), (i - 1) >> 1, kTimeoutRole);  // the last tile of the segment before
                     const uint32_t bam = pipe_bar(pp, BAR_AM), am = base + OFF_AM;
                     mbar_arrive_expect_tx(bam, 2 * kTerms * kMat);
@@ -210,7 +221,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
         int groups = 0;
         for (int i = 0; i < count && !pipe_dead(pp); ++i, advance()) {
             const int b = i & 1;
-            if (fresh) wait_spin(pp, BAR_AM, groups++, kTimeoutTile);
+            if (is_fresh(i)) wait_spin(pp, BAR_AM, groups++, kTimeoutTile);
             wait_spin(pp, BAR_FULL + b, i >> 1, kTimeoutTile);
             if (i > 0) wait_spin(pp, BAR_READ, i - 1, kTimeoutRole);
             tc_fence_after_sync();
@@ -317,13 +328,13 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
                         for (int j = 0; j < 8; ++j) {
                             if (8 * j >= d) break;
                             const float2 v = make_float2(scale * o[4 * j + 2 * h], scale * o[4 * j + 2 * h + 1]);
-                            if (p.blocks == 1) *reinterpret_cast<float2*>(r + 8 * j) = v;
+                            if (p.blocks == 1 || (all && ab == 0)) *reinterpret_cast<float2*>(r + 8 * j) = v;      // (the others follow from the same thread)
                             else red_add2(r + 8 * j, v.x, v.y);
                         }
                     }
                 }
             }
-            if (sums && left == 1) {                                   // the last tile of the segment
+            if (sums && is_last(i)) {                                  // the last tile of the segment
                 float* dst = second ? p.outer1 : p.outer0;
                 const float scale = second ? p.scale : 1.f;
 #pragma unroll
@@ -348,7 +359,6 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
         float2* s_stat = reinterpret_cast<float2*>(smem + OFF_STAT);
         int parity = 0;
         const float2 none = make_float2(INFINITY, 0.f);                // (a token or an agent that does not exist: its probabilities are zero)
-        const int c0 = ab * 64 + 32 * half, lim = n - c0;              // columns of this half that exist
         float2 next = none;
         if (BCAST && tile * kTok + r < N) next = __ldg(p.stats + (size_t)slab * N + tile * kTok + r);
         uint32_t bw[16];                                               // 32 biases as pairs, read a tile ahead
@@ -380,18 +390,19 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
         };
         load_bias(0);
         for (int i = 0; i < count; ++i) {
-            const int now = slab, at_tile = tile;                      // this tile; the role's state goes on to the next
-            const bool first_tile = fresh;
+            const int now = slab, at_tile = tile, block = ab;          // this tile; the role's state goes on to the next
+            const int c0 = block * 64 + 32 * half, lim = n - c0;       // columns of this half that exist
+            const bool first_tile = is_fresh(i);
             if (i + 1 < count) advance();
             const int b = i & 1, tok = at_tile * kTok + r, head = now % p.heads;
-            const bool ok = tok < N, store = p.slabs == p.heads || (p.owned && now < p.heads);      // a head's first batch entry, here before the others
+            const bool ok = tok < N, store = p.slabs == p.heads || (OWN && now < p.heads);      // a head's first batch entry, here before the others
             const float2 st = next;
             if (BCAST) {
                 next = none;
                 if (i + 1 < count && tile * kTok + r < N) next = __ldg(p.stats + (size_t)slab * N + tile * kTok + r);
             } else if (AGG && first_tile) {                                 // another segment: its statistics
                 parity ^= 1;
-                if (tid < 64) s_stat[parity * 64 + tid] = ab * 64 + tid < n ? __ldg(p.stats + (size_t)now * n + ab * 64 + tid) : none;
+                if (tid < 64) s_stat[parity * 64 + tid] = block * 64 + tid < n ? __ldg(p.stats + (size_t)now * n + block * 64 + tid) : none;
                 bar_named(1, kRowThreads);
             }
             wait_par(pp, BAR_S, i, kTimeoutTile);
@@ -434,7 +445,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
                     const float mm = fmaxf(m, o.x), f = m == -INFINITY ? 0.f : exp2f(m - mm), fo = o.x == -INFINITY ? 0.f : exp2f(o.x - mm);
                     const float tot = fmaf(l, f, o.y * fo), dt = fmaf(dot, f, o.z * fo);
                     if (p.blocks == 1) p.tok_stats[(size_t)now * N + tok] = make_float2(mm + log2f(tot), dt / tot);
-                    else p.partial[((size_t)ab * p.slabs + now) * N + tok] = make_float4(mm, tot, dt, 0.f);
+                    else p.partial[((size_t)block * p.slabs + now) * N + tok] = make_float4(mm, tot, dt, 0.f);
                 }
                 if (i + 1 < count) load_bias(i + 1);
                 continue;
@@ -548,12 +559,13 @@ __global__ void __launch_bounds__(256) bwd_stats_merge_kernel(const float4* part
     stats[i] = make_float2(m + log2f(l), dot / l);
 }
 
-template <int MODE> cudaError_t launch(const Args& a, int sm_count, cudaStream_t st) {
+template <int MODE, bool OWN> cudaError_t launch(const Args& a, int sm_count, cudaStream_t st) {
     static std::atomic<unsigned long long> done;
-    cudaError_t e = allow_smem(bwd_terms_umma_kernel<MODE>, done, kSmemBytes);
+    cudaError_t e = allow_smem(bwd_terms_umma_kernel<MODE, OWN>, done, kSmemBytes);
     if (e != cudaSuccess) return e;
-    const long long total = (long long)(a.owned ? a.heads : a.slabs) * a.tiles, lanes = std::min<long long>(total, std::max(1, sm_count / a.blocks));
-    return launch_dependent(bwd_terms_umma_kernel<MODE>, dim3((unsigned)(lanes * a.blocks)), kThreads, kSmemBytes, st, a);
+    const int side = a.all ? 1 : a.blocks;
+    const long long total = (long long)(OWN ? a.heads : a.slabs) * a.tiles, lanes = std::min<long long>(total, std::max(1, sm_count / side));
+    return launch_dependent(bwd_terms_umma_kernel<MODE, OWN>, dim3((unsigned)(lanes * side)), kThreads, kSmemBytes, st, a);
 }
 
 }  // namespace
@@ -574,15 +586,28 @@ bool backward_terms_umma_eligible(int dtype, int slabs, int n, int N, int d) {
     return n > 16 && (N >= 8192 || (N <= 256 && tokens >= 28000));
 }
 
-// Tiles of a stretch of the token axis whose batch entries one block takes in turn (0: runs of slabs).  A block that has all batch entries of its tiles
-// stores the first one's bias gradients and adds the others' to them: nothing is cleared, and what is added to is still in L2 (a reduction of 32 KB
-// on every SM: 1650 cycles where L2 holds the sums, 3400 where it does not).  A stretch ends with a change of A and M; two batch entries of
-// eight heads on a 128 x 128 grid, 256 agents, whole pass: 1176 us in the natural order; stretches of 28, 10, 4 and 2 tiles 1126, 1108, 1096 and 1084.
-int backward_terms_umma_owned(int slabs, int heads, int n, int N, int sm_count) {
-    constexpr int kStretch = 4;
+// Order of the work (see the kernel).  A block that has all batch entries of its tiles stores the first one's bias gradients and adds the others' to them:
+// nothing is cleared, and what is added to is still in L2 (a reduction of 32 KB on every SM: 1650 cycles where L2 holds the sums, 3400 where it
+// does not).  The same goes for the rows of dQ, dK and dV and a block that has all blocks of agents.  A stretch ends with a change of A and M, so
+// runs have to be long and even.  Whole pass in us, 148 SMs, natural order / all batch entries, stretches of 4, 8 and 16 tiles / all agents, too,
+// stretches of 2, 4 and 8:
+//   two batch entries of 8 heads, 128 x 128 tokens, 256 agents (6.9 tiles a block)   1248 / 1147 1149 1173 / 1064 1083 1188
+//   one of 8 heads, 128 x 128, 256                                                    602 /  596  597  603 /  563  568  626
+//   two of 8 heads, 92 x 151, 81 (5.9)                                                667 /  640  641  652 /  604  605  606
+//   two of 8 heads, 75 x 117, 144 (3.7)                                               600 /  591  595  601 /  555  591  589
+//   one of 8 heads, 75 x 117, 256 agents of 40 channels (3.7)                         393 /  398  397  392 /  416  425  427
+//   eight of 2 heads, 128 x 128, 196 agents of 40 channels (6.9 a run of four)       1152 / 1115 1197 1202
+//   fourteen of 2 heads, 75 x 117, 144 agents of 40 channels (2.8 a run of three)     864 /  995
+//   four of 4 heads, 128 x 128, 144 agents of 40 channels (10.4 a run of three)       887 /  931
+//   one of 8 heads, 92 x 151, 256 agents of 40 channels (5.9)                         549 /   -              /  584
+UmmaOrder backward_terms_umma_order(int slabs, int heads, int n, int N, int d, int sm_count) {
     const long long tiles = (long long)heads * ((N + kTok - 1) / kTok), blocks = (n + 63) / 64, lanes = std::max<long long>(1, sm_count / blocks);
-    if (slabs == heads || tiles < 8 * lanes) return 0;                  // (blocks have whole tiles of the axis: one more for some than for others)
-    return kStretch;
+    // blocks have whole tiles of the axis, one more for some than for others: at most an eighth above the average
+    auto even = [&](long long runs) { return (tiles + runs - 1) / runs * runs * 8 <= tiles * 9; };
+    const bool wide = d > 48;                                           // (narrow rows: less to clear)
+    if (blocks > 1 && tiles >= (slabs == heads ? 5 : 3) * (long long)sm_count && even(sm_count) && (wide || slabs != heads)) return {2, 1};
+    if (wide && slabs != heads && tiles >= 4 * lanes && even(lanes) && 4LL * heads * n * N >= 24 << 20) return {4, 0};
+    return {0, 0};
 }
 
 size_t backward_terms_umma_bytes(int slabs, int heads, int n, int N) {
@@ -611,7 +636,8 @@ cudaError_t launch_backward_terms_umma(BwdTermsUmma stage, const BwdCall& c, con
     a.row0 = queries ? c.dq : c.dk; a.row1 = c.dv;
     a.dbias = queries ? c.db2 : c.db1;
     a.chain = backward_values_eligible(c.slabs, c.n, N);
-    a.owned = a.dbias && stage != kUmmaStats ? backward_terms_umma_owned(c.slabs, c.heads, c.n, N, c.sm_count) : 0;
+    const UmmaOrder order = backward_terms_umma_order(c.slabs, c.heads, c.n, N, c.d, c.sm_count);
+    if (stage != kUmmaStats) { a.owned = order.stretch; a.all = order.all_agents; }
     a.scale = queries ? c.scale2 : c.scale1;
     if (!make_map_3d_u16(&a.tm_x, queries ? c.q : c.k, c.slabs, N, c.d, kTok) || !make_map_3d_u16(&a.tm_y, queries ? c.d_out : c.v, c.slabs, N, c.d, kTok) ||
         !make_map_3d_u16(&a.tm_a, a_t, (uint64_t)kTerms * c.slabs, c.n, c.d, 64) || !make_map_3d_u16(&a.tm_m, m_t, (uint64_t)kTerms * c.slabs, c.n, c.d, 64))
@@ -619,9 +645,9 @@ cudaError_t launch_backward_terms_umma(BwdTermsUmma stage, const BwdCall& c, con
     if (bias && !(padded ? make_map_3d_u16(&a.tm_b, padded, c.heads, N, bias_width(c.n), kTok)
                   : queries ? make_map_3d_u16(&a.tm_b, bias, c.heads, N, c.n, kTok) : make_map_3d_u16(&a.tm_b, bias, c.heads, c.n, N, 64)))
         return cudaErrorInvalidValue;
-    if (stage == kUmmaBroadcast) return launch<kBcast>(a, c.sm_count, st);
-    if (stage == kUmmaAggregate) return launch<kAgg>(a, c.sm_count, st);
-    cudaError_t e = launch<kStats>(a, c.sm_count, st);
+    if (stage == kUmmaBroadcast) return a.owned ? launch<kBcast, true>(a, c.sm_count, st) : launch<kBcast, false>(a, c.sm_count, st);
+    if (stage == kUmmaAggregate) return a.owned ? launch<kAgg, true>(a, c.sm_count, st) : launch<kAgg, false>(a, c.sm_count, st);
+    cudaError_t e = launch<kStats, false>(a, c.sm_count, st);
     if (e != cudaSuccess || a.blocks == 1) return e;
     const long long tokens = (long long)c.slabs * N;
     return launch_dependent(bwd_stats_merge_kernel, dim3((unsigned)((tokens + 255) / 256)), 256, 0, st, (const float4*)a.partial, stats, tokens, a.blocks);

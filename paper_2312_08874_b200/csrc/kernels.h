@@ -293,8 +293,10 @@ cudaError_t launch_backward_terms(int dtype, const BwdCall& c, void* ws, cudaStr
 // the gradient stages of that on the 5th-generation tensor cores (bf16 inputs of up to 64 channels)
 bool backward_terms_umma_eligible(int dtype, int slabs, int n, int N, int d);
 enum BwdTermsUmma { kUmmaStats, kUmmaBroadcast, kUmmaAggregate };
-// whether (and in stretches of how many tiles) their blocks own the bias gradients of their tiles, which then need not be cleared
-int backward_terms_umma_owned(int slabs, int heads, int n, int N, int sm_count);
+// Order of their work: stretches of so many tiles whose batch entries a block takes in turn (0: slab by slab), and with them all blocks of 64 agents.
+// It owns their bias gradients then, or the rows of dQ, dK and dV, which need not be cleared.
+struct UmmaOrder { int stretch, all_agents; };
+UmmaOrder backward_terms_umma_order(int slabs, int heads, int n, int N, int d, int sm_count);
 // Workspace: biases as token rows (null where they are read as they are), token statistics per block of agents
 size_t backward_terms_umma_bytes(int slabs, int heads, int n, int N);
 void backward_terms_umma_padded(int heads, int n, int N, void* ws, void** b1, void** b2, void** partial);

@@ -22,7 +22,9 @@ SHAPES = [
     (3, 2, 64, 43, 64, 13, "bf16", False),    # two blocks, runs that hold parts of two slabs
     (1, 1, 70, 41, 64, 9, "bf16", True),      # agent values: 24 states a row, three for a warp
     (1, 2, 64, 65, 40, 6, "bf16", True),      # two rows per agent, 66 states, slabs that begin inside a run
-    (3, 4, 95, 100, 32, 16, "bf16", True),    # 300 tiles of the axis on 37 runs: blocks own their bias gradients, stretches that end with a run or a head
+    (3, 4, 95, 100, 56, 16, "bf16", True),    # 300 tiles of the axis on 37 runs: blocks own their bias gradients, stretches that end with a run or a head
+    (2, 2, 168, 169, 32, 9, "bf16", True),    # three tiles of the axis a block, with both blocks of agents and batch entries; the last one is ragged
+    (1, 8, 111, 128, 56, 9, "bf16", True),    # six, one batch entry
 ]
 
 
