@@ -30,7 +30,7 @@ namespace {
 constexpr int TH = 8, TW = 16, QT = TH * TW;             // tile
 constexpr int NROW = 512, NOUT = 256;                    // threads: two teams of 256, output warps
 constexpr int NT = NROW + NOUT + 256;                    // + five warps of roles (three idle: register splits go by four warps)
-constexpr int kRowRegs = 72, kOutRegs = 72, kRoleRegs = 32;        // of 64 at launch
+constexpr int kRowRegs = 72, kOutRegs = 80, kRoleRegs = 32;        // of 64 at launch
 static_assert(NROW * kRowRegs + NOUT * kOutRegs + 256 * kRoleRegs <= NT * 64, "register split");
 constexpr int kTile = 64 * 128;                          // swizzled [64][64] tile of 16-bit elements
 constexpr float kTau = 5.5f;
@@ -211,7 +211,8 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
         set_regs_inc<kOutRegs>();
         const int q = warp & 3, half = (warp >> 2) & 1, c0 = 32 * half, lg = lane >> 2;
         const uint32_t* tab = filter_lane(reinterpret_cast<const uint32_t*>(smem + OFF_TAB) + c0, reinterpret_cast<const uint32_t*>(smem + OFF_ZEROS), lane);
-        const uint32_t zeros = smem_u32(smem + OFF_ZEROS);
+        uint32_t at[6];
+        patch_offsets<TW + 2>(at, 2 * q * (TW + 2), 64 * half, lane);
         T* gO = static_cast<T*>(p.out) + tok_offset(p.lout, slab, p.heads, 0);
         const size_t so = (size_t)p.lout.st;
         wait_par(pp, BAR_PREP, 0, kTimeoutLoads);
@@ -226,8 +227,7 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
                     for (int e = 0; e < 4; ++e) o[mt][jj][e] = 0.f;
             if (has_dwc) {
                 wait_par(pp, BAR_H_FULL + team, k, kTimeoutLoads);
-                // rows 16 mt .. of the warp are a row of the patch; those of the next one sit a row of the window on
-                dwc_rows<T, TW + 2>(o, sH + team * kHalo, 2 * q * (TW + 2) + (lane & 15), 64 * half, tab, lane, [](int u, int v) { return u * (TW + 2) + v; });
+                dwc_patch<T>(o, at, sH + team * kHalo, tab);
                 // The window goes back to TMA: an arrival overtakes loads that are still queued, so the arriving lane hangs on the products of
                 // what was loaded.
                 uint32_t x = 0u;

@@ -406,7 +406,7 @@ __global__ void __launch_bounds__(NT, 2) slab_umma_kernel(const __grid_constant_
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt) in[mt] = window_taps(16 * mt + (lane & 15) < limit ? t0 + 16 * mt : N, N, p.H, p.W, 1.f / (float)p.W, lane);
         const uint32_t* tab = filter_lane(sTab + c0, reinterpret_cast<const uint32_t*>(smem + OFF_ZERO), lane);
-        dwc_rows<T, 16>(o, sV, t0, 2 * c0, in, base + OFF_ZERO, tab, lane, [&](int u, int v) { return (u - 1) * p.W + v - 1; });
+        dwc_rows<T>(o, sV, t0, 2 * c0, in, base + OFF_ZERO, tab, lane, [&](int u, int v) { return (u - 1) * p.W + v - 1; });
     }
     wait_par(pp, BAR_O, 0, kTimeoutTile);
     tc_fence_after_sync();
