@@ -20,12 +20,11 @@
 // bwd_values_umma.cu made the statistics.  (With the pairs apart there, and a common part of 8 in the logits, dV of four slabs of 64 x 64 tokens,
 // 81 agents, was 3.8e-7 too large; 5e-8 in one chain.  With statistics from bwd_sums_kernel it is the other way round: 4e-8 and 4.5e-7.)
 //
-// What bounds it: the broadcast, fp32 reductions, about 2 TB/s (a tile adds 32 KB of bias gradients and 32 KB of dQ): without them a tile takes
-// 6000 cycles of 9400, of which splitting and storing terms is 2000 beside operand reads of the tensor pipe.  The aggregation takes as long
-// without any: it waits 4000 cycles of a tile for products, whose operands are read from shared memory again for every pair of terms.
-// 16 slabs of a 128 x 128 grid, 256 agents, biases: broadcast 336 us, aggregation 412 us, statistics 88 + 6 us; on mma.sync (bwd_sums_kernel,
-// bwd_rows_kernel) 828, 1010 and 242 us.  192 slabs of 14 x 14, 81 agents, whole pass: 313 -> 187 us; one slab of 40 x 23, 49 agents of 32
-// channels: 62 -> 51 us.
+// What bounds it: the products, whose operands are read from shared memory again for every pair of terms (3900 to 4700 cycles of the tensor pipe a tile),
+// beside splitting and storing terms (2000), and fp32 reductions (a tile adds 32 KB of bias gradients and 32 or 64 KB of rows): see
+// backward_terms_umma_order.  16 slabs of a 128 x 128 grid, 256 agents, biases: broadcast 355 us, aggregation 447 us with nothing cleared before them
+// (342 and 420 after 107 us of clearing), statistics 87 + 6 us; on mma.sync (bwd_sums_kernel, bwd_rows_kernel) 828, 1010 and 242 us.  192 slabs of
+// 14 x 14, 81 agents, whole pass: 313 -> 187 us; one slab of 40 x 23, 49 agents of 32 channels: 62 -> 51 us.
 #include "bwd_terms_launch.cuh"
 #include "stream_common.cuh"
 
