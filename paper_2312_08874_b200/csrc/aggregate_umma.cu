@@ -68,7 +68,8 @@ struct UmmaAggArgs {
 };
 }  // namespace
 
-template <typename T>
+// ROUNDED: see umma_sums_rounded
+template <typename T, bool ROUNDED>
 __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_constant__ UmmaAggArgs g) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ int s_dead;
@@ -231,9 +232,10 @@ __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_cons
                         const float2 a1 = ffma2(make_float2(sv[2 * i + 2], sv[2 * i + 3]), l2e, nb2);
                         const float2 p01 = make_float2(fast_exp2(a0.x), fast_exp2(a0.y));     // exp2(-inf) = 0 past the range
                         const float2 p23 = make_float2(fast_exp2(a1.x), fast_exp2(a1.y));
-                        s01 = fadd2(s01, p01); s23 = fadd2(s23, p23);
                         pk[i] = pack2<T>(p01.x, p01.y);
                         pk[i + 1] = pack2<T>(p23.x, p23.y);
+                        if (ROUNDED) { add_pair<T>(s01, pk[i]); add_pair<T>(s23, pk[i + 1]); }
+                        else { s01 = fadd2(s01, p01); s23 = fadd2(s23, p23); }
                     }
                     l += (s01.x + s01.y) + (s23.x + s23.y);
                 }
@@ -404,7 +406,7 @@ AggPlan plan_aggregate_umma(int slabs, int n_agents, int n_tokens, int d, int sm
 
 template <typename T>
 static cudaError_t launch_umma_t(const UmmaAggArgs& g, cudaStream_t st) {
-    auto kern = aggregate_umma_kernel<T>;
+    auto kern = umma_sums_rounded(g.a.cols, g.a.d) ? aggregate_umma_kernel<T, true> : aggregate_umma_kernel<T, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     dim3 grid(g.a.splits, g.a.slabs);

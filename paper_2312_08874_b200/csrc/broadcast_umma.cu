@@ -81,7 +81,8 @@ struct UmmaBcArgs {
 };
 }  // namespace
 
-template <typename T>
+// ROUNDED: see umma_sums_rounded
+template <typename T, bool ROUNDED>
 __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_constant__ UmmaBcArgs g) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -353,9 +354,10 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
                         const float2 a1 = ffma2(make_float2(sv[2 * k + 2], sv[2 * k + 3]), l2e, nb2);
                         const float2 p01 = make_float2(fast_exp2(a0.x), fast_exp2(a0.y));     // exp2(-inf) = 0 past the last agent
                         const float2 p23 = make_float2(fast_exp2(a1.x), fast_exp2(a1.y));
-                        s01 = fadd2(s01, p01); s23 = fadd2(s23, p23);
                         pk[k] = pack2<T>(p01.x, p01.y);
                         pk[k + 1] = pack2<T>(p23.x, p23.y);
+                        if (ROUNDED) { add_pair<T>(s01, pk[k]); add_pair<T>(s23, pk[k + 1]); }
+                        else { s01 = fadd2(s01, p01); s23 = fadd2(s23, p23); }
                     }
                     l += (s01.x + s01.y) + (s23.x + s23.y);
                 }
@@ -400,7 +402,7 @@ bool broadcast_umma_eligible(int dtype, int n_agents, int n_tokens, int d) {
 
 template <typename T>
 static cudaError_t launch_bc_umma_t(const UmmaBcArgs& g, int splits, cudaStream_t st) {
-    auto kern = broadcast_umma_kernel<T>;
+    auto kern = umma_sums_rounded(g.a.rows, g.a.d) ? broadcast_umma_kernel<T, true> : broadcast_umma_kernel<T, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     dim3 grid(splits, g.a.slabs);

@@ -108,6 +108,14 @@ template <> __device__ __forceinline__ float2 unpack2<__nv_bfloat16>(uint32_t w)
 template <> __device__ __forceinline__ float2 unpack2<__half>(uint32_t w) {
     return __half22float2(*reinterpret_cast<const __half2*>(&w));
 }
+// s += the pair
+template <typename T> __device__ __forceinline__ void add_pair(float2& s, uint32_t w);
+template <> __device__ __forceinline__ void add_pair<__nv_bfloat16>(float2& s, uint32_t w) {
+    asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %2;\n\tadd.rn.f32.bf16 %0, l, %0;\n\tadd.rn.f32.bf16 %1, h, %1;\n\t}\n" : "+f"(s.x), "+f"(s.y) : "r"(w));
+}
+template <> __device__ __forceinline__ void add_pair<__half>(float2& s, uint32_t w) {
+    asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %2;\n\tadd.rn.f32.f16 %0, l, %0;\n\tadd.rn.f32.f16 %1, h, %1;\n\t}\n" : "+f"(s.x), "+f"(s.y) : "r"(w));
+}
 
 // ------------------------------------------------------------------------------- small PTX
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {

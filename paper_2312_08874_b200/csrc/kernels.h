@@ -116,6 +116,10 @@ AggPlan plan_aggregate_simt(int slabs, int n_agents, int n_tokens, int d, int sm
 cudaError_t launch_aggregate_simt(int dtype, const AttnArgs& p, const AggPlan& plan, cudaStream_t st);
 cudaError_t launch_broadcast_simt(int dtype, const AttnArgs& p, cudaStream_t st);
 // tensor-memory (tcgen05) kernels for large agent counts (aggregate_umma.cu)
+// Whether the kernels for large agent counts add up their probabilities as rounded, so that weights and normaliser agree, as on register tiles
+// (else they are up to 2^-9 / sqrt(agents) apart in bf16).  It costs 2 % of the whole pass (16 slabs of 64 x 64 tokens, 256 agents of 40
+// channels 41.0 -> 41.9 us, of 128 x 128, 64 channels 110.8 -> 112.7), so wide rows on long axes, which never ran on register tiles, go without.
+inline bool umma_sums_rounded(int n_tokens, int d) { return n_tokens < 8192 || d <= 48; }
 bool aggregate_umma_eligible(int dtype, int n_agents, int n_tokens, int d, bool has_bias);
 AggPlan plan_aggregate_umma(int slabs, int n_agents, int n_tokens, int d, int sm_count);
 cudaError_t launch_aggregate_umma(int dtype, const AttnArgs& p, const AggPlan& plan, cudaStream_t st);

@@ -49,3 +49,21 @@ def test_patches_and_steps(case, rising):
         hd = lambda x: None if x is None else to_np(x[h:h + 1])
         ref = orc.forward(one(inp["q"]), one(inp["k"]), one(inp["v"]), H, W, agents=one(agents), b1=hd(b1), b2=hd(b2), dwc_weight=hd(inp["dwc"]), threads=orc.max_threads())
         assert_close(out[b:b + 1, h:h + 1], ref, dtype, f"{case} slab {(b, h)}")
+
+
+@pytest.mark.parametrize("n,dtype", [(256, "bf16"), (128, "bf16"), (256, "f16")])
+def test_partial_states_of_the_aggregation_hold_the_weights_as_rounded(n, dtype):
+    """With values of one, a row of a partial state's sums of products and its sum of weights are the same numbers added up: 8 tiles of 64 tokens a
+    block, so at most 19 fp32 roundings of one and 16 of the other, 35 x 2^-23 = 4.2e-6 apart.  (Weights before rounding: 2^-9 / sqrt(512) in bf16.)"""
+    w = Workload("states", 4, 8, 32, 64, 64, 16, dtype, True, False, 1.0, seed=77)
+    inp = make_inputs(w, bias_std=0.5)
+    mod = make_module(w, max_agents=n)
+    a, k = (torch.randn((4, 8, m, 64), generator=torch.Generator().manual_seed(m)).to(inp["q"].dtype).cuda() for m in (n, 2048))
+    ws = torch.zeros(mod.workspace_bytes(1, 2048, n), dtype=torch.uint8, device="cuda")
+    mod.aggregate(a, k, torch.ones_like(k), b1=to_dev(inp["b1"][:, :n].contiguous()), workspace=ws)
+    assert mod.last_launch_count() == 2 and mod.query_status() == 0
+    rows = (n + 127) // 128 * 128
+    state = ws[2 * a.numel() * 2:].view(torch.float32)[:rows * 66]                # the first block's: maxima, sums, products [rows][64]
+    sums, products = state[rows:2 * rows][:n], state[2 * rows:].view(rows, 64)[:n]
+    assert float(sums.min()) > 0
+    assert float((products / sums[:, None] - 1).abs().max()) <= 4.2e-6

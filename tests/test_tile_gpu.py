@@ -37,7 +37,15 @@ def test_tile_edges_match_oracle(case):
     assert torch.equal(out, gpu_forward(mod, w, inp)), "bit-reproducible"
 
 
-@pytest.mark.parametrize("case", [(2, 2, 14, 14, 64, 7, "bf16"), (1, 2, 45, 45, 64, 11, "f16"), (1, 1, 33, 32, 40, 16, "bf16")], ids=["one_kernel", "three_kernels", "d40"])
+WEIGHTS = {
+    "one_kernel": (2, 2, 14, 14, 64, 7, "bf16"), "three_kernels": (1, 2, 45, 45, 64, 11, "f16"), "d40": (1, 1, 33, 32, 40, 16, "bf16"),
+    # tensor memory, where register tiles are the other choice
+    "short_slabs": (128, 3, 14, 14, 64, 7, "bf16"), "latent_grid": (2, 8, 64, 64, 40, 16, "bf16"), "latent_grid_f16": (2, 8, 64, 64, 40, 16, "f16"),
+    "short_axis": (4, 8, 32, 64, 64, 16, "bf16"), "half_filled": (1, 2, 56, 144, 64, 12, "bf16"),
+}
+
+
+@pytest.mark.parametrize("case", list(WEIGHTS.values()), ids=list(WEIGHTS))
 def test_weights_and_their_sums_agree(case):
     """Values that are all one, less themselves through the depthwise term: what is left is how far the rounded weights are from adding up to
     their normaliser.  Both are sums of the same 16-bit numbers, rounded once per 16 of at most 256: 2 x 16 x 2^-23 = 4e-6.  (A normaliser of
