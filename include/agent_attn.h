@@ -56,7 +56,7 @@ typedef enum {
 
 typedef enum {
     AA_PATH_AUTO = 0,         /* bf16/f16: three streaming kernels for long token grids with few agents (n <= 64, d = 64,
-                                 N >= 1024, W >= 8), tensor-memory kernels for many agents (72 <= n <= 256, d <= 64)
+                                 N >= 1024 a multiple of 8, 8 <= W <= 64, pooling windows of one size), tensor-memory kernels for many agents (72 <= n <= 256, d <= 64)
                                  on long axes or large batches, one tensor-memory block per slab for batches of short
                                  slabs (N <= 256, n <= 64, d <= 64), register-tiled kernels for everything else, in one
                                  kernel on short grids.  f32: operands as three bf16 terms on the tensor cores (fp32

@@ -118,7 +118,7 @@ const StreamPlan& stream_plan_for(agent_attn_handle* h, int grid_h, int grid_w, 
     if (h->stream_key[0] != grid_h || h->stream_key[1] != grid_w || h->stream_key[2] != n_agents ||
         h->stream_key[3] != (pooled ? 1 : 2)) {
         h->stream_plan = (h->cfg.path == AA_PATH_AUTO && h->cfg.dtype != AA_F32)
-                             ? plan_stream(h->cfg.dtype, h->cfg.batch * h->cfg.heads, h->cfg.heads, grid_h, grid_w, h->cfg.head_dim,
+                             ? plan_stream(h->cfg.dtype, h->cfg.batch * h->cfg.heads, grid_h, grid_w, h->cfg.head_dim,
                                            n_agents, pooled, h->sm_count)
                              : StreamPlan{};
         h->stream_key[0] = grid_h; h->stream_key[1] = grid_w; h->stream_key[2] = n_agents;
@@ -152,7 +152,7 @@ WsLayout ws_layout(const agent_attn_handle* h, int n_tokens, int n_agents, int g
         // the larger of the plans for pooled and for caller-supplied agents (the size must not depend on A)
         for (int pooled = 0; pooled < 2; ++pooled) {
             const StreamPlan sp = (h->cfg.path == AA_PATH_AUTO && h->cfg.dtype != AA_F32)
-                                      ? plan_stream(h->cfg.dtype, (int)slabs, h->cfg.heads, grid_h, grid_w, h->cfg.head_dim, n_agents, pooled != 0, h->sm_count)
+                                      ? plan_stream(h->cfg.dtype, (int)slabs, grid_h, grid_w, h->cfg.head_dim, n_agents, pooled != 0, h->sm_count)
                                       : StreamPlan{};
             if (sp.ok) extra = stream_extra_bytes((int)slabs, h->cfg.heads, n_tokens, n_agents);
         }

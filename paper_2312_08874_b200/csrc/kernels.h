@@ -203,8 +203,8 @@ struct StreamPlan {
     bool ok;
     int splits;          // aggregation blocks per slab
     int tiles_per_split; // 128-token tiles per aggregation block
-    int rows_b, cols_b;  // grid rows and columns of a broadcast tile (at most 128 tokens)
-    int tiles_x, tiles_b;    // broadcast tiles per band of rows, and per slab
+    int rows_b;          // grid rows per broadcast tile (rows_b * W <= 128 tokens)
+    int tiles_b;         // broadcast tiles per slab
     int grid_b;          // broadcast blocks (persistent)
     int smem_b;          // dynamic shared memory of a broadcast block
 };
@@ -224,7 +224,7 @@ struct StreamArgs {
     StreamPlan plan;
     alignas(64) CUtensorMap tm_k, tm_v, tm_b1, tm_q, tm_b2, tm_h, tm_a2, tm_va;
 };
-StreamPlan plan_stream(int dtype, int slabs, int heads, int H, int W, int d, int n_agents, bool pooled, int sm_count);
+StreamPlan plan_stream(int dtype, int slabs, int H, int W, int d, int n_agents, bool pooled, int sm_count);
 // workspace beyond A and V_A: bytes of (a1s | a2s | b1c | b2p), each 256-byte aligned, in this order
 size_t stream_extra_bytes(int slabs, int heads, int N, int n_agents);
 bool stream_make_maps(StreamArgs* a);

@@ -2,13 +2,13 @@
 // for small agent counts (n <= 64, d = 64, 16-bit elements) as a streaming kernel on the 5th-generation
 // tensor cores: both attention products AND the depthwise 3x3 term run on tcgen05.
 //
-// Persistent blocks, one per SM; block c walks a contiguous run of the (slab, tile) sequence.  A tile is R
-// grid rows by C columns (all of them up to 64, else an even share) in a padded token index: row i of every 128-row operand is (tile row r, padded column xp) with
-// i = r (C + 2) + xp, xp = 0 and xp = C + 1 being pad positions whose results are dropped (R (C + 2) <= 128).
+// Persistent blocks, one per SM; block c walks a contiguous run of the (slab, row tile) sequence.  A tile is R
+// whole grid rows in a padded token index: row i of every 128-row operand is (tile row r, padded column xp) with
+// i = r (W + 2) + xp, xp = 0 and xp = W + 1 being pad positions whose results are dropped (R (W + 2) <= 128).
 // The depthwise term on the tensor core: for tap (u, v) the V rows of the tile, with one grid row above and
-// below and a column more at either end (all filled in by one TMA box: coordinates outside the grid read zero),
+// below and a zero column at either end (all filled in by one TMA box: coordinates outside the grid read zero),
 // sit in shared memory as a K-major, 128-byte-swizzled tile; the swizzle is a function of the address, so an
-// operand may start at any row: the tap's operand is the same tile started u (C + 2) + v - 1 rows later.  Times
+// operand may start at any row: the tap's operand is the same tile started u (W + 2) + v - 1 rows later.  Times
 // a diagonal weight slice (16 channels at a time) it accumulates w[c][u][v] V[y+u-1][x+v-1][c] over the nine
 // taps into its own tensor-memory accumulator, in fp32: 36 small instructions per tile and no stencil code.
 //   warp 8 "producer":  one lane issues every TMA copy: Q tile and padded-B2 tile (two stages), V rows (two
@@ -24,8 +24,6 @@
 //       rounded once, stored (pad positions skipped).
 // Every wait is bounded.  No TMA multicast, no clusters.
 #include "stream_common.cuh"
-
-#include <algorithm>
 
 namespace aa {
 
@@ -48,12 +46,12 @@ static_assert(OFF_QB % 1024 == 0, "swizzled tiles need 1024-byte alignment");
 struct BcLayout {
     int wp, tq, qsz, hsz, off_h, total;
 };
-__host__ __device__ inline BcLayout bc_layout(int R, int C) {
+__host__ __device__ inline BcLayout bc_layout(int R, int W) {
     BcLayout l;
-    l.wp = C + 2;
+    l.wp = W + 2;
     l.tq = R * l.wp;                                         // operand rows that hold (padded) tokens
     l.qsz = (l.tq * 128 + 1023) / 1024 * 1024;
-    // V rows: (R + 2) (C + 2) rows, one guard KB before (tap (0,0) starts one row early) and room after for
+    // V rows: (R + 2) (W + 2) rows, one guard KB before (tap (0,0) starts one row early) and room after for
     // the 128-row operand of the last tap (read, never used)
     l.hsz = 1024 + ((2 * l.wp + 1 + 128) * 128 + 1023) / 1024 * 1024;
     if (l.hsz < 1024 + ((R + 2) * l.wp * 128 + 1023) / 1024 * 1024) l.hsz = 1024 + ((R + 2) * l.wp * 128 + 1023) / 1024 * 1024;
@@ -83,22 +81,14 @@ constexpr uint32_t TM_S = 0, TM_O = 128, TM_D = 256;
 __device__ __forceinline__ int swz16(int row, int col) {
     return row * 128 + ((((col >> 3) ^ row) & 7) << 4) + (col & 7) * 2;
 }
-// Slab, band of rows and (CUT: rows are cut into shares) share of a block's i-th tile, advanced without divisions.  (Whole rows have
-// an instantiation of their own: with the shares' bookkeeping 64 slabs of 56 x 56 took 58.5 us instead of 56.5.)
-template <bool CUT> struct TileIter {
-    int slab, tb, TB, tx, TX;
-    __device__ __forceinline__ void next() {
-        if (CUT) {
-            if (++tx < TX) return;
-            tx = 0;
-        }
-        if (++tb == TB) { tb = 0; ++slab; }
-    }
-    __device__ __forceinline__ int x(int C) const { return CUT ? tx * C : 0; }
+// The (slab, tile) pair of a block's i-th tile, advanced without divisions.
+struct TileIter {
+    int slab, tb, TB;
+    __device__ __forceinline__ void next() { if (++tb == TB) { tb = 0; ++slab; } }
 };
 }  // namespace
 
-template <typename T, bool CUT>
+template <typename T>
 __global__ void __launch_bounds__(NT, 1) stream_broadcast_kernel(const __grid_constant__ StreamArgs p) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ int s_dead;
@@ -107,16 +97,15 @@ __global__ void __launch_bounds__(NT, 1) stream_broadcast_kernel(const __grid_co
     constexpr int fmt = Elem<T>::kIsBf16 ? 1 : 0;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int H = p.H, W = p.W, N = H * W, n = p.n;
-    const int R = p.plan.rows_b, C = CUT ? p.plan.cols_b : W, TX = CUT ? p.plan.tiles_x : 1, TB = p.plan.tiles_b;
-    const BcLayout L = bc_layout(R, C);
+    const int R = p.plan.rows_b, TB = p.plan.tiles_b;
+    const BcLayout L = bc_layout(R, W);
     const bool has_dwc = p.dwc_w != nullptr;
     // this block's run of the (slab, tile) sequence
     const int total = p.slabs * TB;
     const int g0 = (int)((long long)total * blockIdx.x / gridDim.x), g1 = (int)((long long)total * (blockIdx.x + 1) / gridDim.x);
     const int T_ = g1 - g0;
-    TileIter<CUT> it;
-    it.slab = g0 / TB; it.tb = (g0 - it.slab * TB) / TX; it.TB = TB / TX;
-    it.tx = g0 - it.slab * TB - it.tb * TX; it.TX = TX;
+    TileIter it;
+    it.slab = g0 / TB; it.tb = g0 - it.slab * TB; it.TB = TB;
 
     Pipe pp;
     pp.status = p.status;
@@ -158,12 +147,12 @@ __global__ void __launch_bounds__(NT, 1) stream_broadcast_kernel(const __grid_co
         if (lane == 0) {
             // V is an input of the call: its first two stages are requested before the wait for the preceding kernels
             const uint32_t h_tx = (uint32_t)(R + 2) * L.wp * 128u;
-            TileIter<CUT> ih = it;
+            TileIter ih = it;
             if (has_dwc)
                 for (int i = 0; i < min(T_, 2); ++i, ih.next()) {
                     const uint32_t bar = pipe_bar(pp, BAR_H_FULL + i);
                     mbar_arrive_expect_tx(bar, h_tx);
-                    tma_load_grid(sH + i * L.hsz + 1024, &p.tm_h, p.hf, ih.x(C) - 1, ih.tb * R - 1, ih.slab % p.heads, ih.slab / p.heads, bar);
+                    tma_load_grid(sH + i * L.hsz + 1024, &p.tm_h, p.hf, -1, ih.tb * R - 1, ih.slab % p.heads, ih.slab / p.heads, bar);
                 }
             pdl_wait();      // A, V_A, the padded B2 and the weight slices come from the preceding kernels
             int cur = -1, ord = -1;
@@ -185,13 +174,13 @@ __global__ void __launch_bounds__(NT, 1) stream_broadcast_kernel(const __grid_co
                 if (i >= 2) wait_spin(pp, BAR_QB_EMPTY + s2, (i >> 1) - 1, kTimeoutRole);
                 const uint32_t bar = pipe_bar(pp, BAR_QB_FULL + s2), dst = sQB + s2 * 2 * L.qsz;
                 mbar_arrive_expect_tx(bar, qb_tx);
-                tma_load_grid(dst, &p.tm_q, p.hf, it.x(C) - 1, it.tb * R, it.slab % p.heads, it.slab / p.heads, bar);
-                tma_load_4d(dst + L.qsz, &p.tm_b2, 0, it.x(C) - 1, it.tb * R, p.b2 ? it.slab % p.heads : 0, bar);
+                tma_load_grid(dst, &p.tm_q, p.hf, -1, it.tb * R, it.slab % p.heads, it.slab / p.heads, bar);
+                tma_load_4d(dst + L.qsz, &p.tm_b2, 0, -1, it.tb * R, p.b2 ? it.slab % p.heads : 0, bar);
                 if (has_dwc && i >= 2) {
                     wait_spin(pp, BAR_H_EMPTY + s2, (i >> 1) - 1, kTimeoutRole);
                     const uint32_t hb = pipe_bar(pp, BAR_H_FULL + s2);
                     mbar_arrive_expect_tx(hb, h_tx);
-                    tma_load_grid(sH + s2 * L.hsz + 1024, &p.tm_h, p.hf, it.x(C) - 1, it.tb * R - 1, it.slab % p.heads, it.slab / p.heads, hb);
+                    tma_load_grid(sH + s2 * L.hsz + 1024, &p.tm_h, p.hf, -1, it.tb * R - 1, it.slab % p.heads, it.slab / p.heads, hb);
                 }
             }
         }
@@ -206,7 +195,7 @@ __global__ void __launch_bounds__(NT, 1) stream_broadcast_kernel(const __grid_co
             const uint64_t dQ0 = umma_desc_sw128(sQB), dQ1 = dQ0 + (uint64_t)(2 * L.qsz >> 4);
             const uint64_t dB0 = dQ0 + (uint64_t)(L.qsz >> 4), dB1 = dQ1 + (uint64_t)(L.qsz >> 4);
             const uint32_t tS = pp.tmem + TM_S, tO = pp.tmem + TM_O;
-            TileIter<CUT> is = it;                    // slab bookkeeping of the logits (one tile ahead) ...
+            TileIter is = it;                    // slab bookkeeping of the logits (one tile ahead) ...
             int cur_s = -1, ord_s = -1;
             int cur_o = -1, ord_o = -1;          // ... and of the products
             // descriptor start addresses count 16-byte units: + 2 per K-step of a K-major operand (32 bytes),
@@ -281,7 +270,7 @@ __global__ void __launch_bounds__(NT, 1) stream_broadcast_kernel(const __grid_co
                         const uint64_t dh = (b ? dH1 : dH0) - 8;         // tap (0, 0) starts one row before the tile
                         const uint64_t dw = dWT + (uint64_t)((ord & 1) * (kWtBytes >> 4));
                         const uint32_t dd = tD + 64 * b;
-                        // tap (u, v): the V tile started u (C + 2) + v - 1 rows later, times the tap's diagonal slices
+                        // tap (u, v): the V tile started u (W + 2) + v - 1 rows later, times the tap's diagonal slices
 #pragma unroll
                         for (int t = 0; t < 5; ++t) {
                             const int tap = t + 5 * half;        // (the second issuer's fifth slot is empty)
@@ -352,10 +341,9 @@ __global__ void __launch_bounds__(NT, 1) stream_broadcast_kernel(const __grid_co
         for (int i = 0; i < T_; ++i, it.next()) {
             const int b = i & 1;
             const int rows = min(R, H - it.tb * R);
-            const int x = it.x(C) + xp - 1;
-            const bool live = r < rows && xp >= 1 && xp <= C && (!CUT || x < W);
+            const bool live = r < rows && xp >= 1 && xp <= W;
             const uint32_t tO = pp.tmem + TM_O + 64 * b + lane_base, tD = pp.tmem + TM_D + 64 * b + lane_base;
-            uint4* dst = reinterpret_cast<uint4*>(static_cast<T*>(p.out) + tok_offset(p.lout, it.slab, p.heads, (long long)(it.tb * R + r) * W + x));
+            uint4* dst = reinterpret_cast<uint4*>(static_cast<T*>(p.out) + tok_offset(p.lout, it.slab, p.heads, (long long)(it.tb * R + r) * W + (xp - 1)));
             wait_par(pp, BAR_O_FULL + b, i >> 1, kTimeoutTile);
             if (has_dwc) wait_par(pp, BAR_D_FULL + b, i >> 1, kTimeoutTile);
             tc_fence_after_sync();
@@ -393,31 +381,21 @@ __global__ void __launch_bounds__(NT, 1) stream_broadcast_kernel(const __grid_co
 }
 
 // ------------------------------------------------------------------------------------- host
-// Windows that tile a grid of whole rows up to 64 columns: always.  Elsewhere register tiles over these kernels (64 channels, with and without biases, 1 to
-// 128 slabs of 1610 to 40200 tokens, whole pass; the biases are padded once per head, which batches share):
-//   49 and 64 agents 0.92 to 1.74, one slab of 1610 to 5280 tokens 0.86 to 1.09
-//   25 agents: 16384 tokens in all, up to two heads or four batch entries 0.96 to 1.47; two batch entries of eight heads 0.87 to 1.09
-//   9 and 16 agents: 40000 tokens in all on 5120 and more 1.00 to 1.38, two batch entries of eight heads 0.80 to 1.03
-static bool stream_faster(int slabs, int heads, long long N, int W, int H, int n, int pool) {
-    if (W <= 64 && N % 8 == 0 && (!pool || (H % pool == 0 && W % pool == 0))) return true;
-    const long long work = slabs * N;
-    if (n > 32) return N >= 8192 || (slabs >= 2 && work >= 4096);
-    const bool shared = heads <= 2 || slabs >= 4 * heads;
-    return n > 16 ? shared && work >= 16384 : shared && N >= 5120 && work >= 40000;
-}
-
-StreamPlan plan_stream(int dtype, int slabs, int heads, int H, int W, int d, int n_agents, bool pooled, int sm_count) {
+// Windows that tile a grid of whole rows up to 64 columns, tokens a multiple of eight.  Wider grids, other windows and other token counts stay on
+// register tiles.  (Tiles of shares of a row took any grid, 4 x 2 slabs of 75 x 117 tokens, 49 agents, in 48 us instead of 61.  But scale A is
+// rounded to 16 bits here, biases are clamped, weights are summed before they are rounded and an infinity reaches 16 channels, all of which
+// those grids are spared there.)
+StreamPlan plan_stream(int dtype, int slabs, int H, int W, int d, int n_agents, bool pooled, int sm_count) {
     StreamPlan pl;
     memset(&pl, 0, sizeof(pl));
     if (dtype != kBF16 && dtype != kF16) return pl;
     const long long N = (long long)H * W;
-    if (d != 64 || n_agents < 1 || n_agents > 64 || W < 8 || N < 1024 || N > (1 << 24)) return pl;
-    int pw = 0;
+    if (d != 64 || n_agents < 1 || n_agents > 64 || W < 8 || W > 64 || N < 1024 || N % 8 != 0 || N > (1 << 24)) return pl;
     if (pooled) {
+        int pw = 1;
         while (pw * pw < n_agents) ++pw;
-        if (pw * pw != n_agents || pw > H || pw > W) return pl;
+        if (pw * pw != n_agents || H % pw != 0 || W % pw != 0) return pl;
     }
-    if (!stream_faster(slabs, heads, N, W, H, n_agents, pw)) return pl;
     if (!encode_tiled_fn()) return pl;
     // aggregation: about one block per SM, ranges of whole 128-token tiles
     const int tiles = (int)((N + 127) / 128);
@@ -427,19 +405,15 @@ StreamPlan plan_stream(int dtype, int slabs, int heads, int H, int W, int d, int
     if (splits > tiles / 4) splits = tiles / 4 > 0 ? tiles / 4 : 1;
     pl.tiles_per_split = (tiles + splits - 1) / splits;
     pl.splits = (tiles + pl.tiles_per_split - 1) / pl.tiles_per_split;
-    // broadcast: tiles of grid rows, whole or in even shares: the cut with the fewest tiles (operand rows are padded token positions)
-    for (int most = std::min(W, 126); most >= std::min(W, 8); --most) {
-        const int tiles_x = (W + most - 1) / most, C = (W + tiles_x - 1) / tiles_x, R = std::min(std::min(128 / (C + 2), 16), H);
-        if (R < 1 || bc_layout(R, C).total + 1024 > 232448 - 1024) continue;
-        const int count = tiles_x * ((H + R - 1) / R);
-        if (pl.tiles_b && (W <= 64 || count >= pl.tiles_b)) continue;
-        pl.rows_b = R;
-        pl.cols_b = C;
-        pl.tiles_x = tiles_x;
-        pl.tiles_b = count;
-    }
-    if (!pl.tiles_b) return pl;
-    pl.smem_b = bc_layout(pl.rows_b, pl.cols_b).total + 1024;
+    // broadcast: tiles of whole grid rows
+    int R = 128 / (W + 2);                                   // operand rows are padded token positions
+    if (R > 16) R = 16;
+    if (R > H) R = H;
+    if (R < 1) return pl;
+    pl.rows_b = R;
+    pl.tiles_b = (H + R - 1) / R;
+    pl.smem_b = bc_layout(R, W).total + 1024;
+    if (pl.smem_b > 232448 - 1024) return pl;
     const long long total = (long long)slabs * pl.tiles_b;
     pl.grid_b = (int)(total < sm_count ? total : sm_count);
     pl.ok = true;
@@ -457,9 +431,9 @@ bool stream_make_maps(StreamArgs* a) {
     const int batch = a->slabs / a->heads;
     if (!make_map_tok_u16(&a->tm_k, &a->hf, a->k, a->lin, batch, a->heads, (long long)N, 64, 128, true)) return false;
     if (!make_map_tok_u16(&a->tm_v, &a->hf, a->v, a->lin, batch, a->heads, (long long)N, 64, 128, true)) return false;
-    if (!make_map_grid5d_u16(&a->tm_q, a->hf, a->q, a->lin, batch, a->heads, (uint64_t)a->H, (uint64_t)a->W, (uint32_t)a->plan.rows_b, (uint32_t)(a->plan.cols_b + 2))) return false;
-    if (!make_map_grid4d_u16(&a->tm_b2, a->b2p, a->b2 ? (uint64_t)a->heads : 1u, (uint64_t)a->H, (uint64_t)a->W, (uint32_t)a->plan.rows_b, (uint32_t)(a->plan.cols_b + 2), true)) return false;
-    if (a->dwc_w && !make_map_grid5d_u16(&a->tm_h, a->hf, a->v, a->lin, batch, a->heads, (uint64_t)a->H, (uint64_t)a->W, (uint32_t)(a->plan.rows_b + 2), (uint32_t)(a->plan.cols_b + 2))) return false;
+    if (!make_map_grid5d_u16(&a->tm_q, a->hf, a->q, a->lin, batch, a->heads, (uint64_t)a->H, (uint64_t)a->W, (uint32_t)a->plan.rows_b, (uint32_t)(a->W + 2))) return false;
+    if (!make_map_grid4d_u16(&a->tm_b2, a->b2p, a->b2 ? (uint64_t)a->heads : 1u, (uint64_t)a->H, (uint64_t)a->W, (uint32_t)a->plan.rows_b, (uint32_t)(a->W + 2), true)) return false;
+    if (a->dwc_w && !make_map_grid5d_u16(&a->tm_h, a->hf, a->v, a->lin, batch, a->heads, (uint64_t)a->H, (uint64_t)a->W, (uint32_t)(a->plan.rows_b + 2), (uint32_t)(a->W + 2))) return false;
     if (a->b1 && !make_map_rows3d_u16(&a->tm_b1, a->b1c, (uint64_t)a->heads, N, 128, true)) return false;
     if (!make_map_2d_u16(&a->tm_a2, a->a2s, S * a->n, 64, (uint32_t)a->n, 64)) return false;
     if (!make_map_2d_u16(&a->tm_va, a->va_ws, S * a->n, 64, (uint32_t)a->n, 64)) return false;
@@ -478,13 +452,19 @@ cudaError_t launch_stream_broadcast(int dtype, const StreamArgs& a, cudaStream_t
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    auto go = [&](auto kern) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, a.plan.smem_b);
-        return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, kern, a);
-    };
-    const bool cut = a.plan.tiles_x > 1;
-    if (dtype == kBF16) return cut ? go(stream_broadcast_kernel<__nv_bfloat16, true>) : go(stream_broadcast_kernel<__nv_bfloat16, false>);
-    if (dtype == kF16) return cut ? go(stream_broadcast_kernel<__half, true>) : go(stream_broadcast_kernel<__half, false>);
+    cudaError_t e;
+    if (dtype == kBF16) {
+        auto kern = stream_broadcast_kernel<__nv_bfloat16>;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, a.plan.smem_b);
+        if (e != cudaSuccess) return e;
+        return cudaLaunchKernelEx(&cfg, kern, a);
+    }
+    if (dtype == kF16) {
+        auto kern = stream_broadcast_kernel<__half>;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, a.plan.smem_b);
+        if (e != cudaSuccess) return e;
+        return cudaLaunchKernelEx(&cfg, kern, a);
+    }
     return cudaErrorInvalidValue;
 }
 

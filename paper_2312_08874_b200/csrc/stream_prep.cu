@@ -37,8 +37,8 @@ __global__ void __launch_bounds__(NT, 4) stream_prep_kernel(const StreamArgs p, 
         if (p.a_user) {
             if (ts == 0) unpack16<T>(__ldg(reinterpret_cast<const uint4*>(static_cast<const T*>(p.a_user) + ((size_t)slab * n + a) * 64) + c), acc);
         } else {
-            const int ay = a / p.p, ax = a - ay * p.p;
-            const int y0 = ay * p.H / p.p, x0 = ax * p.W / p.p, win_w = ((ax + 1) * p.W + p.p - 1) / p.p - x0, cnt = (((ay + 1) * p.H + p.p - 1) / p.p - y0) * win_w;
+            const int win_h = p.H / p.p, win_w = p.W / p.p, cnt = win_h * win_w;
+            const int y0 = (a / p.p) * win_h, x0 = (a % p.p) * win_w;
             // lane (c, ts) walks the window's tokens ts, ts + 4, ... in row-major order; (wy, wx) is kept
             // incrementally, so the loads of a batch cost an add and a compare each
             const uint4* gq = reinterpret_cast<const uint4*>(static_cast<const T*>(p.q) + tok_offset(p.lin, slab, p.heads, (long long)y0 * p.W + x0)) + c;
@@ -82,10 +82,9 @@ __global__ void __launch_bounds__(NT, 4) stream_prep_kernel(const StreamArgs p, 
                 for (int k = 0; k < 8; ++k) part[warp][8 * c + k] = acc[k];
             __syncthreads();
             if (warp != 0) return;
-            if (!p.a_user)
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    for (int w = 1; w < NT / 32; ++w) acc[k] += part[w][8 * c + k];
+            for (int k = 0; k < 8; ++k)
+                for (int w = 1; w < NT / 32; ++w) acc[k] += part[w][8 * c + k];
         }
         if (ts == 0) {
             float m[8], s1[8], s2[8];

@@ -39,6 +39,7 @@ def test_tile_edges_match_oracle(case):
 
 WEIGHTS = {
     "one_kernel": (2, 2, 14, 14, 64, 7, "bf16"), "three_kernels": (1, 2, 45, 45, 64, 11, "f16"), "d40": (1, 1, 33, 32, 40, 16, "bf16"),
+    "wide_grid": (2, 1, 75, 117, 64, 7, "bf16"), "odd_tokens": (2, 2, 45, 47, 64, 7, "f16"), "ragged_windows": (2, 1, 40, 46, 64, 7, "bf16"),
     # tensor memory, where register tiles are the other choice
     "short_slabs": (128, 3, 14, 14, 64, 7, "bf16"), "latent_grid": (2, 8, 64, 64, 40, 16, "bf16"), "latent_grid_f16": (2, 8, 64, 64, 40, 16, "f16"),
     "short_axis": (4, 8, 32, 64, 64, 16, "bf16"), "half_filled": (1, 2, 56, 144, 64, 12, "bf16"),
