@@ -3,8 +3,8 @@
 //
 // Grid: (splits, slabs), one block per SM.  The slab's agents A and agent features V_A stay resident in shared memory; a block walks its
 // share of the slab's tiles, patches of 8 x 16 tokens of the grid (a window with its halo is 180 tokens there, 390 for 128 tokens of a row, and
-// zeros outside the grid are what TMA fills in).  Two teams of eight warps work on a tile each (even and odd ones); per tile the agents
-// are taken in steps of 64, whose logits alternate between two buffers: while the softmax of one step runs, the other buffer's
+// zeros outside the grid are what TMA fills in) or, on grids that do not fill patches, runs of 128 tokens.  Two teams of eight warps work on a
+// tile each (even and odd ones); per tile the agents are taken in steps of 64, whose logits alternate between two buffers: while the softmax of one step runs, the other buffer's
 // products and next logits are under way.
 //   warps 0-15 "row warps", a team each eight: thread (query row, half of a step's agents): online softmax over the steps with its own running
 //                         maximum, sum and accumulator O_h in tensor memory (no reduction crosses threads); the probabilities go back
@@ -46,10 +46,11 @@ constexpr int OFF_VA = OFF_A + 4 * kTile;                // agent features [256]
 constexpr int OFF_Q = OFF_VA + 4 * kTile;                // a query tile [128][128 B] per team
 constexpr int OFF_B2 = OFF_Q + 4 * kTile;                // biases of a step [128][128 B], two per team
 constexpr int kHaloRows = (TH + 2) * (TW + 2), kHaloBytes = kHaloRows * 128, kHalo = (kHaloBytes + 1023) / 1024 * 1024;
-constexpr int OFF_H = OFF_B2 + 4 * 2 * kTile;            // two windows of V tokens [10][18][128 B]
-constexpr int kSmemBytes = OFF_H + 2 * kHalo + 1024;
+constexpr int OFF_H = OFF_B2 + 4 * 2 * kTile;            // two windows of V tokens [10][18][128 B]; runs: one [3][136][128 B]
+constexpr int kRunRows = (QT + 2 + 7) / 8 * 8;           // (eight rows: a period of the swizzle)
+constexpr int smem_bytes(bool run) { return OFF_H + (run ? 3 * kRunRows * 128 : 2 * kHalo) + 1024; }
 static_assert(OFF_ZEROS % 128 == 0 && OFF_TAB + kFilterWords * 4 <= OFF_A, "small buffers");
-static_assert(kSmemBytes <= 232448 && kSmemBytes > 116 * 1024, "one block per SM");
+static_assert(smem_bytes(true) <= 232448 && smem_bytes(false) <= 232448 && smem_bytes(false) > 116 * 1024, "one block per SM");
 
 // mbarriers (t: + team; ts: + 2 team + step parity; i: + tile parity)   count       waiter
 constexpr int BAR_AG = 0;          //             tx          row warps
@@ -64,7 +65,7 @@ constexpr int BAR_PV = 22;         // ts          commit      row warps       pr
 constexpr int BAR_O_FULL = 26;     // t           commit      output warps    every product of a tile
 constexpr int BAR_O_EMPTY = 28;    // t           8 warps     MMA issuer, row warps    accumulators and (max, sum) read
 constexpr int BAR_ML = 30;         // t           8 warps     output warps
-constexpr int BAR_H_FULL = 32;     // i           tx          output warps    V tokens of the tile's depthwise window
+constexpr int BAR_H_FULL = 32;     // i           tx          output warps    V tokens of the tile's depthwise window (runs: of index 0 only)
 constexpr int BAR_H_EMPTY = 34;    // i           8 warps     their producer
 constexpr int BAR_DRAIN = 36;      // t           commit      MMA issuer, once, at its end
 constexpr int kBars = 38;
@@ -81,12 +82,13 @@ struct UmmaBcArgs {
 };
 }  // namespace
 
-// ROUNDED: see umma_sums_rounded
-template <typename T, bool ROUNDED>
+// RUN: a tile is a run of 128 tokens; ROUNDED: see umma_sums_rounded
+template <typename T, bool RUN, bool ROUNDED>
 __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_constant__ UmmaBcArgs g) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     constexpr int fmt = Elem<T>::kIsBf16 ? 1 : 0;
+    constexpr int th = RUN ? 1 : TH, tw = RUN ? QT : TW;       // (runs: the grid is one row to the maps of Q, B2 and V)
     const AttnArgs& p = g.a;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int split = blockIdx.x, slab = blockIdx.y;
@@ -135,7 +137,7 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
                 }
                 int j = 0;
                 for (int i = team; i < tiles; i += 2) {
-                    const int ty = (i0 + i) / g.tiles_x, y = TH * ty, x = TW * (i0 + i - ty * g.tiles_x);
+                    const int ty = (i0 + i) / g.tiles_x, y = th * ty, x = tw * (i0 + i - ty * g.tiles_x);
                     if (i >= 2) wait_spin(pp, BAR_Q_EMPTY + team, (i >> 1) - 1, kTimeoutRole);
                     const uint32_t qb = pipe_bar(pp, BAR_Q_FULL + team);
                     mbar_arrive_expect_tx(qb, 2 * kTile);
@@ -156,7 +158,14 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
             // ------------------------------------------------------------------ producer of the V tokens
             if (has_dwc && lane == 0)
                 for (int i = 0; i < tiles && !pipe_dead(pp); ++i) {
-                    const int ty = (i0 + i) / g.tiles_x, y = TH * ty, x = TW * (i0 + i - ty * g.tiles_x);
+                    const int ty = (i0 + i) / g.tiles_x, y = th * ty, x = tw * (i0 + i - ty * g.tiles_x);
+                    if (RUN) {                                         // the rows above, of and below the run
+                        const uint32_t bar = pipe_bar(pp, BAR_H_FULL);
+                        if (i >= 1) wait_spin(pp, BAR_H_EMPTY, i - 1, kTimeoutRole);
+                        mbar_arrive_expect_tx(bar, 3 * kRunRows * 128);
+                        for (int u = 0; u < 3; ++u) tma_load_grid(sH + u * kRunRows * 128, &g.tm_h, g.hf, x - 1 + (u - 1) * p.W, 0, head, slab / p.heads, bar);
+                        continue;
+                    }
                     const uint32_t bar = pipe_bar(pp, BAR_H_FULL + (i & 1));
                     if (i >= 2) wait_spin(pp, BAR_H_EMPTY + (i & 1), (i >> 1) - 1, kTimeoutRole);
                     mbar_arrive_expect_tx(bar, kHaloBytes);
@@ -213,7 +222,7 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
         const int q = warp & 3, half = (warp >> 2) & 1, c0 = 32 * half, lg = lane >> 2;
         const uint32_t* tab = filter_lane(reinterpret_cast<const uint32_t*>(smem + OFF_TAB) + c0, reinterpret_cast<const uint32_t*>(smem + OFF_ZEROS), lane);
         uint32_t at[6];
-        patch_offsets<TW + 2>(at, 2 * q * (TW + 2), 64 * half, lane);
+        if (!RUN) patch_offsets<TW + 2>(at, 2 * q * (TW + 2), 64 * half, lane);
         T* gO = static_cast<T*>(p.out) + tok_offset(p.lout, slab, p.heads, 0);
         const size_t so = (size_t)p.lout.st;
         wait_par(pp, BAR_PREP, 0, kTimeoutLoads);
@@ -227,14 +236,25 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
 #pragma unroll
                     for (int e = 0; e < 4; ++e) o[mt][jj][e] = 0.f;
             if (has_dwc) {
-                wait_par(pp, BAR_H_FULL + team, k, kTimeoutLoads);
-                dwc_patch<T>(o, at, sH + team * kHalo, tab);
+                const int ib = RUN ? 0 : team;
+                wait_par(pp, BAR_H_FULL + ib, RUN ? i : k, kTimeoutLoads);
+                if constexpr (RUN) {
+                    uint32_t in[2];
+#pragma unroll
+                    for (int mt = 0; mt < 2; ++mt) {               // (past the last token: anything, not stored)
+                        const int t = QT * (i0 + i) + 32 * q + 16 * mt + (lane & 15), y = t / p.W;
+                        in[mt] = grid_taps(t - y * p.W, y, p.H, p.W, lane);
+                    }
+                    dwc_rows<T>(o, sH, 32 * q + (lane & 15), 64 * half, in, smem_u32(smem + OFF_ZEROS), tab, lane, [](int u, int v) { return u * kRunRows + v; });
+                } else {
+                    dwc_patch<T>(o, at, sH + team * kHalo, tab);
+                }
                 // The window goes back to TMA: an arrival overtakes loads that are still queued, so the arriving lane hangs on the products of
                 // what was loaded.
                 uint32_t x = 0u;
 #pragma unroll
                 for (int k = 0; k < 8; ++k) x ^= __float_as_uint(o[k >> 2][k & 3][0]);
-                if (lane == (__all_sync(0xffffffffu, x == 0x5bd1e995u) ? 31 : 0)) pipe_arrive(pp, BAR_H_EMPTY + team);
+                if (lane == (__all_sync(0xffffffffu, x == 0x5bd1e995u) ? 31 : 0)) pipe_arrive(pp, BAR_H_EMPTY + ib);
             }
             wait_par(pp, BAR_ML + team, k, kTimeoutTile);
             float w0, w1;                                      // weights of row 32 q + lane's two accumulators
@@ -269,6 +289,15 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
             }
             tc_fence_before_sync();
             pipe_arrive_warp(pp, BAR_O_EMPTY + team, lane);
+            if constexpr (RUN) {
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt) {
+                    const int t = QT * (i0 + i) + 32 * q + 16 * mt;
+                    const bool ok[2] = {t + lg < p.rows, t + 8 + lg < p.rows};
+                    store_rows<T>(o[mt], gO + (size_t)t * so, so, c0, p.d, ok, lane);
+                }
+                continue;
+            }
             const int ty = (i0 + i) / g.tiles_x, y = TH * ty + 2 * q, x = TW * (i0 + i - ty * g.tiles_x);
 #pragma unroll
             for (int mt = 0; mt < 2; ++mt) {
@@ -400,21 +429,20 @@ bool broadcast_umma_eligible(int dtype, int n_agents, int n_tokens, int d) {
     return encode_tiled_fn() != nullptr;
 }
 
-template <typename T>
+template <typename T, bool RUN, bool ROUNDED>
 static cudaError_t launch_bc_umma_t(const UmmaBcArgs& g, int splits, cudaStream_t st) {
-    auto kern = umma_sums_rounded(g.a.rows, g.a.d) ? broadcast_umma_kernel<T, true> : broadcast_umma_kernel<T, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    static std::atomic<unsigned long long> done;
+    cudaError_t e = allow_smem(broadcast_umma_kernel<T, RUN, ROUNDED>, done, smem_bytes(RUN));
     if (e != cudaSuccess) return e;
-    dim3 grid(splits, g.a.slabs);
-    return launch_dependent(kern, grid, NT, kSmemBytes, st, g);
+    return launch_dependent(broadcast_umma_kernel<T, RUN, ROUNDED>, dim3(splits, g.a.slabs), NT, smem_bytes(RUN), st, g);
 }
 
 // Map of B2 [heads][H][W][n] with boxes of 64 agents x a tile of tokens.
-static bool make_map_b2(CUtensorMap* out, const void* base, uint64_t heads, uint64_t H, uint64_t W, uint64_t n) {
+static bool make_map_b2(CUtensorMap* out, const void* base, uint64_t heads, uint64_t H, uint64_t W, uint64_t n, uint32_t th, uint32_t tw) {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn || (reinterpret_cast<uintptr_t>(base) & 15u) || n % 8) return false;
     const cuuint64_t dims[4] = {n, W, H, heads}, strides[3] = {2 * n, 2 * n * W, 2 * n * W * H};
-    const cuuint32_t box[4] = {64, TW, TH, 1}, estr[4] = {1, 1, 1, 1};
+    const cuuint32_t box[4] = {64, tw, th, 1}, estr[4] = {1, 1, 1, 1};
     return fn(out, CU_TENSOR_MAP_DATA_TYPE_UINT16, 4, const_cast<void*>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -425,26 +453,40 @@ cudaError_t launch_broadcast_umma(int dtype, const AttnArgs& p, int sm_count, cu
     memset(&g, 0, sizeof(g));
     g.a = p;
     g.steps = (p.cols + 63) / 64;
-    g.tiles_x = (p.W + TW - 1) / TW;
-    g.tiles = g.tiles_x * ((p.H + TH - 1) / TH);
+    const uint64_t S = p.slabs, n = p.cols;
+    const int batch = p.slabs / p.heads, patches = ((p.W + TW - 1) / TW) * ((p.H + TH - 1) / TH), runs = (p.rows + QT - 1) / QT;
+    unsigned long long dims[2], strides[3];
+    bool hf;
+    if (!tok_map_dims(p.lin, batch, p.heads, (long long)p.rows, &hf, dims, strides)) return cudaErrorNotSupported;
+    g.hf = hf;
+    auto maps = [&](bool run) {
+        const uint64_t H = run ? 1 : p.H, W = run ? p.rows : p.W;
+        const uint32_t th = run ? 1 : TH, tw = run ? QT : TW;
+        g.tiles_x = run ? runs : (p.W + TW - 1) / TW;
+        g.tiles = run ? runs : patches;
+        return make_map_grid5d_u16(&g.tm_q, hf, p.qm, p.lin, batch, p.heads, H, W, th, tw, p.d) && (!p.bias || make_map_b2(&g.tm_b, p.bias, p.heads, H, W, n, th, tw)) &&
+               (!p.dwc_w || make_map_grid5d_u16(&g.tm_h, hf, p.dwc_v, p.lin, batch, p.heads, H, W, run ? 1 : TH + 2, run ? kRunRows : TW + 2, p.d));
+    };
+    if (!make_map_2d_u16(&g.tm_a, p.km, S * n, p.d, 128, 64)) return cudaErrorNotSupported;
+    if (!make_map_2d_u16(&g.tm_va, p.vm, S * n, p.d, 128, 64)) return cudaErrorNotSupported;
+    // Whole pass on patches over that on runs (256 and 144 agents, 1 and 16 slabs): as many patches as runs 0.95 to 1.02 (16 slabs of 128 x 128, 144
+    // agents 95.5 and 100 us), 1.05 times as many 0.97 to 1.02, 1.2 times 1.00 to 1.12, 1.4 times 1.10 to 1.16, twice 1.10 to 1.45, sixteen times
+    // 2.5 to 8 (16 slabs of 16384 x 1, 256 agents 852 and 105 us).  Strides that express patches alone: those.
+    const bool run = 8LL * patches > 9LL * runs && maps(true);
+    if (!run && !maps(false)) return cudaErrorNotSupported;
     int splits = sm_count / p.slabs;                        // one block per SM, one wave
     if (splits < 1) splits = 1;
     if (splits > g.tiles) splits = g.tiles;
     g.tps = (g.tiles + splits - 1) / splits;
     splits = (g.tiles + g.tps - 1) / g.tps;
-    const uint64_t S = p.slabs, H = p.H, W = p.W, n = p.cols;
-    const int batch = p.slabs / p.heads;
-    unsigned long long dims[2], strides[3];
-    bool hf;
-    if (!tok_map_dims(p.lin, batch, p.heads, (long long)p.rows, &hf, dims, strides)) return cudaErrorNotSupported;
-    g.hf = hf;
-    if (!make_map_grid5d_u16(&g.tm_q, hf, p.qm, p.lin, batch, p.heads, H, W, TH, TW, p.d)) return cudaErrorNotSupported;
-    if (!make_map_2d_u16(&g.tm_a, p.km, S * n, p.d, 128, 64)) return cudaErrorNotSupported;
-    if (!make_map_2d_u16(&g.tm_va, p.vm, S * n, p.d, 128, 64)) return cudaErrorNotSupported;
-    if (p.bias && !make_map_b2(&g.tm_b, p.bias, p.heads, H, W, n)) return cudaErrorNotSupported;
-    if (p.dwc_w && !make_map_grid5d_u16(&g.tm_h, hf, p.dwc_v, p.lin, batch, p.heads, H, W, TH + 2, TW + 2, p.d)) return cudaErrorNotSupported;
-    if (dtype == kBF16) return launch_bc_umma_t<__nv_bfloat16>(g, splits, st);
-    if (dtype == kF16) return launch_bc_umma_t<__half>(g, splits, st);
+    auto go = [&](auto t) {
+        using T = decltype(t);
+        const bool rounded = umma_sums_rounded(p.rows, p.d);
+        return run ? rounded ? launch_bc_umma_t<T, true, true>(g, splits, st) : launch_bc_umma_t<T, true, false>(g, splits, st)
+                   : rounded ? launch_bc_umma_t<T, false, true>(g, splits, st) : launch_bc_umma_t<T, false, false>(g, splits, st);
+    };
+    if (dtype == kBF16) return go(__nv_bfloat16{});
+    if (dtype == kF16) return go(__half{});
     return cudaErrorInvalidValue;
 }
 

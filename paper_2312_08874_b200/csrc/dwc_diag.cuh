@@ -20,19 +20,22 @@ __device__ __forceinline__ const uint32_t* filter_lane(const uint32_t* tab, cons
     return (lane & 3) == (lane >> 3) ? tab + (lane >> 2) : zeros;
 }
 
-// Window positions (bit 3 u + v) of a token that lie in the grid; with `lane`'s half of the tap pairs: bit 2 k is the tap that the lane addresses for
-// pair k (lanes 0-15 the even taps, lanes 16-31 the odd ones).
-__device__ __forceinline__ uint32_t window_taps(int tok, int N, int H, int W, float inv_w, int lane) {
-    int y = (int)((float)tok * inv_w), x = tok - y * W;                 // the quotient is off by one at most
-    if (x < 0) { x += W; --y; }
-    if (x >= W) { x -= W; ++y; }
+// Window positions (bit 3 u + v) of the token at (x, y) that lie in the grid; with `lane`'s half of the tap pairs: bit 2 k is the tap that the lane
+// addresses for pair k (lanes 0-15 the even taps, lanes 16-31 the odd ones).
+__device__ __forceinline__ uint32_t grid_taps(int x, int y, int H, int W, int lane) {
     uint32_t in = 0x1ffu;
     if (x == 0) in &= ~0x49u;
     if (x == W - 1) in &= ~0x124u;
     if (y == 0) in &= ~7u;
     if (y == H - 1) in &= ~0x1c0u;
-    if (tok >= N) in = 0u;
     return lane < 16 ? in : in >> 1;
+}
+// The same for token `tok` of a short grid (none from N on).
+__device__ __forceinline__ uint32_t window_taps(int tok, int N, int H, int W, float inv_w, int lane) {
+    int y = (int)((float)tok * inv_w), x = tok - y * W;                 // the quotient is off by one at most
+    if (x < 0) { x += W; --y; }
+    if (x >= W) { x -= W; ++y; }
+    return tok >= N ? 0u : grid_taps(x, y, H, W, lane);
 }
 
 // o[mt][j] += the term of rows 16 mt .. + 15 and channels 8 j .. + 7 (mma.sync accumulator layout), k = (tap of a pair, channel of eight).

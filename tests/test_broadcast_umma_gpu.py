@@ -1,4 +1,4 @@
-"""Broadcast on tensor memory for large agent counts: ragged patches of the grid, agents that do not fill a step, references that move from step
+"""Broadcast on tensor memory for large agent counts: ragged patches of the grid, runs of its tokens, agents that do not fill a step, references that move from step
 to step, against the fp64 oracle."""
 import pytest
 import torch
@@ -10,20 +10,32 @@ from tests.parity_util import assert_close, make_module, to_dev, to_np
 pytestmark = pytest.mark.gpu
 
 SHAPES = [
-    # batch heads H    W   d   agents dtype  bias  dwc
-    (1, 2, 65, 97, 64, 72, "bf16", True, True),       # two steps, the second of eight agents; a last patch of one row, of one column
-    (1, 1, 8, 784, 64, 128, "f16", True, True),       # one row of patches
-    (1, 1, 787, 9, 64, 144, "bf16", True, True),      # patches nine columns wide, three steps
-    (2, 1, 88, 71, 40, 200, "f16", False, True),      # four steps, channels padded
-    (1, 1, 96, 64, 56, 248, "bf16", True, False),
-    (3, 2, 75, 117, 64, 256, "bf16", True, True),
+    # batch heads H    W   d   agents dtype  bias  dwc  launches (3: aggregation, merge and broadcast; 2: register tiles)
+    (1, 2, 65, 97, 64, 72, "bf16", True, True, 2),       # tokens no multiple of eight
+    (1, 1, 8, 784, 64, 128, "f16", True, True, 3),       # one row of patches
+    (1, 1, 787, 9, 64, 144, "bf16", True, True, 2),
+    (2, 1, 88, 71, 40, 200, "f16", False, True, 3),      # four steps, channels padded, a last patch of seven columns
+    (1, 1, 96, 64, 56, 248, "bf16", True, False, 3),
+    (3, 2, 75, 117, 64, 256, "bf16", True, True, 2),
+    # patches
+    (1, 2, 72, 100, 64, 72, "bf16", True, True, 3),      # two steps, the second of eight agents; last patches of four columns
+    (2, 1, 70, 112, 64, 144, "f16", True, True, 3),      # three steps; last patches of six rows
+    (1, 1, 123, 104, 64, 256, "bf16", True, True, 3),    # both, a long axis
+    # runs of 128 tokens
+    (2, 2, 1, 3080, 64, 256, "bf16", True, True, 3),     # one row, a last run of eight tokens
+    (1, 2, 3080, 1, 64, 200, "f16", True, True, 3),      # one column
+    (1, 1, 2, 4100, 64, 144, "bf16", True, True, 3),     # two rows, a long axis
+    (1, 1, 788, 10, 64, 144, "bf16", True, True, 3),     # more rows than one in a run
+    (2, 1, 1048, 3, 56, 248, "bf16", True, True, 3),
+    (2, 1, 3, 2736, 40, 256, "f16", False, True, 3),     # a run in the middle of a row, channels padded
+    (1, 2, 66, 100, 64, 72, "bf16", True, False, 3),     # no window
 ]
 
 
 @pytest.mark.parametrize("rising", [False, True], ids=["", "rising"])
 @pytest.mark.parametrize("case", SHAPES, ids=[f"B{c[0]}h{c[1]}_{c[2]}x{c[3]}_d{c[4]}_n{c[5]}" for c in SHAPES])
 def test_patches_and_steps(case, rising):
-    B, heads, H, W, d, n, dtype, bias, dwc = case
+    B, heads, H, W, d, n, dtype, bias, dwc, launches = case
     w = Workload("patch", B, heads, H, W, d, 9, dtype, False, dwc, 1.0, seed=300 + H * W + n)
     inp = make_inputs(w, bias_std=0.5, dwc_std=0.2)
     g = torch.Generator().manual_seed(n)
@@ -43,7 +55,7 @@ def test_patches_and_steps(case, rising):
     mod.forward(to_dev(inp["q"]), to_dev(inp["k"]), to_dev(inp["v"]), H, W, n, agents=agents.cuda(), b1=to_dev(b1), b2=to_dev(b2),
                 dwc_weight=to_dev(inp["dwc"]), out=out)
     torch.cuda.synchronize()
-    assert mod.query_status() == 0
+    assert mod.query_status() == 0 and mod.last_launch_count() == launches
     for b, h in {(0, 0), (B - 1, heads - 1)}:
         one = lambda x: None if x is None else to_np(x[b:b + 1, h:h + 1])
         hd = lambda x: None if x is None else to_np(x[h:h + 1])
@@ -67,3 +79,24 @@ def test_partial_states_of_the_aggregation_hold_the_weights_as_rounded(n, dtype)
     sums, products = state[rows:2 * rows][:n], state[2 * rows:].view(rows, 64)[:n]
     assert float(sums.min()) > 0
     assert float((products / sums[:, None] - 1).abs().max()) <= 4.2e-6
+
+
+@pytest.mark.parametrize("H,W", [(1, 16384), (16384, 1), (2, 8192), (1640, 10)])
+def test_thin_grids_take_as_long_as_square_ones(H, W):
+    """The same tokens in a row, in a column or in a square are the same work.  (Patches of 8 x 16 tokens alone took 2.4 to 8 times as long.)"""
+    def best(H, W):
+        w = Workload("thin", 1, 16, H, W, 64, 1, "bf16", False, True, 1.0, seed=5)
+        g = torch.Generator(device="cuda")
+        q, k, v = (torch.randn((1, 16, H * W, 64), generator=g, device="cuda").bfloat16() for _ in range(3))
+        a, f = torch.randn((1, 16, 256, 64), device="cuda").bfloat16(), torch.randn((16, 64, 3, 3), device="cuda").bfloat16()
+        mod, times = make_module(w, max_agents=256), []
+        for _ in range(6):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            for _ in range(8):
+                mod.forward(q, k, v, H, W, 256, agents=a, dwc_weight=f)
+            t1.record()
+            t1.synchronize()
+            times.append(t0.elapsed_time(t1))
+        return min(times)
+    assert best(H, W) <= 1.6 * best(128, 128)
