@@ -95,8 +95,9 @@ __device__ __forceinline__ void dwc_patch(float (&o)[2][4][4], const uint32_t (&
         for (int pr = 0; pr < 5; ++pr)
 #pragma unroll
             for (int mt = 0; mt < 2; ++mt) {
-                const int a = 3 * mt + 2 * pr, b = 3 * mt + (pr < 4 ? 2 * pr + 1 : 8);       // (the tenth tap weighs nothing)
-                const uint32_t k[4] = {f[a >> 1][2 * (a & 1)], f[a >> 1][2 * (a & 1) + 1], f[b >> 1][2 * (b & 1)], f[b >> 1][2 * (b & 1) + 1]};
+                const int a = 3 * mt + 2 * pr, b = pr < 4 ? a + 1 : 0;
+                uint32_t k[4] = {f[a >> 1][2 * (a & 1)], f[a >> 1][2 * (a & 1) + 1], f[b >> 1][2 * (b & 1)], f[b >> 1][2 * (b & 1) + 1]};
+                if (pr == 4) k[2] = k[3] = 0u;                         // the tenth tap: no token (nothing times an infinity is NaN)
                 mma16816<T>(o[mt][j], k, w[2 * pr], w[2 * pr + 1]);
             }
     }

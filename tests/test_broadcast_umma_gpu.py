@@ -4,8 +4,9 @@ import pytest
 import torch
 
 from oracle import agent_attention_oracle as orc
-from paper_2312_08874_b200 import Workload, make_inputs
-from tests.parity_util import assert_close, make_module, to_dev, to_np
+from paper_2312_08874_b200 import AA_PATH_UNFUSED, Workload, make_inputs
+from tests.parity_util import assert_close, gpu_forward, make_module, to_dev, to_np
+from tests.test_stream_cut_gpu import KINDS, extreme
 
 pytestmark = pytest.mark.gpu
 
@@ -100,3 +101,20 @@ def test_thin_grids_take_as_long_as_square_ones(H, W):
             times.append(t0.elapsed_time(t1))
         return min(times)
     assert best(H, W) <= 1.6 * best(128, 128)
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("case", [(2, 1, 72, 100, 64, 12), (1, 2, 656, 12, 64, 12), (1, 1, 96, 96, 40, 16)], ids=["patches", "runs", "d40"])
+def test_extreme_numbers_reach_as_far_as_on_register_tiles(case, kind):
+    """Rows of biases that remove everything, finite biases beyond +-30000, an infinite value under a positive filter, NaN: what is not finite is the
+    same, and what is finite as close as the two kernels are otherwise."""
+    B, heads, H, W, d, pool = case
+    w = Workload("extreme", B, heads, H, W, d, pool, "bf16", True, True, 1.0, seed=130 + H * W)
+    inp = make_inputs(w, bias_std=0.5, dwc_std=0.2)
+    extreme(inp, kind, "bf16", W)
+    mod = make_module(w)
+    out, tiles = gpu_forward(mod, w, inp), gpu_forward(make_module(w, path=AA_PATH_UNFUSED), w, inp)
+    assert mod.last_launch_count() == 4
+    assert torch.equal(out.isnan(), tiles.isnan()) and torch.equal(out.isinf(), tiles.isinf())
+    both = out.isfinite()
+    assert not both.any() or float((out[both].float() - tiles[both].float()).abs().max()) <= 2e-2
