@@ -15,14 +15,15 @@
 //                        writes the probabilities back over them as the A operand of P V.
 //                        A row's reference maximum moves only when exceeded by a margin; only then does the thread wait for products, and
 //                        rescales its accumulator row in tensor memory.
-// At the end the two token halves of a row meet in shared memory and each chain (up to 128 agents), or the block, writes one partial state;
+// At the end the two token halves of a row, and the chains of up to 128 agents, meet in shared memory and the block writes one partial state;
 // a second small kernel merges the slab's partials in a fixed order, spread over many blocks (a merge by
 // the slab's last block alone took longer than the streaming part).
 // Every wait is bounded (pipe.cuh).  No TMA multicast, no clusters.
 //
 // What bounds it: the row warps' instructions and exponentials (half of the time at the special-function rate), then HBM.  With probabilities through shared
 // memory, a wait for the products of the tile before in every tile and arrivals of single threads, 16 slabs of a 256 x 256 grid with 256
-// agents took 177 us; this way 133.
+// agents took 177 us; this way 133.  (A state per chain of up to 128 agents gave the merge twice as much to read: one slab of 128 x 128 tokens, 128 agents,
+// whole pass 21.5 us; joined in the block 18.8.)
 #include "merge.cuh"
 #include "stream_common.cuh"
 
@@ -68,8 +69,8 @@ struct UmmaAggArgs {
 };
 }  // namespace
 
-// ROUNDED: see umma_sums_rounded
-template <typename T, bool ROUNDED>
+// ROUNDED: see umma_sums_rounded; MB: 128-row agent blocks
+template <typename T, bool ROUNDED, int MB>
 __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_constant__ UmmaAggArgs g) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ int s_dead;
@@ -81,7 +82,7 @@ __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_cons
     const int split = blockIdx.x, slab = blockIdx.y;
     const int head = slab % p.heads;
     const int n = p.rows, N = p.cols;
-    const int MB = g.rows_pad >> 7;                       // 128-row agent blocks
+    constexpr int rows_pad = 128 * MB;
     const bool has_bias = p.bias != nullptr;
     const int tiles_all = (N + KT - 1) / KT;
     const int t0 = split * g.tps, t1 = min(tiles_all, t0 + g.tps);
@@ -107,8 +108,8 @@ __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_cons
     pdl_release_next();
 
     const uint32_t sA = smem_u32(smem + OFF_A), ring = smem_u32(smem + OFF_RING);
-    const size_t pf = partial_floats(g.rows_pad, 64);
-    float* slab_parts = p.partials + (size_t)slab * gridDim.x * (MB == 1 ? 2 : 1) * pf;
+    const size_t pf = partial_floats(rows_pad, 64);
+    float* part = p.partials + ((size_t)slab * gridDim.x + split) * pf;
 
     if (warp == 16) {
         // ------------------------------------------------------------------ producer
@@ -288,20 +289,34 @@ __global__ void __launch_bounds__(NT, 1) aggregate_umma_kernel(const __grid_cons
         }
         asm volatile("bar.sync %0, 256;\n" ::"r"(1 + m) : "memory");       // the chain's own barrier
         if (c == 0) {
-            const float om = sX[64], ol = sX[65];
-            const float mm = fmaxf(m_ref, om);
-            const float bs = (mm == -INFINITY) ? 0.f : mm;
-            const float wa = fast_exp2((m_ref - bs) * kLog2e), wb = fast_exp2((om - bs) * kLog2e);
-            float* part = slab_parts + (size_t)(MB == 1 ? 2 * split + m : split) * pf;
-            part[row] = mm * kLog2e;                       // the merge works in log2 units
-            part[g.rows_pad + row] = (started ? l : 0.f) * wa + ol * wb;
-            float* pacc = part + 2 * (size_t)g.rows_pad + (size_t)row * 64;
+            // state of the row: (reference, sum, products), joined with another one in shared memory
+            float mm = m_ref, ls = started ? l : 0.f;
+            auto join = [&](const float* x) {
+                const float om = x[64], mn = fmaxf(mm, om), bs = (mn == -INFINITY) ? 0.f : mn;
+                const float wa = fast_exp2((mm - bs) * kLog2e), wb = fast_exp2((om - bs) * kLog2e);
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const float4 xv = *reinterpret_cast<const float4*>(sX + 4 * k);
-                *reinterpret_cast<float4*>(pacc + 4 * k) =
-                    make_float4(o[4 * k] * wa + xv.x * wb, o[4 * k + 1] * wa + xv.y * wb,
-                                o[4 * k + 2] * wa + xv.z * wb, o[4 * k + 3] * wa + xv.w * wb);
+                for (int k = 0; k < 16; ++k) {
+                    const float4 v = *reinterpret_cast<const float4*>(x + 4 * k);
+                    o[4 * k] = o[4 * k] * wa + v.x * wb; o[4 * k + 1] = o[4 * k + 1] * wa + v.y * wb;
+                    o[4 * k + 2] = o[4 * k + 2] * wa + v.z * wb; o[4 * k + 3] = o[4 * k + 3] * wa + v.w * wb;
+                }
+                ls = ls * wa + x[65] * wb;
+                mm = mn;
+            };
+            auto put = [&](float* x) {
+#pragma unroll
+                for (int k = 0; k < 16; ++k) *reinterpret_cast<float4*>(x + 4 * k) = make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+            };
+            join(sX);
+            if (MB == 1) {                                 // and the other chain's (its tiles of the same agents)
+                if (m == 1) { put(sX); sX[64] = mm; sX[65] = ls; }
+                asm volatile("bar.sync 4, 256;\n" ::: "memory");
+                if (m == 0) join(sX + 128 * 68);
+            }
+            if (MB == 2 || m == 0) {
+                part[row] = mm * kLog2e;                   // the merge works in log2 units
+                part[rows_pad + row] = ls;
+                put(part + 2 * rows_pad + row * 64);
             }
         }
     }
@@ -400,22 +415,24 @@ AggPlan plan_aggregate_umma(int slabs, int n_agents, int n_tokens, int d, int sm
     if (splits > 64) splits = 64;
     const int tps = (tiles + splits - 1) / splits;
     pl.splits = (tiles + tps - 1) / tps;
-    pl.parts = pl.splits * (pl.rows_pad == 128 ? 2 : 1);          // (up to 128 agents: each chain writes its own)
+    pl.parts = pl.splits;
     return pl;
 }
 
 template <typename T>
 static cudaError_t launch_umma_t(const UmmaAggArgs& g, cudaStream_t st) {
-    auto kern = umma_sums_rounded(g.a.cols, g.a.d) ? aggregate_umma_kernel<T, true> : aggregate_umma_kernel<T, false>;
+    const bool one = g.rows_pad == 128;
+    auto kern = umma_sums_rounded(g.a.cols, g.a.d) ? (one ? aggregate_umma_kernel<T, true, 1> : aggregate_umma_kernel<T, true, 2>)
+                                                   : (one ? aggregate_umma_kernel<T, false, 1> : aggregate_umma_kernel<T, false, 2>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     dim3 grid(g.a.splits, g.a.slabs);
     e = launch_dependent(kern, grid, NT, kSmemBytes, st, g);
     if (e != cudaSuccess) return e;
-    const int parts = g.a.splits * (g.rows_pad == 128 ? 2 : 1);
-    const bool one = parts <= 16;
-    const int rows = one ? 16 : 4;
-    return launch_dependent(one ? merge_umma_kernel<T, 1> : merge_umma_kernel<T, 4>, dim3((g.a.rows + rows - 1) / rows, g.a.slabs), 256, 0, st,
+    const int parts = g.a.splits;
+    const bool few = parts <= 16;
+    const int rows = few ? 16 : 4;
+    return launch_dependent(few ? merge_umma_kernel<T, 1> : merge_umma_kernel<T, 4>, dim3((g.a.rows + rows - 1) / rows, g.a.slabs), 256, 0, st,
                             (const float*)g.a.partials, parts, g.rows_pad, g.a.rows, g.a.d, static_cast<T*>(g.a.out));
 }
 

@@ -7,6 +7,8 @@ a fixed array inside the library instead of a caller-provided workspace.  It mus
 `agent_attn_aggregate` returns, on consecutive calls that reuse the array, and must refuse
 shapes that do not fit the array.
 """
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -60,3 +62,16 @@ def test_static_scratch_rejects_shapes_beyond_its_size():
     with pytest.raises(AgentAttnError) as e:
         mod.aggregate_static(agents, kv, kv)
     assert e.value.status == 3 and "built-in scratch" in str(e.value)
+
+
+@pytest.mark.parametrize("slabs,tokens,n,d", [(600, 3072, 128, 64)], ids=["both_chains_in_one_state"])
+def test_static_scratch_holds_the_shapes_of_many_slabs(slabs, tokens, n, d):
+    """One partial state of 128 agents a block: 600 x 128 x 66 x 4 bytes fit, two would not."""
+    w = WORKLOADS["cfg3_pvt_bf16"].scaled(batch=slabs)
+    mod = make_module(dataclasses.replace(w, head_dim=d, grid_h=1, grid_w=tokens), max_agents=n)
+    g = torch.Generator(device="cuda")
+    a, k, v = (torch.randn((slabs, w.heads, m, d), generator=g, device="cuda").bfloat16() for m in (n, tokens, tokens))
+    got = mod.aggregate_static(a, k, v)
+    assert mod.query_status() == 0
+    ref = torch.softmax(a[slabs - 1, 0].double() @ k[slabs - 1, 0].double().T * d ** -0.5, -1) @ v[slabs - 1, 0].double()
+    assert_close(got[slabs - 1, 0], ref.cpu().numpy(), "bf16")
