@@ -100,17 +100,20 @@ bool use_umma(const agent_attn_handle* h, int n_tokens, int n_agents) {
     return filled ? n_tokens >= 16384 || (n_tokens >= 8192 && slabs >= 4) : slabs <= 24 && (n_tokens >= 32768 || (n_tokens >= 16384 && slabs >= 8));
 }
 
-AggPlan plan_for(const agent_attn_handle* h, int n_tokens, int n_agents) {
-    const int slabs = h->cfg.batch * h->cfg.heads;
-    if (use_umma(h, n_tokens, n_agents))
-        return plan_aggregate_umma(slabs, n_agents, n_tokens, h->cfg.head_dim, h->sm_count);
-    if (use_simt(h)) return plan_aggregate_simt(slabs, n_agents, n_tokens, h->cfg.head_dim, h->sm_count);
-    AggPlan pl;                     // register tiles: the states of a slab meet in shared memory
+AggPlan plan_tiles(const agent_attn_handle* h, int n_agents) {      // register tiles: the states of a slab meet in shared memory
+    AggPlan pl;
     memset(&pl, 0, sizeof(pl));
     pl.rows_pad = (n_agents + 15) / 16 * 16;
     pl.dpad = h->cfg.head_dim;
     pl.splits = pl.row_blocks = 1;
     return pl;
+}
+AggPlan plan_for(const agent_attn_handle* h, int n_tokens, int n_agents) {
+    const int slabs = h->cfg.batch * h->cfg.heads;
+    if (use_umma(h, n_tokens, n_agents))
+        return plan_aggregate_umma(slabs, n_agents, n_tokens, h->cfg.head_dim, h->sm_count);
+    if (use_simt(h)) return plan_aggregate_simt(slabs, n_agents, n_tokens, h->cfg.head_dim, h->sm_count);
+    return plan_tiles(h, n_agents);
 }
 
 // Plan of the streaming path for a call shape (cached in the handle); ok = false where it does not apply.
@@ -216,8 +219,8 @@ TileArgs tile_args(const agent_attn_handle* h, int gh, int gw, int n, const Call
 
 int do_aggregate(agent_attn_handle* h, const void* A, const void* K, const void* V, const void* b1,
                  int N, int n, void* VA, float* partials, unsigned* tickets, cudaStream_t st,
-                 const CallLayout* cl = nullptr) {
-    const bool umma = use_umma(h, N, n);
+                 const CallLayout* cl = nullptr, bool on_tiles = false) {
+    const bool umma = !on_tiles && use_umma(h, N, n);
     if (!umma && !use_simt(h)) {
         TileArgs t = tile_args(h, 1, N, n, cl ? *cl : dense_call(h, N));
         t.a = A; t.k = K; t.v = V; t.b1 = b1; t.va = VA;
@@ -1024,9 +1027,13 @@ extern "C" int agent_attn_aggregate_static(agent_attn_handle* h, const void* A, 
         return fail(h, AA_ERR_INVALID_ARG, "pointers must be 16-byte aligned");
     // scratch layout: [partials | arrival counters], each 256-byte aligned
     const size_t slabs = (size_t)h->cfg.batch * h->cfg.heads;
-    const AggPlan pl = plan_for(h, n_tokens, n_agents);
-    const size_t part_bytes = align_up(slabs * (pl.parts > 0 ? pl.parts : 1) * partial_floats(pl.rows_pad, pl.dpad) * sizeof(float), 256);
-    const size_t need = part_bytes + align_up(slabs * sizeof(unsigned), 256);
+    auto part_bytes_of = [&](const AggPlan& pl) { return align_up(slabs * (pl.parts > 0 ? pl.parts : 1) * partial_floats(pl.rows_pad, pl.dpad) * sizeof(float), 256); };
+    const size_t ticket_bytes = align_up(slabs * sizeof(unsigned), 256);
+    size_t part_bytes = part_bytes_of(plan_for(h, n_tokens, n_agents));
+    // partial states of the tensor-memory kernel that do not fit: register tiles, which need none (their bytes count as they always have)
+    const bool on_tiles = part_bytes + ticket_bytes > AA_STATIC_SCRATCH_BYTES && use_umma(h, n_tokens, n_agents);
+    if (on_tiles) part_bytes = part_bytes_of(plan_tiles(h, n_agents));
+    const size_t need = part_bytes + ticket_bytes;
     if (need > AA_STATIC_SCRATCH_BYTES)
         return fail(h, AA_ERR_WORKSPACE,
                     "this shape needs %zu bytes of scratch but the built-in scratch holds %u bytes; "
@@ -1044,5 +1051,5 @@ extern "C" int agent_attn_aggregate_static(agent_attn_handle* h, const void* A, 
     // do_aggregate clears the arrival counters on the stream before the kernel; the partials are
     // fully rewritten by every call, so nothing else of the previous call's contents is read.
     return do_aggregate(h, A, K, V, b1, n_tokens, n_agents, VA_out, reinterpret_cast<float*>(s),
-                        reinterpret_cast<unsigned*>(s + part_bytes), (cudaStream_t)stream);
+                        reinterpret_cast<unsigned*>(s + part_bytes), (cudaStream_t)stream, nullptr, on_tiles);
 }

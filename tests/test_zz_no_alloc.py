@@ -64,9 +64,10 @@ def test_static_scratch_rejects_shapes_beyond_its_size():
     assert e.value.status == 3 and "built-in scratch" in str(e.value)
 
 
-@pytest.mark.parametrize("slabs,tokens,n,d", [(600, 3072, 128, 64)], ids=["both_chains_in_one_state"])
+@pytest.mark.parametrize("slabs,tokens,n,d", [(600, 3072, 128, 64), (600, 8192, 144, 40)], ids=["both_chains_in_one_state", "register_tiles"])
 def test_static_scratch_holds_the_shapes_of_many_slabs(slabs, tokens, n, d):
-    """One partial state of 128 agents a block: 600 x 128 x 66 x 4 bytes fit, two would not."""
+    """One partial state of 128 agents a block: 600 x 128 x 66 x 4 bytes fit, two would not.  600 states of 256 rows do not: register tiles, which need
+    none, run the shape."""
     w = WORKLOADS["cfg3_pvt_bf16"].scaled(batch=slabs)
     mod = make_module(dataclasses.replace(w, head_dim=d, grid_h=1, grid_w=tokens), max_agents=n)
     g = torch.Generator(device="cuda")
