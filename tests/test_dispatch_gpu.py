@@ -20,6 +20,11 @@ SHAPES = [
     (17, 1, 64, 96, 64, 12, 3),       # of many: register tiles
     (2, 1, 64, 128, 40, 16, 4),       # filled with agents, 40 channels: tensor memory
     (2, 1, 64, 128, 32, 16, 3),       # 32: register tiles
+    (4, 8, 48, 64, 40, 10, 4),        # 100 agents, 32 slabs: tensor memory, the broadcast on register tiles
+    (8, 8, 48, 64, 40, 10, 3),        # 64 slabs of few channels: register tiles
+    (8, 8, 24, 32, 64, 11, 1),        # a short axis, 121 agents: one kernel
+    (1, 1, 72, 96, 40, 15, 3),        # 225 agents of 40 channels, one slab: register tiles
+    (2, 1, 72, 96, 40, 15, 4),        # two: tensor memory
     (2, 1, 31, 33, 64, 8, 1),         # 1023 tokens: one kernel
     (2, 1, 15, 69, 64, 8, 3),         # 1035 on a grid too wide for the streaming kernels: three
     (48, 6, 9, 9, 128, 5, 1),         # slabs all resident: one kernel
