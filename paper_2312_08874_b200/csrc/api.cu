@@ -909,7 +909,7 @@ bool bwd_layout(const agent_attn_handle* h, int N, int n, BwdPlan* pl, BwdLayout
     w->a = 0; w->va = snd; w->dva = 2 * snd; w->da = 3 * snd;
     w->lse = 4 * snd; w->dot = w->lse + sn;
     w->dwd = w->dot + sn;
-    w->part = w->dwd + align_up((size_t)kFilterCopies * h->cfg.heads * h->cfg.head_dim * 9 * sizeof(float), 256);
+    w->part = w->dwd + align_up((filter_copy_words(h->cfg.heads, h->cfg.head_dim) + 1) * sizeof(float), 256);
     size_t part_floats = (size_t)slabs * pl->chunks * n * 2;
     if (part_floats * sizeof(float) < snd) part_floats = snd / sizeof(float);       // (mixed precision: two 16-bit terms of V_A)
     w->terms = w->part + align_up(part_floats * sizeof(float), 256);

@@ -403,7 +403,8 @@ cudaError_t backward_typed(const BwdCall& c, BwdArgs a, cudaStream_t st) {
     const size_t bias_elems = (size_t)a.heads * a.n * a.N;
     if (c.db1) AA_TRY(cudaMemsetAsync(c.db1, 0, bias_elems * sizeof(float), st));
     if (c.db2) AA_TRY(cudaMemsetAsync(c.db2, 0, bias_elems * sizeof(float), st));
-    if (c.dwd) AA_TRY(cudaMemsetAsync(c.ws_dwd, 0, (size_t)kFilterCopies * a.heads * a.d * 9 * sizeof(float), st));
+    const size_t copies = filter_copy_words(a.heads, a.d);                // and the word behind them
+    if (c.wd) AA_TRY(cudaMemsetAsync(c.ws_dwd + (c.dwd ? 0 : copies), 0, ((c.dwd ? copies : 0) + 1) * sizeof(float), st));
 
     bwd_pool_kernel<T><<<(unsigned)((snd + 255) / 256), 256, 0, st>>>(a, c.q, c.ws_a);
     AA_TRY(cudaGetLastError());

@@ -26,8 +26,16 @@ struct TailArgs {
     const void *v, *go, *wd;
     const float* da;
     float *dq, *dv, *dwd, *dwd_copies;
+    unsigned* handed;                  // nonzero once the gradient stages' results are there for bwd_pool_tail (zero on entry)
     int heads, H, W, d, n, p, strip, strips, passes, batch;
 };
+
+__device__ __forceinline__ void store_release(unsigned* p, unsigned v) { asm volatile("st.release.gpu.global.u32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory"); }
+__device__ __forceinline__ unsigned load_acquire(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 
 // Two channels of a token as loaded (zeros where there is no token; volatile: left to itself the compiler gathers the loads of several
 // rows and spills), and in fp32 on use.
@@ -83,9 +91,10 @@ __device__ __forceinline__ Column column_of(const TailArgs& a, int i) {
     return {i - s * a.W, s * a.strip, min(a.H, (s + 1) * a.strip)};
 }
 
-// BESIDE: the kernel before is bwd_conv_tail, whose blocks release this one once the gradient stages are complete and touch nothing that it
-// does; so it runs beside them, and waits for their end before its own (what comes next waits for this kernel alone).  What the stages wrote
-// is read past L1, which was not emptied since.
+// BESIDE: the kernel before is bwd_conv_tail, whose blocks touch nothing that this one does and release it once the gradient stages are complete;
+// so it runs beside them, and waits for their end before its own (what comes next waits for this kernel alone).  A release of the launch orders
+// no memory: bwd_conv_tail, which has waited for the stages, says so in `handed` with a release, every block here reads that with an acquire, and
+// one that finds nothing waits for the kernel before after all.  What the stages wrote is read past L1, which was not emptied since.
 template <bool BESIDE>
 __global__ void __launch_bounds__(kThreadsQ, 4) bwd_pool_tail_kernel(const TailArgs a) {
     __shared__ Windows yw[kAxis];
@@ -112,8 +121,10 @@ __global__ void __launch_bounds__(kThreadsQ, 4) bwd_pool_tail_kernel(const TailA
     if (!BESIDE) {
         pdl_wait_prior();
         pdl_release_next();
+        __syncthreads();
+    } else if (!__syncthreads_or(threadIdx.x == 0 && load_acquire(a.handed))) {
+        pdl_wait_prior();
     }
-    __syncthreads();
     if (cl < cols) {
     const float* da = a.da + (size_t)slab * a.n * d + 4 * cg;
     const int first = blockIdx.x * a.passes * cols, last = min(first + a.passes * cols, a.strips * W);
@@ -173,6 +184,7 @@ __global__ void __launch_bounds__(kThreadsV, sizeof(T) == 4 ? 4 : 5) bwd_conv_ta
         for (int k = 0; k < 9; ++k) tap[k] = make_float2(Elem<T>::to_f32(w[k]), Elem<T>::to_f32(w[9 + k]));
     }
     pdl_wait_prior();                                             // (before that: inputs only)
+    if (blockIdx.x + blockIdx.y + threadIdx.x == 0) store_release(a.handed, 1u);
     pdl_release_next();
     if (DWD)
 #pragma unroll
@@ -296,6 +308,7 @@ template <typename T> cudaError_t launch_tail(TailArgs a, int sm_count, cudaStre
 cudaError_t launch_backward_tail(int dtype, const BwdCall& c, cudaStream_t st) {
     TailArgs a;
     a.v = c.v; a.go = c.d_out; a.wd = c.wd; a.da = c.ws_da; a.dq = c.dq; a.dv = c.dv; a.dwd = c.dwd; a.dwd_copies = c.ws_dwd;
+    a.handed = reinterpret_cast<unsigned*>(c.ws_dwd) + filter_copy_words(c.heads, c.d);
     a.heads = c.heads; a.H = c.H; a.W = c.W; a.d = c.d; a.n = c.n; a.p = c.p; a.strip = a.strips = a.passes = 0; a.batch = c.slabs / c.heads;
     switch (dtype) {
         case kF32:  return launch_tail<float>(a, c.sm_count, st);

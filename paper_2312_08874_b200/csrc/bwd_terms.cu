@@ -191,7 +191,8 @@ template <typename T, typename E, int NT> cudaError_t pool_and_clear(const BwdCa
     cl.p[0] = c.ws_dva; cl.words[0] = 2 * c.region_bytes / sizeof(float);          // dV_A, dA
     cl.p[1] = c.db1; cl.words[1] = c.db1 ? bias : 0;
     cl.p[2] = c.db2; cl.words[2] = c.db2 ? bias : 0;
-    cl.p[3] = c.ws_dwd; cl.words[3] = c.dwd ? (size_t)kFilterCopies * c.heads * c.d * 9 : 0;
+    const size_t copies = filter_copy_words(c.heads, c.d);                          // and the word behind them
+    cl.p[3] = c.ws_dwd + (c.dwd ? 0 : copies); cl.words[3] = c.wd ? (c.dwd ? copies : 0) + 1 : 0;
     float* const rows[3] = {c.dq, c.dk, c.dv};
     for (int k = 0; k < 3; ++k) { cl.p[4 + k] = rows[k]; cl.words[4 + k] = clear_rows ? (size_t)c.slabs * c.H * c.W * c.d : 0; }
     return launch_pool_terms<T, E, NT>(pa, a_t, cl, pl, st);

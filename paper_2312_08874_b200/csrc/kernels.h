@@ -254,13 +254,14 @@ struct BwdArgs {
 };
 // One backward call: inputs in the handle's element type, gradients and workspace in fp32.
 constexpr int kFilterCopies = 16;
+inline size_t filter_copy_words(int heads, int d) { return (size_t)kFilterCopies * heads * d * 9; }
 struct BwdCall {
     const void *q, *k, *v, *d_out, *b1, *b2, *wd;
     float *dq, *dk, *dv, *db1, *db2, *dwd;
     float *ws_a, *ws_va, *ws_dva, *ws_da;     // [slabs][n][d] each; V_A, dV_A, dA contiguous in this order
     float *ws_lse, *ws_dot;                   // [slabs][n]
     float* ws_part;                           // [slabs][chunks][n][2]
-    float* ws_dwd;                            // [kFilterCopies][heads][d][9]: shares of the filter gradient (added)
+    float* ws_dwd;                            // [kFilterCopies][heads][d][9]: shares of the filter gradient (added), and a word of the tail's
     size_t region_bytes;                      // bytes from ws_va to ws_dva and from ws_dva to ws_da
     int slabs, heads, H, W, d, n, p, sm_count;
     float scale1, scale2;

@@ -64,3 +64,17 @@ def test_filter_gradient_is_shared_by_every_copy(case):
     copies = ws[at:at + 16 * heads * 64 * 9 * 4].view(torch.float32).view(16, heads, 64 * 9)
     used = (copies != 0).any(dim=2).sum(dim=0).tolist()
     assert used == [16] * heads, used
+
+
+@pytest.mark.parametrize("filter_grad", [True, False])
+def test_pooling_beside_the_depthwise_part_changes_nothing(filter_grad):
+    """dQ does not depend on the depthwise term.  Slabs of one tile have sums of a fixed order, so it is the same bit for bit with the term, whose
+    kernel the pooling then runs beside, and without."""
+    w = Workload("beside", 300, 3, 11, 11, 64, 3, "bf16", False, True, 1.0, seed=78)
+    inp, go, mod = make_inputs(w, dwc_std=0.2), to_dev(make_upstream_grad(w)), make_module(w)
+    q, k, v, f = (to_dev(inp[x]) for x in ("q", "k", "v", "dwc"))
+    want = mod.backward(q, k, v, go, 11, 11, 9)["dq"]
+    for _ in range(30):
+        got = mod.backward(q, k, v, go, 11, 11, 9, dwc_weight=f, need_filter_grad=filter_grad)
+        assert torch.equal(got["dq"], want)
+    assert mod.query_status() == 0
