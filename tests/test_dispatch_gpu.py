@@ -25,6 +25,8 @@ SHAPES = [
     (8, 8, 24, 32, 64, 11, 1),        # a short axis, 121 agents: one kernel
     (1, 1, 72, 96, 40, 15, 3),        # 225 agents of 40 channels, one slab: register tiles
     (2, 1, 72, 96, 40, 15, 4),        # two: tensor memory
+    (1, 1, 72, 96, 40, 10, 4),        # one, 100 agents: tensor memory
+    (2, 2, 96, 128, 32, 11, 4),       # 121 agents of 32 channels, four slabs: tensor memory
     (2, 1, 31, 33, 64, 8, 1),         # 1023 tokens: one kernel
     (2, 1, 15, 69, 64, 8, 3),         # 1035 on a grid too wide for the streaming kernels: three
     (48, 6, 9, 9, 128, 5, 1),         # slabs all resident: one kernel
