@@ -89,7 +89,8 @@ bool umma_shape(const agent_attn_handle* h, int n_tokens, int n_agents) {
 //   144 agents of 64 channels: 9216 tokens and more 1.12 to 2.01; 3072 and 4096 tokens 0.71 to 1.42
 //   256 agents of 40 channels: 9216 tokens and more 1.07 to 2.10; 3072 and 4096 tokens, 16 slabs and more 1.04 to 1.35, fewer 0.68 to 1.01; 200 to
 //     232 agents, one slab of 6912 tokens 0.96 to 0.98 (100 to 128 agents 1.05 to 1.19)
-//   144 agents of 40 channels: 16384 tokens and more 0.96 to 1.77; 9216 tokens, 8 slabs and more 1.06 to 1.40, fewer 0.87 to 1.05
+//   144 agents of 40 channels: 16384 tokens and more 1.06 to 1.77, but four slabs of 16384 without biases 0.92; 9216 tokens, 8 slabs and more 1.06 to
+//     1.40, fewer 0.87 to 1.05
 //   72 and 88 agents of 40 channels: 32 and 64 slabs of 9216 to 16384 tokens 0.91 to 0.99, 16 and fewer 1.08 and more
 //   256 agents of 32 channels: 16384 tokens and more 1.04 to 1.75; 9216 tokens, one or two slabs 0.95 to 1.08, more 0.99 to 1.28
 //   104 and 128 agents of 32 channels: 9216 to 16384 tokens, 32 and 64 slabs 0.84 to 0.89, 16 slabs 1.0, 4 slabs of 9216 tokens 0.96 and 0.98, of
@@ -105,7 +106,7 @@ bool use_umma(const agent_attn_handle* h, int n_tokens, int n_agents) {
     if (half && unaligned && (d > 48 ? n_tokens <= 1024 : slabs > 48)) return false;
     if (half && !unaligned && slabs > 24 && (d <= 32 || (d <= 48 && !filled))) return false;
     if (d > 48) return filled ? work >= (n_tokens >= 3072 ? 6144 : 32768) : n_tokens >= 7168 || (n_tokens >= 6144 && slabs <= 16);
-    if (d > 32) return filled ? n_tokens >= (slabs == 1 && !half ? 8192 : 6144) || (n_tokens >= 1536 && work >= 49152) : n_tokens >= 12288 || (n_tokens >= 8192 && slabs >= 8);
+    if (d > 32) return filled ? n_tokens >= (slabs == 1 && !half ? 8192 : 6144) || (n_tokens >= 1536 && work >= 49152) : n_tokens >= (slabs >= 8 ? 8192 : slabs <= 2 ? 12288 : 32768);
     return filled ? n_tokens >= 16384 || (n_tokens >= 8192 && slabs >= (half && !unaligned && n_tokens < 12288 ? 8 : 4)) : slabs <= 24 && (n_tokens >= 32768 || (n_tokens >= 16384 && slabs >= 8));
 }
 

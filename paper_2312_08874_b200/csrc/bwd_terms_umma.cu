@@ -594,6 +594,7 @@ bool backward_terms_umma_eligible(int dtype, int slabs, int n, int N, int d) {
 //   one of 8 heads, 128 x 128, 256                                                    602 /  596  597  603 /  563  568  626
 //   two of 8 heads, 92 x 151, 81 (5.9)                                                667 /  640  641  652 /  604  605  606
 //   two of 8 heads, 75 x 117, 144 (3.7)                                               600 /  591  595  601 /  555  591  589
+//   one of 8 heads, 92 x 151, 81 to 196 agents: 349 to 332, 468 to 459, 616 to 608 (stretches of 2); 256 agents 570 to 588
 //   one of 8 heads, 75 x 117, 256 agents of 40 channels (3.7)                         393 /  398  397  392 /  416  425  427
 //   eight of 2 heads, 128 x 128, 196 agents of 40 channels (6.9 a run of four)       1152 / 1115 1197 1202
 //   fourteen of 2 heads, 75 x 117, 144 agents of 40 channels (2.8 a run of three)     864 /  995
@@ -604,7 +605,7 @@ UmmaOrder backward_terms_umma_order(int slabs, int heads, int n, int N, int d, i
     // blocks have whole tiles of the axis, one more for some than for others: at most an eighth above the average
     auto even = [&](long long runs) { return (tiles + runs - 1) / runs * runs * 8 <= tiles * 9; };
     const bool wide = d > 48;                                           // (narrow rows: less to clear)
-    if (blocks > 1 && tiles >= (slabs == heads ? 5 : 3) * (long long)sm_count && even(sm_count) && (wide || slabs != heads)) return {2, 1};
+    if (blocks > 1 && tiles >= (slabs != heads ? 3 : n % 64 ? 5 : 6) * (long long)sm_count && even(sm_count) && (wide || slabs != heads)) return {2, 1};
     if (wide && slabs != heads && tiles >= 4 * lanes && even(lanes) && 4LL * heads * n * N >= 24 << 20) return {4, 0};
     return {0, 0};
 }
