@@ -101,7 +101,6 @@ __global__ void __launch_bounds__(NT, 1) broadcast_umma_kernel(const __grid_cons
     pp.status = p.status;
     pp.dead = reinterpret_cast<int*>(smem + OFF_DEAD);
     pp.bars = smem_u32(smem + OFF_BAR);
-    pp.ph = 0u;
     if (tid == 0) {
         *pp.dead = 0;
         for (int i = 0; i < kBars; ++i) {

@@ -151,7 +151,6 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_terms_umma_kernel(const __gri
     pp.status = p.status;
     pp.dead = reinterpret_cast<int*>(smem + OFF_DEAD);
     pp.bars = base;
-    pp.ph = 0u;
     if (tid == 0) {
         *pp.dead = 0;
         for (int i = 0; i < kBars; ++i) mbar_init(pp.bars + 8 * i, i == BAR_READ || i == BAR_P || i == BAR_BREAD ? 8u : i == BAR_OUT ? 4u : 1u);

@@ -110,7 +110,6 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_umma_kernel(const __grid_cons
     pp.status = p.status;
     pp.dead = &s_dead;
     pp.bars = base;
-    pp.ph = 0u;
     if (tid == 0) {
         s_dead = 0;
         for (int i = 0; i < kBars; ++i) mbar_init(pp.bars + 8 * i, i >= BAR_P && i < BAR_DONE ? 8u : i == BAR_OUT || i >= BAR_M ? 4u : 1u);

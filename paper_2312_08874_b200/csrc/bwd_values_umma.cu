@@ -104,7 +104,6 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_values_umma_kernel(const __gr
     pp.status = p.status;
     pp.dead = reinterpret_cast<int*>(smem + OFF_DEAD);
     pp.bars = base;
-    pp.ph = 0u;
     if (tid == 0) {
         *pp.dead = 0;
         for (int i = 0; i < kBars; ++i)

@@ -195,7 +195,7 @@ inline size_t fused_counter_words(int slabs) { return 3 * (size_t)slabs + 4; }
 // Whole module (Eq. 6) for small agent counts and long token grids (n <= 64, d = 64, N >= 1024, dense tensors)
 // as three streaming kernels, phase by phase over the batch (the second reads of Q and V come from L2):
 //   prep       agents A = Pooling(Q) (or the caller's A), scaled copies for the two logit products, biases
-//              clamped to finite values (B2 also padded to 64 columns), arrival counters cleared
+//              clamped to finite values (B2 also padded to 64 columns), the filter as diagonal operands
 //   aggregate  V_A = softmax(scale1 A K^T + B1) V: grid (splits, slabs), tcgen05 with the agents and the
 //              probabilities as tensor-memory operands, bias added inside the contraction
 //   broadcast  O = softmax(scale2 Q A^T + B2) V_A + DWC(V): persistent blocks over runs of row tiles

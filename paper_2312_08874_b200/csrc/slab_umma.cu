@@ -107,7 +107,6 @@ __global__ void __launch_bounds__(NT, 2) slab_umma_kernel(const __grid_constant_
     pp.status = p.status;
     pp.dead = reinterpret_cast<int*>(smem + OFF_DEAD);
     pp.bars = base + OFF_BAR;
-    pp.ph = 0u;
     if (tid == 0) {
         *pp.dead = 0;
         for (int i = 0; i < kBars; ++i) mbar_init(pp.bars + 8 * i, 1u);

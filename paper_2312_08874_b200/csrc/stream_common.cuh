@@ -1,19 +1,11 @@
 // Helpers of the streaming kernels for small agent counts (stream_prep.cu, stream_aggregate.cu,
-// stream_broadcast.cu): tcgen05.mma with the A operand in tensor memory, packed 16-bit conversions and
-// exponentials, bounded mbarrier waits with an explicit phase parity.
+// stream_broadcast.cu): packed 16-bit conversions, bounded mbarrier waits with an explicit phase parity, tensor maps.
 #pragma once
 #include "common.cuh"
 #include "kernels.h"
 #include "pipe.cuh"
 
 namespace aa {
-
-// One fp32 column of this thread's tensor-memory row.
-__device__ __forceinline__ uint32_t tmem_ld1(uint32_t taddr) {
-    uint32_t r;
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n" : "=r"(r) : "r"(taddr) : "memory");
-    return r;
-}
 
 // 16 consecutive fp32 columns of this thread's tensor-memory row <- registers
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16]) {
@@ -31,9 +23,7 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
         : "memory");
 }
 
-// Packed 16-bit arithmetic of the element type: two fp32 -> one pair (low half = first value), and the
-// base-2 exponential of a pair in one instruction (its result is the pair of probabilities, already in the
-// operand type of the next product).
+// Constants of the element type, and two fp32 -> one pair (low half = first value).
 template <typename T> struct Pair;
 template <> struct Pair<__nv_bfloat16> {
     static constexpr uint32_t kOne = 0x3F80u;            // 1.0
@@ -45,11 +35,6 @@ template <> struct Pair<__nv_bfloat16> {
         asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
         return d;
     }
-    __device__ static __forceinline__ uint32_t ex2(uint32_t x) {
-        uint32_t d;
-        asm("ex2.approx.ftz.bf16x2 %0, %1;" : "=r"(d) : "r"(x));
-        return d;
-    }
 };
 template <> struct Pair<__half> {
     static constexpr uint32_t kOne = 0x3C00u;
@@ -58,11 +43,6 @@ template <> struct Pair<__half> {
     __device__ static __forceinline__ uint32_t cvt(float lo, float hi) {
         uint32_t d;
         asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
-        return d;
-    }
-    __device__ static __forceinline__ uint32_t ex2(uint32_t x) {
-        uint32_t d;
-        asm("ex2.approx.f16x2 %0, %1;" : "=r"(d) : "r"(x));
         return d;
     }
 };

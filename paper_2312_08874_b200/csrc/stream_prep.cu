@@ -9,7 +9,6 @@
 //     columns make the agents past n drop out of the broadcast softmax without any masking instructions.
 //   * the depthwise filter as diagonal operand slices: the broadcast kernel evaluates the 3x3 term on the tensor
 //     core as nine products of a shifted V tile with diag(w[:, tap]).
-//   * the arrival counters of the aggregation are cleared.
 #include "stream_common.cuh"
 
 namespace aa {

@@ -63,31 +63,13 @@ __device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t a_desc, uint6
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
-// The same with the accumulate flag fixed at compile time (no predicate set-up in the issuing thread).
-template <int kAcc>
-__device__ __forceinline__ void umma_f16_c(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "n"(kAcc) : "memory");
-}
 // Arrive on an mbarrier (count 1) when all MMAs issued so far by this thread have completed.
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
 }
 
-// D[tmem] (+)= A[tmem] * B[smem]: the A operand sits in tensor memory, lane = row, each 32-bit column
-// holding two consecutive K elements (low half first).  Issued by ONE thread.
-__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
-
-// The same instructions for an issuing WARP in uniform control flow: every lane executes the surrounding code
+// D[tmem] (+)= A * B[smem] for an issuing WARP in uniform control flow (umma_ts_w: the A operand sits in tensor memory, lane = row, each 32-bit
+// column holding two consecutive K elements, low half first): every lane executes the surrounding code
 // (waits, address arithmetic), so that the compiler can keep descriptors and addresses in uniform registers, and
 // one elected lane (the same one every time) issues.  With the issue inside an `if (lane == 0)` region every
 // operand takes a detour through per-thread registers, which costs more than the instruction itself.
