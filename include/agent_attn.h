@@ -117,7 +117,9 @@ size_t agent_attn_workspace_bytes(const agent_attn_handle* h, int grid_h, int gr
  *               grid to a p x p agent grid with n = p * p (window of cell (ay, ax): rows
  *               floor(ay*H/p) .. ceil((ay+1)*H/p) - 1, columns likewise); then n_agents must be a
  *               perfect square with p <= min(grid_h, grid_w)
- *   bias        NULL, or biases of Eq. 5 (members may be NULL individually)
+ *   bias        NULL, or biases of Eq. 5 (members may be NULL individually).  -inf, or a type's lowest
+ *               value, removes a key or an agent; a row that is -inf throughout gives NaN.  The streaming
+ *               kernels (AA_PATH_AUTO) clamp biases to +-30000: such a row averages there
  *   dwc_weight  device [heads][d][3][3] or NULL (no DWC term).  tap (u, v) multiplies
  *               V[y + u - 1][x + v - 1]; taps outside the grid contribute zero
  *   out         device [B][heads][N][d]

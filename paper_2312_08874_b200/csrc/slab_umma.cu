@@ -14,8 +14,8 @@
 // Normalisers are sums of the rounded weights, so that the two agree.
 //
 // What bounds it: the chain of copies, products and barriers of a slab, about 14 us with two blocks to an SM (inputs 2.5, either softmax 2, V_A 2,
-// depthwise term 2.3), and code that runs once: 384 slabs of 196 tokens, 49 agents of 64 channels 31 us in two waves, register tiles 47.5 us
-// (14.3 M warp instructions, here 10 M); 147 slabs 14 us against 34.
+// depthwise term 2.3), and code that runs once: 384 slabs of 196 tokens, 49 agents of 64 channels 34 us in two waves, register tiles 47.5 us
+// (14.3 M warp instructions, here 13 M); 147 slabs 14 us against 34.
 #include "dwc_diag.cuh"
 #include "stream_common.cuh"
 #include "tile_pool.cuh"
