@@ -43,9 +43,8 @@ inline bool tok_grid_exists(const TokLayout& l, int batch, int heads, long long 
     bool hf;
     unsigned long long n[2], s[3];
     if (!tok_map_dims(l, batch, heads, H * W, &hf, n, s)) return false;
-    const unsigned long long row = (unsigned long long)l.st * 2 * W;
-    const unsigned long long sh = heads == 1 && s[1] < row * H ? row * H : (unsigned long long)l.sh * 2, last = hf ? row * H : sh * heads;
-    return (hf || sh >= row) && (batch == 1 || s[2] >= (hf ? row : sh)) && last < (1ull << 40);
+    const unsigned long long row = (unsigned long long)l.st * 2 * W, last = hf ? row * H : s[1] * heads;       // (s[1]: that of a single head too)
+    return (hf || s[1] >= row) && (batch == 1 || s[2] >= (hf ? row : s[1])) && last < (1ull << 40);
 }
 __host__ __device__ inline long long tok_offset(const TokLayout& l, int slab, int heads, long long tok) {
     return (long long)(slab / heads) * l.sb + (long long)(slab % heads) * l.sh + tok * l.st;

@@ -118,3 +118,18 @@ def test_extreme_numbers_reach_as_far_as_on_register_tiles(case, kind):
     assert torch.equal(out.isnan(), tiles.isnan()) and torch.equal(out.isinf(), tiles.isinf())
     both = out.isfinite()
     assert not both.any() or float((out[both].float() - tiles[both].float()).abs().max()) <= 2e-2
+
+
+@pytest.mark.parametrize("case", [(2, 2, 656, 12), (3, 1, 656, 12), (1, 2, 14, 568), (2, 1, 64, 128), (2, 2, 64, 128)],
+                         ids=["runs", "runs_one_head", "runs_one_entry", "patches_one_head", "patches"])
+def test_token_major_views_run_on_tensor_memory_as_dense_tensors_do(case):
+    B, heads, H, W = case
+    w = Workload("views", B, heads, H, W, 64, 12, "bf16", True, True, 1.0, seed=170 + H * W)
+    inp = make_inputs(w, bias_std=0.5, dwc_std=0.2)
+    mod = make_module(w)
+    dense = gpu_forward(mod, w, inp)
+    qkv = torch.stack([to_dev(inp[x]).permute(0, 2, 1, 3) for x in "qkv"], dim=2).contiguous()          # [B, N, 3, heads, d]
+    out = mod.forward_strided(*(qkv[:, :, i].permute(0, 2, 1, 3) for i in range(3)), H, W, w.agents, b1=to_dev(inp["b1"]), b2=to_dev(inp["b2"]),
+                              dwc_weight=to_dev(inp["dwc"]))
+    assert mod.last_launch_count() == 4 and mod.query_status() == 0
+    assert torch.equal(out, dense)
